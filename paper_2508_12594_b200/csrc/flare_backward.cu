@@ -1,0 +1,232 @@
+// Backward: plans, workspace layout, launches of the tensor-core and CUDA-core kernels.
+#include "flare_host.h"
+#include "flare_bwd.cuh"
+#include "flare_bwd_tc.cuh"
+
+namespace flare {
+namespace {
+
+template <int D, int DRT, bool kPadded, bool kAlt>
+int launch_bwd_dq_tc_a(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
+                     const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
+                     const float *lse_dec, const float *dd, float *part, uint32_t *status, cudaStream_t st) {
+    CUtensorMap tmK, tmV, tmG, tmQ;
+    int rc;
+    if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmV, V, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
+    if (DRT != 0) tmQ = tmK;   // unused: the narrow forms stage Q with their threads
+    else if ((rc = make_latent_map(&tmQ, Q, d)) != FLARE_OK) return rc;
+    const size_t smem = BwdDqSmem<D, kAlt>::total();
+    static std::atomic<uint64_t> smem_opt_in{0};
+    if (int rc_attr = ensure_big_smem(bwd_dq_tc_kernel<D, DRT, kPadded, kAlt>, smem_opt_in, 227 * 1024)) return rc_attr;
+    BwdDqTcArgs a;
+    a.Q = static_cast<const __nv_bfloat16 *>(Q);
+    a.Z = Z; a.dZ = dZ; a.lse_enc = lse_enc; a.de = de; a.lse_dec = lse_dec; a.dd = dd;
+    a.key_mask = mask; a.part = part; a.status = status;
+    a.B = d->B; a.H = d->H; a.N = d->N; a.M = d->M;
+    a.sl2 = d->scale * kLog2e;
+    a.tiles = p.tiles; a.splits = p.splits; a.pairs = p.pairs; a.partials_per_split = p.per_split;
+    dim3 grid(p.splits, d->H * p.pairs, d->B);
+    bwd_dq_tc_kernel<D, DRT, kPadded, kAlt><<<grid, kTcThreads, smem, st>>>(tmK, tmV, tmG, tmQ, a);
+    FLARE_CUDA(cudaGetLastError());
+    return FLARE_OK;
+}
+
+// (one latent block, M <= 128: the form whose slots take alternate tiles, with a deeper tile ring)
+template <int D, int DRT, bool kPadded>
+int launch_bwd_dq_tc_p(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
+                     const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
+                     const float *lse_dec, const float *dd, float *part, uint32_t *status, cudaStream_t st) {
+    if (d->M <= kTile)
+        return launch_bwd_dq_tc_a<D, DRT, kPadded, true>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st);
+    return launch_bwd_dq_tc_a<D, DRT, kPadded, false>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st);
+}
+
+template <int D, int DRT = 0>
+int launch_bwd_dq_tc(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
+                     const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
+                     const float *lse_dec, const float *dd, float *part, uint32_t *status, cudaStream_t st) {
+    // padded tokens: a key mask, or a last partial tile
+    if (mask != nullptr || d->N % kTile != 0)
+        return launch_bwd_dq_tc_p<D, DRT, true>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st);
+    return launch_bwd_dq_tc_p<D, DRT, false>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st);
+}
+
+template <int D, int DRT, int kMode, int kM, bool kPadded>
+int launch_bwd_token_tc_m(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const void *dY,
+                        const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
+                        const float *lse_dec, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st,
+                        int m0, int mc, float *kvacc) {
+    CUtensorMap tmK, tmV, tmG, tmQ;
+    int rc;
+    if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmV, V, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
+    if (DRT != 0) tmQ = tmK;   // unused: the narrow forms stage Q with their threads
+    else if ((rc = make_latent_map(&tmQ, Q, d)) != FLARE_OK) return rc;
+    BwdTokTcArgs a;
+    a.stages = BwdTokSmem<D>::stages(mc);
+    if (a.stages < 1) return FLARE_ERR_UNSUPPORTED;
+    const size_t smem = BwdTokSmem<D>::total(a.stages, mc);
+    static std::atomic<uint64_t> smem_opt_in{0};
+    if (int rc_attr = ensure_big_smem(bwd_token_tc_kernel<D, DRT, kMode, kM, kPadded>, smem_opt_in, 227 * 1024)) return rc_attr;
+    a.Q = static_cast<const __nv_bfloat16 *>(Q);
+    a.Z = Z; a.dZ = dZ; a.lse_enc = lse_enc; a.de = de; a.lse_dec = lse_dec; a.key_mask = mask;
+    a.dK = (__nv_bfloat16 *)dK; a.dV = (__nv_bfloat16 *)dV; a.dd = dd; a.status = status;
+    a.B = d->B; a.H = d->H; a.N = d->N; a.M = mc;
+    a.mtot = d->M; a.m0 = m0; a.first = m0 == 0; a.last = m0 + mc >= d->M; a.kvacc = kvacc;
+    a.scale = d->scale; a.sl2 = d->scale * kLog2e;
+    a.tiles = (d->N + kTile - 1) / kTile;
+    long per_head = sms / ((long)d->B * d->H);
+    if (per_head < 1) per_head = 1;
+    if (per_head > a.tiles) per_head = a.tiles;
+    bwd_token_tc_kernel<D, DRT, kMode, kM, kPadded><<<dim3((unsigned)per_head, d->H, d->B), kTcThreads, smem, st>>>(tmK, tmV, tmG, tmQ, a);
+    FLARE_CUDA(cudaGetLastError());
+    return FLARE_OK;
+}
+
+// The launch's range of latents is [m0, m0 + mc) (mc = 0: all of them); common sizes have forms of the kernel with
+// the number of latents as a compile-time constant.
+template <int D, int DRT = 0, int kMode = 0>
+int launch_bwd_token_tc(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const void *dY,
+                        const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
+                        const float *lse_dec, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st,
+                        int m0 = 0, int mc = 0, float *kvacc = nullptr) {
+    if (mc == 0) mc = d->M;
+    const bool padded = mask != nullptr || d->N % kTile != 0;   // a key mask, or a last partial tile
+#define FLARE_TOK(MM)                                                                                                     \
+    (padded ? launch_bwd_token_tc_m<D, DRT, kMode, MM, true>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, dd, \
+                                                            status, st, m0, mc, kvacc)                                   \
+            : launch_bwd_token_tc_m<D, DRT, kMode, MM, false>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, dd, \
+                                                             status, st, m0, mc, kvacc))
+    if (mc == 256) return FLARE_TOK(256);
+    if (mc == 128) return FLARE_TOK(128);
+    if (mc == 64) return FLARE_TOK(64);
+    if (mc == 512) return FLARE_TOK(512);
+    return FLARE_TOK(0);
+#undef FLARE_TOK
+}
+template <typename T, int D>
+int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V,
+                         const uint8_t *mask, const void *Y, const void *dY, const float *Z, const float *lse_enc,
+                         const float *lse_dec, float *dQ, void *dK, void *dV, char *ws, cudaStream_t st,
+                         bool skip_pass_a = false) {
+    // skip_pass_a: dZ and de are already in the workspace (the second of the two runs of the separate-queries variant)
+    const BwdLayout w = bwd_layout(d, sms);
+    float *part = reinterpret_cast<float *>(ws + w.part);
+    float *dZ = reinterpret_cast<float *>(ws + w.dz);
+    float *de = reinterpret_cast<float *>(ws + w.de);
+    float *dd = reinterpret_cast<float *>(ws + w.dd);
+    (void)Y;  // dY_n . Y_n is rebuilt from float32 quantities instead of the rounded stored Y
+    const long rows = (long)d->B * d->H * d->M;
+    const SimtPlan pa = simt_plan(d, sms), pb = bwd_dq_plan(d, sms);
+    FLARE_CUDA(cudaMemsetAsync(ws, 0, kHeaderBytes, st));
+    int dz_parts = pa.P;
+    bool dz_on_tc = skip_pass_a;
+    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+        if (!skip_pass_a && bwd_dz_on_tensor_cores(d)) {
+            const TcEncodePlan tp = tc_encode_plan(d, sms);
+            uint32_t *status = reinterpret_cast<uint32_t *>(ws);
+            const int rc = encode_dz_tc(d, tp, Q, K, dY, part, status, st, lse_dec);
+            if (rc != FLARE_OK) return rc;
+            dz_parts = tp.P;
+            dz_on_tc = true;
+        }
+    }
+    if (!dz_on_tc) {
+        bwd_dz_simt_kernel<T, D><<<dim3(pa.splits, d->H, d->B), kBwdThreads, 0, st>>>(
+            (const T *)Q, (const T *)K, (const T *)dY, lse_dec, part, d->B, d->H, d->N, d->M, pa.LM, pa.chunk, d->scale);
+        FLARE_CUDA(cudaGetLastError());
+    }
+    if (!skip_pass_a) {
+        bwd_dz_reduce_kernel<<<(unsigned)((rows * d->D + 255) / 256), 256, 0, st>>>(part, dZ, dz_parts, rows, d->D);
+        FLARE_CUDA(cudaGetLastError());
+        bwd_de_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(dZ, Z, de, rows, d->D);
+        FLARE_CUDA(cudaGetLastError());
+    }
+    bool tok_on_tc = false;
+    if constexpr (std::is_same<T, __nv_bfloat16>::value && D <= 32) {
+        constexpr int DK = D < 16 ? 16 : D;                     // width the kernels multiply (D < 16: narrow forms)
+        constexpr int DRT = D < 16 ? D : 0;
+        uint32_t *status = reinterpret_cast<uint32_t *>(ws);
+        if (bwd_dq_on_tensor_cores(d) && !token_in_ranges(d) && BwdTokSmem<DK>::stages(d->M) >= 1) {
+            const int rc = launch_bwd_token_tc<DK, DRT>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, dd,
+                                                        status, st);
+            if (rc != FLARE_OK) return rc;
+            tok_on_tc = true;
+        } else if (token_in_ranges(d)) {
+            // two series of launches over the latent ranges: dd[n] first, then the rows of dK and dV
+            float *kvacc = reinterpret_cast<float *>(ws + w.kvacc);
+            const int R = token_range(d);
+            for (int mode = 1; mode <= 2; ++mode)
+                for (int m0 = 0; m0 < d->M; m0 += R) {
+                    const int mc = d->M - m0 < R ? d->M - m0 : R;
+                    const int rc = mode == 1 ? launch_bwd_token_tc<DK, DRT, 1>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec,
+                                                                              dK, dV, dd, status, st, m0, mc, kvacc)
+                                             : launch_bwd_token_tc<DK, DRT, 2>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec,
+                                                                              dK, dV, dd, status, st, m0, mc, kvacc);
+                    if (rc != FLARE_OK) return rc;
+                }
+            tok_on_tc = true;
+        }
+    }
+    if (!tok_on_tc) {
+        bwd_token_simt_kernel<T, D><<<dim3((d->N + 127) / 128, d->H, d->B), 128, 0, st>>>(
+            (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, lse_enc, lse_dec, (T *)dK, (T *)dV, dd,
+            d->B, d->H, d->N, d->M, d->scale);
+        FLARE_CUDA(cudaGetLastError());
+    }
+    int dq_parts = pb.P;
+    bool dq_on_tc = false;
+    if constexpr (std::is_same<T, __nv_bfloat16>::value && D <= 32) {
+        if (bwd_dq_on_tensor_cores(d)) {
+            const int rc = launch_bwd_dq_tc<(D < 16 ? 16 : D), (D < 16 ? D : 0)>(d, tc_dq_plan(d, sms), Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part,
+                                               reinterpret_cast<uint32_t *>(ws), st);
+            if (rc != FLARE_OK) return rc;
+            dq_parts = tc_dq_plan(d, sms).P;
+            dq_on_tc = true;
+        }
+    }
+    if (!dq_on_tc) {
+        const size_t dyn = sizeof(float) * 3 * (size_t)pb.LM * (D + 1);
+        static std::atomic<uint64_t> smem_opt_in{0};
+        if (int rc_attr = ensure_big_smem(bwd_dq_simt_kernel<T, D>, smem_opt_in, (int)(sizeof(float) * 3 * 64 * (D + 1)))) return rc_attr;
+        bwd_dq_simt_kernel<T, D><<<dim3(pb.splits, d->H, d->B), kBwdThreads, dyn, st>>>(
+            (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, dd, lse_enc, lse_dec, part, d->B, d->H,
+            d->N, d->M, pb.LM, pb.chunk, d->scale);
+        FLARE_CUDA(cudaGetLastError());
+    }
+    bwd_dq_reduce_kernel<<<(unsigned)((long)d->H * d->M), kDqReduceThreads, 0, st>>>(part, dQ, dq_parts, d->B, d->H, d->M,
+                                                                                     d->D, d->scale);
+    FLARE_CUDA(cudaGetLastError());
+    return FLARE_OK;
+}
+
+template <typename T>
+int backward_simt(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const uint8_t *mask,
+                  const void *Y, const void *dY, const float *Z, const float *lse_enc, const float *lse_dec, float *dQ,
+                  void *dK, void *dV, char *ws, cudaStream_t st, bool skip_pass_a) {
+    switch (d->D) {
+        case 4: return launch_backward_simt<T, 4>(d, sms, Q, K, V, mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a);
+        case 8: return launch_backward_simt<T, 8>(d, sms, Q, K, V, mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a);
+        case 16: return launch_backward_simt<T, 16>(d, sms, Q, K, V, mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a);
+        case 32: return launch_backward_simt<T, 32>(d, sms, Q, K, V, mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a);
+        case 64: return launch_backward_simt<T, 64>(d, sms, Q, K, V, mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a);
+        default: return FLARE_ERR_UNSUPPORTED;
+    }
+}
+
+}  // namespace
+
+int backward_impl(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const uint8_t *mask, const void *Y,
+                  const void *dY, const float *Z, const float *lse_enc, const float *lse_dec, float *dQ, void *dK, void *dV,
+                  char *ws, cudaStream_t st, bool skip_pass_a) {
+    return d->dtype == FLARE_DTYPE_F32
+               ? backward_simt<float>(d, sms, Q, K, V, mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a)
+           : d->dtype == FLARE_DTYPE_F16
+               ? backward_simt<__half>(d, sms, Q, K, V, mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a)
+               : backward_simt<__nv_bfloat16>(d, sms, Q, K, V, mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a);
+}
+
+}  // namespace flare

@@ -22,7 +22,6 @@
 
 namespace flare {
 
-constexpr int kBwdThreads = 256;
 constexpr int kBwdTileN = 32;   // tokens staged in shared memory per step of the latent-parallel kernels
 constexpr int kBwdLatents = 32; // latents staged in shared memory per step of the token-parallel kernel
 
@@ -79,7 +78,7 @@ bwd_dz_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
 }
 
 // dZ[row][d] = sum_p part[p][row][d], partials added in index order.  One thread per (row, d).
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 bwd_dz_reduce_kernel(const float *__restrict__ part, float *__restrict__ dZ, int P, long rows, int D) {
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * D) return;
@@ -89,7 +88,7 @@ bwd_dz_reduce_kernel(const float *__restrict__ part, float *__restrict__ dZ, int
 }
 
 // de[row] = dZ_row . Z_row.  One thread per row.
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 bwd_de_kernel(const float *__restrict__ dZ, const float *__restrict__ Z, float *__restrict__ de, long rows, int D) {
     const long row = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= rows) return;
@@ -284,7 +283,7 @@ bwd_dq_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
 // q = b * P + p with q = slice, slice + S, ... (S = 128 / D) in index order, thread (0, d) the S slice sums in index
 // order: a fixed order, and the B * P loads of a row are spread over the block.
 constexpr int kDqReduceThreads = 128;
-__global__ void __launch_bounds__(kDqReduceThreads)
+static __global__ void __launch_bounds__(kDqReduceThreads)
 bwd_dq_reduce_kernel(const float *__restrict__ part, float *__restrict__ dQ, int P, int B, int H, int M, int D,
                      float scale) {
     __shared__ float s_a[kDqReduceThreads];

@@ -38,6 +38,11 @@ inline WorkspaceLayout make_layout(int P, long rows, int D, bool with_z) {
     return w;
 }
 
+// Shape of the CUDA-core kernels' blocks (their launch plans need it too).
+constexpr int kSimtThreads = 256;
+constexpr int kSimtTileN = 32;  // tokens staged in shared memory per step
+constexpr int kBwdThreads = 256;
+
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ void from_f32(float &dst, float x) { dst = x; }

@@ -1,0 +1,128 @@
+// Encode on the tensor cores: launches of the kernel's forms, the merge of the partial results.
+#include "flare_host.h"
+#include "flare_simt.cuh"
+
+namespace flare {
+namespace {
+
+// kAlt: one latent block (M <= 128), the CTA's two slots take alternate tiles: a form of its own with a deeper K/V ring
+template <int D, bool kPair, bool kDz, int DRT, bool kHiLo, bool kMaskBody, bool kFast, bool kAlt>
+int launch_encode_tc_a(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V,
+                       const uint8_t *mask, float *pm, float *pl, float *pacc, uint32_t *status, cudaStream_t st,
+                       const float *lse_dec, bool fallback) {
+    constexpr int DG = kPair ? 2 * D : D;
+    CUtensorMap tmK, tmV, tmQ;
+    int rc;
+    if ((rc = make_token_map(&tmK, K, d, kTile, DG)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmV, V, d, kTile, DG)) != FLARE_OK) return rc;
+    if (DRT != 0) tmQ = tmK;   // unused: the narrow forms stage Q with their threads
+    else if ((rc = make_latent_map(&tmQ, Q, d)) != FLARE_OK) return rc;
+    const size_t smem = EncodeSmem<DG, kAlt>::total();
+    static std::atomic<uint64_t> smem_opt_in{0};
+    if (int rc_attr = ensure_big_smem(encode_tc_kernel<D, kPair, kDz, DRT, kHiLo, kMaskBody, kFast, kAlt>, smem_opt_in, 227 * 1024)) return rc_attr;
+    EncodeTcArgs a;
+    a.Q = static_cast<const __nv_bfloat16 *>(Q);
+    a.lse_dec = lse_dec;
+    a.key_mask = mask; a.part_m = pm; a.part_l = pl; a.part_acc = pacc; a.status = status;
+    a.run_if = fallback ? status + kRedoEncodeWord : nullptr;
+    a.redo = status + kRedoEncodeWord;
+    a.B = d->B; a.H = d->H; a.N = d->N; a.M = d->M;
+    a.scale = d->scale; a.sl2 = d->scale * kLog2e;
+    a.tiles = p.tiles; a.splits = p.splits; a.pairs = p.pairs; a.partials_per_split = p.per_split;
+    dim3 grid(p.splits, (kPair ? d->H / 2 : d->H) * p.pairs, d->B);
+    encode_tc_kernel<D, kPair, kDz, DRT, kHiLo, kMaskBody, kFast, kAlt><<<grid, kFast ? kTcThreadsGuarded : kTcThreads, smem, st>>>(tmK, tmV, tmQ, a);
+    FLARE_CUDA(cudaGetLastError());
+    return FLARE_OK;
+}
+
+template <int D, bool kPair, bool kDz = false, int DRT = 0, bool kHiLo = false, bool kMaskBody = false, bool kFast = false>
+int launch_encode_tc(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V,
+                     const uint8_t *mask, float *pm, float *pl, float *pacc, uint32_t *status, cudaStream_t st,
+                     const float *lse_dec = nullptr, bool fallback = false) {
+    if constexpr (kPair) {
+        return launch_encode_tc_a<D, kPair, kDz, DRT, kHiLo, kMaskBody, kFast, true>(d, p, Q, K, V, mask, pm, pl, pacc, status, st, lse_dec, fallback);
+    } else {
+        // (one latent block without the element tests is reached by the dZ form only, see encode_impl)
+        if constexpr (kMaskBody || kDz)
+            if (d->M <= kTile)
+                return launch_encode_tc_a<D, kPair, kDz, DRT, kHiLo, kMaskBody, kFast, true>(d, p, Q, K, V, mask, pm, pl, pacc, status, st, lse_dec, fallback);
+        return launch_encode_tc_a<D, kPair, kDz, DRT, kHiLo, kMaskBody, kFast, false>(d, p, Q, K, V, mask, pm, pl, pacc, status, st, lse_dec, fallback);
+    }
+}
+// The fast form first (if wanted), then the exact form, which exits at once unless the fast one raised its flag.
+template <int D, bool kPair, int DRT, bool kHiLo, bool kMaskBody>
+int encode_tc_forms(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V,
+                    const uint8_t *mask, float *pm, float *pl, float *pacc, uint32_t *status, cudaStream_t st, bool fast) {
+    if (fast) {
+        const int rc = launch_encode_tc<D, kPair, false, DRT, kHiLo, kMaskBody, true>(d, p, Q, K, V, mask, pm, pl, pacc, status, st);
+        if (rc != FLARE_OK) return rc;
+    }
+    return launch_encode_tc<D, kPair, false, DRT, kHiLo, kMaskBody, false>(d, p, Q, K, V, mask, pm, pl, pacc, status, st, nullptr, fast);
+}
+
+}  // namespace
+
+int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
+                float *lse_enc, void *ws, cudaStream_t st) {
+    const DeviceView di = device_info();
+    const long rows = (long)d->B * d->H * d->M;
+    const int P = partials_for(d, di.sms);
+    WorkspaceLayout w = make_layout(P, rows, d->D, false);
+    char *base = static_cast<char *>(ws);
+    float *pm = reinterpret_cast<float *>(base + w.part_m);
+    float *pl = reinterpret_cast<float *>(base + w.part_l);
+    float *pacc = reinterpret_cast<float *>(base + w.part_acc);
+    FLARE_CUDA(cudaMemsetAsync(base, 0, kHeaderBytes, st));
+    int rc;
+    if (use_tc(d)) {
+        TcEncodePlan p = tc_encode_plan(d, di.sms);
+        uint32_t *status = reinterpret_cast<uint32_t *>(base);
+        // a caller that asks for lse_enc is saving Z for the backward: weights as two bf16 halves (see exp_chunk_hilo)
+        const bool fast = use_fast(d, kFastEncode);
+#define FLARE_ENC3(DD, PAIR, DRT, MB, HL) encode_tc_forms<DD, PAIR, DRT, HL, MB>(d, p, Q, K, V, mask, pm, pl, pacc, status, st, fast)
+#define FLARE_ENC2(DD, PAIR, DRT, MB) (lse_enc != nullptr ? FLARE_ENC3(DD, PAIR, DRT, MB, true) : FLARE_ENC3(DD, PAIR, DRT, MB, false))
+        // A call with a key mask has padding in every tile and takes the form that tests every element (see
+        // encode_tc_kernel).  Without a mask only a last partial tile has padding and either form serves; which one
+        // is faster was measured (B200): the form without the element tests where a CTA holds two latent blocks
+        // (M > 128: 0.80 -> 0.68 ms on the million-point shape, 223 -> 201 us at N = 131072, M = 512), the other
+        // where two slots share one block (M <= 128: 4-5 % apart).
+        const bool mask_body = mask != nullptr || d->M <= kTile;
+#define FLARE_ENC(DD, PAIR, DRT) (mask_body ? FLARE_ENC2(DD, PAIR, DRT, true) : FLARE_ENC2(DD, PAIR, DRT, false))
+        if (encode_head_pairs(d))
+            rc = d->D == 16 ? FLARE_ENC(16, true, 0) : FLARE_ENC(32, true, 0);
+        else
+            rc = d->D == 4    ? FLARE_ENC(16, false, 4)
+                 : d->D == 8  ? FLARE_ENC(16, false, 8)
+                 : d->D == 16 ? FLARE_ENC(16, false, 0)
+                 : d->D == 32 ? FLARE_ENC(32, false, 0)
+                              : FLARE_ENC(64, false, 0);
+#undef FLARE_ENC
+#undef FLARE_ENC2
+#undef FLARE_ENC3
+    } else {
+        SimtPlan p = simt_plan(d, di.sms);
+        rc = encode_simt(d, p, Q, K, V, mask, pm, pl, pacc, st);
+    }
+    if (rc != FLARE_OK) return rc;
+    if (P > 8)   // many partials (small problems spread over all SMs): a block per row shares the loads
+        merge_kernel<<<(unsigned)rows, kMergeThreads, 0, st>>>(pm, pl, pacc, Z, lse_enc, P, rows, d->D);
+    else
+        merge_serial_kernel<<<(unsigned)((rows * d->D + 255) / 256), 256, 0, st>>>(pm, pl, pacc, Z, lse_enc, P, rows, d->D);
+    FLARE_CUDA(cudaGetLastError());
+    return FLARE_OK;
+}
+
+// Pass A of the backward: the dZ form of the kernel (dY for V, lse_dec the decode log-sum-exp rows); partials to `part`.
+int encode_dz_tc(const flare_desc_t *d, const TcEncodePlan &tp, const void *Q, const void *K, const void *dY, float *part,
+                 uint32_t *status, cudaStream_t st, const float *lse_dec) {
+#define FLARE_DZ(DD, PAIR, DRT) launch_encode_tc<DD, PAIR, true, DRT>(d, tp, Q, K, dY, nullptr, nullptr, nullptr, part, status, st, lse_dec)
+    if (encode_head_pairs(d)) return d->D == 16 ? FLARE_DZ(16, true, 0) : FLARE_DZ(32, true, 0);
+    return d->D == 4    ? FLARE_DZ(16, false, 4)
+           : d->D == 8  ? FLARE_DZ(16, false, 8)
+           : d->D == 16 ? FLARE_DZ(16, false, 0)
+           : d->D == 32 ? FLARE_DZ(32, false, 0)
+                        : FLARE_DZ(64, false, 0);
+#undef FLARE_DZ
+}
+
+}  // namespace flare

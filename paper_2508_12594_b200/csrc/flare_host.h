@@ -1,0 +1,351 @@
+// Host-side helpers shared by the library's translation units: error text, device properties, argument checks, launch
+// plans and TMA descriptors; and the launchers that each translation unit provides to the entry points.
+#pragma once
+
+#include "../../include/flare.h"
+
+#include <algorithm>
+#include <atomic>
+#include <cmath>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+
+#include "flare_bwd_tc.cuh"
+#include "flare_common.cuh"
+#include "flare_ptx.cuh"
+#include "flare_tc.cuh"
+
+namespace flare {
+extern thread_local char g_cuda_error[256];   // text of the last CUDA error of this thread
+
+inline int cuda_fail(cudaError_t e, const char *what) {
+    snprintf(g_cuda_error, sizeof(g_cuda_error), "%s: %s", what, cudaGetErrorString(e));
+    return FLARE_ERR_CUDA;
+}
+
+#define FLARE_CUDA(call)                                      \
+    do {                                                      \
+        cudaError_t e__ = (call);                             \
+        if (e__ != cudaSuccess) return cuda_fail(e__, #call); \
+    } while (0)
+
+struct DeviceInfo {
+    std::atomic<int> checked{0};  // 0 = not yet, 1 = ok, -1 = wrong arch, -2 = no device
+    std::atomic<int> sms{148};
+};
+extern DeviceInfo g_dev[64];
+
+// Properties of the current device (cached per ordinal; concurrent first calls write the same values).  Without
+// a device the plan falls back to 148 SMs so that size queries still answer.
+struct DeviceView {
+    int checked, sms;
+};
+inline DeviceView device_info(int *ordinal_out = nullptr) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        cudaGetLastError();
+        return DeviceView{-2, 148};
+    }
+    if (ordinal_out) *ordinal_out = dev;
+    DeviceInfo &d = g_dev[dev];
+    int checked = d.checked.load(std::memory_order_acquire);
+    if (checked == 0) {
+        int major = 0, sms = 0;
+        if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            return DeviceView{-2, 148};
+        }
+        d.sms.store(sms > 0 ? sms : 148, std::memory_order_relaxed);
+        checked = (major == 10) ? 1 : -1;
+        d.checked.store(checked, std::memory_order_release);
+    }
+    return DeviceView{checked, d.sms.load(std::memory_order_relaxed)};
+}
+
+// The opt-in to more than 48 KB of dynamic shared memory is a property of (kernel, device): one bit per device
+// ordinal in a mask per kernel instantiation.  Setting it twice is harmless, so a race between host threads
+// only repeats the call.
+template <typename Kernel>
+int ensure_big_smem(Kernel kernel, std::atomic<uint64_t> &done, int bytes = 227 * 1024) {
+    int dev = 0;
+    FLARE_CUDA(cudaGetDevice(&dev));
+    const uint64_t bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_acquire) & bit) return FLARE_OK;
+    FLARE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    done.fetch_or(bit, std::memory_order_release);
+    return FLARE_OK;
+}
+
+inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+inline int check_desc(const flare_desc_t *d) {
+    if (d == nullptr) return FLARE_ERR_INVALID_ARG;
+    if (d->B <= 0 || d->H <= 0 || d->N <= 0 || d->M <= 0 || d->D <= 0) return FLARE_ERR_INVALID_ARG;
+    if (!std::isfinite(d->scale)) return FLARE_ERR_INVALID_ARG;
+    if (d->dtype != FLARE_DTYPE_F32 && d->dtype != FLARE_DTYPE_BF16 && d->dtype != FLARE_DTYPE_F16) return FLARE_ERR_UNSUPPORTED;
+    if (d->D != 4 && d->D != 8 && d->D != 16 && d->D != 32 && d->D != 64) return FLARE_ERR_UNSUPPORTED;
+    if (d->dtype == FLARE_DTYPE_BF16 && (d->M % 16 != 0 || d->M < 16 || d->M > 2048)) return FLARE_ERR_UNSUPPORTED;
+    if ((long)d->B * d->N > (1L << 31) - 1 || d->H > 65535 || d->B > 65535) return FLARE_ERR_UNSUPPORTED;
+    return FLARE_OK;
+}
+
+// Launch plan of the CUDA-core encode: LM latents x G token groups per block, `splits` blocks along N.
+struct SimtPlan {
+    int LM, G, splits, chunk, P;
+};
+
+inline SimtPlan simt_plan(const flare_desc_t *d, int sms) {
+    SimtPlan p;
+    p.LM = 1;
+    while (p.LM < d->M && p.LM < kSimtThreads) p.LM *= 2;
+    p.G = kSimtThreads / p.LM;
+    long bh = (long)d->B * d->H;
+    long want = (4L * sms + bh - 1) / bh;                  // about four blocks per SM in total
+    long most = (d->N + 255) / 256;                        // at least 256 tokens per block
+    long s = want < most ? want : most;
+    if (s < 1) s = 1;
+    p.chunk = (int)((d->N + s - 1) / s);
+    p.chunk = (p.chunk + kSimtTileN - 1) / kSimtTileN * kSimtTileN;
+    p.splits = (d->N + p.chunk - 1) / p.chunk;
+    p.P = p.splits * p.G;
+    return p;
+}
+
+// The tensor-core kernels take bfloat16 with D in {16, 32, 64} and a positive scale, and D = 8 or 4 as the narrow
+// forms of the D = 16 kernels: a token tile of 16 feature columns then spans two or four heads, so the tensor must
+// be at least 16 columns wide, and (TMA) its rows a multiple of 16 bytes.  Everything else (float32, non-positive
+// scale, narrower tensors) runs on the CUDA-core kernels.  FLARE_DEBUG_PATH=simt forces the latter.
+inline bool use_tc(const flare_desc_t *d) {
+    static const bool forced_simt = [] {
+        const char *e = std::getenv("FLARE_DEBUG_PATH");
+        return e != nullptr && std::strcmp(e, "simt") == 0;
+    }();
+    // (a scale so small that scale * kMaskedScore no longer dwarfs every real score would let padded tokens through the
+    // form that puts padding into the scores: such calls run on the CUDA cores too)
+    return !forced_simt && d->dtype == FLARE_DTYPE_BF16 && d->scale > 1e-20f &&
+           (d->D == 16 || d->D == 32 || d->D == 64 || (d->D == 8 && d->H >= 2) || (d->D == 4 && d->H >= 4 && d->H % 2 == 0));
+}
+
+// Which form of the tensor-core forward kernels runs (flare_set_path).
+extern std::atomic<int> g_path;
+
+// The fast forms (no running maximum, see kFastMaxLog2 in flare_tc.cuh) are followed by a launch of the exact
+// form that exits at once unless it is needed: two more launches per forward, which pay off from a few tens of
+// microseconds of work.
+enum FastStage { kFastEncode, kFastDecode };
+inline bool use_fast(const flare_desc_t *d, FastStage stage) {
+    if (!use_tc(d)) return false;
+    if (stage == kFastDecode && d->D > 32) return false;           // the streaming decode has no form for head width 64
+    const int path = g_path.load(std::memory_order_relaxed);
+    if (path == FLARE_PATH_EXACT) return false;
+    if (path == FLARE_PATH_FAST) return true;
+    // Measured (forward stage times, fast against exact form): encode wins from 128 latents (3-5 % there, 15 % at 256),
+    // is equal or loses at 32 and 64 latents of width 32; the streaming decode
+    // wins from 64 latents (16 % at 64 and 128) and loses at 32; below some tens of microseconds of work the two extra
+    // launches cost more than the forms gain.
+    // The head-pair form of encode (M <= 64, H even) wins at D = 16 since its K/V ring is deep (0.077 -> 0.062 ms on the
+    // 2-D mesh: its rows are short scans, in which the exact form rescales its accumulator on most units) and is equal
+    // at D = 32, where it has no room for the ones column and sums the weights in registers.
+    const bool pair16 = d->M <= 64 && d->H % 2 == 0 && d->D == 16;
+    const bool big_enough = stage == kFastEncode ? (d->M >= 128 || pair16) : d->M >= 64;
+    return big_enough && (double)d->B * d->H * d->N * d->M >= 3.0e7;
+}
+
+// Launch plan of the tensor-core encode: `pairs` CTAs per head along the latents (two 128-latent blocks each),
+// `splits` CTAs along N, about one CTA per SM in total.
+struct TcEncodePlan {
+    int tiles, pairs, splits, per_split, P;
+};
+
+// With at most 64 latents a CTA encodes two adjacent heads at once (see encode_tc_kernel).
+inline bool encode_head_pairs(const flare_desc_t *d) { return d->M <= 64 && d->H % 2 == 0 && d->D >= 16 && d->D <= 32; }
+
+inline TcEncodePlan tc_encode_plan(const flare_desc_t *d, int sms) {
+    TcEncodePlan p;
+    p.tiles = (d->N + kTile - 1) / kTile;
+    const int mb = (d->M + kTile - 1) / kTile;
+    p.pairs = (mb + 1) / 2;
+    long groups = (long)d->B * (encode_head_pairs(d) ? d->H / 2 : d->H) * p.pairs;
+    long s = sms / groups;
+    if (s < 1) s = 1;
+    if (s > p.tiles) s = p.tiles;
+    p.splits = (int)s;
+    p.per_split = (mb == 1) ? 4 : 2;
+    p.P = p.splits * p.per_split;
+    return p;
+}
+
+inline int partials_for(const flare_desc_t *d, int sms) { return use_tc(d) ? tc_encode_plan(d, sms).P : simt_plan(d, sms).P; }
+
+// ---- TMA descriptors (the driver entry point is looked up at run time; the library does not link libcuda)
+typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+inline EncodeTiledFn encode_tiled_fn() {
+    static EncodeTiledFn fn = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return reinterpret_cast<EncodeTiledFn>(p);
+    }();
+    return fn;
+}
+
+inline CUtensorMapSwizzle swizzle_for(int D) {
+    return D == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : D == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
+}
+
+// [B, N, H*D] bf16 viewed as a 3-D tensor (innermost H*D); box = `cols` columns (one head's D, or two adjacent
+// heads' 2D) x `rows` tokens.
+inline int make_token_map(CUtensorMap *m, const void *base, const flare_desc_t *d, int rows, int cols = 0) {
+    if (cols == 0) cols = d->D;
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) {
+        snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled not available");
+        return FLARE_ERR_CUDA;
+    }
+    const cuuint64_t C = (cuuint64_t)d->H * d->D;
+    cuuint64_t dims[3] = {C, (cuuint64_t)d->N, (cuuint64_t)d->B};
+    cuuint64_t strides[2] = {C * 2, C * 2 * (cuuint64_t)d->N};
+    cuuint32_t box[3] = {(cuuint32_t)cols, (cuuint32_t)rows, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for(cols), CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled(tokens) failed: %d", (int)r);
+        return FLARE_ERR_CUDA;
+    }
+    return FLARE_OK;
+}
+
+// Q_lat [H*M, D] bf16 as a 2-D tensor; box = 16 latent rows.
+inline int make_latent_map(CUtensorMap *m, const void *base, const flare_desc_t *d) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) {
+        snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled not available");
+        return FLARE_ERR_CUDA;
+    }
+    cuuint64_t dims[2] = {(cuuint64_t)d->D, (cuuint64_t)d->H * d->M};
+    cuuint64_t strides[1] = {(cuuint64_t)d->D * 2};
+    cuuint32_t box[2] = {(cuuint32_t)d->D, 16};
+    cuuint32_t estr[2] = {1, 1};
+    CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for(d->D), CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        snprintf(g_cuda_error, sizeof(g_cuda_error), "cuTensorMapEncodeTiled(latents) failed: %d", (int)r);
+        return FLARE_ERR_CUDA;
+    }
+    return FLARE_OK;
+}
+
+constexpr float kLog2e = 1.4426950408889634f;
+
+// Header words of a workspace beyond the error flag: set by the fast form of encode / decode when its inputs are
+// outside the range it is valid for; the exact form that follows runs only then.
+constexpr int kRedoEncodeWord = 2, kRedoDecodeWord = 3;
+
+// Decode over more latents than one launch holds in tensor memory (512 columns) is cut into ranges of latents; their
+// partial results take float32 rows [C][B*N*H][D] and log-sum-exps [C][B*N*H] behind the encode layout of the workspace.
+// One decode launch holds all M score columns of a token tile: up to kDecodeMaxM latents.
+constexpr int kDecodeMaxM = 512;
+
+// Ranges of latents a decode over more than kDecodeMaxM latents is cut into, and the scratch their partial results
+// take after the encode layout of the forward workspace: float32 rows [C][B*N*H][D] and log-sum-exps [C][B*N*H].
+constexpr int kDecodeRange = 256;   // latents per launch when a decode is cut into ranges
+inline int decode_ranges(const flare_desc_t *d) { return (d->M + kDecodeRange - 1) / kDecodeRange; }
+inline bool decode_in_ranges(const flare_desc_t *d) { return use_tc(d) && d->M > kDecodeMaxM; }
+inline size_t decode_range_bytes(const flare_desc_t *d) {
+    if (!decode_in_ranges(d)) return 0;
+    const size_t rows = (size_t)d->B * d->N * d->H;
+    return align_up(sizeof(float) * decode_ranges(d) * rows * d->D) + align_up(sizeof(float) * decode_ranges(d) * rows);
+}
+
+// Launch plans of the CUDA-core backward: pass A (dZ) reuses the encode plan; the dQ pass keeps three latent
+// rows per thread in shared memory and therefore caps its latent block at 64.
+// Pass A (dZ) runs as the dZ form of the tensor-core encode kernel wherever that kernel runs.
+inline bool bwd_dz_on_tensor_cores(const flare_desc_t *d) { return use_tc(d); }
+
+// Pass B for dQ runs on the tensor cores for narrow heads (S, A, C and the partial dQ of a group share its 128
+// TMEM columns: 3 * 32 + D).
+inline bool bwd_dq_on_tensor_cores(const flare_desc_t *d) { return use_tc(d) && d->D <= 32; }
+
+// Plan of the tensor-core dQ kernel: the encode plan without head pairing.
+inline TcEncodePlan tc_dq_plan(const flare_desc_t *d, int sms) {
+    TcEncodePlan p;
+    const int mb = (d->M + kTile - 1) / kTile;
+    p.tiles = (d->N + kTile - 1) / kTile;
+    p.pairs = (mb + 1) / 2;
+    long s = sms / ((long)d->B * d->H * p.pairs);
+    if (s < 1) s = 1;
+    if (s > p.tiles) s = p.tiles;
+    p.splits = (int)s;
+    p.per_split = (mb == 1) ? 4 : 2;
+    p.P = p.splits * p.per_split;
+    return p;
+}
+
+inline SimtPlan bwd_dq_plan(const flare_desc_t *d, int sms) {
+    SimtPlan p = simt_plan(d, sms);
+    if (p.LM > 64) p.LM = 64;
+    p.G = kBwdThreads / p.LM;
+    p.P = p.splits * p.G;
+    return p;
+}
+
+struct BwdLayout {
+    size_t part, dz, de, dd, kvacc, total;
+    int P;
+};
+
+// Latents one launch of the tensor-core token kernel keeps in shared memory (five operands of D-wide bf16 rows,
+// beside at least five tile stages); more are worked off in ranges of this many.
+inline int token_range(const flare_desc_t *d) { return d->D == 32 ? 256 : 512; }
+inline bool token_in_ranges(const flare_desc_t *d) { return bwd_dq_on_tensor_cores(d) && d->M > token_range(d); }
+
+inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
+    BwdLayout w;
+    const long rows = (long)d->B * d->H * d->M;
+    const int pa = simt_plan(d, sms).P, pb = bwd_dq_plan(d, sms).P;
+    w.P = pa > pb ? pa : pb;
+    if (bwd_dz_on_tensor_cores(d) && tc_encode_plan(d, sms).P > w.P) w.P = tc_encode_plan(d, sms).P;
+    if (bwd_dq_on_tensor_cores(d) && tc_dq_plan(d, sms).P > w.P) w.P = tc_dq_plan(d, sms).P;
+    size_t off = kHeaderBytes;
+    w.part = off; off += align_up(sizeof(float) * (size_t)w.P * rows * d->D);
+    w.dz = off;   off += align_up(sizeof(float) * (size_t)rows * d->D);
+    w.de = off;   off += align_up(sizeof(float) * (size_t)rows);
+    w.dd = off;   off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
+    w.kvacc = off;                                             // float32 sums of the rows of dK and dV over latent ranges
+    if (token_in_ranges(d)) off += align_up(sizeof(float) * 2 * (size_t)d->B * d->N * d->H * d->D);
+    w.total = off;
+    return w;
+}
+
+// ---- what the translation units provide
+int encode_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask,
+                float *pm, float *pl, float *pacc, cudaStream_t st);
+int decode_simt(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st);
+int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
+                float *lse_enc, void *ws, cudaStream_t st);
+int encode_dz_tc(const flare_desc_t *d, const TcEncodePlan &tp, const void *Q, const void *K, const void *dY, float *part,
+                 uint32_t *status, cudaStream_t st, const float *lse_dec);
+// range_scratch: decode_range_bytes(d) bytes, or null (then more than kDecodeMaxM latents take the CUDA-core kernel)
+int decode_impl(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec,
+                uint32_t *status, cudaStream_t st, char *range_scratch = nullptr);
+// skip_pass_a: dZ and de are already in the workspace (the second of the two runs of the separate-queries variant)
+int backward_impl(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const uint8_t *mask, const void *Y,
+                  const void *dY, const float *Z, const float *lse_enc, const float *lse_dec, float *dQ, void *dK, void *dV,
+                  char *ws, cudaStream_t st, bool skip_pass_a);
+size_t spectral_bytes(const flare_desc_t *d, int sms);
+int spectral_gram(const flare_desc_t *d, int sms, const void *Q, const void *K, const float *lse_enc, const float *lse_dec, float *G,
+                  void *workspace, cudaStream_t st);
+int spectral_eig(int32_t matrices, int32_t M, float *G, float *eigenvalues, float *U, int32_t sweeps, cudaStream_t st);
+
+
+}  // namespace flare

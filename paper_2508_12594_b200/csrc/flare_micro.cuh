@@ -111,4 +111,21 @@ __global__ void __launch_bounds__(64, 1) micro_mma_kernel(int iters, unsigned lo
     }
 }
 
+// The bounded wait of the kernels above, on its own: one thread waits for at most `budget_ns` on a barrier phase
+// that nothing ever completes, then takes the same way out as a kernel whose wait gave up (code into the block's
+// abort flag, from there into the workspace header).  Lets a caller see FLARE_ERR_TIMEOUT without a hung kernel.
+__global__ void selftest_wait_kernel(uint32_t *status, unsigned long long budget_ns) {
+    __shared__ uint64_t bar_mem;
+    __shared__ uint32_t flag;
+    if (threadIdx.x == 0) {
+        ptx::mbar_init(ptx::smem_u32(&bar_mem), 1);
+        flag = 0;
+        ptx::fence_mbar_init();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) ptx::mbar_wait_for(ptx::smem_u32(&bar_mem), 0, &flag, kErrSelftest | 1, budget_ns);
+    __syncthreads();
+    if (threadIdx.x == 0 && flag != 0 && status != nullptr) atomicCAS(status, 0u, flag);
+}
+
 }  // namespace flare

@@ -28,9 +28,6 @@ __device__ __forceinline__ float score_dot(const float (&a)[D], const float *b) 
     }
 }
 
-constexpr int kSimtThreads = 256;
-constexpr int kSimtTileN = 32;  // tokens staged in shared memory per step
-
 // Encode, split over N.  grid = (splits, H, B).  The block's 256 threads are LM latents x G token groups
 // (G = 256 / LM); thread (lm, g) folds the tokens j of its split with j % G == g into a running
 // (max, sum, row) triple for latent lm and writes it as partial number split*G + g.
@@ -106,7 +103,7 @@ encode_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
 // and the P loads of a row are spread over the block instead of queued in one thread (with P in the hundreds
 // for small problems the serial form took longer than the encode kernel itself).
 constexpr int kMergeThreads = 128;
-__global__ void __launch_bounds__(kMergeThreads)
+static __global__ void __launch_bounds__(kMergeThreads)
 merge_kernel(const float *__restrict__ part_m, const float *__restrict__ part_l, const float *__restrict__ part_acc,
              float *__restrict__ Z, float *__restrict__ lse_enc, int P, long rows, int D) {
     __shared__ float s_a[kMergeThreads], s_b[kMergeThreads];
@@ -147,7 +144,7 @@ merge_kernel(const float *__restrict__ part_m, const float *__restrict__ part_l,
 }
 
 // The same merge with one thread per (row, d), partials added in index order: for few partials and many rows.
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 merge_serial_kernel(const float *__restrict__ part_m, const float *__restrict__ part_l, const float *__restrict__ part_acc,
                     float *__restrict__ Z, float *__restrict__ lse_enc, int P, long rows, int D) {
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;

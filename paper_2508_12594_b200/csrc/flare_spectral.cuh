@@ -238,7 +238,7 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
 }
 
 // Sum of the token splits into G [B,H,M,M].  One thread per element.
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256)
 spectral_gram_reduce_kernel(const float *__restrict__ part, float *__restrict__ Gout, int splits, long heads, int M) {
     const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= heads * M * M) return;
@@ -295,7 +295,7 @@ spectral_gram_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, cons
 // Eigenvalues (descending) and, if U != null, eigenvectors (columns of U) of the symmetric matrices G [heads, M, M],
 // by cyclic two-sided Jacobi rotations on disjoint index pairs (round-robin ordering: M - 1 steps of M / 2 rotations
 // per sweep).  One block per matrix; G is overwritten.  Off the hot path: O(M^3) per sweep, about ten sweeps.
-__global__ void __launch_bounds__(1024)
+static __global__ void __launch_bounds__(1024)
 spectral_jacobi_kernel(float *__restrict__ Gall, float *__restrict__ evals, float *__restrict__ Uall, int M, int sweeps) {
     extern __shared__ float sh[];
     float *cs = sh;                         // [M/2 pairs] cosines, then sines
