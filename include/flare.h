@@ -239,9 +239,10 @@ int flare_spectral_gram(const flare_desc_t *desc, const void *Q_lat, const void 
 
 /*
  * The M x M symmetric eigenproblems of Algorithm 1 (its step "U Sigma^2 U^T = J J^T"), O(M^3) each and off the hot
- * path: cyclic Jacobi rotations, one thread block per matrix.  G [matrices, M, M] float32 is destroyed;
+ * path.  Eigenvalues alone (U = NULL): Householder tridiagonalisation, then bisection on Sturm counts; with eigenvectors:
+ * cyclic Jacobi rotations, one thread block per matrix.  G [matrices, M, M] float32 is destroyed;
  * eigenvalues [matrices, M] come out in descending order; U [matrices, M, M] (may be NULL) gets the eigenvectors as
- * columns, in the same order.  sweeps <= 0 means the default (12).  M <= 1024.  (The eigenvectors of W itself,
+ * columns, in the same order.  sweeps (Jacobi): <= 0 means the default (12).  M <= 1024.  (The eigenvectors of W itself,
  * L_N^{1/2} J^T U Sigma^{-1}, are N x M and are not formed.)
  */
 int flare_spectral_eig(int32_t matrices, int32_t M, float *G, float *eigenvalues, float *U, int32_t sweeps,

@@ -165,6 +165,33 @@ int spectral_gram(const flare_desc_t *desc, int sms, const void *Q_lat, const vo
 }
 
 int spectral_eig(int32_t matrices, int32_t M, float *G, float *eigenvalues, float *U, int32_t sweeps, cudaStream_t stream) {
+    if (U == nullptr) {
+        // in registers while a thread's rows of a column fit (see the kernel), in shared memory while that holds M x M, else in G
+#define FLARE_EIG(CX) spectral_tridiag_reg_kernel<CX><<<(unsigned)matrices, EigReg<CX>::kThreads, 0, stream>>>(G, M)
+        if (M <= 192) {
+            switch ((M + 31) / 32) {
+                case 1: FLARE_EIG(32); break;
+                case 2: FLARE_EIG(64); break;
+                case 3: FLARE_EIG(96); break;
+                case 4: FLARE_EIG(128); break;
+                case 5: FLARE_EIG(160); break;
+                default: FLARE_EIG(192); break;
+            }
+#undef FLARE_EIG
+        } else if (eig_smem(M, true) + 256 <= 227 * 1024) {
+            static std::atomic<uint64_t> opt_in{0};
+            if (int rc = ensure_big_smem(spectral_tridiag_kernel<true>, opt_in, 227 * 1024 - 256)) return rc;
+            spectral_tridiag_kernel<true><<<(unsigned)matrices, eig_threads(M), eig_smem(M, true), stream>>>(G, M);
+        } else {
+            spectral_tridiag_kernel<false><<<(unsigned)matrices, eig_threads(M), eig_smem(M, false), stream>>>(G, M);
+        }
+        FLARE_CUDA(cudaGetLastError());
+        constexpr int per_block = kBisectThreads / kEigSectors;
+        spectral_bisect_kernel<<<dim3((unsigned)((M + per_block - 1) / per_block), (unsigned)matrices), kBisectThreads,
+                                 (sizeof(EigPair<double>) + sizeof(EigPair<float>)) * (size_t)M, stream>>>(G, eigenvalues, M);
+        FLARE_CUDA(cudaGetLastError());
+        return FLARE_OK;
+    }
     if (sweeps <= 0) sweeps = 12;
     const int pairs = ((M + 1) & ~1) / 2;
     const size_t shmem = sizeof(float) * (4 * (size_t)pairs + M);

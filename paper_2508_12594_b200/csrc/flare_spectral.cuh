@@ -17,7 +17,8 @@
 //                              bf16 factors nothing cancels and G is off by 4e-3 of its largest entries).
 //   spectral_gram_simt_kernel  everything else (float32 inputs, other shapes): CUDA cores, a 16 x 16 tile of G per block.
 //   spectral_gram_reduce_kernel sums the token splits and writes the symmetric G.
-//   spectral_jacobi_kernel     eigenvalues (and eigenvectors) of G by cyclic two-sided Jacobi rotations.
+//   spectral_jacobi_kernel     eigenvalues and eigenvectors of G by cyclic two-sided Jacobi rotations.
+//   spectral_tridiag_*kernel, spectral_bisect_kernel   eigenvalues alone: Householder tridiagonalisation, then bisection.
 #pragma once
 
 #include "flare_common.cuh"
@@ -382,6 +383,327 @@ spectral_jacobi_kernel(float *__restrict__ Gall, float *__restrict__ evals, floa
         for (int i = t; i < M * M; i += T) G[(size_t)(i / M) * M + rank[i % M]] = U[i];
         __syncthreads();
         for (int i = t; i < M * M; i += T) U[i] = G[i];
+    }
+}
+
+// Eigenvalues alone (no U): Householder reduction to tridiagonal form, then bisection on Sturm counts.  One block per
+// matrix.  4/3 M^3 multiply-adds in M - 2 dependent steps, against about eight sweeps of M - 1 dependent steps of Jacobi
+// rotations over global memory: M = 128, eight matrices: 9.8 ms (Jacobi) -> 0.21 ms.  Each step is bound by the latency
+// of its four barriers and two sums over a vector, not by arithmetic, so the matrix sits where it is reached fastest: in
+// registers up to M = 192 (spectral_tridiag_reg_kernel), else in shared memory (M <= 236) or in G's own storage.
+// Step k: v = the Householder vector of row k right of the diagonal (every warp forms the norm for itself, a lane its
+// columns lane + 32 t), p = beta A v by columns (A is symmetric; thread (column, group) walks the rows of its group),
+// w = p - (beta / 2) (p . v) v, A -= v w^T + w v^T.  Float32 like the rotations; worst error against float64 over random,
+// low-rank and graded matrices: 3e-7 of the norm (rotations: 4e-6 at M = 16, 5e-5 at 128).
+__host__ __device__ constexpr int eig_threads(int M) { return M > 256 ? 1024 : 512; }
+// columns walked side by side, and groups of rows
+__host__ __device__ constexpr int eig_cols(int M) { const int m = (M + 31) & ~31; return m < eig_threads(M) ? m : eig_threads(M); }
+__host__ __device__ constexpr int eig_groups(int M) { return eig_threads(M) / eig_cols(M); }
+// shared memory: v, w, diagonal, off-diagonal, partial sums, and the matrix if it lives there
+inline size_t eig_smem(int M, bool matrix) { return sizeof(float) * ((size_t)(4 + eig_groups(M)) * M + (matrix ? (size_t)M * M : 0)); }
+
+__device__ __forceinline__ float eig_warp_sum(float x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// Eigenvalues, descending, of symmetric tridiagonal matrices: diagonal d[M], then the M - 1 off-diagonal elements, at the
+// start of each M x M block of `tri`.  Polynomial Sturm sequence p_i = (d_i - x) p_{i-1} - e_i^2 p_{i-2} (no division;
+// brought back to exponent 0 every other step; the matrix is scaled to norm 1 first, and e^2 kept above a floor far below
+// the precision wanted, so that no two p in a row are zero).  A chain of M dependent steps per count, so the counts are
+// spread: 16 eigenvalues to a block of 128 threads.  One pass with every thread at a point of its own brackets all
+// eigenvalues to 2 / 128; then kEigSectors threads share an eigenvalue and cut its interval nine-fold per pass: four passes
+// in float32 (their counts are off by at most a few eps of the norm: the interval is widened by 2^-19 afterwards), four in
+// double down to 2^-31 of the norm.
+constexpr int kEigSectors = 8;
+__device__ __forceinline__ float pow2_to_unit(float big) {       // 2^-exponent(big)
+    return __uint_as_float((254u - (__float_as_uint(big) >> 23)) << 23);
+}
+__device__ __forceinline__ double pow2_to_unit(double big) {
+    return __hiloint2double((int)((2046u - ((unsigned)__double2hiint(big) >> 20)) << 20), 0);
+}
+__device__ __forceinline__ int sign_bit(float x) { return (int)(__float_as_uint(x) >> 31); }
+__device__ __forceinline__ int sign_bit(double x) { return (int)((unsigned)__double2hiint(x) >> 31); }
+template <typename F> struct EigPair { F d, e2; };
+template <typename F>
+__device__ __forceinline__ int sturm_count(const EigPair<F> *q, int M, F x) {
+    F pm = 1, pc = q[0].d - x;
+    int count = sign_bit(pc), i = 1;
+    auto step = [&](const EigPair<F> a) {
+        const F pn = (a.d - x) * pc - a.e2 * pm;
+        count += sign_bit(pn) ^ sign_bit(pc);
+        pm = pc;
+        pc = pn;
+    };
+    auto rescale = [&]() {
+        const F x0 = fabs(pc), x1 = fabs(pm), f = pow2_to_unit(x0 > x1 ? x0 : x1);
+        pc *= f;
+        pm *= f;
+    };
+#pragma unroll 2
+    for (; i + 1 < M; i += 2) {
+        step(q[i]);
+        step(q[i + 1]);
+        rescale();
+    }
+    if (i < M) step(q[i]);
+    return count;
+}
+constexpr int kBisectThreads = 128;
+static __global__ void __launch_bounds__(kBisectThreads)
+spectral_bisect_kernel(const float *__restrict__ tri, float *__restrict__ evals, int M) {
+    extern __shared__ double bis_sh[];
+    __shared__ short counts[kBisectThreads];
+    constexpr int TH = kBisectThreads;
+    EigPair<double> *qd = reinterpret_cast<EigPair<double> *>(bis_sh);
+    EigPair<float> *qf = reinterpret_cast<EigPair<float> *>(qd + M);
+    const float *d = tri + (size_t)blockIdx.y * M * M, *e = d + M;
+    const int t = threadIdx.x, lane = t & 31;
+    float top = 0.f;                                            // Gershgorin, by every warp for itself
+    for (int i = lane; i < M; i += 32) top = fmaxf(top, fabsf(d[i]) + (i + 1 < M ? fabsf(e[i]) : 0.f) + (i > 0 ? fabsf(e[i - 1]) : 0.f));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    int ex = 0;
+    frexpf(top, &ex);
+    const double scale = top > 0.f ? ldexp(1.0, -ex) : 1.0;
+    for (int i = t; i < M; i += TH) {
+        const double di = d[i] * scale, ei = i > 0 ? e[i - 1] * scale : 0.0;
+        qd[i] = {di, fmax(ei * ei, 1e-40)};
+        qf[i] = {(float)di, fmaxf((float)(ei * ei), 1e-16f)};
+    }
+    __syncthreads();
+    counts[t] = (short)sturm_count<float>(qf, M, -1.f + 2.f * (float)(t + 1) / (float)(TH + 1));
+    __syncthreads();
+    const int sub = t % kEigSectors;
+    const int r = blockIdx.x * (TH / kEigSectors) + t / kEigSectors;   // eigenvalue number r, descending: M - 1 - r others lie below it
+    const int below = M - 1 - (r < M ? r : M - 1);
+    int n0 = 0, n1 = TH;                                        // points with at most `below` eigenvalues under them: [0, n0) yes, [n1, TH) no
+    while (n0 < n1) {
+        const int mid = (n0 + n1) >> 1;
+        if (counts[mid] <= below) n0 = mid + 1;
+        else n1 = mid;
+    }
+    double lo = -1.0 + 2.0 * n0 / (TH + 1) - 1.9e-6, hi = -1.0 + 2.0 * (n0 + 1) / (TH + 1) + 1.9e-6;
+    for (int pass = 0; pass < 8; ++pass) {
+        const double step = (hi - lo) * (1.0 / (kEigSectors + 1)), base = lo, x = base + step * (sub + 1);
+        const int count = pass < 4 ? sturm_count<float>(qf, M, (float)x) : sturm_count<double>(qd, M, x);
+        const unsigned left = (__ballot_sync(0xffffffffu, count <= below) >> (lane & ~(kEigSectors - 1))) & ((1u << kEigSectors) - 1);
+        const int n = __popc(left);
+        lo = base + step * n;
+        if (n < kEigSectors) hi = base + step * (n + 1);
+        if (pass == 3) { lo -= 1.9e-6; hi += 1.9e-6; }
+    }
+    if (r < M && sub == 0) evals[(size_t)blockIdx.y * M + r] = top > 0.f ? (float)(0.5 * (lo + hi) / scale) : 0.f;
+}
+
+// Largest magnitude over the block as a power of two to scale by, so that squares of the entries neither overflow nor
+// vanish: returns 2^-e with e the exponent of the largest (1 for a zero or non-finite matrix).  All threads call it.
+__device__ __forceinline__ float eig_block_scale(float mx, float *sh32) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) sh32[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    mx = 0.f;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) mx = fmaxf(mx, sh32[i]);
+    __syncthreads();
+    int e = 0;
+    if (!(mx > 0.f) || !(mx <= 3.0e38f)) return 1.f;
+    frexpf(mx, &e);
+    return ldexpf(1.f, e > 126 ? -126 : -e);
+}
+
+// The matrix in registers: NG groups of CX threads, thread (g, j) holds rows g, g + NG, ... of column j.  Vectors that are
+// read by rows are stored group-major (row g + NG r at g * R + r), so that four rows come with one load.
+template <int CX> struct EigReg {
+    static constexpr int NG = CX <= 64 ? 8 : 4, R = (CX / NG + 3) & ~3, kThreads = CX * NG;
+};
+template <int CX>
+__global__ void __launch_bounds__(EigReg<CX>::kThreads)
+spectral_tridiag_reg_kernel(float *__restrict__ Gall, int M) {
+    constexpr int NG = EigReg<CX>::NG, R = EigReg<CX>::R, CW = CX / 32, TH = EigReg<CX>::kThreads;
+    __shared__ __align__(16) float sx[NG * R], sv[NG * R], sw[NG * R];   // column k as it is, v, w
+    __shared__ float part[NG][CX], diag[CX], off[CX], red[32];
+    const int t = threadIdx.x, lane = t & 31, j = t % CX, g = t / CX;
+    float *G = Gall + (size_t)blockIdx.x * M * M;
+    float A[R], mx = 0.f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int i = g + NG * r;
+        A[r] = (j < M && i < M) ? G[(size_t)i * M + j] : 0.f;
+        mx = fmaxf(mx, fabsf(A[r]));
+    }
+    const float scale = eig_block_scale(mx, red);
+#pragma unroll
+    for (int r = 0; r < R; ++r) A[r] *= scale;
+    auto slot = [](int i) { return (i % NG) * R + i / NG; };    // where row i of a vector sits
+    auto dump = [&](int c) {                                    // column c of A to sx
+        if (j == c) {
+#pragma unroll
+            for (int r = 0; r < R; r += 4) *reinterpret_cast<float4 *>(sx + g * R + r) = make_float4(A[r], A[r + 1], A[r + 2], A[r + 3]);
+        }
+    };
+    for (int i = t; i < NG * R; i += TH) sv[i] = sw[i] = 0.f;   // (rows beyond M stay zero)
+    dump(0);
+    __syncthreads();
+    for (int k = 0; k + 2 < M; ++k) {
+        float vl[CW], s = 0.f;                                  // this lane's elements of v (every warp has them all)
+#pragma unroll
+        for (int c = 0; c < CW; ++c) {
+            const int i = lane + 32 * c;
+            vl[c] = i > k ? sx[slot(i)] : 0.f;
+            s = i > k + 1 ? fmaf(vl[c], vl[c], s) : s;
+        }
+        s = eig_warp_sum(s);
+        const float x0 = sx[slot(k + 1)];
+        const float norm = sqrtf(fmaf(x0, x0, s)), alpha = x0 > 0.f ? -norm : norm;
+        const float v0 = x0 - alpha, beta = s > 0.f ? 2.f / fmaf(v0, v0, s) : 0.f;   // nothing to annihilate: beta = 0, nothing changes
+#pragma unroll
+        for (int c = 0; c < CW; ++c)
+            if (lane + 32 * c == k + 1) vl[c] = v0;
+        if (t < 32) {
+#pragma unroll
+            for (int c = 0; c < CW; ++c) sv[slot(lane + 32 * c)] = vl[c];
+            if (t == 0) {
+                diag[k] = sx[slot(k)];
+                off[k] = s > 0.f ? alpha : x0;
+            }
+        }
+        __syncthreads();
+        float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
+        const float4 *v4 = reinterpret_cast<const float4 *>(sv + g * R), *w4 = reinterpret_cast<const float4 *>(sw + g * R);
+#pragma unroll
+        for (int r = 0; r < R; r += 4) {
+            if (g + NG * (r + 3) <= k) continue;                // these rows are done (uniform over the warp)
+            const float4 v = v4[r / 4];
+            p0 = fmaf(A[r], v.x, p0);
+            p1 = fmaf(A[r + 1], v.y, p1);
+            p2 = fmaf(A[r + 2], v.z, p2);
+            p3 = fmaf(A[r + 3], v.w, p3);
+        }
+        part[g][j] = (p0 + p1) + (p2 + p3);
+        __syncthreads();
+        float pv = 0.f;                                         // p . v, by every warp for itself
+#pragma unroll
+        for (int c = 0; c < CW; ++c) {
+            float p = 0.f;
+#pragma unroll
+            for (int q = 0; q < NG; ++q) p += part[q][lane + 32 * c];
+            pv = fmaf(p, vl[c], pv);
+        }
+        pv = eig_warp_sum(pv);
+        const float half = 0.5f * beta * (beta * pv);
+        float pj = 0.f;
+#pragma unroll
+        for (int q = 0; q < NG; ++q) pj += part[q][j];
+        const float vj = sv[slot(j)];                           // (zero up to k and beyond M)
+        const float wj = j > k ? fmaf(beta, pj, -half * vj) : 0.f;
+        if (g == 0) sw[slot(j)] = wj;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < R; r += 4) {
+            if (g + NG * (r + 3) <= k) continue;
+            const float4 v = v4[r / 4], w = w4[r / 4];
+            A[r] = fmaf(-v.x, wj, fmaf(-w.x, vj, A[r]));
+            A[r + 1] = fmaf(-v.y, wj, fmaf(-w.y, vj, A[r + 1]));
+            A[r + 2] = fmaf(-v.z, wj, fmaf(-w.z, vj, A[r + 2]));
+            A[r + 3] = fmaf(-v.w, wj, fmaf(-w.w, vj, A[r + 3]));
+        }
+        dump(k + 1);
+        __syncthreads();
+    }
+    if (M >= 2) {                                               // the last 2 x 2 block: column M - 2 is in sx
+        if (t == 0) {
+            diag[M - 2] = sx[slot(M - 2)];
+            off[M - 2] = sx[slot(M - 1)];
+        }
+        __syncthreads();
+        dump(M - 1);
+        __syncthreads();
+    }
+    if (t == 0) diag[M - 1] = sx[slot(M - 1)];
+    __syncthreads();
+    for (int i = t; i < M; i += TH) {                           // the result takes the place of the matrix
+        G[i] = diag[i] / scale;
+        if (i + 1 < M) G[M + i] = off[i] / scale;
+    }
+}
+
+// The matrix in shared memory (kShared) or where it is (global memory, overwritten).
+template <bool kShared>
+__global__ void __launch_bounds__(1024)
+spectral_tridiag_kernel(float *__restrict__ Gall, int M) {
+    extern __shared__ float eig_sh[];
+    const int t = threadIdx.x, TH = blockDim.x, lane = t & 31;
+    const int CX = eig_cols(M), NG = eig_groups(M);
+    float *dg = eig_sh, *ee = dg + M, *v = ee + M, *w = v + M, *part = w + M;   // part [NG][M]
+    float *G = Gall + (size_t)blockIdx.x * M * M;
+    float *A = kShared ? part + (size_t)NG * M : G;
+    __shared__ float red[32];
+    float mx = 0.f;
+    for (int i = t; i < M * M; i += TH) mx = fmaxf(mx, fabsf(G[i]));
+    const float scale = eig_block_scale(mx, red);
+    for (int i = t; i < M * M; i += TH) A[i] = G[i] * scale;
+    __syncthreads();
+    const int cx = t % CX, g = t / CX;
+    for (int k = 0; k + 2 < M; ++k) {
+        const float *row = A + (size_t)k * M;
+        float s = 0.f;
+        for (int j = k + 2 + lane; j < M; j += 32) s = fmaf(row[j], row[j], s);
+        s = eig_warp_sum(s);
+        const float x0 = row[k + 1];
+        const float norm = sqrtf(fmaf(x0, x0, s)), alpha = x0 > 0.f ? -norm : norm;
+        const float v0 = x0 - alpha, beta = s > 0.f ? 2.f / fmaf(v0, v0, s) : 0.f;
+        if (t == 0) { dg[k] = row[k]; ee[k] = s > 0.f ? alpha : x0; }
+        for (int j = k + 1 + t; j < M; j += TH) v[j] = j == k + 1 ? v0 : row[j];
+        __syncthreads();
+        if (g < NG)
+            for (int j = cx; j < M; j += CX)
+                if (j > k) {
+                    float p[4] = {0.f, 0.f, 0.f, 0.f};
+                    int i = k + 1 + g;
+                    for (; i + 3 * NG < M; i += 4 * NG)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) p[q] = fmaf(A[(size_t)(i + q * NG) * M + j], v[i + q * NG], p[q]);
+                    for (; i < M; i += NG) p[0] = fmaf(A[(size_t)i * M + j], v[i], p[0]);
+                    part[(size_t)g * M + j] = (p[0] + p[1]) + (p[2] + p[3]);
+                }
+        __syncthreads();
+        float pv = 0.f;
+        for (int j = k + 1 + lane; j < M; j += 32) {
+            float p = 0.f;
+            for (int q = 0; q < NG; ++q) p += part[(size_t)q * M + j];
+            pv = fmaf(p, v[j], pv);
+        }
+        pv = eig_warp_sum(pv);
+        const float half = 0.5f * beta * (beta * pv);
+        for (int j = k + 1 + t; j < M; j += TH) {
+            float p = 0.f;
+            for (int q = 0; q < NG; ++q) p += part[(size_t)q * M + j];
+            w[j] = fmaf(beta, p, -half * v[j]);
+        }
+        __syncthreads();
+        if (g < NG)
+            for (int j = cx; j < M; j += CX)
+                if (j > k) {
+                    const float vj = v[j], wj = w[j];
+#pragma unroll 4
+                    for (int i = k + 1 + g; i < M; i += NG)
+                        A[(size_t)i * M + j] = fmaf(-v[i], wj, fmaf(-w[i], vj, A[(size_t)i * M + j]));
+                }
+        __syncthreads();
+    }
+    if (t == 0) {
+        if (M >= 2) {
+            dg[M - 2] = A[(size_t)(M - 2) * M + M - 2];
+            ee[M - 2] = A[(size_t)(M - 2) * M + M - 1];
+        }
+        dg[M - 1] = A[(size_t)M * M - 1];
+    }
+    __syncthreads();
+    for (int i = t; i < M; i += TH) {                           // the result takes the place of the matrix
+        G[i] = dg[i] / scale;
+        if (i + 1 < M) G[M + i] = ee[i] / scale;
     }
 }
 

@@ -88,3 +88,25 @@ def test_spectral_error_paths():
     rc = flare.load().flare_spectral_eig(1, 4096, G.data_ptr(), G.data_ptr(), None, 0, None)
     assert rc == flare.ERR_INVALID_ARG
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("M", [1, 2, 3, 31, 33, 64, 65, 128, 129, 192, 193, 234, 236, 512])
+def test_eigenvalues_without_vectors(M):
+    """The call without eigenvectors (tridiagonal form, bisection) against numpy in float64: random symmetric matrices, one
+    that is already diagonal with repeated values, one of low rank, a zero one, a graded one with small entries; the sizes where the matrix moves from registers to shared
+    and from there to global memory."""
+    rng = np.random.default_rng(M)
+    X = rng.standard_normal((5, M, M))
+    G = (X + X.transpose(0, 2, 1)) / 2
+    G[1] = np.diag(np.round(rng.standard_normal(M)))
+    G[2] = X[2][:, : max(1, M // 8)] @ X[2][:, : max(1, M // 8)].T
+    G[3] = 0.0
+    grade = 2.0 ** (-20.0 * np.arange(M) / M)
+    G[4] = 1e-12 * (X[4] @ X[4].T) * grade[:, None] * grade[None, :]
+    G32 = torch.from_numpy(G).float()
+    ev = torch.full((5, M), float("nan"), device="cuda")
+    flare.flare_spectral_eig(G32.cuda(), ev)
+    want = np.linalg.eigvalsh(G32.double().numpy())[:, ::-1]
+    got = to_np64(ev)
+    for i in range(5):
+        assert np.abs(got[i] - want[i]).max() <= 1e-6 * np.abs(want[i]).max(), i
