@@ -2,6 +2,7 @@
 #include "flare_host.h"
 #include "flare_bwd.cuh"
 #include "flare_bwd_tc.cuh"
+#include "flare_reduce.cuh"
 
 namespace flare {
 namespace {
@@ -140,10 +141,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
         FLARE_CUDA(cudaGetLastError());
     }
     if (!skip_pass_a) {
-        bwd_dz_reduce_kernel<<<(unsigned)((rows * d->D + 255) / 256), 256, 0, st>>>(part, dZ, dz_parts, rows, d->D);
-        FLARE_CUDA(cudaGetLastError());
-        bwd_de_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(dZ, Z, de, rows, d->D);
-        FLARE_CUDA(cudaGetLastError());
+        FLARE_REDUCE(bwd_dz_reduce_kernel, rows, dz_parts, D, st, part, Z, dZ, de, dz_parts, rows);
     }
     bool tok_on_tc = false;
     if constexpr (std::is_same<T, __nv_bfloat16>::value && D <= 32) {
@@ -197,9 +195,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
             d->N, d->M, pb.LM, pb.chunk, d->scale);
         FLARE_CUDA(cudaGetLastError());
     }
-    bwd_dq_reduce_kernel<<<(unsigned)((long)d->H * d->M), kDqReduceThreads, 0, st>>>(part, dQ, dq_parts, d->B, d->H, d->M,
-                                                                                     d->D, d->scale);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_REDUCE(bwd_dq_reduce_kernel, (long)d->H * d->M, d->B * dq_parts, D, st, part, dQ, dq_parts, d->B, (long)d->H * d->M, d->scale);
     return FLARE_OK;
 }
 

@@ -1,5 +1,5 @@
-// Backward of the FLARE mixer on the CUDA cores (float32 arithmetic, any supported dtype and shape), and the
-// small reduction kernels every backward uses.  bfloat16 inputs take the tensor-core kernels instead (the dZ
+// Backward of the FLARE mixer on the CUDA cores (float32 arithmetic, any supported dtype and shape).
+// bfloat16 inputs take the tensor-core kernels instead (the dZ
 // form of the encode kernel for pass A; the dQ and token kernels of the tensor-core backward for pass B when
 // D <= 32); the formulas are the same.
 //
@@ -75,26 +75,6 @@ bwd_dz_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
             for (int d = 0; d < D; ++d) dst[d] = acc[d];
         }
     }
-}
-
-// dZ[row][d] = sum_p part[p][row][d], partials added in index order.  One thread per (row, d).
-static __global__ void __launch_bounds__(256)
-bwd_dz_reduce_kernel(const float *__restrict__ part, float *__restrict__ dZ, int P, long rows, int D) {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * D) return;
-    float s = 0.f;
-    for (int p = 0; p < P; ++p) s += part[(size_t)p * rows * D + idx];
-    dZ[idx] = s;
-}
-
-// de[row] = dZ_row . Z_row.  One thread per row.
-static __global__ void __launch_bounds__(256)
-bwd_de_kernel(const float *__restrict__ dZ, const float *__restrict__ Z, float *__restrict__ de, long rows, int D) {
-    const long row = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= rows) return;
-    float dot = 0.f;
-    for (int d = 0; d < D; ++d) dot = fmaf(dZ[row * D + d], Z[row * D + d], dot);
-    de[row] = dot;
 }
 
 // Pass B, token side: dK and dV.  One thread per token of head h; grid = (ceil(N/128), H, B).
@@ -276,30 +256,6 @@ bwd_dq_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__
 #pragma unroll
             for (int d = 0; d < D; ++d) dst[d] = acc[d];
         }
-    }
-}
-
-// dQ[h][m][d] = scale * sum_b sum_p part[p][(b,h,m)][d].  One block per (h, m): thread (slice, d) adds the terms
-// q = b * P + p with q = slice, slice + S, ... (S = 128 / D) in index order, thread (0, d) the S slice sums in index
-// order: a fixed order, and the B * P loads of a row are spread over the block.
-constexpr int kDqReduceThreads = 128;
-static __global__ void __launch_bounds__(kDqReduceThreads)
-bwd_dq_reduce_kernel(const float *__restrict__ part, float *__restrict__ dQ, int P, int B, int H, int M, int D,
-                     float scale) {
-    __shared__ float s_a[kDqReduceThreads];
-    const long hm = blockIdx.x;                                  // h * M + m
-    const int t = threadIdx.x, S = kDqReduceThreads / D, d = t % D, slice = t / D;
-    const long per_batch = (long)H * M, rows = (long)B * per_batch;
-    float s = 0.f;
-    for (int q = slice; q < B * P; q += S) {
-        const int b = q / P, p = q % P;
-        s += part[((size_t)p * rows + (size_t)b * per_batch + hm) * D + d];
-    }
-    s_a[t] = s;
-    __syncthreads();
-    if (slice == 0) {
-        for (int k = 1; k < S; ++k) s += s_a[k * D + d];
-        dQ[hm * D + d] = s * scale;
     }
 }
 

@@ -1,6 +1,6 @@
 // Encode on the tensor cores: launches of the kernel's forms, the merge of the partial results.
 #include "flare_host.h"
-#include "flare_simt.cuh"
+#include "flare_reduce.cuh"
 
 namespace flare {
 namespace {
@@ -72,9 +72,9 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
     float *pm = reinterpret_cast<float *>(base + w.part_m);
     float *pl = reinterpret_cast<float *>(base + w.part_l);
     float *pacc = reinterpret_cast<float *>(base + w.part_acc);
-    FLARE_CUDA(cudaMemsetAsync(base, 0, kHeaderBytes, st));
     int rc;
     if (use_tc(d)) {
+        FLARE_CUDA(cudaMemsetAsync(base, 0, kHeaderBytes, st));
         TcEncodePlan p = tc_encode_plan(d, di.sms);
         uint32_t *status = reinterpret_cast<uint32_t *>(base);
         // a caller that asks for lse_enc is saving Z for the backward: weights as two bf16 halves (see exp_chunk_hilo)
@@ -104,11 +104,8 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
         rc = encode_simt(d, p, Q, K, V, mask, pm, pl, pacc, st);
     }
     if (rc != FLARE_OK) return rc;
-    if (P > 8)   // many partials (small problems spread over all SMs): a block per row shares the loads
-        merge_kernel<<<(unsigned)rows, kMergeThreads, 0, st>>>(pm, pl, pacc, Z, lse_enc, P, rows, d->D);
-    else
-        merge_serial_kernel<<<(unsigned)((rows * d->D + 255) / 256), 256, 0, st>>>(pm, pl, pacc, Z, lse_enc, P, rows, d->D);
-    FLARE_CUDA(cudaGetLastError());
+    // (the CUDA-core kernels leave nothing in the header: the merge clears it)
+    FLARE_REDUCE(merge_kernel, rows, P, d->D, st, pm, pl, pacc, Z, lse_enc, P, rows, use_tc(d) ? nullptr : static_cast<uint32_t *>(ws));
     return FLARE_OK;
 }
 
