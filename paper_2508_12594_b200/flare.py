@@ -1,8 +1,9 @@
 """Python binding of libflare: the same entry points as ``include/flare.h``, argument marshalling only.
 
 Every step of the mixer runs in the library's CUDA kernels.  PyTorch is used for device memory and streams:
-the functions take torch tensors, check layout and dtype, and pass raw pointers.  There is no CPU fallback:
-if ``libflare.so`` is missing or cannot be loaded the first call raises.
+the functions take torch tensors, check layout and dtype, and pass raw pointers (in ``csrc/flare_binding.cpp``, an extension
+module, for the calls that enqueue work; through ctypes for the rest).  There is no CPU fallback: if ``libflare.so`` or
+the extension is missing or cannot be loaded the first call raises.
 """
 from __future__ import annotations
 
@@ -81,6 +82,20 @@ def load():
     return _lib
 
 
+_native = None
+
+
+def _bind():
+    """The marshalling extension, with the library's functions handed to it (once)."""
+    global _native
+    if _native is None:
+        lib = load()
+        from . import _binding
+        _binding.bind({name: ctypes.cast(getattr(lib, name), _vp).value for name in _SIGNATURES}, FlareError)
+        _native = _binding
+    return _native
+
+
 def exported_symbols():
     return list(_SIGNATURES)
 
@@ -147,13 +162,8 @@ def alloc_workspace(desc: FlareDesc, op: int, device="cuda") -> torch.Tensor:
 
 
 def flare_encode(desc, Q, K, V, key_mask, Z, lse_enc, workspace, stream=None):
-    dt = K.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    rc = load().flare_encode(ctypes.byref(desc), _ptr(Q, dt, (H, M, D)), _ptr(K, dt, (B, N, H, D)),
-                             _ptr(V, dt, (B, N, H, D)), _ptr(key_mask, torch.uint8, (B, N)),
-                             _ptr(Z, torch.float32, (B, H, M, D)), _ptr(lse_enc, torch.float32, (B, H, M)),
-                             _ptr(workspace, torch.uint8), workspace.numel(), _stream(stream))
-    _raise(rc, "flare_encode")
+    (_native or _bind()).encode(desc, Q, K, V, key_mask, Z, lse_enc, workspace, stream)
+
 
 
 STATIC_SCRATCH_BYTES = 8 << 20
@@ -163,23 +173,13 @@ def flare_encode_static_scratch(desc, Q, K, V, key_mask, Z, lse_enc, stream=None
     """flare_encode for callers that cannot allocate device memory: the partial results go to the library's
     built-in scratch array (STATIC_SCRATCH_BYTES, shared by all calls on the device, so calls must not overlap
     on the GPU).  Larger problems raise FlareError(ERR_WORKSPACE_TOO_SMALL)."""
-    dt = K.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    rc = load().flare_encode_static_scratch(ctypes.byref(desc), _ptr(Q, dt, (H, M, D)), _ptr(K, dt, (B, N, H, D)),
-                                            _ptr(V, dt, (B, N, H, D)), _ptr(key_mask, torch.uint8, (B, N)),
-                                            _ptr(Z, torch.float32, (B, H, M, D)),
-                                            _ptr(lse_enc, torch.float32, (B, H, M)), _stream(stream))
-    _raise(rc, "flare_encode_static_scratch")
+    (_native or _bind()).encode_static_scratch(desc, Q, K, V, key_mask, Z, lse_enc, stream)
+
 
 
 def flare_decode(desc, Q, K, Z, Y, lse_dec, workspace=None, stream=None):
-    dt = K.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    rc = load().flare_decode(ctypes.byref(desc), _ptr(Q, dt, (H, M, D)), _ptr(K, dt, (B, N, H, D)),
-                             _ptr(Z, torch.float32, (B, H, M, D)), _ptr(Y, dt, (B, N, H, D)),
-                             _ptr(lse_dec, torch.float32, (B, N, H)), _ptr(workspace, torch.uint8),
-                             0 if workspace is None else workspace.numel(), _stream(stream))
-    _raise(rc, "flare_decode")
+    (_native or _bind()).decode(desc, Q, K, Z, Y, lse_dec, workspace, stream)
+
 
 
 PATH_AUTO, PATH_EXACT, PATH_FAST = 0, 1, 2
@@ -191,40 +191,19 @@ def flare_set_path(path: int):
 
 
 def flare_forward(desc, Q, K, V, key_mask, Y, Z, lse_enc, lse_dec, workspace, stream=None):
-    dt = K.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    rc = load().flare_forward(ctypes.byref(desc), _ptr(Q, dt, (H, M, D)), _ptr(K, dt, (B, N, H, D)),
-                              _ptr(V, dt, (B, N, H, D)), _ptr(key_mask, torch.uint8, (B, N)),
-                              _ptr(Y, dt, (B, N, H, D)), _ptr(Z, torch.float32, (B, H, M, D)),
-                              _ptr(lse_enc, torch.float32, (B, H, M)), _ptr(lse_dec, torch.float32, (B, N, H)),
-                              _ptr(workspace, torch.uint8), workspace.numel(), _stream(stream))
-    _raise(rc, "flare_forward")
+    (_native or _bind()).forward(desc, Q, K, V, key_mask, Y, Z, lse_enc, lse_dec, workspace, stream)
+
 
 
 def flare_backward(desc, Q, K, V, key_mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, workspace, stream=None):
-    dt = K.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    tok = (B, N, H, D)
-    rc = load().flare_backward(ctypes.byref(desc), _ptr(Q, dt, (H, M, D)), _ptr(K, dt, tok), _ptr(V, dt, tok),
-                               _ptr(key_mask, torch.uint8, (B, N)), _ptr(Y, dt, tok), _ptr(dY, dt, tok),
-                               _ptr(Z, torch.float32, (B, H, M, D)), _ptr(lse_enc, torch.float32, (B, H, M)),
-                               _ptr(lse_dec, torch.float32, (B, N, H)), _ptr(dQ, torch.float32, (H, M, D)),
-                               _ptr(dK, dt, tok), _ptr(dV, dt, tok), _ptr(workspace, torch.uint8),
-                               workspace.numel(), _stream(stream))
-    _raise(rc, "flare_backward")
+    (_native or _bind()).backward(desc, Q, K, V, key_mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, workspace, stream)
+
 
 
 def flare_forward_host(desc, hQ, hK, hV, hmask, hY, dQ, dK, dV, dmask, dY, workspace, stream=None):
     """Host tensors in, host tensor out; the device tensors are the caller's staging buffers."""
-    dt = hK.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    tok = (B, N, H, D)
-    rc = load().flare_forward_host(ctypes.byref(desc), _ptr(hQ, dt, (H, M, D), cuda=False), _ptr(hK, dt, tok, cuda=False),
-                                   _ptr(hV, dt, tok, cuda=False), _ptr(hmask, torch.uint8, (B, N), cuda=False),
-                                   _ptr(hY, dt, tok, cuda=False), _ptr(dQ, dt, (H, M, D)), _ptr(dK, dt, tok),
-                                   _ptr(dV, dt, tok), _ptr(dmask, torch.uint8, (B, N)), _ptr(dY, dt, tok),
-                                   _ptr(workspace, torch.uint8), workspace.numel(), _stream(stream))
-    _raise(rc, "flare_forward_host")
+    (_native or _bind()).forward_host(desc, hQ, hK, hV, hmask, hY, dQ, dK, dV, dmask, dY, workspace, stream)
+
 
 
 def flare_check(workspace, stream=None):
@@ -246,29 +225,15 @@ def flare_variant_workspace_bytes(desc, op, shared_latents, separate) -> int:
 
 def flare_forward_variant(desc, shared_latents, Q_enc, Q_dec, K, V, key_mask, Y, Z, lse_enc, lse_dec, workspace, stream=None):
     """The mixer with one latent sequence for all heads (Q [M, D]) and / or separate decode queries (Q_dec, else None)."""
-    dt = K.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    qs = (M, D) if shared_latents else (H, M, D)
-    rc = load().flare_forward_variant(ctypes.byref(desc), int(shared_latents), _ptr(Q_enc, dt, qs), _ptr(Q_dec, dt, qs),
-                                      _ptr(K, dt, (B, N, H, D)), _ptr(V, dt, (B, N, H, D)), _ptr(key_mask, torch.uint8, (B, N)),
-                                      _ptr(Y, dt, (B, N, H, D)), _ptr(Z, torch.float32, (B, H, M, D)),
-                                      _ptr(lse_enc, torch.float32, (B, H, M)), _ptr(lse_dec, torch.float32, (B, N, H)),
-                                      _ptr(workspace, torch.uint8), workspace.numel(), _stream(stream))
-    _raise(rc, "flare_forward_variant")
+    (_native or _bind()).forward_variant(desc, shared_latents, Q_enc, Q_dec, K, V, key_mask, Y, Z, lse_enc, lse_dec, workspace, stream)
+
 
 
 def flare_backward_variant(desc, shared_latents, Q_enc, Q_dec, K, V, key_mask, Y, dY, Z, lse_enc, lse_dec, dQ_enc, dQ_dec, dK,
                            dV, workspace, stream=None):
-    dt = K.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    tok, qs = (B, N, H, D), ((M, D) if shared_latents else (H, M, D))
-    rc = load().flare_backward_variant(ctypes.byref(desc), int(shared_latents), _ptr(Q_enc, dt, qs), _ptr(Q_dec, dt, qs),
-                                       _ptr(K, dt, tok), _ptr(V, dt, tok), _ptr(key_mask, torch.uint8, (B, N)),
-                                       _ptr(Y, dt, tok), _ptr(dY, dt, tok), _ptr(Z, torch.float32, (B, H, M, D)),
-                                       _ptr(lse_enc, torch.float32, (B, H, M)), _ptr(lse_dec, torch.float32, (B, N, H)),
-                                       _ptr(dQ_enc, torch.float32, qs), _ptr(dQ_dec, torch.float32, qs), _ptr(dK, dt, tok),
-                                       _ptr(dV, dt, tok), _ptr(workspace, torch.uint8), workspace.numel(), _stream(stream))
-    _raise(rc, "flare_backward_variant")
+    (_native or _bind()).backward_variant(desc, shared_latents, Q_enc, Q_dec, K, V, key_mask, Y, dY, Z, lse_enc, lse_dec, dQ_enc,
+                                          dQ_dec, dK, dV, workspace, stream)
+
 
 
 def flare_microbench(which: int, iters: int = 20000, stream=None) -> float:
@@ -281,47 +246,27 @@ def flare_microbench(which: int, iters: int = 20000, stream=None) -> float:
 
 
 def flare_spectral_gram(desc, Q, K, lse_enc, lse_dec, G, workspace, stream=None):
-    dt = K.dtype
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    rc = load().flare_spectral_gram(ctypes.byref(desc), _ptr(Q, dt, (H, M, D)), _ptr(K, dt, (B, N, H, D)),
-                                    _ptr(lse_enc, torch.float32, (B, H, M)), _ptr(lse_dec, torch.float32, (B, N, H)),
-                                    _ptr(G, torch.float32, (B, H, M, M)), _ptr(workspace, torch.uint8), workspace.numel(),
-                                    _stream(stream))
-    _raise(rc, "flare_spectral_gram")
+    (_native or _bind()).spectral_gram(desc, Q, K, lse_enc, lse_dec, G, workspace, stream)
+
 
 
 def flare_spectral_eig(G, eigenvalues, U=None, sweeps=0, stream=None):
     """G [..., M, M] float32 (destroyed) -> eigenvalues [..., M] descending, U [..., M, M] eigenvectors as columns."""
-    M = G.shape[-1]
-    matrices = G.numel() // (M * M)
-    rc = load().flare_spectral_eig(matrices, M, _ptr(G, torch.float32), _ptr(eigenvalues, torch.float32),
-                                   _ptr(U, torch.float32), int(sweeps), _stream(stream))
-    _raise(rc, "flare_spectral_eig")
+    (_native or _bind()).spectral_eig(G, eigenvalues, U, int(sweeps), stream)
+
 
 
 def forward(Q, K, V, key_mask=None, scale=1.0, want_stats=False, stream=None):
     """Convenience: allocate outputs and workspace with torch, call flare_forward, return Y (and Z, lse's)."""
-    desc = make_desc(Q, K, scale)
-    B, H, N, M, D = desc.B, desc.H, desc.N, desc.M, desc.D
-    ws = alloc_workspace(desc, OP_FORWARD, K.device)
-    Y = torch.empty_like(K)
-    Z = torch.empty(B, H, M, D, dtype=torch.float32, device=K.device)
-    le = torch.empty(B, H, M, dtype=torch.float32, device=K.device)
-    ld = torch.empty(B, N, H, dtype=torch.float32, device=K.device)
-    flare_forward(desc, Q, K, V, key_mask, Y, Z, le, ld, ws, stream)
-    return (Y, Z, le, ld) if want_stats else Y
+    return (_native or _bind()).call_forward(Q, K, V, key_mask, scale, want_stats, stream)
+
 
 
 def forward_backward(Q, K, V, dY, key_mask=None, scale=1.0, stream=None, check=False):
     """Convenience: flare_forward (keeping Z and the log-sum-exp rows) then flare_backward.
     Returns (Y, dQ_lat [H,M,D] float32, dK, dV).  With check=True the stream is synchronised and a device-side
     wait that gave up raises."""
-    desc = make_desc(Q, K, scale)
-    Y, Z, le, ld = forward(Q, K, V, key_mask, scale, want_stats=True, stream=stream)
-    ws = alloc_workspace(desc, OP_BACKWARD, K.device)
-    dQ = torch.empty(desc.H, desc.M, desc.D, dtype=torch.float32, device=K.device)
-    dK, dV = torch.empty_like(K), torch.empty_like(V)
-    flare_backward(desc, Q, K, V, key_mask, Y, dY, Z, le, ld, dQ, dK, dV, ws, stream)
+    Y, dQ, dK, dV, ws = (_native or _bind()).call_forward_backward(Q, K, V, dY, key_mask, scale, stream)
     if check:
         (stream or torch.cuda.current_stream()).synchronize()
         flare_check(ws, stream)
