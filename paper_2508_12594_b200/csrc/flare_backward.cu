@@ -1,6 +1,5 @@
 // Backward: plans, workspace layout, launches of the tensor-core and CUDA-core kernels.
 #include "flare_host.h"
-#include "flare_bwd.cuh"
 #include "flare_bwd_tc.cuh"
 #include "flare_reduce.cuh"
 
@@ -136,9 +135,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
         }
     }
     if (!dz_on_tc) {
-        bwd_dz_simt_kernel<T, D><<<dim3(pa.splits, d->H, d->B), kBwdThreads, 0, st>>>(
-            (const T *)Q, (const T *)K, (const T *)dY, lse_dec, part, d->B, d->H, d->N, d->M, pa.LM, pa.chunk, d->scale);
-        FLARE_CUDA(cudaGetLastError());
+        if (const int rc = encode_dz_simt(d, pa, Q, K, dY, lse_dec, part, st)) return rc;
     }
     if (!skip_pass_a) {
         FLARE_REDUCE(bwd_dz_reduce_kernel, rows, dz_parts, D, st, part, Z, dZ, de, dz_parts, rows);
@@ -170,10 +167,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
         }
     }
     if (!tok_on_tc) {
-        bwd_token_simt_kernel<T, D><<<dim3((d->N + 127) / 128, d->H, d->B), 128, 0, st>>>(
-            (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, lse_enc, lse_dec, (T *)dK, (T *)dV, dd,
-            d->B, d->H, d->N, d->M, d->scale);
-        FLARE_CUDA(cudaGetLastError());
+        if (const int rc = bwd_token_simt(d, Q, K, V, mask, dY, Z, dZ, de, lse_enc, lse_dec, dK, dV, dd, st)) return rc;
     }
     int dq_parts = pb.P;
     bool dq_on_tc = false;
@@ -187,13 +181,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
         }
     }
     if (!dq_on_tc) {
-        const size_t dyn = sizeof(float) * 3 * (size_t)pb.LM * (D + 1);
-        static std::atomic<uint64_t> smem_opt_in{0};
-        if (int rc_attr = ensure_big_smem(bwd_dq_simt_kernel<T, D>, smem_opt_in, (int)(sizeof(float) * 3 * 64 * (D + 1)))) return rc_attr;
-        bwd_dq_simt_kernel<T, D><<<dim3(pb.splits, d->H, d->B), kBwdThreads, dyn, st>>>(
-            (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, dd, lse_enc, lse_dec, part, d->B, d->H,
-            d->N, d->M, pb.LM, pb.chunk, d->scale);
-        FLARE_CUDA(cudaGetLastError());
+        if (const int rc = bwd_dq_simt(d, pb, Q, K, V, mask, dY, Z, dZ, de, dd, lse_enc, lse_dec, part, st)) return rc;
     }
     FLARE_REDUCE(bwd_dq_reduce_kernel, (long)d->H * d->M, d->B * dq_parts, D, st, part, dQ, dq_parts, d->B, (long)d->H * d->M, d->scale);
     return FLARE_OK;

@@ -1,20 +1,22 @@
-// Backward of the FLARE mixer on the CUDA cores (float32 arithmetic, any supported dtype and shape).
-// bfloat16 inputs take the tensor-core kernels instead (the dZ
-// form of the encode kernel for pass A; the dQ and token kernels of the tensor-core backward for pass B when
-// D <= 32); the formulas are the same.
+// Backward of the FLARE mixer for float32 and float16 inputs (and the bfloat16 shapes the tensor-core kernels do not take);
+// bfloat16 inputs otherwise take the tensor-core kernels with the same formulas.
 //
 // The paper times a backward pass without writing it out; these kernels apply the chain rule to its encode and
 // decode equations (Section 3.2).  With S[m,n] = scale * q_m . k_n,
 //   W_dec[n,m] = exp(S[m,n] - lse_dec[n]),   W_enc[m,n] = valid(n) ? exp(S[m,n] - lse_enc[m]) : 0,
 // both softmax matrices are recomputed from the saved log-sum-exp rows, one score at a time:
-//   pass A   dZ[m]  = sum_n W_dec[n,m] dY_n                      (reduction over tokens; split over N)
+//   pass A   dZ[m]  = sum_n W_dec[n,m] dY_n                      (the dZ form of encode_simt_kernel; split over N)
 //   pass B   dd[n]  = dY_n . Y_n = sum_m W_dec[n,m] (dY_n . Z_m),   de[m] = dZ_m . Z_m
 //            dS[m,n] = W_dec[n,m] (dY_n . Z_m - dd[n]) + W_enc[m,n] (dZ_m . V_n - de[m])
-//            dV_n   = sum_m W_enc[m,n] dZ_m        dK_n = scale * sum_m dS[m,n] q_m       (one thread per token)
-//            dQ_m   = scale * sum_b sum_n dS[m,n] k_n                                     (split over N, then summed)
-// dd[n] is formed from the float32 dot products dY_n . Z_m rather than from the stored Y: Y has been rounded to
+//            dV_n   = sum_m W_enc[m,n] dZ_m        dK_n = scale * sum_m dS[m,n] q_m       (rows are tokens)
+//            dQ_m   = scale * sum_b sum_n dS[m,n] k_n                                     (rows are latents; split over N, then summed)
+// dd[n] is formed from the dot products dY_n . Z_m rather than from the stored Y: Y has been rounded to
 // the output type, and where the rows Z_m that a token mixes are nearly equal that rounding would dominate dS.
 // Reductions add their partial results in a fixed order, so the gradients are bitwise reproducible.
+//
+// The kernels have the shape of the forward ones: row operands as A fragments in registers, column operands in
+// shared memory, all three products of a pair (q.k, dY.Z, dZ.V) on the double-precision MMA, which bounds them: 2 D double
+// multiply-adds per pair in the first sweep over the latents and 3 D in the second and in the dQ pass.
 #pragma once
 
 #include "flare_common.cuh"
@@ -22,241 +24,262 @@
 
 namespace flare {
 
-constexpr int kBwdTileN = 32;   // tokens staged in shared memory per step of the latent-parallel kernels
-constexpr int kBwdLatents = 32; // latents staged in shared memory per step of the token-parallel kernel
+// Row blocks of 8 per warp: three operands of a row and its accumulators are in registers.
+template <int D> struct BwdSimtGeom {
+    static constexpr int RB = D <= 16 ? 2 : 1;
+    // token side: as many warps as the registers of three operands and two accumulators leave room for
+    static constexpr int kTokThreads = D <= 32 ? 384 : 256, kTokRows = kTokThreads / 32 * 8 * RB;
+};
 
-// Pass A.  grid = (splits, H, B); block = LM latents x G token groups (as in the encode kernel).  Partial
-// number split*G + g of latent row (b,h,m) goes to part[(split*G + g) * rows + row][D].
+// Pass B, token side.  Rows are tokens (8 RB per warp, the block's warps side by side).  grid = (ceil(N / kTokRows), H, B).
 template <typename T, int D>
-__global__ void __launch_bounds__(kBwdThreads)
-bwd_dz_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ dY,
-                   const float *__restrict__ lse_dec, float *__restrict__ part, int B, int H, int N, int M, int LM,
-                   int chunk, float scale) {
-    __shared__ float sK[kBwdTileN][D];
-    __shared__ float sG[kBwdTileN][D];
-    __shared__ float sL[kBwdTileN];
-    const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-    const int G = kBwdThreads / LM;
-    const int lm = threadIdx.x % LM, g = threadIdx.x / LM;
-    const int n0 = split * chunk, n1 = min(N, n0 + chunk);
-    const long rows = (long)B * H * M;
-    for (int mbase = 0; mbase < M; mbase += LM) {
-        const int m = mbase + lm;
-        const bool live = m < M;
-        float q[D], acc[D];
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-            q[d] = live ? to_f32(Q[((size_t)h * M + m) * D + d]) * scale : 0.f;
-            acc[d] = 0.f;
-        }
-        for (int t0 = n0; t0 < n1; t0 += kBwdTileN) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < kBwdTileN * D; i += kBwdThreads) {
-                const int j = i / D, d = i % D, n = t0 + j;
-                const bool in = n < n1;
-                const size_t off = (((size_t)b * N + (in ? n : 0)) * H + h) * D + d;
-                sK[j][d] = in ? to_f32(K[off]) : 0.f;
-                sG[j][d] = in ? to_f32(dY[off]) : 0.f;
-                if (d == 0) sL[j] = in ? lse_dec[((size_t)b * N + n) * H + h] : INFINITY;  // weight 0 past the end
-            }
-            __syncthreads();
-            if (live) {
-                for (int j = g; j < kBwdTileN; j += G) {
-                    const float w = expf(score_dot<T, D>(q, sK[j]) - sL[j]);
-#pragma unroll
-                    for (int d = 0; d < D; ++d) acc[d] = fmaf(w, sG[j][d], acc[d]);
-                }
-            }
-        }
-        if (live) {
-            const size_t row = ((size_t)b * H + h) * M + m;
-            float *dst = part + ((size_t)(split * G + g) * rows + row) * D;
-#pragma unroll
-            for (int d = 0; d < D; ++d) dst[d] = acc[d];
-        }
-    }
-}
-
-// Pass B, token side: dK and dV.  One thread per token of head h; grid = (ceil(N/128), H, B).
-template <typename T, int D>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(BwdSimtGeom<D>::kTokThreads, 1)
 bwd_token_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
                       const uint8_t *__restrict__ key_mask, const T *__restrict__ dY, const float *__restrict__ Z,
                       const float *__restrict__ dZ, const float *__restrict__ de, const float *__restrict__ lse_enc,
                       const float *__restrict__ lse_dec, T *__restrict__ dK, T *__restrict__ dV,
                       float *__restrict__ dd_out, int B, int H, int N, int M, float scale) {
-    __shared__ float sQ[kBwdLatents][D];
-    __shared__ float sZ[kBwdLatents][D];
-    __shared__ float sDZ[kBwdLatents][D];
-    __shared__ float sLe[kBwdLatents], sDe[kBwdLatents];
-    const int h = blockIdx.y, b = blockIdx.z;
-    const int n = blockIdx.x * 128 + threadIdx.x;
-    const bool live = n < N;
-    const size_t tok = (((size_t)b * N + (live ? n : 0)) * H + h) * D;
-    float k[D], v[D], dy[D], dk[D], dv[D];
+    using SG = SimtGeom<D>;
+    constexpr int CT = SG::CT, RB = BwdSimtGeom<D>::RB, TH = BwdSimtGeom<D>::kTokThreads;
+    extern __shared__ __align__(16) unsigned char simt_smem[];
+    double *sQ = reinterpret_cast<double *>(simt_smem), *sZ = sQ + CT * SG::DK, *sDZ = sZ + CT * SG::DK;
+    float *fQ = reinterpret_cast<float *>(sDZ + CT * SG::DK), *fDZ = fQ + CT * SG::DV, *sLe = fDZ + CT * SG::DV, *sDe = sLe + CT;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = blockIdx.y, b = blockIdx.z;
+    const int r0 = (blockIdx.x * (TH / 32) + warp) * 8 * RB;
+    const size_t stride = (size_t)H * D, base = ((size_t)b * N * H + h) * D;
+    const T *Qh = Q + (size_t)h * M * D;
+    const size_t lat = ((size_t)b * H + h) * M;
+    double ak[RB][D / 4], ag[RB][D / 4];
+    load_rows<T, D, RB>(ak, K + base, stride, r0, N, (double)scale);
+    load_rows<T, D, RB>(ag, dY + base, stride, r0, N, 1.0);
+    float ld[RB], dd[RB];
 #pragma unroll
-    for (int d = 0; d < D; ++d) {
-        k[d] = live ? to_f32(K[tok + d]) : 0.f;
-        v[d] = live ? to_f32(V[tok + d]) : 0.f;
-        dy[d] = live ? to_f32(dY[tok + d]) : 0.f;
-        dk[d] = 0.f;
-        dv[d] = 0.f;
+    for (int rb = 0; rb < RB; ++rb) {
+        const int n = r0 + 8 * rb + (lane >> 2);
+        ld[rb] = n < N ? lse_dec[((size_t)b * N + n) * H + h] : INFINITY;
+        dd[rb] = 0.f;
     }
-    const bool valid = live && (key_mask == nullptr || key_mask[(size_t)b * N + n] != 0);
-    const float ld = live ? lse_dec[((size_t)b * N + n) * H + h] : 0.f;
+    unsigned char *raw = reinterpret_cast<unsigned char *>(sDe + CT);
+    TileFetch<T, D, TH> fq(raw);
+    TileFetch<float, D, TH> fz(raw + fq.kBytes), fdz(raw + fq.kBytes + fz.kBytes);
     // first sweep over the latents: dd = sum_m W_dec[n,m] (dY_n . Z_m)
-    float dd = 0.f;
-    for (int m0 = 0; m0 < M; m0 += kBwdLatents) {
-        const int mc = min(kBwdLatents, M - m0);
+    fq.load(Qh, D, M);
+    fz.load(Z + lat * D, D, M);
+    for (int m0 = 0; m0 < M; m0 += CT) {
+        fq.wait();
         __syncthreads();
-        for (int i = threadIdx.x; i < mc * D; i += 128) {
-            const int j = i / D, d = i % D;
-            sQ[j][d] = to_f32(Q[((size_t)h * M + m0 + j) * D + d]);
-            sZ[j][d] = Z[(((size_t)b * H + h) * M + m0 + j) * D + d];
-        }
+        fq.put_double(sQ);
+        fz.put_double(sZ);
         __syncthreads();
-        for (int j = 0; j < mc; ++j) {
-            const float wdec = expf(scale * score_dot<T, D>(k, sQ[j]) - ld);
-            float a = 0.f;
+        const int m1 = m0 + CT < M ? m0 + CT : 0;                   // the next tile; after the last one the second sweep's first
+        fq.load(Qh + (size_t)m1 * D, D, M - m1);
+        fz.load(Z + (lat + m1) * D, D, M - m1);
+        const int mc = min(CT, M - m0);
+        if (r0 < N)
+            for (int nb = 0; nb < (mc + 7) / 8; ++nb) {
+                double2 c[RB], a[RB];
+                mma_block<D, RB>(c, ak, sQ, nb);
+                mma_block<D, RB>(a, ag, sZ, nb);
+                const int col = nb * 8 + 2 * (lane & 3);            // (columns beyond M: Z is zero there)
 #pragma unroll
-            for (int d = 0; d < D; ++d) a = fmaf(dy[d], sZ[j][d], a);
-            dd = fmaf(wdec, a, dd);
-        }
+                for (int rb = 0; rb < RB; ++rb) {
+                    if (col < mc) dd[rb] = fmaf(expf((float)c[rb].x - ld[rb]), (float)a[rb].x, dd[rb]);
+                    if (col + 1 < mc) dd[rb] = fmaf(expf((float)c[rb].y - ld[rb]), (float)a[rb].y, dd[rb]);
+                }
+            }
     }
-    if (live) dd_out[((size_t)b * H + h) * N + n] = dd;
-    for (int m0 = 0; m0 < M; m0 += kBwdLatents) {
-        const int mc = min(kBwdLatents, M - m0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < mc * D; i += 128) {
-            const int j = i / D, d = i % D;
-            const size_t row = ((size_t)b * H + h) * M + m0 + j;
-            sQ[j][d] = to_f32(Q[((size_t)h * M + m0 + j) * D + d]);
-            sZ[j][d] = Z[row * D + d];
-            sDZ[j][d] = dZ[row * D + d];
-            if (d == 0) {
-                sLe[j] = lse_enc[row];
-                sDe[j] = de[row];
-            }
-        }
-        __syncthreads();
-        for (int j = 0; j < mc; ++j) {
-            const float s = scale * score_dot<T, D>(k, sQ[j]);
-            const float wdec = expf(s - ld);
-            const float wenc = (valid && sLe[j] != -INFINITY) ? expf(s - sLe[j]) : 0.f;
-            float a = 0.f, c = 0.f;
+    double av[RB][D / 4];
+    load_rows<T, D, RB>(av, V + base, stride, r0, N, 1.0);
+    bool valid[RB];
+    float2 dk[RB][D / 2], dv[RB][D / 2];
 #pragma unroll
-            for (int d = 0; d < D; ++d) {
-                a = fmaf(dy[d], sZ[j][d], a);
-                c = fmaf(sDZ[j][d], v[d], c);
-            }
-            const float ds = (wdec * (a - dd) + wenc * (c - sDe[j])) * scale;
+    for (int rb = 0; rb < RB; ++rb) {
+        const int n = r0 + 8 * rb + (lane >> 2);
+        dd[rb] = quad_sum(dd[rb]);
+        valid[rb] = n < N && (key_mask == nullptr || key_mask[(size_t)b * N + n] != 0);
+        if (n < N && (lane & 3) == 0) dd_out[((size_t)b * H + h) * N + n] = dd[rb];
 #pragma unroll
-            for (int d = 0; d < D; ++d) {
-                dv[d] = fmaf(wenc, sDZ[j][d], dv[d]);
-                dk[d] = fmaf(ds, sQ[j][d], dk[d]);
-            }
-        }
+        for (int d = 0; d < D / 2; ++d) dk[rb][d] = dv[rb][d] = make_float2(0.f, 0.f);
     }
-    if (live) {
+    // second sweep (its first tile of Q and Z is already on its way)
+    fdz.load(dZ + lat * D, D, M);
+    for (int m0 = 0; m0 < M; m0 += CT) {
+        const int mc = min(CT, M - m0);
+        fq.wait();
+        __syncthreads();
+        fq.put_double(sQ);
+        fq.put_float(fQ);
+        fz.put_double(sZ);
+        fdz.put_double(sDZ);
+        fdz.put_float(fDZ);
+        if (threadIdx.x < CT) {
+            const int m = m0 + threadIdx.x;
+            const float le = m < M ? lse_enc[lat + m] : -INFINITY;
+            sLe[threadIdx.x] = le == -INFINITY ? -INFINITY : -le;   // added to the scores: weight 0 for a latent without valid tokens
+            sDe[threadIdx.x] = m < M ? de[lat + m] : 0.f;
+        }
+        __syncthreads();
+        if (m0 + CT < M) {
+            fq.load(Qh + (size_t)(m0 + CT) * D, D, M - m0 - CT);
+            fz.load(Z + (lat + m0 + CT) * D, D, M - m0 - CT);
+            fdz.load(dZ + (lat + m0 + CT) * D, D, M - m0 - CT);
+        }
+        if (r0 < N)
+            for (int nb = 0; nb < (mc + 7) / 8; ++nb) {
+                double2 s[RB], a[RB], c[RB];
+                mma_block<D, RB>(s, ak, sQ, nb);
+                mma_block<D, RB>(a, ag, sZ, nb);
+                mma_block<D, RB>(c, av, sDZ, nb);
+                const int col = nb * 8 + 2 * (lane & 3);
+                const float2 le = *reinterpret_cast<const float2 *>(sLe + col), dem = *reinterpret_cast<const float2 *>(sDe + col);
 #pragma unroll
-        for (int d = 0; d < D; ++d) {
-            from_f32(dK[tok + d], dk[d]);
-            from_f32(dV[tok + d], dv[d]);
+                for (int e = 0; e < 2; ++e) {
+                    if (col + e >= mc) continue;
+                    float ds[RB], we[RB];
+#pragma unroll
+                    for (int rb = 0; rb < RB; ++rb) {
+                        const float sc = (float)(e ? s[rb].y : s[rb].x);
+                        const float wd = expf(sc - ld[rb]);
+                        we[rb] = valid[rb] ? expf(sc + (e ? le.y : le.x)) : 0.f;
+                        ds[rb] = (wd * ((float)(e ? a[rb].y : a[rb].x) - dd[rb]) +
+                                  we[rb] * ((float)(e ? c[rb].y : c[rb].x) - (e ? dem.y : dem.x))) * scale;
+                    }
+#pragma unroll
+                    for (int rb = 0; rb < RB; ++rb) {
+                        axpy2<D>(dk[rb], ds[rb], fQ + (col + e) * SG::DV);
+                        axpy2<D>(dv[rb], we[rb], fDZ + (col + e) * SG::DV);
+                    }
+                }
+            }
+    }
+#pragma unroll
+    for (int rb = 0; rb < RB; ++rb) {
+        const int n = r0 + 8 * rb + (lane >> 2);
+#pragma unroll
+        for (int d = 0; d < D / 2; ++d) {
+            dk[rb][d] = make_float2(quad_sum(dk[rb][d].x), quad_sum(dk[rb][d].y));
+            dv[rb][d] = make_float2(quad_sum(dv[rb][d].x), quad_sum(dv[rb][d].y));
+        }
+        if (n < N) {
+            write_quarter<T, D>(dK + base + (size_t)n * stride, dk[rb], 1.f);
+            write_quarter<T, D>(dV + base + (size_t)n * stride, dv[rb], 1.f);
         }
     }
 }
+template <typename T, int D> inline size_t bwd_token_simt_smem() {
+    using SG = SimtGeom<D>;
+    return sizeof(double) * 3 * SG::CT * SG::DK + sizeof(float) * (2 * SG::CT * SG::DV + 2 * SG::CT) + (sizeof(T) + 2 * sizeof(float)) * SG::CT * D;
+}
 
-// Pass B, latent side: partial dQ rows.  Same grid and thread map as pass A; q, z and dz of the block's latents
-// sit in shared memory (rows padded by one float so that lanes reading different rows hit different banks).
+// Pass B, latent side: partial dQ rows.  Rows are latents, columns tokens; grid and warps as in encode_simt_kernel.
 template <typename T, int D>
-__global__ void __launch_bounds__(kBwdThreads)
+__global__ void __launch_bounds__(kBwdThreads, D <= 32 ? 2 : 1)
 bwd_dq_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
                    const uint8_t *__restrict__ key_mask, const T *__restrict__ dY, const float *__restrict__ Z,
                    const float *__restrict__ dZ, const float *__restrict__ de, const float *__restrict__ dd,
                    const float *__restrict__ lse_enc, const float *__restrict__ lse_dec, float *__restrict__ part,
-                   int B, int H, int N, int M, int LM, int chunk, float scale) {
-    extern __shared__ float dyn[];
-    float(*sQ)[D + 1] = reinterpret_cast<float(*)[D + 1]>(dyn);
-    float(*sZ)[D + 1] = sQ + LM;
-    float(*sDZ)[D + 1] = sZ + LM;
-    __shared__ float sK[kBwdTileN][D];
-    __shared__ float sV[kBwdTileN][D];
-    __shared__ float sG[kBwdTileN][D];
-    __shared__ float sLd[kBwdTileN], sDd[kBwdTileN];
-    __shared__ uint8_t sValid[kBwdTileN];
-    const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-    const int G = kBwdThreads / LM;
-    const int lm = threadIdx.x % LM, g = threadIdx.x / LM;
+                   int B, int H, int N, int M, int WM, int mblocks, int chunk, float scale) {
+    using SG = SimtGeom<D>;
+    constexpr int CT = SG::CT, RB = BwdSimtGeom<D>::RB, RW = 8 * RB;
+    extern __shared__ __align__(16) unsigned char simt_smem[];
+    double *sK = reinterpret_cast<double *>(simt_smem), *sG = sK + CT * SG::DK, *sV = sG + CT * SG::DK;
+    float *fK = reinterpret_cast<float *>(sV + CT * SG::DK), *sLd = fK + CT * SG::DV, *sDd = sLd + CT, *sMask = sDd + CT;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int split = blockIdx.x, h = blockIdx.y / mblocks, mb = blockIdx.y % mblocks, b = blockIdx.z;
+    const int WT = kBwdThreads / 32 / WM, wm = warp % WM, wt = warp / WM;
+    const int rbase = mb * WM * RW, r0 = rbase + wm * RW;
     const int n0 = split * chunk, n1 = min(N, n0 + chunk);
-    const long rows = (long)B * H * M;
-    for (int mbase = 0; mbase < M; mbase += LM) {
-        const int m = mbase + lm;
-        const bool live = m < M;
-        const size_t row = ((size_t)b * H + h) * M + (live ? m : 0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < LM * D; i += kBwdThreads) {
-            const int j = i / D, d = i % D;
-            const bool in = mbase + j < M;
-            const size_t r = ((size_t)b * H + h) * M + (in ? mbase + j : 0);
-            sQ[j][d] = in ? to_f32(Q[((size_t)h * M + mbase + j) * D + d]) : 0.f;
-            sZ[j][d] = in ? Z[r * D + d] : 0.f;
-            sDZ[j][d] = in ? dZ[r * D + d] : 0.f;
-        }
-        const float le = live ? lse_enc[row] : -INFINITY;
-        const float dem = live ? de[row] : 0.f;
-        float acc[D];
+    const size_t stride = (size_t)H * D, base = ((size_t)b * N * H + h) * D;
+    const size_t lat = ((size_t)b * H + h) * M;
+    double aq[RB][D / 4], az[RB][D / 4], adz[RB][D / 4];
+    load_rows<T, D, RB>(aq, Q + (size_t)h * M * D, D, r0, M, (double)scale);
+    load_rows<float, D, RB>(az, Z + lat * D, D, r0, M, 1.0);
+    load_rows<float, D, RB>(adz, dZ + lat * D, D, r0, M, 1.0);
+    float nle[RB], dem[RB];
+    float2 acc[RB][D / 2];
 #pragma unroll
-        for (int d = 0; d < D; ++d) acc[d] = 0.f;
-        for (int t0 = n0; t0 < n1; t0 += kBwdTileN) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < kBwdTileN * D; i += kBwdThreads) {
-                const int j = i / D, d = i % D, n = t0 + j;
-                const bool in = n < n1;
-                const size_t off = (((size_t)b * N + (in ? n : 0)) * H + h) * D + d;
-                sK[j][d] = in ? to_f32(K[off]) : 0.f;
-                sV[j][d] = in ? to_f32(V[off]) : 0.f;
-                sG[j][d] = in ? to_f32(dY[off]) : 0.f;
-            }
-            if (threadIdx.x < kBwdTileN) {
-                const int j = threadIdx.x, n = t0 + j;
-                const bool in = n < n1;
-                sDd[j] = in ? dd[((size_t)b * H + h) * N + n] : 0.f;
-                sLd[j] = in ? lse_dec[((size_t)b * N + n) * H + h] : INFINITY;
-                sValid[j] = in && (key_mask == nullptr || key_mask[(size_t)b * N + n] != 0);
-            }
-            __syncthreads();
-            if (live) {
-                for (int j = g; j < kBwdTileN; j += G) {
-                    float s0 = 0.f, a = 0.f, c = 0.f;
-                    if constexpr (!std::is_same<T, __nv_bfloat16>::value) {   // float32 and float16 inputs
-                        double sd = 0.0;
+    for (int rb = 0; rb < RB; ++rb) {
+        const int m = r0 + 8 * rb + (lane >> 2);
+        const float le = m < M ? lse_enc[lat + m] : -INFINITY;
+        nle[rb] = le == -INFINITY ? -INFINITY : -le;
+        dem[rb] = m < M ? de[lat + m] : 0.f;
 #pragma unroll
-                        for (int d = 0; d < D; ++d) sd = fma((double)sQ[lm][d], (double)sK[j][d], sd);
-                        s0 = (float)sd;
-                    } else {
-#pragma unroll
-                        for (int d = 0; d < D; ++d) s0 = fmaf(sQ[lm][d], sK[j][d], s0);
-                    }
-#pragma unroll
-                    for (int d = 0; d < D; ++d) {
-                        a = fmaf(sG[j][d], sZ[lm][d], a);
-                        c = fmaf(sDZ[lm][d], sV[j][d], c);
-                    }
-                    const float s = s0 * scale;
-                    const float wdec = expf(s - sLd[j]);
-                    const float wenc = (sValid[j] && le != -INFINITY) ? expf(s - le) : 0.f;
-                    const float ds = wdec * (a - sDd[j]) + wenc * (c - dem);
-#pragma unroll
-                    for (int d = 0; d < D; ++d) acc[d] = fmaf(ds, sK[j][d], acc[d]);
-                }
-            }
-        }
-        if (live) {
-            float *dst = part + ((size_t)(split * G + g) * rows + row) * D;
-#pragma unroll
-            for (int d = 0; d < D; ++d) dst[d] = acc[d];
-        }
+        for (int d = 0; d < D / 2; ++d) acc[rb][d] = make_float2(0.f, 0.f);
     }
+    using Fetch = TileFetch<T, D, kBwdThreads>;
+    unsigned char *raw = reinterpret_cast<unsigned char *>(sMask + CT);
+    Fetch fk(raw), fg(raw + Fetch::kBytes), fv(raw + 2 * Fetch::kBytes);
+    auto fetch = [&](int t0) {
+        const size_t at = base + (size_t)t0 * stride;
+        fk.load(K + at, stride, n1 - t0);
+        fg.load(dY + at, stride, n1 - t0);
+        fv.load(V + at, stride, n1 - t0);
+    };
+    fetch(n0);
+    for (int t0 = n0; t0 < n1; t0 += CT) {
+        Fetch::wait();
+        __syncthreads();
+        fk.put_double(sK);
+        fk.put_float(fK);
+        fg.put_double(sG);
+        fv.put_double(sV);
+        if (threadIdx.x < CT) {
+            const int n = t0 + threadIdx.x;
+            const bool in = n < n1;
+            sLd[threadIdx.x] = in ? -lse_dec[((size_t)b * N + n) * H + h] : -INFINITY;
+            sDd[threadIdx.x] = in ? dd[((size_t)b * H + h) * N + n] : 0.f;
+            sMask[threadIdx.x] = in && (key_mask == nullptr || key_mask[(size_t)b * N + n] != 0) ? 0.f : -INFINITY;
+        }
+        __syncthreads();
+        if (t0 + CT < n1) fetch(t0 + CT);
+        const int blocks = (min(CT, n1 - t0) + 7) / 8;
+        if (r0 < M)
+            for (int nb = wt; nb < blocks; nb += WT) {
+                double2 s[RB], a[RB], c[RB];
+                mma_block<D, RB>(s, aq, sK, nb);
+                mma_block<D, RB>(a, az, sG, nb);
+                mma_block<D, RB>(c, adz, sV, nb);
+                const int col = nb * 8 + 2 * (lane & 3);
+                const float2 nld = *reinterpret_cast<const float2 *>(sLd + col), ddn = *reinterpret_cast<const float2 *>(sDd + col);
+                const float2 msk = *reinterpret_cast<const float2 *>(sMask + col);
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+#pragma unroll
+                    for (int rb = 0; rb < RB; ++rb) {
+                        const float sc = (float)(e ? s[rb].y : s[rb].x);
+                        const float wd = expf(sc + (e ? nld.y : nld.x)), we = expf((sc + nle[rb]) + (e ? msk.y : msk.x));
+                        const float ds = wd * ((float)(e ? a[rb].y : a[rb].x) - (e ? ddn.y : ddn.x)) +
+                                         we * ((float)(e ? c[rb].y : c[rb].x) - dem[rb]);
+                        axpy2<D>(acc[rb], ds, fK + (col + e) * SG::DV);
+                    }
+            }
+    }
+    __syncthreads();
+    // the shares of the columns meet
+    constexpr int ROW = D + 4;
+    float *sR = reinterpret_cast<float *>(simt_smem);
+    const int rows_here = WM * RW;
+#pragma unroll
+    for (int rb = 0; rb < RB; ++rb) {
+#pragma unroll
+        for (int d = 0; d < D / 2; ++d) acc[rb][d] = make_float2(quad_sum(acc[rb][d].x), quad_sum(acc[rb][d].y));
+        write_quarter<float, D>(sR + ((size_t)wt * rows_here + wm * RW + 8 * rb + (lane >> 2)) * ROW, acc[rb], 1.f);
+    }
+    __syncthreads();
+    const long rows = (long)B * H * M;
+    for (int i = threadIdx.x; i < rows_here * D; i += kBwdThreads) {
+        const int r = i / D, d = i % D, m = rbase + r;
+        if (m >= M) continue;
+        float z = 0.f;
+        for (int w = 0; w < WT; ++w) z += sR[((size_t)w * rows_here + r) * ROW + d];
+        part[((size_t)split * rows + lat + m) * D + d] = z;
+    }
+}
+template <typename T, int D> inline size_t bwd_dq_simt_smem() {
+    using SG = SimtGeom<D>;
+    const size_t tiles = sizeof(double) * 3 * SG::CT * SG::DK + sizeof(float) * (SG::CT * SG::DV + 3 * SG::CT) + 3 * sizeof(T) * SG::CT * D;
+    const size_t join = sizeof(float) * (kBwdThreads / 32) * 8 * BwdSimtGeom<D>::RB * (D + 4);
+    return tiles > join ? tiles : join;
 }
 
 }  // namespace flare

@@ -40,7 +40,6 @@ inline WorkspaceLayout make_layout(int P, long rows, int D, bool with_z) {
 
 // Shape of the CUDA-core kernels' blocks (their launch plans need it too).
 constexpr int kSimtThreads = 256;
-constexpr int kSimtTileN = 32;  // tokens staged in shared memory per step
 constexpr int kBwdThreads = 256;
 
 __device__ __forceinline__ float to_f32(float x) { return x; }

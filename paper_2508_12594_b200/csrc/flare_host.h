@@ -91,27 +91,32 @@ inline int check_desc(const flare_desc_t *d) {
     return FLARE_OK;
 }
 
-// Launch plan of the CUDA-core encode: LM latents x G token groups per block, `splits` blocks along N.
+// Launch plan of the CUDA-core kernels whose rows are latents (encode, dZ, dQ): blocks of WM groups of 8 RB latents, `splits`
+// blocks along N.
 struct SimtPlan {
-    int LM, G, splits, chunk, P;
+    int RB, WM, mblocks, splits, chunk, P;
 };
-
-inline SimtPlan simt_plan(const flare_desc_t *d, int sms) {
+inline int simt_row_blocks(int D) { return D <= 16 ? 4 : D == 32 ? 2 : 1; }   // of the forward kernels: 8 RB D values of a warp's accumulators
+inline SimtPlan simt_plan_for(const flare_desc_t *d, int sms, int RB) {
     SimtPlan p;
-    p.LM = 1;
-    while (p.LM < d->M && p.LM < kSimtThreads) p.LM *= 2;
-    p.G = kSimtThreads / p.LM;
-    long bh = (long)d->B * d->H;
-    long want = (4L * sms + bh - 1) / bh;                  // about four blocks per SM in total
-    long most = (d->N + 255) / 256;                        // at least 256 tokens per block
-    long s = want < most ? want : most;
+    p.RB = RB;
+    const int groups = (d->M + 8 * RB - 1) / (8 * RB), tile = d->D <= 32 ? 64 : 32;
+    p.WM = 1;
+    while (p.WM < groups && p.WM < kSimtThreads / 32) p.WM *= 2;
+    p.mblocks = (groups + p.WM - 1) / p.WM;
+    const long per = (long)d->B * d->H * p.mblocks;
+    long s = 2L * sms / per;                                    // two blocks per SM, in one wave
+    const long most = (d->N + tile - 1) / tile;
+    if (s > most) s = most;
     if (s < 1) s = 1;
     p.chunk = (int)((d->N + s - 1) / s);
-    p.chunk = (p.chunk + kSimtTileN - 1) / kSimtTileN * kSimtTileN;
+    p.chunk = (p.chunk + tile - 1) / tile * tile;
     p.splits = (d->N + p.chunk - 1) / p.chunk;
-    p.P = p.splits * p.G;
+    p.P = p.splits;
     return p;
 }
+// (up to 16 latents: single row blocks, so that fewer rows of the MMAs are empty)
+inline SimtPlan simt_plan(const flare_desc_t *d, int sms) { return simt_plan_for(d, sms, d->M <= 16 ? 1 : simt_row_blocks(d->D)); }
 
 // The tensor-core kernels take bfloat16 with D in {16, 32, 64} and a positive scale, and D = 8 or 4 as the narrow
 // forms of the D = 16 kernels: a token tile of 16 feature columns then spans two or four heads, so the tensor must
@@ -267,8 +272,8 @@ inline size_t decode_range_bytes(const flare_desc_t *d) {
     return align_up(sizeof(float) * decode_ranges(d) * rows * d->D) + align_up(sizeof(float) * decode_ranges(d) * rows);
 }
 
-// Launch plans of the CUDA-core backward: pass A (dZ) reuses the encode plan; the dQ pass keeps three latent
-// rows per thread in shared memory and therefore caps its latent block at 64.
+// Launch plans of the CUDA-core backward: pass A (dZ) reuses the encode plan; the dQ pass keeps three operands of a latent row
+// in registers and therefore takes fewer rows per warp.
 // Pass A (dZ) runs as the dZ form of the tensor-core encode kernel wherever that kernel runs.
 inline bool bwd_dz_on_tensor_cores(const flare_desc_t *d) { return use_tc(d); }
 
@@ -291,13 +296,7 @@ inline TcEncodePlan tc_dq_plan(const flare_desc_t *d, int sms) {
     return p;
 }
 
-inline SimtPlan bwd_dq_plan(const flare_desc_t *d, int sms) {
-    SimtPlan p = simt_plan(d, sms);
-    if (p.LM > 64) p.LM = 64;
-    p.G = kBwdThreads / p.LM;
-    p.P = p.splits * p.G;
-    return p;
-}
+inline SimtPlan bwd_dq_plan(const flare_desc_t *d, int sms) { return simt_plan_for(d, sms, d->D <= 16 ? 2 : 1); }
 
 struct BwdLayout {
     size_t part, dz, de, dd, kvacc, total;
@@ -330,7 +329,16 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
 // ---- what the translation units provide
 int encode_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask,
                 float *pm, float *pl, float *pacc, cudaStream_t st);
+// dZ form: lse_dec given, dY in place of V, partial sums of dZ to pacc
+int encode_dz_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *dY, const float *lse_dec,
+                   float *pacc, cudaStream_t st);
 int decode_simt(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st);
+int bwd_token_simt(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, const void *dY,
+                   const float *Z, const float *dZ, const float *de, const float *lse_enc, const float *lse_dec, void *dK, void *dV,
+                   float *dd, cudaStream_t st);
+int bwd_dq_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask,
+                const void *dY, const float *Z, const float *dZ, const float *de, const float *dd, const float *lse_enc,
+                const float *lse_dec, float *part, cudaStream_t st);
 int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
                 float *lse_enc, void *ws, cudaStream_t st);
 int encode_dz_tc(const flare_desc_t *d, const TcEncodePlan &tp, const void *Q, const void *K, const void *dY, float *part,

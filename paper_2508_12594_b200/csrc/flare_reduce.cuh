@@ -141,15 +141,13 @@ bwd_dz_reduce_kernel(const float *__restrict__ part, const float *__restrict__ Z
     for (int p = rm.slice; p < P; p += slices) s = f4_add(s, p4[(size_t)p * rows * L]);
     s = sum_slices<L>(s, slices);
     const float4 z = reinterpret_cast<const float4 *>(Z)[at];
-    // de in the order d = 0, 1, ... of the kernels that form dZ_m . V_n, from lane to lane: where a latent follows a single
-    // token the two cancel exactly
-    float dot = 0.f;
+    // de is summed in double, as the CUDA-core kernels sum dZ_m . V_n: where a latent follows a single token the two cancel
+    double dot = fma((double)s.w, (double)z.w, fma((double)s.z, (double)z.z, fma((double)s.y, (double)z.y, (double)s.x * (double)z.x)));
 #pragma unroll
-    for (int l = 0; l < L; ++l)
-        dot = __shfl_sync(0xffffffffu, fmaf(s.w, z.w, fmaf(s.z, z.z, fmaf(s.y, z.y, fmaf(s.x, z.x, dot)))), l, L);
+    for (int o = 1; o < L; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
     if (!live || rm.slice != 0) return;
     reinterpret_cast<float4 *>(dZ)[at] = s;
-    if (rm.lane == 0) de[rm.row] = dot;
+    if (rm.lane == 0) de[rm.row] = (float)dot;
 }
 
 // dQ[h][m] = scale * sum_b sum_p part[p][(b, h, m)]: the B * P terms of a row in index order per slice.

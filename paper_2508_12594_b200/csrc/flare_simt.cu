@@ -1,59 +1,126 @@
-// The CUDA-core forward kernels: float32 and float16 inputs, and the bfloat16 shapes the tensor-core kernels do not take.
+// Launches of the CUDA-core kernels: float32 and float16 inputs, and the bfloat16 shapes the tensor-core kernels do not take.
 #include "flare_host.h"
 #include "flare_simt.cuh"
+#include "flare_bwd.cuh"
 
 namespace flare {
 namespace {
 
-template <typename T>
-int launch_encode_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V,
-                       const uint8_t *mask, float *pm, float *pl, float *pacc, cudaStream_t st) {
-    dim3 grid(p.splits, d->H, d->B), block(kSimtThreads);
-#define FLARE_CASE(DD)                                                                                          \
-    case DD:                                                                                                    \
-        encode_simt_kernel<T, DD><<<grid, block, 0, st>>>((const T *)Q, (const T *)K, (const T *)V, mask, pm, pl, \
-                                                          pacc, d->B, d->H, d->N, d->M, p.LM, p.chunk, d->scale); \
-        break;
-    switch (d->D) {
-        FLARE_CASE(4) FLARE_CASE(8) FLARE_CASE(16) FLARE_CASE(32) FLARE_CASE(64)
-        default: return FLARE_ERR_UNSUPPORTED;
-    }
-#undef FLARE_CASE
+template <typename T, int D, int RB, bool kDz>
+int launch_encode(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask,
+                  const float *lse_dec, float *pm, float *pl, float *pacc, cudaStream_t st) {
+    const size_t smem = encode_simt_smem<T, D>(RB);
+    static std::atomic<uint64_t> opt_in{0};
+    if (smem > 48 * 1024)
+        if (int rc = ensure_big_smem(encode_simt_kernel<T, D, RB, kDz>, opt_in, (int)smem)) return rc;
+    encode_simt_kernel<T, D, RB, kDz><<<dim3(p.splits, d->H * p.mblocks, d->B), kSimtThreads, smem, st>>>(
+        (const T *)Q, (const T *)K, (const T *)V, mask, lse_dec, pm, pl, pacc, d->B, d->H, d->N, d->M, p.WM, p.mblocks, p.chunk, d->scale);
     FLARE_CUDA(cudaGetLastError());
     return FLARE_OK;
 }
+template <typename T, int D>
+struct Encode {
+    template <typename... A>
+    static int run(bool dz, const flare_desc_t *d, const SimtPlan &p, A... a) {
+        constexpr int RB = D <= 16 ? 4 : D == 32 ? 2 : 1;       // (simt_row_blocks)
+        if (p.RB == 1) return dz ? launch_encode<T, D, 1, true>(d, p, a...) : launch_encode<T, D, 1, false>(d, p, a...);
+        return dz ? launch_encode<T, D, RB, true>(d, p, a...) : launch_encode<T, D, RB, false>(d, p, a...);
+    }
+};
 
-template <typename T>
-int launch_decode_simt(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec,
-                       cudaStream_t st) {
-    dim3 grid((d->N + kDecodeSimtThreads - 1) / kDecodeSimtThreads, d->H, d->B), block(kDecodeSimtThreads);
-#define FLARE_CASE(DD)                                                                                            \
-    case DD:                                                                                                      \
-        decode_simt_kernel<T, DD><<<grid, block, 0, st>>>((const T *)Q, (const T *)K, Z, (T *)Y, lse_dec, d->B, d->H, \
-                                                          d->N, d->M, d->scale);                                  \
-        break;
-    switch (d->D) {
-        FLARE_CASE(4) FLARE_CASE(8) FLARE_CASE(16) FLARE_CASE(32) FLARE_CASE(64)
+template <typename T, int D>
+struct Decode {
+    template <int RB>
+    static int launch(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st) {
+        static_assert(sizeof(double) * 64 * 36 + sizeof(float) * 64 * 36 + 8 * 64 * 32 <= 48 * 1024, "no opt-in needed");
+        decode_simt_kernel<T, D, RB><<<dim3((d->N + 64 * RB - 1) / (64 * RB), d->H, d->B), kSimtThreads, decode_simt_smem<T, D>(), st>>>(
+            (const T *)Q, (const T *)K, Z, (T *)Y, lse_dec, d->B, d->H, d->N, d->M, d->scale);
+        FLARE_CUDA(cudaGetLastError());
+        return FLARE_OK;
+    }
+    static int run(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st) {
+        constexpr int RB = D <= 16 ? 4 : D == 32 ? 2 : 1;
+        // few tokens: smaller blocks of them, so that more SMs take part
+        if ((long)d->B * d->H * ((d->N + 64 * RB - 1) / (64 * RB)) < 2L * device_info().sms) return launch<1>(d, Q, K, Z, Y, lse_dec, st);
+        return launch<RB>(d, Q, K, Z, Y, lse_dec, st);
+    }
+};
+
+template <typename T, int D>
+struct Token {
+    static int run(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, const void *dY, const float *Z,
+                   const float *dZ, const float *de, const float *lse_enc, const float *lse_dec, void *dK, void *dV, float *dd, cudaStream_t st) {
+        constexpr int rows = BwdSimtGeom<D>::kTokRows;
+        static std::atomic<uint64_t> opt_in{0};
+        const size_t smem = bwd_token_simt_smem<T, D>();
+        if (smem > 48 * 1024)
+            if (int rc = ensure_big_smem(bwd_token_simt_kernel<T, D>, opt_in, (int)smem)) return rc;
+        bwd_token_simt_kernel<T, D><<<dim3((d->N + rows - 1) / rows, d->H, d->B), BwdSimtGeom<D>::kTokThreads, smem, st>>>(
+            (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, lse_enc, lse_dec, (T *)dK, (T *)dV, dd, d->B, d->H, d->N,
+            d->M, d->scale);
+        FLARE_CUDA(cudaGetLastError());
+        return FLARE_OK;
+    }
+};
+
+template <typename T, int D>
+struct DQuery {
+    static int run(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask, const void *dY,
+                   const float *Z, const float *dZ, const float *de, const float *dd, const float *lse_enc, const float *lse_dec, float *part,
+                   cudaStream_t st) {
+        static std::atomic<uint64_t> opt_in{0};
+        const size_t smem = bwd_dq_simt_smem<T, D>();
+        if (smem > 48 * 1024)
+            if (int rc = ensure_big_smem(bwd_dq_simt_kernel<T, D>, opt_in, (int)smem)) return rc;
+        bwd_dq_simt_kernel<T, D><<<dim3(p.splits, d->H * p.mblocks, d->B), kBwdThreads, smem, st>>>(
+            (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, dd, lse_enc, lse_dec, part, d->B, d->H, d->N, d->M, p.WM,
+            p.mblocks, p.chunk, d->scale);
+        FLARE_CUDA(cudaGetLastError());
+        return FLARE_OK;
+    }
+};
+
+// Op<T, D>::run(args...) for the call's element type and head width.
+template <template <typename, int> class Op, typename T, typename... A>
+int by_width(int D, A... a) {
+    switch (D) {
+        case 4: return Op<T, 4>::run(a...);
+        case 8: return Op<T, 8>::run(a...);
+        case 16: return Op<T, 16>::run(a...);
+        case 32: return Op<T, 32>::run(a...);
+        case 64: return Op<T, 64>::run(a...);
         default: return FLARE_ERR_UNSUPPORTED;
     }
-#undef FLARE_CASE
-    FLARE_CUDA(cudaGetLastError());
-    return FLARE_OK;
+}
+template <template <typename, int> class Op, typename... A>
+int by_type(const flare_desc_t *d, A... a) {
+    return d->dtype == FLARE_DTYPE_F32   ? by_width<Op, float>(d->D, a...)
+           : d->dtype == FLARE_DTYPE_F16 ? by_width<Op, __half>(d->D, a...)
+                                         : by_width<Op, __nv_bfloat16>(d->D, a...);
 }
 
 }  // namespace
 
 int encode_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask,
                 float *pm, float *pl, float *pacc, cudaStream_t st) {
-    return (d->dtype == FLARE_DTYPE_F32)   ? launch_encode_simt<float>(d, p, Q, K, V, mask, pm, pl, pacc, st)
-           : (d->dtype == FLARE_DTYPE_F16) ? launch_encode_simt<__half>(d, p, Q, K, V, mask, pm, pl, pacc, st)
-                                           : launch_encode_simt<__nv_bfloat16>(d, p, Q, K, V, mask, pm, pl, pacc, st);
+    return by_type<Encode>(d, false, d, p, Q, K, V, mask, (const float *)nullptr, pm, pl, pacc, st);
 }
-
+int encode_dz_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *dY, const float *lse_dec,
+                   float *pacc, cudaStream_t st) {
+    return by_type<Encode>(d, true, d, p, Q, K, dY, (const uint8_t *)nullptr, lse_dec, (float *)nullptr, (float *)nullptr, pacc, st);
+}
 int decode_simt(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st) {
-    return (d->dtype == FLARE_DTYPE_F32)   ? launch_decode_simt<float>(d, Q, K, Z, Y, lse_dec, st)
-           : (d->dtype == FLARE_DTYPE_F16) ? launch_decode_simt<__half>(d, Q, K, Z, Y, lse_dec, st)
-                                           : launch_decode_simt<__nv_bfloat16>(d, Q, K, Z, Y, lse_dec, st);
+    return by_type<Decode>(d, d, Q, K, Z, Y, lse_dec, st);
+}
+int bwd_token_simt(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, const void *dY,
+                   const float *Z, const float *dZ, const float *de, const float *lse_enc, const float *lse_dec, void *dK, void *dV,
+                   float *dd, cudaStream_t st) {
+    return by_type<Token>(d, d, Q, K, V, mask, dY, Z, dZ, de, lse_enc, lse_dec, dK, dV, dd, st);
+}
+int bwd_dq_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask,
+                const void *dY, const float *Z, const float *dZ, const float *de, const float *dd, const float *lse_enc,
+                const float *lse_dec, float *part, cudaStream_t st) {
+    return by_type<DQuery>(d, d, p, Q, K, V, mask, dY, Z, dZ, de, dd, lse_enc, lse_dec, part, st);
 }
 
 }  // namespace flare

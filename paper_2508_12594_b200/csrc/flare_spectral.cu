@@ -1,6 +1,5 @@
 // Spectral analysis: launches of the Gram and eigen-solver kernels.
 #include "flare_host.h"
-#include "flare_simt.cuh"
 #include "flare_spectral.cuh"
 
 namespace flare {

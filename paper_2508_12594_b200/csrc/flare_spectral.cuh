@@ -250,6 +250,23 @@ spectral_gram_reduce_kernel(const float *__restrict__ part, float *__restrict__ 
     Gout[idx] = s;
 }
 
+// Score q.k of one (latent, token) pair.  For float32 and float16 inputs the products are summed in double so that
+// the score, which is exponentiated, carries no float32 summation error; bfloat16 inputs sum in float.
+template <typename T, int D>
+__device__ __forceinline__ float score_dot(const float (&a)[D], const float *b) {
+    if constexpr (!std::is_same<T, __nv_bfloat16>::value) {   // float32 and float16 inputs
+        double s = 0.0;
+#pragma unroll
+        for (int d = 0; d < D; ++d) s = fma((double)a[d], (double)b[d], s);
+        return (float)s;
+    } else {
+        float s = 0.f;
+#pragma unroll
+        for (int d = 0; d < D; ++d) s = fmaf(a[d], b[d], s);
+        return s;
+    }
+}
+
 // G on the CUDA cores, for everything the tensor-core kernel does not take: one block per 16 x 16 tile of G of
 // one (b, h); the tokens are walked in chunks of 64 whose J rows for the tile's 16 + 16 latents sit in shared memory.
 template <typename T, int D>

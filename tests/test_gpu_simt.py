@@ -1,0 +1,21 @@
+"""The float32 / float16 kernels at the edges of their tiles (needs a B200): rows in blocks of 8 per warp and up to 8 warps,
+columns in tiles of 64 (32 at head width 64), against the oracle, forward and backward."""
+import pytest
+
+from paper_2508_12594_b200 import workloads
+from tests._util import assert_forward_close, gpu_forward, oracle_forward
+from tests.test_gpu_backward import assert_grads_close, gpu_backward, oracle_backward
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("B,H,N,M,D,masked", [
+    (1, 2, 63, 8, 16, 0.0), (1, 2, 64, 9, 16, 0.2), (2, 1, 65, 16, 8, 0.0), (1, 2, 127, 17, 32, 0.3), (1, 1, 129, 33, 16, 0.0),
+    (1, 2, 191, 64, 4, 0.0), (1, 1, 193, 65, 64, 0.2), (1, 1, 31, 257, 16, 0.0), (1, 1, 385, 129, 32, 0.0), (3, 8, 700, 20, 16, 0.1),
+])
+def test_tile_edges(oracle, B, H, N, M, D, masked, dtype):
+    inp = workloads.make_random(B, H, N, M, D, dtype=dtype, seed=N + M, masked_fraction=masked, with_dy=True, k_std=0.8)
+    what = f"{dtype} B{B}H{H}N{N}M{M}D{D}"
+    assert_forward_close(gpu_forward(inp, scale=0.7, canary=True), oracle_forward(oracle, inp, 0.7), dtype, what)
+    assert_grads_close(gpu_backward(inp, 0.7), oracle_backward(oracle, inp, 0.7), dtype, what)
