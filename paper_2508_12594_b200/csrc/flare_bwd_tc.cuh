@@ -85,7 +85,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NBARS);
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int M = a.M;
     const int split = blockIdx.x, h = blockIdx.y / a.pairs, pair = blockIdx.y % a.pairs, b = blockIdx.z;
     const int t_begin = (int)((long)a.tiles * split / a.splits);
@@ -160,7 +160,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const uint32_t tm = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             if (kHalf) {
                 ptx::mbar_arrive(bar(Q_FULL));                  // Q was written by the threads before the block barrier
             } else {
@@ -181,7 +181,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     } else if (warp < kFirstSoftmaxWarp) {
         const int g = warp - kFirstIssuerWarp;
         const int j = g >> 1, c = g & 1;
-        if (lane == 0 && j < nslots) {
+        if (j < nslots && ptx::elect_one()) {
             const uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0);
             const uint32_t idescQ = ptx::instr_desc_bf16(128, D, 0, 1);
             const uint64_t blk = (uint64_t)(alternate ? 0 : j * kTile * G::RB / 16);     // the slot's latent block
@@ -468,7 +468,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NBARS);
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int h = blockIdx.y, b = blockIdx.z;
     const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
     const int ng = stages < NG ? stages : NG;                   // groups at work
@@ -543,7 +543,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const uint32_t tm = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             if (kHalf) {
                 ptx::mbar_arrive(bar(Q_FULL));                  // Q was written by the threads before the block barrier
             } else {
@@ -563,7 +563,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         }
     } else if (warp < kFirstSoftmaxWarp) {
         const int g = warp - kFirstIssuerWarp;
-        if (lane == 0 && g < ng) {
+        if (g < ng && ptx::elect_one()) {
             const uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0);
             const uint32_t idescO = ptx::instr_desc_bf16(128, D, 0, 1);
             const uint32_t gcol = tm + g * 128;

@@ -77,7 +77,7 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
     // tensor memory, per group 160 columns: G [0,128)  S [128,160)
     constexpr uint32_t G_AA = 0, S_A = 128, GROUP_COLS = 160, NCOLS = 512;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int M = a.M;
     const int t_begin = (int)((long)a.tiles * split / a.splits), t_end = (int)((long)a.tiles * (split + 1) / a.splits);
@@ -101,7 +101,7 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
     const uint32_t tm = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             ptx::mbar_arrive_expect_tx(bar(Q_FULL), (uint32_t)(M * G::RB));
             for (int r = 0; r < M; r += 16) ptx::tma_load_2d(ptx::smem_u32(sQ + (size_t)r * G::RB), &tmQ, bar(Q_FULL), 0, h * M + r);
             for (int i = 0; i < nt; ++i) {
@@ -115,7 +115,7 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
         const int g = warp - kFirstIssuerWarp;
         const int mytiles = (nt - g + NGS - 1) / NGS;
         const uint32_t gtm = tm + g * GROUP_COLS;
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0), idescG = ptx::instr_desc_bf16(128, 128, 0, 0);
             const uint64_t qdesc = ptx::smem_desc(ptx::smem_u32(sQ), 16, G::SBO, G::SWZ);
             const uint64_t pbdesc = ptx::smem_desc(ptx::smem_u32(sPB + (size_t)g * 2 * SM::kPbBytes), 16, GP::SBO, GP::SWZ);

@@ -442,7 +442,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NBARS);
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int h = blockIdx.y, b = blockIdx.z;
     const int off = kHalf ? narrow_offset(h, DR) : 0;           // the head's first column within a token tile row
     const int t_begin = (int)((long)a.tiles * blockIdx.x / gridDim.x);
@@ -522,7 +522,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const uint32_t tm = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             if (kHalf) {
                 ptx::mbar_arrive(bar(Q_FULL));                  // Q was written by the threads before the block barrier
             } else {
@@ -532,7 +532,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     ptx::tma_load_2d(ptx::smem_u32(sQ + (size_t)r * G::RB), &tmQ, bar(Q_FULL), 0, h * a.mtot + a.m0 + r);
             }
         }
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             for (int i = 0; i < ntiles; ++i) {
                 const int s = i % nstages;
                 if (!ptx::mbar_wait(bar(K_EMPTY + s), ((i / nstages) & 1) ^ 1, abort_flag, kErrDecode | 1)) break;
@@ -543,7 +543,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         }
     } else if (warp < kFirstSoftmaxWarp) {
         const int g = warp - kFirstIssuerWarp;                  // the group this warp issues MMAs for
-        if (lane == 0 && g < nbuf * cs) {
+        if (g < nbuf * cs && ptx::elect_one()) {
             // One issuing thread per group: the scores of the group's next tile as soon as its K tile has landed and
             // its buffer is drained, then the value contraction of each hand-over of weights as it arrives.
             const int j = g / cs, c = g % cs;
@@ -817,7 +817,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     constexpr int YN = 48;                                      // N of the value MMA that carries the ones block
     constexpr int SUM_COL = 32;                                 // accumulator column of the row sum
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int tid = threadIdx.x < kTcThreads ? (int)threadIdx.x : (1 << 30);   // the guard warps stage nothing
     const int h = blockIdx.y, b = blockIdx.z;
     const int off = kHalf ? narrow_offset(h, DR) : 0;
@@ -888,7 +888,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     const uint32_t tm = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             if (kHalf) {
                 ptx::mbar_arrive(bar(Q_FULL));
             } else {
@@ -900,7 +900,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         for (int i = 0; i < ntiles; ++i) {
             const int s = i % nstages;
             if (!warp_wait(bar(K_EMPTY + s), ((i / nstages) & 1) ^ 1, abort_flag, kErrDecode | 1)) break;
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 ptx::mbar_arrive_expect_tx(bar(K_FULL + s), G::TILE_BYTES);
                 ptx::tma_load_3d(ptx::smem_u32(sK + (size_t)s * G::TILE_BYTES), &tmK, bar(K_FULL + s), h * DR - off,
                                  (t_begin + i) * kTile, b);
@@ -927,7 +927,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     } else if (warp < kFirstSoftmaxWarp) {
         const int g = warp - kFirstIssuerWarp;
         const int mytiles = (ntiles - g + NG - 1) / NG;          // tiles g, g + 4, ... of the CTA's range
-        if (lane == 0 && mytiles > 0) {
+        if (mytiles > 0 && ptx::elect_one()) {
             const uint32_t gcol = tm + g * GROUP_COLS;
             const uint32_t idescY = ptx::instr_desc_bf16(128, YN, 0, 1);
             const uint32_t idescLo = ptx::instr_desc_bf16(128, D, 0, 1);       // D = 32: the accumulating Z_lo product
@@ -1326,7 +1326,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NBARS);
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int tid = threadIdx.x < kTcThreads ? (int)threadIdx.x : (1 << 30);   // the guard warps stage nothing
     const int M = a.M;
     // h: the head, or in the head-pair form the first head of the pair
@@ -1422,7 +1422,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const uint32_t tm = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             if (kPair || kHalf) {
                 ptx::mbar_arrive(bar(Q_FULL));                  // Q was written by the threads before the block barrier
             } else {
@@ -1451,7 +1451,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
             }
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 ptx::mbar_arrive(bar(KV_FULL + s));             // the bias tile (or none needed)
                 ptx::mbar_arrive_expect_tx(bar(KV_FULL + s), 2 * G::TILE_BYTES);
                 uint8_t *dst = sKV + (size_t)s * 2 * G::TILE_BYTES;
@@ -1481,7 +1481,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     } else if (warp < kFirstSoftmaxWarp) {
         const int g = warp - kFirstIssuerWarp;                  // the group this warp issues MMAs for
         const int j = g >> 1, c = g & 1;                        // its slot and column half
-        if (lane == 0 && j < nslots) {
+        if (j < nslots && ptx::elect_one()) {
             const uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0);
             const uint32_t idescV = ptx::instr_desc_bf16(128, kOnes ? DG + 16 : DG, 0, 1);
             // Q rows of the slot's latent block (K-major A operand); descriptor address fields are in 16-byte units
