@@ -6,107 +6,94 @@
 namespace flare {
 namespace {
 
-template <int D, int DRT, bool kPadded, bool kAlt>
-int launch_bwd_dq_tc_a(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
+// padded tokens: a key mask, or a last partial tile
+bool has_padding(const flare_desc_t *d, const uint8_t *mask) { return mask != nullptr || d->N % kTile != 0; }
+
+template <int D, bool kPair, int DRT, bool kPadded>
+int launch_bwd_dq_tc_n(const flare_desc_t *d, const TcEncodePlan &p, const void *K, const void *V, const void *dY, const BwdDqTcArgs &args,
+                       cudaStream_t st) {
+    constexpr int DG = kPair ? 2 * D : D;
+    CUtensorMap tmK, tmV, tmG;
+    int rc;
+    if ((rc = make_token_map(&tmK, K, d, kTile, DG)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmV, V, d, kTile, DG)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmG, dY, d, kTile, DG)) != FLARE_OK) return rc;
+    static std::atomic<uint64_t> smem_opt_in{0};
+    if ((rc = ensure_big_smem(bwd_dq_tc_kernel<D, kPair, DRT, kPadded>, smem_opt_in)) != FLARE_OK) return rc;
+    bwd_dq_tc_kernel<D, kPair, DRT, kPadded><<<dim3(p.splits, (kPair ? d->H / 2 : d->H) * p.pairs, d->B), kDqThreads,
+                                                         BwdDqSmem<DG, kPair>::total, st>>>(tmK, tmV, tmG, args);
+    FLARE_CUDA(cudaGetLastError());
+    return FLARE_OK;
+}
+
+template <int D, bool kPair, int DRT>
+int launch_bwd_dq_tc_p(const flare_desc_t *d, const TcEncodePlan &p, bool padded, const void *K, const void *V, const void *dY,
+                       const BwdDqTcArgs &args, cudaStream_t st) {
+    return padded ? launch_bwd_dq_tc_n<D, kPair, DRT, true>(d, p, K, V, dY, args, st) : launch_bwd_dq_tc_n<D, kPair, DRT, false>(d, p, K, V, dY, args, st);
+}
+
+int launch_bwd_dq_tc(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
                      const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
                      const float *lse_dec, const float *dd, float *part, uint32_t *status, cudaStream_t st) {
-    CUtensorMap tmK, tmV, tmG, tmQ;
-    int rc;
-    if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
-    if ((rc = make_token_map(&tmV, V, d, kTile, D)) != FLARE_OK) return rc;
-    if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
-    if (DRT != 0) tmQ = tmK;   // unused: the narrow forms stage Q with their threads
-    else if ((rc = make_latent_map(&tmQ, Q, d)) != FLARE_OK) return rc;
-    const size_t smem = BwdDqSmem<D, kAlt>::total();
-    static std::atomic<uint64_t> smem_opt_in{0};
-    if (int rc_attr = ensure_big_smem(bwd_dq_tc_kernel<D, DRT, kPadded, kAlt>, smem_opt_in, 227 * 1024)) return rc_attr;
     BwdDqTcArgs a;
     a.Q = static_cast<const __nv_bfloat16 *>(Q);
     a.Z = Z; a.dZ = dZ; a.lse_enc = lse_enc; a.de = de; a.lse_dec = lse_dec; a.dd = dd;
     a.key_mask = mask; a.part = part; a.status = status;
     a.B = d->B; a.H = d->H; a.N = d->N; a.M = d->M;
     a.sl2 = d->scale * kLog2e;
-    a.tiles = p.tiles; a.splits = p.splits; a.pairs = p.pairs; a.partials_per_split = p.per_split;
-    dim3 grid(p.splits, d->H * p.pairs, d->B);
-    bwd_dq_tc_kernel<D, DRT, kPadded, kAlt><<<grid, kTcThreads, smem, st>>>(tmK, tmV, tmG, tmQ, a);
-    FLARE_CUDA(cudaGetLastError());
-    return FLARE_OK;
+    a.tiles = p.tiles; a.splits = p.splits; a.blocks = p.pairs;
+    const bool pad = has_padding(d, mask);
+    if (encode_head_pairs(d))
+        return d->D == 16 ? launch_bwd_dq_tc_p<16, true, 0>(d, p, pad, K, V, dY, a, st) : launch_bwd_dq_tc_p<32, true, 0>(d, p, pad, K, V, dY, a, st);
+    switch (d->D) {
+        case 4: return launch_bwd_dq_tc_p<16, false, 4>(d, p, pad, K, V, dY, a, st);
+        case 8: return launch_bwd_dq_tc_p<16, false, 8>(d, p, pad, K, V, dY, a, st);
+        case 16: return launch_bwd_dq_tc_p<16, false, 0>(d, p, pad, K, V, dY, a, st);
+        case 32: return launch_bwd_dq_tc_p<32, false, 0>(d, p, pad, K, V, dY, a, st);
+        default: return launch_bwd_dq_tc_p<64, false, 0>(d, p, pad, K, V, dY, a, st);
+    }
 }
 
-// (one latent block, M <= 128: the form whose slots take alternate tiles, with a deeper tile ring)
-template <int D, int DRT, bool kPadded>
-int launch_bwd_dq_tc_p(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
-                     const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
-                     const float *lse_dec, const float *dd, float *part, uint32_t *status, cudaStream_t st) {
-    if (d->M <= kTile)
-        return launch_bwd_dq_tc_a<D, DRT, kPadded, true>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st);
-    return launch_bwd_dq_tc_a<D, DRT, kPadded, false>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st);
-}
-
-template <int D, int DRT = 0>
-int launch_bwd_dq_tc(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
-                     const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
-                     const float *lse_dec, const float *dd, float *part, uint32_t *status, cudaStream_t st) {
-    // padded tokens: a key mask, or a last partial tile
-    if (mask != nullptr || d->N % kTile != 0)
-        return launch_bwd_dq_tc_p<D, DRT, true>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st);
-    return launch_bwd_dq_tc_p<D, DRT, false>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st);
-}
-
-template <int D, int DRT, int kMode, int kM, bool kPadded>
-int launch_bwd_token_tc_m(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const void *dY,
-                        const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
-                        const float *lse_dec, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st,
-                        int m0, int mc, float *kvacc) {
-    CUtensorMap tmK, tmV, tmG, tmQ;
+template <int D, int DRT, int kMode, bool kPadded>
+int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const void *V, const void *dY, BwdTokTcArgs a, cudaStream_t st) {
+    CUtensorMap tmK, tmV, tmG;
     int rc;
     if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
     if ((rc = make_token_map(&tmV, V, d, kTile, D)) != FLARE_OK) return rc;
     if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
-    if (DRT != 0) tmQ = tmK;   // unused: the narrow forms stage Q with their threads
-    else if ((rc = make_latent_map(&tmQ, Q, d)) != FLARE_OK) return rc;
-    BwdTokTcArgs a;
-    a.stages = BwdTokSmem<D>::stages(mc);
+    a.stages = BwdTokSmem<D>::stages(a.M);
     if (a.stages < 1) return FLARE_ERR_UNSUPPORTED;
-    const size_t smem = BwdTokSmem<D>::total(a.stages, mc);
     static std::atomic<uint64_t> smem_opt_in{0};
-    if (int rc_attr = ensure_big_smem(bwd_token_tc_kernel<D, DRT, kMode, kM, kPadded>, smem_opt_in, 227 * 1024)) return rc_attr;
+    if ((rc = ensure_big_smem(bwd_token_tc_kernel<D, DRT, kMode, kPadded>, smem_opt_in)) != FLARE_OK) return rc;
+    a.tiles = (d->N + kTile - 1) / kTile;
+    long per_head = sms / ((long)d->B * d->H);
+    if (per_head < 1) per_head = 1;
+    if (per_head > a.tiles) per_head = a.tiles;
+    bwd_token_tc_kernel<D, DRT, kMode, kPadded><<<dim3((unsigned)per_head, d->H, d->B), BwdGroups<2 * D>::kThreads, BwdTokSmem<D>::total(a.stages, a.M), st>>>(
+        tmK, tmV, tmG, a);
+    FLARE_CUDA(cudaGetLastError());
+    return FLARE_OK;
+}
+
+// The launch's range of latents is [m0, m0 + mc).  mode: see BwdTokTcArgs.
+template <int D, int DRT>
+int launch_bwd_token_tc(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const void *dY,
+                        const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
+                        const float *lse_dec, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st, int mode, int m0, int mc,
+                        float *kvacc) {
+    BwdTokTcArgs a;
     a.Q = static_cast<const __nv_bfloat16 *>(Q);
     a.Z = Z; a.dZ = dZ; a.lse_enc = lse_enc; a.de = de; a.lse_dec = lse_dec; a.key_mask = mask;
     a.dK = (__nv_bfloat16 *)dK; a.dV = (__nv_bfloat16 *)dV; a.dd = dd; a.status = status;
     a.B = d->B; a.H = d->H; a.N = d->N; a.M = mc;
     a.mtot = d->M; a.m0 = m0; a.first = m0 == 0; a.last = m0 + mc >= d->M; a.kvacc = kvacc;
     a.scale = d->scale; a.sl2 = d->scale * kLog2e;
-    a.tiles = (d->N + kTile - 1) / kTile;
-    long per_head = sms / ((long)d->B * d->H);
-    if (per_head < 1) per_head = 1;
-    if (per_head > a.tiles) per_head = a.tiles;
-    bwd_token_tc_kernel<D, DRT, kMode, kM, kPadded><<<dim3((unsigned)per_head, d->H, d->B), kTcThreads, smem, st>>>(tmK, tmV, tmG, tmQ, a);
-    FLARE_CUDA(cudaGetLastError());
-    return FLARE_OK;
-}
-
-// The launch's range of latents is [m0, m0 + mc) (mc = 0: all of them); common sizes have forms of the kernel with
-// the number of latents as a compile-time constant.
-template <int D, int DRT = 0, int kMode = 0>
-int launch_bwd_token_tc(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const void *dY,
-                        const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
-                        const float *lse_dec, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st,
-                        int m0 = 0, int mc = 0, float *kvacc = nullptr) {
-    if (mc == 0) mc = d->M;
-    const bool padded = mask != nullptr || d->N % kTile != 0;   // a key mask, or a last partial tile
-#define FLARE_TOK(MM)                                                                                                     \
-    (padded ? launch_bwd_token_tc_m<D, DRT, kMode, MM, true>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, dd, \
-                                                            status, st, m0, mc, kvacc)                                   \
-            : launch_bwd_token_tc_m<D, DRT, kMode, MM, false>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, dd, \
-                                                             status, st, m0, mc, kvacc))
-    if (mc == 256) return FLARE_TOK(256);
-    if (mc == 128) return FLARE_TOK(128);
-    if (mc == 64) return FLARE_TOK(64);
-    if (mc == 512) return FLARE_TOK(512);
-    return FLARE_TOK(0);
+    const bool pad = has_padding(d, mask);
+#define FLARE_TOK(MODE) (pad ? launch_bwd_token_tc_n<D, DRT, MODE, true>(d, sms, K, V, dY, a, st) : launch_bwd_token_tc_n<D, DRT, MODE, false>(d, sms, K, V, dY, a, st))
+    return mode == 0 ? FLARE_TOK(0) : mode == 1 ? FLARE_TOK(1) : FLARE_TOK(2);
 #undef FLARE_TOK
 }
+
 template <typename T, int D>
 int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V,
                          const uint8_t *mask, const void *Y, const void *dY, const float *Z, const float *lse_enc,
@@ -140,47 +127,29 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
     if (!skip_pass_a) {
         FLARE_REDUCE(bwd_dz_reduce_kernel, rows, dz_parts, D, st, part, Z, dZ, de, dz_parts, rows);
     }
-    bool tok_on_tc = false;
-    if constexpr (std::is_same<T, __nv_bfloat16>::value && D <= 32) {
+    bool on_tc = false;
+    int dq_parts = pb.P;
+    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         constexpr int DK = D < 16 ? 16 : D;                     // width the kernels multiply (D < 16: narrow forms)
         constexpr int DRT = D < 16 ? D : 0;
         uint32_t *status = reinterpret_cast<uint32_t *>(ws);
-        if (bwd_dq_on_tensor_cores(d) && !token_in_ranges(d) && BwdTokSmem<DK>::stages(d->M) >= 1) {
-            const int rc = launch_bwd_token_tc<DK, DRT>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, dd,
-                                                        status, st);
-            if (rc != FLARE_OK) return rc;
-            tok_on_tc = true;
-        } else if (token_in_ranges(d)) {
-            // two series of launches over the latent ranges: dd[n] first, then the rows of dK and dV
+        on_tc = bwd_dq_on_tensor_cores(d);
+        if (on_tc) {
+            // more latents than one launch holds: two series of launches over ranges of them, dd[n] first, then the rows of dK and dV
             float *kvacc = reinterpret_cast<float *>(ws + w.kvacc);
             const int R = token_range(d);
-            for (int mode = 1; mode <= 2; ++mode)
-                for (int m0 = 0; m0 < d->M; m0 += R) {
-                    const int mc = d->M - m0 < R ? d->M - m0 : R;
-                    const int rc = mode == 1 ? launch_bwd_token_tc<DK, DRT, 1>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec,
-                                                                              dK, dV, dd, status, st, m0, mc, kvacc)
-                                             : launch_bwd_token_tc<DK, DRT, 2>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec,
-                                                                              dK, dV, dd, status, st, m0, mc, kvacc);
-                    if (rc != FLARE_OK) return rc;
-                }
-            tok_on_tc = true;
+            for (int mode = token_in_ranges(d) ? 1 : 0; mode <= (token_in_ranges(d) ? 2 : 0); ++mode)
+                for (int m0 = 0; m0 < d->M; m0 += R)
+                    if (const int rc = launch_bwd_token_tc<DK, DRT>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, dd, status,
+                                                                    st, mode, m0, d->M - m0 < R ? d->M - m0 : R, kvacc))
+                        return rc;
+            const TcEncodePlan p = tc_dq_plan(d, sms);
+            if (const int rc = launch_bwd_dq_tc(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st)) return rc;
+            dq_parts = p.P;
         }
     }
-    if (!tok_on_tc) {
+    if (!on_tc) {
         if (const int rc = bwd_token_simt(d, Q, K, V, mask, dY, Z, dZ, de, lse_enc, lse_dec, dK, dV, dd, st)) return rc;
-    }
-    int dq_parts = pb.P;
-    bool dq_on_tc = false;
-    if constexpr (std::is_same<T, __nv_bfloat16>::value && D <= 32) {
-        if (bwd_dq_on_tensor_cores(d)) {
-            const int rc = launch_bwd_dq_tc<(D < 16 ? 16 : D), (D < 16 ? D : 0)>(d, tc_dq_plan(d, sms), Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part,
-                                               reinterpret_cast<uint32_t *>(ws), st);
-            if (rc != FLARE_OK) return rc;
-            dq_parts = tc_dq_plan(d, sms).P;
-            dq_on_tc = true;
-        }
-    }
-    if (!dq_on_tc) {
         if (const int rc = bwd_dq_simt(d, pb, Q, K, V, mask, dY, Z, dZ, de, dd, lse_enc, lse_dec, part, st)) return rc;
     }
     FLARE_REDUCE(bwd_dq_reduce_kernel, (long)d->H * d->M, d->B * dq_parts, D, st, part, dQ, dq_parts, d->B, (long)d->H * d->M, d->scale);

@@ -1,26 +1,122 @@
-// Tensor-core kernels of the backward for bfloat16 inputs on sm_100a (pass B: the gradient of the latent queries).
+// Tensor-core kernels of the backward for bfloat16 inputs on sm_100a (pass B: the gradients of the latent queries, keys and
+// values).
 //
-// dQ_m = scale * sum_n dS[m,n] k_n with
+// dQ_m = scale * sum_n dS[m,n] k_n,   dK_n = scale * sum_m dS[m,n] q_m,   dV_n = sum_m W_enc[m,n] dZ_m   with
 //   dS[m,n] = W_dec[n,m] (dY_n . Z_m - dd[n]) + W_enc[m,n] (dZ_m . V_n - de[m]),
 //   W_dec[n,m] = exp(S[m,n] - lse_dec[n]),  W_enc[m,n] = valid(n) exp(S[m,n] - lse_enc[m]),  S = scale * q_m . k_n.
-// The kernel has the shape of the encode kernel (latents on the 128 TMEM lanes, tokens on columns, the CTA's
-// token range split over N, one pipeline per softmax group with its own issuing warp): per unit of 16 tokens
-// three MMAs put S, A = Z dY^T and C = dZ V^T side by side in tensor memory, the group's threads turn them into
-// dS (two bf16 halves) over columns they have read, and two more MMAs add dS K_unit to the group's partial dQ.
-// Units alternate between two such buffers, so the tiles of the next unit and the dQ MMAs of the previous one
-// run while the group works on the current one (2 x 48 + D <= 128 columns per group).  Z and dZ enter as two bf16
-// halves each (hi + lo): the products dY.Z_m and dZ_m.V_n are differenced against dd and de.
+//
+// Both kernels turn three tiles that the tensor core puts side by side in tensor memory, S = q.k, A = dY.Z and C = dZ.V, into
+// dS (and W_enc) over the columns just read, which feed the output contractions as their A operand.  One kind of row sits
+// on the 128 lanes (latents in the dQ kernel, tokens in the token kernel), the other on the columns, in units of 64 or 32.
+// Z and dZ, and dS and W_enc, enter as two bf16 halves each: the sums cancel (see the host code's notes on precision).
+//
+// What shapes them.  A tcgen05.mma with both operands in shared memory takes the tensor core 40 cycles at N = 16 or 32, 48 at 64 and 64
+// at 128 (most of it the fetch of its A operand), one with A in tensor memory N / 2; a hand-over between threads and tensor core
+// costs a warp some 100 instructions and a round trip of about 1000 cycles.  Units of 16 columns (dQ kernel at D = 32: ten MMAs of N = 16 for
+// 16 tokens) ran at exactly the tensor limit.  Wider units are either shared by all warps (dQ kernel) or each group of four warps has one
+// of its own (token kernel); which serves better was measured for both.
 #pragma once
 
 #include "flare_tc.cuh"
 
 namespace flare {
 
-constexpr int kBqStages = 3;     // (K, V, dY) tile triples in flight where all four groups of a CTA work on the same tile
-constexpr int kBqMaxStages = 8;  // ... and at most where the two slots take alternate tiles (see kEncMaxStages)
+// dS of a pair of columns as packed bf16 halves hi, lo (and W_enc where it is wanted).  xd = s * sl2 + nd is the decode exponent
+// (log2 units), u = A + na, v = C + nc.  Both weights come from one exponential: with K the smallest lse_enc of the CTA's latents
+// (log2 units),
+//     W_enc = W_dec 2^(lse_dec[n] - K) 2^(K - lse_enc[m]),    fr, fc the two factors (fc 0 for a token that takes no part),
+// exact to float32 rounding wherever it matters as long as lse_dec[n] - K <= kOneExpLog2: the second factor is at most 1, so what
+// underflows on the way (W_dec below 2^-126, a factor below 2^-126) is a weight below 2^(kOneExpLog2 - 126).  Tokens beyond that
+// bound (or with an infinite lse_dec, how the two-query variant switches a stage off) take the form with an exponential of its own for
+// W_enc, kTwo: xe = s * sl2 + ne.  (An exponential costs the special-function unit as much as the rest of a pair costs the
+// issue slots: with two per pair the unit bound both kernels.)
+constexpr float kOneExpLog2 = 40.f;
+struct DsPair { uint32_t hi, lo, whi, wlo; };
+template <bool kWeights, bool kTwo>
+__device__ __forceinline__ DsPair ds_pair(float2 s, float2 av, float2 cv, float2 sl2p, float2 nd, float2 na, float2 nc, float2 fr_ne, float2 fc) {
+    const float2 xd = __ffma2_rn(s, sl2p, nd);
+    const float2 pd = make_float2(ptx::ex2(xd.x), ptx::ex2(xd.y));
+    const float2 u = __fadd2_rn(av, na), v = __fadd2_rn(cv, nc);
+    float2 pe, ds;
+    if (kTwo) {                                                  // fr_ne: -lse_enc[m]; fc: 0, or -inf for a token that takes no part
+        const float2 xe = __ffma2_rn(s, sl2p, __fadd2_rn(fr_ne, fc));
+        pe = make_float2(ptx::ex2(xe.x), ptx::ex2(xe.y));
+        ds = __ffma2_rn(pd, u, __fmul2_rn(pe, v));
+    } else {
+        const float2 r = __fmul2_rn(fr_ne, fc);
+        if (kWeights) pe = __fmul2_rn(pd, r);
+        ds = __fmul2_rn(pd, __ffma2_rn(r, v, u));
+    }
+    DsPair o;
+    o.hi = ptx::pack_bf16(ds.x, ds.y);
+    o.lo = ptx::pack_bf16(ds.x - __uint_as_float(o.hi << 16), ds.y - __uint_as_float(o.hi & 0xffff0000u));
+    if (kWeights) {
+        o.whi = ptx::pack_bf16(pe.x, pe.y);
+        o.wlo = ptx::pack_bf16(pe.x - __uint_as_float(o.whi << 16), pe.y - __uint_as_float(o.whi & 0xffff0000u));
+    }
+    return o;
+}
+constexpr float kBwdLog2e = 1.4426950408889634f;
+// Smallest lse_enc (log2 units) of `rows` latents, leaving out those that saw no valid token (-inf); 0 if there is none.  By a full warp.
+__device__ __forceinline__ float warp_lse_min(const float *lse_enc, int rows) {
+    float k = INFINITY;
+    for (int m = threadIdx.x & 31; m < rows; m += 32) {
+        const float le = lse_enc[m];
+        if (le != -INFINITY) k = fminf(k, le * kBwdLog2e);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) k = fminf(k, __shfl_xor_sync(0xffffffffu, k, o));
+    return k <= 3.0e38f ? k : 0.f;
+}
+
+// rows of a [rows, DR] float matrix -> bf16 halves in swizzled rows (DR >= 8), starting at logical chunk `chunk0` of row r0 + m
+template <int DG, int DR>
+__device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float *src, int rows, int r0, int chunk0, int tid, int threads) {
+    using G = TileGeom<DG>;
+    constexpr int ZC = DR >= 8 ? DR / 8 : 1;
+    for (int i = tid; i < rows * ZC; i += threads) {
+        const int m = i / ZC, c = i % ZC, r = r0 + m;
+        const float4 a = *reinterpret_cast<const float4 *>(src + (size_t)m * DR + c * 8);
+        const float4 b = *reinterpret_cast<const float4 *>(src + (size_t)m * DR + c * 8 + 4);
+        const float z[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        uint32_t vh[4], vl[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            vh[k] = ptx::pack_bf16(z[2 * k], z[2 * k + 1]);
+            vl[k] = ptx::pack_bf16(z[2 * k] - __uint_as_float(vh[k] << 16), z[2 * k + 1] - __uint_as_float(vh[k] & 0xffff0000u));
+        }
+        const size_t o = (size_t)r * G::RB + (((chunk0 + c) ^ G::swz(r)) << 4);
+        *reinterpret_cast<uint4 *>(hi + o) = make_uint4(vh[0], vh[1], vh[2], vh[3]);
+        *reinterpret_cast<uint4 *>(lo + o) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
+    }
+}
+// rows of a [rows, DR] bf16 matrix -> swizzled rows, as above
+template <int DG, int DR>
+__device__ __forceinline__ void stage_bf16(uint8_t *dst, const __nv_bfloat16 *src, int rows, int r0, int chunk0, int tid, int threads) {
+    using G = TileGeom<DG>;
+    constexpr int QC = DR >= 8 ? DR / 8 : 1;
+    for (int i = tid; i < rows * QC; i += threads) {
+        const int m = i / QC, c = i % QC, r = r0 + m;
+        *reinterpret_cast<uint4 *>(dst + (size_t)r * G::RB + (((chunk0 + c) ^ G::swz(r)) << 4)) =
+            *reinterpret_cast<const uint4 *>(src + (size_t)m * DR + c * 8);
+    }
+}
+
+// ------------------------------------------------------------------------------- pass B, latent side (dQ)
+
+// Units of 64 tokens, shared by sixteen warps, 16 columns each, on two alternating buffers of tensor memory (S | A | C; then the
+// accumulators): while the threads work on one unit the tensor core runs the output contractions of the other and the tiles of the one after.
+// Warps: 0 TMA producer, 1 MMA issue, 3 column constants, 4-19 arithmetic (warp & 3 = the quarter of the lanes it can reach).
+// Measured, us, against units of 16 columns with two exponentials per pair (N = 16384, M = 32, D = 32, 8 heads; 32 x 4096, M = 128, 4 heads;
+// 131072, M = 512, 8 heads; 1048576, M = 1024, D = 8, 8 heads): 22.4, 82, 437, 7844 -> 15.9, 65, 392, 5706; D = 64 (2 x 20011, M = 128, 4
+// heads), on the CUDA cores before: 498 -> 27.  Groups of four warps with units and buffers of their own, as in the token kernel:
+// 21.6, 78, 522, 7485; 44.  Issue slots and the latency of tensor-memory loads share the bound (some 14 instructions per pair, two issued
+// per cycle and SM).
+constexpr int kDqUnit = 64, kDqBuf = 3 * kDqUnit, kDqAcc = 2 * kDqBuf;
+constexpr int kDqThreads = 640, kDqFirstMathWarp = 4;
 
 struct BwdDqTcArgs {
-    const __nv_bfloat16 *Q;    // [H,M,D] (read directly in the half-width form)
+    const __nv_bfloat16 *Q;    // [H,M,D]
     const float *Z, *dZ;       // [B,H,M,D]
     const float *lse_enc, *de; // [B,H,M]
     const float *lse_dec;      // [B,N,H]
@@ -30,376 +126,398 @@ struct BwdDqTcArgs {
     uint32_t *status;
     int B, H, N, M;
     float sl2;                 // scale * log2(e)
-    int tiles, splits, pairs, partials_per_split;
+    int tiles, splits, blocks; // blocks: of 128 latents per head
 };
 
-template <int D, bool kAlt>
+template <int DG, bool kPair>
 struct BwdDqSmem {
-    using G = TileGeom<D>;
-    static constexpr size_t kColBytes = 4 * kSoftmaxGroups * 2 * 64 * sizeof(float);   // per softmax warp: 2 x 64 column constants
+    using G = TileGeom<DG>;
+    static constexpr int kCst = 8, kAhead = 4;                                   // tiles of column constants in the ring, of them on their way
+    static constexpr size_t kCstBytes = (size_t)(kPair ? 2 : 1) * 3 * kTile * sizeof(float);   // per head: -lse_dec, -dd, mask
     static constexpr size_t total_for(int n) {
-        return (size_t)n * 3 * G::TILE_BYTES + (size_t)5 * 2 * kTile * G::RB + 512 + kColBytes + 1024;
+        return (size_t)n * 3 * G::TILE_BYTES + (size_t)5 * kTile * G::RB + kCst * kCstBytes + 768 + 1024;
     }
     static constexpr int stages_for() {
-        int n = kAlt ? kBqMaxStages : kBqStages;
-        while (n > kBqStages && total_for(n) > 227 * 1024) --n;
+        int n = 6;
+        while (n > 1 && total_for(n) > 227 * 1024) --n;
         return n;
     }
-    static constexpr int kStages = stages_for();                 // (K, V, dY) tile triples in flight
-    static constexpr size_t tile_off = 0;                        // [stage][K | V | dY]
-    __host__ __device__ static size_t q_off() { return (size_t)kStages * 3 * G::TILE_BYTES; }
-    // Q, Z_hi, Z_lo, dZ_hi, dZ_lo: 256 latent rows each
-    __host__ __device__ static size_t lat_off(int which) { return q_off() + (size_t)which * 2 * kTile * G::RB; }
-    __host__ __device__ static size_t bar_off() { return lat_off(5); }
-    __host__ __device__ static size_t col_off() { return bar_off() + 512; }
-    __host__ __device__ static size_t total() {
-        size_t t = col_off() + kColBytes + 1024;
-        return t < kTcMinSmem ? kTcMinSmem : t;
-    }
+    static constexpr int kStages = stages_for();                                 // (K, V, dY) tile triples in flight
+    __host__ __device__ static constexpr size_t lat_off(int which) { return (size_t)kStages * 3 * G::TILE_BYTES + (size_t)which * kTile * G::RB; }
+    static constexpr size_t cst_off = (size_t)kStages * 3 * G::TILE_BYTES + (size_t)5 * kTile * G::RB;
+    static constexpr size_t bar_off = cst_off + kCst * kCstBytes;
+    static constexpr size_t total = total_for(kStages) < kTcMinSmem ? kTcMinSmem : total_for(kStages);
 };
 
-// grid = (splits, H * pairs, B), as the encode kernel.  DRT = 8 or 4 (with D = 16): the narrow form of the forward
-// kernels (the head is DRT wide in memory; token tiles carry the neighbouring heads' features beside the head's
-// own, every latent operand zeros there, and the other columns of the partial dQ are dropped).
-// kPadded: the launch has padded tokens (a key mask, or N not a multiple of the tile); without it the unit body that
-// tests validity is not compiled in.  kAlt: one latent block (the host picks this form for M <= 128), the two slots take
-// alternate tiles and the tile ring is as deep as fits.
-template <int D, int DRT = 0, bool kPadded = true, bool kAlt = false>
-__global__ void __launch_bounds__(kTcThreads, 1)
+// grid = (splits, heads or head pairs * blocks, B); a CTA takes one block of 128 latents and a contiguous range of token tiles.
+// kPair: two heads of at most 64 latents side by side on the lanes, as in the encode kernel (block-diagonal latent operands over
+// the 2 D columns the heads occupy in a token row).  DRT = 8 or 4 (with D = 16): the narrow form (the head is DRT wide in memory;
+// token tiles carry the neighbouring heads' features beside the head's own, every latent operand zeros there).
+// kPadded: the launch has padded tokens (a key mask, or N not a multiple of the tile): a third constant per column, 0 or -inf.
+template <int D, bool kPair, int DRT, bool kPadded>
+__global__ void __launch_bounds__(kDqThreads, 1)
 bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                 const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmQ, BwdDqTcArgs a) {
-    using G = TileGeom<D>;
-    using SM = BwdDqSmem<D, kAlt>;
-    constexpr int nstages = SM::kStages;                        // depth of the tile ring
-    constexpr bool kHalf = DRT != 0;
-    constexpr int DR = kHalf ? DRT : D;                         // head width in memory
+                 const __grid_constant__ CUtensorMap tmG, BwdDqTcArgs a) {
+    constexpr int DG = kPair ? 2 * D : D;
+    using G = TileGeom<DG>;
+    using SM = BwdDqSmem<DG, kPair>;
+    constexpr int DR = DRT ? DRT : D;                           // head width in memory
+    static_assert(!(kPair && DRT), "head pairs are full width");
+    // The units take turns on as many accumulators as there is room for: the tensor core truncates each of the thousands of sums that a
+    // split adds up in float32, an error that grows with their number.
+    constexpr int kAccs = (512 - kDqAcc) / DG;
+    static_assert(kAccs >= 1 && (kAccs & (kAccs - 1)) == 0, "tensor memory");
+    constexpr int UNIT = kDqUnit, UPT = kTile / UNIT, nstages = SM::kStages;
+    static_assert(nstages >= 2, "one tile is finished while the next begins");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t *sT = smem + SM::tile_off;
-    uint8_t *sQ = smem + SM::lat_off(0);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off());
-    constexpr int NG = kSoftmaxGroups;
-    // per group: S_FULL and P_FULL for each of its two unit buffers
-    enum { T_FULL = 0, T_EMPTY = T_FULL + nstages, S_FULL = T_EMPTY + nstages, P_FULL = S_FULL + 2 * NG,
-           ACC_DONE = P_FULL + 2 * NG, Q_FULL = ACC_DONE + NG, NBARS };
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off);
+    enum { T_FULL = 0, T_EMPTY = T_FULL + nstages, C_FULL = T_EMPTY + nstages, C_EMPTY = C_FULL + SM::kCst, S_FULL = C_EMPTY + SM::kCst,
+           P_FULL = S_FULL + 2, ACC_DONE = P_FULL + 2, NBARS = ACC_DONE + 1 };
+    static_assert(NBARS * 8 + 16 + 8 * SM::kCst <= 768, "barrier area too small");
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NBARS);
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int M = a.M;
-    const int split = blockIdx.x, h = blockIdx.y / a.pairs, pair = blockIdx.y % a.pairs, b = blockIdx.z;
-    const int t_begin = (int)((long)a.tiles * split / a.splits);
-    const int t_end = (int)((long)a.tiles * (split + 1) / a.splits);
+    const int split = blockIdx.x, h = (kPair ? 2 : 1) * (blockIdx.y / a.blocks), lb = blockIdx.y % a.blocks, b = blockIdx.z;
+    const int t_begin = (int)((long)a.tiles * split / a.splits), t_end = (int)((long)a.tiles * (split + 1) / a.splits);
     const int nt = t_end - t_begin;
-    const int MB = (M + kTile - 1) / kTile;
-    const bool alternate = kAlt || MB == 1;                           // one latent block: the two slots take alternate tiles
-    const int lb0 = pair * 2;
-    const int nslots = alternate ? 2 : ((lb0 + 1 < MB) ? 2 : 1);
-    const int nq = alternate ? nt : nt * nslots;
-    const int rows_here = min(M - lb0 * kTile, 2 * kTile);
-    constexpr int SLOT_COLS = 256, HALF = kTile / 2, UNIT = 16, UPH = HALF / UNIT;   // units per half tile
-    constexpr uint32_t NCOLS = 512;
-    // per group (128 columns): two unit buffers of 48 columns (S, A, C: 16 each), partial dQ at 96
+    const int rows_here = kPair ? M : min(M - lb * kTile, kTile);
+    const int off = DRT ? narrow_offset(h, DR) : 0;             // the head's first column within a token tile row
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
 
     if (threadIdx.x == 0) {
-        const uint32_t users = alternate ? 2u : 2u * (uint32_t)nslots;
         for (int i = 0; i < NBARS; ++i)
-            ptx::mbar_init(bar(i), (i >= P_FULL && i < P_FULL + 2 * NG) ? 128u
-                                   : (i >= T_EMPTY && i < T_EMPTY + nstages) ? users : 1u);
+            ptx::mbar_init(bar(i), (i >= P_FULL && i < P_FULL + 2) || (i >= C_EMPTY && i < C_EMPTY + SM::kCst) ? 16u : 1u);
         *abort_flag = 0;
         ptx::fence_mbar_init();
         ptx::prefetch_tensormap(&tmK);
         ptx::prefetch_tensormap(&tmV);
         ptx::prefetch_tensormap(&tmG);
-        ptx::prefetch_tensormap(&tmQ);
     }
-    if (warp == kFirstIssuerWarp) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), NCOLS);
-    // zero the latent rows beyond M (all five operands; in the half-width form all rows, whose upper halves stay
-    // zero), then Z and dZ as bf16 hi/lo rows in the swizzled layout
-    for (int i = threadIdx.x; i < 5 * 2 * kTile * (G::RB / 16); i += kTcThreads) {
-        const int which = i / (2 * kTile * (G::RB / 16)), rem = i % (2 * kTile * (G::RB / 16));
-        if (kHalf || rem / (G::RB / 16) >= rows_here) reinterpret_cast<uint4 *>(smem + SM::lat_off(which))[rem] = make_uint4(0, 0, 0, 0);
-    }
-    const int off = kHalf ? narrow_offset(h, DR) : 0;           // the head's first column within a token tile row
-    if (kHalf) {
-        __syncthreads();
-        if constexpr (DR == 4) {
-            const size_t r0 = ((size_t)b * a.H + h) * M + lb0 * kTile;
-            stage_rows4<D>(sQ, a.Q + ((size_t)h * M + lb0 * kTile) * DR, rows_here, off);
-            stage_rows4_hilo<D>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, off);
-            stage_rows4_hilo<D>(smem + SM::lat_off(3), smem + SM::lat_off(4), a.dZ + r0 * DR, rows_here, off);
-        } else {
-            for (int i = threadIdx.x; i < rows_here * (DR / 8); i += kTcThreads) {
-                const int m = i / (DR / 8), ch = i % (DR / 8);
-                *reinterpret_cast<uint4 *>(sQ + (size_t)m * G::RB + ((ch ^ G::swz(m)) << 4)) =
-                    *reinterpret_cast<const uint4 *>(a.Q + ((size_t)h * M + lb0 * kTile + m) * DR + ch * 8);
-            }
-        }
-    }
-    constexpr int ZC = DR >= 8 ? DR / 8 : 1;                    // 8-float chunks per row (none for DR = 4: staged above)
-    for (int i = threadIdx.x; i < (DR >= 8 ? 2 * rows_here * ZC : 0); i += kTcThreads) {
-        const int which = i / (rows_here * ZC), rem = i % (rows_here * ZC), m = rem / ZC, ch = rem % ZC;
-        const float *src = (which == 0 ? a.Z : a.dZ) + (((size_t)b * a.H + h) * M + lb0 * kTile + m) * DR + ch * 8;
-        const float4 lo4 = *reinterpret_cast<const float4 *>(src), hi4 = *reinterpret_cast<const float4 *>(src + 4);
-        const float z[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
-        uint32_t vh[4], vl[4];
+    float *kmin = reinterpret_cast<float *>(tmem_slot + 2);     // smallest lse_enc, per head of the CTA
+    volatile uint32_t *two_exp = tmem_slot + 4;                 // [kCst][head]: the tile needs an exponential of its own for W_enc
+    if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
+    if (warp == 3) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            vh[k] = ptx::pack_bf16(z[2 * k], z[2 * k + 1]);
-            vl[k] = ptx::pack_bf16(z[2 * k] - __uint_as_float(vh[k] << 16), z[2 * k + 1] - __uint_as_float(vh[k] & 0xffff0000u));
+        for (int w = 0; w < (kPair ? 2 : 1); ++w) {
+            const float k = warp_lse_min(a.lse_enc + ((size_t)b * a.H + h + w) * M + lb * kTile, rows_here);
+            if (lane == 0) kmin[w] = k;
         }
-        const size_t off = (size_t)m * G::RB + ((ch ^ G::swz(m)) << 4);
-        *reinterpret_cast<uint4 *>(smem + SM::lat_off(1 + 2 * which) + off) = make_uint4(vh[0], vh[1], vh[2], vh[3]);
-        *reinterpret_cast<uint4 *>(smem + SM::lat_off(2 + 2 * which) + off) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
+    }
+    // latent operands Q, Z_hi, Z_lo, dZ_hi, dZ_lo: zeros where there is no row (or, pair and narrow forms, no feature), then the rows
+    const bool gaps = kPair || DRT != 0 || rows_here < kTile;
+    if (gaps) {
+        for (int i = threadIdx.x; i < 5 * kTile * (G::RB / 16); i += kDqThreads)
+            reinterpret_cast<uint4 *>(smem + SM::lat_off(0))[i] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int w = 0; w < (kPair ? 2 : 1); ++w) {
+        const size_t q0 = (size_t)(h + w) * M + lb * kTile, r0 = ((size_t)b * a.H + h + w) * M + lb * kTile;
+        if constexpr (DR == 4) {
+            stage_rows4<DG>(smem + SM::lat_off(0), a.Q + q0 * DR, rows_here, off);
+            stage_rows4_hilo<DG>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, off);
+            stage_rows4_hilo<DG>(smem + SM::lat_off(3), smem + SM::lat_off(4), a.dZ + r0 * DR, rows_here, off);
+        } else {
+            stage_bf16<DG, DR>(smem + SM::lat_off(0), a.Q + q0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
+            stage_hilo<DG, DR>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
+            stage_hilo<DG, DR>(smem + SM::lat_off(3), smem + SM::lat_off(4), a.dZ + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
+        }
     }
     ptx::fence_proxy_async_smem();
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tm = *tmem_slot;
+    const float lse_min[2] = {kmin[0], kmin[kPair ? 1 : 0]};
 
     if (warp == 0) {
         if (ptx::elect_one()) {
-            if (kHalf) {
-                ptx::mbar_arrive(bar(Q_FULL));                  // Q was written by the threads before the block barrier
-            } else {
-                ptx::mbar_arrive_expect_tx(bar(Q_FULL), (uint32_t)(rows_here * G::RB));
-                for (int r = 0; r < rows_here; r += 16)
-                    ptx::tma_load_2d(ptx::smem_u32(sQ + (size_t)r * G::RB), &tmQ, bar(Q_FULL), 0, h * M + lb0 * kTile + r);
-            }
             for (int i = 0; i < nt; ++i) {
                 const int s = i % nstages;
                 if (!ptx::mbar_wait(bar(T_EMPTY + s), ((i / nstages) & 1) ^ 1, abort_flag, kErrBwdDq | 1)) break;
                 ptx::mbar_arrive_expect_tx(bar(T_FULL + s), 3 * G::TILE_BYTES);
-                uint8_t *dst = sT + (size_t)s * 3 * G::TILE_BYTES;
+                uint8_t *dst = smem + (size_t)s * 3 * G::TILE_BYTES;
                 ptx::tma_load_3d(ptx::smem_u32(dst), &tmK, bar(T_FULL + s), h * DR - off, (t_begin + i) * kTile, b);
                 ptx::tma_load_3d(ptx::smem_u32(dst + G::TILE_BYTES), &tmV, bar(T_FULL + s), h * DR - off, (t_begin + i) * kTile, b);
                 ptx::tma_load_3d(ptx::smem_u32(dst + 2 * G::TILE_BYTES), &tmG, bar(T_FULL + s), h * DR - off, (t_begin + i) * kTile, b);
             }
         }
-    } else if (warp < kFirstSoftmaxWarp) {
-        const int g = warp - kFirstIssuerWarp;
-        const int j = g >> 1, c = g & 1;
-        if (j < nslots && ptx::elect_one()) {
-            const uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0);
-            const uint32_t idescQ = ptx::instr_desc_bf16(128, D, 0, 1);
-            const uint64_t blk = (uint64_t)(alternate ? 0 : j * kTile * G::RB / 16);     // the slot's latent block
-            uint64_t ldesc[5];
+    } else if (warp == 3) {
+        // Column constants of every tile: -lse_dec, -dd, and the factor 2^(lse_dec - K) of W_enc (0 for a token that takes no part), or,
+        // in a tile with a token beyond kOneExpLog2, the addend of its own exponent.  The values come by asynchronous copies, kAhead
+        // tiles on their way at a time (with one tile's loads in flight this warp held the whole kernel back), and are
+        // turned into constants in place.
+        constexpr int AH = SM::kAhead, NW = kPair ? 2 : 1;
+        uint32_t masks[AH];                                     // mask bytes of this lane's four tokens
+        auto fetch = [&](int i) -> uint32_t {
+            float *cst = reinterpret_cast<float *>(smem + SM::cst_off + (i % SM::kCst) * SM::kCstBytes);
+            uint32_t mk = 0x01010101u;
 #pragma unroll
-            for (int i = 0; i < 5; ++i) ldesc[i] = ptx::smem_desc(ptx::smem_u32(smem + SM::lat_off(i)), 16, G::SBO, G::SWZ) + blk;
-            const uint32_t gcol = tm + j * SLOT_COLS + c * 2 * HALF;
-            const uint32_t dcol = gcol + 96;
-            bool ok = ptx::mbar_wait(bar(Q_FULL), 0, abort_flag, kErrBwdDq | 2);
-            const int jobs = (nq - j + nslots - 1) / nslots;
-            const int units = UPH * jobs;
-            // Order of issue, as in the encode kernel: the three tiles of units 0 and 1, then for every unit n its dQ
-            // MMAs as soon as its dS is handed over, then the tiles of unit n+2 into the buffer that dS has just left.
-            int t_s = alternate ? j : 0, t_v = t_s;                         // tiles of the next tile-unit / dQ-unit
-            const int t_step = alternate ? 2 : 1;
-            auto issue_tiles = [&](int n) -> bool {
-                const int s = t_s % nstages, w = n % UPH;
-                if (w == 0 && !ptx::mbar_wait(bar(T_FULL + s), (t_s / nstages) & 1, abort_flag, kErrBwdDq | 3)) return false;
-                ptx::tc_fence_after();
-                const uint32_t tbase = ptx::smem_u32(sT + (size_t)s * 3 * G::TILE_BYTES);
-                const uint64_t rowoff = (uint64_t)((c * HALF + w * UNIT) * G::RB / 16);   // the unit's 16 token rows
-                const uint64_t kdesc = ptx::smem_desc(tbase, 16, G::SBO, G::SWZ) + rowoff;
-                const uint64_t vdesc = ptx::smem_desc(tbase + G::TILE_BYTES, 16, G::SBO, G::SWZ) + rowoff;
-                const uint64_t gdesc = ptx::smem_desc(tbase + 2 * G::TILE_BYTES, 16, G::SBO, G::SWZ) + rowoff;
-                const uint32_t bcol = gcol + (n & 1) * 3 * UNIT;
-                // S = Q K^T | A = (Z_hi + Z_lo) dY^T | C = (dZ_hi + dZ_lo) V^T, each 128 latents x 16 tokens
+            for (int e = 0; e < kTile / 32; ++e) {
+                const int r = e * 32 + lane, n = min((t_begin + i) * kTile + r, a.N - 1);
+                const size_t nn = (size_t)b * a.N + n;
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) ptx::mma_ss(bcol, ldesc[0] + 2 * k, kdesc + 2 * k, idescS, k > 0);
+                for (int w = 0; w < NW; ++w) {
+                    ptx::copy_async4(ptx::smem_u32(cst + w * 3 * kTile + r), a.lse_dec + nn * a.H + h + w);
+                    ptx::copy_async4(ptx::smem_u32(cst + (w * 3 + 1) * kTile + r), a.dd + ((size_t)b * a.H + h + w) * a.N + n);
+                }
+                if (kPadded && a.key_mask != nullptr && a.key_mask[nn] == 0) mk &= ~(0xffu << (8 * e));
+            }
+            return mk;
+        };
+        bool ok = true;
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) ptx::mma_ss(bcol + UNIT, ldesc[1] + 2 * k, gdesc + 2 * k, idescS, k > 0);
+        for (int k = 0; k < AH; ++k) {
+            masks[k] = k < nt ? fetch(k) : 0u;
+            ptx::copy_async_commit();
+        }
+        for (int i0 = 0; ok && i0 < nt; i0 += AH) {
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) ptx::mma_ss(bcol + UNIT, ldesc[2] + 2 * k, gdesc + 2 * k, idescS, 1u);
+            for (int k = 0; k < AH; ++k) {
+                const int i = i0 + k;
+                if (i >= nt) break;
+                ptx::copy_async_wait<AH - 1>();
+                __syncwarp();
+                const int c = i % SM::kCst;
+                float *cst = reinterpret_cast<float *>(smem + SM::cst_off + c * SM::kCstBytes);
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) ptx::mma_ss(bcol + 2 * UNIT, ldesc[3] + 2 * k, vdesc + 2 * k, idescS, k > 0);
+                for (int w = 0; w < NW; ++w) {
+                    float ld[kTile / 32];
+                    bool part[kTile / 32], far = false;
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) ptx::mma_ss(bcol + 2 * UNIT, ldesc[4] + 2 * k, vdesc + 2 * k, idescS, 1u);
-                ptx::mma_commit(bar(S_FULL + 2 * g + (n & 1)));
-                if (w == UPH - 1) t_s += t_step;
+                    for (int e = 0; e < kTile / 32; ++e) {
+                        const int r = e * 32 + lane;
+                        const bool in = (t_begin + i) * kTile + r < a.N;
+                        ld[e] = in ? cst[w * 3 * kTile + r] * kBwdLog2e : INFINITY;
+                        part[e] = in && ((masks[k] >> (8 * e)) & 0xffu) != 0;
+                        cst[w * 3 * kTile + r] = -ld[e];
+                        cst[(w * 3 + 1) * kTile + r] = in ? -cst[(w * 3 + 1) * kTile + r] : 0.f;
+                        far = far || (part[e] && !(ld[e] - lse_min[w] <= kOneExpLog2));
+                    }
+                    far = __any_sync(0xffffffffu, far);
+#pragma unroll
+                    for (int e = 0; e < kTile / 32; ++e)
+                        cst[(w * 3 + 2) * kTile + e * 32 + lane] = far ? (part[e] ? 0.f : -INFINITY) : (part[e] ? ptx::ex2(ld[e] - lse_min[w]) : 0.f);
+                    if (lane == 0) two_exp[c * 2 + w] = far ? 1u : 0u;
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar(C_FULL + c));
+                const int next = i + AH;
+                if (next < nt) {
+                    if (!(ok = warp_wait(bar(C_EMPTY + next % SM::kCst), ((next / SM::kCst) & 1) ^ 1, abort_flag, kErrBwdDq | 7))) break;
+                    masks[k] = fetch(next);
+                }
+                ptx::copy_async_commit();
+            }
+        }
+        ptx::copy_async_wait<0>();
+    } else if (warp == 1) {
+        const int units = UPT * nt;
+        if (ptx::elect_one()) {
+            constexpr uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0), idescQ = ptx::instr_desc_bf16(128, DG, 0, 1);
+            // (descriptors as 32-bit low words beside a constant high word: see ptx::desc)
+            constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), TILE = G::TILE_BYTES >> 4, STEP16 = (16 * G::RB) >> 4, LAT = (kTile * G::RB) >> 4;
+            const uint32_t lat0 = ptx::desc_lo(ptx::smem_u32(smem + SM::lat_off(0)), 16), k0 = ptx::desc_lo(ptx::smem_u32(smem), 16);
+            constexpr uint32_t MN = ptx::desc_lo(0, G::SBO) - ptx::desc_lo(0, 16);          // K-major to MN-major
+            int s_stage = 0, s_wrap = 0, s_u = 0, o_stage = 0, o_u = 0;
+            // S = Q K^T | A = (Z_hi + Z_lo) dY^T | C = (dZ_hi + dZ_lo) V^T of the next unit, into buffer n & 1
+            auto tiles = [&](int n) -> bool {
+                if (s_u == 0) {
+                    if (!ptx::mbar_wait(bar(T_FULL + s_stage), (uint32_t)s_wrap, abort_flag, kErrBwdDq | 3)) return false;
+                    ptx::tc_fence_after();
+                }
+                uint32_t kd = k0 + (uint32_t)s_stage * 3 * TILE + (uint32_t)s_u * (UNIT / 16) * STEP16, ld = lat0;
+                ptx::opaque(kd);
+                ptx::opaque(ld);
+                const uint32_t bcol = tm + (n & 1) * kDqBuf;
+#pragma unroll
+                for (int w = 0; w < 5; ++w) {                   // Q with K; Z hi, lo with dY; dZ hi, lo with V
+                    const uint32_t col = bcol + (w == 0 ? 0 : w <= 2 ? UNIT : 2 * UNIT), td = kd + (w == 0 ? 0 : w <= 2 ? 2 * TILE : TILE);
+#pragma unroll
+                    for (int k = 0; k < DG / 16; ++k)
+                        ptx::mma_ss(col, ptx::desc(ld + w * LAT + 2 * k, HI), ptx::desc(td + 2 * k, HI), idescS, k > 0 || w == 2 || w == 4);
+                }
+                ptx::mma_commit(bar(S_FULL + (n & 1)));
+                if (++s_u == UPT) {
+                    s_u = 0;
+                    if (++s_stage == nstages) { s_stage = 0; s_wrap ^= 1; }
+                }
                 return true;
             };
-            for (int n = 0; ok && n < 2 && n < units; ++n) ok = issue_tiles(n);
+            bool ok = true;
+            for (int n = 0; ok && n < 2 && n < units; ++n) ok = tiles(n);
             for (int n = 0; ok && n < units; ++n) {
-                const int s = t_v % nstages, w = n % UPH;
-                if (!ptx::mbar_wait(bar(P_FULL + 2 * g + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdDq | 4)) { ok = false; break; }
+                // dQ_part += dS_unit K_unit (hi, then lo half of dS): 16 token rows of the K tile per k-step as the MN-major B operand
+                const uint32_t bcol = tm + (n & 1) * kDqBuf, acc = tm + kDqAcc + (n & (kAccs - 1)) * DG;
+                uint32_t kd = k0 + MN + (uint32_t)o_stage * 3 * TILE + (uint32_t)o_u * (UNIT / 16) * STEP16;
+                ptx::opaque(kd);
+                if (!ptx::mbar_wait(bar(P_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdDq | 4)) break;
                 ptx::tc_fence_after();
-                // dQ_part += dS_unit K_unit (hi, then lo half of dS): the unit's 16 token rows of the K tile as the
-                // MN-major B operand
-                const uint64_t kmn = ptx::smem_desc(ptx::smem_u32(sT + (size_t)s * 3 * G::TILE_BYTES), G::SBO, G::SBO, G::SWZ) +
-                                     (uint64_t)((c * HALF + w * UNIT) * G::RB / 16);
-                const uint32_t bcol = gcol + (n & 1) * 3 * UNIT;
-                ptx::mma_ts(dcol, bcol, kmn, idescQ, n > 0 ? 1u : 0u);
-                ptx::mma_ts(dcol, bcol + UNIT, kmn, idescQ, 1u);
-                if (w == UPH - 1) {
-                    ptx::mma_commit(bar(T_EMPTY + s));
-                    t_v += t_step;
+#pragma unroll
+                for (int k = 0; k < UNIT / 16; ++k) {
+                    ptx::mma_ts(acc, bcol + 16 * k, ptx::desc(kd + k * STEP16, HI), idescQ, (n >= kAccs || k > 0) ? 1u : 0u);
+                    ptx::mma_ts(acc, bcol + UNIT + 16 * k, ptx::desc(kd + k * STEP16, HI), idescQ, 1u);
                 }
-                if (n + 2 < units) ok = issue_tiles(n + 2);
+                if (++o_u == UPT) {
+                    ptx::mma_commit(bar(T_EMPTY + o_stage));
+                    o_u = 0;
+                    if (++o_stage == nstages) o_stage = 0;
+                }
+                if (n + 2 < units) ok = tiles(n + 2);
             }
-            if (ok) ptx::mma_commit(bar(ACC_DONE + g));
+            if (ok) ptx::mma_commit(bar(ACC_DONE));
         }
-    } else {
-        const int g = (warp - kFirstSoftmaxWarp) >> 2;
-        const int j = g >> 1, c = g & 1;
-        const int row = ((warp & 3) << 5) + lane;
-        const uint32_t lane_addr = (uint32_t)((warp & 3) << 5) << 16;
-        const uint32_t gcol = tm + lane_addr + j * SLOT_COLS + c * 2 * HALF;
-        const uint32_t abase = gcol + 96;
+    } else if (warp >= kDqFirstMathWarp) {
+        const int cg = (warp - kDqFirstMathWarp) >> 2;         // the group of 16 columns this warp works on
+        const int row = ((warp & 3) << 5) + lane;               // TMEM lane = latent within the block (or within the pair)
+        const int second = kPair ? row >> 6 : 0;                // the head of this lane's latent (uniform over the warp)
+        const uint32_t gcol = tm + ((uint32_t)((warp & 3) << 5) << 16);
         const float2 sl2p = make_float2(a.sl2, a.sl2);
-        const int lb = alternate ? 0 : lb0 + j;
-        const int m = lb * kTile + row;
+        const int m = kPair ? (row & 63) : lb * kTile + row;
         // this thread's latent: -lse_enc in log2 units (-inf for a latent that saw no valid token or lies beyond M), -de
-        float negle = -INFINITY, negde = 0.f;
-        if (j < nslots && m < M) {
-            const size_t r = ((size_t)b * a.H + h) * M + m;
+        float nle = -INFINITY, nde = 0.f;
+        if (m < M) {
+            const size_t r = ((size_t)b * a.H + h + second) * M + m;
             const float le = a.lse_enc[r];
-            negle = (le == -INFINITY) ? -INFINITY : -le * 1.4426950408889634f;
-            negde = -a.de[r];
+            nle = (le == -INFINITY) ? -INFINITY : -le * kBwdLog2e;
+            nde = -a.de[r];
         }
-        const float2 neglep = make_float2(negle, negle), negdep = make_float2(negde, negde);
-        // this warp's column constants for the 64 tokens of its half tile: -lse_dec (log2 units), then -dd
-        float *cst = reinterpret_cast<float *>(smem + SM::col_off()) + (warp - kFirstSoftmaxWarp) * 128;
-        int done = 0;
+        const float fr = ptx::ex2(nle + lse_min[second]);       // 2^(K - lse_enc)
+        const float2 nlep = make_float2(nle, nle), frp = make_float2(fr, fr), ndep = make_float2(nde, nde);
         bool ok = true;
-        // One unit: 16 token columns on buffer (done & 1).  wv: validity bits of the 16 tokens (kMasked only).
-        auto unit = [&](auto masked, int w, uint32_t wv) -> bool {
-            constexpr bool kMasked = decltype(masked)::value;
-            const int buf = done & 1;
-            const uint32_t bcol = gcol + buf * 3 * UNIT;
-            if (!warp_wait(bar(S_FULL + 2 * g + buf), (done >> 1) & 1, abort_flag, kErrBwdDq | 5)) return false;
-            ptx::tc_fence_after();
-            // 8 tokens at a time: their dS goes back as two bf16 halves over columns the thread has already read
-            // (hi over S, lo over A: 4 packed columns per 8 tokens)
+        int n = 0;
+        for (int tile = 0; ok && tile < nt; ++tile) {
+            const int c = tile % SM::kCst;
+            const float *cst = reinterpret_cast<const float *>(smem + SM::cst_off + c * SM::kCstBytes) + second * 3 * kTile + cg * 16;
+            if (!(ok = warp_wait(bar(C_FULL + c), (tile / SM::kCst) & 1, abort_flag, kErrBwdDq | 8))) break;
+            auto units = [&](auto two) {
+                constexpr bool kTwo = decltype(two)::value;
+#pragma unroll 1
+                for (int u = 0; u < UPT; ++u, ++n, cst += UNIT) {
+                    const uint32_t bcol = gcol + (n & 1) * kDqBuf + cg * 16;
+                    if (!(ok = warp_wait(bar(S_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdDq | 5))) break;
+                    ptx::tc_fence_after();
+                    uint32_t s[2][8], av[2][8], cv[2][8];
+                    auto load = [&](int q) {
+                        ptx::tmem_ld8(bcol + q * 8, s[q]);
+                        ptx::tmem_ld8(bcol + UNIT + q * 8, av[q]);
+                        ptx::tmem_ld8(bcol + 2 * UNIT + q * 8, cv[q]);
+                    };
+                    load(0);
 #pragma unroll
-            for (int qd = 0; qd < 2; ++qd) {
-                uint32_t s[8], av[8], cv[8], pk[4], pl[4];
-                ptx::tmem_ld8(bcol + qd * 8, s);
-                ptx::tmem_ld8(bcol + UNIT + qd * 8, av);
-                ptx::tmem_ld8(bcol + 2 * UNIT + qd * 8, cv);
-                ptx::tmem_wait_ld();
+                    for (int q = 0; q < 2; ++q) {                  // eight columns at a time, the other eight on their way meanwhile
+                        ptx::tmem_wait_ld();
+                        if (q == 0) load(1);
+                        uint32_t hi[4], lo[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int col = qd * 8 + 2 * k;
-                    const float2 sp = make_float2(__uint_as_float(s[2 * k]), __uint_as_float(s[2 * k + 1]));
-                    const float2 nld = *reinterpret_cast<const float2 *>(cst + w * UNIT + col);
-                    const float2 ndd = *reinterpret_cast<const float2 *>(cst + HALF + w * UNIT + col);
-                    const float2 xd = __ffma2_rn(sp, sl2p, nld), xe = __ffma2_rn(sp, sl2p, neglep);
-                    const float2 pd = make_float2(ptx::ex2(xd.x), ptx::ex2(xd.y));
-                    float2 pe = make_float2(ptx::ex2(xe.x), ptx::ex2(xe.y));
-                    if (kMasked) {
-                        if (!((wv >> col) & 1)) pe.x = 0.f;
-                        if (!((wv >> (col + 1)) & 1)) pe.y = 0.f;
+                        for (int k = 0; k < 4; k += 2) {
+                            const float4 nld = *reinterpret_cast<const float4 *>(cst + q * 8 + 2 * k);
+                            const float4 ndd = *reinterpret_cast<const float4 *>(cst + kTile + q * 8 + 2 * k);
+                            const float4 fc = *reinterpret_cast<const float4 *>(cst + 2 * kTile + q * 8 + 2 * k);
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const int j = 2 * (k + e);
+                                const DsPair r = ds_pair<false, kTwo>(
+                                    make_float2(__uint_as_float(s[q][j]), __uint_as_float(s[q][j + 1])),
+                                    make_float2(__uint_as_float(av[q][j]), __uint_as_float(av[q][j + 1])),
+                                    make_float2(__uint_as_float(cv[q][j]), __uint_as_float(cv[q][j + 1])), sl2p,
+                                    e ? make_float2(nld.z, nld.w) : make_float2(nld.x, nld.y), e ? make_float2(ndd.z, ndd.w) : make_float2(ndd.x, ndd.y),
+                                    ndep, kTwo ? nlep : frp, e ? make_float2(fc.z, fc.w) : make_float2(fc.x, fc.y));
+                                hi[k + e] = r.hi;
+                                lo[k + e] = r.lo;
+                            }
+                        }
+                        // over columns this warp has read, 8 packed columns per 16 tokens: hi over S, lo over A
+                        ptx::tmem_st4(bcol + q * 4, hi);
+                        ptx::tmem_st4(bcol + UNIT + q * 4, lo);
                     }
-                    const float2 u = __fadd2_rn(make_float2(__uint_as_float(av[2 * k]), __uint_as_float(av[2 * k + 1])), ndd);
-                    const float2 v = __fadd2_rn(make_float2(__uint_as_float(cv[2 * k]), __uint_as_float(cv[2 * k + 1])), negdep);
-                    const float2 ds = __ffma2_rn(pd, u, __fmul2_rn(pe, v));
-                    const uint32_t hi = ptx::pack_bf16(ds.x, ds.y);
-                    pk[k] = hi;
-                    pl[k] = ptx::pack_bf16(ds.x - __uint_as_float(hi << 16), ds.y - __uint_as_float(hi & 0xffff0000u));
-                }
-                ptx::tmem_st4(bcol + qd * 4, pk);
-                ptx::tmem_st4(bcol + UNIT + qd * 4, pl);
-            }
-            ptx::tmem_wait_st();
-            ptx::tc_fence_before();
-            ptx::mbar_arrive(bar(P_FULL + 2 * g + buf));
-            ++done;
-            return true;
-        };
-        if (j < nslots) {
-            // the constants of a tile are fetched one tile ahead (two tokens per lane) and parked, as loaded, in
-            // registers: nothing waits for the loads until the next tile begins
-            float f_ld[2], f_dd[2];
-            uint32_t f_ok[2];
-            auto fetch = [&](int t) {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int n = t * kTile + c * HALF + e * 32 + lane;
-                    const bool in = n < a.N;
-                    const size_t i = ((size_t)b * a.N + (in ? n : 0)) * a.H + h;
-                    f_ld[e] = a.lse_dec[i];
-                    f_dd[e] = a.dd[((size_t)b * a.H + h) * a.N + (in ? n : 0)];
-                    f_ok[e] = a.key_mask == nullptr ? 1u : (uint32_t)a.key_mask[(size_t)b * a.N + (in ? n : 0)];
+                    ptx::tmem_wait_st();
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(bar(P_FULL + (n & 1)));
                 }
             };
-            if (j < nq) fetch(t_begin + (alternate ? j : j / nslots));
-            for (int q = j; ok && q < nq; q += nslots) {
-                const int t = t_begin + (alternate ? q : q / nslots);
-                const bool plain = a.key_mask == nullptr && (t + 1) * kTile <= a.N;
-                __syncwarp();                                               // the previous tile's reads are done
-                bool v01[2];
+            if (two_exp[c * 2 + second] == 0) units(std::false_type{});
+            else units(std::true_type{});
+            if (lane == 0) ptx::mbar_arrive(bar(C_EMPTY + c));
+        }
+        if (cg == 0) {
+            if (ok) ok = warp_wait(bar(ACC_DONE), 0, abort_flag, kErrBwdDq | 6);
+            ptx::tc_fence_after();
+            float acc[D];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const bool in = t * kTile + c * HALF + e * 32 + lane < a.N;
-                    cst[e * 32 + lane] = in ? -f_ld[e] * 1.4426950408889634f : -INFINITY;
-                    cst[HALF + e * 32 + lane] = in ? -f_dd[e] : 0.f;
-                    v01[e] = in && f_ok[e] != 0;
-                }
-                const uint32_t wv0 = __ballot_sync(0xffffffffu, v01[0]), wv1 = __ballot_sync(0xffffffffu, v01[1]);
-                __syncwarp();
-                if (q + nslots < nq) fetch(t_begin + (alternate ? q + nslots : (q + nslots) / nslots));
+            for (int k = 0; k < D; ++k) acc[k] = 0.f;
 #pragma unroll 1
-                for (int w = 0; ok && w < UPH; ++w) {
-                    const uint32_t wv = ((w < 2 ? wv0 : wv1) >> ((w & 1) * UNIT)) & 0xffffu;
-                    if (kPadded && !plain) ok = unit(std::true_type{}, w, wv);
-                    else ok = unit(std::false_type{}, w, wv);
+            for (int i = 0; i < min(kAccs, UPT * nt); ++i) {
+#pragma unroll
+                for (int dc = 0; dc < D / 16; ++dc) {
+                    uint32_t r[16];
+                    ptx::tmem_ld16(gcol + kDqAcc + i * DG + second * D + dc * 16, r);
+                    ptx::tmem_wait_ld();
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) acc[dc * 16 + k] += __uint_as_float(r[k]);
                 }
             }
-        }
-        if (ok && j < nslots) ok = warp_wait(bar(ACC_DONE + g), 0, abort_flag, kErrBwdDq | 6);
-        ptx::tc_fence_after();
-        uint32_t acc[D];
-        if (done > 0) {
+            if (ok && m < M) {
+                const long rows = (long)a.B * a.H * M;
+                float4 *dst = reinterpret_cast<float4 *>(a.part + ((size_t)split * rows + ((size_t)b * a.H + h + second) * M + m) * DR);
+                if (DR == 4) {
+                    dst[0] = make_float4(off ? acc[4] : acc[0], off ? acc[5] : acc[1], off ? acc[6] : acc[2], off ? acc[7] : acc[3]);
+                } else {
 #pragma unroll
-            for (int dc = 0; dc < D / 16; ++dc) ptx::tmem_ld16(abase + dc * 16, acc + dc * 16);
-            ptx::tmem_wait_ld();
-        } else {
-#pragma unroll
-            for (int k = 0; k < D; ++k) acc[k] = 0u;
-        }
-        if (ok && j < nslots && m < M) {
-            const long rows = (long)a.B * a.H * M;
-            const int part = split * a.partials_per_split + (alternate ? 2 * j + c : c);
-            float4 *dst = reinterpret_cast<float4 *>(a.part + ((size_t)part * rows + ((size_t)b * a.H + h) * M + m) * DR);
-            if (DR == 4) {
-                dst[0] = make_float4(__uint_as_float(off ? acc[4] : acc[0]), __uint_as_float(off ? acc[5] : acc[1]),
-                                     __uint_as_float(off ? acc[6] : acc[2]), __uint_as_float(off ? acc[7] : acc[3]));
-            } else {
-#pragma unroll
-                for (int dc = 0; dc < DR / 4; ++dc)
-                    dst[dc] = make_float4(__uint_as_float(acc[4 * dc]), __uint_as_float(acc[4 * dc + 1]),
-                                          __uint_as_float(acc[4 * dc + 2]), __uint_as_float(acc[4 * dc + 3]));
+                    for (int dc = 0; dc < DR / 4; ++dc) dst[dc] = make_float4(acc[4 * dc], acc[4 * dc + 1], acc[4 * dc + 2], acc[4 * dc + 3]);
+                }
             }
         }
     }
     ptx::tc_fence_before();
     __syncthreads();
-    if (warp == kFirstIssuerWarp) {
+    if (warp == 1) {
         ptx::tc_fence_after();
-        ptx::tmem_dealloc(tm, NCOLS);
+        ptx::tmem_dealloc(tm, 512);
     }
     if (threadIdx.x == 0 && *abort_flag != 0 && a.status != nullptr) atomicCAS(a.status, 0u, *abort_flag);
 }
 
 // ------------------------------------------------------------------------------- pass B, token side (dK, dV)
-// Tokens on the 128 TMEM lanes, latents on columns in units of kUnit, every softmax group a token tile of its
-// own.  Two sweeps over the latents of a tile, as in the CUDA-core kernel: the first needs S^T = K Q^T and
-// A^T = dY Z^T and leaves dd[n] = sum_m W_dec[n,m] A[n,m] in a register; the second adds C^T = V dZ^T, turns the
-// three into dS^T and W_enc^T (two bf16 halves each) over the columns just read, and two more contractions
-// accumulate dK_n = scale * sum_m dS[m,n] q_m and dV_n = sum_m W_enc[m,n] dZ_m.  dd goes to the workspace for
-// the dQ kernel.  Columns of a group: S, A, C (kUnit each), dK (D), dV (D): 3 kUnit + 2 D <= 128.
-template <int D>
-struct BwdTokGeom {
-    static constexpr int kUnit = D == 16 ? 32 : 16;
-    static constexpr int kMaxStages = 8;
+// Tokens on the lanes, latents on the columns.  Two sweeps over the latents of a tile: the first needs S^T = K Q^T and
+// A^T = dY Z^T and leaves dd[n] = sum_m W_dec[n,m] A[n,m]; the second adds C^T = V dZ^T, turns the three into dS^T and W_enc^T and
+// accumulates dK_n = sum_m dS[m,n] q_m and dV_n = sum_m W_enc[m,n] dZ_m.  dd goes to the workspace for the dQ kernel.
+
+// A unit is 32 latents wide, and a CTA is a few independent groups of four warps (one per quarter of the lanes; a thread works on all 32
+// columns of its lane), each with a tile of its own, one buffer S | A | C and its own accumulators: while one group waits for the tensor
+// core the others work, nothing is shared between them, and dd needs no exchange.  There is no issuing warp: the warps of a group
+// take turns issuing the output contractions of a unit, the tiles of the next and one commit, which says that all of them are done.
+// Measured, us, on the shapes named at the dQ kernel, against units of 16 columns, two exponentials per pair and half as many latents per
+// launch: 22.4, 164, 1166, 9254 -> 19.9, 132, 1016, 8936; D = 64: 1049 (CUDA cores) -> 67.  Units of 64 columns shared by sixteen warps, as
+// in the dQ kernel: 39.6, 254, 1154, 16489; 71 (W_enc doubles what a thread holds: it spills).  Bound by issue slots, some 26
+// instructions per pair over both sweeps.
+// Groups of four warps, by accumulator columns: as many as 512 columns of tensor memory hold, at most four.  Warps: 0 TMA producer, from 2
+// on the groups (warp & 3 = the quarter of the lanes a warp can reach).  18, 14 or 10 warps: 96, 128 or 168 registers each.
+constexpr int kUnit = 32, kUnitCols = 3 * kUnit, kBwdFirstMathWarp = 2;
+template <int kAccCols> struct BwdGroups {
+    static constexpr int fit = 512 / (kUnitCols + kAccCols), n = fit > 4 ? 4 : fit, cols = (512 / n) & ~31;   // (whole blocks of 32 columns)
+    static_assert(kUnitCols + kAccCols <= cols, "tensor memory");
+    static constexpr int kThreads = (kBwdFirstMathWarp + 4 * n) * 32;
 };
 
+// Hand-over of a group's unit n: every warp arrives on the group's barrier `full` (count 4); one of them, taking turns, waits for the others
+// and returns true: it then may issue instructions that depend on what all four wrote to (or have read from) tensor memory.
+// (A counter whose last incrementer issues would need no wait, but the acquiring read-modify-write costs every warp 250 to 400 cycles.)
+__device__ __forceinline__ bool hand_over(uint32_t full, uint32_t n, volatile uint32_t *abort_flag, uint32_t code) {
+    ptx::tc_fence_before();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(full);
+    if (((threadIdx.x >> 5) & 3) != (n & 3)) return false;
+    const bool ok = warp_wait(full, n & 1, abort_flag, code);
+    ptx::tc_fence_after();
+    return ok;
+}
 struct BwdTokTcArgs {
-    const __nv_bfloat16 *Q;    // [H,M,D] (read directly in the half-width form)
+    const __nv_bfloat16 *Q;    // [H,M,D]
     const float *Z, *dZ;       // [B,H,M,D]
     const float *lse_enc, *de; // [B,H,M]
     const float *lse_dec;      // [B,N,H]
@@ -422,119 +540,95 @@ struct BwdTokTcArgs {
 template <int D>
 struct BwdTokSmem {
     using G = TileGeom<D>;
-    __host__ __device__ static int padded_m(int M) { return (M + 31) & ~31; }
-    // tiles: [stage][K | V | dY]; latents: Q, Z_hi, Z_lo, dZ_hi, dZ_lo with padded_m rows each; then -lse_enc, -de
+    // tiles: [stage][K | V | dY]; latents: Q, Z_hi, Z_lo, dZ_hi, dZ_lo with M rows each (M a multiple of 16); their constants
     __host__ __device__ static size_t lat_off(int stages, int M, int which) {
-        return (size_t)stages * 3 * G::TILE_BYTES + (size_t)which * padded_m(M) * G::RB;
+        return (size_t)stages * 3 * G::TILE_BYTES + (size_t)which * M * G::RB;
     }
     __host__ __device__ static size_t cst_off(int stages, int M) { return lat_off(stages, M, 5); }
-    __host__ __device__ static size_t bar_off(int stages, int M) { return cst_off(stages, M) + 2 * sizeof(float) * padded_m(M); }
+    __host__ __device__ static size_t bar_off(int stages, int M) { return cst_off(stages, M) + 3 * sizeof(float) * M; }
     __host__ __device__ static size_t total(int stages, int M) {
-        size_t t = bar_off(stages, M) + 512 + 1024;
+        const size_t t = bar_off(stages, M) + 512 + 1024;
         return t < kTcMinSmem ? kTcMinSmem : t;
     }
+    static constexpr int kMaxStages = 8;
     // the most stages (at most kMaxStages) that fit beside the latent operands; 0 if not even one does
     __host__ static int stages(int M) {
-        int s = BwdTokGeom<D>::kMaxStages;
+        int s = kMaxStages;
         while (s > 0 && total(s, M) > (size_t)227 * 1024) --s;
         return s;
     }
 };
 
-// grid = (CTAs per head, H, B); a CTA takes the token tiles blockIdx.x, blockIdx.x + gridDim.x, ...
-// DRT = 8 or 4 (with D = 16): the narrow form (head DRT wide in memory; only the head's columns of the rows of dK
-// and dV are kept).
-// kM: 0, or the number of latents of the launch as a compile-time constant.
-// kPadded: as in the dQ kernel.
-template <int D, int DRT = 0, int kMode = 0, int kM = 0, bool kPadded = true>
-__global__ void __launch_bounds__(kTcThreads, 1)
+// grid = (CTAs per head, H, B); a CTA takes the token tiles blockIdx.x, blockIdx.x + gridDim.x, ..., its groups a tile each in turn.
+// A tile's rows of dK and dV are read from the accumulators after the first sweep of the group's next tile, when the contractions
+// that complete them are long done.  DRT, kPadded: as in the dQ kernel.
+template <int D, int DRT, int kMode, bool kPadded>
+__global__ void __launch_bounds__(BwdGroups<2 * D>::kThreads, 1)
 bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
-                    const __grid_constant__ CUtensorMap tmG, const __grid_constant__ CUtensorMap tmQ, BwdTokTcArgs a) {
+                    const __grid_constant__ CUtensorMap tmG, BwdTokTcArgs a) {
     using G = TileGeom<D>;
     using SM = BwdTokSmem<D>;
-    constexpr int UNIT = BwdTokGeom<D>::kUnit;
-    constexpr int kMaxSt = BwdTokGeom<D>::kMaxStages;
-    constexpr bool kHalf = DRT != 0;
-    constexpr int DR = kHalf ? DRT : D;                         // head width in memory
+    using BG = BwdGroups<2 * D>;
+    constexpr int UNIT = kUnit, NG = BG::n, kThreads = BG::kThreads, kMaxSt = SM::kMaxStages, DR = DRT ? DRT : D;
+    // dV = W_hi (dZ_hi + dZ_lo) + W_lo dZ_hi: with room for 2 D columns W_hi meets [dZ_hi | dZ_lo] in one MMA
+    constexpr bool kWideV = kUnitCols + 3 * D <= BG::cols;
+    constexpr int K_COL = kUnitCols, V_COL = K_COL + D;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const int M = kM ? kM : a.M, MU = SM::padded_m(M), stages = a.stages;
-    uint8_t *sQ = smem + SM::lat_off(stages, M, 0);
-    float *cst = reinterpret_cast<float *>(smem + SM::cst_off(stages, M));      // [MU] -lse_enc (log2 units), [MU] -de
+    const int M = a.M, stages = a.stages;
+    float *cst = reinterpret_cast<float *>(smem + SM::cst_off(stages, M));      // [M] -lse_enc (log2 units), [M] -de, [M] 2^(K - lse_enc)
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off(stages, M));
-    constexpr int NG = kSoftmaxGroups;
-    enum { T_FULL = 0, T_EMPTY = T_FULL + kMaxSt, S_FULL = T_EMPTY + kMaxSt, P_FULL = S_FULL + NG,
-           ACC_FULL = P_FULL + NG, ACC_FREE = ACC_FULL + NG, Q_FULL = ACC_FREE + NG, NBARS };
+    enum { T_FULL = 0, T_EMPTY = T_FULL + kMaxSt, S_FULL = T_EMPTY + kMaxSt, P_FULL = S_FULL + NG, NBARS = P_FULL + NG };
+    static_assert(NBARS * 8 + 32 <= 512, "barrier area too small");
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NBARS);
     volatile uint32_t *abort_flag = tmem_slot + 1;
+    float *kmin = reinterpret_cast<float *>(tmem_slot + 2);     // smallest lse_enc of the launch's latents
 
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int h = blockIdx.y, b = blockIdx.z;
     const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
-    const int ng = stages < NG ? stages : NG;                   // groups at work
-    const int nu = (M + UNIT - 1) / UNIT;                       // latent units per sweep
-    constexpr uint32_t NCOLS = 512;
+    const int nu = (M + UNIT - 1) / UNIT;                       // latent units per sweep; the last may have 16 columns
+    const int off = DRT ? narrow_offset(h, DR) : 0;
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < NBARS; ++i)
-            ptx::mbar_init(bar(i), ((i >= P_FULL && i < P_FULL + NG) || (i >= ACC_FREE && i < ACC_FREE + NG)) ? 128u : 1u);
+        for (int i = 0; i < NBARS; ++i) ptx::mbar_init(bar(i), i >= P_FULL ? 4 : 1);
         *abort_flag = 0;
         ptx::fence_mbar_init();
         ptx::prefetch_tensormap(&tmK);
         ptx::prefetch_tensormap(&tmV);
         ptx::prefetch_tensormap(&tmG);
-        ptx::prefetch_tensormap(&tmQ);
     }
-    if (warp == kFirstIssuerWarp) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), NCOLS);
-    // latent rows M..MU-1 of all five operands are zero; their columns carry -lse_enc = -inf
-    const int zfirst = kHalf ? 0 : M;                           // half-width form: every row, whose upper half stays zero
-    for (int i = threadIdx.x; i < 5 * (MU - zfirst) * (G::RB / 16); i += kTcThreads) {
-        const int which = i / ((MU - zfirst) * (G::RB / 16)), rem = i % ((MU - zfirst) * (G::RB / 16));
-        reinterpret_cast<uint4 *>(smem + SM::lat_off(stages, M, which) + (size_t)zfirst * G::RB)[rem] = make_uint4(0, 0, 0, 0);
-    }
-    const int off = kHalf ? narrow_offset(h, DR) : 0;           // the head's first column within a token tile row
-    if (kHalf) {
-        __syncthreads();
-        if constexpr (DR == 4) {
-            const size_t r0 = ((size_t)b * a.H + h) * a.mtot + a.m0;
-            stage_rows4<D>(sQ, a.Q + ((size_t)h * a.mtot + a.m0) * DR, M, off);
-            stage_rows4_hilo<D>(smem + SM::lat_off(stages, M, 1), smem + SM::lat_off(stages, M, 2), a.Z + r0 * DR, M, off);
-            stage_rows4_hilo<D>(smem + SM::lat_off(stages, M, 3), smem + SM::lat_off(stages, M, 4), a.dZ + r0 * DR, M, off);
-        } else {
-            for (int i = threadIdx.x; i < M * (DR / 8); i += kTcThreads) {
-                const int m = i / (DR / 8), ch = i % (DR / 8);
-                *reinterpret_cast<uint4 *>(sQ + (size_t)m * G::RB + ((ch ^ G::swz(m)) << 4)) =
-                    *reinterpret_cast<const uint4 *>(a.Q + ((size_t)h * a.mtot + a.m0 + m) * DR + ch * 8);
-            }
+    if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
+    {
+        const size_t q0 = (size_t)h * a.mtot + a.m0, r0 = ((size_t)b * a.H + h) * a.mtot + a.m0;
+        if (warp == 2) {
+            const float k = warp_lse_min(a.lse_enc + r0, M);
+            if (lane == 0) *kmin = k;
         }
-    }
-    for (int m = threadIdx.x; m < MU; m += kTcThreads) {
-        float nle = -INFINITY, nde = 0.f;
-        if (m < M) {
-            const size_t r = ((size_t)b * a.H + h) * a.mtot + a.m0 + m;
-            const float le = a.lse_enc[r];
-            nle = (le == -INFINITY) ? -INFINITY : -le * 1.4426950408889634f;
-            nde = -a.de[r];
-        }
-        cst[m] = nle;
-        cst[MU + m] = nde;
-    }
-    constexpr int ZC = DR >= 8 ? DR / 8 : 1;                    // 8-float chunks per row (none for DR = 4: staged above)
-    for (int i = threadIdx.x; i < (DR >= 8 ? 2 * M * ZC : 0); i += kTcThreads) {
-        const int which = i / (M * ZC), rem = i % (M * ZC), m = rem / ZC, ch = rem % ZC;
-        const float *src = (which == 0 ? a.Z : a.dZ) + (((size_t)b * a.H + h) * a.mtot + a.m0 + m) * DR + ch * 8;
-        const float4 lo4 = *reinterpret_cast<const float4 *>(src), hi4 = *reinterpret_cast<const float4 *>(src + 4);
-        const float z[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
-        uint32_t vh[4], vl[4];
+        uint8_t *lat[5];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            vh[k] = ptx::pack_bf16(z[2 * k], z[2 * k + 1]);
-            vl[k] = ptx::pack_bf16(z[2 * k] - __uint_as_float(vh[k] << 16), z[2 * k + 1] - __uint_as_float(vh[k] & 0xffff0000u));
+        for (int w = 0; w < 5; ++w) lat[w] = smem + SM::lat_off(stages, M, w);
+        if (DRT != 0) {                                         // narrow form: the other columns of every row stay zero
+            for (int i = threadIdx.x; i < 5 * M * (G::RB / 16); i += kThreads) reinterpret_cast<uint4 *>(lat[0])[i] = make_uint4(0, 0, 0, 0);
+            __syncthreads();
         }
-        const size_t off = (size_t)m * G::RB + ((ch ^ G::swz(m)) << 4);
-        *reinterpret_cast<uint4 *>(smem + SM::lat_off(stages, M, 1 + 2 * which) + off) = make_uint4(vh[0], vh[1], vh[2], vh[3]);
-        *reinterpret_cast<uint4 *>(smem + SM::lat_off(stages, M, 2 + 2 * which) + off) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
+        if constexpr (DR == 4) {
+            stage_rows4<D>(lat[0], a.Q + q0 * DR, M, off);
+            stage_rows4_hilo<D>(lat[1], lat[2], a.Z + r0 * DR, M, off);
+            stage_rows4_hilo<D>(lat[3], lat[4], a.dZ + r0 * DR, M, off);
+        } else {
+            stage_bf16<D, DR>(lat[0], a.Q + q0 * DR, M, 0, 0, threadIdx.x, kThreads);
+            stage_hilo<D, DR>(lat[1], lat[2], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads);
+            stage_hilo<D, DR>(lat[3], lat[4], a.dZ + r0 * DR, M, 0, 0, threadIdx.x, kThreads);
+        }
+        __syncthreads();
+        for (int m = threadIdx.x; m < M; m += kThreads) {
+            const float le = a.lse_enc[r0 + m], nle = (le == -INFINITY) ? -INFINITY : -le * kBwdLog2e;
+            cst[m] = nle;
+            cst[M + m] = -a.de[r0 + m];
+            cst[2 * M + m] = ptx::ex2(nle + *kmin);
+        }
     }
     ptx::fence_proxy_async_smem();
     ptx::tc_fence_before();
@@ -544,13 +638,6 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
     if (warp == 0) {
         if (ptx::elect_one()) {
-            if (kHalf) {
-                ptx::mbar_arrive(bar(Q_FULL));                  // Q was written by the threads before the block barrier
-            } else {
-                ptx::mbar_arrive_expect_tx(bar(Q_FULL), (uint32_t)(M * G::RB));
-                for (int r = 0; r < M; r += 16)
-                    ptx::tma_load_2d(ptx::smem_u32(sQ + (size_t)r * G::RB), &tmQ, bar(Q_FULL), 0, h * a.mtot + a.m0 + r);
-            }
             for (int i = 0; i < nt; ++i) {
                 const int s = i % stages, t = blockIdx.x + i * gridDim.x;
                 if (!ptx::mbar_wait(bar(T_EMPTY + s), ((i / stages) & 1) ^ 1, abort_flag, kErrBwdTok | 1)) break;
@@ -561,268 +648,283 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 ptx::tma_load_3d(ptx::smem_u32(dst + 2 * G::TILE_BYTES), &tmG, bar(T_FULL + s), h * DR - off, t * kTile, b);
             }
         }
-    } else if (warp < kFirstSoftmaxWarp) {
-        const int g = warp - kFirstIssuerWarp;
-        if (g < ng && ptx::elect_one()) {
-            const uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0);
-            const uint32_t idescO = ptx::instr_desc_bf16(128, D, 0, 1);
-            const uint32_t gcol = tm + g * 128;
-            const uint32_t kcol = gcol + 3 * UNIT, vcol = kcol + D;       // the dK and dV accumulators
-            bool ok = ptx::mbar_wait(bar(Q_FULL), 0, abort_flag, kErrBwdTok | 2);
-            uint32_t cnt = 0;
-            int k_tile = 0;
-            for (int i = g; ok && i < nt; i += ng, ++k_tile) {
-                const int s = i % stages;
-                if (!ptx::mbar_wait(bar(T_FULL + s), (i / stages) & 1, abort_flag, kErrBwdTok | 3)) break;
-                ptx::tc_fence_after();
-                const uint32_t tbase = ptx::smem_u32(smem + (size_t)s * 3 * G::TILE_BYTES);
-                // the tile's token rows as the K-major A operand of the three score-like contractions
-                const uint64_t kdesc = ptx::smem_desc(tbase, 16, G::SBO, G::SWZ);
-                const uint64_t vdesc = ptx::smem_desc(tbase + G::TILE_BYTES, 16, G::SBO, G::SWZ);
-                const uint64_t gdesc = ptx::smem_desc(tbase + 2 * G::TILE_BYTES, 16, G::SBO, G::SWZ);
-                for (int sweep = (kMode == 2 ? 1 : 0); ok && sweep < (kMode == 1 ? 1 : 2); ++sweep) {
-                    for (int u = 0; u < nu; ++u) {
-                        const uint64_t uoff = (uint64_t)(u * UNIT * G::RB / 16);      // the unit's latent rows
-                        uint64_t ld[5];
+    } else if (warp >= kBwdFirstMathWarp) {
+        const int g = (warp - kBwdFirstMathWarp) >> 2;
+        const int row = ((warp & 3) << 5) + lane;               // TMEM lane = token within the tile
+        const uint32_t base = tm + g * BG::cols;                // the group's columns: S | A | C | dK | dV
+        const uint32_t gcol = base + ((uint32_t)((warp & 3) << 5) << 16);
+        const float2 sl2p = make_float2(a.sl2, a.sl2);
+        const float lse_min = *kmin;
+        const uint32_t pfull = bar(P_FULL + g), sfull = bar(S_FULL + g);
+        const int wlast = M - (nu - 1) * UNIT;                  // latents of the last unit
+        // (descriptors as 32-bit low words beside a constant high word: see ptx::desc)
+        constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), TILE = G::TILE_BYTES >> 4, STEP16 = (16 * G::RB) >> 4;
+        constexpr uint32_t MN = ptx::desc_lo(0, G::SBO) - ptx::desc_lo(0, 16);          // K-major to MN-major
+        const uint32_t LAT = (uint32_t)(M * G::RB) >> 4;        // from one latent operand to the next
+        auto lat_desc = [&](int u) {                            // low word of Q's rows of unit u
+            uint32_t d = ptx::desc_lo(ptx::smem_u32(smem + SM::lat_off(stages, M, 0)), 16) + (uint32_t)u * (UNIT / 16) * STEP16;
+            ptx::opaque(d);
+            return d;
+        };
+        // by one thread: S^T = K Q^T | A^T = dY (Z_hi + Z_lo)^T and (kSecond) C^T = V (dZ_hi + dZ_lo)^T of unit u of the tile in `stage`
+        auto issue_tiles = [&](auto second, int stage, int u) {
+            constexpr bool kSecond = decltype(second)::value;
+            const uint32_t idescS = ptx::instr_desc_bf16(128, u == nu - 1 ? wlast : UNIT, 0, 0);
+            uint32_t td = ptx::desc_lo(ptx::smem_u32(smem), 16) + (uint32_t)stage * 3 * TILE, ld = lat_desc(u);
+            ptx::opaque(td);
 #pragma unroll
-                        for (int w = 0; w < 5; ++w)
-                            ld[w] = ptx::smem_desc(ptx::smem_u32(smem + SM::lat_off(stages, M, w)), 16, G::SBO, G::SWZ) + uoff;
+            for (int w = 0; w < (kSecond ? 5 : 3); ++w) {       // K with Q; dY with Z hi, lo; V with dZ hi, lo
+                const uint32_t col = base + (w == 0 ? 0 : w <= 2 ? UNIT : 2 * UNIT), ad = td + (w == 0 ? 0 : w <= 2 ? 2 * TILE : TILE);
 #pragma unroll
-                        for (int k = 0; k < D / 16; ++k) ptx::mma_ss(gcol, kdesc + 2 * k, ld[0] + 2 * k, idescS, k > 0);
+                for (int k = 0; k < D / 16; ++k)
+                    ptx::mma_ss(col, ptx::desc(ad + 2 * k, HI), ptx::desc(ld + 2 * k, HI), idescS, k > 0 || w == 2 || w == 4);
+                ld += LAT;
+            }
+        };
+        // by one thread: dK += dS Q_unit, dV += W_enc dZ_unit
+        auto issue_outputs = [&](int u) {
+            constexpr uint32_t idescO = ptx::instr_desc_bf16(128, D, 0, 1), idescW = ptx::instr_desc_bf16(128, kWideV ? 2 * D : D, 0, 1);
+            const uint32_t ld = lat_desc(u);
+            // (wide form: dZ_hi's next block along N is dZ_lo, M rows further on)
+            const uint32_t qd = ld + MN, zd = ld + 3 * LAT + (kWideV ? (LAT << 16) - ptx::desc_lo(0, 16) : MN), zl = ld + 4 * LAT + MN;
 #pragma unroll
-                        for (int k = 0; k < D / 16; ++k) ptx::mma_ss(gcol + UNIT, gdesc + 2 * k, ld[1] + 2 * k, idescS, k > 0);
+            for (int k = 0; k < UNIT / 16; ++k) {
+                if (k > 0 && u == nu - 1 && 16 * k >= wlast) break;
+                const uint32_t acc = (u > 0 || k > 0) ? 1u : 0u;
+                ptx::mma_ts(base + K_COL, base + 16 * k, ptx::desc(qd + k * STEP16, HI), idescO, acc);                    // dS hi
+                ptx::mma_ts(base + K_COL, base + UNIT + 16 * k, ptx::desc(qd + k * STEP16, HI), idescO, 1u);              // dS lo
+                ptx::mma_ts(base + V_COL, base + 2 * UNIT + 16 * k, ptx::desc(zd + k * STEP16, HI), idescW, acc);         // W_enc hi x dZ hi (and lo)
+                if (!kWideV) ptx::mma_ts(base + V_COL, base + 2 * UNIT + 16 * k, ptx::desc(zl + k * STEP16, HI), idescO, 1u);
+                ptx::mma_ts(base + V_COL, base + 16 * k + 8, ptx::desc(zd + k * STEP16, HI), idescO, 1u);                 // W_enc lo x dZ hi
+            }
+        };
+        // by one thread: the first unit of tile i (of the CTA)
+        auto open_tile = [&](int i) -> bool {
+            if (!ptx::mbar_wait(bar(T_FULL + i % stages), (i / stages) & 1, abort_flag, kErrBwdTok | 3)) return false;
+            if (kMode == 2) issue_tiles(std::true_type{}, i % stages, 0);
+            else issue_tiles(std::false_type{}, i % stages, 0);
+            return true;
+        };
+        // by one thread: tile i has been read for the last time; on to the group's next
+        auto close_tile = [&](int i) -> bool {
+            ptx::mbar_arrive(bar(T_EMPTY + i % stages));
+            return i + NG >= nt || open_tile(i + NG);
+        };
+        bool ok = true;
+        uint32_t n = 0;                                         // units waited for
+        auto token_of = [&](int i) { return (int)(blockIdx.x + i * gridDim.x) * kTile + row; };   // of this lane in tile i
+        // One row of dK (which = 0) or dV (1) of token tok_n, from this thread's lane of the accumulators.
+        auto write_row = [&](int which, int tok_n) {
+            constexpr int LW = DR >= 16 ? DR : 8;               // columns loaded (narrow heads: within the first 8)
+            const uint32_t col = gcol + (which ? V_COL : K_COL);
+            const size_t tok = ((size_t)b * a.N + (tok_n < a.N ? tok_n : 0)) * a.H + h;
+            __nv_bfloat16 *out = which ? a.dV : a.dK;
+            float4 *sum = reinterpret_cast<float4 *>(a.kvacc + ((size_t)which * a.B * a.N * a.H + tok) * DR);
+            const float sc = which ? 1.f : a.scale;
 #pragma unroll
-                        for (int k = 0; k < D / 16; ++k) ptx::mma_ss(gcol + UNIT, gdesc + 2 * k, ld[2] + 2 * k, idescS, 1u);
-                        if (sweep == 1) {
+            for (int c0 = 0; c0 < LW; c0 += 8) {
+                uint32_t x[8], y[8];
+                ptx::tmem_ld8(col + c0, x);
+                if (kWideV && which) ptx::tmem_ld8(col + D + c0, y);
+                ptx::tmem_wait_ld();
+                constexpr int PW = DR == 4 ? 4 : 8;             // columns written
+                float f[PW];
 #pragma unroll
-                            for (int k = 0; k < D / 16; ++k) ptx::mma_ss(gcol + 2 * UNIT, vdesc + 2 * k, ld[3] + 2 * k, idescS, k > 0);
+                for (int c = 0; c < PW; ++c) {                  // the head's columns
+                    const bool up = DR == 4 && off != 0;
+                    f[c] = __uint_as_float(up ? x[(4 + c) & 7] : x[c]);
+                    if (kWideV && which) f[c] += __uint_as_float(up ? y[(4 + c) & 7] : y[c]);
+                }
+                if (tok_n < a.N) {
+                    if (kMode == 2) {
 #pragma unroll
-                            for (int k = 0; k < D / 16; ++k) ptx::mma_ss(gcol + 2 * UNIT, vdesc + 2 * k, ld[4] + 2 * k, idescS, 1u);
+                        for (int c = 0; c < PW; c += 4) {       // the earlier ranges' shares
+                            float4 &at = sum[(c0 + c) / 4];
+                            if (!a.first) {
+                                const float4 e = at;
+                                f[c] += e.x; f[c + 1] += e.y; f[c + 2] += e.z; f[c + 3] += e.w;
+                            }
+                            if (!a.last) at = make_float4(f[c], f[c + 1], f[c + 2], f[c + 3]);
                         }
-                        ptx::mma_commit(bar(S_FULL + g));
-                        if (!ptx::mbar_wait(bar(P_FULL + g), cnt & 1, abort_flag, kErrBwdTok | 4)) { ok = false; break; }
-                        ++cnt;
-                        ptx::tc_fence_after();
-                        if (sweep == 1) {
-                            // the previous tile's accumulators must have been read before they are overwritten
-                            if (u == 0 && k_tile > 0 &&
-                                !ptx::mbar_wait(bar(ACC_FREE + g), (k_tile - 1) & 1, abort_flag, kErrBwdTok | 5)) { ok = false; break; }
-                            ptx::tc_fence_after();
-                            // Q and dZ (hi, lo) rows of the unit as MN-major B operands, 16 latent rows per k-step
-                            const uint64_t qmn = ptx::smem_desc(ptx::smem_u32(smem + SM::lat_off(stages, M, 0)), G::SBO, G::SBO, G::SWZ) + uoff;
-                            const uint64_t zmn = ptx::smem_desc(ptx::smem_u32(smem + SM::lat_off(stages, M, 3)), G::SBO, G::SBO, G::SWZ) + uoff;
-                            const uint64_t zln = ptx::smem_desc(ptx::smem_u32(smem + SM::lat_off(stages, M, 4)), G::SBO, G::SBO, G::SWZ) + uoff;
+                    }
+                    if (kMode != 2 || a.last) {
+                        uint32_t w[PW / 2];
 #pragma unroll
-                            for (int k = 0; k < UNIT / 16; ++k) {
-                                const uint32_t acc = (u > 0 || k > 0) ? 1u : 0u;
-                                ptx::mma_ts(kcol, gcol + k * 8, qmn + (uint64_t)(k * G::RB), idescO, acc);              // dS hi
-                                ptx::mma_ts(kcol, gcol + UNIT + k * 8, qmn + (uint64_t)(k * G::RB), idescO, 1u);        // dS lo
-                                ptx::mma_ts(vcol, gcol + 2 * UNIT + k * 16, zmn + (uint64_t)(k * G::RB), idescO, acc);       // W_enc dZ_hi
-                                ptx::mma_ts(vcol, gcol + 2 * UNIT + k * 16, zln + (uint64_t)(k * G::RB), idescO, 1u);        // W_enc dZ_lo
-                                ptx::mma_ts(vcol, gcol + 2 * UNIT + k * 16 + 8, zmn + (uint64_t)(k * G::RB), idescO, 1u);    // W_enc lo x dZ_hi
+                        for (int c = 0; c < PW / 2; ++c) w[c] = ptx::pack_bf16(f[2 * c] * sc, f[2 * c + 1] * sc);
+                        if constexpr (PW == 4) *reinterpret_cast<uint2 *>(out + tok * DR) = make_uint2(w[0], w[1]);
+                        else *reinterpret_cast<uint4 *>(out + tok * DR + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+                    }
+                }
+                __syncwarp();
+            }
+        };
+        // Second sweep over the latents of tile i: dS^T and W_enc^T of every unit; the unit after the tile's last is the group's next tile's first.
+        auto sweep2 = [&](auto two, int i, float nld, float fct, float dd) -> bool {
+            constexpr bool kTwo = decltype(two)::value;
+            const float2 nldp = make_float2(nld, nld), fctp = make_float2(fct, fct), nddp = make_float2(-dd, -dd);
+#pragma unroll 1
+            for (int u = 0; u < nu; ++u, ++n) {
+                if (!warp_wait(sfull, n & 1, abort_flag, kErrBwdTok | 7)) return false;
+                ptx::tc_fence_after();
+#pragma unroll 1
+                for (int q = 0; q < UNIT; q += 16) {            // 16 latents at a time
+                    if (u * UNIT + q >= M) break;
+                    const float *le_at = cst + (kTwo ? 0 : 2 * M) + u * UNIT + q, *de_at = cst + M + u * UNIT + q;
+                    // the second eight columns on their way while the first are worked on: 2 % at D = 16 without padding, 4 % lost where
+                    // it costs the padded form registers, nothing at D = 32 and 64
+                    constexpr bool kPf = D == 16 && !kPadded;
+                    uint32_t wl0[4], ss[2][8], aa[2][8], cc[2][8];
+                    auto load = [&](int p, int to) {
+                        ptx::tmem_ld8(gcol + q + p * 8, ss[to]);
+                        ptx::tmem_ld8(gcol + UNIT + q + p * 8, aa[to]);
+                        ptx::tmem_ld8(gcol + 2 * UNIT + q + p * 8, cc[to]);
+                    };
+                    if (kPf) {
+                        load(0, 0);
+                        ptx::tmem_wait_ld();
+                        load(1, 1);
+                    }
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        uint32_t hi[4], lo[4], wh[4], wl[4];
+                        uint32_t (&s)[8] = ss[kPf ? p : 0], (&av)[8] = aa[kPf ? p : 0], (&cv)[8] = cc[kPf ? p : 0];
+                        if (!kPf) {
+                            load(p, 0);
+                            ptx::tmem_wait_ld();
+                        }
+#pragma unroll
+                        for (int k = 0; k < 4; k += 2) {
+                            const float4 le = *reinterpret_cast<const float4 *>(le_at + p * 8 + 2 * k);
+                            const float4 nd = *reinterpret_cast<const float4 *>(de_at + p * 8 + 2 * k);
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const int j = 2 * (k + e);
+                                const DsPair r = ds_pair<true, kTwo>(
+                                    make_float2(__uint_as_float(s[j]), __uint_as_float(s[j + 1])), make_float2(__uint_as_float(av[j]), __uint_as_float(av[j + 1])),
+                                    make_float2(__uint_as_float(cv[j]), __uint_as_float(cv[j + 1])), sl2p, nldp, nddp,
+                                    e ? make_float2(nd.z, nd.w) : make_float2(nd.x, nd.y), e ? make_float2(le.z, le.w) : make_float2(le.x, le.y), fctp);
+                                hi[k + e] = r.hi; lo[k + e] = r.lo; wh[k + e] = r.whi; wl[k + e] = r.wlo;
                             }
                         }
-                    }
-                }
-                if (!ok) break;
-                ptx::mma_commit(bar(T_EMPTY + s));
-                if (kMode != 1) ptx::mma_commit(bar(ACC_FULL + g));
-            }
-        }
-    } else {
-        const int g = (warp - kFirstSoftmaxWarp) >> 2;
-        const int row = ((warp & 3) << 5) + lane;               // TMEM lane = token within the tile
-        const uint32_t lane_addr = (uint32_t)((warp & 3) << 5) << 16;
-        const uint32_t gcol = tm + lane_addr + g * 128;
-        const uint32_t kcol = gcol + 3 * UNIT, vcol = kcol + D;
-        const float2 sl2p = make_float2(a.sl2, a.sl2);
-        uint32_t cnt = 0;
-        int k_tile = 0;
-        bool ok = true;
-        // The rows of a tile are written one sweep late: while the issuing warp finishes the tile's last MMAs the
-        // group already works on the first sweep of its next tile, whose MMAs do not touch the accumulators.
-        bool pend = false, p_inside = false;
-        size_t p_tok = 0, p_ddi = 0;
-        float p_dd = 0.f;
-        int p_k = 0;
-        auto write_rows = [&]() -> bool {
-            if (!warp_wait(bar(ACC_FULL + g), p_k & 1, abort_flag, kErrBwdTok | 8)) return false;
-            ptx::tc_fence_after();
-            uint32_t ak[D], avv[D];
+                        if (kPf && p == 0) ptx::tmem_wait_ld();
+                        // over columns this thread has read, 8 packed columns per array: dS hi and W_enc lo over S, dS lo over A, W_enc hi over C
+                        ptx::tmem_st4(gcol + q + p * 4, hi);
+                        ptx::tmem_st4(gcol + UNIT + q + p * 4, lo);
+                        ptx::tmem_st4(gcol + 2 * UNIT + q + p * 4, wh);
+                        if (p == 0) {
 #pragma unroll
-            for (int dc = 0; dc < D / 16; ++dc) {
-                ptx::tmem_ld16(kcol + dc * 16, ak + dc * 16);
-                ptx::tmem_ld16(vcol + dc * 16, avv + dc * 16);
-            }
-            ptx::tmem_wait_ld();
-            ptx::tc_fence_before();
-            ptx::mbar_arrive(bar(ACC_FREE + g));
-            if (p_inside) {
-                if (kMode == 0) a.dd[p_ddi] = p_dd;
-                float fk[DR], fv[DR];
-#pragma unroll
-                for (int i = 0; i < DR; ++i) {                  // the head's columns of the accumulators
-                    fk[i] = __uint_as_float((DR == 4 && off) ? ak[(4 + i) % D] : ak[i]);
-                    fv[i] = __uint_as_float((DR == 4 && off) ? avv[(4 + i) % D] : avv[i]);
-                }
-                float4 *sk = reinterpret_cast<float4 *>(a.kvacc + p_tok * DR);
-                float4 *sv = reinterpret_cast<float4 *>(a.kvacc + ((size_t)a.B * a.N * a.H + p_tok) * DR);
-                if (kMode == 2 && !a.first) {                  // the earlier ranges' shares
-#pragma unroll
-                    for (int i = 0; i < DR / 4; ++i) {
-                        const float4 pk4 = sk[i], pv4 = sv[i];
-                        fk[4 * i] += pk4.x; fk[4 * i + 1] += pk4.y; fk[4 * i + 2] += pk4.z; fk[4 * i + 3] += pk4.w;
-                        fv[4 * i] += pv4.x; fv[4 * i + 1] += pv4.y; fv[4 * i + 2] += pv4.z; fv[4 * i + 3] += pv4.w;
-                    }
-                }
-                if (kMode == 2 && !a.last) {
-#pragma unroll
-                    for (int i = 0; i < DR / 4; ++i) {
-                        sk[i] = make_float4(fk[4 * i], fk[4 * i + 1], fk[4 * i + 2], fk[4 * i + 3]);
-                        sv[i] = make_float4(fv[4 * i], fv[4 * i + 1], fv[4 * i + 2], fv[4 * i + 3]);
-                    }
-                } else {
-                    uint32_t *dk = reinterpret_cast<uint32_t *>(a.dK + p_tok * DR), *dv = reinterpret_cast<uint32_t *>(a.dV + p_tok * DR);
-                    uint32_t wk[DR / 2], wv[DR / 2];
-#pragma unroll
-                    for (int i = 0; i < DR / 2; ++i) {
-                        wk[i] = ptx::pack_bf16(fk[2 * i] * a.scale, fk[2 * i + 1] * a.scale);
-                        wv[i] = ptx::pack_bf16(fv[2 * i], fv[2 * i + 1]);
-                    }
-                    if (DR == 4) {
-                        *reinterpret_cast<uint2 *>(dk) = make_uint2(wk[0], wk[1]);
-                        *reinterpret_cast<uint2 *>(dv) = make_uint2(wv[0], wv[1]);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < DR / 8; ++q) {
-                            reinterpret_cast<uint4 *>(dk)[q] = make_uint4(wk[4 * q], wk[4 * q + 1], wk[4 * q + 2], wk[4 * q + 3]);
-                            reinterpret_cast<uint4 *>(dv)[q] = make_uint4(wv[4 * q], wv[4 * q + 1], wv[4 * q + 2], wv[4 * q + 3]);
+                            for (int k = 0; k < 4; ++k) wl0[k] = wl[k];
+                        } else {
+                            ptx::tmem_st4(gcol + q + 8, wl0);
+                            ptx::tmem_st4(gcol + q + 12, wl);
                         }
                     }
                 }
+                ptx::tmem_wait_st();
+                if (hand_over(pfull, n, abort_flag, kErrBwdTok | 4) && ptx::elect_one()) {
+                    issue_outputs(u);
+                    bool go = true;
+                    if (u + 1 < nu) issue_tiles(std::true_type{}, i % stages, u + 1);
+                    else go = close_tile(i);
+                    if (go) ptx::mma_commit(sfull);
+                }
+                __syncwarp();
             }
-            pend = false;
             return true;
         };
         // this lane's token of a tile: its decode log-sum-exp and mask byte, fetched one tile ahead
         float f_ld = 0.f, f_dd = 0.f;
         uint32_t f_mask = 1u;
         auto fetch = [&](int i) {
-            const int n = (blockIdx.x + i * gridDim.x) * kTile + row;
-            const size_t nn = (size_t)b * a.N + (n < a.N ? n : 0);
+            const int t = token_of(i);
+            const size_t nn = (size_t)b * a.N + (t < a.N ? t : 0);
             f_ld = a.lse_dec[nn * a.H + h];
-            f_mask = a.key_mask == nullptr ? 1u : (uint32_t)a.key_mask[nn];
-            if (kMode == 2) f_dd = a.dd[((size_t)b * a.H + h) * a.N + (n < a.N ? n : 0)];
+            if (kPadded) f_mask = a.key_mask == nullptr ? 1u : (uint32_t)a.key_mask[nn];
+            if (kMode == 2) f_dd = a.dd[((size_t)b * a.H + h) * a.N + (t < a.N ? t : 0)];
         };
-        if (g < ng && g < nt) fetch(g);
-        for (int i = g; ok && g < ng && i < nt; i += ng, ++k_tile) {
-            const int t = blockIdx.x + i * gridDim.x, n = t * kTile + row;
-            const bool inside = n < a.N;
-            const bool valid = inside && f_mask != 0;
-            const size_t tok = ((size_t)b * a.N + (inside ? n : 0)) * a.H + h;
-            const float negld = inside ? -f_ld * 1.4426950408889634f : -INFINITY;
-            const float2 negldp = make_float2(negld, negld);
-            const float dd_given = inside ? f_dd : 0.f;         // mode 2: dd[n] over all latents, from the workspace
-            if (i + ng < nt) fetch(i + ng);
-            const bool plain = a.key_mask == nullptr && (t + 1) * kTile <= a.N;      // uniform over the group
-            // sweep 1: dd[n] = sum_m W_dec[n,m] (dY_n . Z_m)
-            float2 dd2 = make_float2(0.f, 0.f);
-            for (int u = 0; ok && kMode != 2 && u < nu; ++u) {
-                if (!warp_wait(bar(S_FULL + g), cnt & 1, abort_flag, kErrBwdTok | 6)) { ok = false; break; }
-                ++cnt;
-                ptx::tc_fence_after();
-#pragma unroll
-                for (int hb = 0; hb < UNIT / 16; ++hb) {
-                    uint32_t s[16], av[16];
-                    ptx::tmem_ld16(gcol + hb * 16, s);
-                    ptx::tmem_ld16(gcol + UNIT + hb * 16, av);
-                    ptx::tmem_wait_ld();
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(s[2 * k]), __uint_as_float(s[2 * k + 1])), sl2p, negldp);
-                        dd2 = __ffma2_rn(make_float2(ptx::ex2(x.x), ptx::ex2(x.y)),
-                                         make_float2(__uint_as_float(av[2 * k]), __uint_as_float(av[2 * k + 1])), dd2);
-                    }
-                }
-                ptx::tc_fence_before();
-                ptx::mbar_arrive(bar(P_FULL + g));
-            }
-            const float dd = kMode == 2 ? dd_given : dd2.x + dd2.y;
-            const float2 negddp = make_float2(-dd, -dd);
-            if (kMode == 1) {                                  // this range's share of dd[n]; no second sweep
-                if (inside) {
-                    const size_t ddi = ((size_t)b * a.H + h) * a.N + n;
-                    a.dd[ddi] = (a.first ? 0.f : a.dd[ddi]) + dd;
-                }
-                continue;
-            }
-            if (ok && pend) ok = write_rows();                  // the previous tile's rows
-            // sweep 2: dS^T and W_enc^T of every unit, handed to the issuing warp
-            auto unit2 = [&](auto masked, int u) {
-                constexpr bool kMasked = decltype(masked)::value;
-                uint32_t pwl[4];                                    // lo halves of W_enc of an even quarter, kept for one quarter
-#pragma unroll
-                for (int qd = 0; qd < UNIT / 8; ++qd) {
-                    uint32_t s[8], av[8], cv[8], pk[4], pl[4], pw[4], pwo[4];
-                    ptx::tmem_ld8(gcol + qd * 8, s);
-                    ptx::tmem_ld8(gcol + UNIT + qd * 8, av);
-                    ptx::tmem_ld8(gcol + 2 * UNIT + qd * 8, cv);
-                    ptx::tmem_wait_ld();
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int col = u * UNIT + qd * 8 + 2 * k;                  // latent of this pair of columns
-                        const float2 sp = make_float2(__uint_as_float(s[2 * k]), __uint_as_float(s[2 * k + 1]));
-                        const float2 nle = *reinterpret_cast<const float2 *>(cst + col);
-                        const float2 nde = *reinterpret_cast<const float2 *>(cst + MU + col);
-                        const float2 xd = __ffma2_rn(sp, sl2p, negldp), xe = __ffma2_rn(sp, sl2p, nle);
-                        const float2 pd = make_float2(ptx::ex2(xd.x), ptx::ex2(xd.y));
-                        float2 pe = make_float2(ptx::ex2(xe.x), ptx::ex2(xe.y));
-                        if (kMasked && !valid) pe = make_float2(0.f, 0.f);
-                        const float2 uu = __fadd2_rn(make_float2(__uint_as_float(av[2 * k]), __uint_as_float(av[2 * k + 1])), negddp);
-                        const float2 vv = __fadd2_rn(make_float2(__uint_as_float(cv[2 * k]), __uint_as_float(cv[2 * k + 1])), nde);
-                        const float2 ds = __ffma2_rn(pd, uu, __fmul2_rn(pe, vv));
-                        const uint32_t hi = ptx::pack_bf16(ds.x, ds.y);
-                        pk[k] = hi;
-                        pl[k] = ptx::pack_bf16(ds.x - __uint_as_float(hi << 16), ds.y - __uint_as_float(hi & 0xffff0000u));
-                        const uint32_t wh = ptx::pack_bf16(pe.x, pe.y);
-                        pw[k] = wh;
-                        pwo[k] = ptx::pack_bf16(pe.x - __uint_as_float(wh << 16), pe.y - __uint_as_float(wh & 0xffff0000u));
-                    }
-                    // Packed results over columns this thread has already read: dS hi over S, dS lo over A.  W_enc over
-                    // C, per 16 latents (two quarters): hi in the first 8 of their 16 columns, lo in the other 8 - which
-                    // the odd quarter has only just read, so the even quarter's lo waits in four registers.
-                    ptx::tmem_st4(gcol + qd * 4, pk);
-                    ptx::tmem_st4(gcol + UNIT + qd * 4, pl);
-                    ptx::tmem_st4(gcol + 2 * UNIT + (qd >> 1) * 16 + (qd & 1) * 4, pw);
-                    if (qd & 1) {
-                        ptx::tmem_st4(gcol + 2 * UNIT + (qd >> 1) * 16 + 8, pwl);
-                        ptx::tmem_st4(gcol + 2 * UNIT + (qd >> 1) * 16 + 12, pwo);
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) pwl[k] = pwo[k];
-                    }
-                }
-            };
-            for (int u = 0; ok && u < nu; ++u) {
-                if (!warp_wait(bar(S_FULL + g), cnt & 1, abort_flag, kErrBwdTok | 7)) { ok = false; break; }
-                ++cnt;
-                ptx::tc_fence_after();
-                if (kPadded && !plain) unit2(std::true_type{}, u); else unit2(std::false_type{}, u);
-                ptx::tmem_wait_st();
-                ptx::tc_fence_before();
-                ptx::mbar_arrive(bar(P_FULL + g));
-            }
-            if (!ok) break;
-            pend = true; p_inside = inside; p_tok = tok; p_dd = dd; p_k = k_tile;
-            p_ddi = ((size_t)b * a.H + h) * a.N + (inside ? n : 0);
+        if (g < nt) {
+            fetch(g);
+            if ((warp & 3) == 0 && ptx::elect_one() && open_tile(g)) ptx::mma_commit(sfull);
+            __syncwarp();
         }
-        if (ok && pend) ok = write_rows();
+        for (int i = g; ok && i < nt; i += NG) {
+            const int tok_n = token_of(i);
+            const bool inside = tok_n < a.N;
+            const float nld = inside ? -f_ld * kBwdLog2e : -INFINITY;
+            const bool part = inside && (!kPadded || f_mask != 0);   // the token takes part in the encode softmax
+            float dd = inside ? f_dd : 0.f;                     // mode 2: over all latents, from the workspace
+            if (i + NG < nt) fetch(i + NG);
+            if (kMode != 2) {
+                // first sweep: dd[n] = sum_m W_dec[n,m] (dY_n . Z_m)
+                const float2 nldp = make_float2(nld, nld);
+                float2 d2 = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int u = 0; u < nu; ++u, ++n) {
+                    if (!(ok = warp_wait(sfull, n & 1, abort_flag, kErrBwdTok | 6))) break;
+                    ptx::tc_fence_after();
+                    uint32_t x[16], av[16];
+                    auto add = [&]() {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const float2 e = __ffma2_rn(make_float2(__uint_as_float(x[2 * k]), __uint_as_float(x[2 * k + 1])), sl2p, nldp);
+                            d2 = __ffma2_rn(make_float2(ptx::ex2(e.x), ptx::ex2(e.y)),
+                                            make_float2(__uint_as_float(av[2 * k]), __uint_as_float(av[2 * k + 1])), d2);
+                        }
+                    };
+                    const bool both = u * UNIT + 16 < M;
+                    ptx::tmem_ld16(gcol, x);
+                    ptx::tmem_ld16(gcol + UNIT, av);
+                    ptx::tmem_wait_ld();
+                    if (both) {
+                        add();
+                        ptx::tmem_ld16(gcol + 16, x);
+                        ptx::tmem_ld16(gcol + UNIT + 16, av);
+                        ptx::tmem_wait_ld();
+                    }
+                    // the buffer has been read: the next unit's tiles run under the second half's exponentials
+                    if (hand_over(pfull, n, abort_flag, kErrBwdTok | 4) && ptx::elect_one()) {
+                        bool go = true;
+                        if (u + 1 < nu) issue_tiles(std::false_type{}, i % stages, u + 1);
+                        else if (kMode == 0) issue_tiles(std::true_type{}, i % stages, 0);
+                        else go = close_tile(i);
+                        if (go) ptx::mma_commit(sfull);
+                    }
+                    __syncwarp();
+                    add();
+                }
+                if (!ok) break;
+                dd = d2.x + d2.y;
+                if (inside) {
+                    float *at = a.dd + ((size_t)b * a.H + h) * a.N + tok_n;
+                    *at = kMode == 1 && !a.first ? *at + dd : dd;
+                }
+            }
+            if (kMode != 1) {
+                if (i > g && kMode == 0) {                      // the previous tile's rows
+                    write_row(0, token_of(i - NG));
+                    write_row(1, token_of(i - NG));
+                }
+                const bool far = __any_sync(0xffffffffu, part && !(-nld - lse_min <= kOneExpLog2));
+                // this token's factor of W_enc, or (far) the addend of its exponent
+                const float fct = far ? (part ? 0.f : -INFINITY) : (part ? ptx::ex2(-nld - lse_min) : 0.f);
+                ok = far ? sweep2(std::true_type{}, i, nld, fct, dd) : sweep2(std::false_type{}, i, nld, fct, dd);
+                if (!ok) break;
+            }
+            // mode 2 has no first sweep under which a tile's last contractions would finish: its rows are written right away
+            const bool done = i + NG >= nt;
+            if ((done && kMode == 0) || kMode == 2) {
+                if (!(ok = warp_wait(sfull, n & 1, abort_flag, kErrBwdTok | 8))) break;
+                ptx::tc_fence_after();
+                write_row(0, tok_n);
+                write_row(1, tok_n);
+            }
+        }
     }
     ptx::tc_fence_before();
     __syncthreads();
-    if (warp == kFirstIssuerWarp) {
+    if (warp == 1) {
         ptx::tc_fence_after();
-        ptx::tmem_dealloc(tm, NCOLS);
+        ptx::tmem_dealloc(tm, 512);
     }
     if (threadIdx.x == 0 && *abort_flag != 0 && a.status != nullptr) atomicCAS(a.status, 0u, *abort_flag);
 }

@@ -164,6 +164,24 @@ struct TcEncodePlan {
     int tiles, pairs, splits, per_split, P;
 };
 
+// CTAs to split the token tiles of each of `groups` pieces of work over, one CTA per SM at a time.  A CTA costs its share of the tiles
+// and about four tiles' time to start and finish (5 of 1.6 us); a launch costs as many CTAs as its fullest SM runs one after the other, so
+// that one more split than fills the chip once can take twice as long and several times as many less than once (64 pieces: 2 splits leave
+// 20 of 148 SMs idle, 23 in ten rounds 0.5); each split also leaves a partial result of `part_bytes` to be reduced (some 4 MB
+// written and read in a tile's time).  At most 512 tiles per split keep the float32 sums on the tensor core short.
+inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes) {
+    const double start = 4.0, reduce = (double)part_bytes / 4.0e6;
+    const int least = (tiles + 511) / 512, most = tiles < least + sms ? tiles : least + sms;
+    int best = least;
+    double best_cost = 0.0;
+    for (int s = least; s <= most; ++s) {
+        const double rounds = (double)((groups * s + sms - 1) / sms);
+        const double cost = rounds * ((tiles + s - 1) / s + start) + reduce * s;
+        if (s == least || cost < best_cost) { best = s; best_cost = cost; }
+    }
+    return best;
+}
+
 // With at most 64 latents a CTA encodes two adjacent heads at once (see encode_tc_kernel).
 inline bool encode_head_pairs(const flare_desc_t *d) { return d->M <= 64 && d->H % 2 == 0 && d->D >= 16 && d->D <= 32; }
 
@@ -277,22 +295,18 @@ inline size_t decode_range_bytes(const flare_desc_t *d) {
 // Pass A (dZ) runs as the dZ form of the tensor-core encode kernel wherever that kernel runs.
 inline bool bwd_dz_on_tensor_cores(const flare_desc_t *d) { return use_tc(d); }
 
-// Pass B for dQ runs on the tensor cores for narrow heads (S, A, C and the partial dQ of a group share its 128
-// TMEM columns: 3 * 32 + D).
-inline bool bwd_dq_on_tensor_cores(const flare_desc_t *d) { return use_tc(d) && d->D <= 32; }
+// Pass B (dQ; dK and dV) runs on the tensor cores for the same shapes.
+inline bool bwd_dq_on_tensor_cores(const flare_desc_t *d) { return use_tc(d); }
 
-// Plan of the tensor-core dQ kernel: the encode plan without head pairing.
+// Plan of the tensor-core dQ kernel: `pairs` = blocks of 128 latents per head, one partial sum per CTA.
 inline TcEncodePlan tc_dq_plan(const flare_desc_t *d, int sms) {
     TcEncodePlan p;
-    const int mb = (d->M + kTile - 1) / kTile;
     p.tiles = (d->N + kTile - 1) / kTile;
-    p.pairs = (mb + 1) / 2;
-    long s = sms / ((long)d->B * d->H * p.pairs);
-    if (s < 1) s = 1;
-    if (s > p.tiles) s = p.tiles;
-    p.splits = (int)s;
-    p.per_split = (mb == 1) ? 4 : 2;
-    p.P = p.splits * p.per_split;
+    p.pairs = encode_head_pairs(d) ? 1 : (d->M + kTile - 1) / kTile;
+    const long groups = (long)d->B * (encode_head_pairs(d) ? d->H / 2 : d->H) * p.pairs;
+    p.splits = balanced_splits(groups, p.tiles, sms, (size_t)d->B * d->H * d->M * d->D * sizeof(float));
+    p.per_split = 1;
+    p.P = p.splits;
     return p;
 }
 
@@ -303,10 +317,12 @@ struct BwdLayout {
     int P;
 };
 
-// Latents one launch of the tensor-core token kernel keeps in shared memory (five operands of D-wide bf16 rows,
-// beside at least five tile stages); more are worked off in ranges of this many.
-inline int token_range(const flare_desc_t *d) { return d->D == 32 ? 256 : 512; }
-inline bool token_in_ranges(const flare_desc_t *d) { return bwd_dq_on_tensor_cores(d) && d->M > token_range(d); }
+// Latents one launch of the tensor-core token kernel takes: five operands of D-wide bf16 rows beside a tile stage per group (four groups at
+// D <= 16, three at 32, two at 64); more are worked off in ranges of equal size.
+inline int token_range_most(const flare_desc_t *d) { return d->D == 64 ? 192 : d->D == 32 ? 448 : 1024; }
+inline bool token_in_ranges(const flare_desc_t *d) { return bwd_dq_on_tensor_cores(d) && d->M > token_range_most(d); }
+inline int token_ranges(const flare_desc_t *d) { return (d->M + token_range_most(d) - 1) / token_range_most(d); }
+inline int token_range(const flare_desc_t *d) { return ((d->M + token_ranges(d) - 1) / token_ranges(d) + 15) / 16 * 16; }
 
 inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     BwdLayout w;
