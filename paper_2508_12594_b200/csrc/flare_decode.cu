@@ -37,7 +37,7 @@ int launch_decode_tc_m(const flare_desc_t *d, int sms, const void *Q, const void
 
 // The streaming (fast) form of decode: head widths 16 (and narrower) and 32, as many latents as fit shared memory.
 template <int D>
-bool decode_stream_fits(int mc) { return (D == 16 || D == 32) && DecodeStreamSmem<(D == 16 || D == 32) ? D : 16>::fits(mc); }
+bool decode_stream_fits(int mc) { return (D == 16 || D == 32) && DecodeStreamSmem<(D == 16 || D == 32) ? D : 16>::fits((mc + 31) & ~31); }
 
 template <int D, int DRT, bool kPart, int kM, bool kLse>
 int launch_decode_stream_l(const flare_desc_t *d, int sms, const void *Q, const void *K, const float *Z, void *Y,
@@ -48,7 +48,7 @@ int launch_decode_stream_l(const flare_desc_t *d, int sms, const void *Q, const 
         if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
         if (DRT != 0) tmQ = tmK;   // unused: the narrow forms stage Q with their threads
         else if ((rc = make_latent_map(&tmQ, Q, d)) != FLARE_OK) return rc;
-        const size_t smem = DecodeStreamSmem<D>::total(mc);
+        const size_t smem = DecodeStreamSmem<D>::total(DecodeStreamSmem<D>::padded(mc));
         static std::atomic<uint64_t> smem_opt_in{0};
         if (int rc_attr = ensure_big_smem(decode_stream_kernel<D, DRT, kPart, kM, kLse>, smem_opt_in, 227 * 1024)) return rc_attr;
         DecodeTcArgs a;
@@ -122,7 +122,7 @@ int launch_decode_tc(const flare_desc_t *d, int sms, const void *Q, const void *
 template <int D, int DRT>
 int decode_tc_any(const flare_desc_t *d, int sms, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec,
                   uint32_t *status, char *range_scratch, cudaStream_t st) {
-    const bool fast = use_fast(d, kFastDecode) && status != nullptr;
+    const bool fast = use_fast_decode(d) && status != nullptr;
     if (d->M <= kDecodeMaxM) return launch_decode_tc<D, DRT>(d, sms, Q, K, Z, Y, lse_dec, status, st, 0, 0, nullptr, fast);
     constexpr int DR = DRT ? DRT : D;
     const int C = decode_ranges(d);

@@ -78,7 +78,7 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
         TcEncodePlan p = tc_encode_plan(d, di.sms);
         uint32_t *status = reinterpret_cast<uint32_t *>(base);
         // a caller that asks for lse_enc is saving Z for the backward: weights as two bf16 halves (see exp_chunk_hilo)
-        const bool fast = use_fast(d, kFastEncode);
+        const bool fast = use_fast_encode(d, lse_enc != nullptr, mask != nullptr);
 #define FLARE_ENC3(DD, PAIR, DRT, MB, HL) encode_tc_forms<DD, PAIR, DRT, HL, MB>(d, p, Q, K, V, mask, pm, pl, pacc, status, st, fast)
 #define FLARE_ENC2(DD, PAIR, DRT, MB) (lse_enc != nullptr ? FLARE_ENC3(DD, PAIR, DRT, MB, true) : FLARE_ENC3(DD, PAIR, DRT, MB, false))
         // A call with a key mask has padding in every tile and takes the form that tests every element (see

@@ -136,26 +136,37 @@ inline bool use_tc(const flare_desc_t *d) {
 // Which form of the tensor-core forward kernels runs (flare_set_path).
 extern std::atomic<int> g_path;
 
+// With at most 64 latents a CTA encodes two adjacent heads at once (see encode_tc_kernel).
+inline bool encode_head_pairs(const flare_desc_t *d) { return d->M <= 64 && d->H % 2 == 0 && d->D >= 16 && d->D <= 32; }
+
 // The fast forms (no running maximum, see kFastMaxLog2 in flare_tc.cuh) are followed by a launch of the exact
-// form that exits at once unless it is needed: two more launches per forward, which pay off from a few tens of
-// microseconds of work.
-enum FastStage { kFastEncode, kFastDecode };
-inline bool use_fast(const flare_desc_t *d, FastStage stage) {
-    if (!use_tc(d)) return false;
-    if (stage == kFastDecode && d->D > 32) return false;           // the streaming decode has no form for head width 64
+// form that exits at once unless it is needed: two more launches per forward, which pay off from some size on.
+inline bool fast_wanted(const flare_desc_t *d, bool pays) {
     const int path = g_path.load(std::memory_order_relaxed);
-    if (path == FLARE_PATH_EXACT) return false;
-    if (path == FLARE_PATH_FAST) return true;
-    // Measured (forward stage times, fast against exact form): encode wins from 128 latents (3-5 % there, 15 % at 256),
-    // is equal or loses at 32 and 64 latents of width 32; the streaming decode
-    // wins from 64 latents (16 % at 64 and 128) and loses at 32; below some tens of microseconds of work the two extra
-    // launches cost more than the forms gain.
-    // The head-pair form of encode (M <= 64, H even) wins at D = 16 since its K/V ring is deep (0.077 -> 0.062 ms on the
-    // 2-D mesh: its rows are short scans, in which the exact form rescales its accumulator on most units) and is equal
-    // at D = 32, where it has no room for the ones column and sums the weights in registers.
-    const bool pair16 = d->M <= 64 && d->H % 2 == 0 && d->D == 16;
-    const bool big_enough = stage == kFastEncode ? (d->M >= 128 || pair16) : d->M >= 64;
-    return big_enough && (double)d->B * d->H * d->N * d->M >= 3.0e7;
+    return use_tc(d) && path != FLARE_PATH_EXACT && (path == FLARE_PATH_FAST || pays);
+}
+// Encode: the time of either form goes with the blocks of 128 lanes (of latents, or of two heads), whatever part of them is filled.
+// Measured, fast against exact form, us, at B H N = 65536 / 131072 / 262144 / 2.1 million, D = 8 and 16: 9.2 : 8.3 / 11.7 : 12.4 / 16.1 : 19.6
+// / 77 : 104, masked 11.0 : 10.4 / 14.5 : 15.8 / 21.5 : 25.8 / 110 : 151.  The head-pair form at D = 32 and D = 64 have a shallow K/V ring,
+// which the norm check holds longer: the first pays later (masked 26 : 32 at 262144, else 41 : 42 at 524288), D = 64 never (13.6 : 19 at
+// 32768, 72 : 84 at a million).
+inline bool use_fast_encode(const flare_desc_t *d, bool lse, bool masked) {
+    const double work = (double)d->B * d->N * (encode_head_pairs(d) ? d->H / 2 : d->H) * ((d->M + 127) / 128);
+    const double least = encode_head_pairs(d) && d->D == 32 ? (masked ? 2.0e5 : 5.0e5) : lse && !masked ? 2.0e5 : 1.0e5;
+    return d->D <= 32 && fast_wanted(d, work >= least);
+}
+// Decode: the streaming form has no variant for head width 64.  Measured against the exact form, us, at B H N = 524288 (131072): D = 16, M = 48
+// 20 : 29 (11.2 : 10.4), 64 31 : 35 (10.4 : 8.3), 96 26 : 36 (12.9 : 12.6), 144 27 : 33 (15 : 20); the exact form keeps what one chunk
+// of its registers holds (M = 32: 18 : 13) and, at D = 32, 64 latents (48 : 41) and small calls up to there (M = 48: 29 : 35 from 262144 on).
+inline bool use_fast_decode(const flare_desc_t *d) {
+    const double rows = (double)d->B * d->H * d->N;
+    bool pays;
+    if (d->M == 32 || (d->D == 32 && d->M == 64)) pays = false;
+    else if (d->M < 64) pays = rows >= 3.0e5;
+    else if (d->M == 64) pays = rows >= 5.0e5;
+    else if (d->M <= 128) pays = rows >= (d->D == 32 && d->M != 128 ? 6.0e4 : 2.0e5);
+    else pays = rows >= 6.0e4;
+    return d->D <= 32 && fast_wanted(d, pays);
 }
 
 // Launch plan of the tensor-core encode: `pairs` CTAs per head along the latents (two 128-latent blocks each),
@@ -181,9 +192,6 @@ inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes) {
     }
     return best;
 }
-
-// With at most 64 latents a CTA encodes two adjacent heads at once (see encode_tc_kernel).
-inline bool encode_head_pairs(const flare_desc_t *d) { return d->M <= 64 && d->H % 2 == 0 && d->D >= 16 && d->D <= 32; }
 
 inline TcEncodePlan tc_encode_plan(const flare_desc_t *d, int sms) {
     TcEncodePlan p;

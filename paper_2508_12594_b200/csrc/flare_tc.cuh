@@ -172,12 +172,15 @@ __device__ __forceinline__ void exp_chunk_hilo(const uint32_t *r, uint32_t *hi, 
 // ---------------------------------------------------------------------------- softmax without a running maximum
 // The "fast" forms of the kernels evaluate p = 2^(s * sl2) as it stands: no maximum is searched, subtracted or
 // tracked, no accumulator is ever rescaled, and the column ranges of a decode tile need no common reference.
-// float32 and bfloat16 hold 2^x for |x| < 126; with 30 binades kept free for the sums of up to 2^20 such terms times
-// values of ordinary size, that is safe while every |s * sl2| <= kFastMaxLog2.  The kernels check the sufficient
-// condition |q| |k| sl2 <= kFastMaxLog2 (Cauchy-Schwarz) on the rows they hold in shared memory and raise a flag if
-// it fails; the host then runs the exact form (running maximum) of the same kernel, which exits at once while the
-// flag is clear.
-constexpr float kFastMaxLog2 = 96.f;
+// float32 and bfloat16 hold 2^x for |x| < 126, so every weight is exact to its rounding while every |s * sl2| <= kFastMaxLog2; the kernels
+// check the sufficient condition |q| |k| sl2 <= kFastMaxLog2 (Cauchy-Schwarz) on the rows they hold in shared memory.  What the scores
+// really reach is far less, and shows in the sums of weights: a row whose sum lies within [kFastSumMin, kFastSumMax] has lost nothing that
+// matters at either end (no weight below 2^-126 of more than 2^-36 of the sum, values of up to 2^23 times the sum within float32).  Where
+// either check fails a flag is raised; the host then runs the exact form (running maximum) of the same kernel, which exits at once
+// while the flag is clear.  (With the norms alone, and 30 binades kept free for the sums, point clouds of width 32 failed the check
+// at 102 > 96 and ran both forms: decode 65 + 155 us where the first would have done.)
+constexpr float kFastMaxLog2 = 125.f;
+constexpr float kFastSumMin = 8.0779357e-28f, kFastSumMax = 2.0282410e31f;   // 2^-90, 2^104
 
 // Two ways to 2^x share the work.  The special-function unit (ex2.approx) delivers 16 results per clock per SM and
 // is the busiest unit of these kernels; the other half of the column pairs goes through the FMA pipe: with
@@ -769,6 +772,8 @@ template <int D>
 struct DecodeStreamSmem {
     using G = TileGeom<D>;
     static constexpr size_t kBarBytes = 1024;
+    // (M here: the launch's latents rounded up to whole units of 32)
+    __host__ __device__ static int padded(int M) { return (M + 31) & ~31; }
     __host__ __device__ static int stages(int M) {
         int s = 8;
         while (s > 4 && (size_t)s * G::TILE_BYTES + (size_t)4 * M * G::RB + kBarBytes + 2048 > 227 * 1024) --s;
@@ -799,12 +804,13 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     static_assert(kM % 64 == 0, "compile-time latent counts are multiples of 64");
-    const int M = kM ? kM : a.M;
-    const int nstages = SM::stages(M);
+    // M: latents; MP: rows of the latent operands, whole units (rows beyond M are zeros; their weights are left out)
+    const int M = kM ? kM : a.M, MP = kM ? kM : SM::padded(a.M);
+    const int nstages = SM::stages(MP);
     uint8_t *sK = smem;
-    uint8_t *sQ = smem + SM::q_off(M);
-    uint8_t *sZ = smem + SM::z_off(M);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off(M));
+    uint8_t *sQ = smem + SM::q_off(MP);
+    uint8_t *sZ = smem + SM::z_off(MP);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off(MP));
     constexpr int NG = kSoftmaxGroups, kMaxStages = 8, UNIT = 32;
     // S_FULL[2] per group: the scores of a unit are in its buffer (and all earlier MMAs of the group are done);
     // P_FULL[2]: the unit's weights are over them (one arrival per warp); Y_FULL / Y_FREE: a tile's rows are complete / read
@@ -824,7 +830,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     const int t_begin = (int)((long)a.tiles * blockIdx.x / gridDim.x);
     const int t_end = (int)((long)a.tiles * (blockIdx.x + 1) / gridDim.x);
     const int ntiles = t_end - t_begin;
-    const int units = (M + UNIT - 1) / UNIT;                    // per tile; the last may have 16 columns
+    const int units = MP / UNIT;                                // per tile; the last may have 16 latents
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
 
     if (threadIdx.x == 0) {
@@ -841,16 +847,19 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     if (warp == kFirstIssuerWarp) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     {   // Z_bh -> [hi | lo | ones] blocks of M latent-major rows in the swizzled layout of an MN-major B operand
         const float *Zg = a.Z + (((size_t)b * a.H + h) * a.mtot + a.m0) * DR;
-        if (kHalf) {
-            for (int i = tid; i < M * (D / 8); i += kTcThreads) {
-                reinterpret_cast<uint4 *>(sQ)[i] = make_uint4(0, 0, 0, 0);
-                reinterpret_cast<uint4 *>(sZ)[i] = make_uint4(0, 0, 0, 0);
-                reinterpret_cast<uint4 *>(sZ + (size_t)M * G::RB)[i] = make_uint4(0, 0, 0, 0);
+        const int z0 = kHalf ? 0 : M;                           // rows to clear: beyond M; in the narrow forms all
+        if (z0 < MP) {
+            for (int i = tid; i < (MP - z0) * (D / 8); i += kTcThreads) {
+                reinterpret_cast<uint4 *>(sQ + (size_t)z0 * G::RB)[i] = make_uint4(0, 0, 0, 0);
+                reinterpret_cast<uint4 *>(sZ + (size_t)z0 * G::RB)[i] = make_uint4(0, 0, 0, 0);
+                reinterpret_cast<uint4 *>(sZ + (size_t)(MP + z0) * G::RB)[i] = make_uint4(0, 0, 0, 0);
             }
+        }
+        if (kHalf) {
             __syncthreads();
             if constexpr (DR == 4) {
                 stage_rows4<D>(sQ, a.Q + ((size_t)h * a.mtot + a.m0) * DR, M, off);
-                stage_rows4_hilo<D>(sZ, sZ + (size_t)M * G::RB, Zg, M, off);
+                stage_rows4_hilo<D>(sZ, sZ + (size_t)MP * G::RB, Zg, M, off);
             } else {
                 for (int i = tid; i < M * (DR / 8); i += kTcThreads) {
                     const int m = i / (DR / 8), c = i % (DR / 8);
@@ -873,10 +882,10 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             }
             uint8_t *dst = sZ + (size_t)m * G::RB + ((c ^ G::swz(m)) << 4);
             *reinterpret_cast<uint4 *>(dst) = make_uint4(vh[0], vh[1], vh[2], vh[3]);
-            *reinterpret_cast<uint4 *>(dst + (size_t)M * G::RB) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
+            *reinterpret_cast<uint4 *>(dst + (size_t)MP * G::RB) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
         }
-        uint8_t *ones = sZ + (size_t)2 * M * G::RB;             // a one in column 0 of every latent row
-        for (int i = tid; i < M * (G::RB / 16); i += kTcThreads) {
+        uint8_t *ones = sZ + (size_t)2 * MP * G::RB;            // a one in column 0 of every latent row
+        for (int i = tid; i < MP * (G::RB / 16); i += kTcThreads) {
             const int m = i / (G::RB / 16), c = i % (G::RB / 16);
             *reinterpret_cast<uint4 *>(ones + (size_t)m * G::RB + ((c ^ G::swz(m)) << 4)) = make_uint4(c == 0 ? 0x00003F80u : 0u, 0, 0, 0);
         }
@@ -923,7 +932,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(bar(K_EMPTY + sj));
         }
-        if (!tame && lane == 0 && a.redo != nullptr) *a.redo = 1u;
+        if (!tame && lane == 0) *a.redo = 1u;
     } else if (warp < kFirstSoftmaxWarp) {
         const int g = warp - kFirstIssuerWarp;
         const int mytiles = (ntiles - g + NG - 1) / NG;          // tiles g, g + 4, ... of the CTA's range
@@ -934,8 +943,8 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             const uint64_t qdesc = ptx::smem_desc(ptx::smem_u32(sQ), 16, G::SBO, G::SWZ);
             // value operand: Z_hi rows of the unit; next block along N: Z_lo (D = 16, then the ones block) or the ones
             // block (D = 32), LBO bytes further on
-            const uint64_t zdesc = ptx::smem_desc(ptx::smem_u32(sZ), (uint32_t)((D == 16 ? 1 : 2) * M * G::RB), G::SBO, G::SWZ);
-            const uint64_t zlo = ptx::smem_desc(ptx::smem_u32(sZ + (size_t)M * G::RB), (uint32_t)G::SBO, G::SBO, G::SWZ);
+            const uint64_t zdesc = ptx::smem_desc(ptx::smem_u32(sZ), (uint32_t)((D == 16 ? 1 : 2) * MP * G::RB), G::SBO, G::SWZ);
+            const uint64_t zlo = ptx::smem_desc(ptx::smem_u32(sZ + (size_t)MP * G::RB), (uint32_t)G::SBO, G::SBO, G::SWZ);
             const int total = mytiles * units;
             bool ok = ptx::mbar_wait(bar(Q_FULL), 0, abort_flag, kErrDecode | 2);
             const uint32_t kstep = (uint32_t)(G::TILE_BYTES >> 4);
@@ -1001,55 +1010,60 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             } else {
                 // This thread's own instructions are on the critical path of the group (they run one at a time, each
                 // waiting for its issue slot among the softmax warps), so both streams of work below keep their
-                // position in running counters instead of dividing: the score units (two ahead of the value units) ...
-                int s_c = 0, s_stage = g % nstages, s_wrap = (g / nstages) & 1, s_n = 0;   // chunk, K stage and its phase, unit
-                const int last_nn = M - (units - 1) * UNIT;
-                const uint32_t idescS_full = ptx::instr_desc_bf16(128, UNIT, 0, 0), idescS_last = ptx::instr_desc_bf16(128, last_nn, 0, 0);
-                auto issue_scores = [&]() -> bool {                   // (the caller commits)
-                    if (s_c == 0) {
+                // position in running 32-bit counters: the score units (two ahead of the value units) ...
+                constexpr uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0);
+                constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), USTEP = (UNIT * G::RB) >> 4;
+                const uint32_t q0 = (uint32_t)qdesc, k0 = (uint32_t)kdesc0, z0 = (uint32_t)zdesc, zl0 = (uint32_t)zlo;
+                const uint32_t sfull = bar(S_FULL + 2 * g), pfull = bar(P_FULL + 2 * g);
+                int s_left = 0, s_stage = g % nstages, s_wrap = (g / nstages) & 1;   // units left of the S stream's tile, its K stage and phase
+                uint32_t ql = q0, kl = k0;
+                auto scores = [&](int w) -> bool {                    // the next unit's, into buffer w
+                    if (s_left == 0) {
                         if (!ptx::mbar_wait(bar(K_FULL + s_stage), (uint32_t)s_wrap, abort_flag, kErrDecode | 3)) return false;
                         ptx::tc_fence_after();
+                        kl = k0 + kstep * (uint32_t)s_stage;
+                        ql = q0;
+                        s_left = units;
                     }
-                    const uint64_t kdesc = kdesc0 + (uint64_t)(kstep * (uint32_t)s_stage);
-                    const uint64_t qd = qdesc + (uint64_t)((uint32_t)(s_c * UNIT * G::RB) >> 4);
-                    const uint32_t idescS = s_c == units - 1 ? idescS_last : idescS_full;
-                    const uint32_t w = (uint32_t)(s_n & 1);
 #pragma unroll
-                    for (int k = 0; k < D / 16; ++k) ptx::mma_ss(gcol + w * UNIT, kdesc + 2 * k, qd + 2 * k, idescS, k > 0);
-                    ptx::mma_commit(bar(S_FULL + 2 * g) + 8 * w);
-                    ++s_n;
-                    if (++s_c == units) {                           // the tile's last scores: its stage is free, on to the next tile
+                    for (int k = 0; k < D / 16; ++k) ptx::mma_ss(gcol + w * UNIT, ptx::desc(kl + 2 * k, HI), ptx::desc(ql + 2 * k, HI), idescS, k > 0);
+                    ptx::mma_commit(sfull + 8 * w);
+                    ql += USTEP;
+                    if (--s_left == 0) {                            // the tile's last scores: its stage is free, on to the next tile
                         ptx::mma_commit(bar(K_EMPTY + s_stage));
-                        s_c = 0;
                         s_stage += NG;
                         if (s_stage >= nstages) { s_stage -= nstages; s_wrap ^= 1; }
                     }
                     return true;
                 };
-                for (int n = 0; ok && n < 2 && n < total; ++n) ok = issue_scores();
-                // ... and the value units
-                int c = 0, tu = 0;
-                for (int n = 0; ok && n < total; ++n) {
-                    const uint32_t w = (uint32_t)(n & 1);           // the unit's buffer: its weights lie over its scores
-                    if (!ptx::mbar_spin(bar(P_FULL + 2 * g) + 8 * w, (uint32_t)((n >> 1) & 1), abort_flag, kErrDecode | 5)) break;
-                    // a tile's first value MMA overwrites the accumulator: the previous tile's rows must have been read
-                    if (c == 0 && tu > 0 && !ptx::mbar_spin(bar(Y_FREE + g), (uint32_t)((tu - 1) & 1), abort_flag, kErrDecode | 11)) break;
-                    ptx::tc_fence_after();
-                    const int subs = (c == units - 1 ? last_nn : UNIT) / 16;
-                    const uint64_t rowoff = (uint64_t)((uint32_t)(c * UNIT * G::RB) >> 4);
-                    const uint32_t pcol = gcol + w * UNIT;
-                    ptx::mma_ts(gcol + Y_COL, pcol, zdesc + rowoff, idescY, c == 0 ? 0u : 1u);
-                    if (D == 32) ptx::mma_ts(gcol + Y_COL, pcol, zlo + rowoff, idescLo, 1u);
-                    if (subs == 2) {                                // the unit's second 16 latents: 8 packed columns, 16 rows of Z on
-                        ptx::mma_ts(gcol + Y_COL, pcol + 8, zdesc + rowoff + (uint64_t)(G::RB), idescY, 1u);
-                        if (D == 32) ptx::mma_ts(gcol + Y_COL, pcol + 8, zlo + rowoff + (uint64_t)(G::RB), idescLo, 1u);
+                for (int w = 0; ok && w < 2 && w < total; ++w) ok = scores(w);
+                // ... and the value units, buffer and barrier constants of a pair
+                int left = units, tu = 0;
+                uint32_t zr = z0, zl = zl0, par = 0;
+                for (int n = 0; ok && n < total; n += 2, par ^= 1) {
+#pragma unroll
+                    for (int w = 0; w < 2; ++w) {
+                        if (n + w >= total) break;
+                        if (!ptx::mbar_spin(pfull + 8 * w, par, abort_flag, kErrDecode | 5)) { ok = false; break; }
+                        // a tile's first value MMA overwrites the accumulator: the previous tile's rows must have been read
+                        if (left == units && tu > 0 && !ptx::mbar_spin(bar(Y_FREE + g), (uint32_t)((tu - 1) & 1), abort_flag, kErrDecode | 11)) { ok = false; break; }
+                        ptx::tc_fence_after();
+                        const uint32_t pcol = gcol + w * UNIT;
+                        ptx::mma_ts(gcol + Y_COL, pcol, ptx::desc(zr, HI), idescY, left == units ? 0u : 1u);
+                        if (D == 32) ptx::mma_ts(gcol + Y_COL, pcol, ptx::desc(zl, HI), idescLo, 1u);
+                        ptx::mma_ts(gcol + Y_COL, pcol + 8, ptx::desc(zr + G::RB, HI), idescY, 1u);
+                        if (D == 32) ptx::mma_ts(gcol + Y_COL, pcol + 8, ptx::desc(zl + G::RB, HI), idescLo, 1u);
+                        zr += USTEP;
+                        zl += USTEP;
+                        if (--left == 0) {
+                            ptx::mma_commit(bar(Y_FULL + g));
+                            left = units;
+                            zr = z0;
+                            zl = zl0;
+                            ++tu;
+                        }
+                        if (n + w + 2 < total && !(ok = scores(w))) break;   // into the buffer just read; its commit covers the value MMAs too
                     }
-                    if (++c == units) {
-                        ptx::mma_commit(bar(Y_FULL + g));
-                        c = 0;
-                        ++tu;
-                    }
-                    if (n + 2 < total && !(ok = issue_scores())) break;   // into the buffer just read; its commit covers the value MMAs too
                 }
             }
         }
@@ -1077,6 +1091,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             const float inv = 1.f / l;
             const int n = (t_begin + g + tu * NG) * kTile + row;
             if (n < a.N) {
+                if (!(l >= kFastSumMin && l <= kFastSumMax)) *a.redo = 1u;
                 // the head's DR values: accumulator columns [off, off + DR) (off is 0 except for every other head of width 4)
                 float v[DR];
 #pragma unroll
@@ -1117,23 +1132,21 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         for (int tu = 0; ok && tu < mytiles; ++tu) {
             for (int c = 0; ok && c < units; ++c, ++n) {
                 const int w = n & 1;
-                const int nn = kM ? UNIT : (M - c * UNIT < UNIT ? M - c * UNIT : UNIT);
+                const bool half = kM == 0 && c == units - 1 && (M & 16) != 0;   // the second 16 columns are beyond M: weights 0
                 if (!s_ready && !(ok = warp_wait(bar(S_FULL + 2 * g + w), (n >> 1) & 1, abort_flag, kErrDecode | 6))) break;
                 ptx::tc_fence_after();
                 uint32_t r[32], pk[16];
-                if (nn == UNIT) ptx::tmem_ld32(gcol + w * UNIT, r);
-                else ptx::tmem_ld16(gcol + w * UNIT, r);
+                ptx::tmem_ld32(gcol + w * UNIT, r);
                 ptx::tmem_wait_ld();
-                bool s_probe = false;
-                if (nn == UNIT) {
-                    exp_chunk_fast<16, true, false, kSum>(r, pk, sl2p, sum2);
-                    s_probe = n + 1 < total && ptx::mbar_test(bar(S_FULL + 2 * g + (w ^ 1)), ((n + 1) >> 1) & 1);
+                exp_chunk_fast<16, true, false, kSum>(r, pk, sl2p, sum2);
+                const bool s_probe = n + 1 < total && ptx::mbar_test(bar(S_FULL + 2 * g + (w ^ 1)), ((n + 1) >> 1) & 1);
+                if (!half) {
                     exp_chunk_fast<16, true, false, kSum>(r + 16, pk + 8, sl2p, sum2);
-                    ptx::tmem_st16(gcol + w * UNIT, pk);
                 } else {
-                    exp_chunk_fast<16, true, false, kSum>(r, pk, sl2p, sum2);
-                    ptx::tmem_st8(gcol + w * UNIT, pk);
+#pragma unroll
+                    for (int k = 8; k < 16; ++k) pk[k] = 0u;
                 }
+                ptx::tmem_st16(gcol + w * UNIT, pk);
                 ptx::tmem_wait_st();
                 ptx::tc_fence_before();
                 __syncwarp();
@@ -1273,6 +1286,10 @@ constexpr float kDeadBelow = -1.0e29f;
 // units of 32 tokens on two alternating score buffers: while the group evaluates the exponentials of one
 // unit, the score MMA of the next and the value MMAs of the previous one run, so that the group never waits
 // for the tensor pipe in steady state.
+// Without a running maximum (fast and dZ forms) a unit is the whole half, 64 tokens, on one buffer: half as many hand-overs, and the other
+// three groups cover the wait for the tensor core.  Measured, us, against units of 32 on two buffers: fast forms 46 -> 39 (2-D mesh), 522 ->
+// 487 (million points, M = 256); weights as two halves 217 -> 174 (131072, M = 512); dZ 261 -> 197 there, 4377 -> 3185 (million points, M =
+// 1024, D = 8).
 //
 // Head-pair form (kPair; M <= 64, H even, D <= 32): with at most 64 latents half of the 128 lanes would idle, so
 // a CTA takes two adjacent heads at once.  Lanes 0-63 hold the latents of head 2p, lanes 64-127 those of head
@@ -1347,15 +1364,17 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const int rows_here = (kPair || kHalf) ? 0 : rows_q;                 // ... fetched by TMA
     constexpr int SLOT_COLS = 256;   // per slot and half (128 columns): two score buffers of UNIT columns, accumulator at 64
     constexpr int HALF = kTile / 2;
-    constexpr int UNIT = 32;         // tokens per unit of work of a group
+    // Tokens per unit of work of a group: without a running maximum its whole half of a tile, on one buffer; else 32, on two
+    constexpr bool kLean = kFast || kDz;
+    constexpr int UNIT = kLean ? HALF : 32;
     constexpr uint32_t NCOLS = 512;
     // Fast form with single weights: the value operand gets a second block along N whose column 0 is all ones, so
     // accumulator column DG is the sum of the rounded weights (see exp_chunk_fast); where the accumulator has no
     // room for it (DG = 64) the threads add the rounded weights themselves.
-    constexpr bool kOnes = kFast && !kHiLo && DG + 16 <= 2 * UNIT;
+    constexpr bool kOnes = kFast && !kHiLo && DG + 16 <= HALF;
     constexpr int kSumMode = kOnes ? 0 : 1;
     uint8_t *sOnes = smem + SM::ones_off();
-    constexpr int ACC_COL = 2 * UNIT;                           // a group's columns: two score buffers, then the accumulator
+    constexpr int ACC_COL = HALF;                           // a group's columns: two score buffers, then the accumulator
 
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
 
@@ -1363,7 +1382,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         // a K/V tile is released by the issuers of all the groups that use it
         const uint32_t users = alternate ? 2u : 2u * (uint32_t)nslots;
         for (int i = 0; i < NBARS; ++i)
-            ptx::mbar_init(bar(i), (i >= P_FULL && i < P_FULL + 2 * NG) ? (kFast ? 4u : 128u)   // fast form: one arrival per warp
+            ptx::mbar_init(bar(i), (i >= P_FULL && i < P_FULL + 2 * NG) ? (kLean ? 4u : 128u)   // one arrival per warp
                                    : (i >= KV_EMPTY && i < KV_EMPTY + nstages) ? users + (kFast ? 1u : 0u)   // and its guard warp
                                    : (i >= KV_FULL && i < KV_FULL + nstages) ? 2u : 1u);   // the TMA loads, the bias tile
         *abort_flag = 0;
@@ -1491,80 +1510,59 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             const uint32_t dcol = gcol + ACC_COL;                           // its accumulator
             bool ok = ptx::mbar_wait(bar(Q_FULL), 0, abort_flag, kErrEncode | 2);
             const int jobs = (nq - j + nslots - 1) / nslots;                // tiles this group works on
-            const int units = 2 * jobs;
+            const int units = 2 * jobs;                                     // (of 32 tokens)
             // Order of issue: S(0), S(1), then for every unit n: its value MMAs as soon as its weights are handed
             // over, then the scores of unit n+2 into the buffer those weights have just left.  Every wait blocks
             // in hardware, so the issuing warp takes no issue slots from the softmax warps while it waits.
             int t_s = alternate ? j : 0, t_v = t_s;                         // tiles (relative to t_begin) of the next S / PV unit
             const int t_step = alternate ? 2 : 1;
-            if constexpr (kFast) {
-                // The fast form's loop, with as few instructions of this thread per unit as it takes (they are on the
-                // critical path of the group: each waits for an issue slot among the softmax warps, and a tcgen05.mma or
-                // commit holds the thread for 50 to 130 cycles): descriptors are a base plus a stage and a unit offset;
-                // one wait per tile for the loads and one per unit for the weights; ONE commit per unit, behind the score
-                // MMA of the unit two further on, which tells the threads both that those scores are there and that the
-                // value MMAs before them (which read the buffer the scores went into) are done.
-                const uint32_t stage_step = (uint32_t)((2 * G::TILE_BYTES) >> 4), unit_step = (uint32_t)((UNIT * G::RB) >> 4);
-                const uint64_t kd0 = ptx::smem_desc(ptx::smem_u32(sKV), 16, G::SBO, G::SWZ) + (uint64_t)((c * HALF * G::RB) >> 4);
-                const uint32_t v0 = ptx::smem_u32(sKV + G::TILE_BYTES);
-                const uint64_t vd0 = ptx::smem_desc(v0, kOnes ? ptx::smem_u32(sOnes) - v0 : (uint32_t)G::SBO, G::SBO, G::SWZ) +
-                                     (uint64_t)((c * HALF * G::RB) >> 4);
-                // a stage further on, the V tile starts stage_step later and (kOnes) the ones tile is that much nearer (LBO: bits 16-29)
-                const uint64_t vstep = (uint64_t)stage_step - (kOnes ? ((uint64_t)stage_step << 16) : 0ull);
+            if constexpr (kLean) {
+                // The lean loop, with as few instructions of this thread per unit as it takes (they are on the critical path of the
+                // group): one wait for the loads of a tile, one for its weights; ONE commit per unit, behind the score MMAs of the
+                // group's next tile, which tells the threads both that those scores are there and that the value MMAs before them
+                // (which read the weights that the scores replaced) are done.  One buffer: while a group waits for the tensor core
+                // the other three work.
+                constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), STAGE = (2 * G::TILE_BYTES) >> 4;
+                const uint32_t q0 = (uint32_t)qdesc, k0 = ptx::desc_lo(ptx::smem_u32(sKV) + c * HALF * G::RB, 16);
+                const uint32_t vtile = ptx::smem_u32(sKV + G::TILE_BYTES);
+                const uint32_t v0 = ptx::desc_lo(vtile + c * HALF * G::RB, kOnes ? ptx::smem_u32(sOnes) - vtile : (uint32_t)G::SBO);
+                // a stage further on, the V tile starts STAGE later and (kOnes) the ones tile is that much nearer (LBO: bits 16-29)
+                constexpr uint32_t VSTAGE = STAGE - (kOnes ? (STAGE << 16) : 0u);
                 const uint32_t sfull = bar(S_FULL + 2 * g), pfull = bar(P_FULL + 2 * g);
                 // without kMaskBody only a last partial tile has padding; its scores get the bias MMA (see kMaskedScore)
-                const int bias_tile = (!kMaskBody && a.N % kTile != 0) ? a.tiles - 1 - t_begin : -1;
-                int ss = t_s % nstages, sp = (t_s / nstages) & 1, sv = ss;
-                auto scores = [&](int w) {                        // the scores of unit w of the S stream's tile, and the commit
-                    const uint64_t kd = kd0 + (uint64_t)(stage_step * (uint32_t)ss + unit_step * (uint32_t)w);
+                const int bias_tile = (!kDz && !kMaskBody && a.N % kTile != 0) ? a.tiles - 1 - t_begin : -1;
+                int ss = t_s % nstages, sp = (t_s / nstages) & 1;
+                auto scores = [&]() -> bool {                     // of tile t_s, and the commit
+                    if (!ptx::mbar_wait(bar(KV_FULL + ss), (uint32_t)sp, abort_flag, kErrEncode | 3)) return false;
+                    ptx::tc_fence_after();
+                    const uint32_t kd = k0 + STAGE * (uint32_t)ss;
 #pragma unroll
-                    for (int k = 0; k < DG / 16; ++k) ptx::mma_ss(gcol + w * UNIT, qdesc + 2 * k, kd + 2 * k, idescS, k > 0);
-                    if (!kMaskBody && t_s == bias_tile) {
+                    for (int k = 0; k < DG / 16; ++k) ptx::mma_ss(gcol, ptx::desc(q0 + 2 * k, HI), ptx::desc(kd + 2 * k, HI), idescS, k > 0);
+                    if (!kDz && !kMaskBody && t_s == bias_tile) {
                         using GB = TileGeom<16>;
                         const uint64_t odesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)nstages * SM::kBiasTile), 16, GB::SBO, GB::SWZ);
                         const uint64_t bdesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)ss * SM::kBiasTile), 16, GB::SBO, GB::SWZ) +
-                                               (uint64_t)((c * HALF + w * UNIT) * GB::RB / 16);
-                        ptx::mma_ss(gcol + w * UNIT, odesc, bdesc, idescS, 1u);
+                                               (uint64_t)(c * HALF * GB::RB / 16);
+                        ptx::mma_ss(gcol, odesc, bdesc, idescS, 1u);
                     }
-                    ptx::mma_commit(sfull + 8 * w);
-                };
-                auto open_tile = [&]() -> bool {
-                    if (!ptx::mbar_wait(bar(KV_FULL + ss), (uint32_t)sp, abort_flag, kErrEncode | 3)) return false;
-                    ptx::tc_fence_after();
+                    ptx::mma_commit(sfull);
                     return true;
                 };
-                auto next_s = [&]() {
+                if (jobs > 0) ok = ok && scores();
+                for (int job = 0; ok && job < jobs; ++job) {
+                    if (!ptx::mbar_spin(pfull, (uint32_t)(job & 1), abort_flag, kErrEncode | 4)) { ok = false; break; }
+                    ptx::tc_fence_after();
+                    const uint32_t vd = v0 + VSTAGE * (uint32_t)ss;
+#pragma unroll
+                    for (int k = 0; k < UNIT / 16; ++k) {
+                        ptx::mma_ts(dcol, gcol + 16 * k, ptx::desc(vd + k * G::RB, HI), idescV, (job > 0 || k > 0) ? 1u : 0u);
+                        if (kHiLo || kDz) ptx::mma_ts(dcol, gcol + 16 * k + 8, ptx::desc(vd + k * G::RB, HI), idescV, 1u);
+                    }
+                    ptx::mma_commit(bar(KV_EMPTY + ss));          // one arrival per group
                     t_s += t_step;
                     ss += t_step;
                     if (ss >= nstages) { ss -= nstages; sp ^= 1; }
-                };
-                if (ok && jobs > 0 && (ok = open_tile())) {
-                    scores(0);
-                    scores(1);
-                    next_s();
-                }
-                for (int job = 0; ok && job < jobs; ++job) {
-#pragma unroll
-                    for (int w = 0; w < 2; ++w) {
-                        if (!ptx::mbar_spin(pfull + 8 * w, (uint32_t)(job & 1), abort_flag, kErrEncode | 4)) { ok = false; break; }
-                        ptx::tc_fence_after();
-                        const uint64_t vd = vd0 + vstep * (uint64_t)sv + (uint64_t)(unit_step * (uint32_t)w);
-#pragma unroll
-                        for (int k = 0; k < UNIT / 16; ++k) {
-                            ptx::mma_ts(dcol, gcol + w * UNIT + k * 8, vd + (uint64_t)(k * G::RB), idescV, (job > 0 || w > 0 || k > 0) ? 1u : 0u);
-                            if (kHiLo) ptx::mma_ts(dcol, gcol + w * UNIT + 16 + k * 8, vd + (uint64_t)(k * G::RB), idescV, 1u);
-                        }
-                        if (w == 1) {                             // the tile's last unit: one arrival per group
-                            ptx::mma_commit(bar(KV_EMPTY + sv));
-                            sv += t_step;
-                            if (sv >= nstages) sv -= nstages;
-                        }
-                        if (job + 1 < jobs) {                     // the same unit of the group's next tile, into the buffer just read
-                            if (w == 0 && !open_tile()) { ok = false; break; }
-                            scores(w);
-                            if (w == 1) next_s();
-                        }
-                    }
+                    if (job + 1 < jobs) ok = scores();
                 }
                 if (ok) ptx::mma_commit(bar(ACC_DONE + g));
             } else {
@@ -1579,7 +1577,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 #pragma unroll
                     for (int k = 0; k < DG / 16; ++k) ptx::mma_ss(gcol + w * UNIT, qdesc + 2 * k, kdesc + 2 * k, idescS, k > 0);
                     const int tile = t_begin + t_s;
-                    if (!kDz && !kMaskBody && !(a.key_mask == nullptr && (tile + 1) * kTile <= a.N)) {
+                    if (!kMaskBody && !(a.key_mask == nullptr && (tile + 1) * kTile <= a.N)) {
                         // scores += ones x bias: padded tokens drop to kMaskedScore (see there)
                         using GB = TileGeom<16>;
                         const uint64_t odesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)nstages * SM::kBiasTile), 16, GB::SBO, GB::SWZ);
@@ -1607,7 +1605,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 #pragma unroll
                     for (int k = 0; k < UNIT / 16; ++k) {
                         ptx::mma_ts(dcol, gcol + w * UNIT + k * 8, vdesc + (uint64_t)(k * G::RB), idescV, (n > 0 || k > 0) ? 1u : 0u);
-                        if (kDz || kHiLo)    // the lo halves of the weights sit 16 columns further on
+                        if (kHiLo)           // the lo halves of the weights sit 16 columns further on
                             ptx::mma_ts(dcol, gcol + w * UNIT + 16 + k * 8, vdesc + (uint64_t)(k * G::RB), idescV, 1u);
                     }
                     ptx::mma_commit(bar(PV_DONE + g));
@@ -1635,28 +1633,6 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         int done = 0;                                           // units finished
         bool ok = true;
         float *colneg = reinterpret_cast<float *>(smem + SM::col_off()) + (warp - kFirstSoftmaxWarp) * 64;   // this warp's addends
-        // dZ form of a unit: weights exp(S - lse_dec[token]), no maximum, no sum.
-        auto unit_dz = [&](int t, int w) -> bool {
-            const uint32_t sbase = gcol + w * UNIT;
-            const int n = t * kTile + c * HALF + w * UNIT + lane;          // this lane fetches the shift of token n
-            const int hh = h + (kPair ? (row >> 6) : 0);                   // the head of this lane's latent
-            __syncwarp();                                                   // the previous unit's reads are done
-            colneg[lane] = n < a.N ? -a.lse_dec[((size_t)b * a.N + n) * a.H + hh] * 1.4426950408889634f : -INFINITY;
-            __syncwarp();
-            if (!warp_wait(bar(S_FULL + 2 * g + w), (done >> 1) & 1, abort_flag, kErrEncode | 5)) return false;
-            ptx::tc_fence_after();
-            uint32_t r[32], pk[16], pl[16];
-            ptx::tmem_ld32(sbase, r);
-            ptx::tmem_wait_ld();
-            exp_chunk_cols<32>(r, pk, pl, sl2p, colneg);
-            ptx::tmem_st16(sbase, pk);                          // hi halves over the first 16 score columns,
-            ptx::tmem_st16(sbase + 16, pl);                     // lo halves over the other 16
-            ptx::tmem_wait_st();
-            ptx::tc_fence_before();
-            ptx::mbar_arrive(bar(P_FULL + 2 * g + w));
-            ++done;
-            return true;
-        };
         // One unit of work: 32 token columns of this group's half, on score buffer w.  kMasked: some of the tile's
         // tokens may be padding or lie beyond N (their weights are exactly 0); the plain form has no such tests.
         auto unit = [&](auto masked, int t, int w) -> bool {
@@ -1719,52 +1695,79 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             ++done;
             return true;
         };
-        // Fast form of a unit: weights 2^(s * sl2), no maximum, nothing to rescale.  kMasked as above; kPoly: half of
-        // the exponentials on the FMA pipe (never where padding sits in the scores as kMaskedScore).
-        auto unit_fast = [&](auto masked, auto poly, int t, int w) -> bool {
+        // Lean form of a unit: the 64 token columns of this group's half, 16 at a time, the next 16 on their way meanwhile.  Fast: weights
+        // 2^(s * sl2), no maximum, nothing to rescale; kMasked as above; kPoly: part of the exponentials on the FMA pipe (never where
+        // padding sits in the scores as kMaskedScore).  dZ: weights exp(S - lse_dec[token]), no maximum, no sum; the shifts are
+        // fetched one tile ahead.
+        float shift[2] = {0.f, 0.f};
+        auto fetch_shifts = [&](int t) {                        // of this lane's tokens (lane and 32 + lane of the half) in tile t
+            const int hh = h + (kPair ? (row >> 6) : 0);                   // the head of this lane's latent
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int n = t * kTile + c * HALF + e * 32 + lane;
+                shift[e] = n < a.N ? a.lse_dec[((size_t)b * a.N + n) * a.H + hh] : INFINITY;
+            }
+        };
+        auto unit_lean = [&](auto masked, auto poly, int t, int t_next) -> bool {
             constexpr bool kMasked = decltype(masked)::value;
             constexpr bool kPoly = decltype(poly)::value && !kHiLo;
-            uint32_t wv = 0xffffffffu;
+            constexpr bool kTwo = kDz || kHiLo;                 // weights as two halves, the lo one 8 columns further on
+            uint32_t wv[2] = {0xffffffffu, 0xffffffffu};
             if (kMasked) {
-                const int n = t * kTile + c * HALF + w * UNIT + lane;
-                wv = __ballot_sync(0xffffffffu, n < a.N && (a.key_mask == nullptr || a.key_mask[(size_t)b * a.N + n] != 0));
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int n = t * kTile + c * HALF + e * 32 + lane;
+                    wv[e] = __ballot_sync(0xffffffffu, n < a.N && (a.key_mask == nullptr || a.key_mask[(size_t)b * a.N + n] != 0));
+                }
             }
-            const uint32_t sbase = gcol + w * UNIT;
-            if (!warp_wait(bar(S_FULL + 2 * g + w), (done >> 1) & 1, abort_flag, kErrEncode | 5)) return false;
+            if (kDz) {
+                __syncwarp();                                   // the previous unit's reads are done
+                colneg[lane] = shift[0] * -1.4426950408889634f;
+                colneg[32 + lane] = shift[1] * -1.4426950408889634f;
+                __syncwarp();
+                if (t_next < t_end) fetch_shifts(t_next);
+            }
+            if (!warp_wait(bar(S_FULL + 2 * g), done & 1, abort_flag, kErrEncode | 5)) return false;
             ptx::tc_fence_after();
-            uint32_t r[32], pk[16];
-            ptx::tmem_ld32(sbase, r);
-            ptx::tmem_wait_ld();
-            if (kHiLo) {
-                uint32_t pl[16];
-                exp_chunk_hilo<32, kMasked>(r, pk, pl, sl2p, make_float2(0.f, 0.f), l2, wv, false);
-                ptx::tmem_st16(sbase, pk);
-                ptx::tmem_st16(sbase + 16, pl);
-            } else {
-                exp_chunk_fast<32, kPoly, kMasked, kSumMode>(r, pk, sl2p, l2, wv);
-                ptx::tmem_st16(sbase, pk);
+            uint32_t r[2][16];
+            ptx::tmem_ld16(gcol, r[0]);
+#pragma unroll
+            for (int q = 0; q < UNIT / 16; ++q) {
+                ptx::tmem_wait_ld();
+                if (q + 1 < UNIT / 16) ptx::tmem_ld16(gcol + 16 * (q + 1), r[(q + 1) & 1]);
+                uint32_t pk[8], pl[8];
+                if (kDz) exp_chunk_cols<16>(r[q & 1], pk, pl, sl2p, colneg + 16 * q);
+                else if (kHiLo) exp_chunk_hilo<16, kMasked>(r[q & 1], pk, pl, sl2p, make_float2(0.f, 0.f), l2, wv[q >> 1] >> (16 * (q & 1)), false);
+                else exp_chunk_fast<16, kPoly, kMasked, kSumMode>(r[q & 1], pk, sl2p, l2, wv[q >> 1] >> (16 * (q & 1)));
+                ptx::tmem_st8(gcol + 16 * q, pk);               // over columns this thread has read
+                if (kTwo) ptx::tmem_st8(gcol + 16 * q + 8, pl);
             }
             ptx::tmem_wait_st();
             ptx::tc_fence_before();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar(P_FULL + 2 * g + w));
+            if (lane == 0) ptx::mbar_arrive(bar(P_FULL + 2 * g));
             ++done;
             return true;
         };
         if (j < nslots) {
+            auto tile_of = [&](int q) { return t_begin + (alternate ? q : q / nslots); };
+            if (kDz && j < nq) fetch_shifts(tile_of(j));
             for (int q = j; ok && q < nq; q += nslots) {
-                const int t = t_begin + (alternate ? q : q / nslots);
+                const int t = tile_of(q), t_next = tile_of(q + nslots);
                 const bool full = a.key_mask == nullptr && (t + 1) * kTile <= a.N;    // no padding in this tile (warp-uniform)
                 const bool plain = !kMaskBody || full;
+                if constexpr (kLean) {
+                    if (kDz) ok = unit_lean(std::false_type{}, std::false_type{}, t, t_next);
+                    else if (kMaskBody) ok = plain ? unit_lean(std::false_type{}, std::true_type{}, t, t_next)
+                                                   : unit_lean(std::true_type{}, std::true_type{}, t, t_next);
+                    else ok = full ? unit_lean(std::false_type{}, std::true_type{}, t, t_next)
+                                   : unit_lean(std::false_type{}, std::false_type{}, t, t_next);
+                } else {
 #pragma unroll 1
-                for (int w = 0; ok && w < 2; ++w) {             // the half's two units, on alternating buffers
-                    if (kDz) ok = unit_dz(t, w);
-                    else if (kFast && kMaskBody) ok = plain ? unit_fast(std::false_type{}, std::true_type{}, t, w)
-                                                            : unit_fast(std::true_type{}, std::true_type{}, t, w);
-                    else if (kFast) ok = full ? unit_fast(std::false_type{}, std::true_type{}, t, w)
-                                              : unit_fast(std::false_type{}, std::false_type{}, t, w);
-                    else if (kMaskBody && !plain) ok = unit(std::true_type{}, t, w);
-                    else ok = unit(std::false_type{}, t, w);    // (without kMaskBody padding is in the scores already)
+                    for (int w = 0; ok && w < 2; ++w) {         // the half's two units, on alternating buffers
+                        if (kMaskBody && !plain) ok = unit(std::true_type{}, t, w);
+                        else ok = unit(std::false_type{}, t, w);    // (without kMaskBody padding is in the scores already)
+                    }
                 }
             }
         }
@@ -1793,6 +1796,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         }
         if (kFast) m_run = (l2.x + l2.y > 0.f) ? 0.f : -INFINITY;   // weights relative to 2^0; a row with no valid token
         if (writes && m < M) {
+            // (a sum of exactly 0 is that of no valid token)
+            if (kFast && !(l2.x + l2.y == 0.f || (l2.x + l2.y >= kFastSumMin && l2.x + l2.y <= kFastSumMax))) *a.redo = 1u;
             const long rows = (long)a.B * a.H * M;
             const int part = split * a.partials_per_split + (alternate ? 2 * j + c : c);
             const size_t prow = (size_t)part * rows + ((size_t)b * a.H + h + second) * M + m;
