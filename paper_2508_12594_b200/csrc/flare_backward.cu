@@ -20,7 +20,7 @@ int launch_bwd_dq_tc_n(const flare_desc_t *d, const TcEncodePlan &p, const void 
     if ((rc = make_token_map(&tmG, dY, d, kTile, DG)) != FLARE_OK) return rc;
     static std::atomic<uint64_t> smem_opt_in{0};
     if ((rc = ensure_big_smem(bwd_dq_tc_kernel<D, kPair, DRT, kPadded>, smem_opt_in)) != FLARE_OK) return rc;
-    bwd_dq_tc_kernel<D, kPair, DRT, kPadded><<<dim3(p.splits, (kPair ? d->H / 2 : d->H) * p.pairs, d->B), kDqThreads,
+    bwd_dq_tc_kernel<D, kPair, DRT, kPadded><<<dim3((kPair ? d->H / 2 : d->H) * p.pairs, p.splits, d->B), kDqThreads,
                                                          BwdDqSmem<DG, kPair>::total, st>>>(tmK, tmV, tmG, args);
     FLARE_CUDA(cudaGetLastError());
     return FLARE_OK;
@@ -113,11 +113,11 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
     bool dz_on_tc = skip_pass_a;
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         if (!skip_pass_a && bwd_dz_on_tensor_cores(d)) {
-            const TcEncodePlan tp = tc_encode_plan(d, sms);
+            const LeanPlan tp = lean_plan(d, sms);
             uint32_t *status = reinterpret_cast<uint32_t *>(ws);
             const int rc = encode_dz_tc(d, tp, Q, K, dY, part, status, st, lse_dec);
             if (rc != FLARE_OK) return rc;
-            dz_parts = tp.P;
+            dz_parts = tp.splits;
             dz_on_tc = true;
         }
     }

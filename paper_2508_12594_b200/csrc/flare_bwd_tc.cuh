@@ -90,18 +90,6 @@ __device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float
         *reinterpret_cast<uint4 *>(lo + o) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
     }
 }
-// rows of a [rows, DR] bf16 matrix -> swizzled rows, as above
-template <int DG, int DR>
-__device__ __forceinline__ void stage_bf16(uint8_t *dst, const __nv_bfloat16 *src, int rows, int r0, int chunk0, int tid, int threads) {
-    using G = TileGeom<DG>;
-    constexpr int QC = DR >= 8 ? DR / 8 : 1;
-    for (int i = tid; i < rows * QC; i += threads) {
-        const int m = i / QC, c = i % QC, r = r0 + m;
-        *reinterpret_cast<uint4 *>(dst + (size_t)r * G::RB + (((chunk0 + c) ^ G::swz(r)) << 4)) =
-            *reinterpret_cast<const uint4 *>(src + (size_t)m * DR + c * 8);
-    }
-}
-
 // ------------------------------------------------------------------------------- pass B, latent side (dQ)
 
 // Units of 64 tokens, shared by sixteen warps, 16 columns each, on two alternating buffers of tensor memory (S | A | C; then the
@@ -149,7 +137,7 @@ struct BwdDqSmem {
     static constexpr size_t total = total_for(kStages) < kTcMinSmem ? kTcMinSmem : total_for(kStages);
 };
 
-// grid = (splits, heads or head pairs * blocks, B); a CTA takes one block of 128 latents and a contiguous range of token tiles.
+// grid = (heads or head pairs * blocks, splits, B): heads that share token rows run at the same time; a CTA takes one block of 128 latents and a contiguous range of token tiles.
 // kPair: two heads of at most 64 latents side by side on the lanes, as in the encode kernel (block-diagonal latent operands over
 // the 2 D columns the heads occupy in a token row).  DRT = 8 or 4 (with D = 16): the narrow form (the head is DRT wide in memory;
 // token tiles carry the neighbouring heads' features beside the head's own, every latent operand zeros there).
@@ -180,7 +168,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int M = a.M;
-    const int split = blockIdx.x, h = (kPair ? 2 : 1) * (blockIdx.y / a.blocks), lb = blockIdx.y % a.blocks, b = blockIdx.z;
+    const int split = blockIdx.y, h = (kPair ? 2 : 1) * (blockIdx.x / a.blocks), lb = blockIdx.x % a.blocks, b = blockIdx.z;
     const int t_begin = (int)((long)a.tiles * split / a.splits), t_end = (int)((long)a.tiles * (split + 1) / a.splits);
     const int nt = t_end - t_begin;
     const int rows_here = kPair ? M : min(M - lb * kTile, kTile);
@@ -504,18 +492,6 @@ template <int kAccCols> struct BwdGroups {
     static constexpr int kThreads = (kBwdFirstMathWarp + 4 * n) * 32;
 };
 
-// Hand-over of a group's unit n: every warp arrives on the group's barrier `full` (count 4); one of them, taking turns, waits for the others
-// and returns true: it then may issue instructions that depend on what all four wrote to (or have read from) tensor memory.
-// (A counter whose last incrementer issues would need no wait, but the acquiring read-modify-write costs every warp 250 to 400 cycles.)
-__device__ __forceinline__ bool hand_over(uint32_t full, uint32_t n, volatile uint32_t *abort_flag, uint32_t code) {
-    ptx::tc_fence_before();
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(full);
-    if (((threadIdx.x >> 5) & 3) != (n & 3)) return false;
-    const bool ok = warp_wait(full, n & 1, abort_flag, code);
-    ptx::tc_fence_after();
-    return ok;
-}
 struct BwdTokTcArgs {
     const __nv_bfloat16 *Q;    // [H,M,D]
     const float *Z, *dZ;       // [B,H,M,D]

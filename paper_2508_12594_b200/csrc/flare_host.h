@@ -208,7 +208,22 @@ inline TcEncodePlan tc_encode_plan(const flare_desc_t *d, int sms) {
     return p;
 }
 
-inline int partials_for(const flare_desc_t *d, int sms) { return use_tc(d) ? tc_encode_plan(d, sms).P : simt_plan(d, sms).P; }
+// Launch plan of the encode without a running maximum and of dZ: one partial result per CTA.  Up to 64 latents two heads share the lanes.
+struct LeanPlan { int tiles, blocks, splits; };
+inline bool lean_pairs(const flare_desc_t *d) { return d->M <= 64 && d->H % 2 == 0 && d->D >= 8 && d->D <= 32; }
+inline LeanPlan lean_plan(const flare_desc_t *d, int sms) {
+    LeanPlan p;
+    p.tiles = (d->N + kTile - 1) / kTile;
+    p.blocks = lean_pairs(d) ? 1 : (d->M + kTile - 1) / kTile;
+    const long groups = (long)d->B * (lean_pairs(d) ? d->H / 2 : d->H) * p.blocks;
+    p.splits = balanced_splits(groups, p.tiles, sms, (size_t)d->B * d->H * d->M * (d->D + 2) * sizeof(float));
+    return p;
+}
+
+// (either form of encode on the tensor cores may have to leave its partial results in the same workspace)
+inline int partials_for(const flare_desc_t *d, int sms) {
+    return use_tc(d) ? std::max(tc_encode_plan(d, sms).P, lean_plan(d, sms).splits) : simt_plan(d, sms).P;
+}
 
 // ---- TMA descriptors (the driver entry point is looked up at run time; the library does not link libcuda)
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -300,7 +315,7 @@ inline size_t decode_range_bytes(const flare_desc_t *d) {
 
 // Launch plans of the CUDA-core backward: pass A (dZ) reuses the encode plan; the dQ pass keeps three operands of a latent row
 // in registers and therefore takes fewer rows per warp.
-// Pass A (dZ) runs as the dZ form of the tensor-core encode kernel wherever that kernel runs.
+// Pass A (dZ) runs as a form of the tensor-core encode without a running maximum wherever the tensor-core kernels run.
 inline bool bwd_dz_on_tensor_cores(const flare_desc_t *d) { return use_tc(d); }
 
 // Pass B (dQ; dK and dV) runs on the tensor cores for the same shapes.
@@ -337,7 +352,7 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     const long rows = (long)d->B * d->H * d->M;
     const int pa = simt_plan(d, sms).P, pb = bwd_dq_plan(d, sms).P;
     w.P = pa > pb ? pa : pb;
-    if (bwd_dz_on_tensor_cores(d) && tc_encode_plan(d, sms).P > w.P) w.P = tc_encode_plan(d, sms).P;
+    if (bwd_dz_on_tensor_cores(d) && lean_plan(d, sms).splits > w.P) w.P = lean_plan(d, sms).splits;
     if (bwd_dq_on_tensor_cores(d) && tc_dq_plan(d, sms).P > w.P) w.P = tc_dq_plan(d, sms).P;
     size_t off = kHeaderBytes;
     w.part = off; off += align_up(sizeof(float) * (size_t)w.P * rows * d->D);
@@ -365,7 +380,7 @@ int bwd_dq_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const v
                 const float *lse_dec, float *part, cudaStream_t st);
 int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
                 float *lse_enc, void *ws, cudaStream_t st);
-int encode_dz_tc(const flare_desc_t *d, const TcEncodePlan &tp, const void *Q, const void *K, const void *dY, float *part,
+int encode_dz_tc(const flare_desc_t *d, const LeanPlan &p, const void *Q, const void *K, const void *dY, float *part,
                  uint32_t *status, cudaStream_t st, const float *lse_dec);
 // range_scratch: decode_range_bytes(d) bytes, or null (then more than kDecodeMaxM latents take the CUDA-core kernel)
 int decode_impl(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec,

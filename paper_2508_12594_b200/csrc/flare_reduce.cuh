@@ -66,12 +66,14 @@ __device__ __forceinline__ float4 sum_slices(float4 v, int slices) {
 // Log-sum-exp merge of the P partial results of every latent row (b, h, m):
 //   m* = max_p m_p;  l = sum_p l_p exp(m_p - m*);  Z = sum_p acc_p exp(m_p - m*) / l;  lse = m* + log l.
 // One pass: a thread joins its own partials relative to their maximum, four loads in flight, then the slices are joined
-// relative to the row's.  `header`: null, or the workspace header, which is cleared here (for encode kernels that leave no
+// relative to the row's.  `redo`: null, or a word that says, if not 0, that the exact form replaced the partial results
+// by P_redo of its own.  `header`: null, or the workspace header, which is cleared here (for encode kernels that leave no
 // flags in it).
 template <int L>
 __global__ void __launch_bounds__(kReduceThreads)
 merge_kernel(const float *__restrict__ part_m, const float *__restrict__ part_l, const float *__restrict__ part_acc,
-             float *__restrict__ Z, float *__restrict__ lse_enc, int P, long rows, uint32_t *header, int slices) {
+             float *__restrict__ Z, float *__restrict__ lse_enc, int P, const uint32_t *redo, int P_redo, long rows, uint32_t *header, int slices) {
+    if (redo != nullptr && *redo != 0) P = P_redo;
     const RowMap rm = row_map<L>(slices);
     const int T = L * slices;
     if (header != nullptr && blockIdx.x == 0 && threadIdx.x < kHeaderBytes / 4) header[threadIdx.x] = 0u;

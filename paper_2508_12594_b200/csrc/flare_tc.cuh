@@ -98,6 +98,31 @@ __device__ __forceinline__ void stage_rows4_hilo(uint8_t *dst_hi, uint8_t *dst_l
     }
 }
 
+// rows of a [rows, DR] bf16 matrix -> swizzled rows (DR >= 8), starting at logical chunk `chunk0` of row r0 + m
+template <int DG, int DR>
+__device__ __forceinline__ void stage_bf16(uint8_t *dst, const __nv_bfloat16 *src, int rows, int r0, int chunk0, int tid, int threads) {
+    using G = TileGeom<DG>;
+    constexpr int QC = DR >= 8 ? DR / 8 : 1;
+    for (int i = tid; i < rows * QC; i += threads) {
+        const int m = i / QC, c = i % QC, r = r0 + m;
+        *reinterpret_cast<uint4 *>(dst + (size_t)r * G::RB + (((chunk0 + c) ^ G::swz(r)) << 4)) =
+            *reinterpret_cast<const uint4 *>(src + (size_t)m * DR + c * 8);
+    }
+}
+
+// Hand-over of a group's unit n: every warp arrives on the group's barrier `full` (count 4); one of them, taking turns, waits for the others
+// and returns true: it then may issue instructions that depend on what all four wrote to (or have read from) tensor memory.
+// (A counter whose last incrementer issues would need no wait, but the acquiring read-modify-write costs every warp 250 to 400 cycles.)
+__device__ __forceinline__ bool hand_over(uint32_t full, uint32_t n, volatile uint32_t *abort_flag, uint32_t code) {
+    ptx::tc_fence_before();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(full);
+    if (((threadIdx.x >> 5) & 3) != (n & 3)) return false;
+    const bool ok = warp_wait(full, n & 1, abort_flag, code);
+    ptx::tc_fence_after();
+    return ok;
+}
+
 // ------------------------------------------------------------------------------------- softmax arithmetic
 // p = 2^(s * sl2 + neg[k]) with one addend per column (read from shared memory, four at a time): the form the
 // backward needs, where every column (token) carries its own log-sum-exp.  The weights leave as two bf16 halves,
@@ -1221,12 +1246,10 @@ decode_combine_kernel(const float *__restrict__ Ypart, const float *__restrict__
 
 struct EncodeTcArgs {
     const __nv_bfloat16 *Q;   // [H,M,D] (read directly in the head-pair form)
-    const float *lse_dec;     // [B,N,H]: only for the backward's dZ form of the kernel
     const uint8_t *key_mask;  // [B,N] or null
     float *part_m, *part_l, *part_acc;
     uint32_t *status;
     const uint32_t *run_if;   // exact forms: null, or a word that must be non-zero for the kernel to do anything
-    uint32_t *redo;           // fast forms: set to 1 if a score may lie outside the range they are valid for
     int B, H, N, M;
     float scale, sl2;
     int tiles;        // ceil(N / 128)
@@ -1240,16 +1263,12 @@ struct EncodeTcArgs {
 template <int DG, bool kAlt>
 struct EncodeSmem {
     using G = TileGeom<DG>;
-    static constexpr size_t kColBytes = 4 * kSoftmaxGroups * 2 * 32 * sizeof(float);   // per softmax warp: 2 x 32 column addends
     // score bias of padded tokens: per stage a [128 tokens, 16] bf16 tile, then one [128 latents, 16] tile of ones
     static constexpr size_t kBiasTile = kTile * 32;
-    // the tile of ones of the fast form exists only where its accumulator has room for the sum's column (DG + 16 <= 64)
-    static constexpr size_t kOnesBytes = DG + 16 <= 64 ? (size_t)kTile * G::RB : 0;
     static constexpr size_t total_for(int n) {
-        size_t t = (size_t)n * 2 * G::TILE_BYTES + (size_t)2 * kTile * G::RB + 512 + kColBytes;
+        size_t t = (size_t)n * 2 * G::TILE_BYTES + (size_t)2 * kTile * G::RB + 512;
         t = (t + 1023) & ~(size_t)1023;
-        t = (t + (size_t)(n + 1) * kBiasTile + 1023) & ~(size_t)1023;
-        return t + kOnesBytes + 1024;
+        return t + (size_t)(n + 1) * kBiasTile + 1024;
     }
     static constexpr int stages_for() {
         int n = kAlt ? kEncMaxStages : kEncStages;
@@ -1260,12 +1279,9 @@ struct EncodeSmem {
     static constexpr size_t kv_off = 0;                         // [stage][K tile | V tile]
     __host__ __device__ static size_t q_off() { return (size_t)kStages * 2 * G::TILE_BYTES; }
     __host__ __device__ static size_t bar_off() { return q_off() + (size_t)2 * kTile * G::RB; }
-    __host__ __device__ static size_t col_off() { return bar_off() + 512; }
-    __host__ __device__ static size_t bias_off() { return (col_off() + kColBytes + 1023) & ~(size_t)1023; }
-    // fast form: a [128 tokens, DG] tile with a one in column 0 of every row, the value operand's second block along N
-    __host__ __device__ static size_t ones_off() { return (bias_off() + (kStages + 1) * kBiasTile + 1023) & ~(size_t)1023; }
+    __host__ __device__ static size_t bias_off() { return (bar_off() + 512 + 1023) & ~(size_t)1023; }
     __host__ __device__ static size_t total() {
-        size_t t = ones_off() + kOnesBytes + 1024;
+        size_t t = bias_off() + (kStages + 1) * kBiasTile + 1024;
         return t < kTcMinSmem ? kTcMinSmem : t;
     }
 };
@@ -1286,10 +1302,6 @@ constexpr float kDeadBelow = -1.0e29f;
 // units of 32 tokens on two alternating score buffers: while the group evaluates the exponentials of one
 // unit, the score MMA of the next and the value MMAs of the previous one run, so that the group never waits
 // for the tensor pipe in steady state.
-// Without a running maximum (fast and dZ forms) a unit is the whole half, 64 tokens, on one buffer: half as many hand-overs, and the other
-// three groups cover the wait for the tensor core.  Measured, us, against units of 32 on two buffers: fast forms 46 -> 39 (2-D mesh), 522 ->
-// 487 (million points, M = 256); weights as two halves 217 -> 174 (131072, M = 512); dZ 261 -> 197 there, 4377 -> 3185 (million points, M =
-// 1024, D = 8).
 //
 // Head-pair form (kPair; M <= 64, H even, D <= 32): with at most 64 latents half of the 128 lanes would idle, so
 // a CTA takes two adjacent heads at once.  Lanes 0-63 hold the latents of head 2p, lanes 64-127 those of head
@@ -1297,31 +1309,20 @@ constexpr float kDeadBelow = -1.0e29f;
 // side by side in a token row, so one MMA with K = 2D gives every lane its own head's scores, and the value MMA
 // with N = 2D gives lanes 0-63 their rows in accumulator columns [0, D) and lanes 64-127 theirs in [D, 2D).
 //
-// dZ form (kDz; pass A of the backward): the same kernel with dY in place of V and the decode weights in place of
-// the encode weights, dZ_m = sum_n exp(S[m,n] - lse_dec[n]) dY_n.  Every column (token) carries its own shift
-// and the weights are already normalised, so there is no running maximum, no rescaling and no sum; tokens
-// beyond N get the shift -inf.  Every group leaves one partial sum of dZ per split (part_acc).
-//
 // Narrow form (DRT = 8 or 4 with D = 16; not with kPair): the head is DRT wide in memory, as in the decode kernel:
 // K and V tile rows carry the neighbouring heads' features beside the head's own, Q rows zeros there; accumulator
 // columns outside the head's (weights times the neighbours' values) are dropped.
 //
-// kHiLo: the weights go to the value contraction as two bf16 halves (see exp_chunk_hilo), as in the dZ form.
+// kHiLo: the weights go to the value contraction as two bf16 halves (see exp_chunk_hilo).
 //
 // kMaskBody: padded tokens are handled by a second form of the unit body that tests every element (the form for
 // calls with a key mask, where every tile has padding); without it they are handled in the scores (kMaskedScore),
 // which costs a bias tile and one more MMA per unit of the tiles that have padding, and nothing elsewhere.
-//
-// kFast: no running maximum (see kFastMaxLog2): weights 2^(s * sl2) as they stand, half of them by the polynomial
-// on the FMA pipe (not with kHiLo, whose point is accuracy), no rescaling, partial maximum 0.  Three more warps
-// (the guard warps) check the norms of the key rows of every tile against those of the CTA's latent rows; in the
-// producer warp that check sat between two loads and cost 10 % at D = 32 (measured).
-template <int D, bool kPair, bool kDz = false, int DRT = 0, bool kHiLo = false, bool kMaskBody = false, bool kFast = false, bool kAlt = kPair>
-__global__ void __launch_bounds__(kFast ? kTcThreadsGuarded : kTcThreads, 1)
+template <int D, bool kPair, int DRT = 0, bool kHiLo = false, bool kMaskBody = false, bool kAlt = kPair>
+__global__ void __launch_bounds__(kTcThreads, 1)
 encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                  const __grid_constant__ CUtensorMap tmQ, EncodeTcArgs a) {
-    static_assert(!(kFast && kDz), "the dZ form has no maximum to drop");
-    if (!kFast && a.run_if != nullptr && *a.run_if == 0) return;      // the exact form as a fallback that was not needed
+    if (a.run_if != nullptr && *a.run_if == 0) return;      // the exact form as a fallback that was not needed
     constexpr bool kHalf = DRT != 0;
     static_assert(!(kPair && kHalf), "head pairing and the narrow form exclude each other");
     constexpr int DG = kPair ? 2 * D : D;
@@ -1344,7 +1345,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
-    const int tid = threadIdx.x < kTcThreads ? (int)threadIdx.x : (1 << 30);   // the guard warps stage nothing
+    const int tid = threadIdx.x;
     const int M = a.M;
     // h: the head, or in the head-pair form the first head of the pair
     const int split = blockIdx.x, h = (kPair ? 2 : 1) * (blockIdx.y / a.pairs), pair = blockIdx.y % a.pairs, b = blockIdx.z;
@@ -1364,16 +1365,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const int rows_here = (kPair || kHalf) ? 0 : rows_q;                 // ... fetched by TMA
     constexpr int SLOT_COLS = 256;   // per slot and half (128 columns): two score buffers of UNIT columns, accumulator at 64
     constexpr int HALF = kTile / 2;
-    // Tokens per unit of work of a group: without a running maximum its whole half of a tile, on one buffer; else 32, on two
-    constexpr bool kLean = kFast || kDz;
-    constexpr int UNIT = kLean ? HALF : 32;
+    constexpr int UNIT = 32;         // tokens per unit of work of a group
     constexpr uint32_t NCOLS = 512;
-    // Fast form with single weights: the value operand gets a second block along N whose column 0 is all ones, so
-    // accumulator column DG is the sum of the rounded weights (see exp_chunk_fast); where the accumulator has no
-    // room for it (DG = 64) the threads add the rounded weights themselves.
-    constexpr bool kOnes = kFast && !kHiLo && DG + 16 <= HALF;
-    constexpr int kSumMode = kOnes ? 0 : 1;
-    uint8_t *sOnes = smem + SM::ones_off();
     constexpr int ACC_COL = HALF;                           // a group's columns: two score buffers, then the accumulator
 
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
@@ -1382,8 +1375,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         // a K/V tile is released by the issuers of all the groups that use it
         const uint32_t users = alternate ? 2u : 2u * (uint32_t)nslots;
         for (int i = 0; i < NBARS; ++i)
-            ptx::mbar_init(bar(i), (i >= P_FULL && i < P_FULL + 2 * NG) ? (kLean ? 4u : 128u)   // one arrival per warp
-                                   : (i >= KV_EMPTY && i < KV_EMPTY + nstages) ? users + (kFast ? 1u : 0u)   // and its guard warp
+            ptx::mbar_init(bar(i), (i >= P_FULL && i < P_FULL + 2 * NG) ? 128u
+                                   : (i >= KV_EMPTY && i < KV_EMPTY + nstages) ? users
                                    : (i >= KV_FULL && i < KV_FULL + nstages) ? 2u : 1u);   // the TMA loads, the bias tile
         *abort_flag = 0;
         ptx::fence_mbar_init();
@@ -1396,19 +1389,12 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     for (int i = tid; i < (2 * kTile - rows_here) * (G::RB / 16); i += kTcThreads)
         reinterpret_cast<uint4 *>(sQ + (size_t)rows_here * G::RB)[i] = make_uint4(0, 0, 0, 0);
     uint8_t *sBias = smem + SM::bias_off();                     // [stage] bias tiles, then the tile of ones
-    if (!kDz) {
+    {
         using GB = TileGeom<16>;
         uint8_t *ones = sBias + (size_t)nstages * SM::kBiasTile;
         for (int r = tid; r < kTile; r += kTcThreads) {   // row r = [1, 0, ..., 0]: the first 16-byte chunk, swizzled
             reinterpret_cast<uint4 *>(ones + (size_t)r * GB::RB)[GB::swz(r)] = make_uint4(0x00003F80u, 0, 0, 0);
             reinterpret_cast<uint4 *>(ones + (size_t)r * GB::RB)[GB::swz(r) ^ 1] = make_uint4(0, 0, 0, 0);
-        }
-    }
-    if (kOnes) {
-        for (int i = tid; i < kTile * (G::RB / 16); i += kTcThreads) {
-            const int r = i / (G::RB / 16), ch = i % (G::RB / 16);
-            *reinterpret_cast<uint4 *>(sOnes + (size_t)r * G::RB + ((ch ^ G::swz(r)) << 4)) =
-                make_uint4(ch == 0 ? 0x00003F80u : 0u, 0, 0, 0);
         }
     }
     if (kPair) {
@@ -1455,7 +1441,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         for (int i = 0; i < nt; ++i) {
             const int s = i % nstages, t = t_begin + i;
             if (!warp_wait(bar(KV_EMPTY + s), ((i / nstages) & 1) ^ 1, abort_flag, kErrEncode | 1)) break;
-            const bool plain = kDz || kMaskBody || (a.key_mask == nullptr && (t + 1) * kTile <= a.N);
+            const bool plain = kMaskBody || (a.key_mask == nullptr && (t + 1) * kTile <= a.N);
             if (!plain) {
                 using GB = TileGeom<16>;
                 uint8_t *bt = sBias + (size_t)s * SM::kBiasTile;
@@ -1478,31 +1464,12 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 ptx::tma_load_3d(ptx::smem_u32(dst + G::TILE_BYTES), &tmV, bar(KV_FULL + s), h * DR - off, t * kTile, b);
             }
         }
-    } else if (kFast && warp >= kFirstGuardWarp) {
-        // Guard warps (fast form), one tile in three each: the largest |k|^2 a tile may hold so that |q| |k| sl2 <=
-        // kFastMaxLog2 for the CTA's latent rows, checked while the tile sits in its stage; the stage is released by
-        // its users and its guard.  (Whole rows of both operands: in the head-pair and narrow forms they hold the
-        // neighbouring heads' features too, which only makes the check stricter.)
-        bool tame = warp_wait(bar(Q_FULL), 0, abort_flag, kErrEncode | 8);
-        const float q2 = warp_max_nan(tile_max_norm2<G::RB>(sQ, 2 * kTile, lane));
-        const float lim = kFastMaxLog2 / a.sl2;
-        const float k2_limit = lim * lim / fmaxf(q2, 1e-30f);
-        if (!(q2 <= 3.0e38f)) tame = false;                     // NaN or infinity in Q
-        for (int j = warp - kFirstGuardWarp; j < nt; j += kGuardWarps) {
-            const int sj = j % nstages;
-            if (!warp_wait(bar(KV_FULL + sj), (j / nstages) & 1, abort_flag, kErrEncode | 9)) break;
-            const float k2 = warp_max_nan(tile_max_norm2<G::RB, kPair ? 2 : 1>(sKV + (size_t)sj * 2 * G::TILE_BYTES, kTile, lane));
-            if (!(k2 <= k2_limit)) tame = false;
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar(KV_EMPTY + sj));
-        }
-        if (!tame && lane == 0) *a.redo = 1u;
     } else if (warp < kFirstSoftmaxWarp) {
         const int g = warp - kFirstIssuerWarp;                  // the group this warp issues MMAs for
         const int j = g >> 1, c = g & 1;                        // its slot and column half
         if (j < nslots && ptx::elect_one()) {
             const uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0);
-            const uint32_t idescV = ptx::instr_desc_bf16(128, kOnes ? DG + 16 : DG, 0, 1);
+            const uint32_t idescV = ptx::instr_desc_bf16(128, DG, 0, 1);
             // Q rows of the slot's latent block (K-major A operand); descriptor address fields are in 16-byte units
             const uint64_t qdesc = ptx::smem_desc(ptx::smem_u32(sQ), 16, G::SBO, G::SWZ) +
                                    (uint64_t)(alternate ? 0 : j * kTile * G::RB / 16);
@@ -1516,109 +1483,58 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             // in hardware, so the issuing warp takes no issue slots from the softmax warps while it waits.
             int t_s = alternate ? j : 0, t_v = t_s;                         // tiles (relative to t_begin) of the next S / PV unit
             const int t_step = alternate ? 2 : 1;
-            if constexpr (kLean) {
-                // The lean loop, with as few instructions of this thread per unit as it takes (they are on the critical path of the
-                // group): one wait for the loads of a tile, one for its weights; ONE commit per unit, behind the score MMAs of the
-                // group's next tile, which tells the threads both that those scores are there and that the value MMAs before them
-                // (which read the weights that the scores replaced) are done.  One buffer: while a group waits for the tensor core
-                // the other three work.
-                constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), STAGE = (2 * G::TILE_BYTES) >> 4;
-                const uint32_t q0 = (uint32_t)qdesc, k0 = ptx::desc_lo(ptx::smem_u32(sKV) + c * HALF * G::RB, 16);
-                const uint32_t vtile = ptx::smem_u32(sKV + G::TILE_BYTES);
-                const uint32_t v0 = ptx::desc_lo(vtile + c * HALF * G::RB, kOnes ? ptx::smem_u32(sOnes) - vtile : (uint32_t)G::SBO);
-                // a stage further on, the V tile starts STAGE later and (kOnes) the ones tile is that much nearer (LBO: bits 16-29)
-                constexpr uint32_t VSTAGE = STAGE - (kOnes ? (STAGE << 16) : 0u);
-                const uint32_t sfull = bar(S_FULL + 2 * g), pfull = bar(P_FULL + 2 * g);
-                // without kMaskBody only a last partial tile has padding; its scores get the bias MMA (see kMaskedScore)
-                const int bias_tile = (!kDz && !kMaskBody && a.N % kTile != 0) ? a.tiles - 1 - t_begin : -1;
-                int ss = t_s % nstages, sp = (t_s / nstages) & 1;
-                auto scores = [&]() -> bool {                     // of tile t_s, and the commit
-                    if (!ptx::mbar_wait(bar(KV_FULL + ss), (uint32_t)sp, abort_flag, kErrEncode | 3)) return false;
-                    ptx::tc_fence_after();
-                    const uint32_t kd = k0 + STAGE * (uint32_t)ss;
+            int s_stage = t_s % nstages, s_phase = (t_s / nstages) & 1;   // stage and phase of the S stream's tile
+            auto issue_scores = [&](int n) -> bool {
+                const int s = s_stage, w = n & 1;                        // w: which 32 tokens of the half; also the buffer
+                if (!ptx::mbar_wait(bar(KV_FULL + s), s_phase, abort_flag, kErrEncode | 3)) return false;
+                ptx::tc_fence_after();
+                // S_unit = Q_block K_unit^T: the unit's 32 token rows of the K tile are the B operand
+                const uint64_t kdesc = ptx::smem_desc(ptx::smem_u32(sKV + (size_t)s * 2 * G::TILE_BYTES), 16, G::SBO, G::SWZ) +
+                                       (uint64_t)((c * HALF + w * UNIT) * G::RB / 16);
 #pragma unroll
-                    for (int k = 0; k < DG / 16; ++k) ptx::mma_ss(gcol, ptx::desc(q0 + 2 * k, HI), ptx::desc(kd + 2 * k, HI), idescS, k > 0);
-                    if (!kDz && !kMaskBody && t_s == bias_tile) {
-                        using GB = TileGeom<16>;
-                        const uint64_t odesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)nstages * SM::kBiasTile), 16, GB::SBO, GB::SWZ);
-                        const uint64_t bdesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)ss * SM::kBiasTile), 16, GB::SBO, GB::SWZ) +
-                                               (uint64_t)(c * HALF * GB::RB / 16);
-                        ptx::mma_ss(gcol, odesc, bdesc, idescS, 1u);
-                    }
-                    ptx::mma_commit(sfull);
-                    return true;
-                };
-                if (jobs > 0) ok = ok && scores();
-                for (int job = 0; ok && job < jobs; ++job) {
-                    if (!ptx::mbar_spin(pfull, (uint32_t)(job & 1), abort_flag, kErrEncode | 4)) { ok = false; break; }
-                    ptx::tc_fence_after();
-                    const uint32_t vd = v0 + VSTAGE * (uint32_t)ss;
-#pragma unroll
-                    for (int k = 0; k < UNIT / 16; ++k) {
-                        ptx::mma_ts(dcol, gcol + 16 * k, ptx::desc(vd + k * G::RB, HI), idescV, (job > 0 || k > 0) ? 1u : 0u);
-                        if (kHiLo || kDz) ptx::mma_ts(dcol, gcol + 16 * k + 8, ptx::desc(vd + k * G::RB, HI), idescV, 1u);
-                    }
-                    ptx::mma_commit(bar(KV_EMPTY + ss));          // one arrival per group
+                for (int k = 0; k < DG / 16; ++k) ptx::mma_ss(gcol + w * UNIT, qdesc + 2 * k, kdesc + 2 * k, idescS, k > 0);
+                const int tile = t_begin + t_s;
+                if (!kMaskBody && !(a.key_mask == nullptr && (tile + 1) * kTile <= a.N)) {
+                    // scores += ones x bias: padded tokens drop to kMaskedScore (see there)
+                    using GB = TileGeom<16>;
+                    const uint64_t odesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)nstages * SM::kBiasTile), 16, GB::SBO, GB::SWZ);
+                    const uint64_t bdesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)s * SM::kBiasTile), 16, GB::SBO, GB::SWZ) +
+                                           (uint64_t)((c * HALF + w * UNIT) * GB::RB / 16);
+                    ptx::mma_ss(gcol + w * UNIT, odesc, bdesc, idescS, 1u);
+                }
+                ptx::mma_commit(bar(S_FULL + 2 * g + w));
+                if (w == 1) {
                     t_s += t_step;
-                    ss += t_step;
-                    if (ss >= nstages) { ss -= nstages; sp ^= 1; }
-                    if (job + 1 < jobs) ok = scores();
+                    s_stage += t_step;
+                    if (s_stage >= nstages) { s_stage -= nstages; s_phase ^= 1; }
                 }
-                if (ok) ptx::mma_commit(bar(ACC_DONE + g));
-            } else {
-                int s_stage = t_s % nstages, s_phase = (t_s / nstages) & 1;   // stage and phase of the S stream's tile
-                auto issue_scores = [&](int n) -> bool {
-                    const int s = s_stage, w = n & 1;                        // w: which 32 tokens of the half; also the buffer
-                    if (!ptx::mbar_wait(bar(KV_FULL + s), s_phase, abort_flag, kErrEncode | 3)) return false;
-                    ptx::tc_fence_after();
-                    // S_unit = Q_block K_unit^T: the unit's 32 token rows of the K tile are the B operand
-                    const uint64_t kdesc = ptx::smem_desc(ptx::smem_u32(sKV + (size_t)s * 2 * G::TILE_BYTES), 16, G::SBO, G::SWZ) +
-                                           (uint64_t)((c * HALF + w * UNIT) * G::RB / 16);
+                return true;
+            };
+            for (int n = 0; ok && n < 2 && n < units; ++n) ok = issue_scores(n);
+            int v_stage = t_v % nstages;
+            for (int n = 0; ok && n < units; ++n) {
+                const int w = n & 1, s = v_stage;
+                if (!ptx::mbar_wait(bar(P_FULL + 2 * g + w), (n >> 1) & 1, abort_flag, kErrEncode | 4)) break;
+                ptx::tc_fence_after();
+                // acc += P_unit V_unit: V tile as the MN-major B operand, 16 token rows further on per k-step
+                const uint64_t vdesc = ptx::smem_desc(ptx::smem_u32(sKV + (size_t)s * 2 * G::TILE_BYTES + G::TILE_BYTES),
+                                                      G::SBO, G::SBO, G::SWZ) + (uint64_t)((c * HALF + w * UNIT) * G::RB / 16);
 #pragma unroll
-                    for (int k = 0; k < DG / 16; ++k) ptx::mma_ss(gcol + w * UNIT, qdesc + 2 * k, kdesc + 2 * k, idescS, k > 0);
-                    const int tile = t_begin + t_s;
-                    if (!kMaskBody && !(a.key_mask == nullptr && (tile + 1) * kTile <= a.N)) {
-                        // scores += ones x bias: padded tokens drop to kMaskedScore (see there)
-                        using GB = TileGeom<16>;
-                        const uint64_t odesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)nstages * SM::kBiasTile), 16, GB::SBO, GB::SWZ);
-                        const uint64_t bdesc = ptx::smem_desc(ptx::smem_u32(sBias + (size_t)s * SM::kBiasTile), 16, GB::SBO, GB::SWZ) +
-                                               (uint64_t)((c * HALF + w * UNIT) * GB::RB / 16);
-                        ptx::mma_ss(gcol + w * UNIT, odesc, bdesc, idescS, 1u);
-                    }
-                    ptx::mma_commit(bar(S_FULL + 2 * g + w));
-                    if (w == 1) {
-                        t_s += t_step;
-                        s_stage += t_step;
-                        if (s_stage >= nstages) { s_stage -= nstages; s_phase ^= 1; }
-                    }
-                    return true;
-                };
-                for (int n = 0; ok && n < 2 && n < units; ++n) ok = issue_scores(n);
-                int v_stage = t_v % nstages;
-                for (int n = 0; ok && n < units; ++n) {
-                    const int w = n & 1, s = v_stage;
-                    if (!ptx::mbar_wait(bar(P_FULL + 2 * g + w), (n >> 1) & 1, abort_flag, kErrEncode | 4)) break;
-                    ptx::tc_fence_after();
-                    // acc += P_unit V_unit: V tile as the MN-major B operand, 16 token rows further on per k-step
-                    const uint64_t vdesc = ptx::smem_desc(ptx::smem_u32(sKV + (size_t)s * 2 * G::TILE_BYTES + G::TILE_BYTES),
-                                                          G::SBO, G::SBO, G::SWZ) + (uint64_t)((c * HALF + w * UNIT) * G::RB / 16);
-#pragma unroll
-                    for (int k = 0; k < UNIT / 16; ++k) {
-                        ptx::mma_ts(dcol, gcol + w * UNIT + k * 8, vdesc + (uint64_t)(k * G::RB), idescV, (n > 0 || k > 0) ? 1u : 0u);
-                        if (kHiLo)           // the lo halves of the weights sit 16 columns further on
-                            ptx::mma_ts(dcol, gcol + w * UNIT + 16 + k * 8, vdesc + (uint64_t)(k * G::RB), idescV, 1u);
-                    }
-                    ptx::mma_commit(bar(PV_DONE + g));
-                    if (w == 1) {                                           // the tile's last unit: one arrival per group
-                        ptx::mma_commit(bar(KV_EMPTY + s));
-                        t_v += t_step;
-                        v_stage += t_step;
-                        if (v_stage >= nstages) v_stage -= nstages;
-                    }
-                    if (n + 2 < units) ok = issue_scores(n + 2);
+                for (int k = 0; k < UNIT / 16; ++k) {
+                    ptx::mma_ts(dcol, gcol + w * UNIT + k * 8, vdesc + (uint64_t)(k * G::RB), idescV, (n > 0 || k > 0) ? 1u : 0u);
+                    if (kHiLo)           // the lo halves of the weights sit 16 columns further on
+                        ptx::mma_ts(dcol, gcol + w * UNIT + 16 + k * 8, vdesc + (uint64_t)(k * G::RB), idescV, 1u);
                 }
-                if (ok) ptx::mma_commit(bar(ACC_DONE + g));
+                ptx::mma_commit(bar(PV_DONE + g));
+                if (w == 1) {                                           // the tile's last unit: one arrival per group
+                    ptx::mma_commit(bar(KV_EMPTY + s));
+                    t_v += t_step;
+                    v_stage += t_step;
+                    if (v_stage >= nstages) v_stage -= nstages;
+                }
+                if (n + 2 < units) ok = issue_scores(n + 2);
             }
+            if (ok) ptx::mma_commit(bar(ACC_DONE + g));
         }
     } else {
         const int g = (warp - kFirstSoftmaxWarp) >> 2;          // softmax group
@@ -1632,7 +1548,6 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         float2 l2 = make_float2(0.f, 0.f);
         int done = 0;                                           // units finished
         bool ok = true;
-        float *colneg = reinterpret_cast<float *>(smem + SM::col_off()) + (warp - kFirstSoftmaxWarp) * 64;   // this warp's addends
         // One unit of work: 32 token columns of this group's half, on score buffer w.  kMasked: some of the tile's
         // tokens may be padding or lie beyond N (their weights are exactly 0); the plain form has no such tests.
         auto unit = [&](auto masked, int t, int w) -> bool {
@@ -1695,79 +1610,14 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             ++done;
             return true;
         };
-        // Lean form of a unit: the 64 token columns of this group's half, 16 at a time, the next 16 on their way meanwhile.  Fast: weights
-        // 2^(s * sl2), no maximum, nothing to rescale; kMasked as above; kPoly: part of the exponentials on the FMA pipe (never where
-        // padding sits in the scores as kMaskedScore).  dZ: weights exp(S - lse_dec[token]), no maximum, no sum; the shifts are
-        // fetched one tile ahead.
-        float shift[2] = {0.f, 0.f};
-        auto fetch_shifts = [&](int t) {                        // of this lane's tokens (lane and 32 + lane of the half) in tile t
-            const int hh = h + (kPair ? (row >> 6) : 0);                   // the head of this lane's latent
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int n = t * kTile + c * HALF + e * 32 + lane;
-                shift[e] = n < a.N ? a.lse_dec[((size_t)b * a.N + n) * a.H + hh] : INFINITY;
-            }
-        };
-        auto unit_lean = [&](auto masked, auto poly, int t, int t_next) -> bool {
-            constexpr bool kMasked = decltype(masked)::value;
-            constexpr bool kPoly = decltype(poly)::value && !kHiLo;
-            constexpr bool kTwo = kDz || kHiLo;                 // weights as two halves, the lo one 8 columns further on
-            uint32_t wv[2] = {0xffffffffu, 0xffffffffu};
-            if (kMasked) {
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int n = t * kTile + c * HALF + e * 32 + lane;
-                    wv[e] = __ballot_sync(0xffffffffu, n < a.N && (a.key_mask == nullptr || a.key_mask[(size_t)b * a.N + n] != 0));
-                }
-            }
-            if (kDz) {
-                __syncwarp();                                   // the previous unit's reads are done
-                colneg[lane] = shift[0] * -1.4426950408889634f;
-                colneg[32 + lane] = shift[1] * -1.4426950408889634f;
-                __syncwarp();
-                if (t_next < t_end) fetch_shifts(t_next);
-            }
-            if (!warp_wait(bar(S_FULL + 2 * g), done & 1, abort_flag, kErrEncode | 5)) return false;
-            ptx::tc_fence_after();
-            uint32_t r[2][16];
-            ptx::tmem_ld16(gcol, r[0]);
-#pragma unroll
-            for (int q = 0; q < UNIT / 16; ++q) {
-                ptx::tmem_wait_ld();
-                if (q + 1 < UNIT / 16) ptx::tmem_ld16(gcol + 16 * (q + 1), r[(q + 1) & 1]);
-                uint32_t pk[8], pl[8];
-                if (kDz) exp_chunk_cols<16>(r[q & 1], pk, pl, sl2p, colneg + 16 * q);
-                else if (kHiLo) exp_chunk_hilo<16, kMasked>(r[q & 1], pk, pl, sl2p, make_float2(0.f, 0.f), l2, wv[q >> 1] >> (16 * (q & 1)), false);
-                else exp_chunk_fast<16, kPoly, kMasked, kSumMode>(r[q & 1], pk, sl2p, l2, wv[q >> 1] >> (16 * (q & 1)));
-                ptx::tmem_st8(gcol + 16 * q, pk);               // over columns this thread has read
-                if (kTwo) ptx::tmem_st8(gcol + 16 * q + 8, pl);
-            }
-            ptx::tmem_wait_st();
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar(P_FULL + 2 * g));
-            ++done;
-            return true;
-        };
         if (j < nslots) {
-            auto tile_of = [&](int q) { return t_begin + (alternate ? q : q / nslots); };
-            if (kDz && j < nq) fetch_shifts(tile_of(j));
             for (int q = j; ok && q < nq; q += nslots) {
-                const int t = tile_of(q), t_next = tile_of(q + nslots);
-                const bool full = a.key_mask == nullptr && (t + 1) * kTile <= a.N;    // no padding in this tile (warp-uniform)
-                const bool plain = !kMaskBody || full;
-                if constexpr (kLean) {
-                    if (kDz) ok = unit_lean(std::false_type{}, std::false_type{}, t, t_next);
-                    else if (kMaskBody) ok = plain ? unit_lean(std::false_type{}, std::true_type{}, t, t_next)
-                                                   : unit_lean(std::true_type{}, std::true_type{}, t, t_next);
-                    else ok = full ? unit_lean(std::false_type{}, std::true_type{}, t, t_next)
-                                   : unit_lean(std::false_type{}, std::false_type{}, t, t_next);
-                } else {
+                const int t = t_begin + (alternate ? q : q / nslots);
+                const bool plain = !kMaskBody || (a.key_mask == nullptr && (t + 1) * kTile <= a.N);   // no padding in this tile (warp-uniform)
 #pragma unroll 1
-                    for (int w = 0; ok && w < 2; ++w) {         // the half's two units, on alternating buffers
-                        if (kMaskBody && !plain) ok = unit(std::true_type{}, t, w);
-                        else ok = unit(std::false_type{}, t, w);    // (without kMaskBody padding is in the scores already)
-                    }
+                for (int w = 0; ok && w < 2; ++w) {             // the half's two units, on alternating buffers
+                    if (kMaskBody && !plain) ok = unit(std::true_type{}, t, w);
+                    else ok = unit(std::false_type{}, t, w);    // (without kMaskBody padding is in the scores already)
                 }
             }
         }
@@ -1783,28 +1633,17 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         if (done > 0) {
 #pragma unroll
             for (int dc = 0; dc < D / 16; ++dc) ptx::tmem_ld16(abase + second * D + dc * 16, acc + dc * 16);
-            if (kOnes) {                                        // column DG: the sum of the weights
-                uint32_t t8[8];
-                ptx::tmem_ld8(abase + DG, t8);
-                ptx::tmem_wait_ld();
-                l2 = make_float2(__uint_as_float(t8[0]), 0.f);
-            }
             ptx::tmem_wait_ld();
         } else {
 #pragma unroll
             for (int k = 0; k < D; ++k) acc[k] = 0u;
         }
-        if (kFast) m_run = (l2.x + l2.y > 0.f) ? 0.f : -INFINITY;   // weights relative to 2^0; a row with no valid token
         if (writes && m < M) {
-            // (a sum of exactly 0 is that of no valid token)
-            if (kFast && !(l2.x + l2.y == 0.f || (l2.x + l2.y >= kFastSumMin && l2.x + l2.y <= kFastSumMax))) *a.redo = 1u;
             const long rows = (long)a.B * a.H * M;
             const int part = split * a.partials_per_split + (alternate ? 2 * j + c : c);
             const size_t prow = (size_t)part * rows + ((size_t)b * a.H + h + second) * M + m;
-            if (!kDz) {
-                a.part_m[prow] = (m_run < kDeadBelow) ? -INFINITY : m_run * a.scale;
-                a.part_l[prow] = l2.x + l2.y;
-            }
+            a.part_m[prow] = (m_run < kDeadBelow) ? -INFINITY : m_run * a.scale;
+            a.part_l[prow] = l2.x + l2.y;
             float4 *dst = reinterpret_cast<float4 *>(a.part_acc + prow * DR);
             if (DR == 4) {
                 dst[0] = make_float4(__uint_as_float(off ? acc[4] : acc[0]), __uint_as_float(off ? acc[5] : acc[1]),

@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,H,N,M,D,masked", [
     (1, 2, 63, 16, 16, 0.0), (1, 2, 65, 48, 32, 0.2), (2, 3, 129, 80, 8, 0.0), (1, 1, 300, 96, 32, 0.0), (1, 2, 1500, 112, 16, 0.3),
     (1, 2, 191, 144, 32, 0.0), (1, 1, 2700, 176, 16, 0.0), (1, 1, 200, 272, 8, 0.1), (1, 2, 321, 320, 32, 0.0), (1, 1, 130, 528, 16, 0.0),
-    (1, 4, 700, 64, 4, 0.1)])
+    (1, 4, 700, 64, 4, 0.1), (1, 2, 200, 48, 8, 0.2), (2, 4, 129, 64, 8, 0.0), (1, 2, 2600, 16, 8, 0.0)])
 def test_unit_edges(oracle, B, H, N, M, D, masked, stats):
     inp = workloads.make_random(B, H, N, M, D, dtype="bf16", seed=N + M, masked_fraction=masked, k_std=0.8)
     got = gpu_forward(inp, stats=stats, path=flare.PATH_FAST)
@@ -41,3 +41,21 @@ def test_sums_out_of_range_hand_over(oracle, score, redo):
     words = ws[:16].view(torch.int32).cpu()
     assert words[0] == 0 and bool(words[2]) == redo and bool(words[3]) == redo
     assert_stored_close(to_np64(Y), oracle_forward(oracle, inp)["Y"], "bf16", f"scores near {score}")
+
+
+def test_masked_stretches_do_not_hand_over(oracle):
+    """Whole tiles of masked tokens leave sums of exactly 0 behind, which are no reason for the exact form."""
+    inp = workloads.make_random(1, 2, 3000, 48, 16, dtype="bf16", seed=9, masked_fraction=0.1, k_std=0.8)
+    inp.key_mask[:, 300:2100] = 0
+    Q, K, V, mask = dev(inp.Q), dev(inp.K), dev(inp.V), dev(inp.key_mask)
+    desc = flare.make_desc(Q, K)
+    ws = flare.alloc_workspace(desc, flare.OP_FORWARD)
+    Y, le = torch.empty_like(K), torch.empty(1, 2, 48, device="cuda")
+    flare.flare_set_path(flare.PATH_FAST)
+    try:
+        flare.flare_forward(desc, Q, K, V, mask, Y, None, le, None, ws)
+    finally:
+        flare.flare_set_path(flare.PATH_AUTO)
+    torch.cuda.synchronize()
+    assert not ws[:16].view(torch.int32).cpu()[[0, 2, 3]].any()
+    assert_stored_close(to_np64(Y), oracle_forward(oracle, inp)["Y"], "bf16", "masked stretches")
