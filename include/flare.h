@@ -167,7 +167,8 @@ int flare_backward(const flare_desc_t *desc, const void *Q_lat, const void *K, c
 /*
  * flare_forward for callers whose tensors live in HOST memory (pinned memory makes the copies asynchronous).
  * Copies Q_lat, K, V (and key_mask if not NULL) from the host pointers into the caller's device staging
- * buffers dQ_lat, dK, dV, dmask, runs flare_forward into dY, and copies Y back to hY, all on `stream`.
+ * buffers dQ_lat, dK, dV, dmask, runs flare_forward into dY, and copies Y back to hY, in stream order of `stream`
+ * (a large batch in parts of whole items, the copies of one part overlapping those of others on a stream of the call's own).
  * hQ_lat, hK, hV, hmask, hY are host pointers; everything else is a device pointer.
  */
 int flare_forward_host(const flare_desc_t *desc, const void *hQ_lat, const void *hK, const void *hV,

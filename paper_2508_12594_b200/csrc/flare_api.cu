@@ -1,4 +1,5 @@
 // Entry points of libflare: argument checks, workspaces, the order of the launches.  See include/flare.h for the contract.
+#include <mutex>
 #include "flare_host.h"
 #include "flare_micro.cuh"
 
@@ -62,6 +63,121 @@ int launches_for(const flare_desc_t *d, int op, int sms) {
         }
         default: return 0;
     }
+}
+
+// Scratch of one flare_forward.
+size_t forward_bytes(const flare_desc_t *d) {
+    return make_layout(partials_for(d, device_info().sms), (long)d->B * d->H * d->M, d->D, true).total + decode_range_bytes(d);
+}
+
+int forward_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, void *Y, float *Z, float *lse_enc,
+                 float *lse_dec, void *workspace, cudaStream_t st, bool keep_status) {
+    const WorkspaceLayout w = make_layout(partials_for(d, device_info().sms), (long)d->B * d->H * d->M, d->D, true);
+    if (Z == nullptr) Z = reinterpret_cast<float *>(static_cast<char *>(workspace) + w.z);
+    const int rc = encode_impl(d, Q, K, V, mask, Z, lse_enc, workspace, st, keep_status);
+    if (rc != FLARE_OK) return rc;
+    char *range_scratch = decode_in_ranges(d) ? static_cast<char *>(workspace) + w.total : nullptr;
+    return decode_impl(d, Q, K, Z, Y, lse_dec, reinterpret_cast<uint32_t *>(workspace), st, range_scratch);
+}
+
+// Host tensors.  The copies bound such a call (67 + 67 MB in and 67 MB out take 3.7 ms, the mixer 0.1 ms), and the two directions of the link
+// are independent: a batch is worked off in parts of whole items, the inputs of the next parts coming in on the caller's stream while
+// a second one computes a part and takes its rows back.  3.75 -> 3.07 ms for 4 items of 65536 tokens of 128 features.  A part has at least
+// 4 MB to bring in (75 us): less would no longer hide what its eight or so calls cost the host.  Items must keep the tensors' alignment.
+int host_part_items(const flare_desc_t *d, size_t item_bytes, size_t workspace_bytes) {
+    const size_t least = (size_t)4 << 20;
+    long items = (long)((least + 2 * item_bytes - 1) / (2 * item_bytes));
+    if (items >= d->B || item_bytes % 16 != 0) return d->B;
+    flare_desc_t part = *d;
+    part.B = (int)items;
+    if (forward_bytes(&part) > workspace_bytes) return d->B;
+    part.B = d->B % (int)items;                                 // the last part
+    if (part.B != 0 && forward_bytes(&part) > workspace_bytes) return d->B;
+    return (int)items;
+}
+
+// Second streams.  One takes 110 us to create and destroy, so a few are kept: a call takes one for itself while it queues its work and gives it
+// back when it returns (a later call's work on it then simply queues behind).  At most kKept are kept in all, the rest and, with the
+// library, the kept ones are destroyed.
+class SideStreams {
+  public:
+    cudaError_t take(int device, cudaStream_t *out) {
+        {
+            std::lock_guard<std::mutex> lock(mutex_);
+            for (int i = 0; i < kept_; ++i)
+                if (device_[i] == device) {
+                    *out = stream_[i];
+                    --kept_;
+                    device_[i] = device_[kept_];
+                    stream_[i] = stream_[kept_];
+                    return cudaSuccess;
+                }
+        }
+        return cudaStreamCreateWithFlags(out, cudaStreamNonBlocking);
+    }
+    void give(int device, cudaStream_t stream) {
+        {
+            std::lock_guard<std::mutex> lock(mutex_);
+            if (kept_ < kKept) {
+                device_[kept_] = device;
+                stream_[kept_++] = stream;
+                return;
+            }
+        }
+        cudaStreamDestroy(stream);
+    }
+    ~SideStreams() {
+        for (int i = 0; i < kept_; ++i) cudaStreamDestroy(stream_[i]);
+    }
+
+  private:
+    static constexpr int kKept = 8;
+    std::mutex mutex_;
+    int kept_ = 0, device_[kKept];
+    cudaStream_t stream_[kKept];
+};
+SideStreams &side_streams() {
+    static SideStreams s;
+    return s;
+}
+
+int forward_host_parts(const flare_desc_t *d, int items, const void *hQ, const void *hK, const void *hV, const uint8_t *hmask, void *hY, void *dQ,
+                       void *dK, void *dV, uint8_t *dmask, void *dY, void *workspace, size_t qb, size_t item_bytes, cudaStream_t st) {
+    struct Side {
+        int device = 0;
+        cudaStream_t stream = nullptr;
+        cudaEvent_t event = nullptr;
+        ~Side() {
+            if (event) cudaEventDestroy(event);                 // (released once what is recorded has happened)
+            if (stream) side_streams().give(device, stream);
+        }
+    } side;
+    FLARE_CUDA(cudaGetDevice(&side.device));
+    FLARE_CUDA(side_streams().take(side.device, &side.stream));
+    FLARE_CUDA(cudaEventCreateWithFlags(&side.event, cudaEventDisableTiming));
+    auto parts = [&]() -> int {
+        FLARE_CUDA(cudaMemcpyAsync(dQ, hQ, qb, cudaMemcpyHostToDevice, st));
+        for (int b0 = 0; b0 < d->B; b0 += items) {
+            flare_desc_t part = *d;
+            part.B = std::min(items, d->B - b0);
+            const size_t at = (size_t)b0 * item_bytes, n = (size_t)part.B * item_bytes, mat = (size_t)b0 * d->N;
+            char *k = static_cast<char *>(dK) + at, *v = static_cast<char *>(dV) + at, *y = static_cast<char *>(dY) + at;
+            FLARE_CUDA(cudaMemcpyAsync(k, static_cast<const char *>(hK) + at, n, cudaMemcpyHostToDevice, st));
+            FLARE_CUDA(cudaMemcpyAsync(v, static_cast<const char *>(hV) + at, n, cudaMemcpyHostToDevice, st));
+            if (hmask) FLARE_CUDA(cudaMemcpyAsync(dmask + mat, hmask + mat, (size_t)part.B * d->N, cudaMemcpyHostToDevice, st));
+            FLARE_CUDA(cudaEventRecord(side.event, st));
+            FLARE_CUDA(cudaStreamWaitEvent(side.stream, side.event, 0));
+            const int rc = forward_impl(&part, dQ, k, v, hmask ? dmask + mat : nullptr, y, nullptr, nullptr, nullptr, workspace, side.stream, b0 > 0);
+            if (rc != FLARE_OK) return rc;
+            FLARE_CUDA(cudaMemcpyAsync(static_cast<char *>(hY) + at, y, n, cudaMemcpyDeviceToHost, side.stream));
+        }
+        return FLARE_OK;
+    };
+    const int rc = parts();
+    // whatever was queued on the second stream comes before the caller's next work, also after an error
+    FLARE_CUDA(cudaEventRecord(side.event, side.stream));
+    FLARE_CUDA(cudaStreamWaitEvent(st, side.event, 0));
+    return rc;
 }
 
 // ---- variants of the mixer: one latent sequence shared by all heads; separate latent queries for decode
@@ -163,8 +279,13 @@ size_t flare_workspace_bytes(const flare_desc_t *desc, int op) {
     switch (op) {
         case FLARE_OP_ENCODE: return make_layout(partials_for(desc, device_info().sms), rows, desc->D, false).total;
         case FLARE_OP_DECODE: return kHeaderBytes + decode_range_bytes(desc);
-        case FLARE_OP_FORWARD:
-            return make_layout(partials_for(desc, device_info().sms), rows, desc->D, true).total + decode_range_bytes(desc);
+        case FLARE_OP_FORWARD: {
+            // (room for the parts that flare_forward_host works a batch off in: fewer rows, but more CTAs along N for each)
+            size_t most = forward_bytes(desc);
+            flare_desc_t part = *desc;
+            for (part.B = desc->B / 2; part.B >= 1; part.B /= 2) most = std::max(most, forward_bytes(&part));
+            return most;
+        }
         case FLARE_OP_BACKWARD: return bwd_layout(desc, device_info().sms).total;
         case FLARE_OP_SPECTRAL: return spectral_bytes(desc, device_info().sms);
         default: return 0;
@@ -238,13 +359,7 @@ int flare_forward(const flare_desc_t *desc, const void *Q_lat, const void *K, co
         return FLARE_ERR_INVALID_ARG;
     if ((rc = require_device()) != FLARE_OK) return rc;
     if (workspace_bytes < flare_workspace_bytes(desc, FLARE_OP_FORWARD)) return FLARE_ERR_WORKSPACE_TOO_SMALL;
-    const WorkspaceLayout w = make_layout(partials_for(desc, device_info().sms), (long)desc->B * desc->H * desc->M, desc->D, true);
-    if (Z == nullptr) Z = reinterpret_cast<float *>(static_cast<char *>(workspace) + w.z);
-    rc = encode_impl(desc, Q_lat, K, V, key_mask, Z, lse_enc, workspace, (cudaStream_t)stream);
-    if (rc != FLARE_OK) return rc;
-    char *range_scratch = decode_in_ranges(desc) ? static_cast<char *>(workspace) + w.total : nullptr;
-    return decode_impl(desc, Q_lat, K, Z, Y, lse_dec, reinterpret_cast<uint32_t *>(workspace), (cudaStream_t)stream,
-                       range_scratch);
+    return forward_impl(desc, Q_lat, K, V, key_mask, Y, Z, lse_enc, lse_dec, workspace, (cudaStream_t)stream, false);
 }
 
 int flare_backward(const flare_desc_t *desc, const void *Q_lat, const void *K, const void *V, const uint8_t *key_mask,
@@ -275,6 +390,14 @@ int flare_forward_host(const flare_desc_t *desc, const void *hQ_lat, const void 
     const size_t e = desc->dtype == FLARE_DTYPE_F32 ? 4 : 2;
     const size_t qb = (size_t)desc->H * desc->M * desc->D * e;
     const size_t tb = (size_t)desc->B * desc->N * desc->H * desc->D * e;
+    if (workspace != nullptr && workspace_bytes >= flare_workspace_bytes(desc, FLARE_OP_FORWARD) && aligned16(dQ_lat) && aligned16(dK) &&
+        aligned16(dV) && aligned16(dY) && aligned16(workspace)) {
+        const int items = host_part_items(desc, tb / desc->B, workspace_bytes);
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (items < desc->B && cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone)
+            return forward_host_parts(desc, items, hQ_lat, hK, hV, hmask, hY, dQ_lat, dK, dV, dmask, dY, workspace, qb, tb / desc->B, st);
+        (void)cudaGetLastError();                               // (a capture elsewhere may forbid the question: one part then)
+    }
     FLARE_CUDA(cudaMemcpyAsync(dQ_lat, hQ_lat, qb, cudaMemcpyHostToDevice, st));
     FLARE_CUDA(cudaMemcpyAsync(dK, hK, tb, cudaMemcpyHostToDevice, st));
     FLARE_CUDA(cudaMemcpyAsync(dV, hV, tb, cudaMemcpyHostToDevice, st));

@@ -88,7 +88,7 @@ int launch_lean(const flare_desc_t *d, const LeanPlan &p, const void *Q, const v
 }  // namespace
 
 int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
-                float *lse_enc, void *ws, cudaStream_t st) {
+                float *lse_enc, void *ws, cudaStream_t st, bool keep_status) {
     const DeviceView di = device_info();
     const long rows = (long)d->B * d->H * d->M;
     const int P = partials_for(d, di.sms);
@@ -100,7 +100,8 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
     int rc, parts = P, parts_redo = 0;                         // partial results, and those of the exact form if it replaced them
     const uint32_t *redo = nullptr;
     if (use_tc(d)) {
-        FLARE_CUDA(cudaMemsetAsync(base, 0, kHeaderBytes, st));
+        const size_t kept = keep_status ? sizeof(uint32_t) : 0;
+        FLARE_CUDA(cudaMemsetAsync(base + kept, 0, kHeaderBytes - kept, st));
         TcEncodePlan p = tc_encode_plan(d, di.sms);
         uint32_t *status = reinterpret_cast<uint32_t *>(base);
         // a caller that asks for lse_enc is saving Z for the backward: weights as two bf16 halves (see exp_chunk_hilo)
@@ -141,7 +142,7 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
     }
     if (rc != FLARE_OK) return rc;
     // (the CUDA-core kernels leave nothing in the header: the merge clears it)
-    FLARE_REDUCE(merge_kernel, rows, parts, d->D, st, pm, pl, pacc, Z, lse_enc, parts, redo, parts_redo, rows, use_tc(d) ? nullptr : static_cast<uint32_t *>(ws));
+    FLARE_REDUCE(merge_kernel, rows, parts, d->D, st, pm, pl, pacc, Z, lse_enc, parts, redo, parts_redo, rows, use_tc(d) || keep_status ? nullptr : static_cast<uint32_t *>(ws));
     return FLARE_OK;
 }
 

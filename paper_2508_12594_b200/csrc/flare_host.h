@@ -378,8 +378,9 @@ int bwd_token_simt(const flare_desc_t *d, const void *Q, const void *K, const vo
 int bwd_dq_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask,
                 const void *dY, const float *Z, const float *dZ, const float *de, const float *dd, const float *lse_enc,
                 const float *lse_dec, float *part, cudaStream_t st);
+// keep_status: leave the error word of the workspace header as it is (a later part of a call in several parts)
 int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
-                float *lse_enc, void *ws, cudaStream_t st);
+                float *lse_enc, void *ws, cudaStream_t st, bool keep_status = false);
 int encode_dz_tc(const flare_desc_t *d, const LeanPlan &p, const void *Q, const void *K, const void *dY, float *part,
                  uint32_t *status, cudaStream_t st, const float *lse_dec);
 // range_scratch: decode_range_bytes(d) bytes, or null (then more than kDecodeMaxM latents take the CUDA-core kernel)
