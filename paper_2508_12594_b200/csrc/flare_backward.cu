@@ -20,9 +20,7 @@ int launch_bwd_dq_tc_n(const flare_desc_t *d, const TcEncodePlan &p, const void 
     if ((rc = make_token_map(&tmG, dY, d, kTile, DG)) != FLARE_OK) return rc;
     static std::atomic<uint64_t> smem_opt_in{0};
     if ((rc = ensure_big_smem(bwd_dq_tc_kernel<D, kPair, DRT, kPadded>, smem_opt_in)) != FLARE_OK) return rc;
-    bwd_dq_tc_kernel<D, kPair, DRT, kPadded><<<dim3((kPair ? d->H / 2 : d->H) * p.pairs, p.splits, d->B), kDqThreads,
-                                                         BwdDqSmem<DG, kPair>::total, st>>>(tmK, tmV, tmG, args);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_CUDA(launch_after(bwd_dq_tc_kernel<D, kPair, DRT, kPadded>, dim3((kPair ? d->H / 2 : d->H) * p.pairs, p.splits, d->B), kDqThreads, BwdDqSmem<DG, kPair>::total, st, tmK, tmV, tmG, args));
     return FLARE_OK;
 }
 
@@ -69,9 +67,7 @@ int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const v
     long per_head = sms / ((long)d->B * d->H);
     if (per_head < 1) per_head = 1;
     if (per_head > a.tiles) per_head = a.tiles;
-    bwd_token_tc_kernel<D, DRT, kMode, kPadded><<<dim3((unsigned)per_head, d->H, d->B), BwdGroups<2 * D>::kThreads, BwdTokSmem<D>::total(a.stages, a.M), st>>>(
-        tmK, tmV, tmG, a);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_CUDA(launch_after(bwd_token_tc_kernel<D, DRT, kMode, kPadded>, dim3((unsigned)per_head, d->H, d->B), BwdGroups<2 * D>::kThreads, BwdTokSmem<D>::total(a.stages, a.M), st,  tmK, tmV, tmG, a));
     return FLARE_OK;
 }
 

@@ -187,6 +187,8 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     float *kmin = reinterpret_cast<float *>(tmem_slot + 2);     // smallest lse_enc, per head of the CTA
     volatile uint32_t *two_exp = tmem_slot + 4;                 // [kCst][head]: the tile needs an exponential of its own for W_enc
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
+    ptx::grid_launch();
+    ptx::grid_wait();
     if (warp == 3) {
 #pragma unroll
         for (int w = 0; w < (kPair ? 2 : 1); ++w) {
@@ -576,6 +578,8 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         ptx::prefetch_tensormap(&tmG);
     }
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
+    ptx::grid_launch();
+    ptx::grid_wait();
     {
         const size_t q0 = (size_t)h * a.mtot + a.m0, r0 = ((size_t)b * a.H + h) * a.mtot + a.m0;
         if (warp == 2) {

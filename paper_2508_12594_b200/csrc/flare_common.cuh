@@ -8,6 +8,22 @@
 
 namespace flare {
 
+// Launch of a kernel that calls ptx::grid_wait() before it touches global memory: its CTAs may be placed, set up their barriers and
+// tensor memory and wait while the launch before it runs out, instead of starting when that has ended altogether.
+// Measured, whole calls, us: training step of 16384 tokens 94.6 -> 88.2, padded batch 333 -> 317, D = 64 194 -> 182, 2-D mesh forward 113 -> 107.
+// (Such kernels take no __restrict__ inputs: a read-only load might be moved ahead of the wait.)
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+
 // Workspace header: 256 bytes at the start of every workspace.
 //   word 0: error flag (0 = fine; otherwise a code naming the wait that gave up)
 //   word 1: detail (which barrier / iteration)

@@ -30,8 +30,7 @@ int launch_decode_tc_m(const flare_desc_t *d, int sms, const void *Q, const void
     if (per_head < 1) per_head = 1;
     if (per_head > a.tiles) per_head = a.tiles;
     dim3 grid((unsigned)per_head, d->H, d->B);
-    decode_tc_kernel<D, DRT, kPart, kM><<<grid, kTcThreads, smem, st>>>(tmK, tmQ, a);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_CUDA(launch_after(decode_tc_kernel<D, DRT, kPart, kM>, grid, kTcThreads, smem, st, tmK, tmQ, a));
     return FLARE_OK;
 }
 
@@ -65,8 +64,7 @@ int launch_decode_stream_l(const flare_desc_t *d, int sms, const void *Q, const 
         const long four = (a.tiles + 3) / 4;                    // a CTA works on four tiles at a time
         if (per_head > four) per_head = four;
         if (per_head < 1) per_head = 1;
-        decode_stream_kernel<D, DRT, kPart, kM, kLse><<<dim3((unsigned)per_head, d->H, d->B), kTcThreadsGuarded, smem, st>>>(tmK, tmQ, a);
-        FLARE_CUDA(cudaGetLastError());
+        FLARE_CUDA(launch_after(decode_stream_kernel<D, DRT, kPart, kM, kLse>, dim3((unsigned)per_head, d->H, d->B), kTcThreadsGuarded, smem, st, tmK, tmQ, a));
         return FLARE_OK;
     } else {
         return FLARE_ERR_UNSUPPORTED;
@@ -135,9 +133,7 @@ int decode_tc_any(const flare_desc_t *d, int sms, const void *Q, const void *K, 
                                                 Ypart + (size_t)c * rows * DR, fast);
         if (rc != FLARE_OK) return rc;
     }
-    decode_combine_kernel<DR><<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Ypart, lpart, C, (long)rows,
-                                                                             (__nv_bfloat16 *)Y, lse_dec);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_CUDA(launch_after(decode_combine_kernel<DR>, (unsigned)((rows + 255) / 256), 256, 0, st, Ypart, lpart, C, (long)rows, (__nv_bfloat16 *)Y, lse_dec));
     return FLARE_OK;
 }
 

@@ -167,6 +167,8 @@ encode_lean_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constan
             *reinterpret_cast<uint4 *>(ones + (size_t)r * G::RB + ((ch ^ G::swz(r)) << 4)) = make_uint4(ch == 0 ? 0x00003F80u : 0u, 0, 0, 0);
         }
     }
+    ptx::grid_launch();
+    ptx::grid_wait();
     // rows of Q: zeros where there is no latent (or, pair and narrow forms, no feature), then the rows
     if (kPair || DRT != 0 || rows_here < kTile) {
         for (int i = threadIdx.x; i < kTile * (G::RB / 16); i += kThreads) reinterpret_cast<uint4 *>(sQ)[i] = make_uint4(0, 0, 0, 0);

@@ -28,8 +28,7 @@ int launch_encode_tc_a(const flare_desc_t *d, const TcEncodePlan &p, const void 
     a.scale = d->scale; a.sl2 = d->scale * kLog2e;
     a.tiles = p.tiles; a.splits = p.splits; a.pairs = p.pairs; a.partials_per_split = p.per_split;
     dim3 grid(p.splits, (kPair ? d->H / 2 : d->H) * p.pairs, d->B);
-    encode_tc_kernel<D, kPair, DRT, kHiLo, kMaskBody, kAlt><<<grid, kTcThreads, smem, st>>>(tmK, tmV, tmQ, a);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_CUDA(launch_after(encode_tc_kernel<D, kPair, DRT, kHiLo, kMaskBody, kAlt>, grid, kTcThreads, smem, st, tmK, tmV, tmQ, a));
     return FLARE_OK;
 }
 
@@ -61,8 +60,7 @@ int launch_lean_m(const flare_desc_t *d, const LeanPlan &p, const void *Q, const
     a.B = d->B; a.H = d->H; a.N = d->N; a.M = d->M;
     a.sl2 = d->scale * kLog2e;
     a.tiles = p.tiles; a.splits = p.splits; a.blocks = p.blocks;
-    encode_lean_kernel<D, kPair, kKind, DRT, kMask><<<dim3((kPair ? d->H / 2 : d->H) * p.blocks, p.splits, d->B), LG::kThreads, LG::total, st>>>(tmK, tmV, a);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_CUDA(launch_after(encode_lean_kernel<D, kPair, kKind, DRT, kMask>, dim3((kPair ? d->H / 2 : d->H) * p.blocks, p.splits, d->B), LG::kThreads, LG::total, st, tmK, tmV, a));
     return FLARE_OK;
 }
 template <int D, bool kPair, int kKind, int DRT>

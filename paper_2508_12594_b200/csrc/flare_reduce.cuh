@@ -8,6 +8,7 @@
 #pragma once
 
 #include "flare_common.cuh"
+#include "flare_ptx.cuh"
 
 namespace flare {
 
@@ -71,8 +72,10 @@ __device__ __forceinline__ float4 sum_slices(float4 v, int slices) {
 // flags in it).
 template <int L>
 __global__ void __launch_bounds__(kReduceThreads)
-merge_kernel(const float *__restrict__ part_m, const float *__restrict__ part_l, const float *__restrict__ part_acc,
-             float *__restrict__ Z, float *__restrict__ lse_enc, int P, const uint32_t *redo, int P_redo, long rows, uint32_t *header, int slices) {
+merge_kernel(const float *part_m, const float *part_l, const float *part_acc,
+             float *Z, float *lse_enc, int P, const uint32_t *redo, int P_redo, long rows, uint32_t *header, int slices) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     if (redo != nullptr && *redo != 0) P = P_redo;
     const RowMap rm = row_map<L>(slices);
     const int T = L * slices;
@@ -132,8 +135,10 @@ merge_kernel(const float *__restrict__ part_m, const float *__restrict__ part_l,
 // dZ[row] = sum_p part[p][row] and de[row] = dZ_row . Z_row.
 template <int L>
 __global__ void __launch_bounds__(kReduceThreads)
-bwd_dz_reduce_kernel(const float *__restrict__ part, const float *__restrict__ Z, float *__restrict__ dZ, float *__restrict__ de,
+bwd_dz_reduce_kernel(const float *part, const float *Z, float *dZ, float *de,
                      int P, long rows, int slices) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     const RowMap rm = row_map<L>(slices);
     const bool live = rm.row < rows;
     const long at = (live ? rm.row : rows - 1) * L + rm.lane;
@@ -155,7 +160,9 @@ bwd_dz_reduce_kernel(const float *__restrict__ part, const float *__restrict__ Z
 // dQ[h][m] = scale * sum_b sum_p part[p][(b, h, m)]: the B * P terms of a row in index order per slice.
 template <int L>
 __global__ void __launch_bounds__(kReduceThreads)
-bwd_dq_reduce_kernel(const float *__restrict__ part, float *__restrict__ dQ, int P, int B, long per_batch, float scale, int slices) {
+bwd_dq_reduce_kernel(const float *part, float *dQ, int P, int B, long per_batch, float scale, int slices) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     const RowMap rm = row_map<L>(slices);
     const bool live = rm.row < per_batch;
     const long at = (live ? rm.row : per_batch - 1) * L + rm.lane;
@@ -169,18 +176,18 @@ bwd_dq_reduce_kernel(const float *__restrict__ part, float *__restrict__ dQ, int
 }
 
 // Launch of one of the kernels above with L = D / 4 as a template parameter.
-#define FLARE_REDUCE(kernel, rows_, P_, D_, st_, ...)                                                              \
-    do {                                                                                                           \
-        const int slices__ = reduce_slices(P_, D_);                                                                \
-        const unsigned blocks__ = reduce_blocks(rows_, D_, slices__);                                              \
-        switch (D_) {                                                                                              \
-            case 4: kernel<1><<<blocks__, kReduceThreads, 0, st_>>>(__VA_ARGS__, slices__); break;                  \
-            case 8: kernel<2><<<blocks__, kReduceThreads, 0, st_>>>(__VA_ARGS__, slices__); break;                  \
-            case 16: kernel<4><<<blocks__, kReduceThreads, 0, st_>>>(__VA_ARGS__, slices__); break;                 \
-            case 32: kernel<8><<<blocks__, kReduceThreads, 0, st_>>>(__VA_ARGS__, slices__); break;                 \
-            default: kernel<16><<<blocks__, kReduceThreads, 0, st_>>>(__VA_ARGS__, slices__); break;                \
-        }                                                                                                          \
-        FLARE_CUDA(cudaGetLastError());                                                                            \
+#define FLARE_REDUCE(kernel, rows_, P_, D_, st_, ...)                                            \
+    do {                                                                                         \
+        const int slices__ = reduce_slices(P_, D_);                                              \
+        const unsigned blocks__ = reduce_blocks(rows_, D_, slices__);                            \
+        switch (D_) {                                                                            \
+            case 4: FLARE_CUDA(launch_after(kernel<1>, blocks__, kReduceThreads, 0, st_, __VA_ARGS__, slices__)); break;\
+            case 8: FLARE_CUDA(launch_after(kernel<2>, blocks__, kReduceThreads, 0, st_, __VA_ARGS__, slices__)); break;\
+            case 16: FLARE_CUDA(launch_after(kernel<4>, blocks__, kReduceThreads, 0, st_, __VA_ARGS__, slices__)); break;                 \
+            case 32: FLARE_CUDA(launch_after(kernel<8>, blocks__, kReduceThreads, 0, st_, __VA_ARGS__, slices__)); break;                 \
+            default: FLARE_CUDA(launch_after(kernel<16>, blocks__, kReduceThreads, 0, st_, __VA_ARGS__, slices__)); break;                \
+        }                                                                                        \
+        FLARE_CUDA(cudaGetLastError());                                                          \
     } while (0)
 
 }  // namespace flare

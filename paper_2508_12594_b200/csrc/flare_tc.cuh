@@ -447,6 +447,8 @@ struct DecodeSmem {
 template <int D, int DRT = 0, bool kPart = false, int kM = 0>
 __global__ void __launch_bounds__(kTcThreads, 1)
 decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ, DecodeTcArgs a) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     if (a.run_if != nullptr && *a.run_if == 0) return;          // behind the streaming form, as a fallback that was not needed
     constexpr bool kHalf = DRT != 0;
     constexpr int DR = kHalf ? DRT : D;                         // head width in memory
@@ -870,6 +872,8 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         ptx::prefetch_tensormap(&tmQ);
     }
     if (warp == kFirstIssuerWarp) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
+    ptx::grid_launch();
+    ptx::grid_wait();
     {   // Z_bh -> [hi | lo | ones] blocks of M latent-major rows in the swizzled layout of an MN-major B operand
         const float *Zg = a.Z + (((size_t)b * a.H + h) * a.mtot + a.m0) * DR;
         const int z0 = kHalf ? 0 : M;                           // rows to clear: beyond M; in the narrow forms all
@@ -1202,8 +1206,9 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
 // the same algebra as the split-N merge of the encode stage.  One thread per (token, head) row of DR elements.
 template <int DR>
 __global__ void __launch_bounds__(256)
-decode_combine_kernel(const float *__restrict__ Ypart, const float *__restrict__ lse_part, int C, long rows,
-                      __nv_bfloat16 *__restrict__ Y, float *__restrict__ lse_dec) {
+decode_combine_kernel(const float *Ypart, const float *lse_part, int C, long rows, __nv_bfloat16 *Y, float *lse_dec) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     const long row = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= rows) return;
     float lc[8], mx = -INFINITY;
@@ -1322,6 +1327,8 @@ template <int D, bool kPair, int DRT = 0, bool kHiLo = false, bool kMaskBody = f
 __global__ void __launch_bounds__(kTcThreads, 1)
 encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                  const __grid_constant__ CUtensorMap tmQ, EncodeTcArgs a) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     if (a.run_if != nullptr && *a.run_if == 0) return;      // the exact form as a fallback that was not needed
     constexpr bool kHalf = DRT != 0;
     static_assert(!(kPair && kHalf), "head pairing and the narrow form exclude each other");
