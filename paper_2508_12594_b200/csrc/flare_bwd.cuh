@@ -19,6 +19,7 @@
 // multiply-adds per pair in the first sweep over the latents and 3 D in the second and in the dQ pass.
 #pragma once
 
+#include "flare_ptx.cuh"
 #include "flare_common.cuh"
 #include "flare_simt.cuh"
 
@@ -34,11 +35,13 @@ template <int D> struct BwdSimtGeom {
 // Pass B, token side.  Rows are tokens (8 RB per warp, the block's warps side by side).  grid = (ceil(N / kTokRows), H, B).
 template <typename T, int D>
 __global__ void __launch_bounds__(BwdSimtGeom<D>::kTokThreads, 1)
-bwd_token_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
-                      const uint8_t *__restrict__ key_mask, const T *__restrict__ dY, const float *__restrict__ Z,
-                      const float *__restrict__ dZ, const float *__restrict__ de, const float *__restrict__ lse_enc,
-                      const float *__restrict__ lse_dec, T *__restrict__ dK, T *__restrict__ dV,
-                      float *__restrict__ dd_out, int B, int H, int N, int M, float scale) {
+bwd_token_simt_kernel(const T *Q, const T *K, const T *V,
+                      const uint8_t *key_mask, const T *dY, const float *Z,
+                      const float *dZ, const float *de, const float *lse_enc,
+                      const float *lse_dec, T *dK, T *dV,
+                      float *dd_out, int B, int H, int N, int M, float scale) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     using SG = SimtGeom<D>;
     constexpr int CT = SG::CT, RB = BwdSimtGeom<D>::RB, TH = BwdSimtGeom<D>::kTokThreads;
     extern __shared__ __align__(16) unsigned char simt_smem[];
@@ -174,11 +177,13 @@ template <typename T, int D> inline size_t bwd_token_simt_smem() {
 // Pass B, latent side: partial dQ rows.  Rows are latents, columns tokens; grid and warps as in encode_simt_kernel.
 template <typename T, int D>
 __global__ void __launch_bounds__(kBwdThreads, D <= 32 ? 2 : 1)
-bwd_dq_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
-                   const uint8_t *__restrict__ key_mask, const T *__restrict__ dY, const float *__restrict__ Z,
-                   const float *__restrict__ dZ, const float *__restrict__ de, const float *__restrict__ dd,
-                   const float *__restrict__ lse_enc, const float *__restrict__ lse_dec, float *__restrict__ part,
+bwd_dq_simt_kernel(const T *Q, const T *K, const T *V,
+                   const uint8_t *key_mask, const T *dY, const float *Z,
+                   const float *dZ, const float *de, const float *dd,
+                   const float *lse_enc, const float *lse_dec, float *part,
                    int B, int H, int N, int M, int WM, int mblocks, int chunk, float scale) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     using SG = SimtGeom<D>;
     constexpr int CT = SG::CT, RB = BwdSimtGeom<D>::RB, RW = 8 * RB;
     extern __shared__ __align__(16) unsigned char simt_smem[];

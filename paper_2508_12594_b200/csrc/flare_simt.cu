@@ -13,9 +13,8 @@ int launch_encode(const flare_desc_t *d, const SimtPlan &p, const void *Q, const
     static std::atomic<uint64_t> opt_in{0};
     if (smem > 48 * 1024)
         if (int rc = ensure_big_smem(encode_simt_kernel<T, D, RB, kDz>, opt_in, (int)smem)) return rc;
-    encode_simt_kernel<T, D, RB, kDz><<<dim3(p.splits, d->H * p.mblocks, d->B), kSimtThreads, smem, st>>>(
-        (const T *)Q, (const T *)K, (const T *)V, mask, lse_dec, pm, pl, pacc, d->B, d->H, d->N, d->M, p.WM, p.mblocks, p.chunk, d->scale);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_CUDA(launch_after(encode_simt_kernel<T, D, RB, kDz>, dim3(p.splits, d->H * p.mblocks, d->B), kSimtThreads, smem, st,
+                            (const T *)Q, (const T *)K, (const T *)V, mask, lse_dec, pm, pl, pacc, d->B, d->H, d->N, d->M, p.WM, p.mblocks, p.chunk, d->scale));
     return FLARE_OK;
 }
 template <typename T, int D>
@@ -33,9 +32,8 @@ struct Decode {
     template <int RB>
     static int launch(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st) {
         static_assert(sizeof(double) * 64 * 36 + sizeof(float) * 64 * 36 + 8 * 64 * 32 <= 48 * 1024, "no opt-in needed");
-        decode_simt_kernel<T, D, RB><<<dim3((d->N + 64 * RB - 1) / (64 * RB), d->H, d->B), kSimtThreads, decode_simt_smem<T, D>(), st>>>(
-            (const T *)Q, (const T *)K, Z, (T *)Y, lse_dec, d->B, d->H, d->N, d->M, d->scale);
-        FLARE_CUDA(cudaGetLastError());
+        FLARE_CUDA(launch_after(decode_simt_kernel<T, D, RB>, dim3((d->N + 64 * RB - 1) / (64 * RB), d->H, d->B), kSimtThreads, decode_simt_smem<T, D>(), st,
+                                (const T *)Q, (const T *)K, Z, (T *)Y, lse_dec, d->B, d->H, d->N, d->M, d->scale));
         return FLARE_OK;
     }
     static int run(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st) {
@@ -55,10 +53,8 @@ struct Token {
         const size_t smem = bwd_token_simt_smem<T, D>();
         if (smem > 48 * 1024)
             if (int rc = ensure_big_smem(bwd_token_simt_kernel<T, D>, opt_in, (int)smem)) return rc;
-        bwd_token_simt_kernel<T, D><<<dim3((d->N + rows - 1) / rows, d->H, d->B), BwdSimtGeom<D>::kTokThreads, smem, st>>>(
-            (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, lse_enc, lse_dec, (T *)dK, (T *)dV, dd, d->B, d->H, d->N,
-            d->M, d->scale);
-        FLARE_CUDA(cudaGetLastError());
+        FLARE_CUDA(launch_after(bwd_token_simt_kernel<T, D>, dim3((d->N + rows - 1) / rows, d->H, d->B), BwdSimtGeom<D>::kTokThreads, smem, st,
+                                (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, lse_enc, lse_dec, (T *)dK, (T *)dV, dd, d->B, d->H, d->N, d->M, d->scale));
         return FLARE_OK;
     }
 };
@@ -72,10 +68,8 @@ struct DQuery {
         const size_t smem = bwd_dq_simt_smem<T, D>();
         if (smem > 48 * 1024)
             if (int rc = ensure_big_smem(bwd_dq_simt_kernel<T, D>, opt_in, (int)smem)) return rc;
-        bwd_dq_simt_kernel<T, D><<<dim3(p.splits, d->H * p.mblocks, d->B), kBwdThreads, smem, st>>>(
-            (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, dd, lse_enc, lse_dec, part, d->B, d->H, d->N, d->M, p.WM,
-            p.mblocks, p.chunk, d->scale);
-        FLARE_CUDA(cudaGetLastError());
+        FLARE_CUDA(launch_after(bwd_dq_simt_kernel<T, D>, dim3(p.splits, d->H * p.mblocks, d->B), kBwdThreads, smem, st,
+                                (const T *)Q, (const T *)K, (const T *)V, mask, (const T *)dY, Z, dZ, de, dd, lse_enc, lse_dec, part, d->B, d->H, d->N, d->M, p.WM, p.mblocks, p.chunk, d->scale));
         return FLARE_OK;
     }
 };

@@ -15,6 +15,7 @@
 // elements: B fragments and value rows are then read without bank conflicts.
 #pragma once
 
+#include "flare_ptx.cuh"
 #include "flare_common.cuh"
 
 namespace flare {
@@ -201,9 +202,11 @@ __device__ __forceinline__ void write_quarter(T *dst, const float2 (&acc)[D / 2]
 // kDz: the backward's dZ form: dY in place of V, weights exp(score - lse_dec[n]), no maximum and no sum.
 template <typename T, int D, int RB, bool kDz>
 __global__ void __launch_bounds__(kSimtThreads, 2)
-encode_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V, const uint8_t *__restrict__ key_mask,
-                   const float *__restrict__ lse_dec, float *__restrict__ part_m, float *__restrict__ part_l,
-                   float *__restrict__ part_acc, int B, int H, int N, int M, int WM, int mblocks, int chunk, float scale) {
+encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
+                   const float *lse_dec, float *part_m, float *part_l,
+                   float *part_acc, int B, int H, int N, int M, int WM, int mblocks, int chunk, float scale) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     using SG = SimtGeom<D>;
     constexpr int CT = SG::CT, RW = 8 * RB;
     extern __shared__ __align__(16) unsigned char simt_smem[];
@@ -322,8 +325,10 @@ template <typename T, int D> inline size_t encode_simt_smem(int RB) {
 // Decode: rows are tokens (8 RB per warp, the eight warps side by side), columns the latents.  grid = (ceil(N / (64 RB)), H, B).
 template <typename T, int D, int RB>
 __global__ void __launch_bounds__(kSimtThreads, 2)
-decode_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, const float *__restrict__ Z, T *__restrict__ Y,
-                   float *__restrict__ lse_dec, int B, int H, int N, int M, float scale) {
+decode_simt_kernel(const T *Q, const T *K, const float *Z, T *Y,
+                   float *lse_dec, int B, int H, int N, int M, float scale) {
+    ptx::grid_launch();
+    ptx::grid_wait();
     using SG = SimtGeom<D>;
     constexpr int CT = SG::CT;
     extern __shared__ __align__(16) unsigned char simt_smem[];
