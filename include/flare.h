@@ -125,8 +125,9 @@ int flare_decode(const flare_desc_t *desc, const void *Q_lat, const void *K, con
  * Both stages are softmaxes, and a softmax is usually stabilised by subtracting the row maximum before every
  * exponential (the exact forms: a running maximum in encode, a first pass over the scores in decode).  The fast
  * forms skip that: float32 and bfloat16 hold 2^x for |x| < 126, so exp(score) can be formed as it stands while
- * every |scale * q.k| stays below 96 binades (66.5 in natural units).  They check the sufficient condition
- * |q| |k| scale log2(e) <= 96 on every key row they load, and raise a flag in the workspace header if it fails;
+ * every |scale * q.k| stays below 125 binades (86 in natural units).  They check the sufficient condition
+ * |q| |k| scale log2(e) <= 125 on the key rows they load (where a saturating exponential makes that needless: not),
+ * and that every sum of weights lies between 2^-90 and 2^104, and raise a flag in the workspace header if either fails;
  * the exact form is launched right behind and exits at once unless the flag is up, in which case it redoes the
  * stage.  Results of the two forms agree within the forward's error bound, not bit for bit.
  *   FLARE_PATH_AUTO   (default) fast forms for problems large enough to hide the extra launches
@@ -153,11 +154,11 @@ int flare_forward(const flare_desc_t *desc, const void *Q_lat, const void *K, co
  * Z, lse_enc, lse_dec are the ones flare_forward wrote; Y is its output (part of the saved set; the present
  * kernels rebuild dY_n.Y_n = sum_m W_dec[n,m] (dY_n.Z_m) in float32 instead of reading the rounded Y, which
  * is markedly more accurate where the latent rows a token mixes are nearly equal).
- * bfloat16 inputs run all three passes (dZ; dK, dV; dQ_lat) on the tensor cores (the last two for D <= 32), with
+ * bfloat16 inputs run all three passes (dZ; dK, dV; dQ_lat) on the tensor cores, with
  * every rounded factor of a cancelling sum carried as two bfloat16 halves; float32 inputs run on the CUDA cores.
  * dQ_lat, dK, dV are overwritten.  Workspace: flare_workspace_bytes(desc, FLARE_OP_BACKWARD) bytes holding dZ,
- * per-split partial sums of dZ and dQ_lat, one float per (b, n, h), and, beyond 512 bfloat16 latents (256 at
- * D = 32), float32 sums of the rows of dK and dV; nothing of size N x M.
+ * per-split partial sums of dZ and dQ_lat, one float per (b, n, h), and, beyond 1024 bfloat16 latents (448 at
+ * D = 32, 192 at D = 64), float32 sums of the rows of dK and dV; nothing of size N x M.
  */
 int flare_backward(const flare_desc_t *desc, const void *Q_lat, const void *K, const void *V,
                    const uint8_t *key_mask, const void *Y, const void *dY, const float *Z, const float *lse_enc,

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) micro_softmax_kernel(int iters,
                 mx = max_of<32>(r, mx);
                 exp_chunk<32, false>(r, pk, sl2p, make_float2(-mx * sl2, -mx * sl2), sum2);
             } else {
-                exp_chunk_fast<32, kBody == 2, false, 0>(r, pk, sl2p, sum2);
+                exp_chunk_fast<32, kBody == 2, 0>(r, pk, sl2p, sum2);
             }
             ptx::tmem_st16(sbase + 64, pk);
             ptx::tmem_wait_st();

@@ -8,11 +8,9 @@
 // feed the second contraction as its A operand.
 //
 // Two resources limit both kernels, and neither is the one a roofline of FLOPs and bytes names.  Every
-// (latent, token) pair needs one exponential on the special-function unit (16 per clock per SM), and every
-// tcgen05.mma of this shape (M = 128, K = 16) holds the tensor pipe for about 107 cycles whatever its N
-// (measured), so the value contraction costs one such slot per 16 latents (decode) or tokens (encode): about
-// as long as the exponentials of the same block.  That cost is a latency of the issuing thread, not an occupancy
-// of the pipe: four threads issuing side by side get about three times the instructions through (measured).
+// (latent, token) pair needs one exponential on the special-function unit (16 per clock per SM), and every tcgen05.mma of this
+// shape (M = 128, K = 16) takes its issuing thread 18 to 58 cycles (113 where the compiler does not know that one lane of a uniform
+// warp issues it) and the tensor core 40 cycles or more with both operands in shared memory, N / 2 with one in tensor memory.
 // The CTA is therefore four pipelines side by side: warp 0 issues TMA loads; sixteen softmax warps (four per
 // scheduler) form four groups of four warps, and each group has an issuing warp of its own (warps 1-4; warp 1
 // also owns the TMEM allocation).  A group owns one TMEM score buffer, or a range of columns of a shared one,
@@ -32,7 +30,7 @@ constexpr int kSoftmaxGroups = 4;                            // groups of 4 warp
 constexpr int kFirstIssuerWarp = 1;                          // warps 1..4: one MMA-issuing warp per group
 constexpr int kFirstSoftmaxWarp = kFirstIssuerWarp + kSoftmaxGroups;
 constexpr int kTcThreads = (kFirstSoftmaxWarp + 4 * kSoftmaxGroups) * 32;  // 672
-// The fast form of encode adds three guard warps behind the softmax warps (they check the norms of the key rows while a
+// The streaming decode adds three guard warps behind the softmax warps (they check the norms of the key rows while a
 // tile waits in its stage; 24 warps still get 80 registers each: six per scheduler either way).
 constexpr int kGuardWarps = 3;
 constexpr int kFirstGuardWarp = kTcThreads / 32;
@@ -124,28 +122,6 @@ __device__ __forceinline__ bool hand_over(uint32_t full, uint32_t n, volatile ui
 }
 
 // ------------------------------------------------------------------------------------- softmax arithmetic
-// p = 2^(s * sl2 + neg[k]) with one addend per column (read from shared memory, four at a time): the form the
-// backward needs, where every column (token) carries its own log-sum-exp.  The weights leave as two bf16 halves,
-// hi = round(p) and lo = round(p - hi): dZ feeds differences (dZ.V - dZ.Z) downstream, and with one half its
-// rounding alone moved dK, dV and dQ by 2e-2 to 4e-2 of their RMS (measured).
-template <int NV>
-__device__ __forceinline__ void exp_chunk_cols(const uint32_t *r, uint32_t *hi, uint32_t *lo, float2 sl2p, const float *neg) {
-#pragma unroll
-    for (int k = 0; k < NV / 4; ++k) {
-        const float4 ng = *reinterpret_cast<const float4 *>(neg + 4 * k);
-        const float2 x0 = __ffma2_rn(make_float2(__uint_as_float(r[4 * k]), __uint_as_float(r[4 * k + 1])), sl2p,
-                                     make_float2(ng.x, ng.y));
-        const float2 x1 = __ffma2_rn(make_float2(__uint_as_float(r[4 * k + 2]), __uint_as_float(r[4 * k + 3])), sl2p,
-                                     make_float2(ng.z, ng.w));
-        const float p0 = ptx::ex2(x0.x), p1 = ptx::ex2(x0.y), p2 = ptx::ex2(x1.x), p3 = ptx::ex2(x1.y);
-        const uint32_t h0 = ptx::pack_bf16(p0, p1), h1 = ptx::pack_bf16(p2, p3);
-        hi[2 * k] = h0;
-        hi[2 * k + 1] = h1;
-        lo[2 * k] = ptx::pack_bf16(p0 - __uint_as_float(h0 << 16), p1 - __uint_as_float(h0 & 0xffff0000u));
-        lo[2 * k + 1] = ptx::pack_bf16(p2 - __uint_as_float(h1 << 16), p3 - __uint_as_float(h1 & 0xffff0000u));
-    }
-}
-
 // Row maximum over NV (16 or 32) float32 scores held as raw bits.
 template <int NV>
 __device__ __forceinline__ float max_of(const uint32_t *r, float m) {
@@ -248,12 +224,10 @@ __device__ __forceinline__ float2 exp2_fma_pipe(float2 s, float2 sl2p) {
 // some 2^x with a full mantissa, and a sum of the unrounded values would normalise it away from the rounded one
 // that multiplies the values (measured: Y off by 1.5e-2 of its RMS where one weight dominates a row, against 4e-3).
 // kSum = 0: no sum here (a ones column of the value operand lets the tensor core add the rounded weights);
-// kSum = 1: the rounded weights are widened again and added into sum2;
-// kSum = 2: as 0, and the unrounded weights are added into sum2 (for a log-sum-exp output, which must not carry the
+// kSum = 2: the unrounded weights are added into sum2 as well (for a log-sum-exp output, which must not carry the
 //           rounding of the weights: the backward rebuilds every weight from it).
-template <int NV, bool kPoly, bool kMasked, int kSum>
-__device__ __forceinline__ void exp_chunk_fast(const uint32_t *r, uint32_t *pk, float2 sl2p, float2 &sum2,
-                                               uint32_t valid = 0xffffffffu) {
+template <int NV, bool kPoly, int kSum>
+__device__ __forceinline__ void exp_chunk_fast(const uint32_t *r, uint32_t *pk, float2 sl2p, float2 &sum2) {
 #pragma unroll
     for (int k = 0; k < NV / 2; ++k) {
         const float2 s = make_float2(__uint_as_float(r[2 * k]), __uint_as_float(r[2 * k + 1]));
@@ -264,12 +238,7 @@ __device__ __forceinline__ void exp_chunk_fast(const uint32_t *r, uint32_t *pk, 
             const float2 x = __fmul2_rn(s, sl2p);
             p = make_float2(ptx::ex2(x.x), ptx::ex2(x.y));
         }
-        if (kMasked) {
-            if (!((valid >> (2 * k)) & 1)) p.x = 0.f;
-            if (!((valid >> (2 * k + 1)) & 1)) p.y = 0.f;
-        }
         pk[k] = ptx::pack_bf16(p.x, p.y);
-        if (kSum == 1) sum2 = __fadd2_rn(sum2, make_float2(__uint_as_float(pk[k] << 16), __uint_as_float(pk[k] & 0xffff0000u)));
         if (kSum == 2) sum2 = __fadd2_rn(sum2, p);
     }
 }
@@ -1167,10 +1136,10 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
                 uint32_t r[32], pk[16];
                 ptx::tmem_ld32(gcol + w * UNIT, r);
                 ptx::tmem_wait_ld();
-                exp_chunk_fast<16, true, false, kSum>(r, pk, sl2p, sum2);
+                exp_chunk_fast<16, true, kSum>(r, pk, sl2p, sum2);
                 const bool s_probe = n + 1 < total && ptx::mbar_test(bar(S_FULL + 2 * g + (w ^ 1)), ((n + 1) >> 1) & 1);
                 if (!half) {
-                    exp_chunk_fast<16, true, false, kSum>(r + 16, pk + 8, sl2p, sum2);
+                    exp_chunk_fast<16, true, kSum>(r + 16, pk + 8, sl2p, sum2);
                 } else {
 #pragma unroll
                     for (int k = 8; k < 16; ++k) pk[k] = 0u;
