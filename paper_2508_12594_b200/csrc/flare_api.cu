@@ -49,7 +49,7 @@ int static_scratch_address(void **out) {
 // Kernels one call of `op` launches (the memset of the workspace header is not a kernel).
 int launches_for(const flare_desc_t *d, int op, int sms) {
     // a fast form is followed by the exact form (which may exit at once)
-    const int fe = use_fast_encode(d, false, false) ? 2 : 1, f = use_fast_decode(d) ? 2 : 1;
+    const int fe = use_fast_encode(d) ? 2 : 1, f = use_fast_decode(d) ? 2 : 1;
     const int enc = fe + 1;                                     // encode, merge
     const int dec = decode_in_ranges(d) ? f * decode_ranges(d) + 1 : f;   // ranges of latents and their combination
     switch (op) {

@@ -103,7 +103,7 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
         TcEncodePlan p = tc_encode_plan(d, di.sms);
         uint32_t *status = reinterpret_cast<uint32_t *>(base);
         // a caller that asks for lse_enc is saving Z for the backward: weights as two bf16 halves (see exp_chunk_hilo)
-        const bool fast = use_fast_encode(d, lse_enc != nullptr, mask != nullptr);
+        const bool fast = use_fast_encode(d);
         if (fast) {                                             // the exact form, behind it, exits at once unless the fast one raised its flag
             const LeanPlan lp = lean_plan(d, di.sms);
             EncodeLeanArgs a{};

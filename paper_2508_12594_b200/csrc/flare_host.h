@@ -146,17 +146,17 @@ inline bool fast_wanted(const flare_desc_t *d, bool pays) {
     return use_tc(d) && path != FLARE_PATH_EXACT && (path == FLARE_PATH_FAST || pays);
 }
 // Encode: the time of either form goes with the blocks of 128 lanes (of latents, or of two heads), whatever part of them is filled.
-// Measured, fast against exact form, us, at B H N = 65536 / 131072 / 262144 / 2.1 million, D = 8 and 16: 9.2 : 8.3 / 11.7 : 12.4 / 16.1 : 19.6
-// / 77 : 104, masked 11.0 : 10.4 / 14.5 : 15.8 / 21.5 : 25.8 / 110 : 151.  The head-pair form at D = 32 and D = 64 have a shallow K/V ring,
-// which the norm check holds longer: the first pays later (masked 26 : 32 at 262144, else 41 : 42 at 524288), D = 64 never (13.6 : 19 at
-// 32768, 72 : 84 at a million).
-inline bool use_fast_encode(const flare_desc_t *d, bool lse, bool masked) {
-    const double work = (double)d->B * d->N * (encode_head_pairs(d) ? d->H / 2 : d->H) * ((d->M + 127) / 128);
-    const double least = encode_head_pairs(d) && d->D == 32 ? (masked ? 2.0e5 : 5.0e5) : lse && !masked ? 2.0e5 : 1.0e5;
-    return d->D <= 32 && fast_wanted(d, work >= least);
+// Measured, exact against fast form with the merge behind it, us, at 65536 / 131072 / 524288 tokens x heads x blocks: D = 16, M = 96 17.8 : 16.5 /
+// 21 : 18.6 / 41 : 31, masked 18.5 : 16.5 / 25 : 20.5 / 51 : 33, with log-sum-exp 18.5 : 17.7 / 22.6 : 20.7 / 43 : 37; D = 32 20.5 : 16.6 / 24 :
+// 20 / 45 : 33; head pairs, at 32768 / 65536 tokens x pairs: D = 8 18.6 : 15.2 / 22 : 16.6, D = 16 14.5 : 15.8 / 16.7 : 16.5, D = 32 18.5 : 16.5 /
+// 20.5 : 18.5.  D = 64: the norm check holds a tile longer than its scores (72 : 84 at a million).
+inline bool lean_pairs(const flare_desc_t *d) { return d->M <= 64 && d->H % 2 == 0 && d->D >= 8 && d->D <= 32; }
+inline bool use_fast_encode(const flare_desc_t *d) {
+    const double work = (double)d->B * d->N * (lean_pairs(d) ? d->H / 2 : d->H) * ((d->M + 127) / 128);
+    return d->D <= 32 && fast_wanted(d, work >= (lean_pairs(d) && d->D != 16 ? 3.0e4 : 6.0e4));
 }
 // Decode: the streaming form has no variant for head width 64.  Measured against the exact form, us, at B H N = 524288 (131072): D = 16, M = 48
-// 20 : 29 (11.2 : 10.4), 64 31 : 35 (10.4 : 8.3), 96 26 : 36 (12.9 : 12.6), 144 27 : 33 (15 : 20); the exact form keeps what one chunk
+// 20 : 29 (11.2 : 10.4), 64 31 : 35 (10.4 : 8.3), 96 26 : 36 (14.4 : 15.8), 144 27 : 33 (15 : 20); the exact form keeps what one chunk
 // of its registers holds (M = 32: 18 : 13) and, at D = 32, 64 latents (48 : 41) and small calls up to there (M = 48: 29 : 35 from 262144 on).
 inline bool use_fast_decode(const flare_desc_t *d) {
     const double rows = (double)d->B * d->H * d->N;
@@ -164,7 +164,7 @@ inline bool use_fast_decode(const flare_desc_t *d) {
     if (d->M == 32 || (d->D == 32 && d->M == 64)) pays = false;
     else if (d->M < 64) pays = rows >= 3.0e5;
     else if (d->M == 64) pays = rows >= 5.0e5;
-    else if (d->M <= 128) pays = rows >= (d->D == 32 && d->M != 128 ? 6.0e4 : 2.0e5);
+    else if (d->M <= 128) pays = rows >= (d->M == 128 ? 2.0e5 : d->D == 32 ? 6.0e4 : 1.2e5);
     else pays = rows >= 6.0e4;
     return d->D <= 32 && fast_wanted(d, pays);
 }
@@ -210,7 +210,6 @@ inline TcEncodePlan tc_encode_plan(const flare_desc_t *d, int sms) {
 
 // Launch plan of the encode without a running maximum and of dZ: one partial result per CTA.  Up to 64 latents two heads share the lanes.
 struct LeanPlan { int tiles, blocks, splits; };
-inline bool lean_pairs(const flare_desc_t *d) { return d->M <= 64 && d->H % 2 == 0 && d->D >= 8 && d->D <= 32; }
 inline LeanPlan lean_plan(const flare_desc_t *d, int sms) {
     LeanPlan p;
     p.tiles = (d->N + kTile - 1) / kTile;
