@@ -363,8 +363,10 @@ BINDING_END
 // G, eigenvalues, U, sweeps, stream
 BINDING(spectral_eig, 5)
     const at::Tensor &G = tensor(a[0]);
-    const int64_t M = G.size(-1);
-    const int32_t matrices = (int32_t)(G.numel() / (M * M));
+    const int64_t M = G.dim() > 0 ? G.size(-1) : 0;
+    if (M < 1) fail(PyExc_ValueError, "expected matrices [..., M, M], got shape " + shape_text(G.sizes()));
+    // (rows longer than the library takes are left to it to refuse: their square might not even be a number of elements)
+    const int32_t matrices = M <= 1024 ? (int32_t)(G.numel() / (M * M)) : 0;
     const long sweeps = PyLong_AsLong(a[3]);
     if (sweeps == -1 && PyErr_Occurred()) throw PythonError{};
     auto ptr = [](PyObject *o) -> float * {

@@ -83,3 +83,11 @@ def test_workspace_never_scales_with_n_times_m(lib):
     rows = 8 * 256
     assert wb <= 256 + 4096 + flare.flare_encode_partials(big) * rows * (16 + 2) * 4 + rows * 16 * 4 + 4 * 256
     assert ws <= wb
+
+
+def test_eigenvalues_of_empty_matrices_are_refused(lib):
+    """The number of matrices is a quotient of sizes: no size may make it one by zero (the sixth: 2^32 squared is 0 in 64 bits)."""
+    import torch
+    for shape in ((0, 0), (3, 0, 0), (5, 0), (0,), (), (0, 1 << 32)):
+        with pytest.raises((ValueError, flare.FlareError)):
+            flare.flare_spectral_eig(torch.empty(shape), torch.empty(0))
