@@ -366,18 +366,20 @@ BINDING(spectral_eig, 5)
     const int64_t M = G.dim() > 0 ? G.size(-1) : 0;
     if (M < 1) fail(PyExc_ValueError, "expected matrices [..., M, M], got shape " + shape_text(G.sizes()));
     // (rows longer than the library takes are left to it to refuse: their square might not even be a number of elements)
-    const int32_t matrices = M <= 1024 ? (int32_t)(G.numel() / (M * M)) : 0;
+    const int64_t matrices = M <= 1024 ? G.numel() / (M * M) : 0;
     const long sweeps = PyLong_AsLong(a[3]);
     if (sweeps == -1 && PyErr_Occurred()) throw PythonError{};
-    auto ptr = [](PyObject *o) -> float * {
+    // (the library is told sizes of G alone: what it writes must have room)
+    auto ptr = [](PyObject *o, int64_t least) -> float * {
         if (o == Py_None) return nullptr;
         const at::Tensor &t = tensor(o);
         check(t, at::kFloat, t.sizes());
+        if (t.numel() < least) fail(PyExc_ValueError, "expected at least " + std::to_string(least) + " elements, got shape " + shape_text(t.sizes()));
         return (float *)t.data_ptr();
     };
-    float *g = ptr(a[0]), *ev = ptr(a[1]), *u = ptr(a[2]);
+    float *g = ptr(a[0], 0), *ev = ptr(a[1], matrices * M), *u = ptr(a[2], matrices * M * M);
     flare_stream_t st = stream_of(a[4]);
-    check_status(unlocked([&] { return lib.spectral_eig(matrices, (int32_t)M, g, ev, u, (int32_t)sweeps, st); }), "flare_spectral_eig");
+    check_status(unlocked([&] { return lib.spectral_eig((int32_t)matrices, (int32_t)M, g, ev, u, (int32_t)sweeps, st); }), "flare_spectral_eig");
 BINDING_END
 
 // bind(addresses: dict name -> int, FlareError)

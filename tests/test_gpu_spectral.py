@@ -90,6 +90,18 @@ def test_spectral_error_paths():
     torch.cuda.synchronize()
 
 
+def test_eigenvalue_outputs_without_room_are_refused():
+    """Eigenvalues or eigenvectors shorter than the matrices need raise before anything is launched."""
+    G = torch.eye(16, device="cuda").repeat(3, 1, 1)
+    ev, U = torch.zeros(3, 16, device="cuda"), torch.zeros(3, 16, 16, device="cuda")
+    for short_ev, short_u in ((ev[:2].contiguous(), None), (ev, U[:2].contiguous())):
+        with pytest.raises(ValueError, match="elements"):
+            flare.flare_spectral_eig(G, short_ev, short_u)
+    assert torch.equal(G, torch.eye(16, device="cuda").repeat(3, 1, 1))
+    flare.flare_spectral_eig(G, ev.view(-1))                    # enough elements, whatever their shape
+    assert (ev - 1).abs().max().item() <= 1e-6
+
+
 @pytest.mark.parametrize("M", [1, 2, 3, 31, 33, 64, 65, 128, 129, 192, 193, 234, 236, 512])
 def test_eigenvalues_without_vectors(M):
     """The call without eigenvectors (tridiagonal form, bisection) against numpy in float64: random symmetric matrices, one
