@@ -310,6 +310,16 @@ spectral_gram_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, cons
     if (mi < M && mj < M) Gout[(((size_t)b * H + h) * M + mi) * M + mj] = acc;
 }
 
+// A matrix that holds a NaN or an infinity has no eigenvalues: every output for it is NaN.  (Maxima, comparisons and rotations
+// drop a NaN: without this test a matrix of NaN came out with eigenvalues 0, as if of rank 0.)  One more pass over G, beside M.
+constexpr float kEigNan = __builtin_nanf("");
+// All threads of the block call it.
+__device__ __forceinline__ bool eig_broken(const float *G, int M) {
+    bool bad = false;
+    for (int i = threadIdx.x; i < M * M; i += blockDim.x) bad |= !isfinite(G[i]);
+    return __syncthreads_or(bad);
+}
+
 // Eigenvalues (descending) and, if U != null, eigenvectors (columns of U) of the symmetric matrices G [heads, M, M],
 // by cyclic two-sided Jacobi rotations on disjoint index pairs (round-robin ordering: M - 1 steps of M / 2 rotations
 // per sweep).  One block per matrix; G is overwritten.  Off the hot path: O(M^3) per sweep, about ten sweeps.
@@ -321,6 +331,12 @@ spectral_jacobi_kernel(float *__restrict__ Gall, float *__restrict__ evals, floa
     float *G = Gall + (size_t)blockIdx.x * M * M;
     float *U = Uall ? Uall + (size_t)blockIdx.x * M * M : nullptr;
     const int Me = (M + 1) & ~1, pairs = Me / 2, t = threadIdx.x, T = blockDim.x;
+    if (eig_broken(G, M)) {
+        for (int i = t; i < M; i += T) evals[(size_t)blockIdx.x * M + i] = kEigNan;
+        if (U)
+            for (int i = t; i < M * M; i += T) U[i] = kEigNan;
+        return;
+    }
     if (U)
         for (int i = t; i < M * M; i += T) U[i] = (i / M == i % M) ? 1.f : 0.f;
     __syncthreads();
@@ -477,13 +493,23 @@ spectral_bisect_kernel(const float *__restrict__ tri, float *__restrict__ evals,
     EigPair<float> *qf = reinterpret_cast<EigPair<float> *>(qd + M);
     const float *d = tri + (size_t)blockIdx.y * M * M, *e = d + M;
     const int t = threadIdx.x, lane = t & 31;
-    float top = 0.f;                                            // Gershgorin, by every warp for itself
-    for (int i = lane; i < M; i += 32) top = fmaxf(top, fabsf(d[i]) + (i + 1 < M ? fabsf(e[i]) : 0.f) + (i > 0 ? fabsf(e[i - 1]) : 0.f));
+    double top = 0.0;                                           // Gershgorin, by every warp for itself
+    bool bad = false;                                           // (see eig_broken: the tridiagonal form of such a matrix)
+    for (int i = lane; i < M; i += 32) {
+        const double ei = i + 1 < M ? e[i] : 0.f, eb = i > 0 ? e[i - 1] : 0.f;
+        bad |= !isfinite(d[i]) || !isfinite(ei);
+        top = fmax(top, fabs((double)d[i]) + fabs(ei) + fabs(eb));
+    }
+    if (__any_sync(0xffffffffu, bad)) {                         // (the same in every warp)
+        const int r = blockIdx.x * (TH / kEigSectors) + t;
+        if (t < TH / kEigSectors && r < M) evals[(size_t)blockIdx.y * M + r] = kEigNan;
+        return;
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    for (int o = 16; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
     int ex = 0;
-    frexpf(top, &ex);
-    const double scale = top > 0.f ? ldexp(1.0, -ex) : 1.0;
+    frexp(top, &ex);
+    const double scale = top > 0.0 ? ldexp(1.0, -ex) : 1.0;
     for (int i = t; i < M; i += TH) {
         const double di = d[i] * scale, ei = i > 0 ? e[i - 1] * scale : 0.0;
         qd[i] = {di, fmax(ei * ei, 1e-40)};
@@ -511,11 +537,12 @@ spectral_bisect_kernel(const float *__restrict__ tri, float *__restrict__ evals,
         if (n < kEigSectors) hi = base + step * (n + 1);
         if (pass == 3) { lo -= 1.9e-6; hi += 1.9e-6; }
     }
-    if (r < M && sub == 0) evals[(size_t)blockIdx.y * M + r] = top > 0.f ? (float)(0.5 * (lo + hi) / scale) : 0.f;
+    if (r < M && sub == 0) evals[(size_t)blockIdx.y * M + r] = top > 0.0 ? (float)(0.5 * (lo + hi) / scale) : 0.f;
 }
 
 // Largest magnitude over the block as a power of two to scale by, so that squares of the entries neither overflow nor
-// vanish: returns 2^-e with e the exponent of the largest (1 for a zero or non-finite matrix).  All threads call it.
+// vanish: returns 2^-e with e the exponent of the largest, as near to it as 2^-e is a normal number (1 for a zero matrix; the
+// entries are finite).  All threads call it.
 __device__ __forceinline__ float eig_block_scale(float mx, float *sh32) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -525,9 +552,9 @@ __device__ __forceinline__ float eig_block_scale(float mx, float *sh32) {
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) mx = fmaxf(mx, sh32[i]);
     __syncthreads();
     int e = 0;
-    if (!(mx > 0.f) || !(mx <= 3.0e38f)) return 1.f;
+    if (!(mx > 0.f)) return 1.f;
     frexpf(mx, &e);
-    return ldexpf(1.f, e > 126 ? -126 : -e);
+    return ldexpf(1.f, e > 126 ? -126 : e < -126 ? 126 : -e);
 }
 
 // The matrix in registers: NG groups of CX threads, thread (g, j) holds rows g, g + NG, ... of column j.  Vectors that are
@@ -544,11 +571,17 @@ spectral_tridiag_reg_kernel(float *__restrict__ Gall, int M) {
     const int t = threadIdx.x, lane = t & 31, j = t % CX, g = t / CX;
     float *G = Gall + (size_t)blockIdx.x * M * M;
     float A[R], mx = 0.f;
+    bool bad = false;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = g + NG * r;
         A[r] = (j < M && i < M) ? G[(size_t)i * M + j] : 0.f;
         mx = fmaxf(mx, fabsf(A[r]));
+        bad |= !isfinite(A[r]);
+    }
+    if (__syncthreads_or(bad)) {                                // (see eig_broken)
+        if (t == 0) G[0] = kEigNan;
+        return;
     }
     const float scale = eig_block_scale(mx, red);
 #pragma unroll
@@ -657,6 +690,10 @@ spectral_tridiag_kernel(float *__restrict__ Gall, int M) {
     float *G = Gall + (size_t)blockIdx.x * M * M;
     float *A = kShared ? part + (size_t)NG * M : G;
     __shared__ float red[32];
+    if (eig_broken(G, M)) {
+        if (t == 0) G[0] = kEigNan;                             // (one is enough for spectral_bisect_kernel)
+        return;
+    }
     float mx = 0.f;
     for (int i = t; i < M * M; i += TH) mx = fmaxf(mx, fabsf(G[i]));
     const float scale = eig_block_scale(mx, red);

@@ -122,3 +122,31 @@ def test_eigenvalues_without_vectors(M):
     got = to_np64(ev)
     for i in range(5):
         assert np.abs(got[i] - want[i]).max() <= 1e-6 * np.abs(want[i]).max(), i
+
+
+@pytest.mark.parametrize("vectors", [False, True])
+@pytest.mark.parametrize("M", [1, 2, 33, 192, 200, 300])
+def test_matrices_without_eigenvalues(M, vectors):
+    """A matrix with a NaN or an infinity anywhere gives NaN throughout, its neighbours in the same call are not touched by it,
+    and finite matrices at either end of the float32 range are not taken for one.  (Bound of the finite ones: as above; the last is
+    subnormal, in steps of 2^-149, so an absolute error of a few steps is allowed; only without eigenvectors, where entries are scaled.)"""
+    rng = np.random.default_rng(M)
+    X = rng.standard_normal((8, M, M))
+    G = ((X + X.transpose(0, 2, 1)) / 2).astype(np.float32)
+    G[1] = np.nan
+    G[2, M - 1, M // 2] = np.nan
+    G[3, M // 2, M - 1] = G[3, M - 1, M // 2] = np.inf
+    G[4, 0, 0] = -np.inf
+    G[6] = np.diag(np.linspace(-3.3e38, 3.3e38, M)) if M > 1 else 3.3e38
+    G[7] *= 1e-41
+    ev = torch.zeros(8, M, device="cuda")
+    U = torch.zeros(8, M, M, device="cuda") if vectors else None
+    flare.flare_spectral_eig(torch.from_numpy(G).cuda(), ev, U)
+    got = to_np64(ev)
+    assert np.isnan(got[1:5]).all()
+    if vectors:
+        assert np.isnan(to_np64(U)[1:5]).all() and np.isfinite(to_np64(U)[[0, 5]]).all()
+    for i in (0, 5) if vectors else (0, 5, 6, 7):
+        want = np.linalg.eigvalsh(G[i].astype(np.float64))[::-1]
+        bound = max(2e-4, 4e-6 * M) if vectors else 1e-6           # (rotations: as in test_gram_and_eigenvalues)
+        assert np.abs(got[i] - want).max() <= bound * np.abs(want).max() + (M + 4) * 2.0 ** -149, i
