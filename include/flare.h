@@ -88,7 +88,11 @@ const char *flare_last_cuda_error(void);
  */
 size_t flare_workspace_bytes(const flare_desc_t *desc, int op);
 
-/* Number of partial results per (b, h, latent) that encode produces and the merge step combines. */
+/*
+ * Number of partial results per (b, h, latent) that flare_encode has room for and the merge step combines.  (The encode of a
+ * flare_forward may split the tokens finer where that is faster: flare_encode keeps its scratch small enough for
+ * flare_encode_static_scratch wherever that is possible.)
+ */
 int flare_encode_partials(const flare_desc_t *desc);
 
 /*

@@ -67,14 +67,14 @@ int launches_for(const flare_desc_t *d, int op, int sms) {
 
 // Scratch of one flare_forward.
 size_t forward_bytes(const flare_desc_t *d) {
-    return make_layout(partials_for(d, device_info().sms), (long)d->B * d->H * d->M, d->D, true).total + decode_range_bytes(d);
+    return make_layout(partials_for(d, device_info().sms, false), (long)d->B * d->H * d->M, d->D, true).total + decode_range_bytes(d);
 }
 
 int forward_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, void *Y, float *Z, float *lse_enc,
                  float *lse_dec, void *workspace, cudaStream_t st, bool keep_status) {
-    const WorkspaceLayout w = make_layout(partials_for(d, device_info().sms), (long)d->B * d->H * d->M, d->D, true);
+    const WorkspaceLayout w = make_layout(partials_for(d, device_info().sms, false), (long)d->B * d->H * d->M, d->D, true);
     if (Z == nullptr) Z = reinterpret_cast<float *>(static_cast<char *>(workspace) + w.z);
-    const int rc = encode_impl(d, Q, K, V, mask, Z, lse_enc, workspace, st, keep_status);
+    const int rc = encode_impl(d, Q, K, V, mask, Z, lse_enc, workspace, st, false, keep_status);
     if (rc != FLARE_OK) return rc;
     char *range_scratch = decode_in_ranges(d) ? static_cast<char *>(workspace) + w.total : nullptr;
     return decode_impl(d, Q, K, Z, Y, lse_dec, reinterpret_cast<uint32_t *>(workspace), st, range_scratch);
@@ -265,7 +265,7 @@ const char *flare_last_cuda_error(void) { return g_cuda_error; }
 
 int flare_encode_partials(const flare_desc_t *desc) {
     if (check_desc(desc) != FLARE_OK) return 0;
-    return partials_for(desc, device_info().sms);
+    return partials_for(desc, device_info().sms, true);
 }
 
 int flare_launch_count(const flare_desc_t *desc, int op) {
@@ -277,7 +277,7 @@ size_t flare_workspace_bytes(const flare_desc_t *desc, int op) {
     if (check_desc(desc) != FLARE_OK) return 0;
     const long rows = (long)desc->B * desc->H * desc->M;
     switch (op) {
-        case FLARE_OP_ENCODE: return make_layout(partials_for(desc, device_info().sms), rows, desc->D, false).total;
+        case FLARE_OP_ENCODE: return make_layout(partials_for(desc, device_info().sms, true), rows, desc->D, false).total;
         case FLARE_OP_DECODE: return kHeaderBytes + decode_range_bytes(desc);
         case FLARE_OP_FORWARD: {
             // (room for the parts that flare_forward_host works a batch off in: fewer rows, but more CTAs along N for each)
@@ -302,7 +302,7 @@ int flare_encode(const flare_desc_t *desc, const void *Q_lat, const void *K, con
         return FLARE_ERR_INVALID_ARG;
     if ((rc = require_device()) != FLARE_OK) return rc;
     if (workspace_bytes < flare_workspace_bytes(desc, FLARE_OP_ENCODE)) return FLARE_ERR_WORKSPACE_TOO_SMALL;
-    return encode_impl(desc, Q_lat, K, V, key_mask, Z, lse_enc, workspace, (cudaStream_t)stream);
+    return encode_impl(desc, Q_lat, K, V, key_mask, Z, lse_enc, workspace, (cudaStream_t)stream, true);
 }
 
 int flare_encode_static_scratch(const flare_desc_t *desc, const void *Q_lat, const void *K, const void *V,
@@ -322,7 +322,7 @@ int flare_encode_static_scratch(const flare_desc_t *desc, const void *Q_lat, con
     void *scratch = nullptr;
     if ((rc = static_scratch_address(&scratch)) != FLARE_OK) return rc;
     // encode_impl zeroes the header words that must start at zero; every partial it later reads it first writes
-    return encode_impl(desc, Q_lat, K, V, key_mask, Z, lse_enc, scratch, (cudaStream_t)stream);
+    return encode_impl(desc, Q_lat, K, V, key_mask, Z, lse_enc, scratch, (cudaStream_t)stream, true);
 }
 
 int flare_decode(const flare_desc_t *desc, const void *Q_lat, const void *K, const float *Z, void *Y, float *lse_dec,
@@ -441,9 +441,9 @@ int flare_forward_variant(const flare_desc_t *desc, int shared_latents, const vo
             qd = ws + v.qd;
         }
     }
-    const WorkspaceLayout w = make_layout(partials_for(desc, device_info().sms), (long)desc->B * desc->H * desc->M, desc->D, true);
+    const WorkspaceLayout w = make_layout(partials_for(desc, device_info().sms, false), (long)desc->B * desc->H * desc->M, desc->D, true);
     if (Z == nullptr) Z = reinterpret_cast<float *>(ws + w.z);
-    if ((rc = encode_impl(desc, qe, K, V, key_mask, Z, lse_enc, workspace, st)) != FLARE_OK) return rc;
+    if ((rc = encode_impl(desc, qe, K, V, key_mask, Z, lse_enc, workspace, st, false)) != FLARE_OK) return rc;
     char *range_scratch = decode_in_ranges(desc) ? ws + w.total : nullptr;
     return decode_impl(desc, qd, K, Z, Y, lse_dec, reinterpret_cast<uint32_t *>(workspace), st, range_scratch);
 }

@@ -109,7 +109,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
     bool dz_on_tc = skip_pass_a;
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         if (!skip_pass_a && bwd_dz_on_tensor_cores(d)) {
-            const LeanPlan tp = lean_plan(d, sms);
+            const LeanPlan tp = dz_plan(d, sms);
             uint32_t *status = reinterpret_cast<uint32_t *>(ws);
             const int rc = encode_dz_tc(d, tp, Q, K, dY, part, status, st, lse_dec);
             if (rc != FLARE_OK) return rc;

@@ -86,10 +86,10 @@ int launch_lean(const flare_desc_t *d, const LeanPlan &p, const void *Q, const v
 }  // namespace
 
 int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
-                float *lse_enc, void *ws, cudaStream_t st, bool keep_status) {
+                float *lse_enc, void *ws, cudaStream_t st, bool alone, bool keep_status) {
     const DeviceView di = device_info();
     const long rows = (long)d->B * d->H * d->M;
-    const int P = partials_for(d, di.sms);
+    const int P = partials_for(d, di.sms, alone);
     WorkspaceLayout w = make_layout(P, rows, d->D, false);
     char *base = static_cast<char *>(ws);
     float *pm = reinterpret_cast<float *>(base + w.part_m);
@@ -105,7 +105,7 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
         // a caller that asks for lse_enc is saving Z for the backward: weights as two bf16 halves (see exp_chunk_hilo)
         const bool fast = use_fast_encode(d);
         if (fast) {                                             // the exact form, behind it, exits at once unless the fast one raised its flag
-            const LeanPlan lp = lean_plan(d, di.sms);
+            const LeanPlan lp = encode_lean_plan(d, di.sms, alone);
             EncodeLeanArgs a{};
             a.key_mask = mask; a.part_m = pm; a.part_l = pl; a.part_acc = pacc; a.status = status; a.redo = status + kRedoEncodeWord;
             rc = lse_enc != nullptr ? launch_lean<kLeanHiLo>(d, lp, Q, K, V, a, st) : launch_lean<kLeanFast>(d, lp, Q, K, V, a, st);

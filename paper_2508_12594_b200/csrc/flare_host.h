@@ -180,9 +180,10 @@ struct TcEncodePlan {
 // that one more split than fills the chip once can take twice as long and several times as many less than once (64 pieces: 2 splits leave
 // 20 of 148 SMs idle, 23 in ten rounds 0.5); each split also leaves a partial result of `part_bytes` to be reduced (some 4 MB
 // written and read in a tile's time).  At most 512 tiles per split keep the float32 sums on the tensor core short.
-inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes) {
+// At most `cap` splits, whatever the sums' length.
+inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes, int cap) {
     const double start = 4.0, reduce = (double)part_bytes / 4.0e6;
-    const int least = (tiles + 511) / 512, most = tiles < least + sms ? tiles : least + sms;
+    const int least = std::min((tiles + 511) / 512, cap), most = std::min(std::min(tiles, least + sms), cap);
     int best = least;
     double best_cost = 0.0;
     for (int s = least; s <= most; ++s) {
@@ -210,18 +211,32 @@ inline TcEncodePlan tc_encode_plan(const flare_desc_t *d, int sms) {
 
 // Launch plan of the encode without a running maximum and of dZ: one partial result per CTA.  Up to 64 latents two heads share the lanes.
 struct LeanPlan { int tiles, blocks, splits; };
-inline LeanPlan lean_plan(const flare_desc_t *d, int sms) {
+inline LeanPlan lean_plan(const flare_desc_t *d, int sms, int cap) {
     LeanPlan p;
     p.tiles = (d->N + kTile - 1) / kTile;
     p.blocks = lean_pairs(d) ? 1 : (d->M + kTile - 1) / kTile;
     const long groups = (long)d->B * (lean_pairs(d) ? d->H / 2 : d->H) * p.blocks;
-    p.splits = balanced_splits(groups, p.tiles, sms, (size_t)d->B * d->H * d->M * (d->D + 2) * sizeof(float));
+    p.splits = balanced_splits(groups, p.tiles, sms, (size_t)d->B * d->H * d->M * (d->D + 2) * sizeof(float), cap);
     return p;
 }
+inline LeanPlan dz_plan(const flare_desc_t *d, int sms) { return lean_plan(d, sms, d->N); }   // (no more splits than tokens: no cap)
+// alone: a call of encode by itself.  Its scratch decides whether flare_encode_static_scratch takes a problem: what the exact form brings
+// into the built-in array must fit it in this form too, whose plan often splits finer (1048576 tokens, 8 heads, 2048 latents, D = 8: 4 partial
+// results against 22, 2.5 MB against 14.4).  The encode of a forward, in a workspace of the caller's, keeps the finer plan.
+inline LeanPlan encode_lean_plan(const flare_desc_t *d, int sms, bool alone) {
+    const long rows = (long)d->B * d->H * d->M;
+    const int exact = tc_encode_plan(d, sms).P;
+    if (!alone || make_layout(exact, rows, d->D, false).total > FLARE_STATIC_SCRATCH_BYTES) return lean_plan(d, sms, d->N);
+    const size_t part = sizeof(float) * (size_t)rows * (d->D + 2);   // (beside the header; three sections are rounded up)
+    return lean_plan(d, sms, std::max(exact, (int)std::min<size_t>(d->N, (FLARE_STATIC_SCRATCH_BYTES - kHeaderBytes - 3 * kAlign) / part)));
+}
 
-// (either form of encode on the tensor cores may have to leave its partial results in the same workspace)
-inline int partials_for(const flare_desc_t *d, int sms) {
-    return use_tc(d) ? std::max(tc_encode_plan(d, sms).P, lean_plan(d, sms).splits) : simt_plan(d, sms).P;
+// (either form of encode on the tensor cores may have to leave its partial results in the same workspace; which one runs may change with
+// flare_set_path while a caller keeps the workspace.  At D = 64 there is only the exact form, see use_fast_encode.)
+inline int partials_for(const flare_desc_t *d, int sms, bool alone) {
+    if (!use_tc(d)) return simt_plan(d, sms).P;
+    const int exact = tc_encode_plan(d, sms).P;
+    return d->D <= 32 ? std::max(exact, encode_lean_plan(d, sms, alone).splits) : exact;
 }
 
 // ---- TMA descriptors (the driver entry point is looked up at run time; the library does not link libcuda)
@@ -326,7 +341,7 @@ inline TcEncodePlan tc_dq_plan(const flare_desc_t *d, int sms) {
     p.tiles = (d->N + kTile - 1) / kTile;
     p.pairs = encode_head_pairs(d) ? 1 : (d->M + kTile - 1) / kTile;
     const long groups = (long)d->B * (encode_head_pairs(d) ? d->H / 2 : d->H) * p.pairs;
-    p.splits = balanced_splits(groups, p.tiles, sms, (size_t)d->B * d->H * d->M * d->D * sizeof(float));
+    p.splits = balanced_splits(groups, p.tiles, sms, (size_t)d->B * d->H * d->M * d->D * sizeof(float), p.tiles);
     p.per_split = 1;
     p.P = p.splits;
     return p;
@@ -351,7 +366,7 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     const long rows = (long)d->B * d->H * d->M;
     const int pa = simt_plan(d, sms).P, pb = bwd_dq_plan(d, sms).P;
     w.P = pa > pb ? pa : pb;
-    if (bwd_dz_on_tensor_cores(d) && lean_plan(d, sms).splits > w.P) w.P = lean_plan(d, sms).splits;
+    if (bwd_dz_on_tensor_cores(d) && dz_plan(d, sms).splits > w.P) w.P = dz_plan(d, sms).splits;
     if (bwd_dq_on_tensor_cores(d) && tc_dq_plan(d, sms).P > w.P) w.P = tc_dq_plan(d, sms).P;
     size_t off = kHeaderBytes;
     w.part = off; off += align_up(sizeof(float) * (size_t)w.P * rows * d->D);
@@ -377,9 +392,10 @@ int bwd_token_simt(const flare_desc_t *d, const void *Q, const void *K, const vo
 int bwd_dq_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *V, const uint8_t *mask,
                 const void *dY, const float *Z, const float *dZ, const float *de, const float *dd, const float *lse_enc,
                 const float *lse_dec, float *part, cudaStream_t st);
-// keep_status: leave the error word of the workspace header as it is (a later part of a call in several parts)
+// alone: not as part of a forward (see encode_lean_plan).  keep_status: leave the error word of the workspace header as it is (a later
+// part of a call in several parts)
 int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
-                float *lse_enc, void *ws, cudaStream_t st, bool keep_status = false);
+                float *lse_enc, void *ws, cudaStream_t st, bool alone, bool keep_status = false);
 int encode_dz_tc(const flare_desc_t *d, const LeanPlan &p, const void *Q, const void *K, const void *dY, float *part,
                  uint32_t *status, cudaStream_t st, const float *lse_dec);
 // range_scratch: decode_range_bytes(d) bytes, or null (then more than kDecodeMaxM latents take the CUDA-core kernel)

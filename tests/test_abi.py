@@ -91,3 +91,22 @@ def test_eigenvalues_of_empty_matrices_are_refused(lib):
     for shape in ((0, 0), (3, 0, 0), (5, 0), (0,), (), (0, 1 << 32)):
         with pytest.raises((ValueError, flare.FlareError)):
             flare.flare_spectral_eig(torch.empty(shape), torch.empty(0))
+
+
+# Shapes whose partial results in the exact form take 1.3 to 6.4 MB (splits x partial results a split x rows x (D + 2) floats).
+STATIC_SCRATCH_SHAPES = [(2, 8, 16384, 2048, 16), (4, 16, 16384, 512, 16), (32, 4, 65536, 32, 64), (32, 4, 65536, 96, 32), (1, 8, 65536, 2048, 16),
+                         (1, 8, 262144, 1024, 16), (1, 8, 1048576, 2048, 8), (4, 16, 1048576, 272, 8), (4, 4, 1048576, 1024, 4)]
+
+
+@pytest.mark.parametrize("shape", STATIC_SCRATCH_SHAPES, ids=str)
+def test_many_latents_fit_the_built_in_scratch(lib, shape):
+    """flare_encode_static_scratch takes what fits its array in the exact form, also where another form runs."""
+    desc = flare.FlareDesc(*shape, flare.DTYPE_BF16, 1.0)
+    assert 0 < flare.flare_workspace_bytes(desc, flare.OP_ENCODE) <= flare.STATIC_SCRATCH_BYTES
+    assert flare.flare_workspace_bytes(desc, flare.OP_FORWARD) >= flare.flare_workspace_bytes(desc, flare.OP_ENCODE)
+
+
+def test_scratch_at_head_width_64_is_that_of_the_exact_form(lib):
+    """D = 64 has no other form: one partial result per split and pair of latent blocks, up to 148 / (B H) splits."""
+    desc = flare.FlareDesc(1, 4, 65536, 256, 64, flare.DTYPE_BF16, 1.0)
+    assert flare.flare_encode_partials(desc) == 2 * (148 // 4)

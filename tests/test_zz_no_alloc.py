@@ -54,6 +54,24 @@ def test_static_scratch_encode_matches_encode_twice_in_a_row(oracle):
         assert np.abs(to_np64(le)[fin] - leo[fin]).max() <= (1e-4 if dtype == "f32" else 2e-2), w.name
 
 
+def test_static_scratch_with_many_latents():
+    """Shapes whose plan without a cap would take 9 MB: the same numbers as flare_encode, and those of the exact form within the forward's
+    bound on either."""
+    for w in (workloads.CONFIGS["field_1m"].with_(N=65536, M=2048, D=16), workloads.CONFIGS["field_1m"].with_(B=4, H=16, N=16384, M=512, D=16)):
+        inp = workloads.make_inputs(w)
+        flare.flare_set_path(flare.PATH_FAST)
+        try:
+            (Z, le), (Z_ref, le_ref) = _encode_both(inp)
+            flare.flare_check(None)
+            flare.flare_set_path(flare.PATH_EXACT)
+            (Z_exact, le_exact), _ = _encode_both(inp)
+        finally:
+            flare.flare_set_path(flare.PATH_AUTO)
+        assert torch.equal(Z, Z_ref) and torch.equal(le, le_ref), w.name
+        assert rel_err(to_np64(Z), to_np64(Z_exact)) <= 2 * TOL["bf16"], w.name
+        assert (le - le_exact).abs().max().item() <= 4e-2, w.name
+
+
 def test_static_scratch_refuses_what_does_not_fit():
     big = flare.FlareDesc(64, 8, 4096, 512, 64, flare.DTYPE_BF16, 1.0)
     assert flare.flare_workspace_bytes(big, flare.OP_ENCODE) > flare.STATIC_SCRATCH_BYTES
