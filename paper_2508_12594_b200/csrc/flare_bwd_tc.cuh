@@ -8,7 +8,7 @@
 // Both kernels turn three tiles that the tensor core puts side by side in tensor memory, S = q.k, A = dY.Z and C = dZ.V, into
 // dS (and W_enc) over the columns just read, which feed the output contractions as their A operand.  One kind of row sits
 // on the 128 lanes (latents in the dQ kernel, tokens in the token kernel), the other on the columns, in units of 64 or 32.
-// Z and dZ, and dS and W_enc, enter as two bf16 halves each: the sums cancel (see the host code's notes on precision).
+// Z and dZ, and dS and W_enc, enter as two bf16 halves each, because the sums cancel; for dQ at D = 64 Z, dZ and dS as three.
 //
 // What shapes them.  A tcgen05.mma with both operands in shared memory takes the tensor core 40 cycles at N = 16 or 32, 48 at 64 and 64
 // at 128 (most of it the fetch of its A operand), one with A in tensor memory N / 2; a hand-over between threads and tensor core
@@ -31,8 +31,9 @@ namespace flare {
 // W_enc, kTwo: xe = s * sl2 + ne.  (An exponential costs the special-function unit as much as the rest of a pair costs the
 // issue slots: with two per pair the unit bound both kernels.)
 constexpr float kOneExpLog2 = 40.f;
-struct DsPair { uint32_t hi, lo, whi, wlo; };
-template <bool kWeights, bool kTwo>
+// kThird: dS in three parts (24 bits: all of the float32 value).
+struct DsPair { uint32_t hi, lo, lo2, whi, wlo; };
+template <bool kWeights, bool kTwo, bool kThird>
 __device__ __forceinline__ DsPair ds_pair(float2 s, float2 av, float2 cv, float2 sl2p, float2 nd, float2 na, float2 nc, float2 fr_ne, float2 fc) {
     const float2 xd = __ffma2_rn(s, sl2p, nd);
     const float2 pd = make_float2(ptx::ex2(xd.x), ptx::ex2(xd.y));
@@ -49,7 +50,9 @@ __device__ __forceinline__ DsPair ds_pair(float2 s, float2 av, float2 cv, float2
     }
     DsPair o;
     o.hi = ptx::pack_bf16(ds.x, ds.y);
-    o.lo = ptx::pack_bf16(ds.x - __uint_as_float(o.hi << 16), ds.y - __uint_as_float(o.hi & 0xffff0000u));
+    const float2 rest = make_float2(ds.x - __uint_as_float(o.hi << 16), ds.y - __uint_as_float(o.hi & 0xffff0000u));
+    o.lo = ptx::pack_bf16(rest.x, rest.y);
+    if (kThird) o.lo2 = ptx::pack_bf16(rest.x - __uint_as_float(o.lo << 16), rest.y - __uint_as_float(o.lo & 0xffff0000u));
     if (kWeights) {
         o.whi = ptx::pack_bf16(pe.x, pe.y);
         o.wlo = ptx::pack_bf16(pe.x - __uint_as_float(o.whi << 16), pe.y - __uint_as_float(o.whi & 0xffff0000u));
@@ -69,9 +72,11 @@ __device__ __forceinline__ float warp_lse_min(const float *lse_enc, int rows) {
     return k <= 3.0e38f ? k : 0.f;
 }
 
-// rows of a [rows, DR] float matrix -> bf16 halves in swizzled rows (DR >= 8), starting at logical chunk `chunk0` of row r0 + m
-template <int DG, int DR>
-__device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float *src, int rows, int r0, int chunk0, int tid, int threads) {
+// rows of a [rows, DR] float matrix -> bf16 halves (kThird: three parts, the third in lo2) in swizzled rows (DR >= 8), starting at
+// logical chunk `chunk0` of row r0 + m
+template <int DG, int DR, bool kThird = false>
+__device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float *src, int rows, int r0, int chunk0, int tid, int threads,
+                                           uint8_t *lo2 = nullptr) {
     using G = TileGeom<DG>;
     constexpr int ZC = DR >= 8 ? DR / 8 : 1;
     for (int i = tid; i < rows * ZC; i += threads) {
@@ -79,15 +84,18 @@ __device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float
         const float4 a = *reinterpret_cast<const float4 *>(src + (size_t)m * DR + c * 8);
         const float4 b = *reinterpret_cast<const float4 *>(src + (size_t)m * DR + c * 8 + 4);
         const float z[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        uint32_t vh[4], vl[4];
+        uint32_t vh[4], vl[4], vl2[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             vh[k] = ptx::pack_bf16(z[2 * k], z[2 * k + 1]);
-            vl[k] = ptx::pack_bf16(z[2 * k] - __uint_as_float(vh[k] << 16), z[2 * k + 1] - __uint_as_float(vh[k] & 0xffff0000u));
+            const float x = z[2 * k] - __uint_as_float(vh[k] << 16), y = z[2 * k + 1] - __uint_as_float(vh[k] & 0xffff0000u);
+            vl[k] = ptx::pack_bf16(x, y);
+            if (kThird) vl2[k] = ptx::pack_bf16(x - __uint_as_float(vl[k] << 16), y - __uint_as_float(vl[k] & 0xffff0000u));
         }
         const size_t o = (size_t)r * G::RB + (((chunk0 + c) ^ G::swz(r)) << 4);
         *reinterpret_cast<uint4 *>(hi + o) = make_uint4(vh[0], vh[1], vh[2], vh[3]);
         *reinterpret_cast<uint4 *>(lo + o) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
+        if (kThird) *reinterpret_cast<uint4 *>(lo2 + o) = make_uint4(vl2[0], vl2[1], vl2[2], vl2[3]);
     }
 }
 // ------------------------------------------------------------------------------- pass B, latent side (dQ)
@@ -97,7 +105,8 @@ __device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float
 // Warps: 0 TMA producer, 1 MMA issue, 3 column constants, 4-19 arithmetic (warp & 3 = the quarter of the lanes it can reach).
 // Measured, us, against units of 16 columns with two exponentials per pair (N = 16384, M = 32, D = 32, 8 heads; 32 x 4096, M = 128, 4 heads;
 // 131072, M = 512, 8 heads; 1048576, M = 1024, D = 8, 8 heads): 22.4, 82, 437, 7844 -> 15.9, 65, 392, 5706; D = 64 (2 x 20011, M = 128, 4
-// heads), on the CUDA cores before: 498 -> 27.  Groups of four warps with units and buffers of their own, as in the token kernel:
+// heads), on the CUDA cores before: 498 -> 27 (in three
+// parts, see kThird, 31).  Groups of four warps with units and buffers of their own, as in the token kernel:
 // 21.6, 78, 522, 7485; 44.  Issue slots and the latency of tensor-memory loads share the bound (some 14 instructions per pair, two issued
 // per cycle and SM).
 constexpr int kDqUnit = 64, kDqBuf = 3 * kDqUnit, kDqAcc = 2 * kDqBuf;
@@ -120,10 +129,11 @@ struct BwdDqTcArgs {
 template <int DG, bool kPair>
 struct BwdDqSmem {
     using G = TileGeom<DG>;
+    static constexpr int kParts = DG == 64 && !kPair ? 3 : 2, kLat = 1 + 2 * kParts;   // parts of Z and dZ (see the kernel); with Q, latent operands
     static constexpr int kCst = 8, kAhead = 4;                                   // tiles of column constants in the ring, of them on their way
     static constexpr size_t kCstBytes = (size_t)(kPair ? 2 : 1) * 3 * kTile * sizeof(float);   // per head: -lse_dec, -dd, mask
     static constexpr size_t total_for(int n) {
-        return (size_t)n * 3 * G::TILE_BYTES + (size_t)5 * kTile * G::RB + kCst * kCstBytes + 768 + 1024;
+        return (size_t)n * 3 * G::TILE_BYTES + (size_t)kLat * kTile * G::RB + kCst * kCstBytes + 768 + 1024;
     }
     static constexpr int stages_for() {
         int n = 6;
@@ -132,7 +142,7 @@ struct BwdDqSmem {
     }
     static constexpr int kStages = stages_for();                                 // (K, V, dY) tile triples in flight
     __host__ __device__ static constexpr size_t lat_off(int which) { return (size_t)kStages * 3 * G::TILE_BYTES + (size_t)which * kTile * G::RB; }
-    static constexpr size_t cst_off = (size_t)kStages * 3 * G::TILE_BYTES + (size_t)5 * kTile * G::RB;
+    static constexpr size_t cst_off = lat_off(kLat);
     static constexpr size_t bar_off = cst_off + kCst * kCstBytes;
     static constexpr size_t total = total_for(kStages) < kTcMinSmem ? kTcMinSmem : total_for(kStages);
 };
@@ -154,6 +164,15 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     // The units take turns on as many accumulators as there is room for: the tensor core truncates each of the thousands of sums that a
     // split adds up in float32, an error that grows with their number.
     constexpr int kAccs = (512 - kDqAcc) / DG;
+    // D = 64: the three products carry all 24 bits of Z, dZ and dS, in three parts each, and a unit's sums go to float32 sums in registers
+    // two units later, when their accumulator is free again: 16 of the 64 columns to each of the four warps that share a quarter of the lanes.
+    // (This width used to run in float32 arithmetic on the CUDA cores, twenty times slower.  In halves, summed in tensor memory, as the
+    // other widths are, dQ was 1.5 to 2.3 times as far from float64 as there; now 0.5 to 1.04 times, what is left being the weights in halves
+    // that Z and dZ were formed with.  2 x 20011 tokens, M = 128, 4 heads, relative to the norm, float32 / halves / parts: 2.6e-6 / 4.9e-6 /
+    // 2.6e-6, on features of point clouds 5.1e-6 / 7.2e-6 / 2.9e-6.  That training step: 182 us in halves, 186 with this, 192 with
+    // the token kernel's third part.)
+    constexpr bool kThird = SM::kParts == 3;
+    static_assert(!kThird || (kAccs == 2 && D == 64 && DRT == 0), "a warp's columns, and the buffer's accumulator");
     static_assert(kAccs >= 1 && (kAccs & (kAccs - 1)) == 0, "tensor memory");
     constexpr int UNIT = kDqUnit, UPT = kTile / UNIT, nstages = SM::kStages;
     static_assert(nstages >= 2, "one tile is finished while the next begins");
@@ -196,10 +215,10 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             if (lane == 0) kmin[w] = k;
         }
     }
-    // latent operands Q, Z_hi, Z_lo, dZ_hi, dZ_lo: zeros where there is no row (or, pair and narrow forms, no feature), then the rows
+    // latent operands Q, Z_hi, Z_lo, dZ_hi, dZ_lo (D = 64: three parts of Z and dZ): zeros where there is no row (or, pair and narrow forms, no feature), then the rows
     const bool gaps = kPair || DRT != 0 || rows_here < kTile;
     if (gaps) {
-        for (int i = threadIdx.x; i < 5 * kTile * (G::RB / 16); i += kDqThreads)
+        for (int i = threadIdx.x; i < SM::kLat * kTile * (G::RB / 16); i += kDqThreads)
             reinterpret_cast<uint4 *>(smem + SM::lat_off(0))[i] = make_uint4(0, 0, 0, 0);
         __syncthreads();
     }
@@ -212,8 +231,11 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             stage_rows4_hilo<DG>(smem + SM::lat_off(3), smem + SM::lat_off(4), a.dZ + r0 * DR, rows_here, off);
         } else {
             stage_bf16<DG, DR>(smem + SM::lat_off(0), a.Q + q0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
-            stage_hilo<DG, DR>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
-            stage_hilo<DG, DR>(smem + SM::lat_off(3), smem + SM::lat_off(4), a.dZ + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
+            stage_hilo<DG, DR, kThird>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads,
+                                       smem + SM::lat_off(3));
+            constexpr int dz0 = 1 + SM::kParts;
+            stage_hilo<DG, DR, kThird>(smem + SM::lat_off(dz0), smem + SM::lat_off(dz0 + 1), a.dZ + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x,
+                                       kDqThreads, smem + SM::lat_off(SM::kLat - 1));
         }
     }
     ptx::fence_proxy_async_smem();
@@ -313,7 +335,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             const uint32_t lat0 = ptx::desc_lo(ptx::smem_u32(smem + SM::lat_off(0)), 16), k0 = ptx::desc_lo(ptx::smem_u32(smem), 16);
             constexpr uint32_t MN = ptx::desc_lo(0, G::SBO) - ptx::desc_lo(0, 16);          // K-major to MN-major
             int s_stage = 0, s_wrap = 0, s_u = 0, o_stage = 0, o_u = 0;
-            // S = Q K^T | A = (Z_hi + Z_lo) dY^T | C = (dZ_hi + dZ_lo) V^T of the next unit, into buffer n & 1
+            // S = Q K^T | A = (Z_hi + Z_lo) dY^T | C = (dZ_hi + dZ_lo) V^T of the next unit, into buffer n & 1 (D = 64: three parts)
             auto tiles = [&](int n) -> bool {
                 if (s_u == 0) {
                     if (!ptx::mbar_wait(bar(T_FULL + s_stage), (uint32_t)s_wrap, abort_flag, kErrBwdDq | 3)) return false;
@@ -324,11 +346,14 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 ptx::opaque(ld);
                 const uint32_t bcol = tm + (n & 1) * kDqBuf;
 #pragma unroll
-                for (int w = 0; w < 5; ++w) {                   // Q with K; Z hi, lo with dY; dZ hi, lo with V
-                    const uint32_t col = bcol + (w == 0 ? 0 : w <= 2 ? UNIT : 2 * UNIT), td = kd + (w == 0 ? 0 : w <= 2 ? 2 * TILE : TILE);
+                for (int i = 0; i < SM::kLat; ++i) {            // Q with K; the parts of Z with dY; those of dZ with V
+                    const int of = i == 0 ? 0 : i <= SM::kParts ? 1 : 2, at = of == 0 ? 0 : (i - 1) % SM::kParts;
+                    const int w = of == 0 ? 0 : 1 + (of - 1) * SM::kParts + (kThird ? SM::kParts - 1 - at : at);   // (kThird: small parts first)
+                    const uint32_t col = bcol + of * UNIT, td = kd + (of == 0 ? 0 : of == 1 ? 2 * TILE : TILE);
+                    const bool more = at > 0;                   // adds to an earlier part's product
 #pragma unroll
                     for (int k = 0; k < DG / 16; ++k)
-                        ptx::mma_ss(col, ptx::desc(ld + w * LAT + 2 * k, HI), ptx::desc(td + 2 * k, HI), idescS, k > 0 || w == 2 || w == 4);
+                        ptx::mma_ss(col, ptx::desc(ld + w * LAT + 2 * k, HI), ptx::desc(td + 2 * k, HI), idescS, k > 0 || more);
                 }
                 ptx::mma_commit(bar(S_FULL + (n & 1)));
                 if (++s_u == UPT) {
@@ -340,16 +365,24 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             bool ok = true;
             for (int n = 0; ok && n < 2 && n < units; ++n) ok = tiles(n);
             for (int n = 0; ok && n < units; ++n) {
-                // dQ_part += dS_unit K_unit (hi, then lo half of dS): 16 token rows of the K tile per k-step as the MN-major B operand
+                // dQ_part += dS_unit K_unit (the parts of dS in turn): 16 token rows of the K tile per k-step as the MN-major B operand
                 const uint32_t bcol = tm + (n & 1) * kDqBuf, acc = tm + kDqAcc + (n & (kAccs - 1)) * DG;
                 uint32_t kd = k0 + MN + (uint32_t)o_stage * 3 * TILE + (uint32_t)o_u * (UNIT / 16) * STEP16;
                 ptx::opaque(kd);
                 if (!ptx::mbar_wait(bar(P_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdDq | 4)) break;
                 ptx::tc_fence_after();
+                if constexpr (kThird) {                         // the small parts first: fewer sums are truncated at their full size
 #pragma unroll
-                for (int k = 0; k < UNIT / 16; ++k) {
-                    ptx::mma_ts(acc, bcol + 16 * k, ptx::desc(kd + k * STEP16, HI), idescQ, (n >= kAccs || k > 0) ? 1u : 0u);
-                    ptx::mma_ts(acc, bcol + UNIT + 16 * k, ptx::desc(kd + k * STEP16, HI), idescQ, 1u);
+                    for (int i = 2; i >= 0; --i)
+#pragma unroll
+                        for (int k = 0; k < UNIT / 16; ++k)
+                            ptx::mma_ts(acc, bcol + i * UNIT + 16 * k, ptx::desc(kd + k * STEP16, HI), idescQ, (i < 2 || k > 0) ? 1u : 0u);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < UNIT / 16; ++k) {
+                        ptx::mma_ts(acc, bcol + 16 * k, ptx::desc(kd + k * STEP16, HI), idescQ, (n >= kAccs || k > 0) ? 1u : 0u);
+                        ptx::mma_ts(acc, bcol + UNIT + 16 * k, ptx::desc(kd + k * STEP16, HI), idescQ, 1u);
+                    }
                 }
                 if (++o_u == UPT) {
                     ptx::mma_commit(bar(T_EMPTY + o_stage));
@@ -379,6 +412,15 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         const float2 nlep = make_float2(nle, nle), frp = make_float2(fr, fr), ndep = make_float2(nde, nde);
         bool ok = true;
         int n = 0;
+        float sum[kThird ? 16 : 1] = {};                        // (kThird) this warp's columns of the sums so far
+        // (kThird) the sums of unit i, complete when the tiles of unit i + 2 are
+        auto drain = [&](int i) {
+            uint32_t r[16];
+            ptx::tmem_ld16(gcol + kDqAcc + (i & 1) * DG + cg * 16, r);
+            ptx::tmem_wait_ld();
+#pragma unroll
+            for (int k = 0; k < 16; ++k) sum[kThird ? k : 0] += __uint_as_float(r[k]);
+        };
         for (int tile = 0; ok && tile < nt; ++tile) {
             const int c = tile % SM::kCst;
             const float *cst = reinterpret_cast<const float *>(smem + SM::cst_off + c * SM::kCstBytes) + second * 3 * kTile + cg * 16;
@@ -401,7 +443,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     for (int q = 0; q < 2; ++q) {                  // eight columns at a time, the other eight on their way meanwhile
                         ptx::tmem_wait_ld();
                         if (q == 0) load(1);
-                        uint32_t hi[4], lo[4];
+                        uint32_t hi[4], lo[4], lo2[4];
 #pragma unroll
                         for (int k = 0; k < 4; k += 2) {
                             const float4 nld = *reinterpret_cast<const float4 *>(cst + q * 8 + 2 * k);
@@ -410,7 +452,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
                                 const int j = 2 * (k + e);
-                                const DsPair r = ds_pair<false, kTwo>(
+                                const DsPair r = ds_pair<false, kTwo, kThird>(
                                     make_float2(__uint_as_float(s[q][j]), __uint_as_float(s[q][j + 1])),
                                     make_float2(__uint_as_float(av[q][j]), __uint_as_float(av[q][j + 1])),
                                     make_float2(__uint_as_float(cv[q][j]), __uint_as_float(cv[q][j + 1])), sl2p,
@@ -418,12 +460,15 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                                     ndep, kTwo ? nlep : frp, e ? make_float2(fc.z, fc.w) : make_float2(fc.x, fc.y));
                                 hi[k + e] = r.hi;
                                 lo[k + e] = r.lo;
+                                if (kThird) lo2[k + e] = r.lo2;
                             }
                         }
-                        // over columns this warp has read, 8 packed columns per 16 tokens: hi over S, lo over A
+                        // over columns this warp has read, 8 packed columns per 16 tokens: hi over S, lo over A, a third part over C
                         ptx::tmem_st4(bcol + q * 4, hi);
                         ptx::tmem_st4(bcol + UNIT + q * 4, lo);
+                        if (kThird) ptx::tmem_st4(bcol + 2 * UNIT + q * 4, lo2);
                     }
+                    if (kThird && n >= 2) drain(n - 2);
                     ptx::tmem_wait_st();
                     ptx::tc_fence_before();
                     __syncwarp();
@@ -434,7 +479,17 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             else units(std::true_type{});
             if (lane == 0) ptx::mbar_arrive(bar(C_EMPTY + c));
         }
-        if (cg == 0) {
+        if constexpr (kThird) {
+            if (ok) ok = warp_wait(bar(ACC_DONE), 0, abort_flag, kErrBwdDq | 6);
+            ptx::tc_fence_after();
+            for (int i = n > 2 ? n - 2 : 0; i < n; ++i) drain(i);
+            if (ok && m < M) {
+                const long rows = (long)a.B * a.H * M;
+                float4 *dst = reinterpret_cast<float4 *>(a.part + ((size_t)split * rows + ((size_t)b * a.H + h) * M + m) * D + cg * 16);
+#pragma unroll
+                for (int k = 0; k < 16; k += 4) dst[k / 4] = make_float4(sum[k], sum[k + 1], sum[k + 2], sum[k + 3]);
+            }
+        } else if (cg == 0) {
             if (ok) ok = warp_wait(bar(ACC_DONE), 0, abort_flag, kErrBwdDq | 6);
             ptx::tc_fence_after();
             float acc[D];
@@ -482,7 +537,8 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // core the others work, nothing is shared between them, and dd needs no exchange.  There is no issuing warp: the warps of a group
 // take turns issuing the output contractions of a unit, the tiles of the next and one commit, which says that all of them are done.
 // Measured, us, on the shapes named at the dQ kernel, against units of 16 columns, two exponentials per pair and half as many latents per
-// launch: 22.4, 164, 1166, 9254 -> 19.9, 132, 1016, 8936; D = 64: 1049 (CUDA cores) -> 67.  Units of 64 columns shared by sixteen warps, as
+// launch: 22.4, 164, 1166, 9254 -> 19.9, 132, 1016, 8936; D = 64: 1049 (CUDA cores) -> 67
+// (with the third part of Z 73).  Units of 64 columns shared by sixteen warps, as
 // in the dQ kernel: 39.6, 254, 1154, 16489; 71 (W_enc doubles what a thread holds: it spills).  Bound by issue slots, some 26
 // instructions per pair over both sweeps.
 // Groups of four warps, by accumulator columns: as many as 512 columns of tensor memory hold, at most four.  Warps: 0 TMA producer, from 2
@@ -518,11 +574,15 @@ struct BwdTokTcArgs {
 template <int D>
 struct BwdTokSmem {
     using G = TileGeom<D>;
-    // tiles: [stage][K | V | dY]; latents: Q, Z_hi, Z_lo, dZ_hi, dZ_lo with M rows each (M a multiple of 16); their constants
+    // D = 64: dd[n] is subtracted from products that the dQ kernel forms of three parts of Z, so the first sweep takes three as well (with two,
+    // dQ on features of point clouds was 4.7e-6 to 5.4e-6 of its norm from float64 instead of 2.6e-6 to 3.0e-6), as long as the third fits
+    // beside two tile stages.
+    static constexpr int kThirdMost = D == 64 ? 160 : 0;
+    // tiles: [stage][K | V | dY]; latents: Q, Z_hi, Z_lo, dZ_hi, dZ_lo (and a third part of Z) with M rows each (M a multiple of 16); their constants
     __host__ __device__ static size_t lat_off(int stages, int M, int which) {
         return (size_t)stages * 3 * G::TILE_BYTES + (size_t)which * M * G::RB;
     }
-    __host__ __device__ static size_t cst_off(int stages, int M) { return lat_off(stages, M, 5); }
+    __host__ __device__ static size_t cst_off(int stages, int M) { return lat_off(stages, M, M <= kThirdMost ? 6 : 5); }
     __host__ __device__ static size_t bar_off(int stages, int M) { return cst_off(stages, M) + 3 * sizeof(float) * M; }
     __host__ __device__ static size_t total(int stages, int M) {
         const size_t t = bar_off(stages, M) + 512 + 1024;
@@ -567,6 +627,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
     const int nu = (M + UNIT - 1) / UNIT;                       // latent units per sweep; the last may have 16 columns
     const int off = DRT ? narrow_offset(h, DR) : 0;
+    const bool third = D == 64 && kMode != 2 && M <= SM::kThirdMost;
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
 
     if (threadIdx.x == 0) {
@@ -599,7 +660,8 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             stage_rows4_hilo<D>(lat[3], lat[4], a.dZ + r0 * DR, M, off);
         } else {
             stage_bf16<D, DR>(lat[0], a.Q + q0 * DR, M, 0, 0, threadIdx.x, kThreads);
-            stage_hilo<D, DR>(lat[1], lat[2], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads);
+            if (third) stage_hilo<D, DR, true>(lat[1], lat[2], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, smem + SM::lat_off(stages, M, 5));
+            else stage_hilo<D, DR>(lat[1], lat[2], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads);
             stage_hilo<D, DR>(lat[3], lat[4], a.dZ + r0 * DR, M, 0, 0, threadIdx.x, kThreads);
         }
         __syncthreads();
@@ -652,13 +714,23 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             const uint32_t idescS = ptx::instr_desc_bf16(128, u == nu - 1 ? wlast : UNIT, 0, 0);
             uint32_t td = ptx::desc_lo(ptx::smem_u32(smem), 16) + (uint32_t)stage * 3 * TILE, ld = lat_desc(u);
             ptx::opaque(td);
+            auto product = [&](int of, uint32_t lat, bool more) {   // of: S, A or C
+                const uint32_t col = base + of * UNIT, ad = td + (of == 0 ? 0 : of == 1 ? 2 * TILE : TILE);
 #pragma unroll
-            for (int w = 0; w < (kSecond ? 5 : 3); ++w) {       // K with Q; dY with Z hi, lo; V with dZ hi, lo
-                const uint32_t col = base + (w == 0 ? 0 : w <= 2 ? UNIT : 2 * UNIT), ad = td + (w == 0 ? 0 : w <= 2 ? 2 * TILE : TILE);
-#pragma unroll
-                for (int k = 0; k < D / 16; ++k)
-                    ptx::mma_ss(col, ptx::desc(ad + 2 * k, HI), ptx::desc(ld + 2 * k, HI), idescS, k > 0 || w == 2 || w == 4);
-                ld += LAT;
+                for (int k = 0; k < D / 16; ++k) ptx::mma_ss(col, ptx::desc(ad + 2 * k, HI), ptx::desc(lat + 2 * k, HI), idescS, k > 0 || more);
+            };
+            product(0, ld, false);                              // K with Q; dY with the parts of Z; V with dZ hi, lo
+            if (D == 64 && !kSecond) {
+                if (third) product(1, ld + 5 * LAT, false);     // (small parts first: fewer sums are truncated at their full size)
+                product(1, ld + 2 * LAT, third);
+                product(1, ld + LAT, true);
+            } else {
+                product(1, ld + LAT, false);
+                product(1, ld + 2 * LAT, true);
+            }
+            if (kSecond) {
+                product(2, ld + 3 * LAT, false);
+                product(2, ld + 4 * LAT, true);
             }
         };
         // by one thread: dK += dS Q_unit, dV += W_enc dZ_unit
@@ -779,7 +851,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
                                 const int j = 2 * (k + e);
-                                const DsPair r = ds_pair<true, kTwo>(
+                                const DsPair r = ds_pair<true, kTwo, false>(
                                     make_float2(__uint_as_float(s[j]), __uint_as_float(s[j + 1])), make_float2(__uint_as_float(av[j]), __uint_as_float(av[j + 1])),
                                     make_float2(__uint_as_float(cv[j]), __uint_as_float(cv[j + 1])), sl2p, nldp, nddp,
                                     e ? make_float2(nd.z, nd.w) : make_float2(nd.x, nd.y), e ? make_float2(le.z, le.w) : make_float2(le.x, le.y), fctp);
