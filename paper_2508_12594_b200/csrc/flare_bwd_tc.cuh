@@ -608,8 +608,6 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     using SM = BwdTokSmem<D>;
     using BG = BwdGroups<2 * D>;
     constexpr int UNIT = kUnit, NG = BG::n, kThreads = BG::kThreads, kMaxSt = SM::kMaxStages, DR = DRT ? DRT : D;
-    // dV = W_hi (dZ_hi + dZ_lo) + W_lo dZ_hi: with room for 2 D columns W_hi meets [dZ_hi | dZ_lo] in one MMA
-    constexpr bool kWideV = kUnitCols + 3 * D <= BG::cols;
     constexpr int K_COL = kUnitCols, V_COL = K_COL + D;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -735,18 +733,16 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         };
         // by one thread: dK += dS Q_unit, dV += W_enc dZ_unit
         auto issue_outputs = [&](int u) {
-            constexpr uint32_t idescO = ptx::instr_desc_bf16(128, D, 0, 1), idescW = ptx::instr_desc_bf16(128, kWideV ? 2 * D : D, 0, 1);
-            const uint32_t ld = lat_desc(u);
-            // (wide form: dZ_hi's next block along N is dZ_lo, M rows further on)
-            const uint32_t qd = ld + MN, zd = ld + 3 * LAT + (kWideV ? (LAT << 16) - ptx::desc_lo(0, 16) : MN), zl = ld + 4 * LAT + MN;
+            constexpr uint32_t idescO = ptx::instr_desc_bf16(128, D, 0, 1);
+            const uint32_t ld = lat_desc(u), qd = ld + MN, zd = ld + 3 * LAT + MN, zl = ld + 4 * LAT + MN;
 #pragma unroll
             for (int k = 0; k < UNIT / 16; ++k) {
                 if (k > 0 && u == nu - 1 && 16 * k >= wlast) break;
                 const uint32_t acc = (u > 0 || k > 0) ? 1u : 0u;
                 ptx::mma_ts(base + K_COL, base + 16 * k, ptx::desc(qd + k * STEP16, HI), idescO, acc);                    // dS hi
                 ptx::mma_ts(base + K_COL, base + UNIT + 16 * k, ptx::desc(qd + k * STEP16, HI), idescO, 1u);              // dS lo
-                ptx::mma_ts(base + V_COL, base + 2 * UNIT + 16 * k, ptx::desc(zd + k * STEP16, HI), idescW, acc);         // W_enc hi x dZ hi (and lo)
-                if (!kWideV) ptx::mma_ts(base + V_COL, base + 2 * UNIT + 16 * k, ptx::desc(zl + k * STEP16, HI), idescO, 1u);
+                ptx::mma_ts(base + V_COL, base + 2 * UNIT + 16 * k, ptx::desc(zd + k * STEP16, HI), idescO, acc);         // W_enc hi x dZ hi
+                ptx::mma_ts(base + V_COL, base + 2 * UNIT + 16 * k, ptx::desc(zl + k * STEP16, HI), idescO, 1u);          // W_enc hi x dZ lo
                 ptx::mma_ts(base + V_COL, base + 16 * k + 8, ptx::desc(zd + k * STEP16, HI), idescO, 1u);                 // W_enc lo x dZ hi
             }
         };
@@ -775,18 +771,13 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             const float sc = which ? 1.f : a.scale;
 #pragma unroll
             for (int c0 = 0; c0 < LW; c0 += 8) {
-                uint32_t x[8], y[8];
+                uint32_t x[8];
                 ptx::tmem_ld8(col + c0, x);
-                if (kWideV && which) ptx::tmem_ld8(col + D + c0, y);
                 ptx::tmem_wait_ld();
                 constexpr int PW = DR == 4 ? 4 : 8;             // columns written
                 float f[PW];
 #pragma unroll
-                for (int c = 0; c < PW; ++c) {                  // the head's columns
-                    const bool up = DR == 4 && off != 0;
-                    f[c] = __uint_as_float(up ? x[(4 + c) & 7] : x[c]);
-                    if (kWideV && which) f[c] += __uint_as_float(up ? y[(4 + c) & 7] : y[c]);
-                }
+                for (int c = 0; c < PW; ++c) f[c] = __uint_as_float(DR == 4 && off != 0 ? x[(4 + c) & 7] : x[c]);   // the head's columns
                 if (tok_n < a.N) {
                     if (kMode == 2) {
 #pragma unroll
