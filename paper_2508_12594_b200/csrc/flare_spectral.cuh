@@ -6,8 +6,7 @@
 //     J[m,n] = exp(S[m,n] - lse_enc[m] / 2 - lse_dec[n] / 2),        G[m,m'] = sum_n J[m,n] J[m',n],
 // so G is one more reduction over the tokens in which every (latent, token) pair costs one exponential (as in
 // encode) and every pair of latents one multiply-add per token: 2 N M^2 FLOP per head, O(M^2) memory.  Nothing
-// of size M x N or N x N is written.  The M x M symmetric eigenproblem (O(M^3), off the hot path) is solved by a
-// small Jacobi kernel.
+// of size M x N or N x N is written.  The M x M symmetric eigenproblem is O(M^3), off the hot path.
 //
 //   spectral_gram_tc_kernel    bfloat16, M <= 128, D in {16, 32}: tcgen05.  A CTA takes one head and a range of
 //                              tokens; the head's latents sit on the 128 TMEM lanes.  Per 32 tokens: S = Q K^T; 128
@@ -311,7 +310,8 @@ spectral_gram_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, cons
 }
 
 // A matrix that holds a NaN or an infinity has no eigenvalues: every output for it is NaN.  (Maxima, comparisons and rotations
-// drop a NaN: without this test a matrix of NaN came out with eigenvalues 0, as if of rank 0.)  One more pass over G, beside M.
+// drop a NaN: without this test a matrix of NaN came out with eigenvalues 0, as if of rank 0.)  One pass over G, where the
+// solvers take M and more.
 constexpr float kEigNan = __builtin_nanf("");
 // All threads of the block call it.
 __device__ __forceinline__ bool eig_broken(const float *G, int M) {
@@ -320,25 +320,22 @@ __device__ __forceinline__ bool eig_broken(const float *G, int M) {
     return __syncthreads_or(bad);
 }
 
-// Eigenvalues (descending) and, if U != null, eigenvectors (columns of U) of the symmetric matrices G [heads, M, M],
-// by cyclic two-sided Jacobi rotations on disjoint index pairs (round-robin ordering: M - 1 steps of M / 2 rotations
-// per sweep).  One block per matrix; G is overwritten.  Off the hot path: O(M^3) per sweep, about ten sweeps.
+// Eigenvalues (descending) and eigenvectors (columns of U) of the symmetric matrices G [heads, M, M], by cyclic two-sided Jacobi
+// rotations on disjoint index pairs (round-robin ordering: M - 1 steps of M / 2 rotations per sweep).  One block per matrix; G is overwritten.  Off the hot path: O(M^3) per sweep, about ten sweeps.
 static __global__ void __launch_bounds__(1024)
 spectral_jacobi_kernel(float *__restrict__ Gall, float *__restrict__ evals, float *__restrict__ Uall, int M, int sweeps) {
     extern __shared__ float sh[];
     float *cs = sh;                         // [M/2 pairs] cosines, then sines
     int *pp = reinterpret_cast<int *>(sh + 2 * ((M + 1) / 2));   // [pairs] p, then q; then [M] ranks
     float *G = Gall + (size_t)blockIdx.x * M * M;
-    float *U = Uall ? Uall + (size_t)blockIdx.x * M * M : nullptr;
+    float *U = Uall + (size_t)blockIdx.x * M * M;
     const int Me = (M + 1) & ~1, pairs = Me / 2, t = threadIdx.x, T = blockDim.x;
     if (eig_broken(G, M)) {
         for (int i = t; i < M; i += T) evals[(size_t)blockIdx.x * M + i] = kEigNan;
-        if (U)
-            for (int i = t; i < M * M; i += T) U[i] = kEigNan;
+        for (int i = t; i < M * M; i += T) U[i] = kEigNan;
         return;
     }
-    if (U)
-        for (int i = t; i < M * M; i += T) U[i] = (i / M == i % M) ? 1.f : 0.f;
+    for (int i = t; i < M * M; i += T) U[i] = (i / M == i % M) ? 1.f : 0.f;
     __syncthreads();
     // A sweep that met no off-diagonal element above 2^-22 of the largest diagonal one (float32 rotations change nothing
     // below that) was the last: six to eight sweeps in practice instead of the twelve allowed.
@@ -367,7 +364,7 @@ spectral_jacobi_kernel(float *__restrict__ Gall, float *__restrict__ evals, floa
                 cs[k] = c; cs[pairs + k] = s; pp[k] = p; pp[pairs + k] = q;
             }
             __syncthreads();
-            // columns: G <- G R (and U <- U R), every row independently.  Neighbouring threads take the pairs of one row:
+            // columns: G <- G R and U <- U R, every row independently.  Neighbouring threads take the pairs of one row:
             // a step's pairs cover every column once, so the row's sectors are all used while they are in the cache
             // (pair-major order touched one element per sector and was 3 times slower at M = 512).
             for (int i = t; i < pairs * M; i += T) {
@@ -377,11 +374,9 @@ spectral_jacobi_kernel(float *__restrict__ Gall, float *__restrict__ evals, floa
                 const float gp = G[(size_t)row * M + p], gq = G[(size_t)row * M + q];
                 G[(size_t)row * M + p] = c * gp - s * gq;
                 G[(size_t)row * M + q] = s * gp + c * gq;
-                if (U) {
-                    const float up = U[(size_t)row * M + p], uq = U[(size_t)row * M + q];
-                    U[(size_t)row * M + p] = c * up - s * uq;
-                    U[(size_t)row * M + q] = s * up + c * uq;
-                }
+                const float up = U[(size_t)row * M + p], uq = U[(size_t)row * M + q];
+                U[(size_t)row * M + p] = c * up - s * uq;
+                U[(size_t)row * M + q] = s * up + c * uq;
             }
             __syncthreads();
             // rows: G <- R^T G, every column independently
@@ -412,11 +407,9 @@ spectral_jacobi_kernel(float *__restrict__ Gall, float *__restrict__ evals, floa
         ev[r] = v;
     }
     __syncthreads();
-    if (U) {
-        for (int i = t; i < M * M; i += T) G[(size_t)(i / M) * M + rank[i % M]] = U[i];
-        __syncthreads();
-        for (int i = t; i < M * M; i += T) U[i] = G[i];
-    }
+    for (int i = t; i < M * M; i += T) G[(size_t)(i / M) * M + rank[i % M]] = U[i];
+    __syncthreads();
+    for (int i = t; i < M * M; i += T) U[i] = G[i];
 }
 
 // Eigenvalues alone (no U): Householder reduction to tridiagonal form, then bisection on Sturm counts.  One block per
