@@ -108,7 +108,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
     int dz_parts = pa.P;
     bool dz_on_tc = skip_pass_a;
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-        if (!skip_pass_a && bwd_dz_on_tensor_cores(d)) {
+        if (!skip_pass_a && use_tc(d)) {
             const LeanPlan tp = dz_plan(d, sms);
             uint32_t *status = reinterpret_cast<uint32_t *>(ws);
             const int rc = encode_dz_tc(d, tp, Q, K, dY, part, status, st, lse_dec);
@@ -129,7 +129,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
         constexpr int DK = D < 16 ? 16 : D;                     // width the kernels multiply (D < 16: narrow forms)
         constexpr int DRT = D < 16 ? D : 0;
         uint32_t *status = reinterpret_cast<uint32_t *>(ws);
-        on_tc = bwd_dq_on_tensor_cores(d);
+        on_tc = use_tc(d);
         if (on_tc) {
             // more latents than one launch holds: two series of launches over ranges of them, dd[n] first, then the rows of dK and dV
             float *kvacc = reinterpret_cast<float *>(ws + w.kvacc);

@@ -311,9 +311,7 @@ constexpr float kLog2e = 1.4426950408889634f;
 // outside the range it is valid for; the exact form that follows runs only then.
 constexpr int kRedoEncodeWord = 2, kRedoDecodeWord = 3;
 
-// Decode over more latents than one launch holds in tensor memory (512 columns) is cut into ranges of latents; their
-// partial results take float32 rows [C][B*N*H][D] and log-sum-exps [C][B*N*H] behind the encode layout of the workspace.
-// One decode launch holds all M score columns of a token tile: up to kDecodeMaxM latents.
+// One decode launch holds all M score columns of a token tile in tensor memory: up to kDecodeMaxM latents.
 constexpr int kDecodeMaxM = 512;
 
 // Ranges of latents a decode over more than kDecodeMaxM latents is cut into, and the scratch their partial results
@@ -327,13 +325,9 @@ inline size_t decode_range_bytes(const flare_desc_t *d) {
     return align_up(sizeof(float) * decode_ranges(d) * rows * d->D) + align_up(sizeof(float) * decode_ranges(d) * rows);
 }
 
-// Launch plans of the CUDA-core backward: pass A (dZ) reuses the encode plan; the dQ pass keeps three operands of a latent row
-// in registers and therefore takes fewer rows per warp.
-// Pass A (dZ) runs as a form of the tensor-core encode without a running maximum wherever the tensor-core kernels run.
-inline bool bwd_dz_on_tensor_cores(const flare_desc_t *d) { return use_tc(d); }
-
-// Pass B (dQ; dK and dV) runs on the tensor cores for the same shapes.
-inline bool bwd_dq_on_tensor_cores(const flare_desc_t *d) { return use_tc(d); }
+// Plans of the backward, whose passes run on the tensor cores for the same shapes as the forward (use_tc): dz_plan for pass A, a form of
+// the encode without a running maximum; tc_dq_plan for dQ.  On the CUDA cores pass A has the encode's plan, and the dQ pass, which keeps
+// three operands of a latent row in registers, one with fewer rows per warp.
 
 // Plan of the tensor-core dQ kernel: `pairs` = blocks of 128 latents per head, one partial sum per CTA.
 inline TcEncodePlan tc_dq_plan(const flare_desc_t *d, int sms) {
@@ -354,10 +348,10 @@ struct BwdLayout {
     int P;
 };
 
-// Latents one launch of the tensor-core token kernel takes: five operands of D-wide bf16 rows beside a tile stage per group (four groups at
+// Latents one launch of the tensor-core token kernel takes: five operands of D-wide bf16 rows (six at D = 64 up to 160 latents) beside a tile stage per group (four groups at
 // D <= 16, three at 32, two at 64); more are worked off in ranges of equal size.
 inline int token_range_most(const flare_desc_t *d) { return d->D == 64 ? 192 : d->D == 32 ? 448 : 1024; }
-inline bool token_in_ranges(const flare_desc_t *d) { return bwd_dq_on_tensor_cores(d) && d->M > token_range_most(d); }
+inline bool token_in_ranges(const flare_desc_t *d) { return use_tc(d) && d->M > token_range_most(d); }
 inline int token_ranges(const flare_desc_t *d) { return (d->M + token_range_most(d) - 1) / token_range_most(d); }
 inline int token_range(const flare_desc_t *d) { return ((d->M + token_ranges(d) - 1) / token_ranges(d) + 15) / 16 * 16; }
 
@@ -366,8 +360,7 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     const long rows = (long)d->B * d->H * d->M;
     const int pa = simt_plan(d, sms).P, pb = bwd_dq_plan(d, sms).P;
     w.P = pa > pb ? pa : pb;
-    if (bwd_dz_on_tensor_cores(d) && dz_plan(d, sms).splits > w.P) w.P = dz_plan(d, sms).splits;
-    if (bwd_dq_on_tensor_cores(d) && tc_dq_plan(d, sms).P > w.P) w.P = tc_dq_plan(d, sms).P;
+    if (use_tc(d)) w.P = std::max(w.P, std::max(dz_plan(d, sms).splits, tc_dq_plan(d, sms).P));
     size_t off = kHeaderBytes;
     w.part = off; off += align_up(sizeof(float) * (size_t)w.P * rows * d->D);
     w.dz = off;   off += align_up(sizeof(float) * (size_t)rows * d->D);
@@ -409,6 +402,5 @@ size_t spectral_bytes(const flare_desc_t *d, int sms);
 int spectral_gram(const flare_desc_t *d, int sms, const void *Q, const void *K, const float *lse_enc, const float *lse_dec, float *G,
                   void *workspace, cudaStream_t st);
 int spectral_eig(int32_t matrices, int32_t M, float *G, float *eigenvalues, float *U, int32_t sweeps, cudaStream_t st);
-
 
 }  // namespace flare

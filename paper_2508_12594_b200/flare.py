@@ -165,7 +165,6 @@ def flare_encode(desc, Q, K, V, key_mask, Z, lse_enc, workspace, stream=None):
     (_native or _bind()).encode(desc, Q, K, V, key_mask, Z, lse_enc, workspace, stream)
 
 
-
 STATIC_SCRATCH_BYTES = 8 << 20
 
 
@@ -176,10 +175,8 @@ def flare_encode_static_scratch(desc, Q, K, V, key_mask, Z, lse_enc, stream=None
     (_native or _bind()).encode_static_scratch(desc, Q, K, V, key_mask, Z, lse_enc, stream)
 
 
-
 def flare_decode(desc, Q, K, Z, Y, lse_dec, workspace=None, stream=None):
     (_native or _bind()).decode(desc, Q, K, Z, Y, lse_dec, workspace, stream)
-
 
 
 PATH_AUTO, PATH_EXACT, PATH_FAST = 0, 1, 2
@@ -194,16 +191,13 @@ def flare_forward(desc, Q, K, V, key_mask, Y, Z, lse_enc, lse_dec, workspace, st
     (_native or _bind()).forward(desc, Q, K, V, key_mask, Y, Z, lse_enc, lse_dec, workspace, stream)
 
 
-
 def flare_backward(desc, Q, K, V, key_mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, workspace, stream=None):
     (_native or _bind()).backward(desc, Q, K, V, key_mask, Y, dY, Z, lse_enc, lse_dec, dQ, dK, dV, workspace, stream)
-
 
 
 def flare_forward_host(desc, hQ, hK, hV, hmask, hY, dQ, dK, dV, dmask, dY, workspace, stream=None):
     """Host tensors in, host tensor out; the device tensors are the caller's staging buffers."""
     (_native or _bind()).forward_host(desc, hQ, hK, hV, hmask, hY, dQ, dK, dV, dmask, dY, workspace, stream)
-
 
 
 def flare_check(workspace, stream=None):
@@ -228,12 +222,10 @@ def flare_forward_variant(desc, shared_latents, Q_enc, Q_dec, K, V, key_mask, Y,
     (_native or _bind()).forward_variant(desc, shared_latents, Q_enc, Q_dec, K, V, key_mask, Y, Z, lse_enc, lse_dec, workspace, stream)
 
 
-
 def flare_backward_variant(desc, shared_latents, Q_enc, Q_dec, K, V, key_mask, Y, dY, Z, lse_enc, lse_dec, dQ_enc, dQ_dec, dK,
                            dV, workspace, stream=None):
     (_native or _bind()).backward_variant(desc, shared_latents, Q_enc, Q_dec, K, V, key_mask, Y, dY, Z, lse_enc, lse_dec, dQ_enc,
                                           dQ_dec, dK, dV, workspace, stream)
-
 
 
 def flare_microbench(which: int, iters: int = 20000, stream=None) -> float:
@@ -249,17 +241,14 @@ def flare_spectral_gram(desc, Q, K, lse_enc, lse_dec, G, workspace, stream=None)
     (_native or _bind()).spectral_gram(desc, Q, K, lse_enc, lse_dec, G, workspace, stream)
 
 
-
 def flare_spectral_eig(G, eigenvalues, U=None, sweeps=0, stream=None):
     """G [..., M, M] float32 (destroyed) -> eigenvalues [..., M] descending, U [..., M, M] eigenvectors as columns."""
     (_native or _bind()).spectral_eig(G, eigenvalues, U, int(sweeps), stream)
 
 
-
 def forward(Q, K, V, key_mask=None, scale=1.0, want_stats=False, stream=None):
     """Convenience: allocate outputs and workspace with torch, call flare_forward, return Y (and Z, lse's)."""
     return (_native or _bind()).call_forward(Q, K, V, key_mask, scale, want_stats, stream)
-
 
 
 def forward_backward(Q, K, V, dY, key_mask=None, scale=1.0, stream=None, check=False):
