@@ -20,10 +20,10 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 
 // Index of this thread's warp in the block, in a form the compiler knows to be the same for the whole warp.
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
-// True in one lane of a converged warp.  The thread that issues tensor-core instructions must be chosen this way (and its
-// role by warp_index): their operands live in warp-uniform registers, and behind a test of the lane number every
-// one of them is moved there through a loop over the active lanes.  Measured, one issuing thread: 113 cycles per
-// tcgen05.mma with `lane == 0`, 18 (A in tensor memory, N = 16), 26 (N = 32) and 51 to 58 (A in shared memory) with this.
+// True in one lane of a converged warp.  The thread that issues tensor-core instructions is chosen this way, and its role by
+// warp_index, because it measured faster: one issuing thread is held 113 cycles per tcgen05.mma behind `lane == 0`, 18 (A in
+// tensor memory, N = 16), 26 (N = 32) and 51 to 58 (A in shared memory) behind this.  The likely reason is that the compiler
+// can tell that one lane issues for a whole warp.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));

@@ -9,8 +9,8 @@
 //
 // Two resources limit both kernels, and neither is the one a roofline of FLOPs and bytes names.  Every
 // (latent, token) pair needs one exponential on the special-function unit (16 per clock per SM), and every tcgen05.mma of this
-// shape (M = 128, K = 16) takes its issuing thread 18 to 58 cycles (113 where the compiler does not know that one lane of a uniform
-// warp issues it) and the tensor core 40 cycles or more with both operands in shared memory, N / 2 with one in tensor memory.
+// shape (M = 128, K = 16) takes its issuing thread 18 to 58 cycles (113 where a test of the lane number chooses it, see
+// elect_one) and the tensor core 40 cycles or more with both operands in shared memory, N / 2 with one in tensor memory.
 // The CTA is therefore four pipelines side by side: warp 0 issues TMA loads; sixteen softmax warps (four per
 // scheduler) form four groups of four warps, and each group has an issuing warp of its own (warps 1-4; warp 1
 // also owns the TMEM allocation).  A group owns one TMEM score buffer, or a range of columns of a shared one,
