@@ -156,8 +156,11 @@ inline bool use_fast_encode(const flare_desc_t *d) {
     return d->D <= 32 && fast_wanted(d, work >= (lean_pairs(d) && d->D != 16 ? 3.0e4 : 6.0e4));
 }
 // Decode: the streaming form has no variant for head width 64.  Measured against the exact form, us, at B H N = 524288 (131072): D = 16, M = 48
-// 20 : 29 (11.2 : 10.4), 64 31 : 35 (10.4 : 8.3), 96 26 : 36 (14.4 : 15.8), 144 27 : 33 (15 : 20); the exact form keeps what one chunk
-// of its registers holds (M = 32: 18 : 13) and, at D = 32, 64 latents (48 : 41) and small calls up to there (M = 48: 29 : 35 from 262144 on).
+// 20 : 29 (11.2 : 10.4), 64 31 : 35 (10.4 : 8.3), 96 26 : 36 (14.4 : 15.8), 144 27 : 33 (15 : 20); the exact form keeps what fills one chunk
+// of its registers (M = 32: 18 : 13) and, at D = 32, 64 latents (48 : 41) and small calls up to there (M = 48: 29 : 35 from 262144 on).
+// 16 latents leave half of a chunk, or of a unit, empty in either form, and the exact form, which has no form of its own for them, is slower
+// than at 32: 262144 / 524288 / 2097152 rows, D = 8 18.4 : 18.4 / 22.5 : 26.7 / 43 : 68, D = 16 18.5 : 20.5 / 24.6 : 30.7 / 53 : 78, D = 32
+// 24.6 : 22.5 / 32.8 : 34.8 / 90 : 96.
 inline bool use_fast_decode(const flare_desc_t *d) {
     const double rows = (double)d->B * d->H * d->N;
     bool pays;
