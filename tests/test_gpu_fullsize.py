@@ -119,3 +119,34 @@ def test_backward_full_size_sampled(oracle, w):
     idx = torch.from_numpy(rows).cuda()
     got = dict(dQ=to_np64(dQ), dK=to_np64(dK.view(w.B * w.N, w.H, w.D)[idx]), dV=to_np64(dV.view(w.B * w.N, w.H, w.D)[idx]))
     assert_grads_close(got, dict(dQ=ref["dQ"], dK=ref["dK_rows"], dV=ref["dV_rows"]), w.dtype, f"{w.name} (sampled rows)")
+
+
+def _float64_z_and_dq(Q, K, V, dY):
+    """Z and dQ of one head in float64 by plain torch, on the device (the oracle would take minutes here), a slice of tokens at a time."""
+    Q, step = Q.double(), 1 << 17
+    S = lambda a: Q @ K[a:a + step].double().T
+    at = range(0, K.shape[0], step)
+    le = torch.logsumexp(torch.stack([torch.logsumexp(S(a), 1) for a in at]), 0)
+    Z = sum(torch.exp(S(a) - le[:, None]) @ V[a:a + step].double() for a in at)
+    dZ = sum(torch.softmax(S(a), 0) @ dY[a:a + step].double() for a in at)
+    de, dQ = (dZ * Z).sum(1, keepdim=True), torch.zeros_like(Q)
+    for a in at:
+        k, v, g = (x[a:a + step].double() for x in (K, V, dY))
+        s = S(a)
+        Wd, A = torch.softmax(s, 0), Z @ g.T
+        dQ += (Wd * (A - (Wd * A).sum(0, keepdim=True)) + torch.exp(s - le[:, None]) * (dZ @ v.T - de)) @ k
+    return Z, dQ
+
+
+def test_sums_over_a_million_tokens():
+    """The tensor core truncates every float32 sum, so the number of sums in a row bounds how far Z and dQ drift at a million tokens:
+    with at most 512 tiles to a split, five groups of warps and two halves of 8 steps to a tile, 1640 truncations of less than 2^-23 of a
+    sum that is half its size on average: 1e-4 of Z.  dQ: eight accumulators of 1024 truncations, 6e-5, beside what Z and dZ carry."""
+    inp = workloads.make_inputs(workloads.CONFIGS["field_1m"])
+    Q, K, V, dY = dev(inp.Q), dev(inp.K), dev(inp.V), dev(inp.dY)
+    _, dQ, _, _ = flare.forward_backward(Q, K, V, dY, check=True)
+    _, Z, _, _ = flare.forward(Q, K, V, want_stats=True)
+    for h in (0, 5):
+        Z_ref, dQ_ref = _float64_z_and_dq(Q[h], K[0, :, h], V[0, :, h], dY[0, :, h])
+        assert (Z[0, h] - Z_ref).norm() <= 1e-4 * Z_ref.norm()
+        assert (dQ[h] - dQ_ref).norm() <= 2.6e-4 * dQ_ref.norm()
