@@ -310,8 +310,7 @@ spectral_gram_simt_kernel(const T *__restrict__ Q, const T *__restrict__ K, cons
 }
 
 // A matrix that holds a NaN or an infinity has no eigenvalues: every output for it is NaN.  (Maxima, comparisons and rotations
-// drop a NaN: without this test a matrix of NaN came out with eigenvalues 0, as if of rank 0.)  One pass over G, where the
-// solvers take M and more.
+// drop a NaN: left to them, a matrix of NaN comes out with eigenvalues 0, as if of rank 0.)
 constexpr float kEigNan = __builtin_nanf("");
 // All threads of the block call it.
 __device__ __forceinline__ bool eig_broken(const float *G, int M) {
@@ -487,7 +486,7 @@ spectral_bisect_kernel(const float *__restrict__ tri, float *__restrict__ evals,
     const float *d = tri + (size_t)blockIdx.y * M * M, *e = d + M;
     const int t = threadIdx.x, lane = t & 31;
     double top = 0.0;                                           // Gershgorin, by every warp for itself
-    bool bad = false;                                           // (see eig_broken: the tridiagonal form of such a matrix)
+    bool bad = false;                                           // (the tridiagonal form of a matrix that was not finite)
     for (int i = lane; i < M; i += 32) {
         const double ei = i + 1 < M ? e[i] : 0.f, eb = i > 0 ? e[i - 1] : 0.f;
         bad |= !isfinite(d[i]) || !isfinite(ei);
@@ -533,22 +532,25 @@ spectral_bisect_kernel(const float *__restrict__ tri, float *__restrict__ evals,
     if (r < M && sub == 0) evals[(size_t)blockIdx.y * M + r] = top > 0.0 ? (float)(0.5 * (lo + hi) / scale) : 0.f;
 }
 
-// Largest magnitude over the block as a power of two to scale by, so that squares of the entries neither overflow nor
-// vanish: returns 2^-e with e the exponent of the largest, as near to it as 2^-e is a normal number (1 for a zero matrix; the
-// entries are finite).  All threads call it.
-__device__ __forceinline__ float eig_block_scale(float mx, float *sh32) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+// Largest magnitude over the block as a power of two to scale by, so that squares of the entries neither overflow nor vanish: returns
+// 2^-e with e the exponent of the largest, as near to it as 2^-e is a normal number (1 for a zero matrix).  NaN if an entry is not
+// finite: what is scaled by it is NaN throughout, and so are the eigenvalues.  mx: the largest |entry| of this thread, as its bits (which order
+// like the magnitudes, infinity and NaN on top).  All threads call it.  (A test of the entries with a return of its own took the kernel
+// below from 67 registers a thread to 98 and from 184 to 227 us at M = 128.)
+__device__ __forceinline__ float eig_block_scale(unsigned mx, unsigned *sh32) {
+    mx = __reduce_max_sync(0xffffffffu, mx);
     if ((threadIdx.x & 31) == 0) sh32[threadIdx.x >> 5] = mx;
     __syncthreads();
-    mx = 0.f;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) mx = fmaxf(mx, sh32[i]);
+    mx = 0u;
+    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) mx = max(mx, sh32[i]);
     __syncthreads();
+    if (mx == 0u) return 1.f;
+    if (mx >= 0x7f800000u) return kEigNan;
     int e = 0;
-    if (!(mx > 0.f)) return 1.f;
-    frexpf(mx, &e);
+    frexpf(__uint_as_float(mx), &e);
     return ldexpf(1.f, e > 126 ? -126 : e < -126 ? 126 : -e);
 }
+__device__ __forceinline__ unsigned eig_magnitude(float x) { return __float_as_uint(fabsf(x)); }
 
 // The matrix in registers: NG groups of CX threads, thread (g, j) holds rows g, g + NG, ... of column j.  Vectors that are
 // read by rows are stored group-major (row g + NG r at g * R + r), so that four rows come with one load.
@@ -560,21 +562,17 @@ __global__ void __launch_bounds__(EigReg<CX>::kThreads)
 spectral_tridiag_reg_kernel(float *__restrict__ Gall, int M) {
     constexpr int NG = EigReg<CX>::NG, R = EigReg<CX>::R, CW = CX / 32, TH = EigReg<CX>::kThreads;
     __shared__ __align__(16) float sx[NG * R], sv[NG * R], sw[NG * R];   // column k as it is, v, w
-    __shared__ float part[NG][CX], diag[CX], off[CX], red[32];
+    __shared__ float part[NG][CX], diag[CX], off[CX];
+    __shared__ unsigned red[32];
     const int t = threadIdx.x, lane = t & 31, j = t % CX, g = t / CX;
     float *G = Gall + (size_t)blockIdx.x * M * M;
-    float A[R], mx = 0.f;
-    bool bad = false;
+    float A[R];
+    unsigned mx = 0u;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = g + NG * r;
         A[r] = (j < M && i < M) ? G[(size_t)i * M + j] : 0.f;
-        mx = fmaxf(mx, fabsf(A[r]));
-        bad |= !isfinite(A[r]);
-    }
-    if (__syncthreads_or(bad)) {                                // (see eig_broken)
-        if (t == 0) G[0] = kEigNan;
-        return;
+        mx = max(mx, eig_magnitude(A[r]));
     }
     const float scale = eig_block_scale(mx, red);
 #pragma unroll
@@ -682,13 +680,9 @@ spectral_tridiag_kernel(float *__restrict__ Gall, int M) {
     float *dg = eig_sh, *ee = dg + M, *v = ee + M, *w = v + M, *part = w + M;   // part [NG][M]
     float *G = Gall + (size_t)blockIdx.x * M * M;
     float *A = kShared ? part + (size_t)NG * M : G;
-    __shared__ float red[32];
-    if (eig_broken(G, M)) {
-        if (t == 0) G[0] = kEigNan;                             // (one is enough for spectral_bisect_kernel)
-        return;
-    }
-    float mx = 0.f;
-    for (int i = t; i < M * M; i += TH) mx = fmaxf(mx, fabsf(G[i]));
+    __shared__ unsigned red[32];
+    unsigned mx = 0u;
+    for (int i = t; i < M * M; i += TH) mx = max(mx, eig_magnitude(G[i]));
     const float scale = eig_block_scale(mx, red);
     for (int i = t; i < M * M; i += TH) A[i] = G[i] * scale;
     __syncthreads();
