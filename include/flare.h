@@ -159,7 +159,8 @@ int flare_forward(const flare_desc_t *desc, const void *Q_lat, const void *K, co
  * kernels rebuild dY_n.Y_n = sum_m W_dec[n,m] (dY_n.Z_m) in float32 instead of reading the rounded Y, which
  * is markedly more accurate where the latent rows a token mixes are nearly equal).
  * bfloat16 inputs run all three passes (dZ; dK, dV; dQ_lat) on the tensor cores, with
- * every rounded factor of a cancelling sum carried as two bfloat16 halves; float32 inputs run on the CUDA cores.
+ * every rounded factor of a cancelling sum carried as two bfloat16 halves (for dQ_lat at D = 64 as three parts, all 24
+ * bits of a float32); float32 inputs run on the CUDA cores.
  * dQ_lat, dK, dV are overwritten.  Workspace: flare_workspace_bytes(desc, FLARE_OP_BACKWARD) bytes holding dZ,
  * per-split partial sums of dZ and dQ_lat, one float per (b, n, h), and, beyond 1024 bfloat16 latents (448 at
  * D = 32, 192 at D = 64), float32 sums of the rows of dK and dV; nothing of size N x M.
@@ -248,7 +249,8 @@ int flare_spectral_gram(const flare_desc_t *desc, const void *Q_lat, const void 
  * path.  Eigenvalues alone (U = NULL): Householder tridiagonalisation, then bisection on Sturm counts; with eigenvectors:
  * cyclic Jacobi rotations, one thread block per matrix.  G [matrices, M, M] float32 is destroyed;
  * eigenvalues [matrices, M] come out in descending order; U [matrices, M, M] (may be NULL) gets the eigenvectors as
- * columns, in the same order.  sweeps (Jacobi): <= 0 means the default (12).  M <= 1024.  (The eigenvectors of W itself,
+ * columns, in the same order.  A matrix that holds a NaN or an infinity gets NaN for all of its eigenvalues (and eigenvectors).
+ * sweeps (Jacobi): <= 0 means the default (12).  M <= 1024.  (The eigenvectors of W itself,
  * L_N^{1/2} J^T U Sigma^{-1}, are N x M and are not formed.)
  */
 int flare_spectral_eig(int32_t matrices, int32_t M, float *G, float *eigenvalues, float *U, int32_t sweeps,
