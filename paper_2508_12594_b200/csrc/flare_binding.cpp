@@ -9,6 +9,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 
 #include <map>
@@ -310,6 +311,14 @@ double number(PyObject *o) {
     return x;
 }
 
+// Scratch that is dropped when the call returns, with its kernels still queued: allocated on the stream it is used on (none given: the
+// current one), so that nothing of another stream takes its place before they have run, or is still at work on it when they start.
+at::Tensor scratch(size_t bytes, const at::Tensor &like, PyObject *stream, flare_stream_t st) {
+    c10::cuda::OptionalCUDAStreamGuard guard;
+    if (stream != Py_None) guard.reset_stream(c10::cuda::getStreamFromExternal((cudaStream_t)st, like.device().index()));
+    return at::empty({(int64_t)bytes}, like.options().dtype(at::kByte));
+}
+
 // Q, K, V, key_mask, scale, want_stats, stream -> Y, or (Y, Z, lse_enc, lse_dec)
 BINDING(call_forward, 7)
     const at::Tensor &Q = tensor(a[0]), &K = tensor(a[1]);
@@ -324,14 +333,14 @@ BINDING(call_forward, 7)
     const auto f32 = K.options().dtype(at::kFloat);
     if (stats) {
         const at::Tensor Z = at::empty({d.B, d.H, d.M, d.D}, f32), le = at::empty({d.B, d.H, d.M}, f32), ld = at::empty({d.B, d.N, d.H}, f32);
-        const at::Tensor w = at::empty({(int64_t)ws}, K.options().dtype(at::kByte));
+        const at::Tensor w = scratch(ws, K, a[6], st);
         check_status(unlocked([&] { return lib.forward(&d, q, k, v, m, Y.data_ptr(), (float *)Z.data_ptr(), (float *)le.data_ptr(),
                                                        (float *)ld.data_ptr(), w.data_ptr(), ws, st); }), "flare_forward");
         return Py_BuildValue("(NNNN)", THPVariable_Wrap(Y), THPVariable_Wrap(Z), THPVariable_Wrap(le), THPVariable_Wrap(ld));
     }
     // Z lives in the workspace, the statistics (asked for: the encode weights are then as accurate as in training) behind it
     const size_t le_at = round256(ws), ld_at = round256(le_at + 4 * (size_t)d.B * d.H * d.M), total = ld_at + 4 * (size_t)d.B * d.N * d.H;
-    const at::Tensor w = at::empty({(int64_t)total}, K.options().dtype(at::kByte));
+    const at::Tensor w = scratch(total, K, a[6], st);
     char *base = (char *)w.data_ptr();
     check_status(unlocked([&] { return lib.forward(&d, q, k, v, m, Y.data_ptr(), nullptr, (float *)(base + le_at), (float *)(base + ld_at), base, ws, st); }),
                  "flare_forward");
@@ -351,7 +360,7 @@ BINDING(call_forward_backward, 7)
     const at::Tensor Y = at::empty({d.B, d.N, d.H, d.D}, K.options()), dK = at::empty({d.B, d.N, d.H, d.D}, K.options());
     const at::Tensor dV = at::empty({d.B, d.N, d.H, d.D}, K.options()), dQ = at::empty({d.H, d.M, d.D}, K.options().dtype(at::kFloat));
     const size_t z_at = round256(ws), le_at = round256(z_at + 4 * (size_t)d.B * d.H * d.M * d.D), ld_at = round256(le_at + 4 * (size_t)d.B * d.H * d.M);
-    const at::Tensor w = at::empty({(int64_t)(ld_at + 4 * (size_t)d.B * d.N * d.H)}, K.options().dtype(at::kByte));
+    const at::Tensor w = scratch(ld_at + 4 * (size_t)d.B * d.N * d.H, K, a[6], st);
     char *base = (char *)w.data_ptr();
     float *z = (float *)(base + z_at), *le = (float *)(base + le_at), *ld = (float *)(base + ld_at);
     check_status(unlocked([&] { return lib.forward(&d, q, k, v, m, Y.data_ptr(), z, le, ld, base, ws, st); }), "flare_forward");

@@ -108,3 +108,24 @@ def test_calls_behind_one_another(specs):
     graph.replay()                                              # two replays without a pause between them
     graph.replay()
     check("replayed twice")
+
+
+@pytest.mark.parametrize("train", [False, True])
+def test_scratch_belongs_to_the_stream_of_the_call(train):
+    """What a one-line call drops on return while its kernels are queued was allocated on their stream: the allocator may hand memory of the
+    current stream on at once."""
+    inp = workloads.make_random(1, 2, 3000, 64, 32, dtype="bf16", seed=3, with_dy=True)
+    Q, K, V, dY = dev(inp.Q), dev(inp.K), dev(inp.V), dev(inp.dY)
+
+    def call(stream=None):
+        return flare.forward_backward(Q, K, V, dY, stream=stream) if train else flare.forward(Q, K, V, want_stats=True, stream=stream)
+
+    want = [t.clone() for t in call()]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    side = torch.cuda.Stream()
+    got = call(side)
+    torch.cuda.synchronize()
+    assert all(torch.equal(g, w) for g, w in zip(got, want))
+    held = sum(s["total_size"] for s in torch.cuda.memory_snapshot() if s["stream"] == side.cuda_stream)
+    assert held >= flare.flare_workspace_bytes(flare.make_desc(Q, K), flare.OP_BACKWARD if train else flare.OP_FORWARD)
