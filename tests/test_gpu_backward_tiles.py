@@ -36,7 +36,8 @@ def test_backward_tile_edges(oracle, B, H, N, M, D, masked, k_std):
 
 
 @pytest.mark.parametrize("B,H,N,M,masked", [(1, 1, 64, 16, 0.0), (1, 2, 129, 48, 0.0), (2, 2, 700, 128, 0.2), (1, 2, 900, 144, 0.0),
-                                            (4, 2, 2048, 64, 0.0), (1, 2, 20011, 32, 0.1), (1, 1, 40000, 256, 0.0)])
+                                            (4, 2, 2048, 64, 0.0), (1, 2, 20011, 32, 0.1), (1, 1, 40000, 256, 0.0),
+                                            (1, 2, 1500, 160, 0.1), (1, 2, 1500, 176, 0.0)])
 def test_wide_heads_keep_float32_accuracy_of_dq(oracle, B, H, N, M, masked):
     """dQ at D = 64: its kernel multiplies Z, dZ and dS in three parts, so that what is left is the forward's and the dZ pass' weights in
     two bf16 halves.  A factor in two halves is off by at most 2^-18 of itself, with random sign: less than 2^-18 of the norm in all.  (One
