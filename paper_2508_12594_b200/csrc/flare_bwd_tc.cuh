@@ -177,7 +177,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     constexpr int UNIT = kDqUnit, UPT = kTile / UNIT, nstages = SM::kStages;
     static_assert(nstages >= 2, "one tile is finished while the next begins");
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = ptx::align_1024(smem_raw);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off);
     enum { T_FULL = 0, T_EMPTY = T_FULL + nstages, C_FULL = T_EMPTY + nstages, C_EMPTY = C_FULL + SM::kCst, S_FULL = C_EMPTY + SM::kCst,
            P_FULL = S_FULL + 2, ACC_DONE = P_FULL + 2, NBARS = ACC_DONE + 1 };
@@ -610,7 +610,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     constexpr int UNIT = kUnit, NG = BG::n, kThreads = BG::kThreads, kMaxSt = SM::kMaxStages, DR = DRT ? DRT : D;
     constexpr int K_COL = kUnitCols, V_COL = K_COL + D;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = ptx::align_1024(smem_raw);
     const int M = a.M, stages = a.stages;
     float *cst = reinterpret_cast<float *>(smem + SM::cst_off(stages, M));      // [M] -lse_enc (log2 units), [M] -de, [M] 2^(K - lse_enc)
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off(stages, M));

@@ -131,7 +131,7 @@ encode_lean_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constan
     constexpr bool kDz = kKind == kLeanDz, kTwo = kKind != kLeanFast;
     constexpr int UNIT = LG::UNIT, NG = LG::NG, nstages = LG::kStages, kThreads = LG::kThreads;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = ptx::align_1024(smem_raw);
     uint8_t *sQ = smem + LG::q_off;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + LG::bar_off);
     enum { KV_FULL = 0, KV_EMPTY = KV_FULL + nstages, S_FULL = KV_EMPTY + nstages, P_FULL = S_FULL + NG, NBARS = P_FULL + NG };

@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) micro_softmax_kernel(int iters,
 // out[1] = cycles from the commit to the barrier's flip (averages over `iters` rounds).  Operands are zeros.
 __global__ void __launch_bounds__(64, 1) micro_mma_kernel(int iters, unsigned long long *out) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = ptx::align_1024(smem_raw);
     __shared__ uint64_t bar_mem;
     __shared__ uint32_t tmem_slot, flag;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

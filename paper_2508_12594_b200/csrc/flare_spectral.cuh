@@ -63,7 +63,7 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
     using GP = TileGeom<32>;                                    // the J tiles in shared memory: 32 tokens = 64 bytes per latent row
     using SM = SpectralSmem<D>;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = ptx::align_1024(smem_raw);
     uint8_t *sK = smem + SM::k_off, *sQ = smem + SM::q_off, *sPB = smem + SM::pb_off;
     float *colneg = reinterpret_cast<float *>(smem + SM::col_off);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off);

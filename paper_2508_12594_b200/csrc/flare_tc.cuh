@@ -424,7 +424,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     using G = TileGeom<D>;
     using SM = DecodeSmem<D>;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = ptx::align_1024(smem_raw);
     const int M = kM ? kM : a.M;
     uint8_t *sK = smem + SM::k_off;
     uint8_t *sQ = smem + SM::q_off(M);
@@ -798,7 +798,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     using G = TileGeom<D>;
     using SM = DecodeStreamSmem<D>;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = ptx::align_1024(smem_raw);
     static_assert(kM % 64 == 0, "compile-time latent counts are multiples of 64");
     // M: latents; MP: rows of the latent operands, whole units (rows beyond M are zeros; their weights are left out)
     const int M = kM ? kM : a.M, MP = kM ? kM : SM::padded(a.M);
@@ -1308,7 +1308,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     static_assert(kAlt || !kPair, "head pairs share one latent block");
     constexpr int nstages = SM::kStages;                        // depth of the K/V ring
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *smem = ptx::align_1024(smem_raw);
     uint8_t *sKV = smem + SM::kv_off;
     uint8_t *sQ = smem + SM::q_off();
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off());
