@@ -49,13 +49,13 @@ __device__ __forceinline__ DsPair ds_pair(float2 s, float2 av, float2 cv, float2
         ds = __fmul2_rn(pd, __ffma2_rn(r, v, u));
     }
     DsPair o;
-    o.hi = ptx::pack_bf16(ds.x, ds.y);
-    const float2 rest = make_float2(ds.x - __uint_as_float(o.hi << 16), ds.y - __uint_as_float(o.hi & 0xffff0000u));
-    o.lo = ptx::pack_bf16(rest.x, rest.y);
-    if (kThird) o.lo2 = ptx::pack_bf16(rest.x - __uint_as_float(o.lo << 16), rest.y - __uint_as_float(o.lo & 0xffff0000u));
+    o.hi = ptx::pack_bf16(ds);
+    const float2 rest = ptx::rest_of(ds, o.hi);
+    o.lo = ptx::pack_bf16(rest);
+    if (kThird) o.lo2 = ptx::pack_bf16(ptx::rest_of(rest, o.lo));
     if (kWeights) {
-        o.whi = ptx::pack_bf16(pe.x, pe.y);
-        o.wlo = ptx::pack_bf16(pe.x - __uint_as_float(o.whi << 16), pe.y - __uint_as_float(o.whi & 0xffff0000u));
+        o.whi = ptx::pack_bf16(pe);
+        o.wlo = ptx::pack_bf16(ptx::rest_of(pe, o.whi));
     }
     return o;
 }

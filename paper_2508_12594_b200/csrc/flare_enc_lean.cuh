@@ -91,7 +91,7 @@ __device__ __forceinline__ void lean_chunk(const uint32_t *r, uint32_t *pk, uint
             pk[j] = ptx::pack_bf16(p.x, p.y);
             if (kKind == kLeanHiLo) sum2 = __fadd2_rn(sum2, p);
             if (kKind == kLeanFast && !kOnes) sum2 = __fadd2_rn(sum2, make_float2(__uint_as_float(pk[j] << 16), __uint_as_float(pk[j] & 0xffff0000u)));
-            if (kKind != kLeanFast) pl[j] = ptx::pack_bf16(p.x - __uint_as_float(pk[j] << 16), p.y - __uint_as_float(pk[j] & 0xffff0000u));
+            if (kKind != kLeanFast) pl[j] = ptx::pack_bf16(ptx::rest_of(p, pk[j]));
         }
     }
 }

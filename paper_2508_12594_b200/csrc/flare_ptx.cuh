@@ -271,5 +271,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return r;
 }
 
+// What rounding the pair x to the packed bf16 pair h left, exactly: the low halves of a split in two (one packed instruction, where two
+// subtractions took two).
+__device__ __forceinline__ float2 rest_of(float2 x, uint32_t h) {
+    return __ffma2_rn(make_float2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)), make_float2(-1.f, -1.f), x);
+}
+__device__ __forceinline__ uint32_t pack_bf16(float2 x) { return pack_bf16(x.x, x.y); }
+
 }  // namespace ptx
 }  // namespace flare

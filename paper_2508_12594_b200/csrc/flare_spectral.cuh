@@ -189,8 +189,8 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
                 const uint32_t h0 = ptx::pack_bf16(p0, p1), h1 = ptx::pack_bf16(p2, p3);
                 hi[2 * k] = h0;
                 hi[2 * k + 1] = h1;
-                lo[2 * k] = ptx::pack_bf16(p0 - __uint_as_float(h0 << 16), p1 - __uint_as_float(h0 & 0xffff0000u));
-                lo[2 * k + 1] = ptx::pack_bf16(p2 - __uint_as_float(h1 << 16), p3 - __uint_as_float(h1 & 0xffff0000u));
+                lo[2 * k] = ptx::pack_bf16(ptx::rest_of(make_float2(p0, p1), h0));
+                lo[2 * k + 1] = ptx::pack_bf16(ptx::rest_of(make_float2(p2, p3), h1));
             }
             ptx::tmem_st16(scol, hi);                           // A operand: back over the scores, hi then lo
             ptx::tmem_st16(scol + 16, lo);

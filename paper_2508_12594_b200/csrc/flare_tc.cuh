@@ -166,7 +166,7 @@ __device__ __forceinline__ void exp_chunk_hilo(const uint32_t *r, uint32_t *hi, 
         sum2 = __fadd2_rn(sum2, p);
         const uint32_t h = ptx::pack_bf16(p.x, p.y);
         hi[k] = h;
-        lo[k] = ptx::pack_bf16(p.x - __uint_as_float(h << 16), p.y - __uint_as_float(h & 0xffff0000u));
+        lo[k] = ptx::pack_bf16(ptx::rest_of(p, h));
     }
 }
 
