@@ -58,7 +58,7 @@ int launches_for(const flare_desc_t *d, int op, int sms) {
         case FLARE_OP_FORWARD: return enc + dec;
         case FLARE_OP_BACKWARD: {
             (void)sms;
-            const int tok = token_in_ranges(d) ? 2 * ((d->M + token_range(d) - 1) / token_range(d)) : 1;
+            const int tok = (d->M + token_range(d) - 1) / token_range(d);
             return 2 + tok + 2;                                 // dZ, its reduction; token kernel(s); dQ, its reduction
         }
         default: return 0;

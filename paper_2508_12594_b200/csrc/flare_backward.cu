@@ -52,7 +52,7 @@ int launch_bwd_dq_tc(const flare_desc_t *d, const TcEncodePlan &p, const void *Q
     }
 }
 
-template <int D, int DRT, int kMode, bool kPadded>
+template <int D, int DRT, bool kRanges>
 int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const void *V, const void *dY, BwdTokTcArgs a, cudaStream_t st) {
     CUtensorMap tmK, tmV, tmG;
     int rc;
@@ -62,32 +62,29 @@ int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const v
     a.stages = BwdTokSmem<D>::stages(a.M);
     if (a.stages < 1) return FLARE_ERR_UNSUPPORTED;
     static std::atomic<uint64_t> smem_opt_in{0};
-    if ((rc = ensure_big_smem(bwd_token_tc_kernel<D, DRT, kMode, kPadded>, smem_opt_in)) != FLARE_OK) return rc;
+    if ((rc = ensure_big_smem(bwd_token_tc_kernel<D, DRT, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
     a.tiles = (d->N + kTile - 1) / kTile;
     long per_head = sms / ((long)d->B * d->H);
     if (per_head < 1) per_head = 1;
     if (per_head > a.tiles) per_head = a.tiles;
-    FLARE_CUDA(launch_after(bwd_token_tc_kernel<D, DRT, kMode, kPadded>, dim3((unsigned)per_head, d->H, d->B), BwdGroups<2 * D>::kThreads, BwdTokSmem<D>::total(a.stages, a.M), st,  tmK, tmV, tmG, a));
+    FLARE_CUDA(launch_after(bwd_token_tc_kernel<D, DRT, kRanges>, dim3((unsigned)per_head, d->H, d->B), BwdTokSmem<D>::kThreads, BwdTokSmem<D>::total(a.stages, a.M), st,  tmK, tmV, tmG, a));
     return FLARE_OK;
 }
 
-// The launch's range of latents is [m0, m0 + mc).  mode: see BwdTokTcArgs.
+// The launch's range of latents is [m0, m0 + mc); dd_sums, kvacc: see BwdTokTcArgs.
 template <int D, int DRT>
 int launch_bwd_token_tc(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const void *dY,
                         const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
-                        const float *lse_dec, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st, int mode, int m0, int mc,
-                        float *kvacc) {
+                        const float *lse_dec, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st, int m0, int mc,
+                        const float *dd_sums, float *kvacc) {
     BwdTokTcArgs a;
     a.Q = static_cast<const __nv_bfloat16 *>(Q);
     a.Z = Z; a.dZ = dZ; a.lse_enc = lse_enc; a.de = de; a.lse_dec = lse_dec; a.key_mask = mask;
     a.dK = (__nv_bfloat16 *)dK; a.dV = (__nv_bfloat16 *)dV; a.dd = dd; a.status = status;
     a.B = d->B; a.H = d->H; a.N = d->N; a.M = mc;
-    a.mtot = d->M; a.m0 = m0; a.first = m0 == 0; a.last = m0 + mc >= d->M; a.kvacc = kvacc;
+    a.mtot = d->M; a.m0 = m0; a.first = m0 == 0; a.last = m0 + mc >= d->M; a.kvacc = kvacc; a.dd_sums = dd_sums;
     a.scale = d->scale; a.sl2 = d->scale * kLog2e;
-    const bool pad = has_padding(d, mask);
-#define FLARE_TOK(MODE) (pad ? launch_bwd_token_tc_n<D, DRT, MODE, true>(d, sms, K, V, dY, a, st) : launch_bwd_token_tc_n<D, DRT, MODE, false>(d, sms, K, V, dY, a, st))
-    return mode == 0 ? FLARE_TOK(0) : mode == 1 ? FLARE_TOK(1) : FLARE_TOK(2);
-#undef FLARE_TOK
+    return token_in_ranges(d) ? launch_bwd_token_tc_n<D, DRT, true>(d, sms, K, V, dY, a, st) : launch_bwd_token_tc_n<D, DRT, false>(d, sms, K, V, dY, a, st);
 }
 
 template <typename T, int D>
@@ -131,14 +128,16 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
         uint32_t *status = reinterpret_cast<uint32_t *>(ws);
         on_tc = use_tc(d);
         if (on_tc) {
-            // more latents than one launch holds: two series of launches over ranges of them, dd[n] first, then the rows of dK and dV
-            float *kvacc = reinterpret_cast<float *>(ws + w.kvacc);
-            const int R = token_range(d);
-            for (int mode = token_in_ranges(d) ? 1 : 0; mode <= (token_in_ranges(d) ? 2 : 0); ++mode)
-                for (int m0 = 0; m0 < d->M; m0 += R)
-                    if (const int rc = launch_bwd_token_tc<DK, DRT>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, dd, status,
-                                                                    st, mode, m0, d->M - m0 < R ? d->M - m0 : R, kvacc))
-                        return rc;
+            // more latents than one launch holds are worked off in ranges; dd alternates between two arrays, the last range's is w.dd
+            float *kvacc = reinterpret_cast<float *>(ws + w.kvacc), *dd_other = reinterpret_cast<float *>(ws + w.dd_other);
+            const int R = token_range(d), ranges = (d->M + R - 1) / R;
+            for (int k = 0; k < ranges; ++k) {
+                const int m0 = k * R;
+                const bool to_dd = (ranges - 1 - k) % 2 == 0;
+                if (const int rc = launch_bwd_token_tc<DK, DRT>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, to_dd ? dd : dd_other, status,
+                                                                st, m0, d->M - m0 < R ? d->M - m0 : R, to_dd ? dd_other : dd, kvacc))
+                    return rc;
+            }
             const TcEncodePlan p = tc_dq_plan(d, sms);
             if (const int rc = launch_bwd_dq_tc(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st)) return rc;
             dq_parts = p.P;

@@ -73,17 +73,24 @@ __device__ __forceinline__ float warp_lse_min(const float *lse_enc, int rows) {
 }
 
 // rows of a [rows, DR] float matrix -> bf16 halves (kThird: three parts, the third in lo2) in swizzled rows (DR >= 8), starting at
-// logical chunk `chunk0` of row r0 + m
-template <int DG, int DR, bool kThird = false>
+// logical chunk `chunk0` of row r0 + m; each less `centre` (null: nothing), row m times factor(m)
+template <int DG, int DR, bool kThird = false, class Factor = UnitFactor>
 __device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float *src, int rows, int r0, int chunk0, int tid, int threads,
-                                           uint8_t *lo2 = nullptr) {
+                                           const float *centre = nullptr, Factor factor = Factor(), uint8_t *lo2 = nullptr) {
     using G = TileGeom<DG>;
     constexpr int ZC = DR >= 8 ? DR / 8 : 1;
     for (int i = tid; i < rows * ZC; i += threads) {
         const int m = i / ZC, c = i % ZC, r = r0 + m;
         const float4 a = *reinterpret_cast<const float4 *>(src + (size_t)m * DR + c * 8);
         const float4 b = *reinterpret_cast<const float4 *>(src + (size_t)m * DR + c * 8 + 4);
-        const float z[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        float4 ca = make_float4(0.f, 0.f, 0.f, 0.f), cb = ca;
+        if (centre != nullptr) {
+            ca = *reinterpret_cast<const float4 *>(centre + c * 8);
+            cb = *reinterpret_cast<const float4 *>(centre + c * 8 + 4);
+        }
+        const float f = factor(m);
+        const float z[8] = {(a.x - ca.x) * f, (a.y - ca.y) * f, (a.z - ca.z) * f, (a.w - ca.w) * f,
+                            (b.x - cb.x) * f, (b.y - cb.y) * f, (b.z - cb.z) * f, (b.w - cb.w) * f};
         uint32_t vh[4], vl[4], vl2[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -217,25 +224,28 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     }
     // latent operands Q, Z_hi, Z_lo, dZ_hi, dZ_lo (D = 64: three parts of Z and dZ): zeros where there is no row (or, pair and narrow forms, no feature), then the rows
     const bool gaps = kPair || DRT != 0 || rows_here < kTile;
+    float *centre = reinterpret_cast<float *>(smem + SM::cst_off);                        // (the ring of constants is not in use yet)
+#pragma unroll
+    for (int w = 0; w < (kPair ? 2 : 1); ++w) z_centre<DR>(centre + w * DR, a.Z + ((size_t)b * a.H + h + w) * M * DR, M);
     if (gaps) {
         for (int i = threadIdx.x; i < SM::kLat * kTile * (G::RB / 16); i += kDqThreads)
             reinterpret_cast<uint4 *>(smem + SM::lat_off(0))[i] = make_uint4(0, 0, 0, 0);
-        __syncthreads();
     }
+    __syncthreads();
 #pragma unroll
     for (int w = 0; w < (kPair ? 2 : 1); ++w) {
         const size_t q0 = (size_t)(h + w) * M + lb * kTile, r0 = ((size_t)b * a.H + h + w) * M + lb * kTile;
         if constexpr (DR == 4) {
             stage_rows4<DG>(smem + SM::lat_off(0), a.Q + q0 * DR, rows_here, off);
-            stage_rows4_hilo<DG>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, off);
+            stage_rows4_hilo<DG>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, off, centre);
             stage_rows4_hilo<DG>(smem + SM::lat_off(3), smem + SM::lat_off(4), a.dZ + r0 * DR, rows_here, off);
         } else {
             stage_bf16<DG, DR>(smem + SM::lat_off(0), a.Q + q0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
             stage_hilo<DG, DR, kThird>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads,
-                                       smem + SM::lat_off(3));
+                                       centre + w * DR, UnitFactor(), smem + SM::lat_off(3));
             constexpr int dz0 = 1 + SM::kParts;
             stage_hilo<DG, DR, kThird>(smem + SM::lat_off(dz0), smem + SM::lat_off(dz0 + 1), a.dZ + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x,
-                                       kDqThreads, smem + SM::lat_off(SM::kLat - 1));
+                                       kDqThreads, nullptr, UnitFactor(), smem + SM::lat_off(SM::kLat - 1));
         }
     }
     ptx::fence_proxy_async_smem();
@@ -528,27 +538,29 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 }
 
 // ------------------------------------------------------------------------------- pass B, token side (dK, dV)
-// Tokens on the lanes, latents on the columns.  Two sweeps over the latents of a tile: the first needs S^T = K Q^T and
-// A^T = dY Z^T and leaves dd[n] = sum_m W_dec[n,m] A[n,m]; the second adds C^T = V dZ^T, turns the three into dS^T and W_enc^T and
-// accumulates dK_n = sum_m dS[m,n] q_m and dV_n = sum_m W_enc[m,n] dZ_m.  dd goes to the workspace for the dQ kernel.
-
-// A unit is 32 latents wide, and a CTA is a few independent groups of four warps (one per quarter of the lanes; a thread works on all 32
-// columns of its lane), each with a tile of its own, one buffer S | A | C and its own accumulators: while one group waits for the tensor
-// core the others work, nothing is shared between them, and dd needs no exchange.  There is no issuing warp: the warps of a group
-// take turns issuing the output contractions of a unit, the tiles of the next and one commit, which says that all of them are done.
-// Measured, us, on the shapes named at the dQ kernel, against units of 16 columns, two exponentials per pair and half as many latents per
-// launch: 22.4, 164, 1166, 9254 -> 19.9, 132, 1016, 8936; D = 64: 1049 (CUDA cores) -> 67
-// (with the third part of Z 73).  Units of 64 columns shared by sixteen warps, as
-// in the dQ kernel: 39.6, 254, 1154, 16489; 71 (W_enc doubles what a thread holds: it spills).  Bound by issue slots, some 26
-// instructions per pair over both sweeps.
-// Groups of four warps, by accumulator columns: as many as 512 columns of tensor memory hold, at most four.  Warps: 0 TMA producer, from 2
-// on the groups (warp & 3 = the quarter of the lanes a warp can reach).  18, 14 or 10 warps: 96, 128 or 168 registers each.
-constexpr int kUnit = 32, kUnitCols = 3 * kUnit, kBwdFirstMathWarp = 2;
-template <int kAccCols> struct BwdGroups {
-    static constexpr int fit = 512 / (kUnitCols + kAccCols), n = fit > 4 ? 4 : fit, cols = (512 / n) & ~31;   // (whole blocks of 32 columns)
-    static_assert(kUnitCols + kAccCols <= cols, "tensor memory");
-    static constexpr int kThreads = (kBwdFirstMathWarp + 4 * n) * 32;
-};
+// Tokens on the lanes, latents on the columns, one sweep over the latents of a tile.  dd[n] = sum_m W_dec[n,m] A[n,m], which every dS of the
+// row needs, is known only when the row is done; but it enters linearly, so it is put in at the end:
+//     dK_n = scale (T_n - dd[n] U_n),   T_n = sum_m (W_dec A + W_enc (C - de))[n,m] q_m,   U_n = sum_m W_dec[n,m] q_m.
+// And W_enc = W_dec r[n] c[m] with r = 2^(lse_dec[n] - K), c = 2^(K - lse_enc[m]) and K in the middle of the latents' lse_enc, so that with
+// c dZ in the place of dZ one weight serves everything:
+//     T_n = sum_m W_dec (A + r (C' - c de)) q_m,   C' = V (c dZ)^T,     dV_n = r sum_m W_dec (c dZ)_m,
+// one exponential and one split of a weight per pair, and [dV | U] one accumulator whose contractions share their A operand.  dd goes to the
+// workspace for the dQ kernel.
+//
+// What the factors may lose: W_dec below 2^-126 is flushed, which is a W_enc below 2^-126 r c <= 2^(range of lse_enc + log2 M - 126) (log2
+// units; lse_dec[n] <= log2 M + the largest lse_enc, since lse_enc[m] >= S[m,n]); with that sum at most kFoldLog2 a weight below
+// 2^-46.  Wider ranges (c is 1 then), and tiles with a token whose lse_dec lies further above K than consistent statistics put it
+// (kFarLog2; an infinite lse_dec is how the two-query variant switches a stage off) take a form of the body with an exponential of its
+// own for W_enc, whose halves are a third pair of operands (kTwo).
+//
+// Sixteen warps share units of 64 latents, 16 columns each, on two alternating buffers of tensor memory (S | A | C), as in the dQ kernel; up
+// to 32 latents two sets of eight warps take a tile each, so that no warp idles.  Rows leave the accumulators after the first unit of the next tile.
+// D = 64: units of 32 shared by eight warps (the accumulators take 192 columns).
+// Two sweeps over the latents (dd first; two exponentials and 26 instructions per pair, here one and 20), by groups of four warps with units of their
+// own, took, us per training step -> now: 131072 tokens, M = 512, D = 32 (in two ranges, 448 latents at most) 1905 -> 1513; 1048576, M = 1024, D = 8 20967 -> 20025;
+// 32 x 4096, M = 128, D = 32 300 -> 283; 2 x 20011, M = 128, D = 64 187 -> 178; 16384, M = 32, D = 32 84.2 -> 85.1.
+constexpr float kFoldLog2 = 80.f, kFarLog2 = 46.f;
+constexpr int kTokFirstMathWarp = 4;                            // warps: 0 TMA producer, 1 MMA issue, 2 token constants, 4 on arithmetic
 
 struct BwdTokTcArgs {
     const __nv_bfloat16 *Q;    // [H,M,D]
@@ -557,16 +569,16 @@ struct BwdTokTcArgs {
     const float *lse_dec;      // [B,N,H]
     const uint8_t *key_mask;   // [B,N] or null
     __nv_bfloat16 *dK, *dV;    // [B,N,H,D]
-    float *dd;                 // [B,H,N] (workspace): written in modes 0 and 1, read in mode 2
+    float *dd;                 // [B,H,N] (workspace)
     uint32_t *status;
     int B, H, N, M;            // M: latents this launch works on (all of them, or a range)
     int mtot, m0;              // latents per head in memory, and the first one of this launch's range
-    // More latents than one launch can keep in shared memory are worked off in ranges, by two series of launches:
-    // mode 1 (first sweep only) adds the range's share of dd[n] to the workspace; mode 2 (second sweep only, dd
-    // complete) adds the range's share of the rows of dK and dV to float32 sums in kvacc [2][B*N*H][D] and, in the
-    // last range, writes the rows.  Mode 0 does both sweeps over all latents in one launch.
-    int first, last;           // (the mode is a template parameter of the kernel)
+    // More latents than one launch can keep in shared memory are worked off in ranges: T, dV, U and dd of a range add up with the earlier
+    // ranges' in float32 sums, kvacc [3][B*N*H][D] and dd_sums (read) / dd (written: another array, since several threads
+    // read what one of them replaces), and the last range writes the rows.
+    int first, last;           // (without ranges both)
     float *kvacc;
+    const float *dd_sums;
     float scale, sl2;
     int tiles, stages;
 };
@@ -574,21 +586,33 @@ struct BwdTokTcArgs {
 template <int D>
 struct BwdTokSmem {
     using G = TileGeom<D>;
-    // D = 64: dd[n] is subtracted from products that the dQ kernel forms of three parts of Z, so the first sweep takes three as well (with two,
+    static constexpr int UNIT = D == 64 ? 32 : 64, NCG = UNIT / 16, kThreads = (kTokFirstMathWarp + 4 * NCG) * 32;
+    static constexpr int kAccStride = D == 16 ? 64 : 3 * D;     // columns of an accumulator dV | U | T (whole blocks of 32)
+    // accumulators beside two buffers of three regions of ucols columns: the largest power of two up to four (as a logarithm)
+    __device__ static __forceinline__ int log2_accs(int ucols) {
+        const int fit = (512 - 6 * ucols) / kAccStride;
+        return fit >= 4 ? 2 : fit >= 2 ? 1 : 0;
+    }
+    static constexpr int kRing = 4;                             // tiles of token constants on their way or in use
+    // D = 64: dd[n] is subtracted from products that the dQ kernel forms of three parts of Z, so A is formed of three as well (with two,
     // dQ on features of point clouds was 4.7e-6 to 5.4e-6 of its norm from float64 instead of 2.6e-6 to 3.0e-6), as long as the third fits
     // beside two tile stages.
     static constexpr int kThirdMost = D == 64 ? 160 : 0;
-    // tiles: [stage][K | V | dY]; latents: Q, Z_hi, Z_lo, dZ_hi, dZ_lo (and a third part of Z) with M rows each (M a multiple of 16); their constants
+    enum { ZH = 0, ZL = 1, DL = 2, DH = 3, QR = 4, Z3 = 5 };    // latent operands: Z hi, lo, c dZ lo, hi, Q (behind c dZ hi: see issue_outputs), third part of Z
+    // tiles: [stage][K | V | dY]; latent operands with M rows each (M a multiple of 16); per latent the exponent's addend and -c de;
+    // per token -lse_dec and r; the column groups' shares of dd
     __host__ __device__ static size_t lat_off(int stages, int M, int which) {
         return (size_t)stages * 3 * G::TILE_BYTES + (size_t)which * M * G::RB;
     }
     __host__ __device__ static size_t cst_off(int stages, int M) { return lat_off(stages, M, M <= kThirdMost ? 6 : 5); }
-    __host__ __device__ static size_t bar_off(int stages, int M) { return cst_off(stages, M) + 3 * sizeof(float) * M; }
+    __host__ __device__ static size_t ring_off(int stages, int M) { return cst_off(stages, M) + 2 * sizeof(float) * M; }
+    __host__ __device__ static size_t dds_off(int stages, int M) { return ring_off(stages, M) + kRing * 2 * kTile * sizeof(float); }
+    __host__ __device__ static size_t bar_off(int stages, int M) { return dds_off(stages, M) + 4 * NCG * kTile * sizeof(float); }
     __host__ __device__ static size_t total(int stages, int M) {
         const size_t t = bar_off(stages, M) + 512 + 1024;
         return t < kTcMinSmem ? kTcMinSmem : t;
     }
-    static constexpr int kMaxStages = 8;
+    static constexpr int kMaxStages = 6;
     // the most stages (at most kMaxStages) that fit beside the latent operands; 0 if not even one does
     __host__ static int stages(int M) {
         int s = kMaxStages;
@@ -597,39 +621,48 @@ struct BwdTokSmem {
     }
 };
 
-// grid = (CTAs per head, H, B); a CTA takes the token tiles blockIdx.x, blockIdx.x + gridDim.x, ..., its groups a tile each in turn.
-// A tile's rows of dK and dV are read from the accumulators after the first sweep of the group's next tile, when the contractions
-// that complete them are long done.  DRT, kPadded: as in the dQ kernel.
-template <int D, int DRT, int kMode, bool kPadded>
-__global__ void __launch_bounds__(BwdGroups<2 * D>::kThreads, 1)
+// grid = (CTAs per head, H, B); a CTA takes the token tiles blockIdx.x, blockIdx.x + gridDim.x, ...  kRanges: see BwdTokTcArgs.  DRT: as in
+// the dQ kernel.
+template <int D, int DRT, bool kRanges>
+__global__ void __launch_bounds__(BwdTokSmem<D>::kThreads, 1)
 bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                     const __grid_constant__ CUtensorMap tmG, BwdTokTcArgs a) {
     using G = TileGeom<D>;
     using SM = BwdTokSmem<D>;
-    using BG = BwdGroups<2 * D>;
-    constexpr int UNIT = kUnit, NG = BG::n, kThreads = BG::kThreads, kMaxSt = SM::kMaxStages, DR = DRT ? DRT : D;
-    constexpr int K_COL = kUnitCols, V_COL = K_COL + D;
+    constexpr int UNIT = SM::UNIT, NCG = SM::NCG, kThreads = SM::kThreads, kMaxSt = SM::kMaxStages, RING = SM::kRing, DR = DRT ? DRT : D;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = ptx::align_1024(smem_raw);
     const int M = a.M, stages = a.stages;
-    float *cst = reinterpret_cast<float *>(smem + SM::cst_off(stages, M));      // [M] -lse_enc (log2 units), [M] -de, [M] 2^(K - lse_enc)
+    float *cst = reinterpret_cast<float *>(smem + SM::cst_off(stages, M));      // [M] addend of W_enc's own exponent, [M] -c de
+    float *ring = reinterpret_cast<float *>(smem + SM::ring_off(stages, M));    // [RING][-lse_dec (log2 units) | r][token]
+    float *dds = reinterpret_cast<float *>(smem + SM::dds_off(stages, M));      // [4][column group][token]
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off(stages, M));
-    enum { T_FULL = 0, T_EMPTY = T_FULL + kMaxSt, S_FULL = T_EMPTY + kMaxSt, P_FULL = S_FULL + NG, NBARS = P_FULL + NG };
-    static_assert(NBARS * 8 + 32 <= 512, "barrier area too small");
+    enum { T_FULL = 0, T_EMPTY = T_FULL + kMaxSt, S_FULL = T_EMPTY + kMaxSt, P_FULL = S_FULL + 2, C_FULL = P_FULL + 2, C_EMPTY = C_FULL + RING,
+           ACC_FULL = C_EMPTY + RING, ACC_EMPTY = ACC_FULL + 4, DD_FULL = ACC_EMPTY + 4, NBARS = DD_FULL + 8 };
+    static_assert(NBARS * 8 + 8 + 4 * RING + 8 * kThreads / 32 <= 512 + 0, "barrier area too small");
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NBARS);
     volatile uint32_t *abort_flag = tmem_slot + 1;
-    float *kmin = reinterpret_cast<float *>(tmem_slot + 2);     // smallest lse_enc of the launch's latents
+    volatile uint32_t *two_exp = tmem_slot + 2;                 // [RING]: the tile takes the form with two exponentials
+    float *extremes = reinterpret_cast<float *>(tmem_slot + 2 + RING);          // [warp][least, greatest lse_enc]
 
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int h = blockIdx.y, b = blockIdx.z;
     const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
-    const int nu = (M + UNIT - 1) / UNIT;                       // latent units per sweep; the last may have 16 columns
+    const int nu = (M + UNIT - 1) / UNIT;                       // latent units of a tile; the last may be narrower
+    const int wlast = M - (nu - 1) * UNIT;
+    // Sets of warps that take the units in turn: two where a unit fills no more than half of the column groups (then a tile is one unit).
+    const int sets = NCG == 4 && M <= 32 ? 2 : 1, cps = sets == 2 ? 2 : NCG;
+    const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S, A or C
+    const int log_accs = SM::log2_accs(ucols);                  // accumulators in turn for the tiles
     const int off = DRT ? narrow_offset(h, DR) : 0;
-    const bool third = D == 64 && kMode != 2 && M <= SM::kThirdMost;
+    const bool third = D == 64 && M <= SM::kThirdMost;
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
 
     if (threadIdx.x == 0) {
-        for (int i = 0; i < NBARS; ++i) ptx::mbar_init(bar(i), i >= P_FULL ? 4 : 1);
+        const uint32_t math = 4 * cps;                          // warps that work on a unit
+        for (int i = 0; i < NBARS; ++i)
+            ptx::mbar_init(bar(i), i >= DD_FULL || (i >= ACC_EMPTY && i < DD_FULL) || (i >= P_FULL && i < C_FULL) ? math
+                                   : i >= C_EMPTY && i < ACC_FULL ? math + 1u : 1u);
         *abort_flag = 0;
         ptx::fence_mbar_init();
         ptx::prefetch_tensormap(&tmK);
@@ -639,35 +672,60 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     ptx::grid_launch();
     ptx::grid_wait();
+    const size_t q0 = (size_t)h * a.mtot + a.m0, r0 = ((size_t)b * a.H + h) * a.mtot + a.m0;
+    z_centre<DR>(dds, a.Z + ((size_t)b * a.H + h) * a.mtot * DR, a.mtot);                    // (dds is not in use yet)
+    float K, unfolded;                                          // (unfolded != 0: c is 1)
     {
-        const size_t q0 = (size_t)h * a.mtot + a.m0, r0 = ((size_t)b * a.H + h) * a.mtot + a.m0;
-        if (warp == 2) {
-            const float k = warp_lse_min(a.lse_enc + r0, M);
-            if (lane == 0) *kmin = k;
+        // K: the middle of the latents' lse_enc (log2 units), leaving out those that saw no valid token and those whose encode is switched off
+        float lo = INFINITY, hi = -INFINITY;
+        for (int m = threadIdx.x; m < M; m += kThreads) {
+            const float le = a.lse_enc[r0 + m] * kBwdLog2e;
+            if (le != -INFINITY && le != INFINITY) {
+                lo = fminf(lo, le);
+                hi = fmaxf(hi, le);
+            }
         }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        if (lane == 0) {
+            extremes[2 * warp] = lo;
+            extremes[2 * warp + 1] = hi;
+        }
+        if (DRT != 0)                                           // narrow form: the other columns of every row stay zero
+            for (int i = threadIdx.x; i < 5 * M * (G::RB / 16); i += kThreads) reinterpret_cast<uint4 *>(smem + SM::lat_off(stages, M, 0))[i] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+        for (int w = 0; w < kThreads / 32; ++w) {
+            lo = fminf(lo, extremes[2 * w]);
+            hi = fmaxf(hi, extremes[2 * w + 1]);
+        }
+        K = lo <= hi ? 0.5f * (lo + hi) : 0.f;
+        unfolded = lo > hi || hi - lo + ptx::lg2((float)M) <= kFoldLog2 ? 0.f : 1.f;
+    }
+    auto factor = [&](int m) {                                  // c of latent m; 0 for those left out
+        const float le = a.lse_enc[r0 + m] * kBwdLog2e;
+        return le == -INFINITY || le == INFINITY ? 0.f : unfolded != 0.f ? 1.f : ptx::ex2(K - le);
+    };
+    {
         uint8_t *lat[5];
 #pragma unroll
         for (int w = 0; w < 5; ++w) lat[w] = smem + SM::lat_off(stages, M, w);
-        if (DRT != 0) {                                         // narrow form: the other columns of every row stay zero
-            for (int i = threadIdx.x; i < 5 * M * (G::RB / 16); i += kThreads) reinterpret_cast<uint4 *>(lat[0])[i] = make_uint4(0, 0, 0, 0);
-            __syncthreads();
-        }
         if constexpr (DR == 4) {
-            stage_rows4<D>(lat[0], a.Q + q0 * DR, M, off);
-            stage_rows4_hilo<D>(lat[1], lat[2], a.Z + r0 * DR, M, off);
-            stage_rows4_hilo<D>(lat[3], lat[4], a.dZ + r0 * DR, M, off);
+            stage_rows4<D>(lat[SM::QR], a.Q + q0 * DR, M, off);
+            stage_rows4_hilo<D>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, off, dds);
+            stage_rows4_hilo<D>(lat[SM::DH], lat[SM::DL], a.dZ + r0 * DR, M, off, nullptr, factor);
         } else {
-            stage_bf16<D, DR>(lat[0], a.Q + q0 * DR, M, 0, 0, threadIdx.x, kThreads);
-            if (third) stage_hilo<D, DR, true>(lat[1], lat[2], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, smem + SM::lat_off(stages, M, 5));
-            else stage_hilo<D, DR>(lat[1], lat[2], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads);
-            stage_hilo<D, DR>(lat[3], lat[4], a.dZ + r0 * DR, M, 0, 0, threadIdx.x, kThreads);
+            stage_bf16<D, DR>(lat[SM::QR], a.Q + q0 * DR, M, 0, 0, threadIdx.x, kThreads);
+            if (third) stage_hilo<D, DR, true>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, dds, UnitFactor(), smem + SM::lat_off(stages, M, SM::Z3));
+            else stage_hilo<D, DR>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, dds);
+            stage_hilo<D, DR>(lat[SM::DH], lat[SM::DL], a.dZ + r0 * DR, M, 0, 0, threadIdx.x, kThreads, nullptr, factor);
         }
-        __syncthreads();
         for (int m = threadIdx.x; m < M; m += kThreads) {
-            const float le = a.lse_enc[r0 + m], nle = (le == -INFINITY) ? -INFINITY : -le * kBwdLog2e;
-            cst[m] = nle;
-            cst[M + m] = -a.de[r0 + m];
-            cst[2 * M + m] = ptx::ex2(nle + *kmin);
+            const float c = factor(m);
+            cst[m] = c == 0.f ? -INFINITY : unfolded != 0.f ? -a.lse_enc[r0 + m] * kBwdLog2e : -K;
+            cst[M + m] = -c * a.de[r0 + m];
         }
     }
     ptx::fence_proxy_async_smem();
@@ -675,6 +733,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tm = *tmem_slot;
+    const uint32_t bcols = 3 * ucols, acc0 = 2 * bcols;         // columns of a buffer; the first accumulator
 
     if (warp == 0) {
         if (ptx::elect_one()) {
@@ -688,278 +747,322 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 ptx::tma_load_3d(ptx::smem_u32(dst + 2 * G::TILE_BYTES), &tmG, bar(T_FULL + s), h * DR - off, t * kTile, b);
             }
         }
-    } else if (warp >= kBwdFirstMathWarp) {
-        const int g = (warp - kBwdFirstMathWarp) >> 2;
-        const int row = ((warp & 3) << 5) + lane;               // TMEM lane = token within the tile
-        const uint32_t base = tm + g * BG::cols;                // the group's columns: S | A | C | dK | dV
-        const uint32_t gcol = base + ((uint32_t)((warp & 3) << 5) << 16);
-        const float2 sl2p = make_float2(a.sl2, a.sl2);
-        const float lse_min = *kmin;
-        const uint32_t pfull = bar(P_FULL + g), sfull = bar(S_FULL + g);
-        const int wlast = M - (nu - 1) * UNIT;                  // latents of the last unit
-        // (descriptors as 32-bit low words beside a constant high word: see ptx::desc)
-        constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), TILE = G::TILE_BYTES >> 4, STEP16 = (16 * G::RB) >> 4;
-        constexpr uint32_t MN = ptx::desc_lo(0, G::SBO) - ptx::desc_lo(0, 16);          // K-major to MN-major
-        const uint32_t LAT = (uint32_t)(M * G::RB) >> 4;        // from one latent operand to the next
-        auto lat_desc = [&](int u) {                            // low word of Q's rows of unit u
-            uint32_t d = ptx::desc_lo(ptx::smem_u32(smem + SM::lat_off(stages, M, 0)), 16) + (uint32_t)u * (UNIT / 16) * STEP16;
-            ptx::opaque(d);
-            return d;
-        };
-        // by one thread: S^T = K Q^T | A^T = dY (Z_hi + Z_lo)^T and (kSecond) C^T = V (dZ_hi + dZ_lo)^T of unit u of the tile in `stage`
-        auto issue_tiles = [&](auto second, int stage, int u) {
-            constexpr bool kSecond = decltype(second)::value;
-            const uint32_t idescS = ptx::instr_desc_bf16(128, u == nu - 1 ? wlast : UNIT, 0, 0);
-            uint32_t td = ptx::desc_lo(ptx::smem_u32(smem), 16) + (uint32_t)stage * 3 * TILE, ld = lat_desc(u);
-            ptx::opaque(td);
-            auto product = [&](int of, uint32_t lat, bool more) {   // of: S, A or C
-                const uint32_t col = base + of * UNIT, ad = td + (of == 0 ? 0 : of == 1 ? 2 * TILE : TILE);
+    } else if (warp == 2) {
+        // Token constants of every tile: -lse_dec and r (0 for a token that takes no part in the encode softmax), or, in a tile that takes
+        // two exponentials, 0 or -inf in the place of r.  Fetched by asynchronous copies three tiles ahead.
+        constexpr int AH = RING - 1;
+        auto fetch = [&](int i) {
+            float *at = ring + (i % RING) * 2 * kTile;
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) ptx::mma_ss(col, ptx::desc(ad + 2 * k, HI), ptx::desc(lat + 2 * k, HI), idescS, k > 0 || more);
+            for (int e = 0; e < kTile / 32; ++e) {
+                const int r = e * 32 + lane, n = min((int)(blockIdx.x + i * gridDim.x) * kTile + r, a.N - 1);
+                ptx::copy_async4(ptx::smem_u32(at + r), a.lse_dec + ((size_t)b * a.N + n) * a.H + h);
+            }
+        };
+        for (int k = 0; k < AH; ++k) {
+            if (k < nt) fetch(k);
+            ptx::copy_async_commit();
+        }
+        for (int i = 0; i < nt; ++i) {
+            ptx::copy_async_wait<AH - 1>();
+            __syncwarp();
+            float *at = ring + (i % RING) * 2 * kTile;
+            float ld[kTile / 32];
+            bool part[kTile / 32], far = unfolded != 0.f;
+#pragma unroll
+            for (int e = 0; e < kTile / 32; ++e) {
+                const int r = e * 32 + lane, n = (int)(blockIdx.x + i * gridDim.x) * kTile + r;
+                const bool in = n < a.N;
+                ld[e] = in ? at[r] * kBwdLog2e : INFINITY;
+                part[e] = in && (a.key_mask == nullptr || a.key_mask[(size_t)b * a.N + n] != 0);
+                at[r] = -ld[e];
+                far = far || (part[e] && !(ld[e] - K <= kFarLog2));
+            }
+            far = __any_sync(0xffffffffu, far);
+#pragma unroll
+            for (int e = 0; e < kTile / 32; ++e)
+                at[kTile + e * 32 + lane] = far ? (part[e] ? 0.f : -INFINITY) : (part[e] ? ptx::ex2(ld[e] - K) : 0.f);
+            if (lane == 0) two_exp[i % RING] = far ? 1u : 0u;
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar(C_FULL + i % RING));
+            const int next = i + AH;
+            if (next < nt) {
+                if (!warp_wait(bar(C_EMPTY + next % RING), ((next / RING) & 1) ^ 1, abort_flag, kErrBwdTok | 2)) break;
+                fetch(next);
+            }
+            ptx::copy_async_commit();
+        }
+        ptx::copy_async_wait<0>();
+    } else if (warp == 1) {
+        if (ptx::elect_one()) {
+            // (descriptors as 32-bit low words beside a constant high word: see ptx::desc)
+            constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), TILE = G::TILE_BYTES >> 4, STEP16 = (16 * G::RB) >> 4;
+            const uint32_t LAT = (uint32_t)(M * G::RB) >> 4;    // from one latent operand to the next
+            const uint32_t lat0 = ptx::desc_lo(ptx::smem_u32(smem + SM::lat_off(stages, M, 0)), 16), td0 = ptx::desc_lo(ptx::smem_u32(smem), 16);
+            // K-major to MN-major; the second block along N of [c dZ hi | Q] is one operand further on (LBO, bits 16-29)
+            constexpr uint32_t MN = ptx::desc_lo(0, G::SBO) - ptx::desc_lo(0, 16);
+            const uint32_t MN2 = (LAT << 16) - ptx::desc_lo(0, 16);
+            const int units = nu * nt;
+            int s_stage = 0, s_wrap = 0, s_u = 0, o_u = 0, o_tile = 0, o_acc = 0, o_wrap = 0;
+            bool o_two = false;
+            // S^T = K Q^T | A^T = dY Z^T | C'^T = V (c dZ)^T of the next unit, into buffer n & 1
+            auto tiles = [&](int n) -> bool {
+                if (s_u == 0) {
+                    if (!ptx::mbar_wait(bar(T_FULL + s_stage), (uint32_t)s_wrap, abort_flag, kErrBwdTok | 3)) return false;
+                    ptx::tc_fence_after();
+                }
+                const uint32_t idescS = ptx::instr_desc_bf16(128, 0, 0, 0) | (uint32_t)((s_u == nu - 1 ? wlast : UNIT) >> 3) << 17;
+                uint32_t td = td0 + (uint32_t)s_stage * 3 * TILE, ld = lat0 + (uint32_t)s_u * (UNIT / 16) * STEP16;
+                ptx::opaque(td);
+                ptx::opaque(ld);
+                const uint32_t bcol = tm + (n & 1) * bcols;
+                auto product = [&](int of, int lat, bool more) {   // of: S, A or C
+                    const uint32_t col = bcol + of * ucols, ad = td + (of == 0 ? 0 : of == 1 ? 2 * TILE : TILE), bd = ld + lat * LAT;
+#pragma unroll
+                    for (int k = 0; k < D / 16; ++k) ptx::mma_ss(col, ptx::desc(ad + 2 * k, HI), ptx::desc(bd + 2 * k, HI), idescS, k > 0 || more);
+                };
+                product(0, SM::QR, false);
+                if (D == 64 && third) product(1, SM::Z3, false);   // (small parts first: fewer sums are truncated at their full size)
+                product(1, SM::ZL, D == 64 && third);
+                product(1, SM::ZH, true);
+                product(2, SM::DL, false);
+                product(2, SM::DH, true);
+                ptx::mma_commit(bar(S_FULL + (n & 1)));
+                if (++s_u == nu) {
+                    ptx::mma_commit(bar(T_EMPTY + s_stage));
+                    s_u = 0;
+                    if (++s_stage == stages) { s_stage = 0; s_wrap ^= 1; }
+                }
+                return true;
             };
-            product(0, ld, false);                              // K with Q; dY with the parts of Z; V with dZ hi, lo
-            if (D == 64 && !kSecond) {
-                if (third) product(1, ld + 5 * LAT, false);     // (small parts first: fewer sums are truncated at their full size)
-                product(1, ld + 2 * LAT, third);
-                product(1, ld + LAT, true);
-            } else {
-                product(1, ld + LAT, false);
-                product(1, ld + 2 * LAT, true);
-            }
-            if (kSecond) {
-                product(2, ld + 3 * LAT, false);
-                product(2, ld + 4 * LAT, true);
-            }
-        };
-        // by one thread: dK += dS Q_unit, dV += W_enc dZ_unit
-        auto issue_outputs = [&](int u) {
-            constexpr uint32_t idescO = ptx::instr_desc_bf16(128, D, 0, 1);
-            const uint32_t ld = lat_desc(u), qd = ld + MN, zd = ld + 3 * LAT + MN, zl = ld + 4 * LAT + MN;
+            // [dV | U] += W_dec [c dZ | Q], T += dS Q of unit o_u (kTwo: dV += W_enc (c dZ))
+            auto outputs = [&](int n) {
+                constexpr uint32_t idesc1 = ptx::instr_desc_bf16(128, D, 0, 1), idesc2 = ptx::instr_desc_bf16(128, 2 * D, 0, 1);
+                const uint32_t bcol = tm + (n & 1) * bcols, V = tm + acc0 + o_acc * SM::kAccStride, U = V + D, T = V + 2 * D;
+                uint32_t ld = lat0 + (uint32_t)o_u * (UNIT / 16) * STEP16;
+                ptx::opaque(ld);
+                const int steps = (o_u == nu - 1 ? wlast : UNIT) / 16;
+                auto step = [&](auto two, int k) {
+                    constexpr bool kTwo = decltype(two)::value;
+                    const uint32_t acc = (o_u > 0 || k > 0) ? 1u : 0u, s = bcol + 16 * k, w = s + ucols, e = w + ucols;   // (hi, and lo 8 columns on)
+                    const uint32_t qd = ld + SM::QR * LAT + MN + k * STEP16, dl = ld + SM::DL * LAT + MN + k * STEP16, dh = ld + SM::DH * LAT + k * STEP16;
+                    if constexpr (!kTwo) {
+                        ptx::mma_ts(V, w, ptx::desc(dh + MN2, HI), idesc2, acc);
+                        ptx::mma_ts(V, w + 8, ptx::desc(dh + MN2, HI), idesc2, 1u);
+                        ptx::mma_ts(V, w, ptx::desc(dl, HI), idesc1, 1u);
+                    } else {
+                        ptx::mma_ts(V, e, ptx::desc(dh + MN, HI), idesc1, acc);
+                        ptx::mma_ts(V, e + 8, ptx::desc(dh + MN, HI), idesc1, 1u);
+                        ptx::mma_ts(V, e, ptx::desc(dl, HI), idesc1, 1u);
+                        ptx::mma_ts(U, w, ptx::desc(qd, HI), idesc1, acc);
+                        ptx::mma_ts(U, w + 8, ptx::desc(qd, HI), idesc1, 1u);
+                    }
+                    ptx::mma_ts(T, s, ptx::desc(qd, HI), idesc1, acc);
+                    ptx::mma_ts(T, s + 8, ptx::desc(qd, HI), idesc1, 1u);
+                };
+                if (!o_two) {
+                    if (steps == UNIT / 16) {
 #pragma unroll
-            for (int k = 0; k < UNIT / 16; ++k) {
-                if (k > 0 && u == nu - 1 && 16 * k >= wlast) break;
-                const uint32_t acc = (u > 0 || k > 0) ? 1u : 0u;
-                ptx::mma_ts(base + K_COL, base + 16 * k, ptx::desc(qd + k * STEP16, HI), idescO, acc);                    // dS hi
-                ptx::mma_ts(base + K_COL, base + UNIT + 16 * k, ptx::desc(qd + k * STEP16, HI), idescO, 1u);              // dS lo
-                ptx::mma_ts(base + V_COL, base + 2 * UNIT + 16 * k, ptx::desc(zd + k * STEP16, HI), idescO, acc);         // W_enc hi x dZ hi
-                ptx::mma_ts(base + V_COL, base + 2 * UNIT + 16 * k, ptx::desc(zl + k * STEP16, HI), idescO, 1u);          // W_enc hi x dZ lo
-                ptx::mma_ts(base + V_COL, base + 16 * k + 8, ptx::desc(zd + k * STEP16, HI), idescO, 1u);                 // W_enc lo x dZ hi
+                        for (int k = 0; k < UNIT / 16; ++k) step(std::false_type{}, k);
+                    } else {
+                        for (int k = 0; k < steps; ++k) step(std::false_type{}, k);
+                    }
+                } else {
+                    for (int k = 0; k < steps; ++k) step(std::true_type{}, k);
+                }
+            };
+            bool ok = true;
+            for (int n = 0; ok && n < 2 && n < units; ++n) ok = tiles(n);
+            for (int n = 0; ok && n < units; ++n) {
+                if (!ptx::mbar_wait(bar(P_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdTok | 4)) break;
+                if (o_u == 0) {
+                    const int c = o_tile % RING;
+                    if (!ptx::mbar_wait(bar(C_FULL + c), (o_tile / RING) & 1, abort_flag, kErrBwdTok | 5)) break;
+                    o_two = two_exp[c] != 0;
+                    ptx::mbar_arrive(bar(C_EMPTY + c));
+                    if (!ptx::mbar_wait(bar(ACC_EMPTY + o_acc), (uint32_t)o_wrap ^ 1u, abort_flag, kErrBwdTok | 6)) break;
+                }
+                ptx::tc_fence_after();
+                outputs(n);
+                if (++o_u == nu) {
+                    ptx::mma_commit(bar(ACC_FULL + o_acc));
+                    o_u = 0;
+                    ++o_tile;
+                    if (++o_acc == 1 << log_accs) { o_acc = 0; o_wrap ^= 1; }
+                }
+                if (n + 2 < units) ok = tiles(n + 2);
             }
-        };
-        // by one thread: the first unit of tile i (of the CTA)
-        auto open_tile = [&](int i) -> bool {
-            if (!ptx::mbar_wait(bar(T_FULL + i % stages), (i / stages) & 1, abort_flag, kErrBwdTok | 3)) return false;
-            if (kMode == 2) issue_tiles(std::true_type{}, i % stages, 0);
-            else issue_tiles(std::false_type{}, i % stages, 0);
-            return true;
-        };
-        // by one thread: tile i has been read for the last time; on to the group's next
-        auto close_tile = [&](int i) -> bool {
-            ptx::mbar_arrive(bar(T_EMPTY + i % stages));
-            return i + NG >= nt || open_tile(i + NG);
-        };
-        bool ok = true;
-        uint32_t n = 0;                                         // units waited for
-        auto token_of = [&](int i) { return (int)(blockIdx.x + i * gridDim.x) * kTile + row; };   // of this lane in tile i
-        // One row of dK (which = 0) or dV (1) of token tok_n, from this thread's lane of the accumulators.
-        auto write_row = [&](int which, int tok_n) {
-            constexpr int LW = DR >= 16 ? DR : 8;               // columns loaded (narrow heads: within the first 8)
-            const uint32_t col = gcol + (which ? V_COL : K_COL);
-            const size_t tok = ((size_t)b * a.N + (tok_n < a.N ? tok_n : 0)) * a.H + h;
-            __nv_bfloat16 *out = which ? a.dV : a.dK;
-            float4 *sum = reinterpret_cast<float4 *>(a.kvacc + ((size_t)which * a.B * a.N * a.H + tok) * DR);
-            const float sc = which ? 1.f : a.scale;
-#pragma unroll
-            for (int c0 = 0; c0 < LW; c0 += 8) {
-                uint32_t x[8];
-                ptx::tmem_ld8(col + c0, x);
+        }
+    } else if (warp >= kTokFirstMathWarp) {
+        const int cg = (warp - kTokFirstMathWarp) >> 2, set = sets == 2 ? cg >> 1 : 0, mine = sets == 2 ? cg & 1 : cg;   // columns: 16 from 16 mine on
+        const int row = ((warp & 3) << 5) + lane;               // TMEM lane = token within the tile
+        const uint32_t gcol = tm + ((uint32_t)((warp & 3) << 5) << 16);
+        const float2 sl2p = make_float2(a.sl2, a.sl2);
+        const float *nle = cst + 16 * mine, *nde = nle + M;
+        // Rows of dK and dV of the set's k-th tile: pieces of eight columns, in turn to the warps that share the tokens.
+        auto write_rows = [&](int k, float r) -> bool {
+            constexpr int COLS = DR >= 16 ? DR : 8, PIECES = COLS / 4, PW = DR == 4 ? 4 : 8;
+            const int i = set + k * sets, acc = i & ((1 << log_accs) - 1), tok_n = (int)(blockIdx.x + i * gridDim.x) * kTile + row;
+            const bool in = tok_n < a.N;
+            const size_t tok = ((size_t)b * a.N + (in ? tok_n : 0)) * a.H + h;
+            const uint32_t V = gcol + acc0 + acc * SM::kAccStride;
+            if (!warp_wait(bar(DD_FULL + (k & 3) + 4 * set), (k >> 2) & 1, abort_flag, kErrBwdTok | 7)) return false;
+            if (!warp_wait(bar(ACC_FULL + acc), (i >> log_accs) & 1, abort_flag, kErrBwdTok | 8)) return false;
+            ptx::tc_fence_after();
+            const size_t plane = (size_t)a.B * a.N * a.H * DR;  // of the sums over ranges
+#pragma unroll 1
+            for (int p = PIECES <= 2 ? (mine + 2 * k) & (cps - 1) : mine; p < PIECES; p += cps) {
+                const int which = (p ^ (p >> 2)) & 1, c0 = (p >> 1) * 8;   // dK or dV, and the first column
+                uint32_t x[8], y[8];
+                float dd = 0.f;
+                ptx::tmem_ld8(V + (which == 0 ? 2 * D : 0) + c0, x);
+                if (which == 0) {
+                    ptx::tmem_ld8(V + D + c0, y);
+                    const float *part = dds + ((k & 3) * NCG + set * cps) * kTile + row;
+                    dd = part[0] + part[kTile];
+                    if (cps == 4) dd += part[2 * kTile] + part[3 * kTile];
+                    const size_t at = ((size_t)b * a.H + h) * a.N + (in ? tok_n : 0);
+                    if (kRanges && !a.first) dd += a.dd_sums[at];
+                    if (in && c0 == 0) a.dd[at] = dd;
+                }
                 ptx::tmem_wait_ld();
-                constexpr int PW = DR == 4 ? 4 : 8;             // columns written
-                float f[PW];
+                float f[PW], u[PW];
 #pragma unroll
-                for (int c = 0; c < PW; ++c) f[c] = __uint_as_float(DR == 4 && off != 0 ? x[(4 + c) & 7] : x[c]);   // the head's columns
-                if (tok_n < a.N) {
-                    if (kMode == 2) {
+                for (int c = 0; c < PW; ++c) {                  // (narrow heads: the head's own columns)
+                    f[c] = __uint_as_float(DR == 4 && off != 0 ? x[(4 + c) & 7] : x[c]);
+                    u[c] = which == 0 ? __uint_as_float(DR == 4 && off != 0 ? y[(4 + c) & 7] : y[c]) : 0.f;
+                    if (which != 0) f[c] *= r;
+                }
+                if (in && kRanges) {
+                    auto sums = [&](int at, float *v) {
+                        float4 *sum = reinterpret_cast<float4 *>(a.kvacc + at * plane + tok * DR + c0);
 #pragma unroll
                         for (int c = 0; c < PW; c += 4) {       // the earlier ranges' shares
-                            float4 &at = sum[(c0 + c) / 4];
                             if (!a.first) {
-                                const float4 e = at;
-                                f[c] += e.x; f[c + 1] += e.y; f[c + 2] += e.z; f[c + 3] += e.w;
+                                const float4 e = sum[c / 4];
+                                v[c] += e.x; v[c + 1] += e.y; v[c + 2] += e.z; v[c + 3] += e.w;
                             }
-                            if (!a.last) at = make_float4(f[c], f[c + 1], f[c + 2], f[c + 3]);
+                            if (!a.last) sum[c / 4] = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
                         }
-                    }
-                    if (kMode != 2 || a.last) {
-                        uint32_t w[PW / 2];
-#pragma unroll
-                        for (int c = 0; c < PW / 2; ++c) w[c] = ptx::pack_bf16(f[2 * c] * sc, f[2 * c + 1] * sc);
-                        if constexpr (PW == 4) *reinterpret_cast<uint2 *>(out + tok * DR) = make_uint2(w[0], w[1]);
-                        else *reinterpret_cast<uint4 *>(out + tok * DR + c0) = make_uint4(w[0], w[1], w[2], w[3]);
-                    }
-                }
-                __syncwarp();
-            }
-        };
-        // Second sweep over the latents of tile i: dS^T and W_enc^T of every unit; the unit after the tile's last is the group's next tile's first.
-        auto sweep2 = [&](auto two, int i, float nld, float fct, float dd) -> bool {
-            constexpr bool kTwo = decltype(two)::value;
-            const float2 nldp = make_float2(nld, nld), fctp = make_float2(fct, fct), nddp = make_float2(-dd, -dd);
-#pragma unroll 1
-            for (int u = 0; u < nu; ++u, ++n) {
-                if (!warp_wait(sfull, n & 1, abort_flag, kErrBwdTok | 7)) return false;
-                ptx::tc_fence_after();
-#pragma unroll 1
-                for (int q = 0; q < UNIT; q += 16) {            // 16 latents at a time
-                    if (u * UNIT + q >= M) break;
-                    const float *le_at = cst + (kTwo ? 0 : 2 * M) + u * UNIT + q, *de_at = cst + M + u * UNIT + q;
-                    // the second eight columns on their way while the first are worked on: 2 % at D = 16 without padding, 4 % lost where
-                    // it costs the padded form registers, nothing at D = 32 and 64
-                    constexpr bool kPf = D == 16 && !kPadded;
-                    uint32_t wl0[4], ss[2][8], aa[2][8], cc[2][8];
-                    auto load = [&](int p, int to) {
-                        ptx::tmem_ld8(gcol + q + p * 8, ss[to]);
-                        ptx::tmem_ld8(gcol + UNIT + q + p * 8, aa[to]);
-                        ptx::tmem_ld8(gcol + 2 * UNIT + q + p * 8, cc[to]);
                     };
-                    if (kPf) {
-                        load(0, 0);
-                        ptx::tmem_wait_ld();
-                        load(1, 1);
-                    }
-#pragma unroll
-                    for (int p = 0; p < 2; ++p) {
-                        uint32_t hi[4], lo[4], wh[4], wl[4];
-                        uint32_t (&s)[8] = ss[kPf ? p : 0], (&av)[8] = aa[kPf ? p : 0], (&cv)[8] = cc[kPf ? p : 0];
-                        if (!kPf) {
-                            load(p, 0);
-                            ptx::tmem_wait_ld();
-                        }
-#pragma unroll
-                        for (int k = 0; k < 4; k += 2) {
-                            const float4 le = *reinterpret_cast<const float4 *>(le_at + p * 8 + 2 * k);
-                            const float4 nd = *reinterpret_cast<const float4 *>(de_at + p * 8 + 2 * k);
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const int j = 2 * (k + e);
-                                const DsPair r = ds_pair<true, kTwo, false>(
-                                    make_float2(__uint_as_float(s[j]), __uint_as_float(s[j + 1])), make_float2(__uint_as_float(av[j]), __uint_as_float(av[j + 1])),
-                                    make_float2(__uint_as_float(cv[j]), __uint_as_float(cv[j + 1])), sl2p, nldp, nddp,
-                                    e ? make_float2(nd.z, nd.w) : make_float2(nd.x, nd.y), e ? make_float2(le.z, le.w) : make_float2(le.x, le.y), fctp);
-                                hi[k + e] = r.hi; lo[k + e] = r.lo; wh[k + e] = r.whi; wl[k + e] = r.wlo;
-                            }
-                        }
-                        if (kPf && p == 0) ptx::tmem_wait_ld();
-                        // over columns this thread has read, 8 packed columns per array: dS hi and W_enc lo over S, dS lo over A, W_enc hi over C
-                        ptx::tmem_st4(gcol + q + p * 4, hi);
-                        ptx::tmem_st4(gcol + UNIT + q + p * 4, lo);
-                        ptx::tmem_st4(gcol + 2 * UNIT + q + p * 4, wh);
-                        if (p == 0) {
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) wl0[k] = wl[k];
-                        } else {
-                            ptx::tmem_st4(gcol + q + 8, wl0);
-                            ptx::tmem_st4(gcol + q + 12, wl);
-                        }
-                    }
+                    sums(which, f);
+                    if (which == 0) sums(2, u);
                 }
-                ptx::tmem_wait_st();
-                if (hand_over(pfull, n, abort_flag, kErrBwdTok | 4) && ptx::elect_one()) {
-                    issue_outputs(u);
-                    bool go = true;
-                    if (u + 1 < nu) issue_tiles(std::true_type{}, i % stages, u + 1);
-                    else go = close_tile(i);
-                    if (go) ptx::mma_commit(sfull);
+                if (in && (!kRanges || a.last)) {
+                    const float sc = which == 0 ? a.scale : 1.f;
+                    uint32_t w[PW / 2];
+#pragma unroll
+                    for (int c = 0; c < PW / 2; ++c)
+                        w[c] = ptx::pack_bf16(fmaf(-dd, u[2 * c], f[2 * c]) * sc, fmaf(-dd, u[2 * c + 1], f[2 * c + 1]) * sc);
+                    __nv_bfloat16 *out = (which ? a.dV : a.dK) + tok * DR + c0;
+                    if constexpr (PW == 4) *reinterpret_cast<uint2 *>(out) = make_uint2(w[0], w[1]);
+                    else *reinterpret_cast<uint4 *>(out) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
                 __syncwarp();
             }
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar(ACC_EMPTY + acc));
             return true;
         };
-        // this lane's token of a tile: its decode log-sum-exp and mask byte, fetched one tile ahead
-        float f_ld = 0.f, f_dd = 0.f;
-        uint32_t f_mask = 1u;
-        auto fetch = [&](int i) {
-            const int t = token_of(i);
-            const size_t nn = (size_t)b * a.N + (t < a.N ? t : 0);
-            f_ld = a.lse_dec[nn * a.H + h];
-            if (kPadded) f_mask = a.key_mask == nullptr ? 1u : (uint32_t)a.key_mask[nn];
-            if (kMode == 2) f_dd = a.dd[((size_t)b * a.H + h) * a.N + (t < a.N ? t : 0)];
-        };
-        if (g < nt) {
-            fetch(g);
-            if ((warp & 3) == 0 && ptx::elect_one() && open_tile(g)) ptx::mma_commit(sfull);
-            __syncwarp();
-        }
-        for (int i = g; ok && i < nt; i += NG) {
-            const int tok_n = token_of(i);
-            const bool inside = tok_n < a.N;
-            const float nld = inside ? -f_ld * kBwdLog2e : -INFINITY;
-            const bool part = inside && (!kPadded || f_mask != 0);   // the token takes part in the encode softmax
-            float dd = inside ? f_dd : 0.f;                     // mode 2: over all latents, from the workspace
-            if (i + NG < nt) fetch(i + NG);
-            if (kMode != 2) {
-                // first sweep: dd[n] = sum_m W_dec[n,m] (dY_n . Z_m)
-                const float2 nldp = make_float2(nld, nld);
-                float2 d2 = make_float2(0.f, 0.f);
-#pragma unroll 1
-                for (int u = 0; u < nu; ++u, ++n) {
-                    if (!(ok = warp_wait(sfull, n & 1, abort_flag, kErrBwdTok | 6))) break;
-                    ptx::tc_fence_after();
-                    uint32_t x[16], av[16];
-                    auto add = [&]() {
+        // Sixteen columns of a unit, over which its weights go: dS over S, W_dec over A, W_enc (kTwo) over C, hi and lo of 16 latents side by side.
+        auto unit = [&](auto two, uint32_t col, int m, float2 nldp, float2 rp, float2 &d2) {
+            constexpr bool kTwo = decltype(two)::value;
+            uint32_t s[2][8], av[2][8], cv[2][8];
+            auto load = [&](int p) {
+                ptx::tmem_ld8(col + 8 * p, s[p]);
+                ptx::tmem_ld8(col + ucols + 8 * p, av[p]);
+                ptx::tmem_ld8(col + 2 * ucols + 8 * p, cv[p]);
+            };
+            load(0);
+            ptx::tmem_wait_ld();
+            load(1);                                            // eight columns on their way while eight are worked on
 #pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const float2 e = __ffma2_rn(make_float2(__uint_as_float(x[2 * k]), __uint_as_float(x[2 * k + 1])), sl2p, nldp);
-                            d2 = __ffma2_rn(make_float2(ptx::ex2(e.x), ptx::ex2(e.y)),
-                                            make_float2(__uint_as_float(av[2 * k]), __uint_as_float(av[2 * k + 1])), d2);
+            for (int p = 0; p < 2; ++p) {
+                uint32_t hi[4], lo[4], wh[4], wl[4], eh[4], el[4];
+#pragma unroll
+                for (int q = 0; q < 4; q += 2) {
+                    const float4 ne = *reinterpret_cast<const float4 *>(nde + m + 8 * p + 2 * q);
+                    float4 le = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (kTwo) le = *reinterpret_cast<const float4 *>(nle + m + 8 * p + 2 * q);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int j = 2 * (q + e), o = q + e;
+                        const float2 sv = make_float2(__uint_as_float(s[p][j]), __uint_as_float(s[p][j + 1]));
+                        const float2 A = make_float2(__uint_as_float(av[p][j]), __uint_as_float(av[p][j + 1]));
+                        const float2 C = make_float2(__uint_as_float(cv[p][j]), __uint_as_float(cv[p][j + 1]));
+                        const float2 x = __ffma2_rn(sv, sl2p, nldp);
+                        const float2 pd = make_float2(ptx::ex2(x.x), ptx::ex2(x.y));
+                        const float2 v = __fadd2_rn(C, e ? make_float2(ne.z, ne.w) : make_float2(ne.x, ne.y));
+                        float2 ds;
+                        if (kTwo) {
+                            const float2 y = __ffma2_rn(sv, sl2p, __fadd2_rn(e ? make_float2(le.z, le.w) : make_float2(le.x, le.y), rp));
+                            const float2 pe = make_float2(ptx::ex2(y.x), ptx::ex2(y.y));
+                            ds = __ffma2_rn(pd, A, __fmul2_rn(pe, v));
+                            eh[o] = ptx::pack_bf16(pe);
+                            el[o] = ptx::pack_bf16(ptx::rest_of(pe, eh[o]));
+                        } else {
+                            ds = __fmul2_rn(pd, __ffma2_rn(rp, v, A));
                         }
-                    };
-                    const bool both = u * UNIT + 16 < M;
-                    ptx::tmem_ld16(gcol, x);
-                    ptx::tmem_ld16(gcol + UNIT, av);
-                    ptx::tmem_wait_ld();
-                    if (both) {
-                        add();
-                        ptx::tmem_ld16(gcol + 16, x);
-                        ptx::tmem_ld16(gcol + UNIT + 16, av);
-                        ptx::tmem_wait_ld();
+                        d2 = __ffma2_rn(pd, A, d2);
+                        hi[o] = ptx::pack_bf16(ds);
+                        lo[o] = ptx::pack_bf16(ptx::rest_of(ds, hi[o]));
+                        wh[o] = ptx::pack_bf16(pd);
+                        wl[o] = ptx::pack_bf16(ptx::rest_of(pd, wh[o]));
                     }
-                    // the buffer has been read: the next unit's tiles run under the second half's exponentials
-                    if (hand_over(pfull, n, abort_flag, kErrBwdTok | 4) && ptx::elect_one()) {
-                        bool go = true;
-                        if (u + 1 < nu) issue_tiles(std::false_type{}, i % stages, u + 1);
-                        else if (kMode == 0) issue_tiles(std::true_type{}, i % stages, 0);
-                        else go = close_tile(i);
-                        if (go) ptx::mma_commit(sfull);
-                    }
+                }
+                if (p == 0) ptx::tmem_wait_ld();                // (all sixteen have been read)
+                ptx::tmem_st4(col + 4 * p, hi);
+                ptx::tmem_st4(col + 8 + 4 * p, lo);
+                ptx::tmem_st4(col + ucols + 4 * p, wh);
+                ptx::tmem_st4(col + ucols + 8 + 4 * p, wl);
+                if (kTwo) {
+                    ptx::tmem_st4(col + 2 * ucols + 4 * p, eh);
+                    ptx::tmem_st4(col + 2 * ucols + 8 + 4 * p, el);
+                }
+            }
+            ptx::tmem_wait_st();
+        };
+        // All units of the set's tiles in one loop; one more turn writes the last tile's rows.
+        int k = 0, u = 0;                                       // tiles of this set done, unit of the next
+        float nld = 0.f, rr = 0.f, r_before = 0.f;
+        bool far = false;
+        float2 d2 = make_float2(0.f, 0.f);
+        while (true) {
+            const int i = set + k * sets;
+            if (i < nt) {
+                if (u == 0) {
+                    const int c = i % RING;
+                    if (!warp_wait(bar(C_FULL + c), (i / RING) & 1, abort_flag, kErrBwdTok | 9)) break;
+                    nld = ring[c * 2 * kTile + row];
+                    rr = ring[(c * 2 + 1) * kTile + row];
+                    far = two_exp[c] != 0;
+                    d2 = make_float2(0.f, 0.f);
                     __syncwarp();
-                    add();
+                    if (lane == 0) ptx::mbar_arrive(bar(C_EMPTY + c));
                 }
-                if (!ok) break;
-                dd = d2.x + d2.y;
-                if (inside) {
-                    float *at = a.dd + ((size_t)b * a.H + h) * a.N + tok_n;
-                    *at = kMode == 1 && !a.first ? *at + dd : dd;
-                }
-            }
-            if (kMode != 1) {
-                if (i > g && kMode == 0) {                      // the previous tile's rows
-                    write_row(0, token_of(i - NG));
-                    write_row(1, token_of(i - NG));
-                }
-                const bool far = __any_sync(0xffffffffu, part && !(-nld - lse_min <= kOneExpLog2));
-                // this token's factor of W_enc, or (far) the addend of its exponent
-                const float fct = far ? (part ? 0.f : -INFINITY) : (part ? ptx::ex2(-nld - lse_min) : 0.f);
-                ok = far ? sweep2(std::true_type{}, i, nld, fct, dd) : sweep2(std::false_type{}, i, nld, fct, dd);
-                if (!ok) break;
-            }
-            // mode 2 has no first sweep under which a tile's last contractions would finish: its rows are written right away
-            const bool done = i + NG >= nt;
-            if ((done && kMode == 0) || kMode == 2) {
-                if (!(ok = warp_wait(sfull, n & 1, abort_flag, kErrBwdTok | 8))) break;
+                const int n = i * nu + u;
+                const uint32_t col = gcol + (n & 1) * bcols + 16 * mine;
+                if (!warp_wait(bar(S_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdTok | 10)) break;
                 ptx::tc_fence_after();
-                write_row(0, tok_n);
-                write_row(1, tok_n);
+                if (u * UNIT + 16 * mine < M) {
+                    if (far) unit(std::true_type{}, col, u * UNIT, make_float2(nld, nld), make_float2(rr, rr), d2);
+                    else unit(std::false_type{}, col, u * UNIT, make_float2(nld, nld), make_float2(rr, rr), d2);
+                }
+                if (u == nu - 1) dds[((k & 3) * NCG + cg) * kTile + row] = d2.x + d2.y;
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    ptx::mbar_arrive(bar(P_FULL + (n & 1)));
+                    if (u == nu - 1) ptx::mbar_arrive(bar(DD_FULL + (k & 3) + 4 * set));
+                }
+            }
+            if (u == 0 && k > 0 && !write_rows(k - 1, r_before)) break;
+            if (i >= nt) break;
+            if (++u == nu) {
+                u = 0;
+                ++k;
+                r_before = far ? 1.f : rr;
             }
         }
     }

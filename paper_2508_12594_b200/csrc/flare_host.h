@@ -347,13 +347,13 @@ inline TcEncodePlan tc_dq_plan(const flare_desc_t *d, int sms) {
 inline SimtPlan bwd_dq_plan(const flare_desc_t *d, int sms) { return simt_plan_for(d, sms, d->D <= 16 ? 2 : 1); }
 
 struct BwdLayout {
-    size_t part, dz, de, dd, kvacc, total;
+    size_t part, dz, de, dd, dd_other, kvacc, total;
     int P;
 };
 
-// Latents one launch of the tensor-core token kernel takes: five operands of D-wide bf16 rows (six at D = 64 up to 160 latents) beside a tile stage per group (four groups at
-// D <= 16, three at 32, two at 64); more are worked off in ranges of equal size.
-inline int token_range_most(const flare_desc_t *d) { return d->D == 64 ? 192 : d->D == 32 ? 448 : 1024; }
+// Latents one launch of the tensor-core token kernel takes: five operands of D-wide bf16 rows (six at D = 64 up to 160 latents) beside two
+// tile stages; more are worked off in ranges of equal size.
+inline int token_range_most(const flare_desc_t *d) { return d->D == 64 ? 192 : d->D == 32 ? 512 : 1024; }
 inline bool token_in_ranges(const flare_desc_t *d) { return use_tc(d) && d->M > token_range_most(d); }
 inline int token_ranges(const flare_desc_t *d) { return (d->M + token_range_most(d) - 1) / token_range_most(d); }
 inline int token_range(const flare_desc_t *d) { return ((d->M + token_ranges(d) - 1) / token_ranges(d) + 15) / 16 * 16; }
@@ -369,8 +369,11 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     w.dz = off;   off += align_up(sizeof(float) * (size_t)rows * d->D);
     w.de = off;   off += align_up(sizeof(float) * (size_t)rows);
     w.dd = off;   off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
-    w.kvacc = off;                                             // float32 sums of the rows of dK and dV over latent ranges
-    if (token_in_ranges(d)) off += align_up(sizeof(float) * 2 * (size_t)d->B * d->N * d->H * d->D);
+    w.dd_other = w.kvacc = off;                                // over latent ranges: dd so far, and float32 sums of the rows
+    if (token_in_ranges(d)) {
+        w.kvacc = off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
+        off += align_up(sizeof(float) * 3 * (size_t)d->B * d->N * d->H * d->D);
+    }
     w.total = off;
     return w;
 }

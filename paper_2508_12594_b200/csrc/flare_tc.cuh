@@ -81,12 +81,20 @@ __device__ __forceinline__ void stage_rows4(uint8_t *dst, const __nv_bfloat16 *s
         *reinterpret_cast<uint2 *>(dst + (size_t)m * G::RB + (G::swz(m) << 4) + off * 2) =
             *reinterpret_cast<const uint2 *>(src + (size_t)m * 4);
 }
-// rows of a [rows, 4] float matrix -> two bf16 halves (hi = round(z), lo = round(z - hi)) at columns [off, off + 4)
-template <int D>
-__device__ __forceinline__ void stage_rows4_hilo(uint8_t *dst_hi, uint8_t *dst_lo, const float *src, int rows, int off) {
+// rows of a [rows, 4] float matrix less `centre` (null: nothing), each times its factor -> two bf16 halves (hi = round(z), lo = round(z - hi)) at columns [off, off + 4)
+struct UnitFactor {
+    __device__ __forceinline__ float operator()(int) const { return 1.f; }
+};
+template <int D, class Factor = UnitFactor>
+__device__ __forceinline__ void stage_rows4_hilo(uint8_t *dst_hi, uint8_t *dst_lo, const float *src, int rows, int off, const float *centre = nullptr,
+                                                 Factor factor = Factor()) {
     using G = TileGeom<D>;
+    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (centre != nullptr) c = *reinterpret_cast<const float4 *>(centre);
     for (int m = threadIdx.x; m < rows; m += blockDim.x) {
-        const float4 z = *reinterpret_cast<const float4 *>(src + (size_t)m * 4);
+        float4 z = *reinterpret_cast<const float4 *>(src + (size_t)m * 4);
+        const float f = factor(m);
+        z = make_float4((z.x - c.x) * f, (z.y - c.y) * f, (z.z - c.z) * f, (z.w - c.w) * f);
         const uint32_t h0 = ptx::pack_bf16(z.x, z.y), h1 = ptx::pack_bf16(z.z, z.w);
         const uint32_t l0 = ptx::pack_bf16(z.x - __uint_as_float(h0 << 16), z.y - __uint_as_float(h0 & 0xffff0000u));
         const uint32_t l1 = ptx::pack_bf16(z.z - __uint_as_float(h1 << 16), z.w - __uint_as_float(h1 & 0xffff0000u));
