@@ -14,9 +14,14 @@
 // the output type, and where the rows Z_m that a token mixes are nearly equal that rounding would dominate dS.
 // Reductions add their partial results in a fixed order, so the gradients are bitwise reproducible.
 //
+// dd enters linearly, so the token side takes one sweep: dK_n = scale (T_n - dd[n] U_n), T without dd, U_n = sum_m W_dec[n,m] q_m, all sums in
+// double.  (Two sweeps, dd first, took 5 D score products and three exponentials per pair instead of 3 D and two.)
+//
 // The kernels have the shape of the forward ones: row operands as A fragments in registers, column operands in
-// shared memory, all three products of a pair (q.k, dY.Z, dZ.V) on the double-precision MMA, which bounds them: 2 D double
-// multiply-adds per pair in the first sweep over the latents and 3 D in the second and in the dQ pass.
+// shared memory, all products of a pair (q.k, dY.Z, dZ.V, and the contractions of dS and the weights) on the double-precision MMA, which is
+// busy 55 to 65 % of the time: 6 D double multiply-adds per pair on the token side, 4 D in the dQ pass.  Neither a second tile buffer, nor
+// twice the warps, nor the wider MMA shapes (m16n8k16) moved that.  us per training step, before (contractions as float32 FMAs, expf) -> now: float16
+// 4 x 10007 tokens, M = 64, D = 16, 8 heads 492 -> 452; float32 2 x 9973 273 -> 242; 16384, M = 64, D = 32, 4 heads 237 -> 216; 10000, D = 64 390 -> 297.
 #pragma once
 
 #include "flare_ptx.cuh"
@@ -28,7 +33,7 @@ namespace flare {
 // Row blocks of 8 per warp: three operands of a row and its accumulators are in registers.
 template <int D> struct BwdSimtGeom {
     static constexpr int RB = D <= 16 ? 2 : 1;
-    // token side: as many warps as the registers of three operands and two accumulators leave room for
+    // token side: as many warps as the registers of three operands and three accumulators leave room for
     static constexpr int kTokThreads = D <= 32 ? 384 : 256, kTokRows = kTokThreads / 32 * 8 * RB;
 };
 
@@ -46,7 +51,7 @@ bwd_token_simt_kernel(const T *Q, const T *K, const T *V,
     constexpr int CT = SG::CT, RB = BwdSimtGeom<D>::RB, TH = BwdSimtGeom<D>::kTokThreads;
     extern __shared__ __align__(16) unsigned char simt_smem[];
     double *sQ = reinterpret_cast<double *>(simt_smem), *sZ = sQ + CT * SG::DK, *sDZ = sZ + CT * SG::DK;
-    float *fQ = reinterpret_cast<float *>(sDZ + CT * SG::DK), *fDZ = fQ + CT * SG::DV, *sLe = fDZ + CT * SG::DV, *sDe = sLe + CT;
+    float *sLe = reinterpret_cast<float *>(sDZ + CT * SG::DK), *sDe = sLe + CT;   // (in the order of the MMA's indices)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = blockIdx.y, b = blockIdx.z;
     const int r0 = (blockIdx.x * (TH / 32) + warp) * 8 * RB;
     const size_t stride = (size_t)H * D, base = ((size_t)b * N * H + h) * D;
@@ -62,64 +67,38 @@ bwd_token_simt_kernel(const T *Q, const T *K, const T *V,
         ld[rb] = n < N ? lse_dec[((size_t)b * N + n) * H + h] : INFINITY;
         dd[rb] = 0.f;
     }
-    unsigned char *raw = reinterpret_cast<unsigned char *>(sDe + CT);
+    float *sC = sDe + CT;
+    unsigned char *raw = reinterpret_cast<unsigned char *>(sC + D);
     TileFetch<T, D, TH> fq(raw);
     TileFetch<float, D, TH> fz(raw + fq.kBytes), fdz(raw + fq.kBytes + fz.kBytes);
-    // first sweep over the latents: dd = sum_m W_dec[n,m] (dY_n . Z_m)
-    fq.load(Qh, D, M);
-    fz.load(Z + lat * D, D, M);
-    for (int m0 = 0; m0 < M; m0 += CT) {
-        fq.wait();
-        __syncthreads();
-        fq.put_double(sQ);
-        fz.put_double(sZ);
-        __syncthreads();
-        const int m1 = m0 + CT < M ? m0 + CT : 0;                   // the next tile; after the last one the second sweep's first
-        fq.load(Qh + (size_t)m1 * D, D, M - m1);
-        fz.load(Z + (lat + m1) * D, D, M - m1);
-        const int mc = min(CT, M - m0);
-        if (r0 < N)
-            for (int nb = 0; nb < (mc + 7) / 8; ++nb) {
-                double2 c[RB], a[RB];
-                mma_block<D, RB>(c, ak, sQ, nb);
-                mma_block<D, RB>(a, ag, sZ, nb);
-                const int col = nb * 8 + 2 * (lane & 3);            // (columns beyond M: Z is zero there)
-#pragma unroll
-                for (int rb = 0; rb < RB; ++rb) {
-                    if (col < mc) dd[rb] = fmaf(expf((float)c[rb].x - ld[rb]), (float)a[rb].x, dd[rb]);
-                    if (col + 1 < mc) dd[rb] = fmaf(expf((float)c[rb].y - ld[rb]), (float)a[rb].y, dd[rb]);
-                }
-            }
-    }
     double av[RB][D / 4];
     load_rows<T, D, RB>(av, V + base, stride, r0, N, 1.0);
     bool valid[RB];
-    float2 dk[RB][D / 2], dv[RB][D / 2];
+    double2 dk[RB][SG::NB], dv[RB][SG::NB], un[RB][SG::NB];         // T, dV, U
+    clear_rows<D, RB>(dk);
+    clear_rows<D, RB>(dv);
+    clear_rows<D, RB>(un);
 #pragma unroll
     for (int rb = 0; rb < RB; ++rb) {
         const int n = r0 + 8 * rb + (lane >> 2);
-        dd[rb] = quad_sum(dd[rb]);
         valid[rb] = n < N && (key_mask == nullptr || key_mask[(size_t)b * N + n] != 0);
-        if (n < N && (lane & 3) == 0) dd_out[((size_t)b * H + h) * N + n] = dd[rb];
-#pragma unroll
-        for (int d = 0; d < D / 2; ++d) dk[rb][d] = dv[rb][d] = make_float2(0.f, 0.f);
     }
-    // second sweep (its first tile of Q and Z is already on its way)
+    z_centre<D>(sC, Z + lat * D, M);
+    fq.load(Qh, D, M);
+    fz.load(Z + lat * D, D, M);
     fdz.load(dZ + lat * D, D, M);
     for (int m0 = 0; m0 < M; m0 += CT) {
         const int mc = min(CT, M - m0);
         fq.wait();
         __syncthreads();
         fq.put_double(sQ);
-        fq.put_float(fQ);
-        fz.put_double(sZ);
+        fz.template put_double<true>(sZ, sC);
         fdz.put_double(sDZ);
-        fdz.put_float(fDZ);
         if (threadIdx.x < CT) {
             const int m = m0 + threadIdx.x;
             const float le = m < M ? lse_enc[lat + m] : -INFINITY;
-            sLe[threadIdx.x] = le == -INFINITY ? -INFINITY : -le;   // added to the scores: weight 0 for a latent without valid tokens
-            sDe[threadIdx.x] = m < M ? de[lat + m] : 0.f;
+            sLe[column_slot(threadIdx.x)] = le == -INFINITY ? -INFINITY : -le;   // added to the scores: weight 0 for a latent without valid tokens
+            sDe[column_slot(threadIdx.x)] = m < M ? de[lat + m] : 0.f;
         }
         __syncthreads();
         if (m0 + CT < M) {
@@ -133,45 +112,44 @@ bwd_token_simt_kernel(const T *Q, const T *K, const T *V,
                 mma_block<D, RB>(s, ak, sQ, nb);
                 mma_block<D, RB>(a, ag, sZ, nb);
                 mma_block<D, RB>(c, av, sDZ, nb);
-                const int col = nb * 8 + 2 * (lane & 3);
-                const float2 le = *reinterpret_cast<const float2 *>(sLe + col), dem = *reinterpret_cast<const float2 *>(sDe + col);
+                const int at = nb * 8 + 2 * (lane & 3);
+                const float2 le = *reinterpret_cast<const float2 *>(sLe + at), dem = *reinterpret_cast<const float2 *>(sDe + at);
+                const bool in0 = nb * 8 + column_slot(2 * (lane & 3)) < mc, in1 = nb * 8 + column_slot(2 * (lane & 3) + 1) < mc;
+                float2 t[RB], wd[RB], we[RB];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    if (col + e >= mc) continue;
-                    float ds[RB], we[RB];
-#pragma unroll
-                    for (int rb = 0; rb < RB; ++rb) {
-                        const float sc = (float)(e ? s[rb].y : s[rb].x);
-                        const float wd = expf(sc - ld[rb]);
-                        we[rb] = valid[rb] ? expf(sc + (e ? le.y : le.x)) : 0.f;
-                        ds[rb] = (wd * ((float)(e ? a[rb].y : a[rb].x) - dd[rb]) +
-                                  we[rb] * ((float)(e ? c[rb].y : c[rb].x) - (e ? dem.y : dem.x))) * scale;
-                    }
-#pragma unroll
-                    for (int rb = 0; rb < RB; ++rb) {
-                        axpy2<D>(dk[rb], ds[rb], fQ + (col + e) * SG::DV);
-                        axpy2<D>(dv[rb], we[rb], fDZ + (col + e) * SG::DV);
-                    }
+                for (int rb = 0; rb < RB; ++rb) {
+                    const float s0 = (float)s[rb].x, s1 = (float)s[rb].y;
+                    wd[rb] = make_float2(in0 ? exp_diff(s0 - ld[rb]) : 0.f, in1 ? exp_diff(s1 - ld[rb]) : 0.f);
+                    we[rb] = make_float2(in0 && valid[rb] ? exp_diff(s0 + le.x) : 0.f, in1 && valid[rb] ? exp_diff(s1 + le.y) : 0.f);
+                    const float wa0 = wd[rb].x * (float)a[rb].x, wa1 = wd[rb].y * (float)a[rb].y;
+                    dd[rb] += wa0 + wa1;
+                    t[rb] = make_float2(wa0 + we[rb].x * ((float)c[rb].x - dem.x), wa1 + we[rb].y * ((float)c[rb].y - dem.y));
                 }
+                double v[2][SG::NB];
+                load_values<D>(v, sQ, nb);
+                add_values<D, RB>(dk, t, v);
+                add_values<D, RB>(un, wd, v);
+                load_values<D>(v, sDZ, nb);
+                add_values<D, RB>(dv, we, v);
             }
     }
 #pragma unroll
     for (int rb = 0; rb < RB; ++rb) {
         const int n = r0 + 8 * rb + (lane >> 2);
+        dd[rb] = quad_sum(dd[rb]);
 #pragma unroll
-        for (int d = 0; d < D / 2; ++d) {
-            dk[rb][d] = make_float2(quad_sum(dk[rb][d].x), quad_sum(dk[rb][d].y));
-            dv[rb][d] = make_float2(quad_sum(dv[rb][d].x), quad_sum(dv[rb][d].y));
-        }
+        for (int j = 0; j < SG::NB; ++j)
+            dk[rb][j] = make_double2(dk[rb][j].x - (double)dd[rb] * un[rb][j].x, dk[rb][j].y - (double)dd[rb] * un[rb][j].y);
         if (n < N) {
-            write_quarter<T, D>(dK + base + (size_t)n * stride, dk[rb], 1.f);
-            write_quarter<T, D>(dV + base + (size_t)n * stride, dv[rb], 1.f);
+            if ((lane & 3) == 0) dd_out[((size_t)b * H + h) * N + n] = dd[rb];
+            write_row<T, D>(dK + base + (size_t)n * stride, dk[rb], scale);
+            write_row<T, D>(dV + base + (size_t)n * stride, dv[rb], 1.0);
         }
     }
 }
 template <typename T, int D> inline size_t bwd_token_simt_smem() {
     using SG = SimtGeom<D>;
-    return sizeof(double) * 3 * SG::CT * SG::DK + sizeof(float) * (2 * SG::CT * SG::DV + 2 * SG::CT) + (sizeof(T) + 2 * sizeof(float)) * SG::CT * D;
+    return sizeof(double) * 3 * SG::CT * SG::DK + sizeof(float) * (2 * SG::CT + D) + (sizeof(T) + 2 * sizeof(float)) * SG::CT * D;
 }
 
 // Pass B, latent side: partial dQ rows.  Rows are latents, columns tokens; grid and warps as in encode_simt_kernel.
@@ -188,7 +166,7 @@ bwd_dq_simt_kernel(const T *Q, const T *K, const T *V,
     constexpr int CT = SG::CT, RB = BwdSimtGeom<D>::RB, RW = 8 * RB;
     extern __shared__ __align__(16) unsigned char simt_smem[];
     double *sK = reinterpret_cast<double *>(simt_smem), *sG = sK + CT * SG::DK, *sV = sG + CT * SG::DK;
-    float *fK = reinterpret_cast<float *>(sV + CT * SG::DK), *sLd = fK + CT * SG::DV, *sDd = sLd + CT, *sMask = sDd + CT;
+    float *sLd = reinterpret_cast<float *>(sV + CT * SG::DK), *sDd = sLd + CT, *sMask = sDd + CT;   // (in the order of the MMA's indices)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int split = blockIdx.x, h = blockIdx.y / mblocks, mb = blockIdx.y % mblocks, b = blockIdx.z;
     const int WT = kBwdThreads / 32 / WM, wm = warp % WM, wt = warp / WM;
@@ -198,21 +176,23 @@ bwd_dq_simt_kernel(const T *Q, const T *K, const T *V,
     const size_t lat = ((size_t)b * H + h) * M;
     double aq[RB][D / 4], az[RB][D / 4], adz[RB][D / 4];
     load_rows<T, D, RB>(aq, Q + (size_t)h * M * D, D, r0, M, (double)scale);
-    load_rows<float, D, RB>(az, Z + lat * D, D, r0, M, 1.0);
+    float *sC = sMask + CT;
+    z_centre<D>(sC, Z + lat * D, M);
+    __syncthreads();
+    load_rows<float, D, RB>(az, Z + lat * D, D, r0, M, 1.0, sC);
     load_rows<float, D, RB>(adz, dZ + lat * D, D, r0, M, 1.0);
     float nle[RB], dem[RB];
-    float2 acc[RB][D / 2];
+    double2 acc[RB][SG::NB];
+    clear_rows<D, RB>(acc);
 #pragma unroll
     for (int rb = 0; rb < RB; ++rb) {
         const int m = r0 + 8 * rb + (lane >> 2);
         const float le = m < M ? lse_enc[lat + m] : -INFINITY;
         nle[rb] = le == -INFINITY ? -INFINITY : -le;
         dem[rb] = m < M ? de[lat + m] : 0.f;
-#pragma unroll
-        for (int d = 0; d < D / 2; ++d) acc[rb][d] = make_float2(0.f, 0.f);
     }
     using Fetch = TileFetch<T, D, kBwdThreads>;
-    unsigned char *raw = reinterpret_cast<unsigned char *>(sMask + CT);
+    unsigned char *raw = reinterpret_cast<unsigned char *>(sC + D);
     Fetch fk(raw), fg(raw + Fetch::kBytes), fv(raw + 2 * Fetch::kBytes);
     auto fetch = [&](int t0) {
         const size_t at = base + (size_t)t0 * stride;
@@ -225,15 +205,14 @@ bwd_dq_simt_kernel(const T *Q, const T *K, const T *V,
         Fetch::wait();
         __syncthreads();
         fk.put_double(sK);
-        fk.put_float(fK);
         fg.put_double(sG);
         fv.put_double(sV);
         if (threadIdx.x < CT) {
             const int n = t0 + threadIdx.x;
             const bool in = n < n1;
-            sLd[threadIdx.x] = in ? -lse_dec[((size_t)b * N + n) * H + h] : -INFINITY;
-            sDd[threadIdx.x] = in ? dd[((size_t)b * H + h) * N + n] : 0.f;
-            sMask[threadIdx.x] = in && (key_mask == nullptr || key_mask[(size_t)b * N + n] != 0) ? 0.f : -INFINITY;
+            sLd[column_slot(threadIdx.x)] = in ? -lse_dec[((size_t)b * N + n) * H + h] : -INFINITY;
+            sDd[column_slot(threadIdx.x)] = in ? dd[((size_t)b * H + h) * N + n] : 0.f;
+            sMask[column_slot(threadIdx.x)] = in && (key_mask == nullptr || key_mask[(size_t)b * N + n] != 0) ? 0.f : -INFINITY;
         }
         __syncthreads();
         if (t0 + CT < n1) fetch(t0 + CT);
@@ -244,19 +223,20 @@ bwd_dq_simt_kernel(const T *Q, const T *K, const T *V,
                 mma_block<D, RB>(s, aq, sK, nb);
                 mma_block<D, RB>(a, az, sG, nb);
                 mma_block<D, RB>(c, adz, sV, nb);
-                const int col = nb * 8 + 2 * (lane & 3);
-                const float2 nld = *reinterpret_cast<const float2 *>(sLd + col), ddn = *reinterpret_cast<const float2 *>(sDd + col);
-                const float2 msk = *reinterpret_cast<const float2 *>(sMask + col);
+                const int at = nb * 8 + 2 * (lane & 3);
+                const float2 nld = *reinterpret_cast<const float2 *>(sLd + at), ddn = *reinterpret_cast<const float2 *>(sDd + at);
+                const float2 msk = *reinterpret_cast<const float2 *>(sMask + at);
+                float2 ds[RB];
 #pragma unroll
-                for (int e = 0; e < 2; ++e)
-#pragma unroll
-                    for (int rb = 0; rb < RB; ++rb) {
-                        const float sc = (float)(e ? s[rb].y : s[rb].x);
-                        const float wd = expf(sc + (e ? nld.y : nld.x)), we = expf((sc + nle[rb]) + (e ? msk.y : msk.x));
-                        const float ds = wd * ((float)(e ? a[rb].y : a[rb].x) - (e ? ddn.y : ddn.x)) +
-                                         we * ((float)(e ? c[rb].y : c[rb].x) - dem[rb]);
-                        axpy2<D>(acc[rb], ds, fK + (col + e) * SG::DV);
-                    }
+                for (int rb = 0; rb < RB; ++rb) {
+                    const float s0 = (float)s[rb].x, s1 = (float)s[rb].y;
+                    const float we0 = exp_diff((s0 + nle[rb]) + msk.x), we1 = exp_diff((s1 + nle[rb]) + msk.y);
+                    ds[rb] = make_float2(exp_diff(s0 + nld.x) * ((float)a[rb].x - ddn.x) + we0 * ((float)c[rb].x - dem[rb]),
+                                         exp_diff(s1 + nld.y) * ((float)a[rb].y - ddn.y) + we1 * ((float)c[rb].y - dem[rb]));
+                }
+                double v[2][SG::NB];
+                load_values<D>(v, sK, nb);
+                add_values<D, RB>(acc, ds, v);
             }
     }
     __syncthreads();
@@ -266,9 +246,7 @@ bwd_dq_simt_kernel(const T *Q, const T *K, const T *V,
     const int rows_here = WM * RW;
 #pragma unroll
     for (int rb = 0; rb < RB; ++rb) {
-#pragma unroll
-        for (int d = 0; d < D / 2; ++d) acc[rb][d] = make_float2(quad_sum(acc[rb][d].x), quad_sum(acc[rb][d].y));
-        write_quarter<float, D>(sR + ((size_t)wt * rows_here + wm * RW + 8 * rb + (lane >> 2)) * ROW, acc[rb], 1.f);
+        write_row<float, D>(sR + ((size_t)wt * rows_here + wm * RW + 8 * rb + (lane >> 2)) * ROW, acc[rb], 1.0);
     }
     __syncthreads();
     const long rows = (long)B * H * M;
@@ -282,7 +260,7 @@ bwd_dq_simt_kernel(const T *Q, const T *K, const T *V,
 }
 template <typename T, int D> inline size_t bwd_dq_simt_smem() {
     using SG = SimtGeom<D>;
-    const size_t tiles = sizeof(double) * 3 * SG::CT * SG::DK + sizeof(float) * (SG::CT * SG::DV + 3 * SG::CT) + 3 * sizeof(T) * SG::CT * D;
+    const size_t tiles = sizeof(double) * 3 * SG::CT * SG::DK + sizeof(float) * (3 * SG::CT + D) + 3 * sizeof(T) * SG::CT * D;
     const size_t join = sizeof(float) * (kBwdThreads / 32) * 8 * BwdSimtGeom<D>::RB * (D + 4);
     return tiles > join ? tiles : join;
 }

@@ -31,8 +31,11 @@ template <typename T, int D>
 struct Decode {
     template <int RB>
     static int launch(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st) {
-        static_assert(sizeof(double) * 64 * 36 + sizeof(float) * 64 * 36 + 8 * 64 * 32 <= 48 * 1024, "no opt-in needed");
-        FLARE_CUDA(launch_after(decode_simt_kernel<T, D, RB>, dim3((d->N + 64 * RB - 1) / (64 * RB), d->H, d->B), kSimtThreads, decode_simt_smem<T, D>(), st,
+        const size_t smem = decode_simt_smem<T, D>();
+        static std::atomic<uint64_t> opt_in{0};
+        if (smem > 48 * 1024)
+            if (int rc = ensure_big_smem(decode_simt_kernel<T, D, RB>, opt_in, (int)smem)) return rc;
+        FLARE_CUDA(launch_after(decode_simt_kernel<T, D, RB>, dim3((d->N + 64 * RB - 1) / (64 * RB), d->H, d->B), kSimtThreads, smem, st,
                                 (const T *)Q, (const T *)K, Z, (T *)Y, lse_dec, d->B, d->H, d->N, d->M, d->scale));
         return FLARE_OK;
     }

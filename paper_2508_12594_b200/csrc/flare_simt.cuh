@@ -2,17 +2,16 @@
 //
 // float32 inputs must meet a 1e-5 relative tolerance, which the tensor cores' reduced-mantissa float32 mode cannot.  Here
 // every score q.k is summed in double precision, by the double-precision MMA (m8n8k4), and rounded once; exponentials
-// are expf, the value contractions float32 FMAs.  What bounds them is the double-precision pipe: 64 multiply-adds per clock
-// per SM, D of them per (row, column) pair and product, so 0.25 clocks per pair and SM at D = 16 (a thread per row with
-// scalar double FMAs took 2.1 to 2.4: converting both operands of every product in the inner loop, 16 conversions per clock, was
-// most of it; 0.9 now, encode and decode at D = 16).
+// are expf; the value contractions run on the double-precision MMA too, their sums in double.  What bounds them is that pipe:
+// 64 multiply-adds per clock per SM, D of them per (row, column) pair and product, 0.25 clocks per pair, product and SM at D = 16.
 //
 // All of them share one shape.  "Rows" (latents in encode, dZ and dQ; tokens in decode and the token pass) stay in
 // registers as A fragments, RB blocks of 8 rows per warp; "columns" (the other kind) stream through shared memory in tiles
-// of CT, as doubles for the B fragments and as floats for the value contraction.  In a C fragment a thread holds row
-// lane / 4 and columns 2 (lane % 4), + 1, so it weights two rows of the value tile per MMA and keeps a partial
-// accumulator of its row over its own columns; the four lanes of a row meet once, at the end.  Row strides are padded by four
-// elements: B fragments and value rows are then read without bank conflicts.
+// of CT, as doubles.  In a C fragment a thread holds row g = lane / 4 and two columns, what an A fragment asks of it with those two as the
+// K index of two steps: the weights go from one MMA into the next in the same registers, only rounded to float and back on the way.
+// (As float32 FMAs, every thread adding up whole rows over its own columns, the contractions and their shared-memory reads took
+// as long again as the scores.)  Which two columns is chosen (column_slot) so that neither the fragments of the scores nor those of the values
+// meet bank conflicts, with rows of D + 4 doubles.
 #pragma once
 
 #include "flare_ptx.cuh"
@@ -22,25 +21,19 @@ namespace flare {
 
 template <int D> struct SimtGeom {
     static constexpr int CT = D <= 32 ? 64 : 32;                     // columns per tile
-    static constexpr int DK = D + (D == 4 ? 0 : 4), DV = D + 4;      // padded row lengths of double and float tiles
+    static constexpr int DK = D + (D == 4 ? 0 : 4);                  // padded row length of a tile of doubles
+    static constexpr int NB = D < 8 ? 1 : D / 8;                     // blocks of 8 features of a row
 };
+// The column of a block of eight that is index j of the scores' MMA, and the other way round.  Thread q of a quad then has columns 0,1 | 2,3 | 5,4 |
+// 7,6: as rows of a tile, of 8 (mod 32) banks each, the first of the four (second likewise) lie in different banks, and so do those of
+// indices 0-3 and 4-7.
+__host__ __device__ constexpr int column_slot(int j) { return j ^ ((j >> 2) & 1); }
 
 // D (8x8, f64) += A (8x4, row lane / 4, k lane % 4) * B (4x8, k lane % 4, column lane / 4)
 __device__ __forceinline__ void dmma(double2 &c, double a, double b) {
     asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c.x), "+d"(c.y) : "d"(a), "d"(b));
 }
 
-// Packed-pair helpers: value rows are read four floats at a time and accumulated two at a time.
-template <int D>
-__device__ __forceinline__ void axpy2(float2 *acc, float w, const float *row) {
-    const float2 wp = make_float2(w, w);
-#pragma unroll
-    for (int d = 0; d < D; d += 4) {
-        const float4 v = *reinterpret_cast<const float4 *>(row + d);
-        acc[d / 2] = __ffma2_rn(wp, make_float2(v.x, v.y), acc[d / 2]);
-        acc[d / 2 + 1] = __ffma2_rn(wp, make_float2(v.z, v.w), acc[d / 2 + 1]);
-    }
-}
 __device__ __forceinline__ float quad_sum(float x) {
     x += __shfl_xor_sync(0xffffffffu, x, 1);
     return x + __shfl_xor_sync(0xffffffffu, x, 2);
@@ -85,47 +78,46 @@ struct TileFetch {
         }
     }
     // (pairs of doubles, neighbouring rows in opposite order: a quarter warp then covers all banks)
-    __device__ __forceinline__ void put_double(double *dst) const {
+    // kCentred: less `centre`
+    template <bool kCentred = false>
+    __device__ __forceinline__ void put_double(double *dst, const float *centre = nullptr) const {
         each([&](int r, int c, const Vec &x) {
             double2 *p = reinterpret_cast<double2 *>(dst + r * SimtGeom<D>::DK + c);
+            auto at = [&](int k) { return (double)to_f32(x.e[k]) - (kCentred ? (double)centre[c + k] : 0.0); };
             if constexpr (VE == 4) {
                 const bool odd = r & 1;
-                const double2 lo = make_double2((double)to_f32(x.e[0]), (double)to_f32(x.e[1]));
-                const double2 hi = make_double2((double)to_f32(x.e[2]), (double)to_f32(x.e[3]));
+                const double2 lo = make_double2(at(0), at(1)), hi = make_double2(at(2), at(3));
                 p[odd] = odd ? hi : lo;
                 p[!odd] = odd ? lo : hi;
             } else {
 #pragma unroll
-                for (int k = 0; k < VE / 2; ++k) p[k] = make_double2((double)to_f32(x.e[2 * k]), (double)to_f32(x.e[2 * k + 1]));
+                for (int k = 0; k < VE / 2; ++k) p[k] = make_double2(at(2 * k), at(2 * k + 1));
             }
-        });
-    }
-    __device__ __forceinline__ void put_float(float *dst) const {
-        each([&](int r, int c, const Vec &x) {
-            float4 *p = reinterpret_cast<float4 *>(dst + r * SimtGeom<D>::DV + c);
-#pragma unroll
-            for (int k = 0; k < VE / 4; ++k)
-                p[k] = make_float4(to_f32(x.e[4 * k]), to_f32(x.e[4 * k + 1]), to_f32(x.e[4 * k + 2]), to_f32(x.e[4 * k + 3]));
         });
     }
 };
 
-// A fragments of RB row blocks: row r0 + 8 rb + lane / 4, element 4 kk + lane % 4, times f; rows from `rows` on are zeros.
+// A fragments of RB row blocks: row r0 + 8 rb + lane / 4, element 4 kk + lane % 4, less `centre` (null: nothing), times f; rows from `rows` on
+// are zeros.
 template <typename T, int D, int RB>
-__device__ __forceinline__ void load_rows(double (&a)[RB][D / 4], const T *src, size_t stride, int r0, int rows, double f) {
+__device__ __forceinline__ void load_rows(double (&a)[RB][D / 4], const T *src, size_t stride, int r0, int rows, double f,
+                                          const float *centre = nullptr) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int rb = 0; rb < RB; ++rb) {
         const int r = r0 + 8 * rb + (lane >> 2);
 #pragma unroll
-        for (int kk = 0; kk < D / 4; ++kk) a[rb][kk] = r < rows ? (double)to_f32(src[(size_t)r * stride + 4 * kk + (lane & 3)]) * f : 0.0;
+        for (int kk = 0; kk < D / 4; ++kk) {
+            const double c = centre != nullptr ? (double)centre[4 * kk + (lane & 3)] : 0.0;
+            a[rb][kk] = r < rows ? ((double)to_f32(src[(size_t)r * stride + 4 * kk + (lane & 3)]) - c) * f : 0.0;
+        }
     }
 }
 // c[rb] = the 8 x 8 products of the row blocks with columns nb * 8 ... of a double tile
 template <int D, int RB>
 __device__ __forceinline__ void mma_block(double2 (&c)[RB], const double (&a)[RB][D / 4], const double *tile, int nb) {
     const int lane = threadIdx.x & 31;
-    const double *b = tile + (nb * 8 + (lane >> 2)) * SimtGeom<D>::DK + (lane & 3);
+    const double *b = tile + (nb * 8 + column_slot(lane >> 2)) * SimtGeom<D>::DK + (lane & 3);
 #pragma unroll
     for (int rb = 0; rb < RB; ++rb) c[rb] = make_double2(0.0, 0.0);
 #pragma unroll
@@ -135,67 +127,97 @@ __device__ __forceinline__ void mma_block(double2 (&c)[RB], const double (&a)[RB
         for (int rb = 0; rb < RB; ++rb) dmma(c[rb], a[rb][kk], bk);
     }
 }
+// B fragments of a block of eight columns for the value contractions: v[e][j] = element 8 j + lane / 4 of the row that is the thread's
+// (quad lane's) column e.
+template <int D>
+__device__ __forceinline__ void load_values(double (&v)[2][SimtGeom<D>::NB], const double *tile, int nb) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const double *b = tile + (nb * 8 + column_slot(2 * (lane & 3) + e)) * SimtGeom<D>::DK + (lane >> 2);
+#pragma unroll
+        for (int j = 0; j < SimtGeom<D>::NB; ++j) v[e][j] = D >= 8 || lane < 4 * D ? b[8 * j] : 0.0;
+    }
+}
+// acc += weights of the thread's two columns * values: row lane / 4 of a block, elements 8 j + 2 (lane % 4), + 1
+template <int D, int RB>
+__device__ __forceinline__ void add_values(double2 (&acc)[RB][SimtGeom<D>::NB], const float2 (&w)[RB], const double (&v)[2][SimtGeom<D>::NB]) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+#pragma unroll
+        for (int rb = 0; rb < RB; ++rb) {
+            const double we = (double)(e ? w[rb].y : w[rb].x);
+#pragma unroll
+            for (int j = 0; j < SimtGeom<D>::NB; ++j) dmma(acc[rb][j], we, v[e][j]);
+        }
+}
+template <int D, int RB>
+__device__ __forceinline__ void clear_rows(double2 (&acc)[RB][SimtGeom<D>::NB]) {
+#pragma unroll
+    for (int rb = 0; rb < RB; ++rb)
+#pragma unroll
+        for (int j = 0; j < SimtGeom<D>::NB; ++j) acc[rb][j] = make_double2(0.0, 0.0);
+}
+// The row a quad holds, times f, written by its four threads.
+template <typename T, int D>
+__device__ __forceinline__ void write_row(T *dst, const double2 (&acc)[SimtGeom<D>::NB], double f) {
+    const int q = threadIdx.x & 3;
+    if (D < 8 && 2 * q >= D) return;
+    struct alignas(2 * sizeof(T)) Pair { T x, y; };
+#pragma unroll
+    for (int j = 0; j < SimtGeom<D>::NB; ++j) {
+        Pair p;
+        from_f32(p.x, (float)(acc[j].x * f));
+        from_f32(p.y, (float)(acc[j].y * f));
+        *reinterpret_cast<Pair *>(dst + 8 * j + 2 * q) = p;
+    }
+}
 
-// Running softmax state of the rows of a thread, over its own columns.  The reference m is not the running maximum but a
-// score within kSlack of it: exp(score - m) stays below e^20, and rescaling (a divergent branch) is rare.
+// exp of a score, once rounded to float, less a reference or a log-sum-exp (which was formed from scores rounded the same way: the rounding of the
+// largest ones cancels; with the difference taken in double and rounded after it a weight near 1 was off by the log-sum-exp's last place,
+// the largest entries of dV three times as much).  The product's rounding is x / 2^24, and e^x x small.
+__device__ __forceinline__ float exp_diff(float x) { return ptx::ex2(x * 1.4426950408889634f); }
+
+// Running softmax state of the rows of a warp.  The reference m of a row (the same in the four threads of its quad) is not the running maximum
+// but a score within kSlack of it: exp(score - m) stays below e^20, and rescaling (a branch of the whole warp) is rare.
 constexpr float kNoScore = -1.0e30f, kSlack = 20.f;
 template <int D, int RB>
 struct RowState {
-    float m[RB], l[RB];
-    float2 acc[RB][D / 2];
+    float m[RB], l[RB];                                              // (l: over the thread's own columns)
+    double2 acc[RB][SimtGeom<D>::NB];
     __device__ __forceinline__ void clear() {
 #pragma unroll
         for (int rb = 0; rb < RB; ++rb) {
             m[rb] = kNoScore;
             l[rb] = 0.f;
-#pragma unroll
-            for (int d = 0; d < D / 2; ++d) acc[rb][d] = make_float2(0.f, 0.f);
         }
+        clear_rows<D, RB>(acc);
     }
-    __device__ __forceinline__ void rescale(int rb, float f) {
-        l[rb] *= f;
+    // s: scores of the thread's two columns; their weights (0 for a score of -inf)
+    __device__ __forceinline__ void weights(const float2 (&s)[RB], float2 (&p)[RB]) {
+        bool far = false;
 #pragma unroll
-        for (int d = 0; d < D / 2; ++d) acc[rb][d] = make_float2(acc[rb][d].x * f, acc[rb][d].y * f);
-    }
-    // the weights of two columns of row block rb (scores of -inf weigh nothing)
-    __device__ __forceinline__ float2 weights(int rb, float s0, float s1) {
-        const float mx = fmaxf(s0, s1);
-        if (mx > m[rb] + kSlack) {
-            rescale(rb, expf(m[rb] - mx));
-            m[rb] = mx;
+        for (int rb = 0; rb < RB; ++rb) far = far || fmaxf(s[rb].x, s[rb].y) > m[rb] + kSlack;
+        if (__any_sync(0xffffffffu, far)) {
+#pragma unroll
+            for (int rb = 0; rb < RB; ++rb) {
+                const float mx = quad_max(fmaxf(s[rb].x, s[rb].y));
+                if (mx > m[rb] + kSlack) {
+                    const float f = exp_diff(m[rb] - mx);
+                    m[rb] = mx;
+                    l[rb] *= f;
+#pragma unroll
+                    for (int j = 0; j < SimtGeom<D>::NB; ++j) acc[rb][j] = make_double2(acc[rb][j].x * f, acc[rb][j].y * f);
+                }
+            }
         }
-        const float2 p = make_float2(expf(s0 - m[rb]), expf(s1 - m[rb]));
-        l[rb] += p.x + p.y;
-        return p;
-    }
-    // the four lanes of every row joined; all four hold the result
-    __device__ __forceinline__ void join_quad() {
 #pragma unroll
         for (int rb = 0; rb < RB; ++rb) {
-            const float top = quad_max(m[rb]);
-            rescale(rb, expf(m[rb] - top));
-            m[rb] = top;
-            l[rb] = quad_sum(l[rb]);
-#pragma unroll
-            for (int d = 0; d < D / 2; ++d) acc[rb][d] = make_float2(quad_sum(acc[rb][d].x), quad_sum(acc[rb][d].y));
+            p[rb] = make_float2(exp_diff(s[rb].x - m[rb]), exp_diff(s[rb].y - m[rb]));
+            l[rb] += p[rb].x + p[rb].y;
         }
     }
 };
-// Element d of a row as float (d a constant after unrolling).
-template <int D> __device__ __forceinline__ float pick(const float2 (&acc)[D / 2], int d) { return d & 1 ? acc[d / 2].y : acc[d / 2].x; }
-// Lane q of a quad writes its quarter of a row of D elements.
-template <typename T, int D>
-__device__ __forceinline__ void write_quarter(T *dst, const float2 (&acc)[D / 2], float f) {
-    constexpr int QD = D / 4;
-    const int q = threadIdx.x & 3;
-    struct alignas(sizeof(T) * QD < 16 ? sizeof(T) * QD : 16) Out { T e[QD]; } out;
-#pragma unroll
-    for (int k = 0; k < QD; ++k) {
-        const float x01 = q & 1 ? pick<D>(acc, QD + k) : pick<D>(acc, k), x23 = q & 1 ? pick<D>(acc, 3 * QD + k) : pick<D>(acc, 2 * QD + k);
-        from_f32(out.e[k], (q & 2 ? x23 : x01) * f);
-    }
-    *reinterpret_cast<Out *>(dst + q * QD) = out;
-}
 
 // Encode, split over N.  grid = (splits, H * mblocks, B); the block's eight warps are WM groups of 8 RB latents x WT = 8 / WM
 // shares of a tile's columns.  The shares are joined in shared memory: one partial (m, l, row) per latent and split.
@@ -211,8 +233,8 @@ encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
     constexpr int CT = SG::CT, RW = 8 * RB;
     extern __shared__ __align__(16) unsigned char simt_smem[];
     double *sK = reinterpret_cast<double *>(simt_smem);             // [CT][DK]
-    float *sV = reinterpret_cast<float *>(sK + CT * SG::DK);        // [CT][DV]
-    float *sBias = sV + CT * SG::DV;                                // [CT]: added to a column's scores
+    double *sV = sK + CT * SG::DK;                                  // [CT][DK]
+    float *sBias = reinterpret_cast<float *>(sV + CT * SG::DK);     // [CT]: added to a column's scores (in the order of the MMA's indices)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int split = blockIdx.x, h = blockIdx.y / mblocks, mb = blockIdx.y % mblocks, b = blockIdx.z;
     const int WT = kSimtThreads / 32 / WM, wm = warp % WM, wt = warp / WM;
@@ -233,7 +255,7 @@ encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
         Fetch::wait();
         __syncthreads();
         fk.put_double(sK);
-        fv.put_float(sV);
+        fv.put_double(sV);
         if (threadIdx.x < CT) {
             const int n = t0 + threadIdx.x;
             float bias = -INFINITY;
@@ -241,7 +263,7 @@ encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
                 if (kDz) bias = -lse_dec[((size_t)b * N + n) * H + h];
                 else if (key_mask == nullptr || key_mask[(size_t)b * N + n] != 0) bias = 0.f;
             }
-            sBias[threadIdx.x] = bias;
+            sBias[column_slot(threadIdx.x)] = bias;
         }
         __syncthreads();
         if (t0 + CT < n1) {
@@ -253,33 +275,24 @@ encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
             for (int nb = wt; nb < blocks; nb += WT) {
                 double2 c[RB];
                 mma_block<D, RB>(c, aq, sK, nb);
-                const int col = nb * 8 + 2 * (lane & 3);
-                const float2 bias = *reinterpret_cast<const float2 *>(sBias + col);
-                float2 p[RB];
+                const float2 bias = *reinterpret_cast<const float2 *>(sBias + nb * 8 + 2 * (lane & 3));
+                float2 sc[RB], p[RB];
+                double v[2][SG::NB];
+                load_values<D>(v, sV, nb);
 #pragma unroll
                 for (int rb = 0; rb < RB; ++rb) {
-                    const float s0 = (float)c[rb].x + bias.x, s1 = (float)c[rb].y + bias.y;
-                    p[rb] = kDz ? make_float2(expf(s0), expf(s1)) : st.weights(rb, s0, s1);
+                    sc[rb] = make_float2((float)c[rb].x + bias.x, (float)c[rb].y + bias.y);
+                    if (kDz) p[rb] = make_float2(exp_diff(sc[rb].x), exp_diff(sc[rb].y));
                 }
-#pragma unroll
-                for (int d = 0; d < D; d += 4) {
-                    const float4 v0 = *reinterpret_cast<const float4 *>(sV + col * SG::DV + d);
-                    const float4 v1 = *reinterpret_cast<const float4 *>(sV + (col + 1) * SG::DV + d);
-#pragma unroll
-                    for (int rb = 0; rb < RB; ++rb) {
-                        const float2 p0 = make_float2(p[rb].x, p[rb].x), p1 = make_float2(p[rb].y, p[rb].y);
-                        float2 &x = st.acc[rb][d / 2], &y = st.acc[rb][d / 2 + 1];
-                        x = __ffma2_rn(p1, make_float2(v1.x, v1.y), __ffma2_rn(p0, make_float2(v0.x, v0.y), x));
-                        y = __ffma2_rn(p1, make_float2(v1.z, v1.w), __ffma2_rn(p0, make_float2(v0.z, v0.w), y));
-                    }
-                }
+                if (!kDz) st.weights(sc, p);
+                add_values<D, RB>(st.acc, p, v);
             }
     }
-    if (kDz) {
 #pragma unroll
-        for (int rb = 0; rb < RB; ++rb) st.m[rb] = 0.f;
+    for (int rb = 0; rb < RB; ++rb) {
+        if (kDz) st.m[rb] = 0.f;
+        st.l[rb] = quad_sum(st.l[rb]);
     }
-    st.join_quad();
     // the shares of the columns meet: [WT][WM * RW rows] rows of (acc, m, l)
     __syncthreads();
     constexpr int ROW = D + 4;
@@ -292,7 +305,7 @@ encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
             dst[D] = st.m[rb];
             dst[D + 1] = st.l[rb];
         }
-        write_quarter<float, D>(dst, st.acc[rb], 1.f);
+        write_row<float, D>(dst, st.acc[rb], 1.0);
     }
     __syncthreads();
     const long rows = (long)B * H * M;
@@ -303,7 +316,7 @@ encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
         for (int w = 0; w < WT; ++w) top = fmaxf(top, sR[((size_t)w * rows_here + r) * ROW + D]);
         for (int w = 0; w < WT; ++w) {
             const float *src = sR + ((size_t)w * rows_here + r) * ROW;
-            const float f = kDz ? 1.f : expf(src[D] - top);
+            const float f = kDz ? 1.f : exp_diff(src[D] - top);
             l = fmaf(src[D + 1], f, l);
             z = fmaf(src[d], f, z);
         }
@@ -317,7 +330,7 @@ encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
 }
 template <typename T, int D> inline size_t encode_simt_smem(int RB) {
     using SG = SimtGeom<D>;
-    const size_t tiles = sizeof(double) * SG::CT * SG::DK + sizeof(float) * (SG::CT * SG::DV + SG::CT) + 2 * sizeof(T) * SG::CT * D;
+    const size_t tiles = sizeof(double) * 2 * SG::CT * SG::DK + sizeof(float) * SG::CT + 2 * sizeof(T) * SG::CT * D;
     const size_t join = sizeof(float) * (kSimtThreads / 32) * 8 * RB * (D + 4);
     return tiles > join ? tiles : join;
 }
@@ -333,7 +346,7 @@ decode_simt_kernel(const T *Q, const T *K, const float *Z, T *Y,
     constexpr int CT = SG::CT;
     extern __shared__ __align__(16) unsigned char simt_smem[];
     double *sQ = reinterpret_cast<double *>(simt_smem);
-    float *sZ = reinterpret_cast<float *>(sQ + CT * SG::DK);
+    double *sZ = sQ + CT * SG::DK;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, h = blockIdx.y, b = blockIdx.z;
     const int r0 = (blockIdx.x * (kSimtThreads / 32) + warp) * 8 * RB;
     const T *Qh = Q + (size_t)h * M * D;
@@ -342,7 +355,7 @@ decode_simt_kernel(const T *Q, const T *K, const float *Z, T *Y,
     load_rows<T, D, RB>(ak, K + ((size_t)b * N * H + h) * D, (size_t)H * D, r0, N, (double)scale);
     RowState<D, RB> st;
     st.clear();
-    unsigned char *raw = reinterpret_cast<unsigned char *>(sZ + CT * SG::DV);
+    unsigned char *raw = reinterpret_cast<unsigned char *>(sZ + CT * SG::DK);
     TileFetch<T, D, kSimtThreads> fq(raw);
     TileFetch<float, D, kSimtThreads> fz(raw + fq.kBytes);
     fq.load(Qh, D, M);
@@ -351,7 +364,7 @@ decode_simt_kernel(const T *Q, const T *K, const float *Z, T *Y,
         fq.wait();
         __syncthreads();
         fq.put_double(sQ);
-        fz.put_float(sZ);
+        fz.put_double(sZ);
         __syncthreads();
         if (m0 + CT < M) {
             fq.load(Qh + (size_t)(m0 + CT) * D, D, M - m0 - CT);
@@ -362,38 +375,28 @@ decode_simt_kernel(const T *Q, const T *K, const float *Z, T *Y,
             for (int nb = 0; nb < (mc + 7) / 8; ++nb) {
                 double2 c[RB];
                 mma_block<D, RB>(c, ak, sQ, nb);
-                const int col = nb * 8 + 2 * (lane & 3);
-                float2 p[RB];
+                const bool in0 = nb * 8 + column_slot(2 * (lane & 3)) < mc, in1 = nb * 8 + column_slot(2 * (lane & 3) + 1) < mc;
+                float2 sc[RB], p[RB];
+                double v[2][SG::NB];
+                load_values<D>(v, sZ, nb);
 #pragma unroll
-                for (int rb = 0; rb < RB; ++rb)
-                    p[rb] = st.weights(rb, col < mc ? (float)c[rb].x : -INFINITY, col + 1 < mc ? (float)c[rb].y : -INFINITY);
-#pragma unroll
-                for (int d = 0; d < D; d += 4) {
-                    const float4 v0 = *reinterpret_cast<const float4 *>(sZ + col * SG::DV + d);
-                    const float4 v1 = *reinterpret_cast<const float4 *>(sZ + (col + 1) * SG::DV + d);
-#pragma unroll
-                    for (int rb = 0; rb < RB; ++rb) {
-                        const float2 p0 = make_float2(p[rb].x, p[rb].x), p1 = make_float2(p[rb].y, p[rb].y);
-                        float2 &x = st.acc[rb][d / 2], &y = st.acc[rb][d / 2 + 1];
-                        x = __ffma2_rn(p1, make_float2(v1.x, v1.y), __ffma2_rn(p0, make_float2(v0.x, v0.y), x));
-                        y = __ffma2_rn(p1, make_float2(v1.z, v1.w), __ffma2_rn(p0, make_float2(v0.z, v0.w), y));
-                    }
-                }
+                for (int rb = 0; rb < RB; ++rb) sc[rb] = make_float2(in0 ? (float)c[rb].x : -INFINITY, in1 ? (float)c[rb].y : -INFINITY);
+                st.weights(sc, p);
+                add_values<D, RB>(st.acc, p, v);
             }
     }
-    st.join_quad();
 #pragma unroll
     for (int rb = 0; rb < RB; ++rb) {
         const int n = r0 + 8 * rb + (lane >> 2);
+        const float l = quad_sum(st.l[rb]);
         if (n >= N) continue;
         const size_t tok = ((size_t)b * N + n) * H + h;
-        write_quarter<T, D>(Y + tok * D, st.acc[rb], 1.f / st.l[rb]);
-        if (lse_dec != nullptr && (lane & 3) == 0) lse_dec[tok] = st.m[rb] + logf(st.l[rb]);
+        write_row<T, D>(Y + tok * D, st.acc[rb], 1.0 / (double)l);
+        if (lse_dec != nullptr && (lane & 3) == 0) lse_dec[tok] = st.m[rb] + logf(l);
     }
 }
 template <typename T, int D> inline size_t decode_simt_smem() {
-    return sizeof(double) * SimtGeom<D>::CT * SimtGeom<D>::DK + sizeof(float) * SimtGeom<D>::CT * SimtGeom<D>::DV +
-           (sizeof(T) + sizeof(float)) * SimtGeom<D>::CT * D;
+    return sizeof(double) * 2 * SimtGeom<D>::CT * SimtGeom<D>::DK + (sizeof(T) + sizeof(float)) * SimtGeom<D>::CT * D;
 }
 
 }  // namespace flare

@@ -1,6 +1,7 @@
 """The float32 / float16 kernels at the edges of their tiles (needs a B200): rows in blocks of 8 per warp and up to 8 warps,
 columns in tiles of 64 (32 at head width 64), against the oracle, forward and backward."""
 import pytest
+import torch
 
 from paper_2508_12594_b200 import workloads
 from tests._util import assert_forward_close, gpu_forward, oracle_forward
@@ -19,3 +20,15 @@ def test_tile_edges(oracle, B, H, N, M, D, masked, dtype):
     what = f"{dtype} B{B}H{H}N{N}M{M}D{D}"
     assert_forward_close(gpu_forward(inp, scale=0.7, canary=True), oracle_forward(oracle, inp, 0.7), dtype, what)
     assert_grads_close(gpu_backward(inp, 0.7), oracle_backward(oracle, inp, 0.7), dtype, what)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("B,H,N,M,D", [(1, 2, 700, 24, 4), (1, 1, 520, 40, 8), (1, 2, 1300, 16, 16), (1, 1, 600, 72, 32), (1, 1, 300, 33, 64)])
+def test_scores_climb(oracle, B, H, N, M, D, dtype):
+    """Scores that grow by tens along the tokens and along the latents: the softmax references move several times, in encode and decode.  A
+    score of 64 is rounded by 2^-19, which the bounds of the other cases allow for."""
+    inp = workloads.make_random(B, H, N, M, D, dtype=dtype, seed=N + M, k_std=0.8)
+    inp.K.mul_(torch.linspace(0.05, 4.0, N)[None, :, None, None].to(inp.K.dtype))
+    inp.Q.mul_(torch.linspace(0.5, 2.0, M)[None, :, None].to(inp.Q.dtype))
+    scale = 2.0 * D ** -0.5
+    assert_forward_close(gpu_forward(inp, scale), oracle_forward(oracle, inp, scale), dtype, f"climb {dtype} B{B}H{H}N{N}M{M}D{D}")
