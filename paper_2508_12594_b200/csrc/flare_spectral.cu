@@ -55,11 +55,9 @@ int launch_spectral_gram_tc(const flare_desc_t *d, int sms, const void *Q, const
     a.sl2 = d->scale * kLog2e;
     a.tiles = (d->N + kTile - 1) / kTile;
     a.splits = spectral_splits(d, sms);
-    spectral_gram_tc_kernel<D><<<dim3(a.splits, d->H, d->B), kTcThreads, SpectralSmem<D>::total, st>>>(tmK, tmQ, a);
-    FLARE_CUDA(cudaGetLastError());
-    const long n = (long)d->B * d->H * d->M * d->M;
-    spectral_gram_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(a.part, G, a.splits * kSpectralGroups, (long)d->B * d->H, d->M);
-    FLARE_CUDA(cudaGetLastError());
+    FLARE_CUDA(launch_after(spectral_gram_tc_kernel<D>, dim3(a.splits, d->H, d->B), kTcThreads, SpectralSmem<D>::total, st, tmK, tmQ, a));
+    FLARE_CUDA(launch_after(spectral_gram_reduce_kernel, dim3(gram_tile_pairs(d->M), (unsigned)(d->B * d->H)), kGramTile * kGramTile, 0, st, a.part, G,
+                            a.splits * kSpectralGroups, (long)d->B * d->H, d->M));
     return FLARE_OK;
 }
 
@@ -166,16 +164,14 @@ int spectral_gram(const flare_desc_t *desc, int sms, const void *Q_lat, const vo
 int spectral_eig(int32_t matrices, int32_t M, float *G, float *eigenvalues, float *U, int32_t sweeps, cudaStream_t stream) {
     if (U == nullptr) {
         // in registers while a thread's rows of a column fit (see the kernel), in shared memory while that holds M x M, else in G
-#define FLARE_EIG(CX) spectral_tridiag_reg_kernel<CX><<<(unsigned)matrices, EigReg<CX>::kThreads, 0, stream>>>(G, M)
+#define FLARE_EIG(CX) do { FLARE_CUDA(launch_after(spectral_tridiag_reg_kernel<CX>, dim3((unsigned)matrices), EigReg<CX>::kThreads, 0, stream, G, M)); } while (0)
         if (M <= 192) {
-            switch ((M + 31) / 32) {
-                case 1: FLARE_EIG(32); break;
-                case 2: FLARE_EIG(64); break;
-                case 3: FLARE_EIG(96); break;
-                case 4: FLARE_EIG(128); break;
-                case 5: FLARE_EIG(160); break;
-                default: FLARE_EIG(192); break;
-            }
+            if (M <= 32) FLARE_EIG(32);
+            else if (M <= 64) FLARE_EIG(64);
+            else if (M <= 96) FLARE_EIG(96);
+            else if (M <= 128) FLARE_EIG(128);
+            else if (M <= 160) FLARE_EIG(160);
+            else FLARE_EIG(192);
 #undef FLARE_EIG
         } else if (eig_smem(M, true) + 256 <= 227 * 1024) {
             static std::atomic<uint64_t> opt_in{0};
@@ -186,9 +182,8 @@ int spectral_eig(int32_t matrices, int32_t M, float *G, float *eigenvalues, floa
         }
         FLARE_CUDA(cudaGetLastError());
         constexpr int per_block = kBisectThreads / kEigSectors;
-        spectral_bisect_kernel<<<dim3((unsigned)((M + per_block - 1) / per_block), (unsigned)matrices), kBisectThreads,
-                                 (sizeof(EigPair<double>) + sizeof(EigPair<float>)) * (size_t)M, stream>>>(G, eigenvalues, M);
-        FLARE_CUDA(cudaGetLastError());
+        FLARE_CUDA(launch_after(spectral_bisect_kernel, dim3((unsigned)((M + per_block - 1) / per_block), (unsigned)matrices), kBisectThreads,
+                                (sizeof(EigPair<double>) + sizeof(EigPair<float>)) * (size_t)M, stream, G, eigenvalues, M));
         return FLARE_OK;
     }
     if (sweeps <= 0) sweeps = 12;

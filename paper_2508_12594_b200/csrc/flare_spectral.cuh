@@ -10,10 +10,12 @@
 //
 //   spectral_gram_tc_kernel    bfloat16, M <= 128, D in {16, 32}: tcgen05.  A CTA takes one head and a range of
 //                              tokens; the head's latents sit on the 128 TMEM lanes.  Per 32 tokens: S = Q K^T; 128
-//                              threads form J as two bf16 halves (hi + lo), back over the scores (the A operand of the
-//                              next MMAs) and into shared memory (their B operand); G += J J^T with the accumulator in
-//                              TMEM, as hi hi^T + hi lo^T + lo hi^T (the diagonal of G is a sum of squares: with single
-//                              bf16 factors nothing cancels and G is off by 4e-3 of its largest entries).
+//                              threads form J as two bf16 halves (hi + lo): hi back over the scores (the A operand of the
+//                              next MMAs), hi and 2 lo into shared memory (their B operands); X += hi hi^T + 2 hi lo^T with
+//                              the accumulator in TMEM.  G = (X + X^T) / 2 = hi hi^T + hi lo^T + lo hi^T, taken when the
+//                              splits are summed: two products instead of three (eight heads of 131072 tokens, M = 128,
+//                              D = 32: 113 -> 106 us).  (The diagonal of G is a sum of squares: with single
+//                              bf16 factors nothing cancels and G is off by 4e-3 of its largest entries.)
 //   spectral_gram_simt_kernel  everything else (float32 inputs, other shapes): CUDA cores, a 16 x 16 tile of G per block.
 //   spectral_gram_reduce_kernel sums the token splits and writes the symmetric G.
 //   spectral_jacobi_kernel     eigenvalues and eigenvectors of G by cyclic two-sided Jacobi rotations.
@@ -91,6 +93,8 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
         ptx::prefetch_tensormap(&tmQ);
     }
     if (warp == kFirstIssuerWarp) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), NCOLS);
+    ptx::grid_launch();
+    ptx::grid_wait();
     for (int i = threadIdx.x; i < kTile * (G::RB / 16); i += kTcThreads)          // latent rows beyond M stay zero
         reinterpret_cast<uint4 *>(sQ)[i] = make_uint4(0, 0, 0, 0);
     ptx::fence_proxy_async_smem();
@@ -136,17 +140,15 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
             for (int u = 0; ok && u < units; ++u) {
                 if (!ptx::mbar_wait(bar(P_FULL + g), u & 1, abort_flag, kErrSpectral | 4)) break;
                 ptx::tc_fence_after();
-                // G += J J^T over the unit's 32 tokens (two k-steps of 16): A = J in tensor memory (hi in the first 16 columns
-                // of the score buffer, lo in the other 16), B = J in shared memory (hi tile, then lo tile)
+                // X += hi (hi + 2 lo)^T over the unit's 32 tokens (two k-steps of 16): A = hi in tensor memory (the first 16 columns
+                // of the score buffer), B in shared memory (hi tile, then 2 lo tile)
                 constexpr uint64_t LO = (uint64_t)(SM::kPbBytes >> 4);
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
 #pragma unroll
-                    for (int t = 0; t < 3; ++t) {               // hi hi^T, hi lo^T, lo hi^T
-                        const uint32_t acol = (t == 2 ? 16u : 0u) + 8 * k;
-                        const uint64_t bsel = (t == 1 ? LO : 0) + 2 * k;
+                    for (int t = 0; t < 2; ++t) {
                         const uint32_t acc = (u > 0 || k > 0 || t > 0) ? 1u : 0u;
-                        ptx::mma_ts(gtm + G_AA, gtm + S_A + acol, pbdesc + bsel, idescG, acc);
+                        ptx::mma_ts(gtm + G_AA, gtm + S_A + 8 * k, pbdesc + (t == 1 ? LO : 0) + 2 * k, idescG, acc);
                     }
                 }
                 // the next unit's scores overwrite J in tensor memory after those MMAs (a thread's MMAs run in order); the
@@ -165,13 +167,18 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
         float *cn = colneg + (warp - kFirstSoftmaxWarp) * 32;
         const float rowneg = m < M ? -0.5f * 1.4426950408889634f * a.lse_enc[((size_t)b * a.H + h) * M + m] : -INFINITY;
         const float2 sl2p = make_float2(a.sl2, a.sl2);
-        uint8_t *pb = sPB + (size_t)g * 2 * SM::kPbBytes + (size_t)row * GP::RB;   // this latent's row of the group's hi tile; lo: kPbBytes on
+        uint8_t *pb = sPB + (size_t)g * 2 * SM::kPbBytes + (size_t)row * GP::RB;   // this latent's row of the group's hi tile; 2 lo: kPbBytes on
         bool ok = true;
         const int units = 4 * mytiles;
+        auto column = [&](int u) {                              // lse_dec of this lane's token of unit u
+            const int n = (t_begin + g + NGS * (u >> 2)) * kTile + (u & 3) * UNIT + lane;
+            return u < units && n < a.N ? a.lse_dec[((size_t)b * a.N + n) * a.H + h] : INFINITY;
+        };
+        float ld = column(0);                                   // (fetched a unit ahead)
         for (int u = 0; ok && u < units; ++u) {
-            const int n = (t_begin + g + NGS * (u >> 2)) * kTile + (u & 3) * UNIT + lane;   // this lane fetches the shift of token n
             __syncwarp();
-            cn[lane] = n < a.N ? -0.5f * 1.4426950408889634f * a.lse_dec[((size_t)b * a.N + n) * a.H + h] : -INFINITY;
+            cn[lane] = -0.5f * 1.4426950408889634f * ld;
+            ld = column(u + 1);
             __syncwarp();
             if (!(ok = warp_wait(bar(S_FULL + g), u & 1, abort_flag, kErrSpectral | 5))) break;
             ptx::tc_fence_after();
@@ -189,11 +196,11 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
                 const uint32_t h0 = ptx::pack_bf16(p0, p1), h1 = ptx::pack_bf16(p2, p3);
                 hi[2 * k] = h0;
                 hi[2 * k + 1] = h1;
-                lo[2 * k] = ptx::pack_bf16(ptx::rest_of(make_float2(p0, p1), h0));
-                lo[2 * k + 1] = ptx::pack_bf16(ptx::rest_of(make_float2(p2, p3), h1));
+                const float2 l0 = ptx::rest_of(make_float2(p0, p1), h0), l1 = ptx::rest_of(make_float2(p2, p3), h1);
+                lo[2 * k] = ptx::pack_bf16(__fadd2_rn(l0, l0));
+                lo[2 * k + 1] = ptx::pack_bf16(__fadd2_rn(l1, l1));
             }
-            ptx::tmem_st16(scol, hi);                           // A operand: back over the scores, hi then lo
-            ptx::tmem_st16(scol + 16, lo);
+            ptx::tmem_st16(scol, hi);                           // A operand: back over the scores
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {                    // B operand: this latent's 64-byte rows, 16-byte chunks swizzled
                 *reinterpret_cast<uint4 *>(pb + ((ch ^ GP::swz(row)) << 4)) = make_uint4(hi[4 * ch], hi[4 * ch + 1], hi[4 * ch + 2], hi[4 * ch + 3]);
@@ -206,7 +213,7 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(bar(P_FULL + g));
         }
-        // the partial sum of G: this thread's lane holds row m
+        // the partial sum X: this thread's lane holds row m
         if (ok && units > 0) ok = warp_wait(bar(G_DONE + g), 0, abort_flag, kErrSpectral | 6);
         ptx::tc_fence_after();
         if (ok) {
@@ -237,16 +244,38 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
     if (threadIdx.x == 0 && *abort_flag != 0 && a.status != nullptr) atomicCAS(a.status, 0u, *abort_flag);
 }
 
-// Sum of the token splits into G [B,H,M,M].  One thread per element.
-static __global__ void __launch_bounds__(256)
-spectral_gram_reduce_kernel(const float *__restrict__ part, float *__restrict__ Gout, int splits, long heads, int M) {
-    const long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= heads * M * M) return;
-    const long bh = idx / ((long)M * M);
-    const int i = (int)((idx / M) % M), j = (int)(idx % M);
-    float s = 0.f;
-    for (int p = 0; p < splits; ++p) s += part[((size_t)p * heads + bh) * (size_t)kTile * kTile + (size_t)i * kTile + j];
-    Gout[idx] = s;
+// Sum of the token splits X into G [B,H,M,M] = (X + X^T) / 2.  grid = (pairs of 16 x 16 blocks (i, j), i <= j, heads): both blocks of X are
+// read by rows and meet in shared memory.
+constexpr int kGramTile = 16;
+__host__ __device__ constexpr int gram_tile_pairs(int M) { return ((M + kGramTile - 1) / kGramTile) * ((M + kGramTile - 1) / kGramTile + 1) / 2; }
+static __global__ void __launch_bounds__(kGramTile *kGramTile)
+spectral_gram_reduce_kernel(const float *part, float *Gout, int splits, long heads, int M) {
+    ptx::grid_launch();
+    ptx::grid_wait();
+    __shared__ float lower[kGramTile][kGramTile + 1], upper[kGramTile][kGramTile + 1];
+    int ti = 0, tj = blockIdx.x;                                // pair number -> (ti, tj), tj >= ti
+    for (int row = (M + kGramTile - 1) / kGramTile; tj >= row; --row) {
+        tj -= row;
+        ++ti;
+    }
+    tj += ti;
+    const int r = threadIdx.x / kGramTile, c = threadIdx.x % kGramTile;
+    const float *x = part + (size_t)blockIdx.y * kTile * kTile;
+    const size_t up = (size_t)(ti * kGramTile + r) * kTile + tj * kGramTile + c, low = (size_t)(tj * kGramTile + r) * kTile + ti * kGramTile + c;
+    float u = 0.f, l = 0.f;
+#pragma unroll 6
+    for (int p = 0; p < splits; ++p) {
+        const float *xp = x + (size_t)p * heads * kTile * kTile;
+        u += xp[up];
+        l += xp[low];
+    }
+    upper[r][c] = u;
+    lower[r][c] = l;
+    __syncthreads();
+    float *g = Gout + (size_t)blockIdx.y * M * M;
+    const int i = ti * kGramTile + r, j = tj * kGramTile + c, i2 = tj * kGramTile + r, j2 = ti * kGramTile + c;
+    if (i < M && j < M) g[(size_t)i * M + j] = 0.5f * (u + lower[c][r]);
+    if (ti != tj && i2 < M && j2 < M) g[(size_t)i2 * M + j2] = 0.5f * (upper[c][r] + l);
 }
 
 // Score q.k of one (latent, token) pair.  For float32 and float16 inputs the products are summed in double so that
@@ -413,9 +442,9 @@ spectral_jacobi_kernel(float *__restrict__ Gall, float *__restrict__ evals, floa
 
 // Eigenvalues alone (no U): Householder reduction to tridiagonal form, then bisection on Sturm counts.  One block per
 // matrix.  4/3 M^3 multiply-adds in M - 2 dependent steps, against about eight sweeps of M - 1 dependent steps of Jacobi
-// rotations over global memory: M = 128, eight matrices: 9.8 ms (Jacobi) -> 0.21 ms.  Each step is bound by the latency
+// rotations over global memory: M = 128, eight matrices: 9.8 ms (Jacobi) -> 0.16 ms.  Each step is bound by the latency
 // of its four barriers and two sums over a vector, not by arithmetic, so the matrix sits where it is reached fastest: in
-// registers up to M = 192 (spectral_tridiag_reg_kernel), else in shared memory (M <= 236) or in G's own storage.
+// registers up to M = 192 (spectral_tridiag_reg_kernel, which takes one barrier), else in shared memory (M <= 236) or in G's own storage.
 // Step k: v = the Householder vector of row k right of the diagonal (every warp forms the norm for itself, a lane its
 // columns lane + 32 t), p = beta A v by columns (A is symmetric; thread (column, group) walks the rows of its group),
 // w = p - (beta / 2) (p . v) v, A -= v w^T + w v^T.  Float32 like the rotations; worst error against float64 over random,
@@ -477,7 +506,7 @@ __device__ __forceinline__ int sturm_count(const EigPair<F> *q, int M, F x) {
 }
 constexpr int kBisectThreads = 128;
 static __global__ void __launch_bounds__(kBisectThreads)
-spectral_bisect_kernel(const float *__restrict__ tri, float *__restrict__ evals, int M) {
+spectral_bisect_kernel(const float *tri, float *evals, int M) {
     extern __shared__ double bis_sh[];
     __shared__ short counts[kBisectThreads];
     constexpr int TH = kBisectThreads;
@@ -485,6 +514,8 @@ spectral_bisect_kernel(const float *__restrict__ tri, float *__restrict__ evals,
     EigPair<float> *qf = reinterpret_cast<EigPair<float> *>(qd + M);
     const float *d = tri + (size_t)blockIdx.y * M * M, *e = d + M;
     const int t = threadIdx.x, lane = t & 31;
+    ptx::grid_launch();
+    ptx::grid_wait();
     double top = 0.0;                                           // Gershgorin, by every warp for itself
     bool bad = false;                                           // (the tridiagonal form of a matrix that was not finite)
     for (int i = lane; i < M; i += 32) {
@@ -552,117 +583,177 @@ __device__ __forceinline__ float eig_block_scale(unsigned mx, unsigned *sh32) {
 }
 __device__ __forceinline__ unsigned eig_magnitude(float x) { return __float_as_uint(fabsf(x)); }
 
-// The matrix in registers: NG groups of CX threads, thread (g, j) holds rows g, g + NG, ... of column j.  Vectors that are
-// read by rows are stored group-major (row g + NG r at g * R + r), so that four rows come with one load.
+// The matrix in registers: NG groups of CX / COLS threads, thread (g, j) holds rows g, g + NG, ... of column j (and j + CX / 2).  Columns that
+// are read by rows are stored group-major (row g + NG r at g * RP + r; RP, 4 or 8 mod 16 and odd multiples of these, keeps the groups' banks apart), so that four rows come with one load.
+// A step k takes one barrier.  Every warp holds v_k (a lane its elements lane + 32 c) and, from shared memory, the groups' sums of p = A v_k and
+// column k + 1 as it was before this step; so it has w_k, that column after the step, and with it v_(k+1) by itself.  It puts the rows
+// of its group where its lanes read them, updates its part of A while the norm's sum goes round, and multiplies it with the next v.  What every
+// warp does for itself costs shared-memory cycles by the warp, so there are few of them with much of A each.
+// With the bisection, us for eight matrices of 64 / 96 / 128 / 160 / 192: four barriers and two passes over A per step, 16 to 24 warps, a column per
+// thread 78 / 122 / 211 / 289 / 558; now 65 / 104 / 162 / 284 / 385 (128: with a column per thread 275, with two 170).
 template <int CX> struct EigReg {
-    static constexpr int NG = CX <= 64 ? 8 : 4, R = (CX / NG + 3) & ~3, kThreads = CX * NG;
+    static constexpr int NG = CX == 96 || CX == 192 ? 4 : 8, COLS = CX == 32 || CX == 96 ? 1 : CX == 64 || CX == 192 ? 2 : CX / 32, R = CX / NG;
+    static constexpr int RP = NG == 4 ? (R % 16 == 8 ? R : R + 8) : (R % 8 == 4 ? R : R + 4);
+    static constexpr int kThreads = CX / COLS * NG;
 };
 template <int CX>
 __global__ void __launch_bounds__(EigReg<CX>::kThreads)
-spectral_tridiag_reg_kernel(float *__restrict__ Gall, int M) {
-    constexpr int NG = EigReg<CX>::NG, R = EigReg<CX>::R, CW = CX / 32, TH = EigReg<CX>::kThreads;
-    __shared__ __align__(16) float sx[NG * R], sv[NG * R], sw[NG * R];   // column k as it is, v, w
-    __shared__ float part[NG][CX], diag[CX], off[CX];
+spectral_tridiag_reg_kernel(float *Gall, int M) {
+    using E = EigReg<CX>;
+    constexpr int NG = E::NG, R = E::R, RP = E::RP, COLS = E::COLS, CT = CX / COLS, CW = CX / 32, TH = E::kThreads;
+    static_assert(CT % 32 == 0 && R % 4 == 0, "a warp has one group's rows, four at a time");
+    __shared__ __align__(16) float sx[2][NG * RP];              // a column of A
+    __shared__ __align__(16) float rows[TH / 32][3][R];         // per warp: its group's rows of v, w and the next v
+    __shared__ float part[2][NG][CX], diag[CX], off[CX];
     __shared__ unsigned red[32];
-    const int t = threadIdx.x, lane = t & 31, j = t % CX, g = t / CX;
+    const int t = threadIdx.x, lane = t & 31, j = t % CT, g = t / CT, jc = j >> 5;
+    ptx::grid_launch();
+    ptx::grid_wait();
     float *G = Gall + (size_t)blockIdx.x * M * M;
-    float A[R];
+    float A[COLS][R];
     unsigned mx = 0u;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int i = g + NG * r;
-        A[r] = (j < M && i < M) ? G[(size_t)i * M + j] : 0.f;
-        mx = max(mx, eig_magnitude(A[r]));
-    }
+    for (int q = 0; q < COLS; ++q)
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = g + NG * r, c = j + q * CT;
+            A[q][r] = (c < M && i < M) ? G[(size_t)i * M + c] : 0.f;
+            mx = max(mx, eig_magnitude(A[q][r]));
+        }
     const float scale = eig_block_scale(mx, red);
 #pragma unroll
-    for (int r = 0; r < R; ++r) A[r] *= scale;
-    auto slot = [](int i) { return (i % NG) * R + i / NG; };    // where row i of a vector sits
-    auto dump = [&](int c) {                                    // column c of A to sx
-        if (j == c) {
+    for (int q = 0; q < COLS; ++q)
 #pragma unroll
-            for (int r = 0; r < R; r += 4) *reinterpret_cast<float4 *>(sx + g * R + r) = make_float4(A[r], A[r + 1], A[r + 2], A[r + 3]);
+        for (int r = 0; r < R; ++r) A[q][r] *= scale;
+    auto slot = [](int i) { return (i % NG) * RP + i / NG; };   // where row i of a column sits
+    auto dump = [&](float *to, int c) {                         // column c of A
+#pragma unroll
+        for (int q = 0; q < COLS; ++q)
+            if (j + q * CT == c) {
+#pragma unroll
+                for (int r = 0; r < R; r += 4) *reinterpret_cast<float4 *>(to + g * RP + r) = make_float4(A[q][r], A[q][r + 1], A[q][r + 2], A[q][r + 3]);
+            }
+    };
+    float *mine = &rows[t >> 5][0][0];
+    float v[CW], w[CW], x[CW], beta = 0.f, v1 = 0.f;            // this lane's elements of v, w and the column the next v is made from; v's first
+    auto select = [&](const float (&a)[CW], int c) {            // a[c], c the same for the whole warp
+        float y = a[0];
+#pragma unroll
+        for (int q = 1; q < CW; ++q) y = c == q ? a[q] : y;
+        return y;
+    };
+    auto put = [&](int which, const float (&a)[CW]) {           // the rows of this warp's group
+        if (lane % NG == g) {
+#pragma unroll
+            for (int c = 0; c < CW; ++c) mine[which * R + (lane + 32 * c) / NG] = a[c];
         }
     };
-    for (int i = t; i < NG * R; i += TH) sv[i] = sw[i] = 0.f;   // (rows beyond M stay zero)
-    dump(0);
-    __syncthreads();
-    for (int k = 0; k + 2 < M; ++k) {
-        float vl[CW], s = 0.f;                                  // this lane's elements of v (every warp has them all)
+    auto skip = [&](int r, int k) { return g + NG * (r + 3) <= k || g + NG * r >= M; };   // rows r ... r + 3 of the group are done, or none
+    float vj[COLS], wj[COLS];
+    auto update = [&](int r, int k) {                           // A -= v w^T + w v^T
+        if (skip(r, k)) return;
+        const float4 vr = *reinterpret_cast<const float4 *>(mine + r), wr = *reinterpret_cast<const float4 *>(mine + R + r);
+#pragma unroll
+        for (int q = 0; q < COLS; ++q) {
+            A[q][r] = fmaf(-vr.x, wj[q], fmaf(-wr.x, vj[q], A[q][r]));
+            A[q][r + 1] = fmaf(-vr.y, wj[q], fmaf(-wr.y, vj[q], A[q][r + 1]));
+            A[q][r + 2] = fmaf(-vr.z, wj[q], fmaf(-wr.z, vj[q], A[q][r + 2]));
+            A[q][r + 3] = fmaf(-vr.w, wj[q], fmaf(-wr.w, vj[q], A[q][r + 3]));
+        }
+    };
+    // x, column k, becomes the Householder vector that annihilates it below the subdiagonal, with beta; `between`(0 ... 4) goes between the
+    // steps of the sum
+    auto reflect = [&](int k, auto between) {
+        float s = 0.f;
+#pragma unroll
+        for (int c = 0; c < CW; ++c) s = lane + 32 * c > k + 1 ? fmaf(x[c], x[c], s) : s;
+        const float x0 = __shfl_sync(0xffffffffu, select(x, (k + 1) >> 5), (k + 1) & 31);
+        if (t == (k & 31)) diag[k] = select(x, k >> 5);
+#pragma unroll
+        for (int o = 0; o < 5; ++o) {
+            s += __shfl_xor_sync(0xffffffffu, s, 16 >> o);
+            between(o);
+        }
+        const float norm = sqrtf(fmaf(x0, x0, s)), alpha = x0 > 0.f ? -norm : norm, v0 = x0 - alpha;
+        beta = s > 0.f ? 2.f / fmaf(v0, v0, s) : 0.f;           // nothing to annihilate: beta = 0, nothing changes
+        if (t == 0) off[k] = s > 0.f ? alpha : x0;
+        v1 = v0;
 #pragma unroll
         for (int c = 0; c < CW; ++c) {
             const int i = lane + 32 * c;
-            vl[c] = i > k ? sx[slot(i)] : 0.f;
-            s = i > k + 1 ? fmaf(vl[c], vl[c], s) : s;
+            x[c] = i > k + 1 ? x[c] : i == k + 1 ? v0 : 0.f;
         }
-        s = eig_warp_sum(s);
-        const float x0 = sx[slot(k + 1)];
-        const float norm = sqrtf(fmaf(x0, x0, s)), alpha = x0 > 0.f ? -norm : norm;
-        const float v0 = x0 - alpha, beta = s > 0.f ? 2.f / fmaf(v0, v0, s) : 0.f;   // nothing to annihilate: beta = 0, nothing changes
+    };
+    // this thread's share of A (next v); column `next` for the step after
+    auto multiply = [&](int k, int buf, int next) {
+        put(2, x);
+        __syncwarp();
+        float p[COLS][4] = {};
 #pragma unroll
-        for (int c = 0; c < CW; ++c)
-            if (lane + 32 * c == k + 1) vl[c] = v0;
-        if (t < 32) {
+        for (int r = 0; r < R; r += 4) {
+            if (skip(r, k)) continue;
+            const float4 nv = *reinterpret_cast<const float4 *>(mine + 2 * R + r);
 #pragma unroll
-            for (int c = 0; c < CW; ++c) sv[slot(lane + 32 * c)] = vl[c];
-            if (t == 0) {
-                diag[k] = sx[slot(k)];
-                off[k] = s > 0.f ? alpha : x0;
+            for (int q = 0; q < COLS; ++q) {
+                p[q][0] = fmaf(A[q][r], nv.x, p[q][0]);
+                p[q][1] = fmaf(A[q][r + 1], nv.y, p[q][1]);
+                p[q][2] = fmaf(A[q][r + 2], nv.z, p[q][2]);
+                p[q][3] = fmaf(A[q][r + 3], nv.w, p[q][3]);
             }
         }
-        __syncthreads();
-        float p0 = 0.f, p1 = 0.f, p2 = 0.f, p3 = 0.f;
-        const float4 *v4 = reinterpret_cast<const float4 *>(sv + g * R), *w4 = reinterpret_cast<const float4 *>(sw + g * R);
 #pragma unroll
-        for (int r = 0; r < R; r += 4) {
-            if (g + NG * (r + 3) <= k) continue;                // these rows are done (uniform over the warp)
-            const float4 v = v4[r / 4];
-            p0 = fmaf(A[r], v.x, p0);
-            p1 = fmaf(A[r + 1], v.y, p1);
-            p2 = fmaf(A[r + 2], v.z, p2);
-            p3 = fmaf(A[r + 3], v.w, p3);
-        }
-        part[g][j] = (p0 + p1) + (p2 + p3);
+        for (int q = 0; q < COLS; ++q) part[buf][g][j + q * CT] = (p[q][0] + p[q][1]) + (p[q][2] + p[q][3]);
+        dump(sx[buf], next);
+    };
+    dump(sx[1], 0);
+    __syncthreads();
+    if (M >= 2) {
+#pragma unroll
+        for (int c = 0; c < CW; ++c) x[c] = sx[1][slot(lane + 32 * c)];
+        reflect(0, [](int) {});
+        multiply(-1, 0, 1);
+    } else if (t == 0) {
+        diag[0] = sx[1][0];
+    }
+    for (int k = 0; k + 2 < M; ++k) {
         __syncthreads();
-        float pv = 0.f;                                         // p . v, by every warp for itself
+        const int buf = k & 1;
+        float pv = 0.f;
 #pragma unroll
         for (int c = 0; c < CW; ++c) {
+            v[c] = x[c];
             float p = 0.f;
 #pragma unroll
-            for (int q = 0; q < NG; ++q) p += part[q][lane + 32 * c];
-            pv = fmaf(p, vl[c], pv);
+            for (int q = 0; q < NG; ++q) p += part[buf][q][lane + 32 * c];
+            x[c] = sx[buf][slot(lane + 32 * c)];
+            w[c] = p;
+            pv = fmaf(p, v[c], pv);
         }
+        put(0, v);
         pv = eig_warp_sum(pv);
         const float half = 0.5f * beta * (beta * pv);
-        float pj = 0.f;
 #pragma unroll
-        for (int q = 0; q < NG; ++q) pj += part[q][j];
-        const float vj = sv[slot(j)];                           // (zero up to k and beyond M)
-        const float wj = j > k ? fmaf(beta, pj, -half * vj) : 0.f;
-        if (g == 0) sw[slot(j)] = wj;
-        __syncthreads();
+        for (int c = 0; c < CW; ++c) w[c] = lane + 32 * c > k ? fmaf(beta, w[c], -half * v[c]) : 0.f;
+        put(1, w);
+        const float w1 = __shfl_sync(0xffffffffu, select(w, (k + 1) >> 5), (k + 1) & 31);
 #pragma unroll
-        for (int r = 0; r < R; r += 4) {
-            if (g + NG * (r + 3) <= k) continue;
-            const float4 v = v4[r / 4], w = w4[r / 4];
-            A[r] = fmaf(-v.x, wj, fmaf(-w.x, vj, A[r]));
-            A[r + 1] = fmaf(-v.y, wj, fmaf(-w.y, vj, A[r + 1]));
-            A[r + 2] = fmaf(-v.z, wj, fmaf(-w.z, vj, A[r + 2]));
-            A[r + 3] = fmaf(-v.w, wj, fmaf(-w.w, vj, A[r + 3]));
+        for (int c = 0; c < CW; ++c) x[c] = fmaf(-v[c], w1, fmaf(-w[c], v1, x[c]));
+#pragma unroll
+        for (int q = 0; q < COLS; ++q) {
+            vj[q] = select(v, jc + q * (CT / 32));
+            wj[q] = select(w, jc + q * (CT / 32));
         }
-        dump(k + 1);
-        __syncthreads();
+        __syncwarp();
+        reflect(k + 1, [&](int o) {
+#pragma unroll
+            for (int r = 0; r < R; r += 4)
+                if (r / 4 * 5 / (R / 4) == o) update(r, k);     // (o a constant after unrolling)
+        });
+        multiply(k, buf ^ 1, k + 2);
+        __syncwarp();                                           // (the rows are written again in the next step)
     }
-    if (M >= 2) {                                               // the last 2 x 2 block: column M - 2 is in sx
-        if (t == 0) {
-            diag[M - 2] = sx[slot(M - 2)];
-            off[M - 2] = sx[slot(M - 1)];
-        }
-        __syncthreads();
-        dump(M - 1);
-        __syncthreads();
-    }
-    if (t == 0) diag[M - 1] = sx[slot(M - 1)];
+    __syncthreads();
+    if (t == 0 && M >= 2) diag[M - 1] = sx[M & 1][slot(M - 1)];
     __syncthreads();
     for (int i = t; i < M; i += TH) {                           // the result takes the place of the matrix
         G[i] = diag[i] / scale;
