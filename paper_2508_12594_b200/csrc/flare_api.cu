@@ -55,7 +55,7 @@ int launches_for(const flare_desc_t *d, int op, int sms) {
     switch (op) {
         case FLARE_OP_ENCODE: return enc;
         case FLARE_OP_DECODE: return dec;                       // (given a workspace)
-        case FLARE_OP_FORWARD: return enc + dec;
+        case FLARE_OP_FORWARD: return small_forward_cluster(d, sms) ? 1 : enc + dec;
         case FLARE_OP_BACKWARD: {
             (void)sms;
             const int tok = (d->M + token_range(d) - 1) / token_range(d);
@@ -73,6 +73,8 @@ size_t forward_bytes(const flare_desc_t *d) {
 int forward_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, void *Y, float *Z, float *lse_enc,
                  float *lse_dec, void *workspace, cudaStream_t st, bool keep_status) {
     const WorkspaceLayout w = make_layout(partials_for(d, device_info().sms, false), (long)d->B * d->H * d->M, d->D, true);
+    if (const int cluster = small_forward_cluster(d, device_info().sms))
+        return forward_small_simt(d, cluster, Q, K, V, mask, Z, lse_enc, Y, lse_dec, keep_status ? nullptr : static_cast<uint32_t *>(workspace), st);
     if (Z == nullptr) Z = reinterpret_cast<float *>(static_cast<char *>(workspace) + w.z);
     const int rc = encode_impl(d, Q, K, V, mask, Z, lse_enc, workspace, st, false, keep_status);
     if (rc != FLARE_OK) return rc;

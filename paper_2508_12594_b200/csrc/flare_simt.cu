@@ -48,6 +48,35 @@ struct Decode {
 };
 
 template <typename T, int D>
+struct SmallForward {
+    static int run(const flare_desc_t *d, int cluster, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z, float *lse_enc,
+                   void *Y, float *lse_dec, uint32_t *header, cudaStream_t st) {
+        if constexpr (D > 32) {
+            return FLARE_ERR_UNSUPPORTED;
+        } else {
+            const size_t partials_at = encode_simt_smem<T, D>(1), smem = forward_small_smem<T, D>();
+            int WM = 1;
+            while (WM * 8 < d->M) WM *= 2;
+            auto launch = [&](auto size) -> int {
+                constexpr int CS = decltype(size)::value;
+                auto kernel = forward_small_simt_kernel<T, D, CS>;
+                static std::atomic<uint64_t> opt_in{0};
+                if (smem > 48 * 1024)
+                    if (int rc = ensure_big_smem(kernel, opt_in, (int)smem)) return rc;
+                static std::atomic<uint64_t> wide_opt_in{0};
+                if (CS > 8)
+                    if (int rc = ensure_wide_cluster(kernel, wide_opt_in)) return rc;
+                const int chunk = ((d->N + CS - 1) / CS + 7) / 8 * 8;
+                FLARE_CUDA(launch_after(kernel, dim3(CS, d->H, d->B), kSimtThreads, smem, st, (const T *)Q, (const T *)K, (const T *)V, mask, Z, lse_enc,
+                                        (T *)Y, lse_dec, header, d->H, d->N, d->M, WM, chunk, d->scale, (int)partials_at));
+                return FLARE_OK;
+            };
+            return cluster == 16 ? launch(std::integral_constant<int, 16>{}) : launch(std::integral_constant<int, 8>{});
+        }
+    }
+};
+
+template <typename T, int D>
 struct Token {
     static int run(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, const void *dY, const float *Z,
                    const float *dZ, const float *de, const float *lse_enc, const float *lse_dec, void *dK, void *dV, float *dd, cudaStream_t st) {
@@ -105,6 +134,10 @@ int encode_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const v
 int encode_dz_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *dY, const float *lse_dec,
                    float *pacc, cudaStream_t st) {
     return by_type<Encode>(d, true, d, p, Q, K, dY, (const uint8_t *)nullptr, lse_dec, (float *)nullptr, (float *)nullptr, pacc, st);
+}
+int forward_small_simt(const flare_desc_t *d, int cluster, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z, float *lse_enc,
+                       void *Y, float *lse_dec, uint32_t *header, cudaStream_t st) {
+    return by_type<SmallForward>(d, d, cluster, Q, K, V, mask, Z, lse_enc, Y, lse_dec, header, st);
 }
 int decode_simt(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st) {
     return by_type<Decode>(d, d, Q, K, Z, Y, lse_dec, st);

@@ -14,6 +14,8 @@
 // meet bank conflicts, with rows of D + 4 doubles.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "flare_ptx.cuh"
 #include "flare_common.cuh"
 
@@ -179,8 +181,9 @@ __device__ __forceinline__ void write_row(T *dst, const double2 (&acc)[SimtGeom<
 __device__ __forceinline__ float exp_diff(float x) { return ptx::ex2(x * 1.4426950408889634f); }
 
 // Running softmax state of the rows of a warp.  The reference m of a row (the same in the four threads of its quad) is not the running maximum
-// but a score within kSlack of it: exp(score - m) stays below e^20, and rescaling (a branch of the whole warp) is rare.
-constexpr float kNoScore = -1.0e30f, kSlack = 20.f;
+// but a score within kSlack of it: what weighs most has a small exponent (see exp_diff; with 20, lse_enc was off by up to 1.6 of its last place), and
+// rescaling, a branch of the whole warp, is rare.
+constexpr float kNoScore = -1.0e30f, kSlack = 6.f;
 template <int D, int RB>
 struct RowState {
     float m[RB], l[RB];                                              // (l: over the thread's own columns)
@@ -219,38 +222,31 @@ struct RowState {
     }
 };
 
-// Encode, split over N.  grid = (splits, H * mblocks, B); the block's eight warps are WM groups of 8 RB latents x WT = 8 / WM
-// shares of a tile's columns.  The shares are joined in shared memory: one partial (m, l, row) per latent and split.
-// kDz: the backward's dZ form: dY in place of V, weights exp(score - lse_dec[n]), no maximum and no sum.
+// What a block of the kernels below does with the tokens n0 ... n1 - 1 (there may be none): its eight warps are WM groups of 8 RB latents, from
+// rbase on, x WT = 8 / WM shares of a tile's columns.  Leaves the shares of every latent in shared memory, [WT][WM * RW rows] rows of (acc, m, l)
+// of D + 4 floats.  kDz: the backward's dZ form: dY in place of V, weights exp(score - lse_dec[n]), no maximum and no sum.
 template <typename T, int D, int RB, bool kDz>
-__global__ void __launch_bounds__(kSimtThreads, 2)
-encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
-                   const float *lse_dec, float *part_m, float *part_l,
-                   float *part_acc, int B, int H, int N, int M, int WM, int mblocks, int chunk, float scale) {
-    ptx::grid_launch();
-    ptx::grid_wait();
+__device__ __forceinline__ void encode_tokens(unsigned char *simt_smem, const T *Q, const T *K, const T *V, const uint8_t *key_mask, const float *lse_dec,
+                                              int b, int h, int H, int N, int M, int WM, int rbase, int n0, int n1, float scale) {
     using SG = SimtGeom<D>;
     constexpr int CT = SG::CT, RW = 8 * RB;
-    extern __shared__ __align__(16) unsigned char simt_smem[];
     double *sK = reinterpret_cast<double *>(simt_smem);             // [CT][DK]
     double *sV = sK + CT * SG::DK;                                  // [CT][DK]
     float *sBias = reinterpret_cast<float *>(sV + CT * SG::DK);     // [CT]: added to a column's scores (in the order of the MMA's indices)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int split = blockIdx.x, h = blockIdx.y / mblocks, mb = blockIdx.y % mblocks, b = blockIdx.z;
     const int WT = kSimtThreads / 32 / WM, wm = warp % WM, wt = warp / WM;
-    const int rbase = mb * WM * RW, r0 = rbase + wm * RW;
-    const int n0 = split * chunk, n1 = min(N, n0 + chunk);
+    const int r0 = rbase + wm * RW;
     const size_t stride = (size_t)H * D;
     const T *Kb = K + ((size_t)b * N * H + h) * D, *Vb = V + ((size_t)b * N * H + h) * D;
-    double aq[RB][D / 4];
-    load_rows<T, D, RB>(aq, Q + (size_t)h * M * D, D, r0, M, (double)scale);
-    RowState<D, RB> st;
-    st.clear();
     using Fetch = TileFetch<T, D, kSimtThreads>;
     unsigned char *raw = reinterpret_cast<unsigned char *>(sBias + CT);
     Fetch fk(raw), fv(raw + Fetch::kBytes);
     fk.load(Kb + n0 * stride, stride, n1 - n0);
     fv.load(Vb + n0 * stride, stride, n1 - n0);
+    double aq[RB][D / 4];
+    load_rows<T, D, RB>(aq, Q + (size_t)h * M * D, D, r0, M, (double)scale);
+    RowState<D, RB> st;
+    st.clear();
     for (int t0 = n0; t0 < n1; t0 += CT) {
         Fetch::wait();
         __syncthreads();
@@ -308,6 +304,22 @@ encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
         write_row<float, D>(dst, st.acc[rb], 1.0);
     }
     __syncthreads();
+}
+// Encode, split over N.  grid = (splits, H * mblocks, B).  One partial (m, l, row) per latent and split.
+template <typename T, int D, int RB, bool kDz>
+__global__ void __launch_bounds__(kSimtThreads, 2)
+encode_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask,
+                   const float *lse_dec, float *part_m, float *part_l,
+                   float *part_acc, int B, int H, int N, int M, int WM, int mblocks, int chunk, float scale) {
+    ptx::grid_launch();
+    ptx::grid_wait();
+    extern __shared__ __align__(16) unsigned char simt_smem[];
+    const int split = blockIdx.x, h = blockIdx.y / mblocks, b = blockIdx.z, rbase = blockIdx.y % mblocks * WM * 8 * RB;
+    const int n0 = split * chunk, n1 = min(N, n0 + chunk);
+    encode_tokens<T, D, RB, kDz>(simt_smem, Q, K, V, key_mask, lse_dec, b, h, H, N, M, WM, rbase, n0, n1, scale);
+    const float *sR = reinterpret_cast<const float *>(simt_smem);
+    constexpr int ROW = D + 4;
+    const int rows_here = WM * 8 * RB, WT = kSimtThreads / 32 / WM;
     const long rows = (long)B * H * M;
     for (int i = threadIdx.x; i < rows_here * D; i += kSimtThreads) {
         const int r = i / D, d = i % D, m = rbase + r;
@@ -335,6 +347,38 @@ template <typename T, int D> inline size_t encode_simt_smem(int RB) {
     return tiles > join ? tiles : join;
 }
 
+// mc latents, in tiles of doubles, against the token rows of a warp
+template <int D, int RB>
+__device__ __forceinline__ void decode_tile(RowState<D, RB> &st, const double (&ak)[RB][D / 4], const double *sQ, const double *sZ, int mc) {
+    const int lane = threadIdx.x & 31;
+    for (int nb = 0; nb < (mc + 7) / 8; ++nb) {
+        double2 c[RB];
+        mma_block<D, RB>(c, ak, sQ, nb);
+        const bool in0 = nb * 8 + column_slot(2 * (lane & 3)) < mc, in1 = nb * 8 + column_slot(2 * (lane & 3) + 1) < mc;
+        float2 sc[RB], p[RB];
+        double v[2][SimtGeom<D>::NB];
+        load_values<D>(v, sZ, nb);
+#pragma unroll
+        for (int rb = 0; rb < RB; ++rb) sc[rb] = make_float2(in0 ? (float)c[rb].x : -INFINITY, in1 ? (float)c[rb].y : -INFINITY);
+        st.weights(sc, p);
+        add_values<D, RB>(st.acc, p, v);
+    }
+}
+// rows r0 ... of Y and lse_dec, up to row `end`
+template <typename T, int D, int RB>
+__device__ __forceinline__ void decode_rows_out(const RowState<D, RB> &st, T *Y, float *lse_dec, int r0, int end, int b, int h, int N, int H) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int rb = 0; rb < RB; ++rb) {
+        const int n = r0 + 8 * rb + (lane >> 2);
+        const float l = quad_sum(st.l[rb]);
+        if (n >= end) continue;
+        const size_t tok = ((size_t)b * N + n) * H + h;
+        write_row<T, D>(Y + tok * D, st.acc[rb], 1.0 / (double)l);
+        if (lse_dec != nullptr && (lane & 3) == 0) lse_dec[tok] = st.m[rb] + logf(l);
+    }
+}
+
 // Decode: rows are tokens (8 RB per warp, the eight warps side by side), columns the latents.  grid = (ceil(N / (64 RB)), H, B).
 template <typename T, int D, int RB>
 __global__ void __launch_bounds__(kSimtThreads, 2)
@@ -351,15 +395,15 @@ decode_simt_kernel(const T *Q, const T *K, const float *Z, T *Y,
     const int r0 = (blockIdx.x * (kSimtThreads / 32) + warp) * 8 * RB;
     const T *Qh = Q + (size_t)h * M * D;
     const float *Zh = Z + ((size_t)b * H + h) * M * D;
-    double ak[RB][D / 4];
-    load_rows<T, D, RB>(ak, K + ((size_t)b * N * H + h) * D, (size_t)H * D, r0, N, (double)scale);
-    RowState<D, RB> st;
-    st.clear();
     unsigned char *raw = reinterpret_cast<unsigned char *>(sZ + CT * SG::DK);
     TileFetch<T, D, kSimtThreads> fq(raw);
     TileFetch<float, D, kSimtThreads> fz(raw + fq.kBytes);
     fq.load(Qh, D, M);
     fz.load(Zh, D, M);
+    double ak[RB][D / 4];
+    load_rows<T, D, RB>(ak, K + ((size_t)b * N * H + h) * D, (size_t)H * D, r0, N, (double)scale);
+    RowState<D, RB> st;
+    st.clear();
     for (int m0 = 0; m0 < M; m0 += CT) {
         fq.wait();
         __syncthreads();
@@ -372,31 +416,106 @@ decode_simt_kernel(const T *Q, const T *K, const float *Z, T *Y,
         }
         const int mc = min(CT, M - m0);
         if (r0 < N)
-            for (int nb = 0; nb < (mc + 7) / 8; ++nb) {
-                double2 c[RB];
-                mma_block<D, RB>(c, ak, sQ, nb);
-                const bool in0 = nb * 8 + column_slot(2 * (lane & 3)) < mc, in1 = nb * 8 + column_slot(2 * (lane & 3) + 1) < mc;
-                float2 sc[RB], p[RB];
-                double v[2][SG::NB];
-                load_values<D>(v, sZ, nb);
-#pragma unroll
-                for (int rb = 0; rb < RB; ++rb) sc[rb] = make_float2(in0 ? (float)c[rb].x : -INFINITY, in1 ? (float)c[rb].y : -INFINITY);
-                st.weights(sc, p);
-                add_values<D, RB>(st.acc, p, v);
-            }
+            decode_tile<D, RB>(st, ak, sQ, sZ, mc);
     }
-#pragma unroll
-    for (int rb = 0; rb < RB; ++rb) {
-        const int n = r0 + 8 * rb + (lane >> 2);
-        const float l = quad_sum(st.l[rb]);
-        if (n >= N) continue;
-        const size_t tok = ((size_t)b * N + n) * H + h;
-        write_row<T, D>(Y + tok * D, st.acc[rb], 1.0 / (double)l);
-        if (lse_dec != nullptr && (lane & 3) == 0) lse_dec[tok] = st.m[rb] + logf(l);
-    }
+    decode_rows_out<T, D, RB>(st, Y, lse_dec, r0, N, b, h, N, H);
 }
 template <typename T, int D> inline size_t decode_simt_smem() {
     return sizeof(double) * 2 * SimtGeom<D>::CT * SimtGeom<D>::DK + (sizeof(T) + sizeof(float)) * SimtGeom<D>::CT * D;
+}
+
+// The whole forward of a small problem in one launch: a cluster of CS blocks per (batch item, head), each with its share of the tokens.
+// Encode as above; the blocks join their partial rows through each other's shared memory, every block its share of the latents, whose Z it
+// hands to all; decode of the block's tokens against that Z.  Three launches take 2 to 3 us each whatever there is to do, and the host as long to
+// queue them.  (Which problems: see small_forward_cluster.)
+constexpr int kSmallMaxM = 64;
+template <int D> struct SmallGeom {
+    using SG = SimtGeom<D>;
+    static constexpr int PS = D + 2;                                 // a partial row in shared memory: acc, m, l
+    static_assert(SG::CT >= kSmallMaxM || D > 32, "all latents are one tile");
+};
+template <typename T, int D> inline size_t forward_small_smem() { return encode_simt_smem<T, D>(1) + sizeof(float) * kSmallMaxM * SmallGeom<D>::PS; }
+template <typename T, int D, int CS>
+__global__ void __cluster_dims__(CS, 1, 1) __launch_bounds__(kSimtThreads, 2)
+forward_small_simt_kernel(const T *Q, const T *K, const T *V, const uint8_t *key_mask, float *Z, float *lse_enc, T *Y, float *lse_dec,
+                          uint32_t *header, int H, int N, int M, int WM, int chunk, float scale, int partials_at) {
+    ptx::grid_launch();
+    ptx::grid_wait();
+    using SG = SimtGeom<D>;
+    constexpr int ROW = D + 4, PS = SmallGeom<D>::PS;
+    extern __shared__ __align__(16) unsigned char simt_smem[];
+    const int rank = blockIdx.x, h = blockIdx.y, b = blockIdx.z, warp = threadIdx.x >> 5;
+    const int n0 = min(N, rank * chunk), n1 = min(N, n0 + chunk);
+    if (header != nullptr && rank == 0 && h == 0 && b == 0 && threadIdx.x < kHeaderBytes / 4) header[threadIdx.x] = 0u;
+    encode_tokens<T, D, 1, false>(simt_smem, Q, K, V, key_mask, nullptr, b, h, H, N, M, WM, 0, n0, n1, scale);
+    const float *sR = reinterpret_cast<const float *>(simt_smem);
+    float *sP = reinterpret_cast<float *>(simt_smem + partials_at);
+    double *sQ = reinterpret_cast<double *>(simt_smem), *sZ = sQ + SG::CT * SG::DK;
+    const int rows_here = WM * 8, WT = kSimtThreads / 32 / WM;
+    for (int i = threadIdx.x; i < M * D; i += kSimtThreads) {
+        const int r = i / D, d = i % D;
+        float top = kNoScore, l = 0.f, z = 0.f;
+        for (int w = 0; w < WT; ++w) top = fmaxf(top, sR[((size_t)w * rows_here + r) * ROW + D]);
+        for (int w = 0; w < WT; ++w) {
+            const float *src = sR + ((size_t)w * rows_here + r) * ROW, f = exp_diff(src[D] - top);
+            l = fmaf(src[D + 1], f, l);
+            z = fmaf(src[d], f, z);
+        }
+        sP[r * PS + d] = z;
+        if (d == 0) {
+            sP[r * PS + D] = top;
+            sP[r * PS + D + 1] = l;
+        }
+    }
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    TileFetch<T, D, kSimtThreads>::wait();                           // (of a block without tokens)
+    TileFetch<T, D, kSimtThreads> fq(simt_smem + sizeof(double) * 2 * SG::CT * SG::DK + sizeof(float) * SG::CT);
+    fq.load(Q + (size_t)h * M * D, D, M);
+    cluster.sync();                                                  // partial rows are there, and tiles and shares are done with
+    fq.wait();
+    fq.put_double(sQ);
+    for (int i = threadIdx.x; i < ((M + 7) / 8 * 8 - M) * SG::DK; i += kSimtThreads) sZ[M * SG::DK + i] = 0.0;
+    const int mine = (M - rank + CS - 1) / CS;  // latents rank, rank + CS, ...
+    for (int i = threadIdx.x; i < mine * D; i += kSimtThreads) {
+        const int m = rank + i / D * CS, d = i % D;
+        float pm[CS], pl[CS], pz[CS], top = kNoScore;
+#pragma unroll
+        for (int p = 0; p < CS; ++p) {
+            const float *row = cluster.map_shared_rank(sP, p) + m * PS;
+            pm[p] = row[D];
+            pl[p] = row[D + 1];
+            pz[p] = row[d];
+        }
+#pragma unroll
+        for (int p = 0; p < CS; ++p) top = fmaxf(top, pm[p]);
+        float l = 0.f, z = 0.f;
+#pragma unroll
+        for (int p = 0; p < CS; ++p) {
+            const float f = exp_diff(pm[p] - top);
+            l = f > 0.f ? fmaf(pl[p], f, l) : l;
+            z = f > 0.f ? fmaf(pz[p], f, z) : z;
+        }
+        const bool none = top == kNoScore;                           // no valid token anywhere
+        z = none ? 0.f : z * (1.f / l);
+#pragma unroll
+        for (int p = 0; p < CS; ++p) cluster.map_shared_rank(sZ, p)[m * SG::DK + d] = (double)z;
+        const size_t row = ((size_t)b * H + h) * M + m;
+        if (Z != nullptr) Z[row * D + d] = z;
+        if (lse_enc != nullptr && d == 0) lse_enc[row] = none ? -INFINITY : top + logf(l);
+    }
+    const T *Kh = K + ((size_t)b * N * H + h) * D;
+    int r0 = n0 + warp * 8;
+    double ak[1][D / 4];
+    load_rows<T, D, 1>(ak, Kh, (size_t)H * D, r0, n1, (double)scale);   // (on their way across the barrier)
+    cluster.sync();
+    for (; r0 < n1; r0 += kSimtThreads / 32 * 8) {
+        if (r0 >= n0 + kSimtThreads / 32 * 8) load_rows<T, D, 1>(ak, Kh, (size_t)H * D, r0, n1, (double)scale);
+        RowState<D, 1> st;
+        st.clear();
+        decode_tile<D, 1>(st, ak, sQ, sZ, M);
+        decode_rows_out<T, D, 1>(st, Y, lse_dec, r0, n1, b, h, N, H);
+    }
 }
 
 }  // namespace flare

@@ -3,7 +3,7 @@ columns in tiles of 64 (32 at head width 64), against the oracle, forward and ba
 import pytest
 import torch
 
-from paper_2508_12594_b200 import workloads
+from paper_2508_12594_b200 import flare, workloads
 from tests._util import assert_forward_close, gpu_forward, oracle_forward
 from tests.test_gpu_backward import assert_grads_close, gpu_backward, oracle_backward
 
@@ -32,3 +32,29 @@ def test_scores_climb(oracle, B, H, N, M, D, dtype):
     inp.Q.mul_(torch.linspace(0.5, 2.0, M)[None, :, None].to(inp.Q.dtype))
     scale = 2.0 * D ** -0.5
     assert_forward_close(gpu_forward(inp, scale), oracle_forward(oracle, inp, scale), dtype, f"climb {dtype} B{B}H{H}N{N}M{M}D{D}")
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("B,H,N,M,D,masked", [
+    (1, 1, 1, 1, 4, 0.0), (1, 2, 7, 9, 16, 0.3), (1, 9, 1023, 64, 32, 0.1), (1, 9, 1024, 64, 32, 0.0), (1, 2, 2048, 32, 16, 0.0), (1, 3, 2041, 33, 8, 0.2),
+    (2, 5, 512, 64, 32, 0.2), (2, 5, 1024, 31, 16, 0.0), (4, 9, 1017, 64, 8, 0.5), (1, 10, 130, 17, 4, 1.0),
+])
+def test_forward_in_one_launch(B, H, N, M, D, masked, dtype):
+    """The form of small forwards against the general kernels (encode, then decode) on the same inputs: either side of the cluster sizes and of
+    the most tokens, lengths that leave blocks a part of a tile or nothing, every token masked.  Both round the same float32 steps in another order:
+    the bound of each against the oracle, twice; a stored float16 may land on the next value."""
+    inp = workloads.make_random(B, H, N, M, D, dtype=dtype, seed=N + M, masked_fraction=masked, k_std=0.8)
+    Q, K, V, mask = (None if t is None else t.cuda() for t in (inp.Q, inp.K, inp.V, inp.key_mask))
+    desc = flare.make_desc(Q, K, 0.7)
+    assert flare.flare_launch_count(desc, flare.OP_FORWARD) == 1
+    Y, Z, le, ld = flare.forward(Q, K, V, mask, 0.7, want_stats=True)
+    assert torch.equal(flare.forward(Q, K, V, mask, 0.7), Y)
+    Z2, le2, Y2, ld2 = torch.empty_like(Z), torch.empty_like(le), torch.empty_like(Y), torch.empty_like(ld)
+    flare.flare_encode(desc, Q, K, V, mask, Z2, le2, flare.alloc_workspace(desc, flare.OP_ENCODE))
+    flare.flare_decode(desc, Q, K, Z2, Y2, ld2)
+    for got, want, stored in ((Z, Z2, 0.0), (Y, Y2, 2.0 ** -10 if dtype == "f16" else 0.0), (le, le2, 0.0), (ld, ld2, 0.0)):
+        got, want = got.double(), want.double()
+        assert torch.equal(torch.isinf(got), torch.isinf(want))
+        got, want = got.nan_to_num(), want.nan_to_num()
+        rms = max(float(want.pow(2).mean().sqrt()), 1e-30)
+        assert float(((got - want).abs() - stored * want.abs()).max()) <= 4e-5 * rms
