@@ -485,7 +485,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     if (lane == 0) ptx::mbar_arrive(bar(P_FULL + (n & 1)));
                 }
             };
-            if (two_exp[c * 2 + second] == 0) units(std::false_type{});
+            if (!__any_sync(0xffffffffu, two_exp[c * 2 + second] != 0)) units(std::false_type{});
             else units(std::true_type{});
             if (lane == 0) ptx::mbar_arrive(bar(C_EMPTY + c));
         }
@@ -560,7 +560,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // own, took, us per training step -> now: 131072 tokens, M = 512, D = 32 (in two ranges, 448 latents at most) 1905 -> 1513; 1048576, M = 1024, D = 8 20967 -> 20025;
 // 32 x 4096, M = 128, D = 32 300 -> 283; 2 x 20011, M = 128, D = 64 187 -> 178; 16384, M = 32, D = 32 84.2 -> 85.1.
 constexpr float kFoldLog2 = 80.f, kFarLog2 = 46.f;
-constexpr int kTokFirstMathWarp = 4;                            // warps: 0 TMA producer, 1 MMA issue, 2 token constants, 4 on arithmetic
+constexpr int kTokFirstMathWarp = 4;                            // warps: 0 TMA producer, 1 and 3 MMA issue, 2 token constants, 4 on arithmetic
 
 struct BwdTokTcArgs {
     const __nv_bfloat16 *Q;    // [H,M,D]
@@ -587,7 +587,7 @@ template <int D>
 struct BwdTokSmem {
     using G = TileGeom<D>;
     static constexpr int UNIT = D == 64 ? 32 : 64, NCG = UNIT / 16, kThreads = (kTokFirstMathWarp + 4 * NCG) * 32;
-    static constexpr int kAccStride = D == 16 ? 64 : 3 * D;     // columns of an accumulator dV | U | T (whole blocks of 32)
+    static constexpr int kAccStride = 4 * D;                    // columns of an accumulator: dV | U | dV's share of c dZ lo | T
     // accumulators beside two buffers of three regions of ucols columns: the largest power of two up to four (as a logarithm)
     __device__ static __forceinline__ int log2_accs(int ucols) {
         const int fit = (512 - 6 * ucols) / kAccStride;
@@ -598,7 +598,7 @@ struct BwdTokSmem {
     // dQ on features of point clouds was 4.7e-6 to 5.4e-6 of its norm from float64 instead of 2.6e-6 to 3.0e-6), as long as the third fits
     // beside two tile stages.
     static constexpr int kThirdMost = D == 64 ? 160 : 0;
-    enum { ZH = 0, ZL = 1, DL = 2, DH = 3, QR = 4, Z3 = 5 };    // latent operands: Z hi, lo, c dZ lo, hi, Q (behind c dZ hi: see issue_outputs), third part of Z
+    enum { ZH = 0, ZL = 1, DH = 2, QR = 3, DL = 4, Z3 = 5 };    // latent operands: Z hi, lo, c dZ hi, Q, c dZ lo (one B operand: see outputs), third part of Z
     // tiles: [stage][K | V | dY]; latent operands with M rows each (M a multiple of 16); per latent the exponent's addend and -c de;
     // per token -lse_dec and r; the column groups' shares of dd
     __host__ __device__ static size_t lat_off(int stages, int M, int which) {
@@ -662,7 +662,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         const uint32_t math = 4 * cps;                          // warps that work on a unit
         for (int i = 0; i < NBARS; ++i)
             ptx::mbar_init(bar(i), i >= DD_FULL || (i >= ACC_EMPTY && i < DD_FULL) || (i >= P_FULL && i < C_FULL) ? math
-                                   : i >= C_EMPTY && i < ACC_FULL ? math + 1u : 1u);
+                                   : i >= C_EMPTY && i < ACC_FULL ? math + 1u : i < T_EMPTY || (i >= C_FULL && i < C_EMPTY) ? 1u : 2u);   // (two issuing warps)
         *abort_flag = 0;
         ptx::fence_mbar_init();
         ptx::prefetch_tensormap(&tmK);
@@ -793,19 +793,22 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             ptx::copy_async_commit();
         }
         ptx::copy_async_wait<0>();
-    } else if (warp == 1) {
-        if (ptx::elect_one()) {
+    } else if (warp == 1 || warp == 3) {
+        // Two issuing warps: warp 1 forms S and adds up T = dS Q, whose operand dS lies over S; warp 3 forms A and C' and adds up [dV | U], whose
+        // weights lie over A (kTwo: and C').  Each overwrites only what its own earlier instructions read.
+        auto issue = [&](auto second) {
+            constexpr bool kSecond = decltype(second)::value;
             // (descriptors as 32-bit low words beside a constant high word: see ptx::desc)
             constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), TILE = G::TILE_BYTES >> 4, STEP16 = (16 * G::RB) >> 4;
             const uint32_t LAT = (uint32_t)(M * G::RB) >> 4;    // from one latent operand to the next
             const uint32_t lat0 = ptx::desc_lo(ptx::smem_u32(smem + SM::lat_off(stages, M, 0)), 16), td0 = ptx::desc_lo(ptx::smem_u32(smem), 16);
-            // K-major to MN-major; the second block along N of [c dZ hi | Q] is one operand further on (LBO, bits 16-29)
+            // K-major to MN-major; the next blocks along N of [c dZ hi | Q | c dZ lo] are one operand further on each (LBO, bits 16-29)
             constexpr uint32_t MN = ptx::desc_lo(0, G::SBO) - ptx::desc_lo(0, 16);
-            const uint32_t MN2 = (LAT << 16) - ptx::desc_lo(0, 16);
+            const uint32_t MN3 = (LAT << 16) - ptx::desc_lo(0, 16);
             const int units = nu * nt;
             int s_stage = 0, s_wrap = 0, s_u = 0, o_u = 0, o_tile = 0, o_acc = 0, o_wrap = 0;
             bool o_two = false;
-            // S^T = K Q^T | A^T = dY Z^T | C'^T = V (c dZ)^T of the next unit, into buffer n & 1
+            // S^T = K Q^T, or A^T = dY Z^T | C'^T = V (c dZ)^T, of the next unit, into buffer n & 1
             auto tiles = [&](int n) -> bool {
                 if (s_u == 0) {
                     if (!ptx::mbar_wait(bar(T_FULL + s_stage), (uint32_t)s_wrap, abort_flag, kErrBwdTok | 3)) return false;
@@ -821,12 +824,15 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k) ptx::mma_ss(col, ptx::desc(ad + 2 * k, HI), ptx::desc(bd + 2 * k, HI), idescS, k > 0 || more);
                 };
-                product(0, SM::QR, false);
-                if (D == 64 && third) product(1, SM::Z3, false);   // (small parts first: fewer sums are truncated at their full size)
-                product(1, SM::ZL, D == 64 && third);
-                product(1, SM::ZH, true);
-                product(2, SM::DL, false);
-                product(2, SM::DH, true);
+                if constexpr (!kSecond) {
+                    product(0, SM::QR, false);
+                } else {
+                    if (D == 64 && third) product(1, SM::Z3, false);   // (small parts first: fewer sums are truncated at their full size)
+                    product(1, SM::ZL, D == 64 && third);
+                    product(1, SM::ZH, true);
+                    product(2, SM::DL, false);
+                    product(2, SM::DH, true);
+                }
                 ptx::mma_commit(bar(S_FULL + (n & 1)));
                 if (++s_u == nu) {
                     ptx::mma_commit(bar(T_EMPTY + s_stage));
@@ -835,10 +841,11 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
                 return true;
             };
-            // [dV | U] += W_dec [c dZ | Q], T += dS Q of unit o_u (kTwo: dV += W_enc (c dZ))
+            // T += dS Q, or [dV | U | dV'] += W_dec [c dZ hi | Q | c dZ lo], of unit o_u (kTwo: dV += W_enc (c dZ))
             auto outputs = [&](int n) {
-                constexpr uint32_t idesc1 = ptx::instr_desc_bf16(128, D, 0, 1), idesc2 = ptx::instr_desc_bf16(128, 2 * D, 0, 1);
-                const uint32_t bcol = tm + (n & 1) * bcols, V = tm + acc0 + o_acc * SM::kAccStride, U = V + D, T = V + 2 * D;
+                constexpr uint32_t idesc1 = ptx::instr_desc_bf16(128, D, 0, 1), idesc2 = ptx::instr_desc_bf16(128, 2 * D, 0, 1),
+                                   idesc3 = ptx::instr_desc_bf16(128, 3 * D, 0, 1);
+                const uint32_t bcol = tm + (n & 1) * bcols, V = tm + acc0 + o_acc * SM::kAccStride, U = V + D, V2 = U + D, T = V2 + D;
                 uint32_t ld = lat0 + (uint32_t)o_u * (UNIT / 16) * STEP16;
                 ptx::opaque(ld);
                 const int steps = (o_u == nu - 1 ? wlast : UNIT) / 16;
@@ -846,28 +853,28 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     constexpr bool kTwo = decltype(two)::value;
                     const uint32_t acc = (o_u > 0 || k > 0) ? 1u : 0u, s = bcol + 16 * k, w = s + ucols, e = w + ucols;   // (hi, and lo 8 columns on)
                     const uint32_t qd = ld + SM::QR * LAT + MN + k * STEP16, dl = ld + SM::DL * LAT + MN + k * STEP16, dh = ld + SM::DH * LAT + k * STEP16;
-                    if constexpr (!kTwo) {
-                        ptx::mma_ts(V, w, ptx::desc(dh + MN2, HI), idesc2, acc);
-                        ptx::mma_ts(V, w + 8, ptx::desc(dh + MN2, HI), idesc2, 1u);
-                        ptx::mma_ts(V, w, ptx::desc(dl, HI), idesc1, 1u);
+                    if constexpr (!kSecond) {
+                        ptx::mma_ts(T, s, ptx::desc(qd, HI), idesc1, acc);
+                        ptx::mma_ts(T, s + 8, ptx::desc(qd, HI), idesc1, 1u);
+                    } else if constexpr (!kTwo) {
+                        ptx::mma_ts(V, w, ptx::desc(dh + MN3, HI), idesc3, acc);
+                        ptx::mma_ts(V, w + 8, ptx::desc(dh + MN3, HI), idesc2, 1u);
                     } else {
                         ptx::mma_ts(V, e, ptx::desc(dh + MN, HI), idesc1, acc);
                         ptx::mma_ts(V, e + 8, ptx::desc(dh + MN, HI), idesc1, 1u);
-                        ptx::mma_ts(V, e, ptx::desc(dl, HI), idesc1, 1u);
+                        ptx::mma_ts(V2, e, ptx::desc(dl, HI), idesc1, acc);
                         ptx::mma_ts(U, w, ptx::desc(qd, HI), idesc1, acc);
                         ptx::mma_ts(U, w + 8, ptx::desc(qd, HI), idesc1, 1u);
                     }
-                    ptx::mma_ts(T, s, ptx::desc(qd, HI), idesc1, acc);
-                    ptx::mma_ts(T, s + 8, ptx::desc(qd, HI), idesc1, 1u);
                 };
-                if (!o_two) {
+                if (!kSecond || !o_two) {
                     if (steps == UNIT / 16) {
 #pragma unroll
                         for (int k = 0; k < UNIT / 16; ++k) step(std::false_type{}, k);
                     } else {
                         for (int k = 0; k < steps; ++k) step(std::false_type{}, k);
                     }
-                } else {
+                } else if constexpr (kSecond) {
                     for (int k = 0; k < steps; ++k) step(std::true_type{}, k);
                 }
             };
@@ -876,10 +883,12 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             for (int n = 0; ok && n < units; ++n) {
                 if (!ptx::mbar_wait(bar(P_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdTok | 4)) break;
                 if (o_u == 0) {
-                    const int c = o_tile % RING;
-                    if (!ptx::mbar_wait(bar(C_FULL + c), (o_tile / RING) & 1, abort_flag, kErrBwdTok | 5)) break;
-                    o_two = two_exp[c] != 0;
-                    ptx::mbar_arrive(bar(C_EMPTY + c));
+                    if (kSecond) {
+                        const int c = o_tile % RING;
+                        if (!ptx::mbar_wait(bar(C_FULL + c), (o_tile / RING) & 1, abort_flag, kErrBwdTok | 5)) break;
+                        o_two = two_exp[c] != 0;
+                        ptx::mbar_arrive(bar(C_EMPTY + c));
+                    }
                     if (!ptx::mbar_wait(bar(ACC_EMPTY + o_acc), (uint32_t)o_wrap ^ 1u, abort_flag, kErrBwdTok | 6)) break;
                 }
                 ptx::tc_fence_after();
@@ -892,6 +901,10 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
                 if (n + 2 < units) ok = tiles(n + 2);
             }
+        };
+        if (ptx::elect_one()) {
+            if (warp == 1) issue(std::false_type{});
+            else issue(std::true_type{});
         }
     } else if (warp >= kTokFirstMathWarp) {
         const int cg = (warp - kTokFirstMathWarp) >> 2, set = sets == 2 ? cg >> 1 : 0, mine = sets == 2 ? cg & 1 : cg;   // columns: 16 from 16 mine on
@@ -915,9 +928,9 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 const int which = (p ^ (p >> 2)) & 1, c0 = (p >> 1) * 8;   // dK or dV, and the first column
                 uint32_t x[8], y[8];
                 float dd = 0.f;
-                ptx::tmem_ld8(V + (which == 0 ? 2 * D : 0) + c0, x);
+                ptx::tmem_ld8(V + (which == 0 ? 3 * D : 0) + c0, x);
+                ptx::tmem_ld8(V + (which == 0 ? D : 2 * D) + c0, y);
                 if (which == 0) {
-                    ptx::tmem_ld8(V + D + c0, y);
                     const float *part = dds + ((k & 3) * NCG + set * cps) * kTile + row;
                     dd = part[0] + part[kTile];
                     if (cps == 4) dd += part[2 * kTile] + part[3 * kTile];
@@ -930,8 +943,11 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 #pragma unroll
                 for (int c = 0; c < PW; ++c) {                  // (narrow heads: the head's own columns)
                     f[c] = __uint_as_float(DR == 4 && off != 0 ? x[(4 + c) & 7] : x[c]);
-                    u[c] = which == 0 ? __uint_as_float(DR == 4 && off != 0 ? y[(4 + c) & 7] : y[c]) : 0.f;
-                    if (which != 0) f[c] *= r;
+                    u[c] = __uint_as_float(DR == 4 && off != 0 ? y[(4 + c) & 7] : y[c]);
+                    if (which != 0) {
+                        f[c] = (f[c] + u[c]) * r;
+                        u[c] = 0.f;
+                    }
                 }
                 if (in && kRanges) {
                     auto sums = [&](int at, float *v) {
@@ -1036,7 +1052,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     if (!warp_wait(bar(C_FULL + c), (i / RING) & 1, abort_flag, kErrBwdTok | 9)) break;
                     nld = ring[c * 2 * kTile + row];
                     rr = ring[(c * 2 + 1) * kTile + row];
-                    far = two_exp[c] != 0;
+                    far = __any_sync(0xffffffffu, two_exp[c] != 0);          // (the same for all: a vote says so to the compiler)
                     d2 = make_float2(0.f, 0.f);
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive(bar(C_EMPTY + c));
