@@ -1,6 +1,7 @@
 // Entry points of libflare: argument checks, workspaces, the order of the launches.  See include/flare.h for the contract.
 #include <mutex>
 #include "flare_host.h"
+#include "flare_reduce.cuh"
 #include "flare_micro.cuh"
 
 namespace flare {
@@ -46,20 +47,20 @@ int static_scratch_address(void **out) {
     return FLARE_OK;
 }
 
-// Kernels one call of `op` launches (the memset of the workspace header is not a kernel).
+// Kernels one call of `op` launches (among them the one that clears the workspace header, where it is not left to the merge).
 int launches_for(const flare_desc_t *d, int op, int sms) {
     // a fast form is followed by the exact form (which may exit at once)
     const int fe = use_fast_encode(d) ? 2 : 1, f = use_fast_decode(d) ? 2 : 1;
-    const int enc = fe + 1;                                     // encode, merge
+    const int enc = fe + 1 + (use_tc(d) ? 1 : 0);               // header, encode, merge
     const int dec = decode_in_ranges(d) ? f * decode_ranges(d) + 1 : f;   // ranges of latents and their combination
     switch (op) {
         case FLARE_OP_ENCODE: return enc;
-        case FLARE_OP_DECODE: return dec;                       // (given a workspace)
+        case FLARE_OP_DECODE: return 1 + dec;                   // header (given a workspace), decode
         case FLARE_OP_FORWARD: return small_forward_cluster(d, sms) ? 1 : enc + dec;
         case FLARE_OP_BACKWARD: {
             (void)sms;
             const int tok = (d->M + token_range(d) - 1) / token_range(d);
-            return 2 + tok + 2;                                 // dZ, its reduction; token kernel(s); dQ, its reduction
+            return 1 + 2 + tok + 2;                             // header; dZ, its reduction; token kernel(s); dQ, its reduction
         }
         default: return 0;
     }
@@ -338,7 +339,7 @@ int flare_decode(const flare_desc_t *desc, const void *Q_lat, const void *K, con
     if ((rc = require_device()) != FLARE_OK) return rc;
     if (workspace == nullptr) return decode_impl(desc, Q_lat, K, Z, Y, lse_dec, nullptr, (cudaStream_t)stream);
     if (workspace_bytes < flare_workspace_bytes(desc, FLARE_OP_DECODE)) return FLARE_ERR_WORKSPACE_TOO_SMALL;
-    FLARE_CUDA(cudaMemsetAsync(workspace, 0, kHeaderBytes, (cudaStream_t)stream));
+    if ((rc = clear_header(workspace, 0, (cudaStream_t)stream)) != FLARE_OK) return rc;
     char *range_scratch = decode_in_ranges(desc) ? static_cast<char *>(workspace) + kHeaderBytes : nullptr;
     return decode_impl(desc, Q_lat, K, Z, Y, lse_dec, static_cast<uint32_t *>(workspace), (cudaStream_t)stream,
                        range_scratch);
@@ -527,7 +528,7 @@ int flare_spectral_gram(const flare_desc_t *desc, const void *Q_lat, const void 
     const int sms = device_info().sms;
     if (workspace_bytes < spectral_bytes(desc, sms)) return FLARE_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = (cudaStream_t)stream;
-    FLARE_CUDA(cudaMemsetAsync(workspace, 0, kHeaderBytes, st));
+    if ((rc = clear_header(workspace, 0, st)) != FLARE_OK) return rc;
     return spectral_gram(desc, sms, Q_lat, K, lse_enc, lse_dec, G, workspace, st);
 }
 

@@ -101,7 +101,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
     (void)Y;  // dY_n . Y_n is rebuilt from float32 quantities instead of the rounded stored Y
     const long rows = (long)d->B * d->H * d->M;
     const SimtPlan pa = simt_plan(d, sms), pb = bwd_dq_plan(d, sms);
-    FLARE_CUDA(cudaMemsetAsync(ws, 0, kHeaderBytes, st));
+    if (const int rc = clear_header(ws, 0, st)) return rc;
     int dz_parts = pa.P;
     bool dz_on_tc = skip_pass_a;
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {

@@ -98,8 +98,7 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
     int rc, parts = P, parts_redo = 0;                         // partial results, and those of the exact form if it replaced them
     const uint32_t *redo = nullptr;
     if (use_tc(d)) {
-        const size_t kept = keep_status ? sizeof(uint32_t) : 0;
-        FLARE_CUDA(cudaMemsetAsync(base + kept, 0, kHeaderBytes - kept, st));
+        if ((rc = clear_header(base, keep_status ? 1 : 0, st)) != FLARE_OK) return rc;
         TcEncodePlan p = tc_encode_plan(d, di.sms);
         uint32_t *status = reinterpret_cast<uint32_t *>(base);
         // a caller that asks for lse_enc is saving Z for the backward: weights as two bf16 halves (see exp_chunk_hilo)
