@@ -56,7 +56,7 @@ int launch_spectral_gram_tc(const flare_desc_t *d, int sms, const void *Q, const
     a.tiles = (d->N + kTile - 1) / kTile;
     a.splits = spectral_splits(d, sms);
     FLARE_CUDA(launch_after(spectral_gram_tc_kernel<D>, dim3(a.splits, d->H, d->B), kTcThreads, SpectralSmem<D>::total, st, tmK, tmQ, a));
-    FLARE_CUDA(launch_after(spectral_gram_reduce_kernel, dim3(gram_tile_pairs(d->M), (unsigned)(d->B * d->H)), kGramTile * kGramTile, 0, st, a.part, G,
+    FLARE_CUDA(launch_after(spectral_gram_reduce_kernel, dim3((unsigned)(d->B * d->H), gram_tile_pairs(d->M)), kGramTile * kGramTile, 0, st, a.part, G,
                             a.splits * kSpectralGroups, (long)d->B * d->H, d->M));
     return FLARE_OK;
 }

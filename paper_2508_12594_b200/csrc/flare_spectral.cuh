@@ -244,7 +244,7 @@ spectral_gram_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
     if (threadIdx.x == 0 && *abort_flag != 0 && a.status != nullptr) atomicCAS(a.status, 0u, *abort_flag);
 }
 
-// Sum of the token splits X into G [B,H,M,M] = (X + X^T) / 2.  grid = (pairs of 16 x 16 blocks (i, j), i <= j, heads): both blocks of X are
+// Sum of the token splits X into G [B,H,M,M] = (X + X^T) / 2.  grid = (heads, pairs of 16 x 16 blocks (i, j), i <= j): both blocks of X are
 // read by rows and meet in shared memory.
 constexpr int kGramTile = 16;
 __host__ __device__ constexpr int gram_tile_pairs(int M) { return ((M + kGramTile - 1) / kGramTile) * ((M + kGramTile - 1) / kGramTile + 1) / 2; }
@@ -253,14 +253,14 @@ spectral_gram_reduce_kernel(const float *part, float *Gout, int splits, long hea
     ptx::grid_launch();
     ptx::grid_wait();
     __shared__ float lower[kGramTile][kGramTile + 1], upper[kGramTile][kGramTile + 1];
-    int ti = 0, tj = blockIdx.x;                                // pair number -> (ti, tj), tj >= ti
+    int ti = 0, tj = blockIdx.y;                                // pair number -> (ti, tj), tj >= ti
     for (int row = (M + kGramTile - 1) / kGramTile; tj >= row; --row) {
         tj -= row;
         ++ti;
     }
     tj += ti;
     const int r = threadIdx.x / kGramTile, c = threadIdx.x % kGramTile;
-    const float *x = part + (size_t)blockIdx.y * kTile * kTile;
+    const float *x = part + (size_t)blockIdx.x * kTile * kTile;
     const size_t up = (size_t)(ti * kGramTile + r) * kTile + tj * kGramTile + c, low = (size_t)(tj * kGramTile + r) * kTile + ti * kGramTile + c;
     float u = 0.f, l = 0.f;
 #pragma unroll 6
@@ -272,7 +272,7 @@ spectral_gram_reduce_kernel(const float *part, float *Gout, int splits, long hea
     upper[r][c] = u;
     lower[r][c] = l;
     __syncthreads();
-    float *g = Gout + (size_t)blockIdx.y * M * M;
+    float *g = Gout + (size_t)blockIdx.x * M * M;
     const int i = ti * kGramTile + r, j = tj * kGramTile + c, i2 = tj * kGramTile + r, j2 = ti * kGramTile + c;
     if (i < M && j < M) g[(size_t)i * M + j] = 0.5f * (u + lower[c][r]);
     if (ti != tj && i2 < M && j2 < M) g[(size_t)i2 * M + j2] = 0.5f * (upper[c][r] + l);

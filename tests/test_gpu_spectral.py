@@ -75,6 +75,22 @@ def test_gram_and_eigenvalues(case):
             assert np.abs(Uh[b, h].T @ Uh[b, h] - np.eye(M)).max() <= max(2e-4, 4e-6 * M)   # (rounding grows with the number of rotations)
 
 
+def test_gram_of_more_heads_than_a_launch_dimension():
+    """65600 matrices in one call (a launch takes 65535 blocks along y and z): the last ones are those of a call of their own, bit for bit."""
+    B, H, N, M, D = 8200, 8, 1, 16, 16
+    inp = workloads.make_random(B, H, N, M, D, dtype="bf16", seed=3)
+    Q, K = dev(inp.Q), dev(inp.K)
+    desc = flare.make_desc(Q, K)
+    le, ld = _forward_stats(Q, K, 1.0)
+    G = torch.empty(B, H, M, M, dtype=torch.float32, device="cuda")
+    flare.flare_spectral_gram(desc, Q, K, le, ld, G, flare.alloc_workspace(desc, flare.OP_SPECTRAL))
+    for b in (0, B - 1):
+        K1, le1, ld1, G1 = K[b:b + 1].clone(), le[b:b + 1].clone(), ld[b:b + 1].clone(), torch.empty(1, H, M, M, device="cuda")
+        d1 = flare.make_desc(Q, K1)
+        flare.flare_spectral_gram(d1, Q, K1, le1, ld1, G1, flare.alloc_workspace(d1, flare.OP_SPECTRAL))
+        assert torch.equal(G[b], G1[0])
+
+
 def test_spectral_error_paths():
     inp = workloads.make_random(1, 2, 64, 16, 16, dtype="bf16", seed=1)
     Q, K = dev(inp.Q), dev(inp.K)
