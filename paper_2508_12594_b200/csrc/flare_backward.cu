@@ -64,10 +64,7 @@ int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const v
     static std::atomic<uint64_t> smem_opt_in{0};
     if ((rc = ensure_big_smem(bwd_token_tc_kernel<D, DRT, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
     a.tiles = (d->N + kTile - 1) / kTile;
-    long per_head = sms / ((long)d->B * d->H);
-    if (per_head < 1) per_head = 1;
-    if (per_head > a.tiles) per_head = a.tiles;
-    FLARE_CUDA(launch_after(bwd_token_tc_kernel<D, DRT, kRanges>, dim3((unsigned)per_head, d->H, d->B), BwdTokSmem<D>::kThreads, BwdTokSmem<D>::total(a.stages, a.M), st,  tmK, tmV, tmG, a));
+    FLARE_CUDA(launch_after(bwd_token_tc_kernel<D, DRT, kRanges>, dim3((unsigned)token_splits(d, a.tiles, a.M, sms), d->H, d->B), BwdTokSmem<D>::kThreads, BwdTokSmem<D>::total(a.stages, a.M), st,  tmK, tmV, tmG, a));
     return FLARE_OK;
 }
 

@@ -222,6 +222,26 @@ inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes, i
     return best;
 }
 
+// CTAs per head of the token kernel of the backward, which leaves no partial results.  As many as fill the chip once, unless that leaves enough SMs
+// idle that several rounds are 2 % quicker; a CTA's start, where the head's latent operands are split and stored, counts as six units of 64
+// latents against a tile, and a fifth of a tile.  us per training step, once : several rounds: 32 heads (128 of 148 CTAs : 288), 50489 tokens, M = 624, D = 16
+// 2793 : 2689, 68334 tokens, M = 80, D = 8 734 : 710, 25344 tokens, M = 336, D = 32 890 : 875; 8 heads (144 : 296) of 1048576 tokens, M = 1024, D = 8
+// 18813 : 18640.
+// (A CTA per SM with a share of all heads' tiles in a row, which needs a loop over heads around the kernel: the loop costs 12 % of the kernel's time.)
+inline int token_splits(const flare_desc_t *d, int tiles, int mc, int sms) {
+    const double units = (double)((mc + 63) / 64);
+    const long heads = (long)d->B * d->H;
+    auto cost = [&](long s) { return (double)((heads * s + sms - 1) / sms) * ((double)((tiles + s - 1) / s) * units + 6.0 + 0.2 * units); };
+    int best = (int)std::min<long>(std::max(1L, sms / heads), tiles);
+    double best_cost = 0.98 * cost(best);
+    for (int s = best + 1; s <= std::min(tiles, sms); ++s)
+        if (cost(s) < best_cost) {
+            best = s;
+            best_cost = cost(s);
+        }
+    return best;
+}
+
 inline TcEncodePlan tc_encode_plan(const flare_desc_t *d, int sms) {
     TcEncodePlan p;
     p.tiles = (d->N + kTile - 1) / kTile;

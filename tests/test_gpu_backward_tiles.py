@@ -33,6 +33,7 @@ CASES = [  # B, H, N, M, D, masked_fraction, k_std
     (1, 2, 40000, 32, 32, 0.1, 0.8),      # two sets of warps, several tiles each
     (2, 1, 40000, 16, 8, 0.0, 0.8),
     (1, 2, 20001, 48, 16, 0.1, 0.8),
+    (8, 4, 20001, 256, 8, 0.0, 0.8),      # several rounds of CTAs over the chip, token side
 ]
 
 
