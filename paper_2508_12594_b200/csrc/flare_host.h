@@ -227,7 +227,7 @@ inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes, i
 // latents against a tile, and a fifth of a tile.  us per training step, once : several rounds: 32 heads (128 of 148 CTAs : 288), 50489 tokens, M = 624, D = 16
 // 2793 : 2689, 68334 tokens, M = 80, D = 8 734 : 710, 25344 tokens, M = 336, D = 32 890 : 875; 8 heads (144 : 296) of 1048576 tokens, M = 1024, D = 8
 // 18813 : 18640.
-// (A CTA per SM with a share of all heads' tiles in a row, which needs a loop over heads around the kernel: the loop costs 12 % of the kernel's time.)
+// (A CTA per SM with a share of all heads' tiles in a row, needs a loop over heads around the kernel's body, which made every training step 5 % slower.)
 inline int token_splits(const flare_desc_t *d, int tiles, int mc, int sms) {
     const double units = (double)((mc + 63) / 64);
     const long heads = (long)d->B * d->H;
