@@ -1,13 +1,24 @@
 // Entry points of libflare: argument checks, workspaces, the order of the launches.  See include/flare.h for the contract.
 #include <mutex>
 #include "flare_host.h"
-#include "flare_reduce.cuh"
 #include "flare_micro.cuh"
 
 namespace flare {
 thread_local char g_cuda_error[256] = "";
 DeviceInfo g_dev[64];
 std::atomic<int> g_path{FLARE_PATH_AUTO};
+
+// Clears the workspace header from word `first` on.  (A memset waits for the launch before it and holds up the one behind: 2 us more than this, which
+// overlaps with both.)
+__global__ void __launch_bounds__(kHeaderBytes / 4) clear_header_kernel(uint32_t *header, int first) {
+    ptx::grid_launch();
+    ptx::grid_wait();
+    if ((int)threadIdx.x >= first) header[threadIdx.x] = 0u;
+}
+int clear_header(void *workspace, int first, cudaStream_t st) {
+    FLARE_CUDA(launch_after(clear_header_kernel, 1, kHeaderBytes / 4, 0, st, static_cast<uint32_t *>(workspace), first));
+    return FLARE_OK;
+}
 }  // namespace flare
 
 using namespace flare;

@@ -429,6 +429,8 @@ int encode_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const v
 // dZ form: lse_dec given, dY in place of V, partial sums of dZ to pacc
 int encode_dz_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *dY, const float *lse_dec,
                    float *pacc, cudaStream_t st);
+// Clears the workspace header from word `first` on (one kernel for all callers: whichever call comes first loads it).
+int clear_header(void *workspace, int first, cudaStream_t st);
 int forward_small_simt(const flare_desc_t *d, int cluster, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z, float *lse_enc,
                        void *Y, float *lse_dec, uint32_t *header, cudaStream_t st);
 int decode_simt(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st);

@@ -12,18 +12,6 @@
 
 namespace flare {
 
-// Clears the workspace header from word `first` on.  (A memset waits for the launch before it and holds up the one behind: 2 us more than this, which
-// overlaps with both.)
-static __global__ void __launch_bounds__(kHeaderBytes / 4) clear_header_kernel(uint32_t *header, int first) {
-    ptx::grid_launch();
-    ptx::grid_wait();
-    if ((int)threadIdx.x >= first) header[threadIdx.x] = 0u;
-}
-inline int clear_header(void *workspace, int first, cudaStream_t st) {
-    FLARE_CUDA(launch_after(clear_header_kernel, 1, kHeaderBytes / 4, 0, st, static_cast<uint32_t *>(workspace), first));
-    return FLARE_OK;
-}
-
 constexpr int kReduceThreads = 256;
 
 // Slices per row: a power of two, P / slices about four, all of a row's lanes in one block.
