@@ -97,7 +97,9 @@ int flare_encode_partials(const flare_desc_t *desc);
 
 /*
  * Number of kernels one call of the given operation launches for `desc` on the current device (0 for an invalid
- * descriptor): e.g. encode, merge and decode for a forward; more where latents are worked off in ranges.
+ * descriptor); FLARE_OP_DECODE: given a workspace.  A forward is one kernel where a cluster per head does all of it (small
+ * float32 and float16 problems), else encode, merge and decode, for bfloat16 with one that clears the workspace header before
+ * them and with the exact form behind each fast one (flare_set_path); more where latents are worked off in ranges.
  */
 int flare_launch_count(const flare_desc_t *desc, int op);
 

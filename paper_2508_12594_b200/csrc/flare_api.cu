@@ -69,8 +69,7 @@ int launches_for(const flare_desc_t *d, int op, int sms) {
         case FLARE_OP_DECODE: return 1 + dec;                   // header (given a workspace), decode
         case FLARE_OP_FORWARD: return small_forward_cluster(d, sms) ? 1 : enc + dec;
         case FLARE_OP_BACKWARD: {
-            (void)sms;
-            const int tok = (d->M + token_range(d) - 1) / token_range(d);
+            const int tok = token_in_ranges(d) ? (d->M + token_range(d) - 1) / token_range(d) : 1;   // (the CUDA-core kernel knows no ranges)
             return 1 + 2 + tok + 2;                             // header; dZ, its reduction; token kernel(s); dQ, its reduction
         }
         default: return 0;

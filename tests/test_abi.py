@@ -110,3 +110,12 @@ def test_scratch_at_head_width_64_is_that_of_the_exact_form(lib):
     """D = 64 has no other form: one partial result per split and pair of latent blocks, up to 148 / (B H) splits."""
     desc = flare.FlareDesc(1, 4, 65536, 256, 64, flare.DTYPE_BF16, 1.0)
     assert flare.flare_encode_partials(desc) == 2 * (148 // 4)
+
+
+@pytest.mark.parametrize("M,D,dtype,kernels", [
+    (256, 64, flare.DTYPE_F32, 6), (528, 32, flare.DTYPE_F16, 6), (2048, 64, flare.DTYPE_F32, 6),     # one token kernel whatever M is
+    (192, 64, flare.DTYPE_BF16, 6), (208, 64, flare.DTYPE_BF16, 7), (400, 64, flare.DTYPE_BF16, 8),   # up to 192 latents a launch at D = 64
+    (512, 32, flare.DTYPE_BF16, 6), (528, 32, flare.DTYPE_BF16, 7)])
+def test_launch_count_of_a_backward(lib, M, D, dtype, kernels):
+    """Header, dZ and its reduction, the token kernel (bfloat16: one per range of latents), dQ and its reduction."""
+    assert flare.flare_launch_count(flare.FlareDesc(1, 2, 1000, M, D, dtype, 1.0), flare.OP_BACKWARD) == kernels
