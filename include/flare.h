@@ -157,15 +157,17 @@ int flare_forward(const flare_desc_t *desc, const void *Q_lat, const void *K, co
  *     dZ = W_dec^T dY;  dV = W_enc^T dZ;
  *     dS[m,n] = W_dec[n,m] (dY_n.Z_m - dY_n.Y_n) + W_enc[m,n] (dZ_m.V_n - dZ_m.Z_m);
  *     dQ_lat = scale * sum_b dS K;  dK = scale * dS^T Q_lat.
- * Z, lse_enc, lse_dec are the ones flare_forward wrote; Y is its output (part of the saved set; the present
- * kernels rebuild dY_n.Y_n = sum_m W_dec[n,m] (dY_n.Z_m) in float32 instead of reading the rounded Y, which
- * is markedly more accurate where the latent rows a token mixes are nearly equal).
+ * Z, lse_enc, lse_dec are the ones flare_forward wrote; Y is its output (part of the saved set).  dY_n.Y_n is formed
+ * from float32 quantities, sum_m W_dec[n,m] (dY_n.Z_m), which is markedly more accurate than the rounded Y where the
+ * latent rows a token mixes are nearly equal; on the tensor cores the rounded Y gives a first guess of it, no more (any
+ * other contents change the last bits of dK and dQ_lat, not what they are sums of).
  * bfloat16 inputs run all three passes (dZ; dK, dV; dQ_lat) on the tensor cores, with
  * every rounded factor of a cancelling sum carried as two bfloat16 halves (for dQ_lat at D = 64 as three parts, all 24
  * bits of a float32); float32 inputs run on the CUDA cores.
  * dQ_lat, dK, dV are overwritten.  Workspace: flare_workspace_bytes(desc, FLARE_OP_BACKWARD) bytes holding dZ,
- * per-split partial sums of dZ and dQ_lat, one float per (b, n, h), and, beyond 1024 bfloat16 latents (448 at
- * D = 32, 192 at D = 64), float32 sums of the rows of dK and dV; nothing of size N x M.
+ * per-split partial sums of dZ and dQ_lat, one float per (b, n, h) (bfloat16: two, and a few rows of D per head), and,
+ * beyond 1024 bfloat16 latents (512 at D = 32, 192 at D = 64), three float32 rows of D and one more float per (b, n, h):
+ * the sums over ranges of latents; nothing of size N x M.
  */
 int flare_backward(const flare_desc_t *desc, const void *Q_lat, const void *K, const void *V,
                    const uint8_t *key_mask, const void *Y, const void *dY, const float *Z, const float *lse_enc,

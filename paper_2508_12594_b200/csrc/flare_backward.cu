@@ -32,8 +32,9 @@ int launch_bwd_dq_tc_p(const flare_desc_t *d, const TcEncodePlan &p, bool padded
 
 int launch_bwd_dq_tc(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
                      const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
-                     const float *lse_dec, const float *dd, float *part, uint32_t *status, cudaStream_t st) {
+                     const float *lse_dec, const float *dd, const float *around, float *part, uint32_t *status, cudaStream_t st) {
     BwdDqTcArgs a;
+    a.around = around; a.around_rows = 1 + latent_blocks(d);
     a.Q = static_cast<const __nv_bfloat16 *>(Q);
     a.Z = Z; a.dZ = dZ; a.lse_enc = lse_enc; a.de = de; a.lse_dec = lse_dec; a.dd = dd;
     a.key_mask = mask; a.part = part; a.status = status;
@@ -59,8 +60,20 @@ int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const v
     if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
     if ((rc = make_token_map(&tmV, V, d, kTile, D)) != FLARE_OK) return rc;
     if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
-    a.stages = BwdTokSmem<D>::stages(a.M);
+    using SM = BwdTokSmem<D>;
+    a.stages = SM::stages(a.M);
     if (a.stages < 1) return FLARE_ERR_UNSUPPORTED;
+    if constexpr (SM::kSplitRegs) {
+        static std::atomic<int> launched_with{0};
+        int regs = launched_with.load(std::memory_order_relaxed);
+        if (regs == 0) {
+            cudaFuncAttributes attr;
+            FLARE_CUDA(cudaFuncGetAttributes(&attr, bwd_token_tc_kernel<D, DRT, kRanges>));
+            launched_with.store(regs = (attr.numRegs + 7) / 8 * 8, std::memory_order_relaxed);
+        }
+        constexpr int few = 32 * kTokFirstMathWarp, many = SM::kThreads - few;
+        if (regs * SM::kThreads < SM::kFewRegs * few + SM::kManyRegs * many) return FLARE_ERR_UNSUPPORTED;
+    }
     static std::atomic<uint64_t> smem_opt_in{0};
     if ((rc = ensure_big_smem(bwd_token_tc_kernel<D, DRT, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
     a.tiles = (d->N + kTile - 1) / kTile;
@@ -72,11 +85,12 @@ int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const v
 template <int D, int DRT>
 int launch_bwd_token_tc(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const void *dY,
                         const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
-                        const float *lse_dec, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st, int m0, int mc,
+                        const float *lse_dec, const float *around, const float *e, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st, int m0, int mc,
                         const float *dd_sums, float *kvacc) {
     BwdTokTcArgs a;
     a.Q = static_cast<const __nv_bfloat16 *>(Q);
     a.Z = Z; a.dZ = dZ; a.lse_enc = lse_enc; a.de = de; a.lse_dec = lse_dec; a.key_mask = mask;
+    a.around = around; a.around_rows = 1 + latent_blocks(d); a.e = e;
     a.dK = (__nv_bfloat16 *)dK; a.dV = (__nv_bfloat16 *)dV; a.dd = dd; a.status = status;
     a.B = d->B; a.H = d->H; a.N = d->N; a.M = mc;
     a.mtot = d->M; a.m0 = m0; a.first = m0 == 0; a.last = m0 + mc >= d->M; a.kvacc = kvacc; a.dd_sums = dd_sums;
@@ -95,9 +109,9 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
     float *dZ = reinterpret_cast<float *>(ws + w.dz);
     float *de = reinterpret_cast<float *>(ws + w.de);
     float *dd = reinterpret_cast<float *>(ws + w.dd);
-    (void)Y;  // dY_n . Y_n is rebuilt from float32 quantities instead of the rounded stored Y
     const long rows = (long)d->B * d->H * d->M;
     const SimtPlan pa = simt_plan(d, sms), pb = bwd_dq_plan(d, sms);
+    float *around = reinterpret_cast<float *>(ws + w.around), *e = reinterpret_cast<float *>(ws + w.e);
     if (const int rc = clear_header(ws, 0, st)) return rc;
     int dz_parts = pa.P;
     bool dz_on_tc = skip_pass_a;
@@ -105,7 +119,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
         if (!skip_pass_a && use_tc(d)) {
             const LeanPlan tp = dz_plan(d, sms);
             uint32_t *status = reinterpret_cast<uint32_t *>(ws);
-            const int rc = encode_dz_tc(d, tp, Q, K, dY, part, status, st, lse_dec);
+            const int rc = encode_dz_tc(d, tp, Q, K, dY, part, status, st, lse_dec, Z, around);
             if (rc != FLARE_OK) return rc;
             dz_parts = tp.splits;
             dz_on_tc = true;
@@ -115,7 +129,17 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
         if (const int rc = encode_dz_simt(d, pa, Q, K, dY, lse_dec, part, st)) return rc;
     }
     if (!skip_pass_a) {
-        FLARE_REDUCE(bwd_dz_reduce_kernel, rows, dz_parts, D, st, part, Z, dZ, de, dz_parts, rows);
+        GuessArgs guess{static_cast<const __nv_bfloat16 *>(Y), static_cast<const __nv_bfloat16 *>(dY), around, e, d->H, d->N, latent_blocks(d), 0, 0, 0};
+        unsigned guess_blocks = 0;                              // (the CUDA-core kernels have no use for e)
+        if (dz_on_tc) {
+            const GuessPlan g = guess_plan(d, sms);
+            guess.chunk = g.chunk; guess.chunks = g.chunks; guess.groups = g.groups;
+            guess_blocks = (unsigned)((long)d->B * g.chunks * g.groups);
+        }
+        const int slices = reduce_slices(dz_parts, D);
+        const unsigned row_blocks = reduce_blocks(rows, D, slices);
+        FLARE_CUDA(launch_after(bwd_dz_reduce_kernel<D / 4>, row_blocks + guess_blocks, kReduceThreads, 0, st, part, Z, dZ, de, dz_parts, rows, slices,
+                                (int)row_blocks, guess));
     }
     bool on_tc = false;
     int dq_parts = pb.P;
@@ -131,12 +155,12 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
             for (int k = 0; k < ranges; ++k) {
                 const int m0 = k * R;
                 const bool to_dd = (ranges - 1 - k) % 2 == 0;
-                if (const int rc = launch_bwd_token_tc<DK, DRT>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dK, dV, to_dd ? dd : dd_other, status,
+                if (const int rc = launch_bwd_token_tc<DK, DRT>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, around, e, dK, dV, to_dd ? dd : dd_other, status,
                                                                 st, m0, d->M - m0 < R ? d->M - m0 : R, to_dd ? dd_other : dd, kvacc))
                     return rc;
             }
             const TcEncodePlan p = tc_dq_plan(d, sms);
-            if (const int rc = launch_bwd_dq_tc(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, part, status, st)) return rc;
+            if (const int rc = launch_bwd_dq_tc(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, around, part, status, st)) return rc;
             dq_parts = p.P;
         }
     }

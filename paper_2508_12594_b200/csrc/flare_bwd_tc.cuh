@@ -125,6 +125,8 @@ struct BwdDqTcArgs {
     const float *lse_enc, *de; // [B,H,M]
     const float *lse_dec;      // [B,N,H]
     const float *dd;           // [B,H,N] (workspace)
+    const float *around;       // (workspace) a centre of the rows of Z at the head of each head's rows, see z_around
+    int around_rows;
     const uint8_t *key_mask;   // [B,N] or null
     float *part;               // [P][B*H*M][D] partial dQ rows (un-scaled)
     uint32_t *status;
@@ -224,9 +226,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     }
     // latent operands Q, Z_hi, Z_lo, dZ_hi, dZ_lo (D = 64: three parts of Z and dZ): zeros where there is no row (or, pair and narrow forms, no feature), then the rows
     const bool gaps = kPair || DRT != 0 || rows_here < kTile;
-    float *centre = reinterpret_cast<float *>(smem + SM::cst_off);                        // (the ring of constants is not in use yet)
-#pragma unroll
-    for (int w = 0; w < (kPair ? 2 : 1); ++w) z_centre<DR>(centre + w * DR, a.Z + ((size_t)b * a.H + h + w) * M * DR, M);
+    const float *centre = a.around + ((size_t)b * a.H + h) * a.around_rows * DR;
     if (gaps) {
         for (int i = threadIdx.x; i < SM::kLat * kTile * (G::RB / 16); i += kDqThreads)
             reinterpret_cast<uint4 *>(smem + SM::lat_off(0))[i] = make_uint4(0, 0, 0, 0);
@@ -242,7 +242,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         } else {
             stage_bf16<DG, DR>(smem + SM::lat_off(0), a.Q + q0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
             stage_hilo<DG, DR, kThird>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads,
-                                       centre + w * DR, UnitFactor(), smem + SM::lat_off(3));
+                                       centre + w * a.around_rows * DR, UnitFactor(), smem + SM::lat_off(3));
             constexpr int dz0 = 1 + SM::kParts;
             stage_hilo<DG, DR, kThird>(smem + SM::lat_off(dz0), smem + SM::lat_off(dz0 + 1), a.dZ + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x,
                                        kDqThreads, nullptr, UnitFactor(), smem + SM::lat_off(SM::kLat - 1));
@@ -540,10 +540,17 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // ------------------------------------------------------------------------------- pass B, token side (dK, dV)
 // Tokens on the lanes, latents on the columns, one sweep over the latents of a tile.  dd[n] = sum_m W_dec[n,m] A[n,m], which every dS of the
 // row needs, is known only when the row is done; but it enters linearly, so it is put in at the end:
-//     dK_n = scale (T_n - dd[n] U_n),   T_n = sum_m (W_dec A + W_enc (C - de))[n,m] q_m,   U_n = sum_m W_dec[n,m] q_m.
+//     dK_n = scale (T_n - (dd - e)[n] U_n),   T_n = sum_m (W_dec (A - e) + W_enc (C - de))[n,m] q_m,   U_n = sum_m W_dec[n,m] q_m.
+// e[n], any number that is near dd[n], keeps the two from being large and nearly equal, each with the rounding of its halves, where the rows of Z
+// that a token weighs are nearly equal or one of them has most of the weight.  It comes from the stored Y (bwd_guess), which is dd up to the rounding of
+// Y; A has had a row near the middle of Z taken out as well (z_around).  Against float64, what is left of dK's error when the rounding of the stored value
+// is taken off, of the norm, with dd formed in a sweep of its own first : e = 0 : e from Y.  M = 64, D = 32, mean largest weight 0.70 4.8e-7 : 1.1e-6 : 5.7e-7
+// (99th percentile of a row's 2.5e-5 : 1.9e-4 : 2.5e-6), 0.93 9.6e-6 : 1.2e-5 : 5.1e-6, 0.97 3.6e-5 : 3.8e-5 : 1.0e-5; features with
+// a mean of 1, M = 128, D = 32 2.3e-4 : 2.2e-6 : 2.2e-6.  e costs a packed addition per pair of columns and a pass over Y and dY, us per training step, e = 0 -> now: 16384 tokens, M = 32,
+// D = 32 77 -> 82; 32 x 4096, M = 128 266 -> 287; 2 x 20011, M = 128, D = 64 173 -> 180; 131072, M = 1024, D = 8 2472 -> 2530.
 // And W_enc = W_dec r[n] c[m] with r = 2^(lse_dec[n] - K), c = 2^(K - lse_enc[m]) and K in the middle of the latents' lse_enc, so that with
 // c dZ in the place of dZ one weight serves everything:
-//     T_n = sum_m W_dec (A + r (C' - c de)) q_m,   C' = V (c dZ)^T,     dV_n = r sum_m W_dec (c dZ)_m,
+//     T_n = sum_m W_dec (A - e + r (C' - c de)) q_m,   C' = V (c dZ)^T,     dV_n = r sum_m W_dec (c dZ)_m,
 // one exponential and one split of a weight per pair, and [dV | U] one accumulator whose contractions share their A operand.  dd goes to the
 // workspace for the dQ kernel.
 //
@@ -568,6 +575,8 @@ struct BwdTokTcArgs {
     const float *lse_enc, *de; // [B,H,M]
     const float *lse_dec;      // [B,N,H]
     const uint8_t *key_mask;   // [B,N] or null
+    const float *around, *e;   // (workspace) see BwdDqTcArgs; [B,N,H], see bwd_guess
+    int around_rows;
     __nv_bfloat16 *dK, *dV;    // [B,N,H,D]
     float *dd;                 // [B,H,N] (workspace)
     uint32_t *status;
@@ -593,23 +602,30 @@ struct BwdTokSmem {
         const int fit = (512 - 6 * ucols) / kAccStride;
         return fit >= 4 ? 2 : fit >= 2 ? 1 : 0;
     }
-    static constexpr int kRing = 4;                             // tiles of token constants on their way or in use
+    static constexpr int kRing = 4, kPlanes = D == 64 ? 2 : 3, kRingTile = kPlanes * kTile;   // tiles of token constants on their way or in use
+    // D = 16 (and the narrow forms): the arithmetic warps take registers that the other four leave.  Without, the pair of constants that e adds
+    // made the compiler put others together again for every pair of columns: 127 instead of 109 us (2 x 65536 tokens, M = 64, D = 16, 8 heads), 1000 instead
+    // of 910 (131072, M = 1024, D = 8).  At D = 32 the issuing warps then have too few: 118 instead of 106 (32 x 4096, M = 128).  The sum is what the
+    // block is launched with (20 warps of 96), which the host checks: the warps that ask for more wait for it.
+    static constexpr bool kSplitRegs = D == 16;
+    static constexpr int kFewRegs = 64, kManyRegs = 104;
+    static constexpr int kAlign = D == 64 ? 1024 : 512;         // (rows of 64 bytes are swizzled alike every 512: that much less to leave room for)
     // D = 64: dd[n] is subtracted from products that the dQ kernel forms of three parts of Z, so A is formed of three as well (with two,
     // dQ on features of point clouds was 4.7e-6 to 5.4e-6 of its norm from float64 instead of 2.6e-6 to 3.0e-6), as long as the third fits
     // beside two tile stages.
     static constexpr int kThirdMost = D == 64 ? 160 : 0;
     enum { ZH = 0, ZL = 1, DH = 2, QR = 3, DL = 4, Z3 = 5 };    // latent operands: Z hi, lo, c dZ hi, Q, c dZ lo (one B operand: see outputs), third part of Z
     // tiles: [stage][K | V | dY]; latent operands with M rows each (M a multiple of 16); per latent the exponent's addend and -c de;
-    // per token -lse_dec and r; the column groups' shares of dd
+    // per token -lse_dec, e and, but at D = 64, r; the column groups' shares of dd
     __host__ __device__ static size_t lat_off(int stages, int M, int which) {
         return (size_t)stages * 3 * G::TILE_BYTES + (size_t)which * M * G::RB;
     }
     __host__ __device__ static size_t cst_off(int stages, int M) { return lat_off(stages, M, M <= kThirdMost ? 6 : 5); }
     __host__ __device__ static size_t ring_off(int stages, int M) { return cst_off(stages, M) + 2 * sizeof(float) * M; }
-    __host__ __device__ static size_t dds_off(int stages, int M) { return ring_off(stages, M) + kRing * 2 * kTile * sizeof(float); }
+    __host__ __device__ static size_t dds_off(int stages, int M) { return ring_off(stages, M) + kRing * kRingTile * sizeof(float); }
     __host__ __device__ static size_t bar_off(int stages, int M) { return dds_off(stages, M) + 4 * NCG * kTile * sizeof(float); }
     __host__ __device__ static size_t total(int stages, int M) {
-        const size_t t = bar_off(stages, M) + 512 + 1024;
+        const size_t t = bar_off(stages, M) + 512 + kAlign;
         return t < kTcMinSmem ? kTcMinSmem : t;
     }
     static constexpr int kMaxStages = 6;
@@ -631,10 +647,10 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     using SM = BwdTokSmem<D>;
     constexpr int UNIT = SM::UNIT, NCG = SM::NCG, kThreads = SM::kThreads, kMaxSt = SM::kMaxStages, RING = SM::kRing, DR = DRT ? DRT : D;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = ptx::align_1024(smem_raw);
+    uint8_t *smem = ptx::align_smem<SM::kAlign>(smem_raw);
     const int M = a.M, stages = a.stages;
     float *cst = reinterpret_cast<float *>(smem + SM::cst_off(stages, M));      // [M] addend of W_enc's own exponent, [M] -c de
-    float *ring = reinterpret_cast<float *>(smem + SM::ring_off(stages, M));    // [RING][-lse_dec (log2 units) | r][token]
+    float *ring = reinterpret_cast<float *>(smem + SM::ring_off(stages, M));    // [RING][-lse_dec (log2 units) | -e | r][token]
     float *dds = reinterpret_cast<float *>(smem + SM::dds_off(stages, M));      // [4][column group][token]
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off(stages, M));
     enum { T_FULL = 0, T_EMPTY = T_FULL + kMaxSt, S_FULL = T_EMPTY + kMaxSt, P_FULL = S_FULL + 2, C_FULL = P_FULL + 2, C_EMPTY = C_FULL + RING,
@@ -673,7 +689,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::grid_launch();
     ptx::grid_wait();
     const size_t q0 = (size_t)h * a.mtot + a.m0, r0 = ((size_t)b * a.H + h) * a.mtot + a.m0;
-    z_centre<DR>(dds, a.Z + ((size_t)b * a.H + h) * a.mtot * DR, a.mtot);                    // (dds is not in use yet)
+    const float *centre = a.around + ((size_t)b * a.H + h) * a.around_rows * DR;
     float K, unfolded;                                          // (unfolded != 0: c is 1)
     {
         // K: the middle of the latents' lse_enc (log2 units), leaving out those that saw no valid token and those whose encode is switched off
@@ -714,12 +730,12 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         for (int w = 0; w < 5; ++w) lat[w] = smem + SM::lat_off(stages, M, w);
         if constexpr (DR == 4) {
             stage_rows4<D>(lat[SM::QR], a.Q + q0 * DR, M, off);
-            stage_rows4_hilo<D>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, off, dds);
+            stage_rows4_hilo<D>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, off, centre);
             stage_rows4_hilo<D>(lat[SM::DH], lat[SM::DL], a.dZ + r0 * DR, M, off, nullptr, factor);
         } else {
             stage_bf16<D, DR>(lat[SM::QR], a.Q + q0 * DR, M, 0, 0, threadIdx.x, kThreads);
-            if (third) stage_hilo<D, DR, true>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, dds, UnitFactor(), smem + SM::lat_off(stages, M, SM::Z3));
-            else stage_hilo<D, DR>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, dds);
+            if (third) stage_hilo<D, DR, true>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, centre, UnitFactor(), smem + SM::lat_off(stages, M, SM::Z3));
+            else stage_hilo<D, DR>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, centre);
             stage_hilo<D, DR>(lat[SM::DH], lat[SM::DL], a.dZ + r0 * DR, M, 0, 0, threadIdx.x, kThreads, nullptr, factor);
         }
         for (int m = threadIdx.x; m < M; m += kThreads) {
@@ -734,6 +750,10 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::tc_fence_after();
     const uint32_t tm = *tmem_slot;
     const uint32_t bcols = 3 * ucols, acc0 = 2 * bcols;         // columns of a buffer; the first accumulator
+    if constexpr (SM::kSplitRegs) {
+        if (warp < kTokFirstMathWarp) ptx::regs_down<SM::kFewRegs>();
+        else ptx::regs_up<SM::kManyRegs>();
+    }
 
     if (warp == 0) {
         if (ptx::elect_one()) {
@@ -748,15 +768,18 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
         }
     } else if (warp == 2) {
-        // Token constants of every tile: -lse_dec and r (0 for a token that takes no part in the encode softmax), or, in a tile that takes
-        // two exponentials, 0 or -inf in the place of r.  Fetched by asynchronous copies three tiles ahead.
+        // Token constants of every tile: -lse_dec, e and r (0 for a token that takes no part in the encode softmax), or, in a tile that takes
+        // two exponentials, 0 or -inf in the place of r.  Fetched by asynchronous copies three tiles ahead.  (D = 64: with a plane for r as well 160
+        // and 192 latents would have one tile stage instead of two.  There the last bit of e says whether a token takes part, and the arithmetic warps,
+        // which have registers to spare, form r.)
         constexpr int AH = RING - 1;
         auto fetch = [&](int i) {
-            float *at = ring + (i % RING) * 2 * kTile;
+            float *at = ring + (i % RING) * SM::kRingTile;
 #pragma unroll
             for (int e = 0; e < kTile / 32; ++e) {
                 const int r = e * 32 + lane, n = min((int)(blockIdx.x + i * gridDim.x) * kTile + r, a.N - 1);
                 ptx::copy_async4(ptx::smem_u32(at + r), a.lse_dec + ((size_t)b * a.N + n) * a.H + h);
+                ptx::copy_async4(ptx::smem_u32(at + kTile + r), a.e + ((size_t)b * a.N + n) * a.H + h);
             }
         };
         for (int k = 0; k < AH; ++k) {
@@ -766,7 +789,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         for (int i = 0; i < nt; ++i) {
             ptx::copy_async_wait<AH - 1>();
             __syncwarp();
-            float *at = ring + (i % RING) * 2 * kTile;
+            float *at = ring + (i % RING) * SM::kRingTile;
             float ld[kTile / 32];
             bool part[kTile / 32], far = unfolded != 0.f;
 #pragma unroll
@@ -776,12 +799,14 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 ld[e] = in ? at[r] * kBwdLog2e : INFINITY;
                 part[e] = in && (a.key_mask == nullptr || a.key_mask[(size_t)b * a.N + n] != 0);
                 at[r] = -ld[e];
+                const float ev = at[kTile + r], ne = fabsf(ev) <= 3.0e38f ? -ev : 0.f;
+                at[kTile + r] = SM::kPlanes == 3 ? ne : __uint_as_float((__float_as_uint(ne) & ~1u) | (part[e] ? 1u : 0u));
                 far = far || (part[e] && !(ld[e] - K <= kFarLog2));
             }
             far = __any_sync(0xffffffffu, far);
 #pragma unroll
-            for (int e = 0; e < kTile / 32; ++e)
-                at[kTile + e * 32 + lane] = far ? (part[e] ? 0.f : -INFINITY) : (part[e] ? ptx::ex2(ld[e] - K) : 0.f);
+            for (int e = 0; SM::kPlanes == 3 && e < kTile / 32; ++e)
+                at[2 * kTile + e * 32 + lane] = far ? (part[e] ? 0.f : -INFINITY) : (part[e] ? ptx::ex2(ld[e] - K) : 0.f);
             if (lane == 0) two_exp[i % RING] = far ? 1u : 0u;
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(bar(C_FULL + i % RING));
@@ -913,7 +938,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         const float2 sl2p = make_float2(a.sl2, a.sl2);
         const float *nle = cst + 16 * mine, *nde = nle + M;
         // Rows of dK and dV of the set's k-th tile: pieces of eight columns, in turn to the warps that share the tokens.
-        auto write_rows = [&](int k, float r) -> bool {
+        auto write_rows = [&](int k, float r, float ne) -> bool {
             constexpr int COLS = DR >= 16 ? DR : 8, PIECES = COLS / 4, PW = DR == 4 ? 4 : 8;
             const int i = set + k * sets, acc = i & ((1 << log_accs) - 1), tok_n = (int)(blockIdx.x + i * gridDim.x) * kTile + row;
             const bool in = tok_n < a.N;
@@ -927,7 +952,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             for (int p = PIECES <= 2 ? (mine + 2 * k) & (cps - 1) : mine; p < PIECES; p += cps) {
                 const int which = (p ^ (p >> 2)) & 1, c0 = (p >> 1) * 8;   // dK or dV, and the first column
                 uint32_t x[8], y[8];
-                float dd = 0.f;
+                float dd = 0.f;                                 // less e
                 ptx::tmem_ld8(V + (which == 0 ? 3 * D : 0) + c0, x);
                 ptx::tmem_ld8(V + (which == 0 ? D : 2 * D) + c0, y);
                 if (which == 0) {
@@ -936,7 +961,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     if (cps == 4) dd += part[2 * kTile] + part[3 * kTile];
                     const size_t at = ((size_t)b * a.H + h) * a.N + (in ? tok_n : 0);
                     if (kRanges && !a.first) dd += a.dd_sums[at];
-                    if (in && c0 == 0) a.dd[at] = dd;
+                    if (in && c0 == 0) a.dd[at] = !kRanges || a.last ? dd - ne : dd;
                 }
                 ptx::tmem_wait_ld();
                 float f[PW], u[PW];
@@ -982,7 +1007,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             return true;
         };
         // Sixteen columns of a unit, over which its weights go: dS over S, W_dec over A, W_enc (kTwo) over C, hi and lo of 16 latents side by side.
-        auto unit = [&](auto two, uint32_t col, int m, float2 nldp, float2 rp, float2 &d2) {
+        auto unit = [&](auto two, uint32_t col, int m, float2 nldp, float2 rp, float2 nep, float2 &d2) {
             constexpr bool kTwo = decltype(two)::value;
             uint32_t s[2][8], av[2][8], cv[2][8];
             auto load = [&](int p) {
@@ -1005,7 +1030,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     for (int e = 0; e < 2; ++e) {
                         const int j = 2 * (q + e), o = q + e;
                         const float2 sv = make_float2(__uint_as_float(s[p][j]), __uint_as_float(s[p][j + 1]));
-                        const float2 A = make_float2(__uint_as_float(av[p][j]), __uint_as_float(av[p][j + 1]));
+                        const float2 A = __fadd2_rn(make_float2(__uint_as_float(av[p][j]), __uint_as_float(av[p][j + 1])), nep);
                         const float2 C = make_float2(__uint_as_float(cv[p][j]), __uint_as_float(cv[p][j + 1]));
                         const float2 x = __ffma2_rn(sv, sl2p, nldp);
                         const float2 pd = make_float2(ptx::ex2(x.x), ptx::ex2(x.y));
@@ -1041,7 +1066,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         };
         // All units of the set's tiles in one loop; one more turn writes the last tile's rows.
         int k = 0, u = 0;                                       // tiles of this set done, unit of the next
-        float nld = 0.f, rr = 0.f, r_before = 0.f;
+        float nld = 0.f, rr = 0.f, ne = 0.f, r_before = 0.f, ne_before = 0.f;
         bool far = false;
         float2 d2 = make_float2(0.f, 0.f);
         while (true) {
@@ -1050,9 +1075,16 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (u == 0) {
                     const int c = i % RING;
                     if (!warp_wait(bar(C_FULL + c), (i / RING) & 1, abort_flag, kErrBwdTok | 9)) break;
-                    nld = ring[c * 2 * kTile + row];
-                    rr = ring[(c * 2 + 1) * kTile + row];
+                    const float *at = ring + c * SM::kRingTile + row;
+                    nld = at[0];
+                    ne = at[kTile];
                     far = __any_sync(0xffffffffu, two_exp[c] != 0);          // (the same for all: a vote says so to the compiler)
+                    if constexpr (SM::kPlanes == 3) {
+                        rr = at[2 * kTile];
+                    } else {
+                        const bool part = __float_as_uint(ne) & 1u;
+                        rr = far ? (part ? 0.f : -INFINITY) : (part ? ptx::ex2(-nld - K) : 0.f);
+                    }
                     d2 = make_float2(0.f, 0.f);
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive(bar(C_EMPTY + c));
@@ -1062,8 +1094,8 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (!warp_wait(bar(S_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdTok | 10)) break;
                 ptx::tc_fence_after();
                 if (u * UNIT + 16 * mine < M) {
-                    if (far) unit(std::true_type{}, col, u * UNIT, make_float2(nld, nld), make_float2(rr, rr), d2);
-                    else unit(std::false_type{}, col, u * UNIT, make_float2(nld, nld), make_float2(rr, rr), d2);
+                    if (far) unit(std::true_type{}, col, u * UNIT, make_float2(nld, nld), make_float2(rr, rr), make_float2(ne, ne), d2);
+                    else unit(std::false_type{}, col, u * UNIT, make_float2(nld, nld), make_float2(rr, rr), make_float2(ne, ne), d2);
                 }
                 if (u == nu - 1) dds[((k & 3) * NCG + cg) * kTile + row] = d2.x + d2.y;
                 ptx::tc_fence_before();
@@ -1073,12 +1105,13 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     if (u == nu - 1) ptx::mbar_arrive(bar(DD_FULL + (k & 3) + 4 * set));
                 }
             }
-            if (u == 0 && k > 0 && !write_rows(k - 1, r_before)) break;
+            if (u == 0 && k > 0 && !write_rows(k - 1, r_before, ne_before)) break;
             if (i >= nt) break;
             if (++u == nu) {
                 u = 0;
                 ++k;
                 r_before = far ? 1.f : rr;
+                ne_before = ne;
             }
         }
     }

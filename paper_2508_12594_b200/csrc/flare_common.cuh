@@ -82,4 +82,39 @@ __device__ __forceinline__ void z_centre(float *centre, const float *Z, int rows
     }
 }
 
+// The same row of a head's Z, and how far the 128 rows from r0 on reach from it, by feature, by one warp: around [1 + blocks of 128 latents][D].
+template <int D>
+__device__ __forceinline__ void z_around(float *around, const float *Z, int rows, int block) {
+    constexpr int L = D / 4, STEP = 32 / L;                     // lanes of a row, rows at a time
+    const int lane = threadIdx.x & 31, r0 = lane / L, r1 = min(rows, block * 128 + 128);
+    const float4 *z4 = reinterpret_cast<const float4 *>(Z) + lane % L;
+    float c[4] = {0.f, 0.f, 0.f, 0.f}, reach[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+        const float4 z = z4[(size_t)((long)(r0 + k * STEP) * rows / 32) * L];
+        c[0] += z.x; c[1] += z.y; c[2] += z.z; c[3] += z.w;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int o = L; o < 32; o <<= 1) c[k] += __shfl_xor_sync(0xffffffffu, c[k], o);
+        c[k] *= 1.f / 32.f;
+    }
+#pragma unroll 8
+    for (int r = block * 128 + r0; r < r1; r += STEP) {
+        const float4 z = z4[(size_t)r * L];
+        reach[0] = fmaxf(reach[0], fabsf(z.x - c[0])); reach[1] = fmaxf(reach[1], fabsf(z.y - c[1]));
+        reach[2] = fmaxf(reach[2], fabsf(z.z - c[2])); reach[3] = fmaxf(reach[3], fabsf(z.w - c[3]));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int o = L; o < 32; o <<= 1) reach[k] = fmaxf(reach[k], __shfl_xor_sync(0xffffffffu, reach[k], o));
+    if (lane < L) {
+        if (block == 0) reinterpret_cast<float4 *>(around)[lane] = make_float4(c[0], c[1], c[2], c[3]);
+        reinterpret_cast<float4 *>(around + (1 + block) * D)[lane] = make_float4(reach[0], reach[1], reach[2], reach[3]);
+    }
+}
+
 }  // namespace flare

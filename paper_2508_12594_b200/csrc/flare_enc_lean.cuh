@@ -35,7 +35,8 @@ struct LeanGeom {
     static constexpr int NG = UNIT + kAccCols <= 96 ? 5 : 4, COLS = NG == 5 ? 96 : 128;
     static_assert(UNIT + kAccCols <= COLS && NG * COLS <= 512, "tensor memory");
     static constexpr int kGuards = kKind == kLeanFast ? (NG == 4 ? 3 : 2) : 0;                  // warps that check the norms of the key rows
-    static constexpr int kFirstGuardWarp = 1 + NG, kFirstMathWarp = kFirstGuardWarp + kGuards;   // (warp 0: TMA; 1 to NG: MMA issue)
+    // (warp 0: TMA; 1 to NG: MMA issue; then the guards, or in the dZ form one warp that looks Z over for the kernels behind)
+    static constexpr int kFirstGuardWarp = 1 + NG, kFirstMathWarp = kFirstGuardWarp + kGuards + (kKind == kLeanDz ? 1 : 0);
     static constexpr int kThreads = (kFirstMathWarp + 4 * NG) * 32;
     static constexpr size_t kOnesBytes = kOnes ? (size_t)UNIT * G::RB : 0, kColBytes = (size_t)4 * NG * UNIT * sizeof(float);
     static constexpr size_t tail = (size_t)kTile * G::RB + ((kOnesBytes + 1023) & ~(size_t)1023) + kColBytes + 512 + 1024;
@@ -53,6 +54,8 @@ struct LeanGeom {
 struct EncodeLeanArgs {
     const __nv_bfloat16 *Q;   // [H,M,D]
     const float *lse_dec;     // [B,N,H]: dZ form
+    const float *Z;           // [B,H,M,D], and
+    float *around;            // [B * H][1 + blocks][D], dZ form: see z_around
     const uint8_t *key_mask;  // [B,N] or null
     float *part_m, *part_l, *part_acc;
     uint32_t *status;
@@ -266,6 +269,13 @@ encode_lean_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constan
                 if (lane == 0) ptx::mbar_arrive(bar(KV_EMPTY + sj));
             }
             if (!tame && lane == 0) *a.redo = 1u;
+        }
+    } else if (kDz && warp < LG::kFirstMathWarp) {
+        if (split == 0) {
+            for (int w = 0; w < (kPair ? 2 : 1); ++w) {
+                const size_t bh = (size_t)b * a.H + h + w;
+                z_around<DR>(a.around + bh * (1 + a.blocks) * DR, a.Z + bh * M * DR, M, lb);
+            }
         }
     } else if (warp >= LG::kFirstMathWarp) {
         const float2 sl2p = make_float2(a.sl2, a.sl2);

@@ -145,8 +145,9 @@ int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void 
 
 // Pass A of the backward: dY for V, lse_dec the decode log-sum-exp rows; partial sums to `part`.
 int encode_dz_tc(const flare_desc_t *d, const LeanPlan &p, const void *Q, const void *K, const void *dY, float *part,
-                 uint32_t *status, cudaStream_t st, const float *lse_dec) {
+                 uint32_t *status, cudaStream_t st, const float *lse_dec, const float *Z, float *around) {
     EncodeLeanArgs a{};
+    a.Z = Z; a.around = around;
     a.lse_dec = lse_dec; a.part_acc = part; a.status = status;
     return launch_lean<kLeanDz>(d, p, Q, K, dY, a, st);
 }

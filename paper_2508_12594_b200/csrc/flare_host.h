@@ -391,8 +391,25 @@ inline TcEncodePlan tc_dq_plan(const flare_desc_t *d, int sms) {
 
 inline SimtPlan bwd_dq_plan(const flare_desc_t *d, int sms) { return simt_plan_for(d, sms, d->D <= 16 ? 2 : 1); }
 
+// Blocks of 128 latents of a head in dZ's kernel.
+inline int latent_blocks(const flare_desc_t *d) { return (d->M + kTile - 1) / kTile; }
+
+// How the tokens are shared out to the blocks that form e (bwd_guess): five blocks an SM, of four turns at least.
+struct GuessPlan {
+    int chunk, chunks, groups;
+};
+inline GuessPlan guess_plan(const flare_desc_t *d, int sms) {
+    const int pieces = d->H * (d->D >= 8 ? d->D / 8 : 1), per = std::max(1, 256 / pieces);
+    GuessPlan p;
+    p.groups = (pieces + 255) / 256;
+    const long most = std::max(1L, 5L * sms / ((long)d->B * p.groups));
+    p.chunk = (int)std::max<long>((d->N + most - 1) / most, 4L * per);
+    p.chunks = (d->N + p.chunk - 1) / p.chunk;
+    return p;
+}
+
 struct BwdLayout {
-    size_t part, dz, de, dd, dd_other, kvacc, total;
+    size_t part, dz, de, dd, e, around, dd_other, kvacc, total;
     int P;
 };
 
@@ -414,6 +431,11 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     w.dz = off;   off += align_up(sizeof(float) * (size_t)rows * d->D);
     w.de = off;   off += align_up(sizeof(float) * (size_t)rows);
     w.dd = off;   off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
+    w.e = w.around = off;                                      // tensor-core kernels: see bwd_guess, z_around
+    if (use_tc(d)) {
+        w.around = off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
+        off += align_up(sizeof(float) * (size_t)(1 + latent_blocks(d)) * d->B * d->H * d->D);
+    }
     w.dd_other = w.kvacc = off;                                // over latent ranges: dd so far, and float32 sums of the rows
     if (token_in_ranges(d)) {
         w.kvacc = off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
@@ -445,7 +467,7 @@ int bwd_dq_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const v
 int encode_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z,
                 float *lse_enc, void *ws, cudaStream_t st, bool alone, bool keep_status = false);
 int encode_dz_tc(const flare_desc_t *d, const LeanPlan &p, const void *Q, const void *K, const void *dY, float *part,
-                 uint32_t *status, cudaStream_t st, const float *lse_dec);
+                 uint32_t *status, cudaStream_t st, const float *lse_dec, const float *Z, float *around);
 // range_scratch: decode_range_bytes(d) bytes, or null (then more than kDecodeMaxM latents take the CUDA-core kernel)
 int decode_impl(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec,
                 uint32_t *status, cudaStream_t st, char *range_scratch = nullptr);

@@ -12,10 +12,11 @@ namespace ptx {
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// The first 1024-byte boundary of dynamic shared memory.  By an offset: a pointer that has been an integer in between is generic to the
+// The first boundary of 1024 bytes (a smaller power of two where swizzled rows are narrower) of dynamic shared memory.  By an offset: a pointer that has been an integer in between is generic to the
 // compiler, and everything read or written through it goes by way of address translation instead of straight to shared memory (column constants in
 // the inner loops of the backward: training of a million points with 1024 latents 22.45 -> 21.23 ms, 32 x 4096 tokens 317 -> 303 us).
-__device__ __forceinline__ uint8_t *align_1024(uint8_t *raw) { return raw + (-smem_u32(raw) & 1023u); }
+template <uint32_t kBytes> __device__ __forceinline__ uint8_t *align_smem(uint8_t *raw) { return raw + (-smem_u32(raw) & (kBytes - 1)); }
+__device__ __forceinline__ uint8_t *align_1024(uint8_t *raw) { return align_smem<1024>(raw); }
 
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
@@ -34,6 +35,11 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
     return p != 0;
 }
+
+// Registers of a thread from here on, by all warps of a warp group (four from a multiple of four on).  The second waits until the block's warps have
+// given up as many.
+template <int n> __device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(n)); }
+template <int n> __device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(n)); }
 
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {

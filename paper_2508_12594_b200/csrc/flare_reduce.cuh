@@ -132,13 +132,66 @@ merge_kernel(const float *part_m, const float *part_l, const float *part_acc,
     if (lse_enc != nullptr && rm.lane == 0) lse_enc[rm.row] = none ? -INFINITY : top + logf(ls.x);
 }
 
-// dZ[row] = sum_p part[p][row] and de[row] = dZ_row . Z_row.
+// A first guess e[n] of dd[n] = dY_n . Y_n for the token kernel of the backward, from the stored Y: of dY_n . (Y_n - centre), with Y_n no further from
+// the centre of the rows of Z than these are (features with a mean: what rounding Y left must not be taken for a difference).  A block takes `chunk`
+// tokens of a batch item, in 16-byte pieces (8 at D = 4) as they lie in memory, so that a thread has the same piece of every token it reads.
+struct GuessArgs {
+    const __nv_bfloat16 *Y, *dY;   // [B,N,H,D]
+    const float *around;           // see z_around
+    float *e;                      // [B,N,H]
+    int H, N, blocks;              // blocks: of latents per head
+    int chunk, chunks, groups;     // groups: of at most kReduceThreads pieces of a token
+};
+template <int D> struct GuessGeom {
+    static constexpr int F = D >= 8 ? 8 : 4, LPR = D / F;       // features of a piece, pieces of a row
+};
+template <int D>
+__device__ __forceinline__ void bwd_guess(int block, const GuessArgs &a) {
+    using G = GuessGeom<D>;
+    const int pieces = a.H * G::LPR, here = min(pieces, kReduceThreads), per = kReduceThreads / here;   // of a token, of a token in a block; tokens at a time
+    const int group = block % a.groups, chunk = block / a.groups % a.chunks, b = block / a.groups / a.chunks;
+    const int piece = group * kReduceThreads + threadIdx.x % here, tok = threadIdx.x / here;
+    const bool live = tok < per && piece < pieces;
+    const int q = live ? piece : (int)threadIdx.x % G::LPR, h = q / G::LPR, f0 = q % G::LPR * G::F;
+    const float *around = a.around + ((size_t)b * a.H + h) * (1 + a.blocks) * D + f0;
+    float cen[G::F], most[G::F];
+#pragma unroll
+    for (int k = 0; k < G::F; ++k) {
+        cen[k] = around[k];
+        most[k] = around[D + k];
+    }
+    for (int m = 2; m <= a.blocks; ++m)
+#pragma unroll
+        for (int k = 0; k < G::F; ++k) most[k] = fmaxf(most[k], around[m * D + k]);
+    struct alignas(2 * G::F) Piece { __nv_bfloat162 w[G::F / 2]; };
+    const Piece *Y = reinterpret_cast<const Piece *>(a.Y) + (size_t)b * a.N * pieces + q, *dY = reinterpret_cast<const Piece *>(a.dY) + (size_t)b * a.N * pieces + q;
+    const int n1 = min(a.N, (chunk + 1) * a.chunk);
+#pragma unroll 4
+    for (int n = chunk * a.chunk + tok; n - tok < n1; n += per) {
+        const size_t at = (size_t)min(n, n1 - 1) * pieces;
+        const Piece y = Y[at], g = dY[at];
+        float sum = 0.f;
+#pragma unroll
+        for (int k = 0; k < G::F; ++k) {
+            const float yk = k & 1 ? __high2float(y.w[k / 2]) : __low2float(y.w[k / 2]), gk = k & 1 ? __high2float(g.w[k / 2]) : __low2float(g.w[k / 2]);
+            sum = fmaf(gk, fminf(fmaxf(yk - cen[k], -most[k]), most[k]), sum);
+        }
+#pragma unroll
+        for (int o = 1; o < G::LPR; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (live && f0 == 0 && n < n1) a.e[((size_t)b * a.N + n) * a.H + h] = sum;
+    }
+}
+
+// dZ[row] = sum_p part[p][row] and de[row] = dZ_row . Z_row; blocks from row_blocks on: e, see bwd_guess.
 template <int L>
 __global__ void __launch_bounds__(kReduceThreads)
-bwd_dz_reduce_kernel(const float *part, const float *Z, float *dZ, float *de,
-                     int P, long rows, int slices) {
+bwd_dz_reduce_kernel(const float *part, const float *Z, float *dZ, float *de, int P, long rows, int slices, int row_blocks, GuessArgs guess) {
     ptx::grid_launch();
     ptx::grid_wait();
+    if ((int)blockIdx.x >= row_blocks) {
+        bwd_guess<4 * L>((int)blockIdx.x - row_blocks, guess);
+        return;
+    }
     const RowMap rm = row_map<L>(slices);
     const bool live = rm.row < rows;
     const long at = (live ? rm.row : rows - 1) * L + rm.lane;

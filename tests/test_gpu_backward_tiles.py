@@ -5,7 +5,8 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2508_12594_b200 import workloads
+from paper_2508_12594_b200 import flare, workloads
+from tests._util import dev, to_np64
 from tests.test_gpu_backward import assert_grads_close, gpu_backward, oracle_backward
 
 pytestmark = pytest.mark.gpu
@@ -77,3 +78,54 @@ def test_wide_heads_keep_float32_accuracy_of_dq(oracle, B, H, N, M, masked):
     inp = workloads.make_random(B, H, N, M, 64, dtype="bf16", seed=N + M, masked_fraction=masked, with_dy=True, k_std=0.125)
     got, want = gpu_backward(inp)["dQ"], oracle_backward(oracle, inp)["dQ"]
     assert np.linalg.norm(got - want) <= 2.0 ** -18 * np.linalg.norm(want)
+
+
+def dk_error_bound(inp):
+    """What dK of one batch item may be off by before it is rounded to bfloat16, element by element (float64).  u = 2^-17 covers two roundings of a
+    value in bf16 halves.  Per (token, latent): the halves of W_dec (A - e) and of W_enc (C - de), |A - e| <= |A - dd| + |dd - e| with e from Y as it is
+    stored (a 2^-7 of |dY| |Y|); those of W_dec against dd - e; the errors of A (Z in halves, and of weights in halves), as far as they do not move
+    all of a token's alike; those of C (dZ, of weights in halves); the weights' own (a rounded score and the exponential)."""
+    u = 2.0 ** -17
+    Q, K, V, dY = (t.double().numpy() for t in (inp.Q, inp.K, inp.V, inp.dY))
+    out = np.zeros(K.shape)
+    for h in range(Q.shape[0]):
+        q, k, v, g = Q[h], K[0, :, h], V[0, :, h], dY[0, :, h]
+        S = k @ q.T
+        dec, enc = np.exp(S - S.max(1, keepdims=True)), np.exp(S - S.max(0))
+        dec /= dec.sum(1, keepdims=True)
+        enc /= enc.sum(0)
+        Z, Z_abs, dZ, dZ_abs = enc.T @ v, enc.T @ np.abs(v), dec.T @ g, dec.T @ np.abs(g)
+        centred = Z - Z.mean(0)
+        A, C = g @ centred.T, v @ dZ.T
+        dd, de = (dec * A).sum(1, keepdims=True), (enc * C).sum(0)
+        guess = 2.0 ** -7 * (np.abs(g) * np.abs(dec @ Z)).sum(1, keepdims=True)
+        weight = 2.0 ** -21 + 2.0 ** -22 * np.abs(S).max(1, keepdims=True)
+        a = u * np.abs(g) @ (np.abs(centred) + Z_abs).T
+        others = (1.0 - dec) * a + (dec * a).sum(1, keepdims=True) - dec * a
+        c = 4 * u * (np.abs(v) @ dZ_abs.T + (dZ_abs * Z_abs).sum(1))
+        out[0, :, h] = (dec * ((u + weight) * np.abs(A - dd) + 2 * u * guess + others) + enc * ((u + weight) * np.abs(C - de) + c)) @ np.abs(q)
+    return out
+
+
+@pytest.mark.parametrize("H,N,M,D,k_std", [(2, 1200, 64, 32, 2.0), (2, 1200, 64, 32, 5.0), (2, 1500, 48, 16, 4.0), (2, 1000, 96, 64, 2.0), (2, 900, 208, 64, 2.0),
+                                           (4, 1100, 64, 8, 6.0), (4, 1000, 32, 4, 8.0), (2, 700, 640, 32, 3.0), (2, 2000, 64, 32, 0.2)])
+def test_rows_of_peaked_softmaxes(oracle, H, N, M, D, k_std):
+    """A token that follows one latent has a small row of dK, left of large numbers: every element of it within what its own terms allow.  (Without
+    e, 20 to 75 times that; with dd formed first, in a sweep of its own, 13 to 70 times; now at most 0.15 of it.)"""
+    inp = workloads.make_random(1, H, N, M, D, dtype="bf16", seed=N + M, with_dy=True, k_std=k_std)
+    got, want = gpu_backward(inp)["dK"], oracle_backward(oracle, inp)["dK"]
+    half_ulp = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(want), 1e-300))) - 8)
+    assert (np.abs(got - want) <= half_ulp + dk_error_bound(inp)).all()
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), 0.0, 1e30])
+@pytest.mark.parametrize("M,D", [(64, 32), (144, 16), (208, 64)])
+def test_any_stored_output(oracle, M, D, value):
+    """The stored Y is a first guess only: what a caller left there has no say in the gradients."""
+    inp = workloads.make_random(2, 2, 300, M, D, dtype="bf16", seed=M, with_dy=True)
+    Q, K, V, dY = (dev(t) for t in (inp.Q, inp.K, inp.V, inp.dY))
+    desc = flare.make_desc(Q, K)
+    Y, Z, le, ld = flare.forward(Q, K, V, want_stats=True)
+    dQ, dK, dV = torch.empty(Q.shape, device="cuda"), torch.empty_like(K), torch.empty_like(V)
+    flare.flare_backward(desc, Q, K, V, None, Y.fill_(value), dY, Z, le, ld, dQ, dK, dV, flare.alloc_workspace(desc, flare.OP_BACKWARD))
+    assert_grads_close(dict(dQ=to_np64(dQ), dK=to_np64(dK), dV=to_np64(dV)), oracle_backward(oracle, inp), "bf16", f"Y = {value}, M = {M}, D = {D}")
