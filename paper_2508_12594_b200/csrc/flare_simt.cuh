@@ -2,7 +2,7 @@
 //
 // float32 inputs must meet a 1e-5 relative tolerance, which the tensor cores' reduced-mantissa float32 mode cannot.  Here
 // every score q.k is summed in double precision, by the double-precision MMA (m8n8k4), and rounded once; exponentials
-// are expf; the value contractions run on the double-precision MMA too, their sums in double.  What bounds them is that pipe:
+// are one ex2 each, put right to first order (exp_diff); the value contractions run on the double-precision MMA too, their sums in double.  What bounds them is that pipe:
 // 64 multiply-adds per clock per SM, D of them per (row, column) pair and product, 0.25 clocks per pair, product and SM at D = 16.
 //
 // All of them share one shape.  "Rows" (latents in encode, dZ and dQ; tokens in decode and the token pass) stay in
@@ -36,7 +36,8 @@ __device__ __forceinline__ void dmma(double2 &c, double a, double b) {
     asm("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c.x), "+d"(c.y) : "d"(a), "d"(b));
 }
 
-__device__ __forceinline__ float quad_sum(float x) {
+template <class F>
+__device__ __forceinline__ F quad_sum(F x) {
     x += __shfl_xor_sync(0xffffffffu, x, 1);
     return x + __shfl_xor_sync(0xffffffffu, x, 2);
 }
@@ -142,8 +143,8 @@ __device__ __forceinline__ void load_values(double (&v)[2][SimtGeom<D>::NB], con
     }
 }
 // acc += weights of the thread's two columns * values: row lane / 4 of a block, elements 8 j + 2 (lane % 4), + 1
-template <int D, int RB>
-__device__ __forceinline__ void add_values(double2 (&acc)[RB][SimtGeom<D>::NB], const float2 (&w)[RB], const double (&v)[2][SimtGeom<D>::NB]) {
+template <int D, int RB, class W>                               // W: float2 or double2
+__device__ __forceinline__ void add_values(double2 (&acc)[RB][SimtGeom<D>::NB], const W (&w)[RB], const double (&v)[2][SimtGeom<D>::NB]) {
 #pragma unroll
     for (int e = 0; e < 2; ++e)
 #pragma unroll
@@ -177,8 +178,14 @@ __device__ __forceinline__ void write_row(T *dst, const double2 (&acc)[SimtGeom<
 
 // exp of a score, once rounded to float, less a reference or a log-sum-exp (which was formed from scores rounded the same way: the rounding of the
 // largest ones cancels; with the difference taken in double and rounded after it a weight near 1 was off by the log-sum-exp's last place,
-// the largest entries of dV three times as much).  The product's rounding is x / 2^24, and e^x x small.
-__device__ __forceinline__ float exp_diff(float x) { return ptx::ex2(x * 1.4426950408889634f); }
+// the largest entries of dV three times as much).  e^x = 2^y e^(x - y ln 2) with y = x log2(e) as it was rounded: what is left of x, some x / 2^24, to
+// first order.  (Without, the weights of the backward over N flat scores, where x is -log N, were off by 4.7e-7 instead of 2.8e-7 at 131072 tokens, root
+// mean square; what is left is the rounding of x.  expf gives the same and takes 3 % of a float16 training step more.)
+__device__ __forceinline__ float exp_diff(float x) {
+    const float y = x * 1.4426950408889634f, w = ptx::ex2(y);
+    const float rest = fmaf(-y, -1.9046542e-9f, fmaf(-y, 0.69314718f, x));   // (ln 2 in two parts)
+    return fmaf(w, fmaxf(rest, -1.f), w);                       // (x = -inf: rest is NaN, w is 0)
+}
 
 // Running softmax state of the rows of a warp.  The reference m of a row (the same in the four threads of its quad) is not the running maximum
 // but a score within kSlack of it: what weighs most has a small exponent (see exp_diff; with 20, lse_enc was off by up to 1.6 of its last place), and

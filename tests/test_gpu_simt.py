@@ -58,3 +58,15 @@ def test_forward_in_one_launch(B, H, N, M, D, masked, dtype):
         got, want = got.nan_to_num(), want.nan_to_num()
         rms = max(float(want.pow(2).mean().sqrt()), 1e-30)
         assert float(((got - want).abs() - stored * want.abs()).max()) <= 4e-5 * rms
+
+
+def test_weights_over_many_tokens():
+    """One latent over 131072 tokens of nearly equal score: a row of dV is the token's weight times one vector, and the weight e^(score - lse) of a distance
+    of 11.8.  That distance is rounded to multiples of 2^-20 (root mean square 2^-20 / sqrt(12) = 2.75e-7); the exponential, the score and the stored
+    value add 2^-23 each at most.  (A product with log2(e) that is rounded once more: 4.7e-7.)"""
+    inp = workloads.make_random(1, 1, 131072, 1, 8, dtype="f32", seed=9, with_dy=True, k_std=0.1)
+    Q, K, V, dY = (t.cuda() for t in (inp.Q, inp.K, inp.V, inp.dY))
+    dV = flare.forward_backward(Q, K, V, dY)[3].double()[0, :, 0]
+    S = (K.double()[0, :, 0] * Q.double()[0, 0]).sum(1)
+    ratio = (dV / (torch.softmax(S, 0)[:, None] * dY.double()[0, :, 0].sum(0))).mean(1)
+    assert float((ratio / ratio.mean() - 1.0).pow(2).mean().sqrt()) <= 2.0 ** -20 / 12 ** 0.5 + 2.0 ** -23 * 0.5
