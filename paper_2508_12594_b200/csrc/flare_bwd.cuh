@@ -14,14 +14,16 @@
 // the output type, and where the rows Z_m that a token mixes are nearly equal that rounding would dominate dS.
 // Reductions add their partial results in a fixed order, so the gradients are bitwise reproducible.
 //
-// dd enters linearly, so the token side takes one sweep: dK_n = scale (T_n - dd[n] U_n), T without dd, U_n = sum_m W_dec[n,m] q_m, all sums in
-// double.  (Two sweeps, dd first, took 5 D score products and three exponentials per pair instead of 3 D and two.)
+// dd enters linearly, so the token side takes one sweep: dK_n = scale (T_n - dd[n] U_n), T without dd, U_n = sum_m W_dec[n,m] q_m, all products and
+// sums in double, and dd[n] over the sum of the weights as they were rounded: where a token follows one latent, T and dd U agree to many digits, and
+// what is left, (1 - W_dec) A q, takes 1 - W_dec from the other latents' weights instead of from the last digits of this one's.  (Two sweeps, dd first, took 5 D score products and three exponentials per pair instead of 3 D and two.)
 //
 // The kernels have the shape of the forward ones: row operands as A fragments in registers, column operands in
 // shared memory, all products of a pair (q.k, dY.Z, dZ.V, and the contractions of dS and the weights) on the double-precision MMA, which is
 // busy 55 to 65 % of the time: 6 D double multiply-adds per pair on the token side, 4 D in the dQ pass.  Neither a second tile buffer, nor
 // twice the warps, nor the wider MMA shapes (m16n8k16) moved that.  us per training step, before (contractions as float32 FMAs, expf) -> now: float16
-// 4 x 10007 tokens, M = 64, D = 16, 8 heads 492 -> 452; float32 2 x 9973 273 -> 242; 16384, M = 64, D = 32, 4 heads 237 -> 216; 10000, D = 64 390 -> 297.
+// 4 x 10007 tokens, M = 64, D = 16, 8 heads 487 -> 470; float32 2 x 9973 272 -> 249; 16384, M = 64, D = 32, 4 heads 236 -> 217; 10000, D = 64 389 -> 295.
+// (Of these 12, 5, 3 and 1 are exp_diff's second term, and as much the products of dd and T in double.)
 #pragma once
 
 #include "flare_ptx.cuh"
@@ -60,12 +62,13 @@ bwd_token_simt_kernel(const T *Q, const T *K, const T *V,
     double ak[RB][D / 4], ag[RB][D / 4];
     load_rows<T, D, RB>(ak, K + base, stride, r0, N, (double)scale);
     load_rows<T, D, RB>(ag, dY + base, stride, r0, N, 1.0);
-    float ld[RB], dd[RB];
+    float ld[RB];
+    double dd[RB], sum[RB];
 #pragma unroll
     for (int rb = 0; rb < RB; ++rb) {
         const int n = r0 + 8 * rb + (lane >> 2);
         ld[rb] = n < N ? lse_dec[((size_t)b * N + n) * H + h] : INFINITY;
-        dd[rb] = 0.f;
+        dd[rb] = sum[rb] = 0.0;
     }
     float *sC = sDe + CT;
     unsigned char *raw = reinterpret_cast<unsigned char *>(sC + D);
@@ -115,15 +118,17 @@ bwd_token_simt_kernel(const T *Q, const T *K, const T *V,
                 const int at = nb * 8 + 2 * (lane & 3);
                 const float2 le = *reinterpret_cast<const float2 *>(sLe + at), dem = *reinterpret_cast<const float2 *>(sDe + at);
                 const bool in0 = nb * 8 + column_slot(2 * (lane & 3)) < mc, in1 = nb * 8 + column_slot(2 * (lane & 3) + 1) < mc;
-                float2 t[RB], wd[RB], we[RB];
+                double2 t[RB], wd[RB], we[RB];
 #pragma unroll
                 for (int rb = 0; rb < RB; ++rb) {
                     const float s0 = (float)s[rb].x, s1 = (float)s[rb].y;
-                    wd[rb] = make_float2(in0 ? exp_diff(s0 - ld[rb]) : 0.f, in1 ? exp_diff(s1 - ld[rb]) : 0.f);
-                    we[rb] = make_float2(in0 && valid[rb] ? exp_diff(s0 + le.x) : 0.f, in1 && valid[rb] ? exp_diff(s1 + le.y) : 0.f);
-                    const float wa0 = wd[rb].x * (float)a[rb].x, wa1 = wd[rb].y * (float)a[rb].y;
+                    wd[rb] = make_double2(in0 ? exp_diff(s0 - ld[rb]) : 0.f, in1 ? exp_diff(s1 - ld[rb]) : 0.f);
+                    we[rb] = make_double2(in0 && valid[rb] ? exp_diff(s0 + le.x) : 0.f, in1 && valid[rb] ? exp_diff(s1 + le.y) : 0.f);
+                    const double wa0 = wd[rb].x * a[rb].x, wa1 = wd[rb].y * a[rb].y;
                     dd[rb] += wa0 + wa1;
-                    t[rb] = make_float2(wa0 + we[rb].x * ((float)c[rb].x - dem.x), wa1 + we[rb].y * ((float)c[rb].y - dem.y));
+                    sum[rb] += wd[rb].x + wd[rb].y;
+                    // (de is a rounded sum: rounded alike, the two cancel where a latent follows a single token)
+                    t[rb] = make_double2(fma(we[rb].x, (double)((float)c[rb].x - dem.x), wa0), fma(we[rb].y, (double)((float)c[rb].y - dem.y), wa1));
                 }
                 double v[2][SG::NB];
                 load_values<D>(v, sQ, nb);
@@ -137,11 +142,13 @@ bwd_token_simt_kernel(const T *Q, const T *K, const T *V,
     for (int rb = 0; rb < RB; ++rb) {
         const int n = r0 + 8 * rb + (lane >> 2);
         dd[rb] = quad_sum(dd[rb]);
+        sum[rb] = quad_sum(sum[rb]);
+        if (fabs(sum[rb] - 1.0) < 1e-3) dd[rb] /= sum[rb];          // (0 where a caller has switched the stage off)
 #pragma unroll
         for (int j = 0; j < SG::NB; ++j)
-            dk[rb][j] = make_double2(dk[rb][j].x - (double)dd[rb] * un[rb][j].x, dk[rb][j].y - (double)dd[rb] * un[rb][j].y);
+            dk[rb][j] = make_double2(dk[rb][j].x - dd[rb] * un[rb][j].x, dk[rb][j].y - dd[rb] * un[rb][j].y);
         if (n < N) {
-            if ((lane & 3) == 0) dd_out[((size_t)b * H + h) * N + n] = dd[rb];
+            if ((lane & 3) == 0) dd_out[((size_t)b * H + h) * N + n] = (float)dd[rb];
             write_row<T, D>(dK + base + (size_t)n * stride, dk[rb], scale);
             write_row<T, D>(dV + base + (size_t)n * stride, dv[rb], 1.0);
         }

@@ -80,12 +80,12 @@ def test_wide_heads_keep_float32_accuracy_of_dq(oracle, B, H, N, M, masked):
     assert np.linalg.norm(got - want) <= 2.0 ** -18 * np.linalg.norm(want)
 
 
-def dk_error_bound(inp):
-    """What dK of one batch item may be off by before it is rounded to bfloat16, element by element (float64).  u = 2^-17 covers two roundings of a
-    value in bf16 halves.  Per (token, latent): the halves of W_dec (A - e) and of W_enc (C - de), |A - e| <= |A - dd| + |dd - e| with e from Y as it is
-    stored (a 2^-7 of |dY| |Y|); those of W_dec against dd - e; the errors of A (Z in halves, and of weights in halves), as far as they do not move
-    all of a token's alike; those of C (dZ, of weights in halves); the weights' own (a rounded score and the exponential)."""
-    u = 2.0 ** -17
+def dk_error_bound(inp, u):
+    """What dK of one batch item may be off by before it is stored, element by element (float64).  u: what an operand of the products loses, 2^-17 for two
+    roundings of bf16 halves, 2^-24 for a float32.  Per (token, latent): W_dec (A - e) and W_enc (C - de) as they enter the last product, |A - e| <= |A - dd| + |dd - e|
+    with e from Y as it is stored (a 2^-7 of |dY| |Y|; bfloat16), and W_dec against dd - e; the errors of A (Z and the weights it was
+    formed with), as far as they do not move all of a token's alike; those of C (dZ likewise); the weights' own (a rounded score, its distance from a
+    rounded log-sum-exp, the exponential)."""
     Q, K, V, dY = (t.double().numpy() for t in (inp.Q, inp.K, inp.V, inp.dY))
     out = np.zeros(K.shape)
     for h in range(Q.shape[0]):
@@ -100,22 +100,28 @@ def dk_error_bound(inp):
         dd, de = (dec * A).sum(1, keepdims=True), (enc * C).sum(0)
         guess = 2.0 ** -7 * (np.abs(g) * np.abs(dec @ Z)).sum(1, keepdims=True)
         weight = 2.0 ** -21 + 2.0 ** -22 * np.abs(S).max(1, keepdims=True)
-        a = u * np.abs(g) @ (np.abs(centred) + Z_abs).T
+        formed = u if inp.Q.dtype == torch.bfloat16 else u + weight.max()
+        a = formed * np.abs(g) @ (np.abs(centred) + Z_abs).T
         others = (1.0 - dec) * a + (dec * a).sum(1, keepdims=True) - dec * a
-        c = 4 * u * (np.abs(v) @ dZ_abs.T + (dZ_abs * Z_abs).sum(1))
+        c = 4 * formed * (np.abs(v) @ dZ_abs.T + (dZ_abs * Z_abs).sum(1))
         out[0, :, h] = (dec * ((u + weight) * np.abs(A - dd) + 2 * u * guess + others) + enc * ((u + weight) * np.abs(C - de) + c)) @ np.abs(q)
     return out
 
 
-@pytest.mark.parametrize("H,N,M,D,k_std", [(2, 1200, 64, 32, 2.0), (2, 1200, 64, 32, 5.0), (2, 1500, 48, 16, 4.0), (2, 1000, 96, 64, 2.0), (2, 900, 208, 64, 2.0),
-                                           (4, 1100, 64, 8, 6.0), (4, 1000, 32, 4, 8.0), (2, 700, 640, 32, 3.0), (2, 2000, 64, 32, 0.2)])
-def test_rows_of_peaked_softmaxes(oracle, H, N, M, D, k_std):
-    """A token that follows one latent has a small row of dK, left of large numbers: every element of it within what its own terms allow.  (Without
-    e, 20 to 75 times that; with dd formed first, in a sweep of its own, 13 to 70 times; now at most 0.15 of it.)"""
-    inp = workloads.make_random(1, H, N, M, D, dtype="bf16", seed=N + M, with_dy=True, k_std=k_std)
+@pytest.mark.parametrize("dtype,H,N,M,D,k_std", [
+    ("bf16", 2, 1200, 64, 32, 2.0), ("bf16", 2, 1200, 64, 32, 5.0), ("bf16", 2, 1500, 48, 16, 4.0), ("bf16", 2, 1000, 96, 64, 2.0),
+    ("bf16", 2, 900, 208, 64, 2.0), ("bf16", 4, 1100, 64, 8, 6.0), ("bf16", 4, 1000, 32, 4, 8.0), ("bf16", 2, 700, 640, 32, 3.0),
+    ("bf16", 2, 2000, 64, 32, 0.2),
+    ("f32", 2, 1200, 64, 32, 5.0), ("f32", 2, 1000, 64, 64, 5.0), ("f32", 2, 1000, 33, 16, 4.0), ("f16", 2, 1200, 64, 32, 5.0), ("f16", 2, 1000, 40, 8, 6.0)])
+def test_rows_of_peaked_softmaxes(oracle, dtype, H, N, M, D, k_std):
+    """A token that follows one latent has a small row of dK, left of large numbers: every element of it within what its own terms allow.  (bfloat16 without
+    e 20 to 75 times that, with dd formed first, in a sweep of its own, 13 to 70 times; now at most 0.15 of it; float32 and
+    float16 with dd summed in float32 and not over the sum of the weights 900 to 2000 times, now 0.05.)"""
+    inp = workloads.make_random(1, H, N, M, D, dtype=dtype, seed=N + M, with_dy=True, k_std=k_std)
     got, want = gpu_backward(inp)["dK"], oracle_backward(oracle, inp)["dK"]
-    half_ulp = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(want), 1e-300))) - 8)
-    assert (np.abs(got - want) <= half_ulp + dk_error_bound(inp)).all()
+    bits, least = {"bf16": (8, -133), "f16": (11, -25), "f32": (24, -149)}[dtype]
+    half_ulp = np.maximum(2.0 ** (np.floor(np.log2(np.maximum(np.abs(want), 1e-300))) - bits), 2.0 ** least)
+    assert (np.abs(got - want) <= half_ulp + dk_error_bound(inp, 2.0 ** (-17 if dtype == "bf16" else -24))).all()
 
 
 @pytest.mark.parametrize("value", [float("nan"), float("inf"), 0.0, 1e30])
