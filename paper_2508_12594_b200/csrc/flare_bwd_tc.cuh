@@ -554,11 +554,12 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // one exponential and one split of a weight per pair, and [dV | U] one accumulator whose contractions share their A operand.  dd goes to the
 // workspace for the dQ kernel.
 //
-// What the factors may lose: W_dec below 2^-126 is flushed, which is a W_enc below 2^-126 r c <= 2^(range of lse_enc + log2 M - 126) (log2
-// units; lse_dec[n] <= log2 M + the largest lse_enc, since lse_enc[m] >= S[m,n]); with that sum at most kFoldLog2 a weight below
-// 2^-46.  Wider ranges (c is 1 then), and tiles with a token whose lse_dec lies further above K than consistent statistics put it
-// (kFarLog2; an infinite lse_dec is how the two-query variant switches a stage off) take a form of the body with an exponential of its
-// own for W_enc, whose halves are a third pair of operands (kTwo).
+// What the factors may lose: W_dec below 2^-126 is flushed, which is a W_enc below 2^-126 r c = 2^(lse_dec[n] - lse_enc[m] - 126) (log2 units): below 2^-86 in
+// tiles whose tokens have an lse_dec within kOneExpLog2 of the least lse_enc, as in the dQ kernel.  (A bound by the range of lse_enc alone would not
+// do: of a range of latents lse_dec may lie far above all, and weights it flushes may then be all there is of a row of dV.)  Tiles beyond that
+// (an infinite lse_dec is how the two-query variant switches a stage off) take a form of the body with an exponential of its own for W_enc,
+// whose halves are a third pair of operands (kTwo): 2^(S - K) against c dZ, c at most 2^(kFoldLog2 / 2); for wider ranges of lse_enc all tiles
+// do, and c is 1.
 //
 // Sixteen warps share units of 64 latents, 16 columns each, on two alternating buffers of tensor memory (S | A | C), as in the dQ kernel; up
 // to 32 latents two sets of eight warps take a tile each, so that no warp idles.  Rows leave the accumulators after the first unit of the next tile.
@@ -566,7 +567,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // Two sweeps over the latents (dd first; two exponentials and 26 instructions per pair, here one and 20), by groups of four warps with units of their
 // own, took, us per training step -> now: 131072 tokens, M = 512, D = 32 (in two ranges, 448 latents at most) 1905 -> 1513; 1048576, M = 1024, D = 8 20967 -> 20025;
 // 32 x 4096, M = 128, D = 32 300 -> 283; 2 x 20011, M = 128, D = 64 187 -> 178; 16384, M = 32, D = 32 84.2 -> 85.1.
-constexpr float kFoldLog2 = 80.f, kFarLog2 = 46.f;
+constexpr float kFoldLog2 = 80.f;
 constexpr int kTokFirstMathWarp = 4;                            // warps: 0 TMA producer, 1 and 3 MMA issue, 2 token constants, 4 on arithmetic
 
 struct BwdTokTcArgs {
@@ -690,7 +691,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::grid_wait();
     const size_t q0 = (size_t)h * a.mtot + a.m0, r0 = ((size_t)b * a.H + h) * a.mtot + a.m0;
     const float *centre = a.around + ((size_t)b * a.H + h) * a.around_rows * DR;
-    float K, unfolded;                                          // (unfolded != 0: c is 1)
+    float K, least, unfolded;                                   // (unfolded != 0: c is 1)
     {
         // K: the middle of the latents' lse_enc (log2 units), leaving out those that saw no valid token and those whose encode is switched off
         float lo = INFINITY, hi = -INFINITY;
@@ -718,7 +719,8 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             hi = fmaxf(hi, extremes[2 * w + 1]);
         }
         K = lo <= hi ? 0.5f * (lo + hi) : 0.f;
-        unfolded = lo > hi || hi - lo + ptx::lg2((float)M) <= kFoldLog2 ? 0.f : 1.f;
+        least = lo <= hi ? lo : 0.f;
+        unfolded = lo > hi || hi - lo <= kFoldLog2 ? 0.f : 1.f;
     }
     auto factor = [&](int m) {                                  // c of latent m; 0 for those left out
         const float le = a.lse_enc[r0 + m] * kBwdLog2e;
@@ -801,7 +803,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 at[r] = -ld[e];
                 const float ev = at[kTile + r], ne = fabsf(ev) <= 3.0e38f ? -ev : 0.f;
                 at[kTile + r] = SM::kPlanes == 3 ? ne : __uint_as_float((__float_as_uint(ne) & ~1u) | (part[e] ? 1u : 0u));
-                far = far || (part[e] && !(ld[e] - K <= kFarLog2));
+                far = far || (part[e] && !(ld[e] - least <= kOneExpLog2));
             }
             far = __any_sync(0xffffffffu, far);
 #pragma unroll

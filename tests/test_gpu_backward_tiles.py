@@ -135,3 +135,18 @@ def test_any_stored_output(oracle, M, D, value):
     dQ, dK, dV = torch.empty(Q.shape, device="cuda"), torch.empty_like(K), torch.empty_like(V)
     flare.flare_backward(desc, Q, K, V, None, Y.fill_(value), dY, Z, le, ld, dQ, dK, dV, flare.alloc_workspace(desc, flare.OP_BACKWARD))
     assert_grads_close(dict(dQ=to_np64(dQ), dK=to_np64(dK), dV=to_np64(dV)), oracle_backward(oracle, inp), "bf16", f"Y = {value}, M = {M}, D = {D}")
+
+
+def test_small_weights_of_a_range_of_latents(oracle):
+    """Latents worked off in two ranges.  The first token's largest decode score is to the second range, 2^91 above its score to the first latent, whose decode
+    weight is below 2^-126; its encode weight there, 2^-48, is 2^55 times any other: its row of dV is that weight times one row of dZ."""
+    N, M, D = 1024, 208, 64
+    inp = workloads.make_random(1, 1, N, M, D, dtype="bf16", seed=4, with_dy=True)
+    inp.Q.zero_()
+    inp.Q[0, 0, 0], inp.Q[0, 1:112, 1], inp.Q[0, 112:, 2] = 1.0, 1.0, 1.0
+    inp.K.zero_()
+    inp.K[0, 0, 0, :3] = torch.tensor([-26.25, -13.875, 59.0])
+    inp.K[0, 200, 0, 1], inp.K[0, 300, 0, 2] = 57.5, 132.0      # (in other tiles) raise lse_enc of the first range's other latents, and of the second range's
+    got, want = gpu_backward(inp)["dV"][0, 0, 0], oracle_backward(oracle, inp)["dV"][0, 0, 0]
+    assert np.linalg.norm(want) > 2.0 ** -60
+    assert np.linalg.norm(got - want) <= 2.0 ** -7 * np.linalg.norm(want)     # (one rounding of the stored value, and as much again)
