@@ -347,7 +347,7 @@ BINDING(call_forward, 7)
     return THPVariable_Wrap(Y);
 BINDING_END
 
-// Q, K, V, dY, key_mask, scale, stream -> (Y, dQ, dK, dV, workspace)
+// Q, K, V, dY, key_mask, scale, stream -> (Y, dQ, dK, dV, workspace: the forward's, and from byte 256 on the backward's)
 BINDING(call_forward_backward, 7)
     const at::Tensor &Q = tensor(a[0]), &K = tensor(a[1]);
     const flare_desc_t d = make_desc(Q, K, number(a[5]));
@@ -355,17 +355,19 @@ BINDING(call_forward_backward, 7)
     void *q = c.q(a[0]), *k = c.tok(a[1]), *v = c.tok(a[2]), *dy = c.tok(a[3]);
     uint8_t *m = c.mask(a[4]);
     flare_stream_t st = stream_of(a[6]);
-    // one workspace: the backward starts when the forward is done with it
-    const size_t ws = std::max(workspace_bytes(d, FLARE_OP_FORWARD), workspace_bytes(d, FLARE_OP_BACKWARD));
+    // one workspace: the backward starts when the forward is done with it.  But for the header, which keeps what the forward reports: the
+    // backward has its own behind it.
+    const size_t fwd_bytes = workspace_bytes(d, FLARE_OP_FORWARD), bwd_bytes = workspace_bytes(d, FLARE_OP_BACKWARD), bwd_at = 256;
+    const size_t ws = std::max(fwd_bytes, bwd_at + bwd_bytes);
     const at::Tensor Y = at::empty({d.B, d.N, d.H, d.D}, K.options()), dK = at::empty({d.B, d.N, d.H, d.D}, K.options());
     const at::Tensor dV = at::empty({d.B, d.N, d.H, d.D}, K.options()), dQ = at::empty({d.H, d.M, d.D}, K.options().dtype(at::kFloat));
     const size_t z_at = round256(ws), le_at = round256(z_at + 4 * (size_t)d.B * d.H * d.M * d.D), ld_at = round256(le_at + 4 * (size_t)d.B * d.H * d.M);
     const at::Tensor w = scratch(ld_at + 4 * (size_t)d.B * d.N * d.H, K, a[6], st);
     char *base = (char *)w.data_ptr();
     float *z = (float *)(base + z_at), *le = (float *)(base + le_at), *ld = (float *)(base + ld_at);
-    check_status(unlocked([&] { return lib.forward(&d, q, k, v, m, Y.data_ptr(), z, le, ld, base, ws, st); }), "flare_forward");
+    check_status(unlocked([&] { return lib.forward(&d, q, k, v, m, Y.data_ptr(), z, le, ld, base, fwd_bytes, st); }), "flare_forward");
     check_status(unlocked([&] { return lib.backward(&d, q, k, v, m, Y.data_ptr(), dy, z, le, ld, (float *)dQ.data_ptr(), dK.data_ptr(), dV.data_ptr(),
-                                                    base, ws, st); }), "flare_backward");
+                                                    base + bwd_at, bwd_bytes, st); }), "flare_backward");
     return Py_BuildValue("(NNNNN)", THPVariable_Wrap(Y), THPVariable_Wrap(dQ), THPVariable_Wrap(dK), THPVariable_Wrap(dV), THPVariable_Wrap(w));
 BINDING_END
 

@@ -259,4 +259,5 @@ def forward_backward(Q, K, V, dY, key_mask=None, scale=1.0, stream=None, check=F
     if check:
         (stream or torch.cuda.current_stream()).synchronize()
         flare_check(ws, stream)
+        flare_check(ws[256:], stream)
     return Y, dQ, dK, dV

@@ -180,3 +180,33 @@ def test_backward_large_scores(oracle, case):
     got = gpu_backward(inp)
     assert all(np.isfinite(v).all() for v in got.values())
     assert_grads_close(got, oracle_backward(oracle, inp), "bf16", str(case))
+
+
+@pytest.mark.parametrize("which", ["flare_forward", "flare_backward"])
+def test_a_wait_that_gave_up_is_reported_for_either_half(which):
+    """check=True raises for a bounded wait that gave up in the forward as well as in the backward: the call named waits, behind its own kernels, for
+    what never comes (flare_selftest_wait), and records that as a kernel of its own would."""
+    import ctypes
+    lib = flare.load()
+    at = {name: ctypes.cast(getattr(lib, name), ctypes.c_void_p).value for name in flare._SIGNATURES}
+    n = len(flare._SIGNATURES[which][1])                     # arguments: ..., workspace, workspace_bytes, stream
+    kind = ctypes.CFUNCTYPE(ctypes.c_int, *([ctypes.c_void_p] * (n - 2) + [ctypes.c_size_t, ctypes.c_void_p]))
+    real = kind(at[which])
+
+    def gives_up(*args):
+        rc = real(*args)
+        return rc or lib.flare_selftest_wait(args[n - 3], 1_000_000, args[n - 1])
+
+    fake = kind(gives_up)
+    inp = workloads.make_random(1, 2, 300, 32, 16, dtype="bf16", seed=2, with_dy=True)
+    args = [dev(t) for t in (inp.Q, inp.K, inp.V, inp.dY)]
+    flare.forward_backward(*args, check=True)
+    native = flare._native
+    try:
+        native.bind({**at, which: ctypes.cast(fake, ctypes.c_void_p).value}, flare.FlareError)
+        with pytest.raises(flare.FlareError) as e:
+            flare.forward_backward(*args, check=True)
+        assert e.value.status == flare.ERR_TIMEOUT
+    finally:
+        native.bind(at, flare.FlareError)
+    flare.forward_backward(*args, check=True)
