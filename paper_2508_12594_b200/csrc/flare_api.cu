@@ -59,7 +59,7 @@ int static_scratch_address(void **out) {
 }
 
 // Kernels one call of `op` launches (among them the one that clears the workspace header, where it is not left to the merge).
-int launches_for(const flare_desc_t *d, int op, int sms) {
+int launches_for(const flare_desc_t *d, int op) {
     // a fast form is followed by the exact form (which may exit at once)
     const int fe = use_fast_encode(d) ? 2 : 1, f = use_fast_decode(d) ? 2 : 1;
     const int enc = fe + 1 + (use_tc(d) ? 1 : 0);               // header, encode, merge
@@ -67,7 +67,7 @@ int launches_for(const flare_desc_t *d, int op, int sms) {
     switch (op) {
         case FLARE_OP_ENCODE: return enc;
         case FLARE_OP_DECODE: return 1 + dec;                   // header (given a workspace), decode
-        case FLARE_OP_FORWARD: return small_forward_cluster(d, sms) ? 1 : enc + dec;
+        case FLARE_OP_FORWARD: return small_forward_cluster(d) ? 1 : enc + dec;
         case FLARE_OP_BACKWARD: {
             const int tok = token_in_ranges(d) ? (d->M + token_range(d) - 1) / token_range(d) : 1;   // (the CUDA-core kernel knows no ranges)
             return 1 + 2 + tok + 2;                             // header; dZ, its reduction; token kernel(s); dQ, its reduction
@@ -84,8 +84,10 @@ size_t forward_bytes(const flare_desc_t *d) {
 int forward_impl(const flare_desc_t *d, const void *Q, const void *K, const void *V, const uint8_t *mask, void *Y, float *Z, float *lse_enc,
                  float *lse_dec, void *workspace, cudaStream_t st, bool keep_status) {
     const WorkspaceLayout w = make_layout(partials_for(d, device_info().sms, false), (long)d->B * d->H * d->M, d->D, true);
-    if (const int cluster = small_forward_cluster(d, device_info().sms))
-        return forward_small_simt(d, cluster, Q, K, V, mask, Z, lse_enc, Y, lse_dec, keep_status ? nullptr : static_cast<uint32_t *>(workspace), st);
+    if (const int cluster = small_forward_cluster(d)) {
+        const int rc = forward_small_simt(d, cluster, Q, K, V, mask, Z, lse_enc, Y, lse_dec, keep_status ? nullptr : static_cast<uint32_t *>(workspace), st);
+        if (rc != FLARE_ERR_UNSUPPORTED) return rc;
+    }
     if (Z == nullptr) Z = reinterpret_cast<float *>(static_cast<char *>(workspace) + w.z);
     const int rc = encode_impl(d, Q, K, V, mask, Z, lse_enc, workspace, st, false, keep_status);
     if (rc != FLARE_OK) return rc;
@@ -283,7 +285,7 @@ int flare_encode_partials(const flare_desc_t *desc) {
 
 int flare_launch_count(const flare_desc_t *desc, int op) {
     if (check_desc(desc) != FLARE_OK) return 0;
-    return launches_for(desc, op, device_info().sms);
+    return launches_for(desc, op);
 }
 
 size_t flare_workspace_bytes(const flare_desc_t *desc, int op) {

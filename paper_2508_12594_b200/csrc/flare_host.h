@@ -78,18 +78,6 @@ int ensure_big_smem(Kernel kernel, std::atomic<uint64_t> &done, int bytes = 227 
     return FLARE_OK;
 }
 
-// The same for clusters of more than eight blocks.
-template <typename Kernel>
-int ensure_wide_cluster(Kernel kernel, std::atomic<uint64_t> &done) {
-    int dev = 0;
-    FLARE_CUDA(cudaGetDevice(&dev));
-    const uint64_t bit = 1ull << (dev & 63);
-    if (done.load(std::memory_order_acquire) & bit) return FLARE_OK;
-    FLARE_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    done.fetch_or(bit, std::memory_order_release);
-    return FLARE_OK;
-}
-
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 inline int check_desc(const flare_desc_t *d) {
@@ -150,7 +138,7 @@ inline bool use_tc(const flare_desc_t *d) {
 // tokens, or two where a tile is quick.  Measured, one launch : three, us (tokens, M, D, heads): sixteen blocks 1024, 16, 16, 2 5.3 : 7.2;
 // 1024, 64, 32, 8 17.4 : 21; 2048, 16, 16, 8 8.5 : 9.7; 2048, 60, 8, 8 12.1 : 12.6; 2048, 64, 16, 4 14.1 : 11.9; 4096, 16, 16, 2 10.4 : 9.7; eight
 // 512, 64, 32, 16 18 : 21; 1024, 16, 16, 32 8.8 : 12.3; 1024, 32, 16, 16 11 : 12.5; 1024, 32, 32, 16 18.5 : 16.3; 1024, 64, 32, 16 29 : 24.
-inline int small_forward_cluster(const flare_desc_t *d, int sms) {
+inline int small_forward_wanted(const flare_desc_t *d, int sms) {
     if (use_tc(d) || d->M > 64 || d->D > 32) return 0;
     const long heads = (long)d->B * d->H;
     const int cluster = 16 * heads <= sms ? 16 : 8 * heads <= 2L * sms ? 8 : 0;
@@ -453,6 +441,9 @@ int encode_dz_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, cons
                    float *pacc, cudaStream_t st);
 // Clears the workspace header from word `first` on (one kernel for all callers: whichever call comes first loads it).
 int clear_header(void *workspace, int first, cudaStream_t st);
+// Blocks per cluster of a forward in one launch on the current device, or 0.  forward_small_simt: FLARE_ERR_UNSUPPORTED, and nothing launched, where the
+// stream has no room for the cluster.
+int small_forward_cluster(const flare_desc_t *d);
 int forward_small_simt(const flare_desc_t *d, int cluster, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z, float *lse_enc,
                        void *Y, float *lse_dec, uint32_t *header, cudaStream_t st);
 int decode_simt(const flare_desc_t *d, const void *Q, const void *K, const float *Z, void *Y, float *lse_dec, cudaStream_t st);

@@ -47,6 +47,43 @@ struct Decode {
     }
 };
 
+// Whether the device can place a cluster of forward_small_simt_kernel, asked once per device: sixteen blocks are not a portable size, and where a
+// partition of the GPU has no group of SMs with room for them a launch is refused.
+template <typename T, int D, int CS>
+bool small_cluster_fits() {
+    static std::atomic<uint64_t> asked{0}, fits{0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaGetLastError(), false;
+    const uint64_t bit = 1ull << dev;
+    if (!(asked.load(std::memory_order_acquire) & bit)) {
+        auto kernel = forward_small_simt_kernel<T, D, CS>;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = CS; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(CS); cfg.blockDim = dim3(kSimtThreads); cfg.dynamicSmemBytes = forward_small_smem<T, D>();
+        cfg.attrs = &attr; cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) != cudaSuccess ||
+            (CS > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) ||
+            cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            clusters = 0;
+        }
+        if (clusters > 0) fits.fetch_or(bit, std::memory_order_relaxed);
+        asked.fetch_or(bit, std::memory_order_release);
+    }
+    return fits.load(std::memory_order_relaxed) & bit;
+}
+
+template <typename T, int D>
+struct SmallFits {
+    static int run(int cluster) {
+        if constexpr (D > 32) return 0;
+        else return cluster == 16 ? small_cluster_fits<T, D, 16>() : small_cluster_fits<T, D, 8>();
+    }
+};
+
 template <typename T, int D>
 struct SmallForward {
     static int run(const flare_desc_t *d, int cluster, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z, float *lse_enc,
@@ -54,21 +91,20 @@ struct SmallForward {
         if constexpr (D > 32) {
             return FLARE_ERR_UNSUPPORTED;
         } else {
-            const size_t partials_at = encode_simt_smem<T, D>(1), smem = forward_small_smem<T, D>();
+            const size_t partials_at = encode_simt_smem<T, D>(1);
             int WM = 1;
             while (WM * 8 < d->M) WM *= 2;
             auto launch = [&](auto size) -> int {
                 constexpr int CS = decltype(size)::value;
-                auto kernel = forward_small_simt_kernel<T, D, CS>;
-                static std::atomic<uint64_t> opt_in{0};
-                if (smem > 48 * 1024)
-                    if (int rc = ensure_big_smem(kernel, opt_in, (int)smem)) return rc;
-                static std::atomic<uint64_t> wide_opt_in{0};
-                if (CS > 8)
-                    if (int rc = ensure_wide_cluster(kernel, wide_opt_in)) return rc;
                 const int chunk = ((d->N + CS - 1) / CS + 7) / 8 * 8;
-                FLARE_CUDA(launch_after(kernel, dim3(CS, d->H, d->B), kSimtThreads, smem, st, (const T *)Q, (const T *)K, (const T *)V, mask, Z, lse_enc,
-                                        (T *)Y, lse_dec, header, d->H, d->N, d->M, WM, chunk, d->scale, (int)partials_at));
+                const cudaError_t e = launch_after(forward_small_simt_kernel<T, D, CS>, dim3(CS, d->H, d->B), kSimtThreads, forward_small_smem<T, D>(), st,
+                                                   (const T *)Q, (const T *)K, (const T *)V, mask, Z, lse_enc, (T *)Y, lse_dec, header, d->H, d->N, d->M,
+                                                   WM, chunk, d->scale, (int)partials_at);
+                if (e == cudaErrorInvalidClusterSize || e == cudaErrorLaunchOutOfResources) {   // (the stream's part of the GPU is smaller than the device's)
+                    cudaGetLastError();
+                    return FLARE_ERR_UNSUPPORTED;
+                }
+                FLARE_CUDA(e);
                 return FLARE_OK;
             };
             return cluster == 16 ? launch(std::integral_constant<int, 16>{}) : launch(std::integral_constant<int, 8>{});
@@ -134,6 +170,11 @@ int encode_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const v
 int encode_dz_simt(const flare_desc_t *d, const SimtPlan &p, const void *Q, const void *K, const void *dY, const float *lse_dec,
                    float *pacc, cudaStream_t st) {
     return by_type<Encode>(d, true, d, p, Q, K, dY, (const uint8_t *)nullptr, lse_dec, (float *)nullptr, (float *)nullptr, pacc, st);
+}
+int small_forward_cluster(const flare_desc_t *d) {
+    const DeviceView di = device_info();
+    const int cluster = small_forward_wanted(d, di.sms);
+    return cluster != 0 && (di.checked != 1 || by_type<SmallFits>(d, cluster)) ? cluster : 0;   // (no device: what a whole one runs)
 }
 int forward_small_simt(const flare_desc_t *d, int cluster, const void *Q, const void *K, const void *V, const uint8_t *mask, float *Z, float *lse_enc,
                        void *Y, float *lse_dec, uint32_t *header, cudaStream_t st) {

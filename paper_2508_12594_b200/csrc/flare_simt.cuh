@@ -434,7 +434,7 @@ template <typename T, int D> inline size_t decode_simt_smem() {
 // The whole forward of a small problem in one launch: a cluster of CS blocks per (batch item, head), each with its share of the tokens.
 // Encode as above; the blocks join their partial rows through each other's shared memory, every block its share of the latents, whose Z it
 // hands to all; decode of the block's tokens against that Z.  Three launches take 2 to 3 us each whatever there is to do, and the host as long to
-// queue them.  (Which problems: see small_forward_cluster.)
+// queue them.  (Which problems: see small_forward_wanted.)
 constexpr int kSmallMaxM = 64;
 template <int D> struct SmallGeom {
     using SG = SimtGeom<D>;
