@@ -30,6 +30,9 @@ CASES = [  # B, H, N, M, D, masked_fraction, k_std
     (1, 1, 300, 64, 64, 0.0, 4.0),
     (1, 1, 300, 512, 32, 0.1, 0.8),       # the most latents of one launch at D = 32, and ranges beyond
     (1, 1, 300, 528, 32, 0.1, 0.8),
+    (1, 1, 260, 400, 64, 0.1, 0.8),       # three and four ranges: launches that neither begin nor end the sums, dd from either array
+    (1, 1, 260, 592, 64, 0.1, 0.8),
+    (1, 2, 200, 1040, 32, 0.1, 0.8),
     (1, 1, 260, 160, 64, 0.0, 0.8),       # third part of Z: the most latents
     (1, 2, 40000, 32, 32, 0.1, 0.8),      # two sets of warps, several tiles each
     (2, 1, 40000, 16, 8, 0.0, 0.8),

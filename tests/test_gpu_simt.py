@@ -54,10 +54,21 @@ def test_forward_in_one_launch(B, H, N, M, D, masked, dtype):
     flare.flare_decode(desc, Q, K, Z2, Y2, ld2)
     for got, want, stored in ((Z, Z2, 0.0), (Y, Y2, 2.0 ** -10 if dtype == "f16" else 0.0), (le, le2, 0.0), (ld, ld2, 0.0)):
         got, want = got.double(), want.double()
-        assert torch.equal(torch.isinf(got), torch.isinf(want))
-        got, want = got.nan_to_num(), want.nan_to_num()
-        rms = max(float(want.pow(2).mean().sqrt()), 1e-30)
-        assert float(((got - want).abs() - stored * want.abs()).max()) <= 4e-5 * rms
+        finite = want.isfinite()
+        assert bool((finite | want.isneginf()).all()) and torch.equal(got.isfinite(), finite) and torch.equal(got.isneginf(), want.isneginf())
+        if finite.any():
+            got, want = got[finite], want[finite]
+            rms = max(float(want.pow(2).mean().sqrt()), 1e-30)
+            assert float(((got - want).abs() - stored * want.abs()).max()) <= 4e-5 * rms
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("B,H,N,M,D,masked", [(1, 9, 1024, 64, 32, 0.1), (1, 2, 2048, 32, 16, 0.0), (2, 5, 512, 64, 32, 0.2), (2, 5, 1024, 64, 8, 0.1)])
+def test_most_tokens_of_one_launch(oracle, B, H, N, M, D, masked, dtype):
+    """The largest problems of that form, of sixteen and of eight blocks, against the oracle."""
+    inp = workloads.make_random(B, H, N, M, D, dtype=dtype, seed=N + M, masked_fraction=masked, k_std=0.8)
+    assert flare.flare_launch_count(flare.make_desc(inp.Q, inp.K, 0.7), flare.OP_FORWARD) == 1
+    assert_forward_close(gpu_forward(inp, scale=0.7, canary=True), oracle_forward(oracle, inp, 0.7), dtype, f"{dtype} B{B}H{H}N{N}M{M}D{D}")
 
 
 def test_weights_over_many_tokens():
