@@ -13,15 +13,15 @@
 // What shapes them.  A tcgen05.mma with both operands in shared memory takes the tensor core 40 cycles at N = 16 or 32, 48 at 64 and 64
 // at 128 (most of it the fetch of its A operand), one with A in tensor memory N / 2; a hand-over between threads and tensor core
 // costs a warp some 100 instructions and a round trip of about 1000 cycles.  Units of 16 columns (dQ kernel at D = 32: ten MMAs of N = 16 for
-// 16 tokens) ran at exactly the tensor limit.  Wider units are either shared by all warps (dQ kernel) or each group of four warps has one
-// of its own (token kernel); which serves better was measured for both.
+// 16 tokens) ran at exactly the tensor limit.  Wider units are shared by all warps (token kernel, up to 32 latents: by half of them, which served better than
+// groups of four warps with units of their own in both kernels).
 #pragma once
 
 #include "flare_tc.cuh"
 
 namespace flare {
 
-// dS of a pair of columns as packed bf16 halves hi, lo (and W_enc where it is wanted).  xd = s * sl2 + nd is the decode exponent
+// dS of a pair of columns as packed bf16 halves hi, lo, for the dQ kernel.  xd = s * sl2 + nd is the decode exponent
 // (log2 units), u = A + na, v = C + nc.  Both weights come from one exponential: with K the smallest lse_enc of the CTA's latents
 // (log2 units),
 //     W_enc = W_dec 2^(lse_dec[n] - K) 2^(K - lse_enc[m]),    fr, fc the two factors (fc 0 for a token that takes no part),
@@ -32,31 +32,24 @@ namespace flare {
 // issue slots: with two per pair the unit bound both kernels.)
 constexpr float kOneExpLog2 = 40.f;
 // kThird: dS in three parts (24 bits: all of the float32 value).
-struct DsPair { uint32_t hi, lo, lo2, whi, wlo; };
-template <bool kWeights, bool kTwo, bool kThird>
+struct DsPair { uint32_t hi, lo, lo2; };
+template <bool kTwo, bool kThird>
 __device__ __forceinline__ DsPair ds_pair(float2 s, float2 av, float2 cv, float2 sl2p, float2 nd, float2 na, float2 nc, float2 fr_ne, float2 fc) {
     const float2 xd = __ffma2_rn(s, sl2p, nd);
     const float2 pd = make_float2(ptx::ex2(xd.x), ptx::ex2(xd.y));
     const float2 u = __fadd2_rn(av, na), v = __fadd2_rn(cv, nc);
-    float2 pe, ds;
+    float2 ds;
     if (kTwo) {                                                  // fr_ne: -lse_enc[m]; fc: 0, or -inf for a token that takes no part
         const float2 xe = __ffma2_rn(s, sl2p, __fadd2_rn(fr_ne, fc));
-        pe = make_float2(ptx::ex2(xe.x), ptx::ex2(xe.y));
-        ds = __ffma2_rn(pd, u, __fmul2_rn(pe, v));
+        ds = __ffma2_rn(pd, u, __fmul2_rn(make_float2(ptx::ex2(xe.x), ptx::ex2(xe.y)), v));
     } else {
-        const float2 r = __fmul2_rn(fr_ne, fc);
-        if (kWeights) pe = __fmul2_rn(pd, r);
-        ds = __fmul2_rn(pd, __ffma2_rn(r, v, u));
+        ds = __fmul2_rn(pd, __ffma2_rn(__fmul2_rn(fr_ne, fc), v, u));
     }
     DsPair o;
     o.hi = ptx::pack_bf16(ds);
     const float2 rest = ptx::rest_of(ds, o.hi);
     o.lo = ptx::pack_bf16(rest);
     if (kThird) o.lo2 = ptx::pack_bf16(ptx::rest_of(rest, o.lo));
-    if (kWeights) {
-        o.whi = ptx::pack_bf16(pe);
-        o.wlo = ptx::pack_bf16(ptx::rest_of(pe, o.whi));
-    }
     return o;
 }
 constexpr float kBwdLog2e = 1.4426950408889634f;
@@ -113,7 +106,7 @@ __device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float
 // Measured, us, against units of 16 columns with two exponentials per pair (N = 16384, M = 32, D = 32, 8 heads; 32 x 4096, M = 128, 4 heads;
 // 131072, M = 512, 8 heads; 1048576, M = 1024, D = 8, 8 heads): 22.4, 82, 437, 7844 -> 15.9, 65, 392, 5706; D = 64 (2 x 20011, M = 128, 4
 // heads), on the CUDA cores before: 498 -> 27 (in three
-// parts, see kThird, 31).  Groups of four warps with units and buffers of their own, as in the token kernel:
+// parts, see kThird, 31).  Groups of four warps with units and buffers of their own:
 // 21.6, 78, 522, 7485; 44.  Issue slots and the latency of tensor-memory loads share the bound (some 14 instructions per pair, two issued
 // per cycle and SM).
 constexpr int kDqUnit = 64, kDqBuf = 3 * kDqUnit, kDqAcc = 2 * kDqBuf;
@@ -462,7 +455,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
                                 const int j = 2 * (k + e);
-                                const DsPair r = ds_pair<false, kTwo, kThird>(
+                                const DsPair r = ds_pair<kTwo, kThird>(
                                     make_float2(__uint_as_float(s[q][j]), __uint_as_float(s[q][j + 1])),
                                     make_float2(__uint_as_float(av[q][j]), __uint_as_float(av[q][j + 1])),
                                     make_float2(__uint_as_float(cv[q][j]), __uint_as_float(cv[q][j + 1])), sl2p,

@@ -122,19 +122,6 @@ __device__ __forceinline__ void stage_bf16(uint8_t *dst, const __nv_bfloat16 *sr
     }
 }
 
-// Hand-over of a group's unit n: every warp arrives on the group's barrier `full` (count 4); one of them, taking turns, waits for the others
-// and returns true: it then may issue instructions that depend on what all four wrote to (or have read from) tensor memory.
-// (A counter whose last incrementer issues would need no wait, but the acquiring read-modify-write costs every warp 250 to 400 cycles.)
-__device__ __forceinline__ bool hand_over(uint32_t full, uint32_t n, volatile uint32_t *abort_flag, uint32_t code) {
-    ptx::tc_fence_before();
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) ptx::mbar_arrive(full);
-    if (((threadIdx.x >> 5) & 3) != (n & 3)) return false;
-    const bool ok = warp_wait(full, n & 1, abort_flag, code);
-    ptx::tc_fence_after();
-    return ok;
-}
-
 // ------------------------------------------------------------------------------------- softmax arithmetic
 // Row maximum over NV (16 or 32) float32 scores held as raw bits.
 template <int NV>
