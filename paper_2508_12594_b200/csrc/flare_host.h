@@ -214,7 +214,8 @@ inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes, i
 // idle that several rounds are 2 % quicker; a CTA's start, where the head's latent operands are split and stored, counts as six units of 64
 // latents against a tile, and a fifth of a tile.  us per training step, once : several rounds: 32 heads (128 of 148 CTAs : 288), 50489 tokens, M = 624, D = 16
 // 2793 : 2689, 68334 tokens, M = 80, D = 8 734 : 710, 25344 tokens, M = 336, D = 32 890 : 875; 8 heads (144 : 296) of 1048576 tokens, M = 1024, D = 8
-// 18813 : 18640.
+// 18813 : 18640; D = 64, where a unit has 32 latents and up to 160 of them three parts to split, 32 heads (128 : 288), 40000 tokens, M = 64 855 : 824; 40
+// (120 : 280), 30000, M = 160 1611 : 1530; 64 (128 : 256), 9000, M = 96 500 : 496; the same number either way 128 heads, M = 192, and 32, 20011, M = 128.
 // (A CTA per SM with a share of all heads' tiles in a row, needs a loop over heads around the kernel's body, which made every training step 5 % slower.)
 inline int token_splits(const flare_desc_t *d, int tiles, int mc, int sms) {
     const double units = (double)((mc + 63) / 64);
@@ -402,7 +403,9 @@ struct BwdLayout {
 };
 
 // Latents one launch of the tensor-core token kernel takes: five operands of D-wide bf16 rows (six at D = 64 up to 160 latents) beside two
-// tile stages; more are worked off in ranges of equal size.
+// tile stages; more are worked off in ranges of equal size, with three float32 planes and dd to read and write between them.  us per backward, two sweeps with
+// two planes and at most 448 latents a range at D = 32 : now, 8 heads of 131072 tokens: D = 32, M = 528 1778 : 1533, 640 1922 : 1587, 1024 3126 : 2284; D = 8,
+// M = 2048 4668 : 3818; 65536, D = 64, M = 208 852 : 874, 256 939 : 904, 400 1654 : 1671; 4 heads of 131072, M = 384 1128 : 1026.
 inline int token_range_most(const flare_desc_t *d) { return d->D == 64 ? 192 : d->D == 32 ? 512 : 1024; }
 inline bool token_in_ranges(const flare_desc_t *d) { return use_tc(d) && d->M > token_range_most(d); }
 inline int token_ranges(const flare_desc_t *d) { return (d->M + token_range_most(d) - 1) / token_range_most(d); }
