@@ -1,5 +1,6 @@
 // Backward: plans, workspace layout, launches of the tensor-core and CUDA-core kernels.
 #include "flare_host.h"
+#include "flare_bwd_sweep.cuh"
 #include "flare_bwd_tc.cuh"
 #include "flare_reduce.cuh"
 
@@ -98,12 +99,83 @@ int launch_bwd_token_tc(const flare_desc_t *d, int sms, const void *Q, const voi
     return token_in_ranges(d) ? launch_bwd_token_tc_n<D, DRT, true>(d, sms, K, V, dY, a, st) : launch_bwd_token_tc_n<D, DRT, false>(d, sms, K, V, dY, a, st);
 }
 
+template <int D, int DRT, bool kRanges>
+int launch_dz_sweep(const flare_desc_t *d, const SweepPlan &p, const void *K, const void *dY, const BwdDzArgs &a, cudaStream_t st) {
+    CUtensorMap tmK, tmG;
+    int rc;
+    if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
+    static std::atomic<uint64_t> smem_opt_in{0};
+    if ((rc = ensure_big_smem(bwd_dz_sweep_kernel<D, DRT, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
+    FLARE_CUDA(launch_after(bwd_dz_sweep_kernel<D, DRT, kRanges>, dim3((unsigned)p.splits, d->H, d->B), kSwThreads, BwdDzSmem<D>::total(p.stages, p.range), st,
+                            tmK, tmG, a));
+    return FLARE_OK;
+}
+
+template <int D, int DRT, bool kRanges>
+int launch_grad_sweep(const flare_desc_t *d, const SweepPlan &p, const void *K, const void *V, const void *dY, const BwdGradArgs &a, cudaStream_t st) {
+    CUtensorMap tmK, tmV, tmG, tmDK, tmDV;
+    int rc;
+    if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmV, V, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
+    constexpr int out = DRT == 4 ? D : DRT ? DRT : D;           // (rows of 8 bytes do not leave by such copies)
+    if ((rc = make_token_map(&tmDK, a.dK, d, kTile, out)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmDV, a.dV, d, kTile, out)) != FLARE_OK) return rc;
+    static std::atomic<uint64_t> smem_opt_in{0};
+    if ((rc = ensure_big_smem(bwd_grad_sweep_kernel<D, DRT, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
+    FLARE_CUDA(launch_after(bwd_grad_sweep_kernel<D, DRT, kRanges>, dim3((unsigned)p.splits, d->H, d->B), kSwThreads, BwdGradSmem<D>::total(p.bufs, p.stages, p.range), st,
+                            tmK, tmV, tmG, tmDK, tmDV, a));
+    return FLARE_OK;
+}
+
+// bfloat16 backward of heads up to 32 wide.  skip_pass_a: as below
+template <int D, int DRT>
+int backward_sweeps(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const uint8_t *mask, const void *dY, const float *Z,
+                    const float *lse_enc, const float *lse_dec, float *dQ, void *dK, void *dV, char *ws, cudaStream_t st, bool skip_pass_a) {
+    const BwdLayout w = bwd_layout(d, sms);
+    auto at = [&](size_t off) { return reinterpret_cast<float *>(ws + off); };
+    const long rows = (long)d->B * d->H * d->M;
+    const int tiles = (d->N + kTile - 1) / kTile;
+    uint32_t *status = reinterpret_cast<uint32_t *>(ws);
+    if (const int rc = clear_header(ws, 0, st)) return rc;
+    if (!skip_pass_a) {
+        const SweepPlan p = dz_sweep_plan(d, sms);
+        if (p.stages < p.bufs) return FLARE_ERR_UNSUPPORTED;
+        for (int m0 = 0; m0 < d->M; m0 += p.range) {
+            const BwdDzArgs a{static_cast<const __nv_bfloat16 *>(Q), Z, lse_dec, at(w.part), at(w.dd), status, d->B, d->H, d->N, std::min(p.range, d->M - m0), d->M, m0, m0 == 0,
+                              m0 + p.range >= d->M, reinterpret_cast<float4 *>(ws + w.dd_other), d->scale * kLog2e, tiles, p.stages};
+            const int rc = p.ranges > 1 ? launch_dz_sweep<D, DRT, true>(d, p, K, dY, a, st) : launch_dz_sweep<D, DRT, false>(d, p, K, dY, a, st);
+            if (rc != FLARE_OK) return rc;
+        }
+        const int slices = reduce_slices(2 * p.splits, d->D);
+        const unsigned row_blocks = reduce_blocks(rows, d->D, slices);
+        FLARE_CUDA(launch_after(bwd_dz_reduce_kernel<(DRT ? DRT : D) / 4>, row_blocks, kReduceThreads, 0, st, at(w.part), Z, at(w.dz), at(w.de), 2 * p.splits, rows, slices,
+                                (int)row_blocks, GuessArgs{}));
+    }
+    const SweepPlan p = grad_sweep_plan(d, sms);
+    if (p.stages < p.bufs || BwdGradSmem<D>::log2_accs(p.range) < 0) return FLARE_ERR_UNSUPPORTED;
+    for (int m0 = 0; m0 < d->M; m0 += p.range) {
+        const BwdGradArgs a{static_cast<const __nv_bfloat16 *>(Q), Z, at(w.dz), lse_enc, at(w.de), lse_dec, at(w.dd), mask, static_cast<__nv_bfloat16 *>(dK),
+                            static_cast<__nv_bfloat16 *>(dV), at(w.part), status, d->B, d->H, d->N, std::min(p.range, d->M - m0), d->M, m0, m0 == 0, m0 + p.range >= d->M,
+                            at(w.kvacc), d->scale, d->scale * kLog2e, tiles, p.stages, p.bufs};
+        const int rc = p.ranges > 1 ? launch_grad_sweep<D, DRT, true>(d, p, K, V, dY, a, st) : launch_grad_sweep<D, DRT, false>(d, p, K, V, dY, a, st);
+        if (rc != FLARE_OK) return rc;
+    }
+    FLARE_REDUCE(bwd_dq_reduce_kernel, (long)d->H * d->M, d->B * 2 * p.splits, d->D, st, at(w.part), dQ, 2 * p.splits, d->B, (long)d->H * d->M, d->scale);
+    return FLARE_OK;
+}
+
 template <typename T, int D>
 int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V,
                          const uint8_t *mask, const void *Y, const void *dY, const float *Z, const float *lse_enc,
                          const float *lse_dec, float *dQ, void *dK, void *dV, char *ws, cudaStream_t st,
                          bool skip_pass_a = false) {
     // skip_pass_a: dZ and de are already in the workspace (the second of the two runs of the separate-queries variant)
+    if constexpr (std::is_same<T, __nv_bfloat16>::value && D <= 32) {
+        if (use_sweeps(d))
+            return backward_sweeps<D < 16 ? 16 : D, D < 16 ? D : 0>(d, sms, Q, K, V, mask, dY, Z, lse_enc, lse_dec, dQ, dK, dV, ws, st, skip_pass_a);
+    }
     const BwdLayout w = bwd_layout(d, sms);
     float *part = reinterpret_cast<float *>(ws + w.part);
     float *dZ = reinterpret_cast<float *>(ws + w.dz);

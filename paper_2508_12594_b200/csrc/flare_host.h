@@ -11,6 +11,7 @@
 #include <cstdlib>
 #include <cstring>
 
+#include "flare_bwd_sweep.cuh"
 #include "flare_bwd_tc.cuh"
 #include "flare_common.cuh"
 #include "flare_ptx.cuh"
@@ -294,11 +295,12 @@ inline EncodeTiledFn encode_tiled_fn() {
 }
 
 inline CUtensorMapSwizzle swizzle_for(int D) {
-    return D == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : D == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
+    return D == 8 ? CU_TENSOR_MAP_SWIZZLE_NONE : D == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : D == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
 }
 
 // [B, N, H*D] bf16 viewed as a 3-D tensor (innermost H*D); box = `cols` columns (one head's D, or two adjacent
 // heads' 2D) x `rows` tokens.
+// (8 columns: rows of 16 bytes as they are, not swizzled)
 inline int make_token_map(CUtensorMap *m, const void *base, const flare_desc_t *d, int rows, int cols = 0) {
     if (cols == 0) cols = d->D;
     EncodeTiledFn fn = encode_tiled_fn();
@@ -411,24 +413,58 @@ inline bool token_in_ranges(const flare_desc_t *d) { return use_tc(d) && d->M > 
 inline int token_ranges(const flare_desc_t *d) { return (d->M + token_range_most(d) - 1) / token_range_most(d); }
 inline int token_range(const flare_desc_t *d) { return ((d->M + token_ranges(d) - 1) / token_ranges(d) + 15) / 16 * 16; }
 
+// Two sweeps over the tokens (flare_bwd_sweep.cuh, where both sides are measured): heads up to 16 wide, and 32 wide as long as one launch takes all latents.
+inline bool use_sweeps(const flare_desc_t *d) { return use_tc(d) && (d->D <= 16 || (d->D == 32 && d->M <= 320)); }
+// Latents one launch of a sweep takes: what its operands leave of shared memory (beside two tile stages) and the sums over tokens of tensor memory; more are
+// worked off in ranges of about equal size, whole units of 64.
+struct SweepPlan { int range, ranges, splits, stages, bufs; };
+inline SweepPlan sweep_ranges(const flare_desc_t *d, int sms) {
+    const int most = d->D == 32 ? 320 : 768;
+    SweepPlan p{};
+    p.ranges = (d->M + most - 1) / most;
+    p.range = p.ranges == 1 ? d->M : ((d->M + p.ranges - 1) / p.ranges + 63) / 64 * 64;
+    p.ranges = (d->M + p.range - 1) / p.range;
+    p.splits = token_splits(d, (d->N + kTile - 1) / kTile, p.range, sms);
+    return p;
+}
+inline SweepPlan dz_sweep_plan(const flare_desc_t *d, int sms) {
+    SweepPlan p = sweep_ranges(d, sms);
+    p.bufs = 3;
+    p.stages = d->D == 32 ? BwdDzSmem<32>::stages(p.range) : BwdDzSmem<16>::stages(p.range);
+    return p;
+}
+inline SweepPlan grad_sweep_plan(const flare_desc_t *d, int sms) {
+    SweepPlan p = sweep_ranges(d, sms);
+    auto stages = [&](int bufs) { return d->D == 32 ? BwdGradSmem<32>::stages(bufs, p.range) : BwdGradSmem<16>::stages(bufs, p.range); };
+    // Three buffers of weights want three tile stages: the issuing warp then waits for a tile before it has issued the sums that release the last but one.
+    p.bufs = stages(3) >= 3 ? 3 : 2;
+    p.stages = stages(p.bufs);
+    return p;
+}
+
 inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     BwdLayout w;
     const long rows = (long)d->B * d->H * d->M;
     const int pa = simt_plan(d, sms).P, pb = bwd_dq_plan(d, sms).P;
     w.P = pa > pb ? pa : pb;
-    if (use_tc(d)) w.P = std::max(w.P, std::max(dz_plan(d, sms).splits, tc_dq_plan(d, sms).P));
+    if (use_sweeps(d)) w.P = 2 * std::max(dz_sweep_plan(d, sms).splits, grad_sweep_plan(d, sms).splits);
+    else if (use_tc(d)) w.P = std::max(w.P, std::max(dz_plan(d, sms).splits, tc_dq_plan(d, sms).P));
     size_t off = kHeaderBytes;
     w.part = off; off += align_up(sizeof(float) * (size_t)w.P * rows * d->D);
     w.dz = off;   off += align_up(sizeof(float) * (size_t)rows * d->D);
     w.de = off;   off += align_up(sizeof(float) * (size_t)rows);
-    w.dd = off;   off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
-    w.e = w.around = off;                                      // tensor-core kernels: see bwd_guess, z_around
-    if (use_tc(d)) {
+    w.dd = off;   off += align_up(sizeof(float) * (use_sweeps(d) ? 2 : 1) * (size_t)d->B * d->N * d->H);
+    w.e = w.around = off;                                      // heads 64 wide: see bwd_guess, z_around
+    if (use_tc(d) && !use_sweeps(d)) {
         w.around = off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
         off += align_up(sizeof(float) * (size_t)(1 + latent_blocks(d)) * d->B * d->H * d->D);
     }
     w.dd_other = w.kvacc = off;                                // over latent ranges: dd so far, and float32 sums of the rows
-    if (token_in_ranges(d)) {
+    if (use_sweeps(d)) {
+        const size_t tokens = (size_t)d->B * d->N * d->H;
+        if (dz_sweep_plan(d, sms).ranges > 1) w.kvacc = off += align_up(sizeof(float4) * tokens);
+        if (grad_sweep_plan(d, sms).ranges > 1) off += align_up(sizeof(float) * 2 * (size_t)d->B * d->H * ((d->N + kTile - 1) / kTile) * kTile * d->D);
+    } else if (token_in_ranges(d)) {
         w.kvacc = off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
         off += align_up(sizeof(float) * 3 * (size_t)d->B * d->N * d->H * d->D);
     }

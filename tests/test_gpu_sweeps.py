@@ -1,0 +1,33 @@
+"""The two sweeps over the tokens of the bfloat16 backward (heads up to 32 wide) where they can go wrong, against the CPU oracle (needs a B200): latents
+around the units of 64 and the most of one launch, ranges of unequal size, more tiles to a CTA than tensor memory adds up in a row (with one and with two
+sets of warps), rows that leave by a tile's copy at the end of a batch item, narrow heads."""
+import pytest
+
+from paper_2508_12594_b200 import workloads
+from tests.test_gpu_backward import assert_grads_close, gpu_backward, oracle_backward
+
+pytestmark = pytest.mark.gpu
+
+CASES = [  # B, H, N, M, D, masked_fraction
+    (1, 2, 60, 16, 32, 0.0),              # less than a tile
+    (3, 2, 255, 32, 32, 0.2),             # rows past the end of an item are another item's
+    (3, 3, 130, 48, 16, 0.1),
+    (2, 2, 640, 112, 32, 0.0),
+    (1, 2, 385, 176, 32, 0.1),
+    (2, 4, 383, 80, 8, 0.1),
+    (2, 4, 385, 64, 4, 0.1),
+    (1, 1, 700, 320, 32, 0.1),            # the most latents at D = 32, and one more (other kernels)
+    (1, 1, 700, 336, 32, 0.1),
+    (1, 1, 300, 768, 16, 0.0),            # the most of one launch at D = 16; two ranges, the second shorter; three
+    (1, 2, 300, 784, 16, 0.1),
+    (1, 2, 260, 1552, 8, 0.0),
+    (37, 4, 8400, 16, 8, 0.0),            # 66 tiles to a CTA, two sets of warps
+    (37, 4, 16500, 16, 32, 0.0),          # 129 tiles, the last by itself
+    (37, 4, 8400, 48, 16, 0.1),           # one set
+]
+
+
+@pytest.mark.parametrize("B,H,N,M,D,masked", CASES)
+def test_backward_in_two_sweeps(oracle, B, H, N, M, D, masked):
+    inp = workloads.make_random(B, H, N, M, D, dtype="bf16", seed=N + M, masked_fraction=masked, with_dy=True, k_std=0.8)
+    assert_grads_close(gpu_backward(inp), oracle_backward(oracle, inp), "bf16", f"{B}x{H}x{N}x{M}x{D}")
