@@ -984,7 +984,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
                     const bool more = tu + 1 < mytiles;
 #pragma unroll
                     for (int c = 0; c < U; ++c) {
-                        if (!ptx::mbar_spin(pfull + 8 * (c & 1), par ^ (uint32_t)((c >> 1) & 1), abort_flag, kErrDecode | 5)) { ok = false; break; }
+                        if (!ptx::mbar_wait(pfull + 8 * (c & 1), par ^ (uint32_t)((c >> 1) & 1), abort_flag, kErrDecode | 5)) { ok = false; break; }
                         if (c == 0 && tu > 0 && !ptx::mbar_spin(bar(Y_FREE + g), (uint32_t)((tu - 1) & 1), abort_flag, kErrDecode | 11)) { ok = false; break; }
                         ptx::tc_fence_after();
                         const uint32_t pcol = gcol + (c & 1) * UNIT;
@@ -1077,6 +1077,7 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         constexpr int kSum = kLse ? 2 : 0;
         // normalise and store the rows of tile tu (this group's tu-th), whose value MMAs are all issued
         auto epilogue = [&](int tu) -> bool {
+            asm volatile("" : "+r"(tu));                        // (nothing of what follows is worked out before the branch that leads here, at every unit)
             if (!warp_wait(bar(Y_FULL + g), tu & 1, abort_flag, kErrDecode | 7)) return false;
             ptx::tc_fence_after();
             uint32_t y[48];
@@ -1122,40 +1123,85 @@ decode_stream_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             return true;
         };
         bool ok = true;
-        int n = 0;                                              // unit counter of this group's stream
-        const int total = mytiles * units;
         // A wait on a barrier costs a warp about 150 cycles even when the phase is long complete, and the warp has
         // nothing else to do meanwhile.  So the wait for the next unit's scores is asked early, without blocking,
         // before the exponentials of this unit, and falls back to a blocking wait only if the answer was no.
         bool s_ready = false;
-        for (int tu = 0; ok && tu < mytiles; ++tu) {
-            for (int c = 0; ok && c < units; ++c, ++n) {
-                const int w = n & 1;
-                const bool half = kM == 0 && c == units - 1 && (M & 16) != 0;   // the second 16 columns are beyond M: weights 0
-                if (!s_ready && !(ok = warp_wait(bar(S_FULL + 2 * g + w), (n >> 1) & 1, abort_flag, kErrDecode | 6))) break;
+        uint32_t sfull = bar(S_FULL + 2 * g);                   // (opaque: an address that can be formed again from the kernel's arguments is, at every use)
+        ptx::opaque(sfull);
+        constexpr uint32_t DONE = 8 * (P_FULL - S_FULL);
+        const uint32_t lead = lane == 0;
+        if constexpr (kM != 0) {
+            // Two units a turn, so that buffers and barriers are constants, and the rows of the tile before between them (nothing of which is worked out ahead:
+            // see epilogue).  us per forward, one unit a turn, addresses formed from the kernel's arguments : this: 1048576 tokens, M = 256, D =
+            // 16 1005 : 979, on features of N(0, 1 / D) 954 : 914, 4 x 65536, M = 64 104 : 100, 131072, M = 512, D = 32 288 : 273, 262144, M = 128 171 : 172.
+            // unit on buffer `which`; next: whether another follows, whose scores have parity_next
+            auto unit = [&](auto which, uint32_t parity, bool next, uint32_t parity_next) -> bool {
+                constexpr int w = decltype(which)::value;
+                if (!s_ready && !warp_wait(sfull + 8 * w, parity, abort_flag, kErrDecode | 6)) return false;
                 ptx::tc_fence_after();
                 uint32_t r[32], pk[16];
                 ptx::tmem_ld32(gcol + w * UNIT, r);
                 ptx::tmem_wait_ld();
                 exp_chunk_fast<16, true, kSum>(r, pk, sl2p, sum2);
-                const bool s_probe = n + 1 < total && ptx::mbar_test(bar(S_FULL + 2 * g + (w ^ 1)), ((n + 1) >> 1) & 1);
-                if (!half) {
-                    exp_chunk_fast<16, true, kSum>(r + 16, pk + 8, sl2p, sum2);
-                } else {
-#pragma unroll
-                    for (int k = 8; k < 16; ++k) pk[k] = 0u;
-                }
+                const bool s_probe = next && ptx::mbar_test(sfull + 8 * (w ^ 1), parity_next);
+                exp_chunk_fast<16, true, kSum>(r + 16, pk + 8, sl2p, sum2);
                 ptx::tmem_st16(gcol + w * UNIT, pk);
                 ptx::tmem_wait_st();
                 ptx::tc_fence_before();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(P_FULL + 2 * g + w));
+                ptx::mbar_arrive_if(sfull + DONE + 8 * w, lead);
                 s_ready = __all_sync(0xffffffffu, s_probe);
-                // the previous tile's rows, while the tensor core works on this unit
-                if (c == 0 && tu > 0) ok = epilogue(tu - 1);
-                if (kLse && c == units - 1) {                   // the tile's sum is complete; the next tile starts its own
+                return true;
+            };
+            uint32_t par = 0;
+            for (int tu = 0; ok && tu < mytiles; ++tu) {
+                bool pending = tu > 0;                          // the rows of the tile before are still to be written
+                for (int left = kM / UNIT / 2; left > 0; --left, par ^= 1u) {
+                    if (!(ok = unit(std::integral_constant<int, 0>{}, par, true, par))) break;
+                    if (pending) {                              // while the tensor core works on this unit
+                        pending = false;
+                        if (!(ok = epilogue(tu - 1))) break;
+                    }
+                    if (!(ok = unit(std::integral_constant<int, 1>{}, par, left > 1 || tu + 1 < mytiles, par ^ 1u))) break;
+                }
+                if (kLse) {                                     // the tile's sum is complete; the next tile starts its own
                     l_exact = sum2.x + sum2.y;
                     sum2 = make_float2(0.f, 0.f);
+                }
+            }
+        } else {
+            int n = 0;                                          // unit counter of this group's stream
+            const int total = mytiles * units;
+            for (int tu = 0; ok && tu < mytiles; ++tu) {
+                for (int c = 0; ok && c < units; ++c, ++n) {
+                    const uint32_t w = n & 1, at = sfull + 8 * w;
+                    const bool half = c == units - 1 && (M & 16) != 0;   // the second 16 columns are beyond M: weights 0
+                    if (!s_ready && !(ok = warp_wait(at, (n >> 1) & 1, abort_flag, kErrDecode | 6))) break;
+                    ptx::tc_fence_after();
+                    uint32_t r[32], pk[16];
+                    ptx::tmem_ld32(gcol + w * UNIT, r);
+                    ptx::tmem_wait_ld();
+                    exp_chunk_fast<16, true, kSum>(r, pk, sl2p, sum2);
+                    const bool s_probe = n + 1 < total && ptx::mbar_test(sfull + 8 * (w ^ 1), ((n + 1) >> 1) & 1);
+                    if (!half) {
+                        exp_chunk_fast<16, true, kSum>(r + 16, pk + 8, sl2p, sum2);
+                    } else {
+#pragma unroll
+                        for (int k = 8; k < 16; ++k) pk[k] = 0u;
+                    }
+                    ptx::tmem_st16(gcol + w * UNIT, pk);
+                    ptx::tmem_wait_st();
+                    ptx::tc_fence_before();
+                    __syncwarp();
+                    ptx::mbar_arrive_if(at + DONE, lead);
+                    s_ready = __all_sync(0xffffffffu, s_probe);
+                    // the previous tile's rows, while the tensor core works on this unit
+                    if (c == 0 && tu > 0) ok = epilogue(tu - 1);
+                    if (kLse && c == units - 1) {               // the tile's sum is complete; the next tile starts its own
+                        l_exact = sum2.x + sum2.y;
+                        sum2 = make_float2(0.f, 0.f);
+                    }
                 }
             }
         }
