@@ -10,27 +10,21 @@ namespace {
 // padded tokens: a key mask, or a last partial tile
 bool has_padding(const flare_desc_t *d, const uint8_t *mask) { return mask != nullptr || d->N % kTile != 0; }
 
-template <int D, bool kPair, int DRT, bool kPadded>
+template <int D, bool kPadded>
 int launch_bwd_dq_tc_n(const flare_desc_t *d, const TcEncodePlan &p, const void *K, const void *V, const void *dY, const BwdDqTcArgs &args,
                        cudaStream_t st) {
-    constexpr int DG = kPair ? 2 * D : D;
     CUtensorMap tmK, tmV, tmG;
     int rc;
-    if ((rc = make_token_map(&tmK, K, d, kTile, DG)) != FLARE_OK) return rc;
-    if ((rc = make_token_map(&tmV, V, d, kTile, DG)) != FLARE_OK) return rc;
-    if ((rc = make_token_map(&tmG, dY, d, kTile, DG)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmK, K, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmV, V, d, kTile, D)) != FLARE_OK) return rc;
+    if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
     static std::atomic<uint64_t> smem_opt_in{0};
-    if ((rc = ensure_big_smem(bwd_dq_tc_kernel<D, kPair, DRT, kPadded>, smem_opt_in)) != FLARE_OK) return rc;
-    FLARE_CUDA(launch_after(bwd_dq_tc_kernel<D, kPair, DRT, kPadded>, dim3((kPair ? d->H / 2 : d->H) * p.pairs, p.splits, d->B), kDqThreads, BwdDqSmem<DG, kPair>::total, st, tmK, tmV, tmG, args));
+    if ((rc = ensure_big_smem(bwd_dq_tc_kernel<D, kPadded>, smem_opt_in)) != FLARE_OK) return rc;
+    FLARE_CUDA(launch_after(bwd_dq_tc_kernel<D, kPadded>, dim3(d->H * p.pairs, p.splits, d->B), kDqThreads, BwdDqSmem<D>::total, st, tmK, tmV, tmG, args));
     return FLARE_OK;
 }
 
-template <int D, bool kPair, int DRT>
-int launch_bwd_dq_tc_p(const flare_desc_t *d, const TcEncodePlan &p, bool padded, const void *K, const void *V, const void *dY,
-                       const BwdDqTcArgs &args, cudaStream_t st) {
-    return padded ? launch_bwd_dq_tc_n<D, kPair, DRT, true>(d, p, K, V, dY, args, st) : launch_bwd_dq_tc_n<D, kPair, DRT, false>(d, p, K, V, dY, args, st);
-}
-
+template <int D>
 int launch_bwd_dq_tc(const flare_desc_t *d, const TcEncodePlan &p, const void *Q, const void *K, const void *V, const void *dY,
                      const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
                      const float *lse_dec, const float *dd, const float *around, float *part, uint32_t *status, cudaStream_t st) {
@@ -42,19 +36,10 @@ int launch_bwd_dq_tc(const flare_desc_t *d, const TcEncodePlan &p, const void *Q
     a.B = d->B; a.H = d->H; a.N = d->N; a.M = d->M;
     a.sl2 = d->scale * kLog2e;
     a.tiles = p.tiles; a.splits = p.splits; a.blocks = p.pairs;
-    const bool pad = has_padding(d, mask);
-    if (encode_head_pairs(d))
-        return d->D == 16 ? launch_bwd_dq_tc_p<16, true, 0>(d, p, pad, K, V, dY, a, st) : launch_bwd_dq_tc_p<32, true, 0>(d, p, pad, K, V, dY, a, st);
-    switch (d->D) {
-        case 4: return launch_bwd_dq_tc_p<16, false, 4>(d, p, pad, K, V, dY, a, st);
-        case 8: return launch_bwd_dq_tc_p<16, false, 8>(d, p, pad, K, V, dY, a, st);
-        case 16: return launch_bwd_dq_tc_p<16, false, 0>(d, p, pad, K, V, dY, a, st);
-        case 32: return launch_bwd_dq_tc_p<32, false, 0>(d, p, pad, K, V, dY, a, st);
-        default: return launch_bwd_dq_tc_p<64, false, 0>(d, p, pad, K, V, dY, a, st);
-    }
+    return has_padding(d, mask) ? launch_bwd_dq_tc_n<D, true>(d, p, K, V, dY, a, st) : launch_bwd_dq_tc_n<D, false>(d, p, K, V, dY, a, st);
 }
 
-template <int D, int DRT, bool kRanges>
+template <int D, bool kRanges>
 int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const void *V, const void *dY, BwdTokTcArgs a, cudaStream_t st) {
     CUtensorMap tmK, tmV, tmG;
     int rc;
@@ -64,26 +49,15 @@ int launch_bwd_token_tc_n(const flare_desc_t *d, int sms, const void *K, const v
     using SM = BwdTokSmem<D>;
     a.stages = SM::stages(a.M);
     if (a.stages < 1) return FLARE_ERR_UNSUPPORTED;
-    if constexpr (SM::kSplitRegs) {
-        static std::atomic<int> launched_with{0};
-        int regs = launched_with.load(std::memory_order_relaxed);
-        if (regs == 0) {
-            cudaFuncAttributes attr;
-            FLARE_CUDA(cudaFuncGetAttributes(&attr, bwd_token_tc_kernel<D, DRT, kRanges>));
-            launched_with.store(regs = (attr.numRegs + 7) / 8 * 8, std::memory_order_relaxed);
-        }
-        constexpr int few = 32 * kTokFirstMathWarp, many = SM::kThreads - few;
-        if (regs * SM::kThreads < SM::kFewRegs * few + SM::kManyRegs * many) return FLARE_ERR_UNSUPPORTED;
-    }
     static std::atomic<uint64_t> smem_opt_in{0};
-    if ((rc = ensure_big_smem(bwd_token_tc_kernel<D, DRT, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
+    if ((rc = ensure_big_smem(bwd_token_tc_kernel<D, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
     a.tiles = (d->N + kTile - 1) / kTile;
-    FLARE_CUDA(launch_after(bwd_token_tc_kernel<D, DRT, kRanges>, dim3((unsigned)token_splits(d, a.tiles, a.M, sms), d->H, d->B), BwdTokSmem<D>::kThreads, BwdTokSmem<D>::total(a.stages, a.M), st,  tmK, tmV, tmG, a));
+    FLARE_CUDA(launch_after(bwd_token_tc_kernel<D, kRanges>, dim3((unsigned)token_splits(d, a.tiles, a.M, sms), d->H, d->B), SM::kThreads, SM::total(a.stages, a.M), st, tmK, tmV, tmG, a));
     return FLARE_OK;
 }
 
 // The launch's range of latents is [m0, m0 + mc); dd_sums, kvacc: see BwdTokTcArgs.
-template <int D, int DRT>
+template <int D>
 int launch_bwd_token_tc(const flare_desc_t *d, int sms, const void *Q, const void *K, const void *V, const void *dY,
                         const uint8_t *mask, const float *Z, const float *dZ, const float *lse_enc, const float *de,
                         const float *lse_dec, const float *around, const float *e, void *dK, void *dV, float *dd, uint32_t *status, cudaStream_t st, int m0, int mc,
@@ -96,7 +70,7 @@ int launch_bwd_token_tc(const flare_desc_t *d, int sms, const void *Q, const voi
     a.B = d->B; a.H = d->H; a.N = d->N; a.M = mc;
     a.mtot = d->M; a.m0 = m0; a.first = m0 == 0; a.last = m0 + mc >= d->M; a.kvacc = kvacc; a.dd_sums = dd_sums;
     a.scale = d->scale; a.sl2 = d->scale * kLog2e;
-    return token_in_ranges(d) ? launch_bwd_token_tc_n<D, DRT, true>(d, sms, K, V, dY, a, st) : launch_bwd_token_tc_n<D, DRT, false>(d, sms, K, V, dY, a, st);
+    return token_in_ranges(d) ? launch_bwd_token_tc_n<D, true>(d, sms, K, V, dY, a, st) : launch_bwd_token_tc_n<D, false>(d, sms, K, V, dY, a, st);
 }
 
 template <int D, int DRT, bool kRanges>
@@ -187,7 +161,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
     if (const int rc = clear_header(ws, 0, st)) return rc;
     int dz_parts = pa.P;
     bool dz_on_tc = skip_pass_a;
-    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+    if constexpr (std::is_same<T, __nv_bfloat16>::value && D >= 32) {
         if (!skip_pass_a && use_tc(d)) {
             const LeanPlan tp = dz_plan(d, sms);
             uint32_t *status = reinterpret_cast<uint32_t *>(ws);
@@ -215,9 +189,7 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
     }
     bool on_tc = false;
     int dq_parts = pb.P;
-    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-        constexpr int DK = D < 16 ? 16 : D;                     // width the kernels multiply (D < 16: narrow forms)
-        constexpr int DRT = D < 16 ? D : 0;
+    if constexpr (std::is_same<T, __nv_bfloat16>::value && D >= 32) {
         uint32_t *status = reinterpret_cast<uint32_t *>(ws);
         on_tc = use_tc(d);
         if (on_tc) {
@@ -227,12 +199,12 @@ int launch_backward_simt(const flare_desc_t *d, int sms, const void *Q, const vo
             for (int k = 0; k < ranges; ++k) {
                 const int m0 = k * R;
                 const bool to_dd = (ranges - 1 - k) % 2 == 0;
-                if (const int rc = launch_bwd_token_tc<DK, DRT>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, around, e, dK, dV, to_dd ? dd : dd_other, status,
+                if (const int rc = launch_bwd_token_tc<D>(d, sms, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, around, e, dK, dV, to_dd ? dd : dd_other, status,
                                                                 st, m0, d->M - m0 < R ? d->M - m0 : R, to_dd ? dd_other : dd, kvacc))
                     return rc;
             }
             const TcEncodePlan p = tc_dq_plan(d, sms);
-            if (const int rc = launch_bwd_dq_tc(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, around, part, status, st)) return rc;
+            if (const int rc = launch_bwd_dq_tc<D>(d, p, Q, K, V, dY, mask, Z, dZ, lse_enc, de, lse_dec, dd, around, part, status, st)) return rc;
             dq_parts = p.P;
         }
     }

@@ -128,12 +128,12 @@ struct BwdDqTcArgs {
     int tiles, splits, blocks; // blocks: of 128 latents per head
 };
 
-template <int DG, bool kPair>
+template <int D>
 struct BwdDqSmem {
-    using G = TileGeom<DG>;
-    static constexpr int kParts = DG == 64 && !kPair ? 3 : 2, kLat = 1 + 2 * kParts;   // parts of Z and dZ (see the kernel); with Q, latent operands
+    using G = TileGeom<D>;
+    static constexpr int kParts = D == 64 ? 3 : 2, kLat = 1 + 2 * kParts;   // parts of Z and dZ (see the kernel); with Q, latent operands
     static constexpr int kCst = 8, kAhead = 4;                                   // tiles of column constants in the ring, of them on their way
-    static constexpr size_t kCstBytes = (size_t)(kPair ? 2 : 1) * 3 * kTile * sizeof(float);   // per head: -lse_dec, -dd, mask
+    static constexpr size_t kCstBytes = (size_t)3 * kTile * sizeof(float);     // -lse_dec, -dd, mask
     static constexpr size_t total_for(int n) {
         return (size_t)n * 3 * G::TILE_BYTES + (size_t)kLat * kTile * G::RB + kCst * kCstBytes + 768 + 1024;
     }
@@ -149,23 +149,17 @@ struct BwdDqSmem {
     static constexpr size_t total = total_for(kStages) < kTcMinSmem ? kTcMinSmem : total_for(kStages);
 };
 
-// grid = (heads or head pairs * blocks, splits, B): heads that share token rows run at the same time; a CTA takes one block of 128 latents and a contiguous range of token tiles.
-// kPair: two heads of at most 64 latents side by side on the lanes, as in the encode kernel (block-diagonal latent operands over
-// the 2 D columns the heads occupy in a token row).  DRT = 8 or 4 (with D = 16): the narrow form (the head is DRT wide in memory;
-// token tiles carry the neighbouring heads' features beside the head's own, every latent operand zeros there).
+// grid = (heads * blocks, splits, B): heads that share token rows run at the same time; a CTA takes one block of 128 latents and a contiguous range of token tiles.
 // kPadded: the launch has padded tokens (a key mask, or N not a multiple of the tile): a third constant per column, 0 or -inf.
-template <int D, bool kPair, int DRT, bool kPadded>
+template <int D, bool kPadded>
 __global__ void __launch_bounds__(kDqThreads, 1)
 bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                  const __grid_constant__ CUtensorMap tmG, BwdDqTcArgs a) {
-    constexpr int DG = kPair ? 2 * D : D;
-    using G = TileGeom<DG>;
-    using SM = BwdDqSmem<DG, kPair>;
-    constexpr int DR = DRT ? DRT : D;                           // head width in memory
-    static_assert(!(kPair && DRT), "head pairs are full width");
+    using G = TileGeom<D>;
+    using SM = BwdDqSmem<D>;
     // The units take turns on as many accumulators as there is room for: the tensor core truncates each of the thousands of sums that a
     // split adds up in float32, an error that grows with their number.
-    constexpr int kAccs = (512 - kDqAcc) / DG;
+    constexpr int kAccs = (512 - kDqAcc) / D;
     // D = 64: the three products carry all 24 bits of Z, dZ and dS, in three parts each, and a unit's sums go to float32 sums in registers
     // two units later, when their accumulator is free again: 16 of the 64 columns to each of the four warps that share a quarter of the lanes.
     // (This width used to run in float32 arithmetic on the CUDA cores, twenty times slower.  In halves, summed in tensor memory, as the
@@ -174,7 +168,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     // 2.6e-6, on features of point clouds 5.1e-6 / 7.2e-6 / 2.9e-6.  That training step: 182 us in halves, 186 with this, 192 with
     // the token kernel's third part.)
     constexpr bool kThird = SM::kParts == 3;
-    static_assert(!kThird || (kAccs == 2 && D == 64 && DRT == 0), "a warp's columns, and the buffer's accumulator");
+    static_assert(!kThird || (kAccs == 2 && D == 64), "a warp's columns, and the buffer's accumulator");
     static_assert(kAccs >= 1 && (kAccs & (kAccs - 1)) == 0, "tensor memory");
     constexpr int UNIT = kDqUnit, UPT = kTile / UNIT, nstages = SM::kStages;
     static_assert(nstages >= 2, "one tile is finished while the next begins");
@@ -189,11 +183,10 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int M = a.M;
-    const int split = blockIdx.y, h = (kPair ? 2 : 1) * (blockIdx.x / a.blocks), lb = blockIdx.x % a.blocks, b = blockIdx.z;
+    const int split = blockIdx.y, h = blockIdx.x / a.blocks, lb = blockIdx.x % a.blocks, b = blockIdx.z;
     const int t_begin = (int)((long)a.tiles * split / a.splits), t_end = (int)((long)a.tiles * (split + 1) / a.splits);
     const int nt = t_end - t_begin;
-    const int rows_here = kPair ? M : min(M - lb * kTile, kTile);
-    const int off = DRT ? narrow_offset(h, DR) : 0;             // the head's first column within a token tile row
+    const int rows_here = min(M - lb * kTile, kTile);
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
 
     if (threadIdx.x == 0) {
@@ -205,48 +198,37 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         ptx::prefetch_tensormap(&tmV);
         ptx::prefetch_tensormap(&tmG);
     }
-    float *kmin = reinterpret_cast<float *>(tmem_slot + 2);     // smallest lse_enc, per head of the CTA
-    volatile uint32_t *two_exp = tmem_slot + 4;                 // [kCst][head]: the tile needs an exponential of its own for W_enc
+    float *kmin = reinterpret_cast<float *>(tmem_slot + 2);     // smallest lse_enc
+    volatile uint32_t *two_exp = tmem_slot + 4;                 // [kCst]: the tile needs an exponential of its own for W_enc
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     ptx::grid_launch();
     ptx::grid_wait();
     if (warp == 3) {
-#pragma unroll
-        for (int w = 0; w < (kPair ? 2 : 1); ++w) {
-            const float k = warp_lse_min(a.lse_enc + ((size_t)b * a.H + h + w) * M + lb * kTile, rows_here);
-            if (lane == 0) kmin[w] = k;
-        }
+        const float k = warp_lse_min(a.lse_enc + ((size_t)b * a.H + h) * M + lb * kTile, rows_here);
+        if (lane == 0) *kmin = k;
     }
-    // latent operands Q, Z_hi, Z_lo, dZ_hi, dZ_lo (D = 64: three parts of Z and dZ): zeros where there is no row (or, pair and narrow forms, no feature), then the rows
-    const bool gaps = kPair || DRT != 0 || rows_here < kTile;
-    const float *centre = a.around + ((size_t)b * a.H + h) * a.around_rows * DR;
-    if (gaps) {
+    // latent operands Q, Z_hi, Z_lo, dZ_hi, dZ_lo (D = 64: three parts of Z and dZ): zeros where there is no row, then the rows
+    const float *centre = a.around + ((size_t)b * a.H + h) * a.around_rows * D;
+    if (rows_here < kTile) {
         for (int i = threadIdx.x; i < SM::kLat * kTile * (G::RB / 16); i += kDqThreads)
             reinterpret_cast<uint4 *>(smem + SM::lat_off(0))[i] = make_uint4(0, 0, 0, 0);
     }
     __syncthreads();
-#pragma unroll
-    for (int w = 0; w < (kPair ? 2 : 1); ++w) {
-        const size_t q0 = (size_t)(h + w) * M + lb * kTile, r0 = ((size_t)b * a.H + h + w) * M + lb * kTile;
-        if constexpr (DR == 4) {
-            stage_rows4<DG>(smem + SM::lat_off(0), a.Q + q0 * DR, rows_here, off);
-            stage_rows4_hilo<DG>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, off, centre);
-            stage_rows4_hilo<DG>(smem + SM::lat_off(3), smem + SM::lat_off(4), a.dZ + r0 * DR, rows_here, off);
-        } else {
-            stage_bf16<DG, DR>(smem + SM::lat_off(0), a.Q + q0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads);
-            stage_hilo<DG, DR, kThird>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x, kDqThreads,
-                                       centre + w * a.around_rows * DR, UnitFactor(), smem + SM::lat_off(3));
-            constexpr int dz0 = 1 + SM::kParts;
-            stage_hilo<DG, DR, kThird>(smem + SM::lat_off(dz0), smem + SM::lat_off(dz0 + 1), a.dZ + r0 * DR, rows_here, 64 * w, w * (D / 8), threadIdx.x,
-                                       kDqThreads, nullptr, UnitFactor(), smem + SM::lat_off(SM::kLat - 1));
-        }
+    {
+        const size_t q0 = (size_t)h * M + lb * kTile, r0 = ((size_t)b * a.H + h) * M + lb * kTile;
+        constexpr int dz0 = 1 + SM::kParts;
+        stage_bf16<D, D>(smem + SM::lat_off(0), a.Q + q0 * D, rows_here, 0, 0, threadIdx.x, kDqThreads);
+        stage_hilo<D, D, kThird>(smem + SM::lat_off(1), smem + SM::lat_off(2), a.Z + r0 * D, rows_here, 0, 0, threadIdx.x, kDqThreads, centre, UnitFactor(),
+                                 smem + SM::lat_off(3));
+        stage_hilo<D, D, kThird>(smem + SM::lat_off(dz0), smem + SM::lat_off(dz0 + 1), a.dZ + r0 * D, rows_here, 0, 0, threadIdx.x, kDqThreads, nullptr,
+                                 UnitFactor(), smem + SM::lat_off(SM::kLat - 1));
     }
     ptx::fence_proxy_async_smem();
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tm = *tmem_slot;
-    const float lse_min[2] = {kmin[0], kmin[kPair ? 1 : 0]};
+    const float lse_min = *kmin;
 
     if (warp == 0) {
         if (ptx::elect_one()) {
@@ -255,9 +237,9 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (!ptx::mbar_wait(bar(T_EMPTY + s), ((i / nstages) & 1) ^ 1, abort_flag, kErrBwdDq | 1)) break;
                 ptx::mbar_arrive_expect_tx(bar(T_FULL + s), 3 * G::TILE_BYTES);
                 uint8_t *dst = smem + (size_t)s * 3 * G::TILE_BYTES;
-                ptx::tma_load_3d(ptx::smem_u32(dst), &tmK, bar(T_FULL + s), h * DR - off, (t_begin + i) * kTile, b);
-                ptx::tma_load_3d(ptx::smem_u32(dst + G::TILE_BYTES), &tmV, bar(T_FULL + s), h * DR - off, (t_begin + i) * kTile, b);
-                ptx::tma_load_3d(ptx::smem_u32(dst + 2 * G::TILE_BYTES), &tmG, bar(T_FULL + s), h * DR - off, (t_begin + i) * kTile, b);
+                ptx::tma_load_3d(ptx::smem_u32(dst), &tmK, bar(T_FULL + s), h * D, (t_begin + i) * kTile, b);
+                ptx::tma_load_3d(ptx::smem_u32(dst + G::TILE_BYTES), &tmV, bar(T_FULL + s), h * D, (t_begin + i) * kTile, b);
+                ptx::tma_load_3d(ptx::smem_u32(dst + 2 * G::TILE_BYTES), &tmG, bar(T_FULL + s), h * D, (t_begin + i) * kTile, b);
             }
         }
     } else if (warp == 3) {
@@ -265,7 +247,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         // in a tile with a token beyond kOneExpLog2, the addend of its own exponent.  The values come by asynchronous copies, kAhead
         // tiles on their way at a time (with one tile's loads in flight this warp held the whole kernel back), and are
         // turned into constants in place.
-        constexpr int AH = SM::kAhead, NW = kPair ? 2 : 1;
+        constexpr int AH = SM::kAhead;
         uint32_t masks[AH];                                     // mask bytes of this lane's four tokens
         auto fetch = [&](int i) -> uint32_t {
             float *cst = reinterpret_cast<float *>(smem + SM::cst_off + (i % SM::kCst) * SM::kCstBytes);
@@ -274,11 +256,8 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             for (int e = 0; e < kTile / 32; ++e) {
                 const int r = e * 32 + lane, n = min((t_begin + i) * kTile + r, a.N - 1);
                 const size_t nn = (size_t)b * a.N + n;
-#pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    ptx::copy_async4(ptx::smem_u32(cst + w * 3 * kTile + r), a.lse_dec + nn * a.H + h + w);
-                    ptx::copy_async4(ptx::smem_u32(cst + (w * 3 + 1) * kTile + r), a.dd + ((size_t)b * a.H + h + w) * a.N + n);
-                }
+                ptx::copy_async4(ptx::smem_u32(cst + r), a.lse_dec + nn * a.H + h);
+                ptx::copy_async4(ptx::smem_u32(cst + kTile + r), a.dd + ((size_t)b * a.H + h) * a.N + n);
                 if (kPadded && a.key_mask != nullptr && a.key_mask[nn] == 0) mk &= ~(0xffu << (8 * e));
             }
             return mk;
@@ -298,26 +277,23 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 __syncwarp();
                 const int c = i % SM::kCst;
                 float *cst = reinterpret_cast<float *>(smem + SM::cst_off + c * SM::kCstBytes);
+                float ld[kTile / 32];
+                bool part[kTile / 32], far = false;
 #pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    float ld[kTile / 32];
-                    bool part[kTile / 32], far = false;
-#pragma unroll
-                    for (int e = 0; e < kTile / 32; ++e) {
-                        const int r = e * 32 + lane;
-                        const bool in = (t_begin + i) * kTile + r < a.N;
-                        ld[e] = in ? cst[w * 3 * kTile + r] * kBwdLog2e : INFINITY;
-                        part[e] = in && ((masks[k] >> (8 * e)) & 0xffu) != 0;
-                        cst[w * 3 * kTile + r] = -ld[e];
-                        cst[(w * 3 + 1) * kTile + r] = in ? -cst[(w * 3 + 1) * kTile + r] : 0.f;
-                        far = far || (part[e] && !(ld[e] - lse_min[w] <= kOneExpLog2));
-                    }
-                    far = __any_sync(0xffffffffu, far);
-#pragma unroll
-                    for (int e = 0; e < kTile / 32; ++e)
-                        cst[(w * 3 + 2) * kTile + e * 32 + lane] = far ? (part[e] ? 0.f : -INFINITY) : (part[e] ? ptx::ex2(ld[e] - lse_min[w]) : 0.f);
-                    if (lane == 0) two_exp[c * 2 + w] = far ? 1u : 0u;
+                for (int e = 0; e < kTile / 32; ++e) {
+                    const int r = e * 32 + lane;
+                    const bool in = (t_begin + i) * kTile + r < a.N;
+                    ld[e] = in ? cst[r] * kBwdLog2e : INFINITY;
+                    part[e] = in && ((masks[k] >> (8 * e)) & 0xffu) != 0;
+                    cst[r] = -ld[e];
+                    cst[kTile + r] = in ? -cst[kTile + r] : 0.f;
+                    far = far || (part[e] && !(ld[e] - lse_min <= kOneExpLog2));
                 }
+                far = __any_sync(0xffffffffu, far);
+#pragma unroll
+                for (int e = 0; e < kTile / 32; ++e)
+                    cst[2 * kTile + e * 32 + lane] = far ? (part[e] ? 0.f : -INFINITY) : (part[e] ? ptx::ex2(ld[e] - lse_min) : 0.f);
+                if (lane == 0) two_exp[c] = far ? 1u : 0u;
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(bar(C_FULL + c));
                 const int next = i + AH;
@@ -332,7 +308,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     } else if (warp == 1) {
         const int units = UPT * nt;
         if (ptx::elect_one()) {
-            constexpr uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0), idescQ = ptx::instr_desc_bf16(128, DG, 0, 1);
+            constexpr uint32_t idescS = ptx::instr_desc_bf16(128, UNIT, 0, 0), idescQ = ptx::instr_desc_bf16(128, D, 0, 1);
             // (descriptors as 32-bit low words beside a constant high word: see ptx::desc)
             constexpr uint32_t HI = ptx::desc_hi(G::SBO, G::SWZ), TILE = G::TILE_BYTES >> 4, STEP16 = (16 * G::RB) >> 4, LAT = (kTile * G::RB) >> 4;
             const uint32_t lat0 = ptx::desc_lo(ptx::smem_u32(smem + SM::lat_off(0)), 16), k0 = ptx::desc_lo(ptx::smem_u32(smem), 16);
@@ -355,7 +331,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     const uint32_t col = bcol + of * UNIT, td = kd + (of == 0 ? 0 : of == 1 ? 2 * TILE : TILE);
                     const bool more = at > 0;                   // adds to an earlier part's product
 #pragma unroll
-                    for (int k = 0; k < DG / 16; ++k)
+                    for (int k = 0; k < D / 16; ++k)
                         ptx::mma_ss(col, ptx::desc(ld + w * LAT + 2 * k, HI), ptx::desc(td + 2 * k, HI), idescS, k > 0 || more);
                 }
                 ptx::mma_commit(bar(S_FULL + (n & 1)));
@@ -369,7 +345,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             for (int n = 0; ok && n < 2 && n < units; ++n) ok = tiles(n);
             for (int n = 0; ok && n < units; ++n) {
                 // dQ_part += dS_unit K_unit (the parts of dS in turn): 16 token rows of the K tile per k-step as the MN-major B operand
-                const uint32_t bcol = tm + (n & 1) * kDqBuf, acc = tm + kDqAcc + (n & (kAccs - 1)) * DG;
+                const uint32_t bcol = tm + (n & 1) * kDqBuf, acc = tm + kDqAcc + (n & (kAccs - 1)) * D;
                 uint32_t kd = k0 + MN + (uint32_t)o_stage * 3 * TILE + (uint32_t)o_u * (UNIT / 16) * STEP16;
                 ptx::opaque(kd);
                 if (!ptx::mbar_wait(bar(P_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdDq | 4)) break;
@@ -399,19 +375,18 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     } else if (warp >= kDqFirstMathWarp) {
         const int cg = (warp - kDqFirstMathWarp) >> 2;         // the group of 16 columns this warp works on
         const int row = ((warp & 3) << 5) + lane;               // TMEM lane = latent within the block (or within the pair)
-        const int second = kPair ? row >> 6 : 0;                // the head of this lane's latent (uniform over the warp)
         const uint32_t gcol = tm + ((uint32_t)((warp & 3) << 5) << 16);
         const float2 sl2p = make_float2(a.sl2, a.sl2);
-        const int m = kPair ? (row & 63) : lb * kTile + row;
+        const int m = lb * kTile + row;
         // this thread's latent: -lse_enc in log2 units (-inf for a latent that saw no valid token or lies beyond M), -de
         float nle = -INFINITY, nde = 0.f;
         if (m < M) {
-            const size_t r = ((size_t)b * a.H + h + second) * M + m;
+            const size_t r = ((size_t)b * a.H + h) * M + m;
             const float le = a.lse_enc[r];
             nle = (le == -INFINITY) ? -INFINITY : -le * kBwdLog2e;
             nde = -a.de[r];
         }
-        const float fr = ptx::ex2(nle + lse_min[second]);       // 2^(K - lse_enc)
+        const float fr = ptx::ex2(nle + lse_min);       // 2^(K - lse_enc)
         const float2 nlep = make_float2(nle, nle), frp = make_float2(fr, fr), ndep = make_float2(nde, nde);
         bool ok = true;
         int n = 0;
@@ -419,14 +394,14 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         // (kThird) the sums of unit i, complete when the tiles of unit i + 2 are
         auto drain = [&](int i) {
             uint32_t r[16];
-            ptx::tmem_ld16(gcol + kDqAcc + (i & 1) * DG + cg * 16, r);
+            ptx::tmem_ld16(gcol + kDqAcc + (i & 1) * D + cg * 16, r);
             ptx::tmem_wait_ld();
 #pragma unroll
             for (int k = 0; k < 16; ++k) sum[kThird ? k : 0] += __uint_as_float(r[k]);
         };
         for (int tile = 0; ok && tile < nt; ++tile) {
             const int c = tile % SM::kCst;
-            const float *cst = reinterpret_cast<const float *>(smem + SM::cst_off + c * SM::kCstBytes) + second * 3 * kTile + cg * 16;
+            const float *cst = reinterpret_cast<const float *>(smem + SM::cst_off + c * SM::kCstBytes) + cg * 16;
             if (!(ok = warp_wait(bar(C_FULL + c), (tile / SM::kCst) & 1, abort_flag, kErrBwdDq | 8))) break;
             auto units = [&](auto two) {
                 constexpr bool kTwo = decltype(two)::value;
@@ -478,7 +453,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                     if (lane == 0) ptx::mbar_arrive(bar(P_FULL + (n & 1)));
                 }
             };
-            if (!__any_sync(0xffffffffu, two_exp[c * 2 + second] != 0)) units(std::false_type{});
+            if (!__any_sync(0xffffffffu, two_exp[c] != 0)) units(std::false_type{});
             else units(std::true_type{});
             if (lane == 0) ptx::mbar_arrive(bar(C_EMPTY + c));
         }
@@ -503,7 +478,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 #pragma unroll
                 for (int dc = 0; dc < D / 16; ++dc) {
                     uint32_t r[16];
-                    ptx::tmem_ld16(gcol + kDqAcc + i * DG + second * D + dc * 16, r);
+                    ptx::tmem_ld16(gcol + kDqAcc + i * D + dc * 16, r);
                     ptx::tmem_wait_ld();
 #pragma unroll
                     for (int k = 0; k < 16; ++k) acc[dc * 16 + k] += __uint_as_float(r[k]);
@@ -511,13 +486,9 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             }
             if (ok && m < M) {
                 const long rows = (long)a.B * a.H * M;
-                float4 *dst = reinterpret_cast<float4 *>(a.part + ((size_t)split * rows + ((size_t)b * a.H + h + second) * M + m) * DR);
-                if (DR == 4) {
-                    dst[0] = make_float4(off ? acc[4] : acc[0], off ? acc[5] : acc[1], off ? acc[6] : acc[2], off ? acc[7] : acc[3]);
-                } else {
+                float4 *dst = reinterpret_cast<float4 *>(a.part + ((size_t)split * rows + ((size_t)b * a.H + h) * M + m) * D);
 #pragma unroll
-                    for (int dc = 0; dc < DR / 4; ++dc) dst[dc] = make_float4(acc[4 * dc], acc[4 * dc + 1], acc[4 * dc + 2], acc[4 * dc + 3]);
-                }
+                for (int dc = 0; dc < D / 4; ++dc) dst[dc] = make_float4(acc[4 * dc], acc[4 * dc + 1], acc[4 * dc + 2], acc[4 * dc + 3]);
             }
         }
     }
@@ -597,12 +568,6 @@ struct BwdTokSmem {
         return fit >= 4 ? 2 : fit >= 2 ? 1 : 0;
     }
     static constexpr int kRing = 4, kPlanes = D == 64 ? 2 : 3, kRingTile = kPlanes * kTile;   // tiles of token constants on their way or in use
-    // D = 16 (and the narrow forms): the arithmetic warps take registers that the other four leave.  Without, the pair of constants that e adds
-    // made the compiler put others together again for every pair of columns: 127 instead of 109 us (2 x 65536 tokens, M = 64, D = 16, 8 heads), 1000 instead
-    // of 910 (131072, M = 1024, D = 8).  At D = 32 the issuing warps then have too few: 118 instead of 106 (32 x 4096, M = 128).  The sum is what the
-    // block is launched with (20 warps of 96), which the host checks: the warps that ask for more wait for it.
-    static constexpr bool kSplitRegs = D == 16;
-    static constexpr int kFewRegs = 64, kManyRegs = 104;
     static constexpr int kAlign = D == 64 ? 1024 : 512;         // (rows of 64 bytes are swizzled alike every 512: that much less to leave room for)
     // D = 64: dd[n] is subtracted from products that the dQ kernel forms of three parts of Z, so A is formed of three as well (with two,
     // dQ on features of point clouds was 4.7e-6 to 5.4e-6 of its norm from float64 instead of 2.6e-6 to 3.0e-6), as long as the third fits
@@ -631,15 +596,14 @@ struct BwdTokSmem {
     }
 };
 
-// grid = (CTAs per head, H, B); a CTA takes the token tiles blockIdx.x, blockIdx.x + gridDim.x, ...  kRanges: see BwdTokTcArgs.  DRT: as in
-// the dQ kernel.
-template <int D, int DRT, bool kRanges>
+// grid = (CTAs per head, H, B); a CTA takes the token tiles blockIdx.x, blockIdx.x + gridDim.x, ...  kRanges: see BwdTokTcArgs.
+template <int D, bool kRanges>
 __global__ void __launch_bounds__(BwdTokSmem<D>::kThreads, 1)
 bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                     const __grid_constant__ CUtensorMap tmG, BwdTokTcArgs a) {
     using G = TileGeom<D>;
     using SM = BwdTokSmem<D>;
-    constexpr int UNIT = SM::UNIT, NCG = SM::NCG, kThreads = SM::kThreads, kMaxSt = SM::kMaxStages, RING = SM::kRing, DR = DRT ? DRT : D;
+    constexpr int UNIT = SM::UNIT, NCG = SM::NCG, kThreads = SM::kThreads, kMaxSt = SM::kMaxStages, RING = SM::kRing;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = ptx::align_smem<SM::kAlign>(smem_raw);
     const int M = a.M, stages = a.stages;
@@ -660,16 +624,13 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
     const int nu = (M + UNIT - 1) / UNIT;                       // latent units of a tile; the last may be narrower
     const int wlast = M - (nu - 1) * UNIT;
-    // Sets of warps that take the units in turn: two where a unit fills no more than half of the column groups (then a tile is one unit).
-    const int sets = NCG == 4 && M <= 32 ? 2 : 1, cps = sets == 2 ? 2 : NCG;
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S, A or C
     const int log_accs = SM::log2_accs(ucols);                  // accumulators in turn for the tiles
-    const int off = DRT ? narrow_offset(h, DR) : 0;
     const bool third = D == 64 && M <= SM::kThirdMost;
     auto bar = [&](int i) { return ptx::smem_u32(bars + i); };
 
     if (threadIdx.x == 0) {
-        const uint32_t math = 4 * cps;                          // warps that work on a unit
+        const uint32_t math = 4 * NCG;                          // warps that work on a unit
         for (int i = 0; i < NBARS; ++i)
             ptx::mbar_init(bar(i), i >= DD_FULL || (i >= ACC_EMPTY && i < DD_FULL) || (i >= P_FULL && i < C_FULL) ? math
                                    : i >= C_EMPTY && i < ACC_FULL ? math + 1u : i < T_EMPTY || (i >= C_FULL && i < C_EMPTY) ? 1u : 2u);   // (two issuing warps)
@@ -683,7 +644,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::grid_launch();
     ptx::grid_wait();
     const size_t q0 = (size_t)h * a.mtot + a.m0, r0 = ((size_t)b * a.H + h) * a.mtot + a.m0;
-    const float *centre = a.around + ((size_t)b * a.H + h) * a.around_rows * DR;
+    const float *centre = a.around + ((size_t)b * a.H + h) * a.around_rows * D;
     float K, least, unfolded;                                   // (unfolded != 0: c is 1)
     {
         // K: the middle of the latents' lse_enc (log2 units), leaving out those that saw no valid token and those whose encode is switched off
@@ -704,8 +665,6 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             extremes[2 * warp] = lo;
             extremes[2 * warp + 1] = hi;
         }
-        if (DRT != 0)                                           // narrow form: the other columns of every row stay zero
-            for (int i = threadIdx.x; i < 5 * M * (G::RB / 16); i += kThreads) reinterpret_cast<uint4 *>(smem + SM::lat_off(stages, M, 0))[i] = make_uint4(0, 0, 0, 0);
         __syncthreads();
         for (int w = 0; w < kThreads / 32; ++w) {
             lo = fminf(lo, extremes[2 * w]);
@@ -723,16 +682,10 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
         uint8_t *lat[5];
 #pragma unroll
         for (int w = 0; w < 5; ++w) lat[w] = smem + SM::lat_off(stages, M, w);
-        if constexpr (DR == 4) {
-            stage_rows4<D>(lat[SM::QR], a.Q + q0 * DR, M, off);
-            stage_rows4_hilo<D>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, off, centre);
-            stage_rows4_hilo<D>(lat[SM::DH], lat[SM::DL], a.dZ + r0 * DR, M, off, nullptr, factor);
-        } else {
-            stage_bf16<D, DR>(lat[SM::QR], a.Q + q0 * DR, M, 0, 0, threadIdx.x, kThreads);
-            if (third) stage_hilo<D, DR, true>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, centre, UnitFactor(), smem + SM::lat_off(stages, M, SM::Z3));
-            else stage_hilo<D, DR>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * DR, M, 0, 0, threadIdx.x, kThreads, centre);
-            stage_hilo<D, DR>(lat[SM::DH], lat[SM::DL], a.dZ + r0 * DR, M, 0, 0, threadIdx.x, kThreads, nullptr, factor);
-        }
+        stage_bf16<D, D>(lat[SM::QR], a.Q + q0 * D, M, 0, 0, threadIdx.x, kThreads);
+        if (third) stage_hilo<D, D, true>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * D, M, 0, 0, threadIdx.x, kThreads, centre, UnitFactor(), smem + SM::lat_off(stages, M, SM::Z3));
+        else stage_hilo<D, D>(lat[SM::ZH], lat[SM::ZL], a.Z + r0 * D, M, 0, 0, threadIdx.x, kThreads, centre);
+        stage_hilo<D, D>(lat[SM::DH], lat[SM::DL], a.dZ + r0 * D, M, 0, 0, threadIdx.x, kThreads, nullptr, factor);
         for (int m = threadIdx.x; m < M; m += kThreads) {
             const float c = factor(m);
             cst[m] = c == 0.f ? -INFINITY : unfolded != 0.f ? -a.lse_enc[r0 + m] * kBwdLog2e : -K;
@@ -745,10 +698,6 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     ptx::tc_fence_after();
     const uint32_t tm = *tmem_slot;
     const uint32_t bcols = 3 * ucols, acc0 = 2 * bcols;         // columns of a buffer; the first accumulator
-    if constexpr (SM::kSplitRegs) {
-        if (warp < kTokFirstMathWarp) ptx::regs_down<SM::kFewRegs>();
-        else ptx::regs_up<SM::kManyRegs>();
-    }
 
     if (warp == 0) {
         if (ptx::elect_one()) {
@@ -757,9 +706,9 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (!ptx::mbar_wait(bar(T_EMPTY + s), ((i / stages) & 1) ^ 1, abort_flag, kErrBwdTok | 1)) break;
                 ptx::mbar_arrive_expect_tx(bar(T_FULL + s), 3 * G::TILE_BYTES);
                 uint8_t *dst = smem + (size_t)s * 3 * G::TILE_BYTES;
-                ptx::tma_load_3d(ptx::smem_u32(dst), &tmK, bar(T_FULL + s), h * DR - off, t * kTile, b);
-                ptx::tma_load_3d(ptx::smem_u32(dst + G::TILE_BYTES), &tmV, bar(T_FULL + s), h * DR - off, t * kTile, b);
-                ptx::tma_load_3d(ptx::smem_u32(dst + 2 * G::TILE_BYTES), &tmG, bar(T_FULL + s), h * DR - off, t * kTile, b);
+                ptx::tma_load_3d(ptx::smem_u32(dst), &tmK, bar(T_FULL + s), h * D, t * kTile, b);
+                ptx::tma_load_3d(ptx::smem_u32(dst + G::TILE_BYTES), &tmV, bar(T_FULL + s), h * D, t * kTile, b);
+                ptx::tma_load_3d(ptx::smem_u32(dst + 2 * G::TILE_BYTES), &tmG, bar(T_FULL + s), h * D, t * kTile, b);
             }
         }
     } else if (warp == 2) {
@@ -927,43 +876,43 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             else issue(std::true_type{});
         }
     } else if (warp >= kTokFirstMathWarp) {
-        const int cg = (warp - kTokFirstMathWarp) >> 2, set = sets == 2 ? cg >> 1 : 0, mine = sets == 2 ? cg & 1 : cg;   // columns: 16 from 16 mine on
+        const int mine = (warp - kTokFirstMathWarp) >> 2;       // columns: 16 from 16 mine on
         const int row = ((warp & 3) << 5) + lane;               // TMEM lane = token within the tile
         const uint32_t gcol = tm + ((uint32_t)((warp & 3) << 5) << 16);
         const float2 sl2p = make_float2(a.sl2, a.sl2);
         const float *nle = cst + 16 * mine, *nde = nle + M;
-        // Rows of dK and dV of the set's k-th tile: pieces of eight columns, in turn to the warps that share the tokens.
+        // Rows of dK and dV of the k-th tile: pieces of eight columns, in turn to the warps that share the tokens.
         auto write_rows = [&](int k, float r, float ne) -> bool {
-            constexpr int COLS = DR >= 16 ? DR : 8, PIECES = COLS / 4, PW = DR == 4 ? 4 : 8;
-            const int i = set + k * sets, acc = i & ((1 << log_accs) - 1), tok_n = (int)(blockIdx.x + i * gridDim.x) * kTile + row;
+            constexpr int PIECES = D / 4;
+            const int acc = k & ((1 << log_accs) - 1), tok_n = (int)(blockIdx.x + k * gridDim.x) * kTile + row;
             const bool in = tok_n < a.N;
             const size_t tok = ((size_t)b * a.N + (in ? tok_n : 0)) * a.H + h;
             const uint32_t V = gcol + acc0 + acc * SM::kAccStride;
-            if (!warp_wait(bar(DD_FULL + (k & 3) + 4 * set), (k >> 2) & 1, abort_flag, kErrBwdTok | 7)) return false;
-            if (!warp_wait(bar(ACC_FULL + acc), (i >> log_accs) & 1, abort_flag, kErrBwdTok | 8)) return false;
+            if (!warp_wait(bar(DD_FULL + (k & 3)), (k >> 2) & 1, abort_flag, kErrBwdTok | 7)) return false;
+            if (!warp_wait(bar(ACC_FULL + acc), (k >> log_accs) & 1, abort_flag, kErrBwdTok | 8)) return false;
             ptx::tc_fence_after();
-            const size_t plane = (size_t)a.B * a.N * a.H * DR;  // of the sums over ranges
+            const size_t plane = (size_t)a.B * a.N * a.H * D;   // of the sums over ranges
 #pragma unroll 1
-            for (int p = PIECES <= 2 ? (mine + 2 * k) & (cps - 1) : mine; p < PIECES; p += cps) {
+            for (int p = mine; p < PIECES; p += NCG) {
                 const int which = (p ^ (p >> 2)) & 1, c0 = (p >> 1) * 8;   // dK or dV, and the first column
                 uint32_t x[8], y[8];
                 float dd = 0.f;                                 // less e
                 ptx::tmem_ld8(V + (which == 0 ? 3 * D : 0) + c0, x);
                 ptx::tmem_ld8(V + (which == 0 ? D : 2 * D) + c0, y);
                 if (which == 0) {
-                    const float *part = dds + ((k & 3) * NCG + set * cps) * kTile + row;
+                    const float *part = dds + (k & 3) * NCG * kTile + row;
                     dd = part[0] + part[kTile];
-                    if (cps == 4) dd += part[2 * kTile] + part[3 * kTile];
+                    if (NCG == 4) dd += part[2 * kTile] + part[3 * kTile];
                     const size_t at = ((size_t)b * a.H + h) * a.N + (in ? tok_n : 0);
                     if (kRanges && !a.first) dd += a.dd_sums[at];
                     if (in && c0 == 0) a.dd[at] = !kRanges || a.last ? dd - ne : dd;
                 }
                 ptx::tmem_wait_ld();
-                float f[PW], u[PW];
+                float f[8], u[8];
 #pragma unroll
-                for (int c = 0; c < PW; ++c) {                  // (narrow heads: the head's own columns)
-                    f[c] = __uint_as_float(DR == 4 && off != 0 ? x[(4 + c) & 7] : x[c]);
-                    u[c] = __uint_as_float(DR == 4 && off != 0 ? y[(4 + c) & 7] : y[c]);
+                for (int c = 0; c < 8; ++c) {
+                    f[c] = __uint_as_float(x[c]);
+                    u[c] = __uint_as_float(y[c]);
                     if (which != 0) {
                         f[c] = (f[c] + u[c]) * r;
                         u[c] = 0.f;
@@ -971,9 +920,9 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
                 if (in && kRanges) {
                     auto sums = [&](int at, float *v) {
-                        float4 *sum = reinterpret_cast<float4 *>(a.kvacc + at * plane + tok * DR + c0);
+                        float4 *sum = reinterpret_cast<float4 *>(a.kvacc + at * plane + tok * D + c0);
 #pragma unroll
-                        for (int c = 0; c < PW; c += 4) {       // the earlier ranges' shares
+                        for (int c = 0; c < 8; c += 4) {        // the earlier ranges' shares
                             if (!a.first) {
                                 const float4 e = sum[c / 4];
                                 v[c] += e.x; v[c + 1] += e.y; v[c + 2] += e.z; v[c + 3] += e.w;
@@ -986,13 +935,11 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
                 if (in && (!kRanges || a.last)) {
                     const float sc = which == 0 ? a.scale : 1.f;
-                    uint32_t w[PW / 2];
+                    uint32_t w[4];
 #pragma unroll
-                    for (int c = 0; c < PW / 2; ++c)
+                    for (int c = 0; c < 4; ++c)
                         w[c] = ptx::pack_bf16(fmaf(-dd, u[2 * c], f[2 * c]) * sc, fmaf(-dd, u[2 * c + 1], f[2 * c + 1]) * sc);
-                    __nv_bfloat16 *out = (which ? a.dV : a.dK) + tok * DR + c0;
-                    if constexpr (PW == 4) *reinterpret_cast<uint2 *>(out) = make_uint2(w[0], w[1]);
-                    else *reinterpret_cast<uint4 *>(out) = make_uint4(w[0], w[1], w[2], w[3]);
+                    *reinterpret_cast<uint4 *>((which ? a.dV : a.dK) + tok * D + c0) = make_uint4(w[0], w[1], w[2], w[3]);
                 }
                 __syncwarp();
             }
@@ -1059,17 +1006,16 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             }
             ptx::tmem_wait_st();
         };
-        // All units of the set's tiles in one loop; one more turn writes the last tile's rows.
-        int k = 0, u = 0;                                       // tiles of this set done, unit of the next
+        // All units of the tiles in one loop; one more turn writes the last tile's rows.
+        int k = 0, u = 0;                                       // tiles done, unit of the next
         float nld = 0.f, rr = 0.f, ne = 0.f, r_before = 0.f, ne_before = 0.f;
         bool far = false;
         float2 d2 = make_float2(0.f, 0.f);
         while (true) {
-            const int i = set + k * sets;
-            if (i < nt) {
+            if (k < nt) {
                 if (u == 0) {
-                    const int c = i % RING;
-                    if (!warp_wait(bar(C_FULL + c), (i / RING) & 1, abort_flag, kErrBwdTok | 9)) break;
+                    const int c = k % RING;
+                    if (!warp_wait(bar(C_FULL + c), (k / RING) & 1, abort_flag, kErrBwdTok | 9)) break;
                     const float *at = ring + c * SM::kRingTile + row;
                     nld = at[0];
                     ne = at[kTile];
@@ -1084,7 +1030,7 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive(bar(C_EMPTY + c));
                 }
-                const int n = i * nu + u;
+                const int n = k * nu + u;
                 const uint32_t col = gcol + (n & 1) * bcols + 16 * mine;
                 if (!warp_wait(bar(S_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdTok | 10)) break;
                 ptx::tc_fence_after();
@@ -1092,16 +1038,16 @@ bwd_token_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     if (far) unit(std::true_type{}, col, u * UNIT, make_float2(nld, nld), make_float2(rr, rr), make_float2(ne, ne), d2);
                     else unit(std::false_type{}, col, u * UNIT, make_float2(nld, nld), make_float2(rr, rr), make_float2(ne, ne), d2);
                 }
-                if (u == nu - 1) dds[((k & 3) * NCG + cg) * kTile + row] = d2.x + d2.y;
+                if (u == nu - 1) dds[((k & 3) * NCG + mine) * kTile + row] = d2.x + d2.y;
                 ptx::tc_fence_before();
                 __syncwarp();
                 if (lane == 0) {
                     ptx::mbar_arrive(bar(P_FULL + (n & 1)));
-                    if (u == nu - 1) ptx::mbar_arrive(bar(DD_FULL + (k & 3) + 4 * set));
+                    if (u == nu - 1) ptx::mbar_arrive(bar(DD_FULL + (k & 3)));
                 }
             }
             if (u == 0 && k > 0 && !write_rows(k - 1, r_before, ne_before)) break;
-            if (i >= nt) break;
+            if (k >= nt) break;
             if (++u == nu) {
                 u = 0;
                 ++k;

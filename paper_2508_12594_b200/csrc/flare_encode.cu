@@ -71,15 +71,16 @@ int launch_lean_k(const flare_desc_t *d, const LeanPlan &p, const void *Q, const
 }
 template <int kKind>
 int launch_lean(const flare_desc_t *d, const LeanPlan &p, const void *Q, const void *K, const void *V, const EncodeLeanArgs &a, cudaStream_t st) {
+    // (dZ: what the two sweeps of the backward do not take, no narrow heads and more than 64 latents or heads 64 wide)
+    if constexpr (kKind == kLeanDz)
+        return d->D == 32 ? launch_lean_k<32, false, kKind, 0>(d, p, Q, K, V, a, st) : launch_lean_k<64, false, kKind, 0>(d, p, Q, K, V, a, st);
     const bool pair = lean_pairs(d);
-    switch (d->D) {
+    if constexpr (kKind != kLeanDz) switch (d->D) {
         case 4: return launch_lean_k<16, false, kKind, 4>(d, p, Q, K, V, a, st);
         case 8: return pair ? launch_lean_k<8, true, kKind, 0>(d, p, Q, K, V, a, st) : launch_lean_k<16, false, kKind, 8>(d, p, Q, K, V, a, st);
         case 16: return pair ? launch_lean_k<16, true, kKind, 0>(d, p, Q, K, V, a, st) : launch_lean_k<16, false, kKind, 0>(d, p, Q, K, V, a, st);
         case 32: return pair ? launch_lean_k<32, true, kKind, 0>(d, p, Q, K, V, a, st) : launch_lean_k<32, false, kKind, 0>(d, p, Q, K, V, a, st);
-        default:
-            if constexpr (kKind == kLeanDz) return launch_lean_k<64, false, kKind, 0>(d, p, Q, K, V, a, st);
-            else return FLARE_ERR_UNSUPPORTED;                  // (use_fast_encode knows none)
+        default: return FLARE_ERR_UNSUPPORTED;                  // (use_fast_encode knows none)
     }
 }
 

@@ -372,9 +372,8 @@ inline size_t decode_range_bytes(const flare_desc_t *d) {
 inline TcEncodePlan tc_dq_plan(const flare_desc_t *d, int sms) {
     TcEncodePlan p;
     p.tiles = (d->N + kTile - 1) / kTile;
-    p.pairs = encode_head_pairs(d) ? 1 : (d->M + kTile - 1) / kTile;
-    const long groups = (long)d->B * (encode_head_pairs(d) ? d->H / 2 : d->H) * p.pairs;
-    p.splits = balanced_splits(groups, p.tiles, sms, (size_t)d->B * d->H * d->M * d->D * sizeof(float), p.tiles);
+    p.pairs = (d->M + kTile - 1) / kTile;
+    p.splits = balanced_splits((long)d->B * d->H * p.pairs, p.tiles, sms, (size_t)d->B * d->H * d->M * d->D * sizeof(float), p.tiles);
     p.per_split = 1;
     p.P = p.splits;
     return p;
@@ -390,7 +389,7 @@ struct GuessPlan {
     int chunk, chunks, groups;
 };
 inline GuessPlan guess_plan(const flare_desc_t *d, int sms) {
-    const int pieces = d->H * (d->D >= 8 ? d->D / 8 : 1), per = std::max(1, 256 / pieces);
+    const int pieces = d->H * (d->D / 8), per = std::max(1, 256 / pieces);
     GuessPlan p;
     p.groups = (pieces + 255) / 256;
     const long most = std::max(1L, 5L * sms / ((long)d->B * p.groups));
@@ -408,7 +407,7 @@ struct BwdLayout {
 // tile stages; more are worked off in ranges of equal size, with three float32 planes and dd to read and write between them.  us per backward, two sweeps with
 // two planes and at most 448 latents a range at D = 32 : now, 8 heads of 131072 tokens: D = 32, M = 528 1778 : 1533, 640 1922 : 1587, 1024 3126 : 2284; D = 8,
 // M = 2048 4668 : 3818; 65536, D = 64, M = 208 852 : 874, 256 939 : 904, 400 1654 : 1671; 4 heads of 131072, M = 384 1128 : 1026.
-inline int token_range_most(const flare_desc_t *d) { return d->D == 64 ? 192 : d->D == 32 ? 512 : 1024; }
+inline int token_range_most(const flare_desc_t *d) { return d->D == 64 ? 192 : 512; }
 inline bool token_in_ranges(const flare_desc_t *d) { return use_tc(d) && d->M > token_range_most(d); }
 inline int token_ranges(const flare_desc_t *d) { return (d->M + token_range_most(d) - 1) / token_range_most(d); }
 inline int token_range(const flare_desc_t *d) { return ((d->M + token_ranges(d) - 1) / token_ranges(d) + 15) / 16 * 16; }

@@ -36,11 +36,6 @@ __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
-// Registers of a thread from here on, by all warps of a warp group (four from a multiple of four on).  The second waits until the block's warps have
-// given up as many.
-template <int n> __device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(n)); }
-template <int n> __device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(n)); }
-
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));

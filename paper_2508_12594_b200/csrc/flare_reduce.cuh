@@ -134,7 +134,7 @@ merge_kernel(const float *part_m, const float *part_l, const float *part_acc,
 
 // A first guess e[n] of dd[n] = dY_n . Y_n for the token kernel of the backward, from the stored Y: of dY_n . (Y_n - centre), with Y_n no further from
 // the centre of the rows of Z than these are (features with a mean: what rounding Y left must not be taken for a difference).  A block takes `chunk`
-// tokens of a batch item, in 16-byte pieces (8 at D = 4) as they lie in memory, so that a thread has the same piece of every token it reads.
+// tokens of a batch item, in 16-byte pieces as they lie in memory, so that a thread has the same piece of every token it reads.
 struct GuessArgs {
     const __nv_bfloat16 *Y, *dY;   // [B,N,H,D]
     const float *around;           // see z_around
@@ -143,7 +143,7 @@ struct GuessArgs {
     int chunk, chunks, groups;     // groups: of at most kReduceThreads pieces of a token
 };
 template <int D> struct GuessGeom {
-    static constexpr int F = D >= 8 ? 8 : 4, LPR = D / F;       // features of a piece, pieces of a row
+    static constexpr int F = 8, LPR = D / F;                    // features of a piece, pieces of a row
 };
 template <int D>
 __device__ __forceinline__ void bwd_guess(int block, const GuessArgs &a) {
@@ -189,7 +189,7 @@ bwd_dz_reduce_kernel(const float *part, const float *Z, float *dZ, float *de, in
     ptx::grid_launch();
     ptx::grid_wait();
     if ((int)blockIdx.x >= row_blocks) {
-        bwd_guess<4 * L>((int)blockIdx.x - row_blocks, guess);
+        if constexpr (L >= 8) bwd_guess<4 * L>((int)blockIdx.x - row_blocks, guess);   // (narrower heads have no use for it)
         return;
     }
     const RowMap rm = row_map<L>(slices);
