@@ -119,7 +119,9 @@ int backward_sweeps(const flare_desc_t *d, int sms, const void *Q, const void *K
         for (int m0 = 0; m0 < d->M; m0 += p.range) {
             const BwdDzArgs a{static_cast<const __nv_bfloat16 *>(Q), Z, lse_dec, at(w.part), at(w.dd), status, d->B, d->H, d->N, std::min(p.range, d->M - m0), d->M, m0, m0 == 0,
                               m0 + p.range >= d->M, reinterpret_cast<float4 *>(ws + w.dd_other), d->scale * kLog2e, tiles, p.stages};
-            const int rc = p.ranges > 1 ? launch_dz_sweep<D, DRT, true>(d, p, K, dY, a, st) : launch_dz_sweep<D, DRT, false>(d, p, K, dY, a, st);
+            int rc = FLARE_ERR_UNSUPPORTED;                     // (ranges at D = 32: see use_sweeps)
+            if (p.ranges == 1) rc = launch_dz_sweep<D, DRT, false>(d, p, K, dY, a, st);
+            else if constexpr (D == 16) rc = launch_dz_sweep<D, DRT, true>(d, p, K, dY, a, st);
             if (rc != FLARE_OK) return rc;
         }
         const int slices = reduce_slices(2 * p.splits, d->D);
@@ -133,7 +135,9 @@ int backward_sweeps(const flare_desc_t *d, int sms, const void *Q, const void *K
         const BwdGradArgs a{static_cast<const __nv_bfloat16 *>(Q), Z, at(w.dz), lse_enc, at(w.de), lse_dec, at(w.dd), mask, static_cast<__nv_bfloat16 *>(dK),
                             static_cast<__nv_bfloat16 *>(dV), at(w.part), status, d->B, d->H, d->N, std::min(p.range, d->M - m0), d->M, m0, m0 == 0, m0 + p.range >= d->M,
                             at(w.kvacc), d->scale, d->scale * kLog2e, tiles, p.stages, p.bufs};
-        const int rc = p.ranges > 1 ? launch_grad_sweep<D, DRT, true>(d, p, K, V, dY, a, st) : launch_grad_sweep<D, DRT, false>(d, p, K, V, dY, a, st);
+        int rc = FLARE_ERR_UNSUPPORTED;
+        if (p.ranges == 1) rc = launch_grad_sweep<D, DRT, false>(d, p, K, V, dY, a, st);
+        else if constexpr (D == 16) rc = launch_grad_sweep<D, DRT, true>(d, p, K, V, dY, a, st);
         if (rc != FLARE_OK) return rc;
     }
     FLARE_REDUCE(bwd_dq_reduce_kernel, (long)d->H * d->M, d->B * 2 * p.splits, d->D, st, at(w.part), dQ, 2 * p.splits, d->B, (long)d->H * d->M, d->scale);

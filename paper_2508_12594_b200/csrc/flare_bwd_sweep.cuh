@@ -11,8 +11,8 @@
 //
 // Three kernels before (dZ with latents on the lanes; dK, dV and dd with tokens; dQ with latents) exponentiated every score three times and formed A and C
 // twice; here it is twice and once, and since dd is known when dS is formed, no first guess of it is needed (a pass over Y and dY) and nothing is put right
-// afterwards.  us per training step, before -> now: 16384 tokens, M = 32, D = 32, 8 heads 81 -> 67; 32 x 4096, M = 128, D = 32, 4 heads 289 -> 235; 131072
-// tokens, 8 heads, D = 32: M = 64 388 -> 306, 256 773 -> 657, 320 1014 -> 826; D = 16: M = 32 238 -> 229, 256 706 -> 624, 1024 2618 -> 2392; D = 8: M = 64 294 -> 262,
+// afterwards.  us per training step, before -> now: 16384 tokens, M = 32, D = 32, 8 heads 81 -> 65; 32 x 4096, M = 128, D = 32, 4 heads 289 -> 235; 131072
+// tokens, 8 heads, D = 32: M = 32 340 -> 233, 64 388 -> 298, 256 773 -> 657, 320 1014 -> 826; D = 16: M = 32 238 -> 215, 256 706 -> 624, 1024 2618 -> 2392; D = 8: M = 64 294 -> 262,
 // 1024 2525 -> 2345, 2048 5133 -> 4626; D = 4, 16 heads, M = 64 596 -> 503.  At D = 32 two ranges of latents, with float32 rows to read and write between
 // them, are no faster (M = 400 1312 : 1309, 512 1391 : 1414): more than 320 latents take the kernels of flare_bwd_tc.cuh, and so do heads 64 wide.
 //
@@ -782,8 +782,8 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             };
             // What says that the products of unit n + 1 are there says as well that a buffer of dS has been read: with two buffers that of unit n - 1,
             // whose sums come before those products; with three that of n - 2, and dQ of unit n - 1 may come behind them.
-            // (D = 32: only where a tile is one unit, us per step, 32 x 4096, M = 128 239 : 236; D = 16: wherever there are three, 131072, M = 256 620 : 645)
-            const bool late = bufs == 3 && (D == 16 || nu == 1);
+            // us per step, in order : late, 131072 tokens: D = 32, M = 32 233 : 262, 64 298 : 302, 32 x 4096, M = 128 236 : 239; D = 16, M = 64 270 : 262, 256 645 : 620.
+            const bool late = bufs == 3 && D == 16;
             bool ok = products(0);
             for (int n = 0; ok && n < units; ++n) {
                 if (n + 1 < units) {
@@ -992,13 +992,16 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         auto unit_wait = [&](uint32_t at, uint32_t parity, uint32_t code) { return D == 16 ? issue_wait(at, parity, abort_flag, code) : warp_wait(at, parity, abort_flag, code); };
         // The loop over the units has nothing else in it: with the rows in a branch of it, it carried some forty instructions of theirs (131072 tokens, M = 256, D =
         // 16 649 -> 622 us per step, 32 x 4096, M = 128 259 -> 239 with what follows dd in a warp of its own).
-        // Rows of a tile leave after the first unit of the next, when they have long been formed; with two sets of warps at once, the other set is at work.
+        // Rows of a tile leave after the first unit of the set's next, when they have long been formed; at D = 32 with two sets of warps at once: the other
+        // set is at work, and four tile stages are all there is room for (us per step at once : after the next unit, 131072 tokens: D = 32, M = 32 233 : 253, D = 16,
+        // M = 16 229 : 213, D = 8, M = 32 230 : 214).
+        const bool at_once = D == 32 && sets == 2;
         int n = set;                                            // unit of all
         float r_before = 0.f;
         bool ok = true;
         for (int i = set, k = 0; ok; i += sets, ++k) {          // one more turn writes the last tile's rows
             const bool more = i < nt;
-            bool pending = sets == 2 ? more : k > 0;
+            bool pending = at_once ? more : k > 0;
             if (!more && !pending) break;
             float2 nldp = make_float2(0.f, 0.f), rp = nldp, nddp = nldp, ndd2p = nldp;
             bool far = false;
@@ -1040,10 +1043,10 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     if (!ok) break;
                 }
                 if (pending) {
-                    int done = sets == 2 ? k : k - 1;
+                    int done = at_once ? k : k - 1;
                     asm volatile("" : "+r"(done));              // (nothing of what follows is worked out ahead)
                     const int before = set + done * sets;
-                    if (!(ok = write_rows(done, sets == 2 ? r : r_before))) break;
+                    if (!(ok = write_rows(done, at_once ? r : r_before))) break;
                     if ((before + 1) % kSwFlush == 0 || before + 1 == nt) {
                         const int window = before / kSwFlush;   // (after the window before, which the other set of warps may be about)
                         if (window > 0 && !(ok = warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdTok | 15))) break;
