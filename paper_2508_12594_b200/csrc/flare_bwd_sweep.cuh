@@ -29,8 +29,9 @@ namespace flare {
 constexpr int kSwThreads = 640, kSwFirstMathWarp = 4, kSwUnit = 64, kSwGroups = kSwUnit / 16;
 constexpr uint32_t kSwHalf = kTile * kSwUnit * 2, kSwBuf = 2 * kSwHalf;     // bytes of a unit's hi (lo) halves, of both
 constexpr int kSwRing = 4, kSwMaxStages = 6;
-// Tiles whose sums over tokens tensor memory adds up: it truncates, an error that grows with the number of sums; then they are added to the float32 partial results.
-constexpr int kSwFlush = 64;
+// Tiles whose sums over tokens (eight of 16 tokens each) tensor memory adds up: it truncates, an error that grows with the number of sums; then they are added to the float32
+// partial results, which stops the pipeline for some 4000 cycles.  A power of two, by units of a tile.
+__host__ __device__ constexpr int sweep_flush_tiles(int nu) { return nu <= 2 ? 16 : nu <= 4 ? 32 : 64; }
 
 // Descriptors of a unit's weights in shared memory: rows of 128 bytes (64 latents of a token), swizzled.
 constexpr uint32_t kSwDescHi = ptx::desc_hi(1024, 2);
@@ -167,7 +168,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     float *ring = reinterpret_cast<float *>(smem + SM::ring_off(stages, M));
     float4 *dds = reinterpret_cast<float4 *>(smem + SM::dds_off(stages, M));
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + SM::bar_off(stages, M));
-    enum { T_FULL = 0, T_EMPTY = T_FULL + kSwMaxStages, S_FULL = T_EMPTY + kSwMaxStages, S_READ = S_FULL + 2, P_FULL = S_READ + 2, C_FULL = P_FULL + 2,
+    enum { T_FULL = 0, T_EMPTY = T_FULL + kSwMaxStages, S_FULL = T_EMPTY + kSwMaxStages, S_READ = S_FULL + 2, P_FULL = S_READ + 2, C_FULL = P_FULL + 4,
            C_EMPTY = C_FULL + RING, DD_FULL = C_EMPTY + RING, DD_EMPTY = DD_FULL + 2, FL_FULL = DD_EMPTY + 2, FL_DONE, NBARS };
     static_assert(NBARS * 8 + 8 <= 512, "barrier area too small");
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + NBARS);
@@ -181,7 +182,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S or A
     const int sets = M <= 32 ? 2 : 1, cps = sets == 2 ? 2 : kSwGroups;                 // sets of warps that take the tiles in turn, column groups of each
     const int off = DRT ? narrow_offset(h, DR) : 0;
-    const int units = nu * nt;
+    const int units = nu * nt, flush = sweep_flush_tiles(nu);
     // (opaque: an address that can be formed again from the kernel's arguments is, at every use, by a dozen instructions)
     uint32_t bars0 = ptx::smem_u32(bars);
     ptx::opaque(bars0);
@@ -336,7 +337,8 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     ptx::tc_fence_after();
                     if (!tiles(n + 2)) break;
                 }
-                if (!issue_wait(bar(P_FULL + (n & 1)), (n >> 1) & 1, abort_flag, kErrBwdDz | 6)) break;
+                // (four barriers in turn: scores two units on are there before all warps are done with this one, and one that is may arrive for that unit first)
+                if (!issue_wait(bar(P_FULL + (n & 3)), (n >> 2) & 1, abort_flag, kErrBwdDz | 6)) break;
                 if (o_u == 0 && o_tile == 0 && window > 0 && !issue_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdDz | 7)) break;
                 ptx::tc_fence_after();
                 // dZ += W^T dY: 16 tokens per step
@@ -350,7 +352,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                     o_u = 0;
                     ptx::mma_commit_by(lead, bar(T_EMPTY + o_stage));
                     if (++o_stage == stages) o_stage = 0;
-                    if (++o_tile == kSwFlush || n + 1 == units) {
+                    if (++o_tile == flush || n + 1 == units) {
                         ptx::mma_commit_by(lead, bar(FL_FULL));
                         o_tile = 0;
                         ++window;
@@ -415,7 +417,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
-                ptx::mbar_arrive_if(read + 8 * (P_FULL - S_READ), lead);
+                ptx::mbar_arrive_if(bar(P_FULL + (n & 3)), lead);
                 w += (uint32_t)sets * kSwBuf;
                 if (w >= w_end) w -= SM::kBufs * kSwBuf;
             }
@@ -423,8 +425,8 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             dds[((i & 1) * kSwGroups + mine) * kTile + row] = sums.get();
             __syncwarp();
             ptx::mbar_arrive_if(bar(DD_FULL + (i & 1)), lead);
-            if ((i + 1) % kSwFlush == 0 || i + 1 == nt) {
-                const int window = i / kSwFlush;                // (after the window before, which the other set of warps may be about)
+            if (((i + 1) & (flush - 1)) == 0 || i + 1 == nt) {
+                const int window = i / flush;                // (after the window before, which the other set of warps may be about)
                 if (window > 0 && !warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdDz | 11)) break;
                 if (!warp_wait(bar(FL_FULL), window & 1, abort_flag, kErrBwdDz | 10)) break;
                 ptx::tc_fence_after();
@@ -527,7 +529,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S, A or C
     const int log_accs = SM::log2_accs(M);
     const int off = DRT ? narrow_offset(h, DR) : 0;
-    const int units = nu * nt;
+    const int units = nu * nt, flush = sweep_flush_tiles(nu);
     // (opaque: an address that can be formed again from the kernel's arguments is, at every use, by a dozen instructions)
     uint32_t bars0 = ptx::smem_u32(bars);
     ptx::opaque(bars0);
@@ -772,7 +774,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     q_u = 0;
                     ptx::mma_commit_by(lead, bar(T_DONE + q_stage));
                     if (++q_stage == stages) q_stage = 0;
-                    if (++q_tile == kSwFlush || q_n == units) {
+                    if (++q_tile == flush || q_n == units) {
                         ptx::mma_commit_by(lead, bar(FL_FULL));
                         q_tile = 0;
                         ++window;
@@ -1047,8 +1049,8 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     asm volatile("" : "+r"(done));              // (nothing of what follows is worked out ahead)
                     const int before = set + done * sets;
                     if (!(ok = write_rows(done, at_once ? r : r_before))) break;
-                    if ((before + 1) % kSwFlush == 0 || before + 1 == nt) {
-                        const int window = before / kSwFlush;   // (after the window before, which the other set of warps may be about)
+                    if (((before + 1) & (flush - 1)) == 0 || before + 1 == nt) {
+                        const int window = before / flush;   // (after the window before, which the other set of warps may be about)
                         if (window > 0 && !(ok = warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdTok | 15))) break;
                         if (!(ok = warp_wait(bar(FL_FULL), window & 1, abort_flag, kErrBwdTok | 14))) break;
                         ptx::tc_fence_after();
