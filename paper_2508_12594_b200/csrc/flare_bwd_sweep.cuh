@@ -11,7 +11,7 @@
 //
 // Three kernels before (dZ with latents on the lanes; dK, dV and dd with tokens; dQ with latents) exponentiated every score three times and formed A and C
 // twice; here it is twice and once, and since dd is known when dS is formed, no first guess of it is needed (a pass over Y and dY) and nothing is put right
-// afterwards.  us per training step, before -> now: 16384 tokens, M = 32, D = 32, 8 heads 81 -> 65; 32 x 4096, M = 128, D = 32, 4 heads 289 -> 235; 131072
+// afterwards.  us per training step, before -> now: 16384 tokens, M = 32, D = 32, 8 heads 81 -> 65; 32 x 4096, M = 128, D = 32, 4 heads 289 -> 245; 131072
 // tokens, 8 heads, D = 32: M = 32 340 -> 233, 64 388 -> 298, 256 773 -> 657, 320 1014 -> 826; D = 16: M = 32 238 -> 215, 256 706 -> 624, 1024 2618 -> 2392; D = 8: M = 64 294 -> 262,
 // 1024 2525 -> 2345, 2048 5133 -> 4626; D = 4, 16 heads, M = 64 596 -> 503.  At D = 32 two ranges of latents, with float32 rows to read and write between
 // them, are no faster (M = 400 1312 : 1309, 512 1391 : 1414): more than 320 latents take the kernels of flare_bwd_tc.cuh, and so do heads 64 wide.
