@@ -29,42 +29,54 @@ namespace flare {
 constexpr int kSwThreads = 640, kSwFirstMathWarp = 4, kSwUnit = 64, kSwGroups = kSwUnit / 16;
 constexpr uint32_t kSwHalf = kTile * kSwUnit * 2, kSwBuf = 2 * kSwHalf;     // bytes of a unit's hi (lo) halves, of both
 constexpr int kSwRing = 4, kSwMaxStages = 6;
-// Tiles whose sums over tokens (eight of 16 tokens each) tensor memory adds up: it truncates, an error that grows with the number of sums; then they are added to the float32
-// partial results, which stops the pipeline for some 4000 cycles.  A power of two, by units of a tile.
-__host__ __device__ constexpr int sweep_flush_tiles(int nu) { return nu <= 2 ? 16 : nu <= 4 ? 32 : 64; }
+// Sums over tokens that take a CTA's tiles in turn, up to four where tensor memory has the columns (as a logarithm; `each`: columns of one).  The tensor core
+// truncates: n parts in a row lose n 2^-24 / 3 of their sum on average, all in one direction.  Distance of dQ from float64, of its norm, one sum : in turn : the
+// three kernels before, 65536 tokens, 8 heads: D = 32, M = 32 5.8e-6 : 4.8e-6 : 5.4e-6, M = 64 5.7e-6 : 4.8e-6 : 5.3e-6; D = 16, M = 32 5.6e-6 : 4.6e-6 : 4.9e-6, M = 128 9.1e-6 : 8.2e-6 : 8.5e-6.
+__host__ __device__ constexpr int sweep_log2_sums(int columns, int each) { return columns >= 4 * each ? 2 : columns >= 2 * each ? 1 : 0; }
+// Tiles (eight parts of 16 tokens each) after which these sums are added to the float32 partial results, which stops the pipeline for some 4000 cycles: a power
+// of two, by units of a tile.  64 to 128 parts in a row up to two units; with more units, whose tiles take longer and are fewer to a CTA at the same time, up
+// to 256 and 512, which leave dQ no further from float64 than the three kernels before (100000 tokens, M = 1024, D = 16 8.9e-6, before 10.7e-6).
+__host__ __device__ constexpr int sweep_flush_tiles(int nu, int sums) { return nu <= 2 && sums < 4 ? 16 : nu <= 4 ? 32 : 64; }
 
 // Descriptors of a unit's weights in shared memory: rows of 128 bytes (64 latents of a token), swizzled.
 constexpr uint32_t kSwDescHi = ptx::desc_hi(1024, 2);
 constexpr uint32_t kSwDescMn = ptx::desc_lo(0, kSwHalf), kSwDescK = ptx::desc_lo(0, 16);   // transposed: the lo halves follow as rows 64 on; as they lie
 
-// The sums over tokens that a CTA has in tensor memory (columns base + u D of unit u; lanes 0-63 hi, 64-127 lo) to partial results 2 part and
-// 2 part + 1, or added to them.  By the warps that worked on the last unit: `mine` of `cps` column groups.
+// The sums over tokens that a CTA has in tensor memory (`sums` of them, columns base + (s nu + u) D of unit u; lanes 0-63 hi, 64-127 lo) to partial results 2 part
+// and 2 part + 1, or added to them.  By the warps that worked on the last unit: `mine` of `cps` column groups.
 template <int D, int DR>
-__device__ __forceinline__ void sweep_flush(uint32_t base, float *part, size_t rows, int cta, size_t row0, int M, int nu, int mine, int cps, int row, int off, bool add) {
+__device__ __forceinline__ void sweep_flush(uint32_t base, float *part, size_t rows, int cta, size_t row0, int M, int nu, int sums, int mine, int cps, int row, int off, bool add) {
     float *dst0 = part + ((size_t)(2 * cta + (row >> 6)) * rows + row0) * DR;
-    for (int u = mine; u < nu; u += cps) {
-        const int m = u * kSwUnit + (row & 63);
+    constexpr int PIECES = DR <= 8 ? 1 : DR / 8;                // of eight columns, in turn to the warps that share the tokens
+    for (int p = mine; p < nu * PIECES; p += cps) {
+        const int u = p / PIECES, c0 = p % PIECES * 8, m = u * kSwUnit + (row & 63);
+        uint32_t x[8];
+        ptx::tmem_ld8(base + u * D + c0, x);
+        ptx::tmem_wait_ld();
 #pragma unroll
-        for (int c0 = 0; c0 < (DR < 8 ? 8 : DR); c0 += 8) {
-            uint32_t x[8];
-            ptx::tmem_ld8(base + u * D + c0, x);
+        for (int s = 1; s < 4; ++s) {
+            if (s >= sums) break;
+            uint32_t y[8];
+            ptx::tmem_ld8(base + (s * nu + u) * D + c0, y);
             ptx::tmem_wait_ld();
-            float4 *dst = reinterpret_cast<float4 *>(dst0 + (size_t)m * DR + c0);
-            if (m < M) {
 #pragma unroll
-                for (int c = 0; c < (DR == 4 ? 1 : 2); ++c) {
-                    float4 v;
-                    if (DR == 4 && off != 0) v = make_float4(__uint_as_float(x[4]), __uint_as_float(x[5]), __uint_as_float(x[6]), __uint_as_float(x[7]));
-                    else v = make_float4(__uint_as_float(x[4 * c]), __uint_as_float(x[4 * c + 1]), __uint_as_float(x[4 * c + 2]), __uint_as_float(x[4 * c + 3]));
-                    if (add) {
-                        const float4 o = dst[c];
-                        v = make_float4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
-                    }
-                    dst[c] = v;
-                }
-            }
-            __syncwarp();
+            for (int c = 0; c < 8; ++c) x[c] = __float_as_uint(__uint_as_float(x[c]) + __uint_as_float(y[c]));
         }
+        float4 *dst = reinterpret_cast<float4 *>(dst0 + (size_t)m * DR + c0);
+        if (m < M) {
+#pragma unroll
+            for (int c = 0; c < (DR == 4 ? 1 : 2); ++c) {
+                float4 v;
+                if (DR == 4 && off != 0) v = make_float4(__uint_as_float(x[4]), __uint_as_float(x[5]), __uint_as_float(x[6]), __uint_as_float(x[7]));
+                else v = make_float4(__uint_as_float(x[4 * c]), __uint_as_float(x[4 * c + 1]), __uint_as_float(x[4 * c + 2]), __uint_as_float(x[4 * c + 3]));
+                if (add) {
+                    const float4 o = dst[c];
+                    v = make_float4(v.x + o.x, v.y + o.y, v.z + o.z, v.w + o.w);
+                }
+                dst[c] = v;
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -139,6 +151,11 @@ struct BwdDzSmem {
     using G = TileGeom<D>;
     enum { QR = 0, ZH = 1, ZL = 2 };                            // latent operands: Q, Z hi, lo
     static constexpr int kBufs = 3;                             // of weights
+    // sums over tokens beside S and A twice
+    __host__ __device__ static int log2_sums(int M) {
+        const int ucols = (M + 31) / 32 * 32 < kSwUnit ? (M + 31) / 32 * 32 : kSwUnit;
+        return sweep_log2_sums(512 - 4 * ucols, (M + kSwUnit - 1) / kSwUnit * D);
+    }
     static constexpr size_t tile_off = (size_t)kBufs * kSwBuf;
     __host__ __device__ static size_t lat_off(int stages, int M, int which) { return tile_off + (size_t)stages * 2 * G::TILE_BYTES + (size_t)which * M * G::RB; }
     __host__ __device__ static size_t ring_off(int stages, int M) { return lat_off(stages, M, 3); }         // [ring][token] -lse_dec
@@ -182,7 +199,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S or A
     const int sets = M <= 32 ? 2 : 1, cps = sets == 2 ? 2 : kSwGroups;                 // sets of warps that take the tiles in turn, column groups of each
     const int off = DRT ? narrow_offset(h, DR) : 0;
-    const int units = nu * nt, flush = sweep_flush_tiles(nu);
+    const int units = nu * nt, sums_in_turn = 1 << SM::log2_sums(M), flush = sweep_flush_tiles(nu, sums_in_turn);
     // (opaque: an address that can be formed again from the kernel's arguments is, at every use, by a dozen instructions)
     uint32_t bars0 = ptx::smem_u32(bars);
     ptx::opaque(bars0);
@@ -344,9 +361,10 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 // dZ += W^T dY: 16 tokens per step
                 constexpr uint32_t idescO = ptx::instr_desc_bf16(128, D, 1, 1);
                 uint32_t wd = w0 + (uint32_t)o_buf * (kSwBuf >> 4), gd = td0 + MN + (uint32_t)o_stage * 2 * TILE + TILE;
+                const uint32_t to = acc0 + ((o_tile & (sums_in_turn - 1)) * nu + o_u) * D;
 #pragma unroll
                 for (int k = 0; k < kTile / 16; ++k)
-                    ptx::mma_ss_by(lead, acc0 + o_u * D, ptx::desc(wd + k * (2048 >> 4), kSwDescHi), ptx::desc(gd + k * STEP16, HI), idescO, (o_tile > 0 || k > 0) ? 1u : 0u);
+                    ptx::mma_ss_by(lead, to, ptx::desc(wd + k * (2048 >> 4), kSwDescHi), ptx::desc(gd + k * STEP16, HI), idescO, (o_tile >= sums_in_turn || k > 0) ? 1u : 0u);
                 if (++o_buf == SM::kBufs) o_buf = 0;
                 if (++o_u == nu) {
                     o_u = 0;
@@ -430,7 +448,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (window > 0 && !warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdDz | 11)) break;
                 if (!warp_wait(bar(FL_FULL), window & 1, abort_flag, kErrBwdDz | 10)) break;
                 ptx::tc_fence_after();
-                sweep_flush<D, DR>(acc0 - tm + gcol, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, mine, cps, row, off, window > 0);
+                sweep_flush<D, DR>(acc0 - tm + gcol, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, min(sums_in_turn, i + 1 - window * flush), mine, cps, row, off, window > 0);
                 ptx::tc_fence_before();
                 __syncwarp();
                 ptx::mbar_arrive_if(bar(FL_DONE), lead);
@@ -483,6 +501,11 @@ struct BwdGradSmem {
         const int ucols = (M + 31) / 32 * 32 < kSwUnit ? (M + 31) / 32 * 32 : kSwUnit, fit = (512 - 4 * ucols - (M + kSwUnit - 1) / kSwUnit * D) / kAccStride;
         return fit >= 4 ? 2 : fit >= 2 ? 1 : fit >= 1 ? 0 : -1;
     }
+    // sums over tokens in what is left
+    __host__ __device__ static int log2_sums(int M) {
+        const int ucols = (M + 31) / 32 * 32 < kSwUnit ? (M + 31) / 32 * 32 : kSwUnit;
+        return sweep_log2_sums(512 - 4 * ucols - (kAccStride << log2_accs(M)), (M + kSwUnit - 1) / kSwUnit * D);
+    }
     __host__ __device__ static size_t tile_off(int bufs) { return (size_t)bufs * kSwBuf; }
     __host__ __device__ static size_t lat_off(int bufs, int stages, int M, int which) { return tile_off(bufs) + (size_t)stages * 3 * G::TILE_BYTES + (size_t)which * M * G::RB; }
     __host__ __device__ static size_t cst_off(int bufs, int stages, int M) { return lat_off(bufs, stages, M, 5); }     // per latent the exponent's addend and -c de
@@ -529,7 +552,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S, A or C
     const int log_accs = SM::log2_accs(M);
     const int off = DRT ? narrow_offset(h, DR) : 0;
-    const int units = nu * nt, flush = sweep_flush_tiles(nu);
+    const int units = nu * nt, sums_in_turn = 1 << SM::log2_sums(M), flush = sweep_flush_tiles(nu, sums_in_turn);
     // (opaque: an address that can be formed again from the kernel's arguments is, at every use, by a dozen instructions)
     uint32_t bars0 = ptx::smem_u32(bars);
     ptx::opaque(bars0);
@@ -765,9 +788,10 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     ptx::tc_fence_after();
                 }
                 uint32_t wd = w0 + kSwDescMn + (uint32_t)q_buf * (kSwBuf >> 4), kd = td0 + MN + (uint32_t)q_stage * 3 * TILE;
+                const uint32_t to = tm + dq0 + ((q_tile & (sums_in_turn - 1)) * nu + q_u) * D;
 #pragma unroll
                 for (int k = 0; k < kTile / 16; ++k)
-                    ptx::mma_ss_by(lead, tm + dq0 + q_u * D, ptx::desc(wd + k * (2048 >> 4), kSwDescHi), ptx::desc(kd + k * STEP16, HI), idesc, (q_tile > 0 || k > 0) ? 1u : 0u);
+                    ptx::mma_ss_by(lead, to, ptx::desc(wd + k * (2048 >> 4), kSwDescHi), ptx::desc(kd + k * STEP16, HI), idesc, (q_tile >= sums_in_turn || k > 0) ? 1u : 0u);
                 if (++q_buf == bufs) q_buf = 0;
                 ++q_n;
                 if (++q_u == nu) {
@@ -1054,7 +1078,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                         if (window > 0 && !(ok = warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdTok | 15))) break;
                         if (!(ok = warp_wait(bar(FL_FULL), window & 1, abort_flag, kErrBwdTok | 14))) break;
                         ptx::tc_fence_after();
-                        sweep_flush<D, DR>(gcol + dq0, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, mine, cps, row, off, window > 0);
+                        sweep_flush<D, DR>(gcol + dq0, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, min(sums_in_turn, before + 1 - window * flush), mine, cps, row, off, window > 0);
                         ptx::tc_fence_before();
                         __syncwarp();
                         ptx::mbar_arrive_if(bar(FL_DONE), lead);

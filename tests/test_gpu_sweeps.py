@@ -2,9 +2,12 @@
 around the units of 64 and the most of one launch, ranges of unequal size, more tiles to a CTA than tensor memory adds up in a row (with one and with two
 sets of warps), rows that leave by a tile's copy at the end of a batch item, narrow heads."""
 import pytest
+import torch
 
-from paper_2508_12594_b200 import workloads
+from paper_2508_12594_b200 import flare, workloads
+from tests._util import dev
 from tests.test_gpu_backward import assert_grads_close, gpu_backward, oracle_backward
+from tests.test_gpu_fullsize import _float64_z_and_dq
 
 pytestmark = pytest.mark.gpu
 
@@ -31,3 +34,14 @@ CASES = [  # B, H, N, M, D, masked_fraction
 def test_backward_in_two_sweeps(oracle, B, H, N, M, D, masked):
     inp = workloads.make_random(B, H, N, M, D, dtype="bf16", seed=N + M, masked_fraction=masked, with_dy=True, k_std=0.8)
     assert_grads_close(gpu_backward(inp), oracle_backward(oracle, inp), "bf16", f"{B}x{H}x{N}x{M}x{D}")
+
+
+@pytest.mark.parametrize("M,D", [(32, 32), (64, 32), (32, 16)])
+def test_sums_over_tokens_are_made_of_few_parts(M, D):
+    """The halves of the factors leave 2^-18 of dQ's norm.  The tensor core truncates its sums: a part added to one of uniform size loses 2^-24 / 3 of the whole on
+    average.  A CTA has 14 tiles of eight parts, shared out to four sums (dQ at D = 32, M = 64: two): some 32 parts, in dZ and again in dQ.  (One sum of all: 5.5e-6 to 5.9e-6.)"""
+    inp = workloads.make_random(1, 8, 65536, M, D, dtype="bf16", seed=65536 + M, with_dy=True, k_std=D ** -0.5)
+    Q, K, V, dY = dev(inp.Q), dev(inp.K), dev(inp.V), dev(inp.dY)
+    _, dQ, _, _ = flare.forward_backward(Q, K, V, dY, check=True)
+    want = torch.stack([_float64_z_and_dq(Q[h], K[0, :, h], V[0, :, h], dY[0, :, h])[1] for h in range(8)])
+    assert (dQ - want).norm() <= (2.0 ** -18 + 2 * 32 * 2.0 ** -24 / 3) * want.norm()
