@@ -159,15 +159,21 @@ int flare_forward(const flare_desc_t *desc, const void *Q_lat, const void *K, co
  *     dQ_lat = scale * sum_b dS K;  dK = scale * dS^T Q_lat.
  * Z, lse_enc, lse_dec are the ones flare_forward wrote; Y is its output (part of the saved set).  dY_n.Y_n is formed
  * from float32 quantities, sum_m W_dec[n,m] (dY_n.Z_m), which is markedly more accurate than the rounded Y where the
- * latent rows a token mixes are nearly equal; on the tensor cores the rounded Y gives a first guess of it, no more (any
- * other contents change the last bits of dK and dQ_lat, not what they are sums of).
- * bfloat16 inputs run all three passes (dZ; dK, dV; dQ_lat) on the tensor cores, with
- * every rounded factor of a cancelling sum carried as two bfloat16 halves (for dQ_lat at D = 64 as three parts, all 24
- * bits of a float32); float32 inputs run on the CUDA cores.
- * dQ_lat, dK, dV are overwritten.  Workspace: flare_workspace_bytes(desc, FLARE_OP_BACKWARD) bytes holding dZ,
- * per-split partial sums of dZ and dQ_lat, one float per (b, n, h) (bfloat16: two, and a few rows of D per head), and,
- * beyond 1024 bfloat16 latents (512 at D = 32, 192 at D = 64), three float32 rows of D and one more float per (b, n, h):
- * the sums over ranges of latents; nothing of size N x M.
+ * latent rows a token mixes are nearly equal; where the tensor-core kernels read Y at all (D = 64, and D = 32 with more than
+ * 320 latents) it is a first guess of that, no more (any other contents change the last bits of dK and dQ_lat, not what they
+ * are sums of).
+ * bfloat16 inputs run on the tensor cores, with every rounded factor of a cancelling sum carried as two bfloat16 halves (for
+ * dQ_lat at D = 64 as three parts, all 24 bits of a float32): D <= 16, and D = 32 with up to 320 latents, in two sweeps over
+ * the tokens (dZ and dY_n.Y_n; dK, dV and dQ_lat), wider heads and more latents in three passes (dZ; dK, dV; dQ_lat).
+ * float32 and float16 inputs run on the CUDA cores.
+ * dQ_lat, dK, dV are overwritten.  Workspace: flare_workspace_bytes(desc, FLARE_OP_BACKWARD) bytes, nothing of size N x M:
+ *   - dZ (and a float per latent);
+ *   - per-split partial sums of dZ and dQ_lat, in the two sweeps two of each per split;
+ *   - one float per (b, n, h), bfloat16 two, and a few rows of D per head;
+ *   - where one launch does not take all bfloat16 latents, what the launches leave to one another.  Two sweeps, more than 768
+ *     latents: two float32 rows of D per (b, n, h), for so many tokens at a time, in whole tiles of 128, that these rows take
+ *     no more than 128 MB (or, should that be more, a tile per thread block).  Three passes, more than 512 latents (192 at
+ *     D = 64): three float32 rows of D and one more float per (b, n, h).
  */
 int flare_backward(const flare_desc_t *desc, const void *Q_lat, const void *K, const void *V,
                    const uint8_t *key_mask, const void *Y, const void *dY, const float *Z, const float *lse_enc,

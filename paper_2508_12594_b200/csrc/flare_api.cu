@@ -69,9 +69,9 @@ int launches_for(const flare_desc_t *d, int op) {
         case FLARE_OP_DECODE: return 1 + dec;                   // header (given a workspace), decode
         case FLARE_OP_FORWARD: return small_forward_cluster(d) ? 1 : enc + dec;
         case FLARE_OP_BACKWARD: {
-            if (use_sweeps(d)) {                                // header; the two sweeps, each over ranges of latents, and their reductions
+            if (use_sweeps(d)) {                                // header; the two sweeps, each over ranges of latents and chunks of tokens, and their reductions
                 const int sms = device_info().sms;
-                return 1 + dz_sweep_plan(d, sms).ranges + 1 + grad_sweep_plan(d, sms).ranges + 1;
+                return 1 + sweep_launches(d, dz_sweep_plan(d, sms)) + 1 + sweep_launches(d, grad_sweep_plan(d, sms)) + 1;
             }
             const int tok = token_in_ranges(d) ? (d->M + token_range(d) - 1) / token_range(d) : 1;   // (the CUDA-core kernel knows no ranges)
             return 1 + 2 + tok + 2;                             // header; dZ, its reduction; token kernel(s); dQ, its reduction

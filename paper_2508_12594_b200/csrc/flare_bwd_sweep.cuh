@@ -141,9 +141,10 @@ struct BwdDzArgs {
     int B, H, N, M;            // M: latents this launch works on (all of them, or a range)
     int mtot, m0;              // latents per head in memory, and the first one of this launch's range
     int first, last;           // range of latents (without ranges both)
-    float4 *sums;              // [B,H,N]: RowSums of the earlier ranges
+    float4 *sums;              // [B,H][tile of this launch][token of the tile]: RowSums of the earlier ranges
     float sl2;                 // scale * log2(e)
-    int tiles, stages;
+    int tiles, stages;         // tiles of tokens this launch works on
+    int t0;                    // the first of them (without ranges 0)
 };
 
 template <int D>
@@ -195,6 +196,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int h = blockIdx.y, b = blockIdx.z;
     const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
+    auto tile_at = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x + (kRanges ? a.t0 : 0); };   // the i-th of them
     const int nu = (M + UNIT - 1) / UNIT, wlast = M - (nu - 1) * UNIT;                 // latent units of a tile; columns of the last
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S or A
     const int sets = M <= 32 ? 2 : 1, cps = sets == 2 ? 2 : kSwGroups;                 // sets of warps that take the tiles in turn, column groups of each
@@ -242,7 +244,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (warp == 0) {
         if (ptx::elect_one()) {
             for (int i = 0; i < nt; ++i) {
-                const int s = i % stages, t = blockIdx.x + i * gridDim.x;
+                const int s = i % stages, t = tile_at(i);
                 if (!ptx::mbar_wait(bar(T_EMPTY + s), ((i / stages) & 1) ^ 1, abort_flag, kErrBwdDz | 1)) break;
                 ptx::mbar_arrive_expect_tx(bar(T_FULL + s), 2 * G::TILE_BYTES);
                 uint8_t *dst = tiles_s + (size_t)s * 2 * G::TILE_BYTES;
@@ -257,7 +259,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             float *at = ring + (i % RING) * kTile;
 #pragma unroll
             for (int e = 0; e < kTile / 32; ++e) {
-                const int r = e * 32 + lane, n = min((int)(blockIdx.x + i * gridDim.x) * kTile + r, a.N - 1);
+                const int r = e * 32 + lane, n = min(tile_at(i) * kTile + r, a.N - 1);
                 ptx::copy_async4(ptx::smem_u32(at + r), a.lse_dec + ((size_t)b * a.N + n) * a.H + h);
             }
         };
@@ -271,7 +273,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             float *at = ring + (i % RING) * kTile;
 #pragma unroll
             for (int e = 0; e < kTile / 32; ++e) {
-                const int r = e * 32 + lane, n = (int)(blockIdx.x + i * gridDim.x) * kTile + r;
+                const int r = e * 32 + lane, n = tile_at(i) * kTile + r;
                 at[r] = n < a.N ? -at[r] * kBwdLog2e : -INFINITY;
             }
             __syncwarp();
@@ -300,16 +302,17 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
             const size_t plane = (size_t)a.B * a.H * a.N;
 #pragma unroll
             for (int e = 0; e < kTile / 32; ++e) {
-                const int n = (int)(blockIdx.x + i * gridDim.x) * kTile + e * 32 + lane;
+                const int n = tile_at(i) * kTile + e * 32 + lane;
                 if (n >= a.N) continue;
                 const size_t at = bh * a.N + n;
-                if (kRanges && !a.first) all[e].join(a.sums[at]);
+                const size_t so_far = ((bh * a.tiles + (tile_at(i) - (kRanges ? a.t0 : 0))) * kTile) + e * 32 + lane;
+                if (kRanges && !a.first) all[e].join(a.sums[so_far]);
                 if (!kRanges || a.last) {
                     const float2 d = all[e].mean();
                     a.dd[at] = d.x;
                     a.dd[plane + at] = d.y;
                 } else {
-                    a.sums[at] = all[e].get();
+                    a.sums[so_far] = all[e].get();
                 }
             }
         }
@@ -448,7 +451,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (window > 0 && !warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdDz | 11)) break;
                 if (!warp_wait(bar(FL_FULL), window & 1, abort_flag, kErrBwdDz | 10)) break;
                 ptx::tc_fence_after();
-                sweep_flush<D, DR>(acc0 - tm + gcol, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, min(sums_in_turn, i + 1 - window * flush), mine, cps, row, off, window > 0);
+                sweep_flush<D, DR>(acc0 - tm + gcol, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, min(sums_in_turn, i + 1 - window * flush), mine, cps, row, off, window > 0 || (kRanges && a.t0 > 0));
                 ptx::tc_fence_before();
                 __syncwarp();
                 ptx::mbar_arrive_if(bar(FL_DONE), lead);
@@ -486,9 +489,9 @@ struct BwdGradArgs {
     float *part;               // [2 * CTAs per head][B*H*M][D] partial dQ rows (un-scaled)
     uint32_t *status;
     int B, H, N, M, mtot, m0, first, last;   // as in BwdDzArgs
-    float *kvacc;              // float32 dK and dV so far, where there are ranges; the last writes the rows.  [2][B,H][tile][D / 4][token of the tile][4]
+    float *kvacc;              // float32 dK and dV so far, where there are ranges; the last writes the rows.  [2][B,H][tile of this launch][D / 4][token of the tile][4]
     float scale, sl2;
-    int tiles, stages, bufs;
+    int tiles, stages, bufs, t0;   // as in BwdDzArgs
 };
 
 template <int D>
@@ -547,6 +550,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int h = blockIdx.y, b = blockIdx.z;
     const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    auto tile_at = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x + (kRanges ? a.t0 : 0); };   // the i-th of them
     const int nu = (M + UNIT - 1) / UNIT, wlast = M - (nu - 1) * UNIT;
     const int sets = M <= 32 ? 2 : 1, cps = sets == 2 ? 2 : kSwGroups;
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S, A or C
@@ -640,7 +644,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         if (ptx::elect_one()) {
             // Rows of dK and dV leave from where K and V of their tile were.
             auto store = [&](int i) -> bool {
-                const int s = i % stages, t = blockIdx.x + i * gridDim.x;
+                const int s = i % stages, t = tile_at(i);
                 if (!ptx::mbar_wait(bar(T_OUT + s), (i / stages) & 1, abort_flag, kErrBwdTok | 16)) return false;
                 if (DR >= 8 && (!kRanges || a.last)) {
                     const uint32_t src = ptx::smem_u32(tiles_s + (size_t)s * 3 * G::TILE_BYTES);
@@ -652,7 +656,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             };
             int i = 0;
             for (; i < nt; ++i) {
-                const int s = i % stages, t = blockIdx.x + i * gridDim.x;
+                const int s = i % stages, t = tile_at(i);
                 if (i >= stages) {
                     if (!store(i - stages)) break;
                     ptx::tma_store_wait<true>();
@@ -675,7 +679,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             float *at = ring + (i % RING) * 4 * kTile;
 #pragma unroll
             for (int e = 0; e < kTile / 32; ++e) {
-                const int r = e * 32 + lane, n = min((int)(blockIdx.x + i * gridDim.x) * kTile + r, a.N - 1);
+                const int r = e * 32 + lane, n = min(tile_at(i) * kTile + r, a.N - 1);
                 ptx::copy_async4(ptx::smem_u32(at + r), a.lse_dec + ((size_t)b * a.N + n) * a.H + h);
                 ptx::copy_async4(ptx::smem_u32(at + kTile + r), a.dd + bh * a.N + n);
                 ptx::copy_async4(ptx::smem_u32(at + 2 * kTile + r), a.dd + ((size_t)a.B * a.H + bh) * a.N + n);
@@ -693,7 +697,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             bool part[kTile / 32], far = unfolded != 0.f;
 #pragma unroll
             for (int e = 0; e < kTile / 32; ++e) {
-                const int r = e * 32 + lane, n = (int)(blockIdx.x + i * gridDim.x) * kTile + r;
+                const int r = e * 32 + lane, n = tile_at(i) * kTile + r;
                 const bool in = n < a.N;
                 ld[e] = in ? at[r] * kBwdLog2e : INFINITY;
                 part[e] = in && (a.key_mask == nullptr || a.key_mask[(size_t)b * a.N + n] != 0);
@@ -900,7 +904,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         uint32_t out_wrap = 0;
         auto write_rows = [&](int k, float r) -> bool {
             constexpr int COLS = DR >= 16 ? DR : 8, PIECES = COLS / 4, PW = DR == 4 ? 4 : 8;
-            const int i = set + k * sets, acc = i & ((1 << log_accs) - 1), s = out_stage, t = (int)blockIdx.x + i * (int)gridDim.x;
+            const int i = set + k * sets, acc = i & ((1 << log_accs) - 1), s = out_stage, t = tile_at(i);
             if (!warp_wait(bar(ACC_FULL + acc), (i >> log_accs) & 1, abort_flag, kErrBwdTok | 11)) return false;
             if (!warp_wait(bar(T_DONE + s), out_wrap, abort_flag, kErrBwdTok | 17)) return false;
             ptx::tc_fence_after();
@@ -919,7 +923,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     float4 *sums = nullptr;
                     float4 before[PW / 4];
                     if (kRanges) {
-                        sums = reinterpret_cast<float4 *>(a.kvacc) + ((((size_t)which * a.B * a.H + bh) * a.tiles + t) * (DR / 4) + c0 / 4) * kTile + row;
+                        sums = reinterpret_cast<float4 *>(a.kvacc) + ((((size_t)which * a.B * a.H + bh) * a.tiles + (t - a.t0)) * (DR / 4) + c0 / 4) * kTile + row;
                         if (!a.first) {
 #pragma unroll
                             for (int c = 0; c < PW / 4; ++c) before[c] = sums[c * kTile];
@@ -1078,7 +1082,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                         if (window > 0 && !(ok = warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdTok | 15))) break;
                         if (!(ok = warp_wait(bar(FL_FULL), window & 1, abort_flag, kErrBwdTok | 14))) break;
                         ptx::tc_fence_after();
-                        sweep_flush<D, DR>(gcol + dq0, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, min(sums_in_turn, before + 1 - window * flush), mine, cps, row, off, window > 0);
+                        sweep_flush<D, DR>(gcol + dq0, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, min(sums_in_turn, before + 1 - window * flush), mine, cps, row, off, window > 0 || (kRanges && a.t0 > 0));
                         ptx::tc_fence_before();
                         __syncwarp();
                         ptx::mbar_arrive_if(bar(FL_DONE), lead);

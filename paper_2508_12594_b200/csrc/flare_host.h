@@ -416,15 +416,34 @@ inline int token_range(const flare_desc_t *d) { return ((d->M + token_ranges(d) 
 inline bool use_sweeps(const flare_desc_t *d) { return use_tc(d) && (d->D <= 16 || (d->D == 32 && d->M <= 320)); }
 // Latents one launch of a sweep takes: what its operands leave of shared memory (beside two tile stages) and the sums over tokens of tensor memory; more are
 // worked off in ranges of about equal size, whole units of 64.
-struct SweepPlan { int range, ranges, splits, stages, bufs; };
+// Ranges leave float32 rows of dK and dV to one another (in the first sweep RowSums): a launch takes a chunk of each item's tokens, so that the rows stay within
+// kRangeBytes (or, if that is more, within a tile to a CTA), and all ranges go over one chunk before the next.  Without a bound they are 1074 MB at 1048576 tokens of
+// 8 heads, D = 16.  us per backward, no bound : 128 : 64 : 32 : 16 MB, 8 heads, M = 1024: 1048576 tokens, D = 8 12408 : 13080 : 13200 : 13450 : 13900, 524288, D = 16
+// 6394 : 6586 : 6791 : 7136 : 7724, 131072, D = 16 1681 : 1644 : 1745 : 1822 : 1972 (a chunk starts and ends as any launch does, and chunks give 144 CTAs to the 148 SMs
+// where one launch of 1048576 tokens gives two rounds of 148).
+constexpr size_t kRangeBytes = (size_t)128 << 20;
+struct SweepPlan { int range, ranges, chunk, splits, stages, bufs; };
+inline size_t range_tile_bytes(const flare_desc_t *d) {         // of one tile of every item
+    return sizeof(float) * kTile * (size_t)d->B * d->H * 2 * d->D;
+}
 inline SweepPlan sweep_ranges(const flare_desc_t *d, int sms) {
     const int most = d->D == 32 ? 320 : 768;
     SweepPlan p{};
     p.ranges = (d->M + most - 1) / most;
     p.range = p.ranges == 1 ? d->M : ((d->M + p.ranges - 1) / p.ranges + 63) / 64 * 64;
     p.ranges = (d->M + p.range - 1) / p.range;
-    p.splits = token_splits(d, (d->N + kTile - 1) / kTile, p.range, sms);
+    const int tiles = (d->N + kTile - 1) / kTile;
+    p.chunk = p.ranges == 1 ? tiles : (int)std::min<size_t>(tiles, std::max<size_t>(1, kRangeBytes / range_tile_bytes(d)));
+    p.splits = token_splits(d, p.chunk, p.range, sms);
+    if (p.chunk < tiles) {                                      // chunks of about equal size, each a whole number of tiles to a CTA
+        const int chunks = (tiles + p.chunk / p.splits * p.splits - 1) / (p.chunk / p.splits * p.splits);
+        p.chunk = ((tiles + chunks - 1) / chunks + p.splits - 1) / p.splits * p.splits;
+    }
     return p;
+}
+inline int sweep_launches(const flare_desc_t *d, const SweepPlan &p) {
+    const int tiles = (d->N + kTile - 1) / kTile;
+    return p.ranges * ((tiles + p.chunk - 1) / p.chunk);
 }
 inline SweepPlan dz_sweep_plan(const flare_desc_t *d, int sms) {
     SweepPlan p = sweep_ranges(d, sms);
@@ -459,10 +478,9 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
         off += align_up(sizeof(float) * (size_t)(1 + latent_blocks(d)) * d->B * d->H * d->D);
     }
     w.dd_other = w.kvacc = off;                                // over latent ranges: dd so far, and float32 sums of the rows
-    if (use_sweeps(d)) {
-        const size_t tokens = (size_t)d->B * d->N * d->H;
-        if (dz_sweep_plan(d, sms).ranges > 1) w.kvacc = off += align_up(sizeof(float4) * tokens);
-        if (grad_sweep_plan(d, sms).ranges > 1) off += align_up(sizeof(float) * 2 * (size_t)d->B * d->H * ((d->N + kTile - 1) / kTile) * kTile * d->D);
+    if (use_sweeps(d)) {                                       // (the two sweeps one after the other, in the same place: a row of either is at least a RowSums)
+        const SweepPlan p = grad_sweep_plan(d, sms);
+        if (p.ranges > 1) off += align_up(range_tile_bytes(d) * p.chunk);
     } else if (token_in_ranges(d)) {
         w.kvacc = off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
         off += align_up(sizeof(float) * 3 * (size_t)d->B * d->N * d->H * d->D);

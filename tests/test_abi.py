@@ -119,3 +119,12 @@ def test_scratch_at_head_width_64_is_that_of_the_exact_form(lib):
 def test_launch_count_of_a_backward(lib, M, D, dtype, kernels):
     """Header, dZ and its reduction, the token kernel (bfloat16: one per range of latents), dQ and its reduction."""
     assert flare.flare_launch_count(flare.FlareDesc(1, 2, 1000, M, D, dtype, 1.0), flare.OP_BACKWARD) == kernels
+
+
+@pytest.mark.parametrize("B,H,N,D", [(1, 8, 1048576, 8), (1, 8, 1048576, 16), (4, 16, 262144, 16), (32, 4, 65536, 16)])
+@pytest.mark.parametrize("M", [784, 1024, 2048])
+def test_ranges_of_latents_take_bounded_scratch(lib, B, H, N, M, D):
+    """Beyond the 768 latents of one launch a backward keeps float32 rows of dK and dV between its ranges of latents: at most 128 MB of them, whatever the number of
+    tokens.  (All else grows as the latents do, or less.)"""
+    need = lambda m: flare.flare_workspace_bytes(flare.FlareDesc(B, H, N, m, D, flare.DTYPE_BF16, 1.0), flare.OP_BACKWARD)
+    assert 0 < need(M) <= need(768) * M / 768 + (128 << 20)

@@ -1,11 +1,12 @@
 """The two sweeps over the tokens of the bfloat16 backward (heads up to 32 wide) where they can go wrong, against the CPU oracle (needs a B200): latents
 around the units of 64 and the most of one launch, ranges of unequal size, more tiles to a CTA than tensor memory adds up in a row (with one and with two
 sets of warps), rows that leave by a tile's copy at the end of a batch item, narrow heads."""
+import numpy as np
 import pytest
 import torch
 
 from paper_2508_12594_b200 import flare, workloads
-from tests._util import dev
+from tests._util import dev, to_np64
 from tests.test_gpu_backward import assert_grads_close, gpu_backward, oracle_backward
 from tests.test_gpu_fullsize import _float64_z_and_dq
 
@@ -45,3 +46,39 @@ def test_sums_over_tokens_are_made_of_few_parts(M, D):
     _, dQ, _, _ = flare.forward_backward(Q, K, V, dY, check=True)
     want = torch.stack([_float64_z_and_dq(Q[h], K[0, :, h], V[0, :, h], dY[0, :, h])[1] for h in range(8)])
     assert (dQ - want).norm() <= (2.0 ** -18 + 2 * 32 * 2.0 ** -24 / 3) * want.norm()
+
+
+def float64_gradients(Q, K, V, dY):
+    """dQ, dK, dV of one head in float64 by plain torch, on the device, a slice of tokens at a time."""
+    Q, step = Q.double(), 1 << 15
+    at = range(0, K.shape[0], step)
+    S = lambda a: K[a:a + step].double() @ Q.T
+    le = torch.logsumexp(torch.stack([torch.logsumexp(S(a), 0) for a in at]), 0)
+    Z = sum(torch.exp(S(a) - le).T @ V[a:a + step].double() for a in at)
+    dZ = sum(torch.softmax(S(a), 1).T @ dY[a:a + step].double() for a in at)
+    de, dQ, dK, dV = (dZ * Z).sum(1), torch.zeros_like(Q), [], []
+    for a in at:
+        k, v, g = (x[a:a + step].double() for x in (K, V, dY))
+        Wd, We, A = torch.softmax(S(a), 1), torch.exp(S(a) - le), g @ Z.T
+        dS = Wd * (A - (Wd * A).sum(1, keepdim=True)) + We * (v @ dZ.T - de)
+        dQ += dS.T @ k
+        dK.append(dS @ Q)
+        dV.append(We @ dZ)
+    return dQ, torch.cat(dK), torch.cat(dV)
+
+
+@pytest.mark.parametrize("B,H,N,M,D", [(1, 8, 150001, 784, 16), (2, 8, 140000, 1040, 8), (1, 32, 40000, 784, 16)])
+def test_chunks_of_tokens_between_ranges_of_latents(B, H, N, M, D):
+    """More tokens than the rows that the ranges leave to one another have room for: several launches per range, each a chunk of the tokens.
+    dQ: 2^-18 from the halves of its factors, and at most 512 parts in a row, in dZ and again in dQ (see above)."""
+    inp = workloads.make_random(B, H, N, M, D, dtype="bf16", seed=N + M, with_dy=True, k_std=D ** -0.5)
+    Q, K, V, dY = dev(inp.Q), dev(inp.K), dev(inp.V), dev(inp.dY)
+    desc = flare.make_desc(Q, K)
+    assert flare.flare_launch_count(desc, flare.OP_BACKWARD) > 3 + 2 * 2
+    _, dQ, dK, dV = flare.forward_backward(Q, K, V, dY, check=True)
+    for h in (0, H - 1):
+        each = [float64_gradients(Q[h], K[b, :, h], V[b, :, h], dY[b, :, h]) for b in range(B)]
+        got = dict(dQ=to_np64(dQ[h]), dK=to_np64(dK[:, :, h]), dV=to_np64(dV[:, :, h]))
+        want = dict(dQ=to_np64(sum(x[0] for x in each)), dK=to_np64(torch.stack([x[1] for x in each])), dV=to_np64(torch.stack([x[2] for x in each])))
+        assert_grads_close(got, want, "bf16", f"{B}x{H}x{N}x{M}x{D}")
+        assert np.linalg.norm(got["dQ"] - want["dQ"]) <= (2.0 ** -18 + 2 * 512 * 2.0 ** -24 / 3) * np.linalg.norm(want["dQ"])
