@@ -211,17 +211,20 @@ inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes, i
     return best;
 }
 
-// CTAs per head of the token kernel of the backward, which leaves no partial results.  As many as fill the chip once, unless that leaves enough SMs
+// CTAs per head of the kernels of the backward that have tokens on the lanes.  As many as fill the chip once, unless that leaves enough SMs
 // idle that several rounds are 2 % quicker; a CTA's start, where the head's latent operands are split and stored, counts as six units of 64
 // latents against a tile, and a fifth of a tile.  us per training step, once : several rounds: 32 heads (128 of 148 CTAs : 288), 50489 tokens, M = 624, D = 16
 // 2793 : 2689, 68334 tokens, M = 80, D = 8 734 : 710, 25344 tokens, M = 336, D = 32 890 : 875; 8 heads (144 : 296) of 1048576 tokens, M = 1024, D = 8
 // 18813 : 18640; D = 64, where a unit has 32 latents and up to 160 of them three parts to split, 32 heads (128 : 288), 40000 tokens, M = 64 855 : 824; 40
 // (120 : 280), 30000, M = 160 1611 : 1530; 64 (128 : 256), 9000, M = 96 500 : 496; the same number either way 128 heads, M = 192, and 32, 20011, M = 128.
 // (A CTA per SM with a share of all heads' tiles in a row, needs a loop over heads around the kernel's body, which made every training step 5 % slower.)
-inline int token_splits(const flare_desc_t *d, int tiles, int mc, int sms) {
+// `part`: what one more CTA per head costs beyond that, in the same units (some 0.65 us): the two sweeps leave partial results of D floats per latent, two per
+// CTA (the token kernel leaves none), which take about a unit per 8 MB to write and add up.  us per backward of 128 heads of 8192 tokens, M = 1024, D = 16, in seven
+// rounds with 134 MB of them : once over the chip with 17 MB 1905 : 1835; M = 512, D = 8, where 34 MB do not decide, 880 : 899.
+inline int token_splits(const flare_desc_t *d, int tiles, int mc, int sms, double part = 0.0) {
     const double units = (double)((mc + 63) / 64);
     const long heads = (long)d->B * d->H;
-    auto cost = [&](long s) { return (double)((heads * s + sms - 1) / sms) * ((double)((tiles + s - 1) / s) * units + 6.0 + 0.2 * units); };
+    auto cost = [&](long s) { return (double)((heads * s + sms - 1) / sms) * ((double)((tiles + s - 1) / s) * units + 6.0 + 0.2 * units) + part * (double)s; };
     int best = (int)std::min<long>(std::max(1L, sms / heads), tiles);
     double best_cost = 0.98 * cost(best);
     for (int s = best + 1; s <= std::min(tiles, sms); ++s)
@@ -434,7 +437,7 @@ inline SweepPlan sweep_ranges(const flare_desc_t *d, int sms) {
     p.ranges = (d->M + p.range - 1) / p.range;
     const int tiles = (d->N + kTile - 1) / kTile;
     p.chunk = p.ranges == 1 ? tiles : (int)std::min<size_t>(tiles, std::max<size_t>(1, kRangeBytes / range_tile_bytes(d)));
-    p.splits = token_splits(d, p.chunk, p.range, sms);
+    p.splits = token_splits(d, p.chunk, p.range, sms, (double)d->B * d->H * d->M * d->D * 2 * sizeof(float) / 8.0e6);
     if (p.chunk < tiles) {                                      // chunks of about equal size, each a whole number of tiles to a CTA
         const int chunks = (tiles + p.chunk / p.splits * p.splits - 1) / (p.chunk / p.splits * p.splits);
         p.chunk = ((tiles + chunks - 1) / chunks + p.splits - 1) / p.splits * p.splits;
