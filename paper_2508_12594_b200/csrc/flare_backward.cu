@@ -81,7 +81,7 @@ int launch_dz_sweep(const flare_desc_t *d, const SweepPlan &p, const void *K, co
     if ((rc = make_token_map(&tmG, dY, d, kTile, D)) != FLARE_OK) return rc;
     static std::atomic<uint64_t> smem_opt_in{0};
     if ((rc = ensure_big_smem(bwd_dz_sweep_kernel<D, DRT, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
-    FLARE_CUDA(launch_after(bwd_dz_sweep_kernel<D, DRT, kRanges>, dim3((unsigned)std::min(p.splits, a.tiles), d->H, d->B), kSwThreads, BwdDzSmem<D>::total(p.stages, p.range), st,
+    FLARE_CUDA(launch_after(bwd_dz_sweep_kernel<D, DRT, kRanges>, dim3((unsigned)(std::min(p.splits, a.tiles) * p.side), d->H, d->B), kSwThreads, BwdDzSmem<D>::total(p.stages, p.range), st,
                             tmK, tmG, a));
     return FLARE_OK;
 }
@@ -98,7 +98,7 @@ int launch_grad_sweep(const flare_desc_t *d, const SweepPlan &p, const void *K, 
     if ((rc = make_token_map(&tmDV, a.dV, d, kTile, out)) != FLARE_OK) return rc;
     static std::atomic<uint64_t> smem_opt_in{0};
     if ((rc = ensure_big_smem(bwd_grad_sweep_kernel<D, DRT, kRanges>, smem_opt_in)) != FLARE_OK) return rc;
-    FLARE_CUDA(launch_after(bwd_grad_sweep_kernel<D, DRT, kRanges>, dim3((unsigned)std::min(p.splits, a.tiles), d->H, d->B), kSwThreads, BwdGradSmem<D>::total(p.bufs, p.stages, p.range), st,
+    FLARE_CUDA(launch_after(bwd_grad_sweep_kernel<D, DRT, kRanges>, dim3((unsigned)(std::min(p.splits, a.tiles) * p.side), d->H, d->B), kSwThreads, BwdGradSmem<D>::total(p.bufs, p.stages, p.range), st,
                             tmK, tmV, tmG, tmDK, tmDV, a));
     return FLARE_OK;
 }
@@ -113,8 +113,9 @@ int backward_sweeps(const flare_desc_t *d, int sms, const void *Q, const void *K
     const int tiles = (d->N + kTile - 1) / kTile;
     uint32_t *status = reinterpret_cast<uint32_t *>(ws);
     if (const int rc = clear_header(ws, 0, st)) return rc;
-    // One launch per range of latents and chunk of tokens: with ranges, all of them over one chunk before the next.
+    // One launch per range of latents and chunk of tokens: all ranges over one chunk before the next.  Side by side all of them in one.
     auto sweep = [&](const SweepPlan &p, auto &&launch) -> int {
+        if (p.side > 1) return launch(0, tiles, 0, p.range);
         for (int t0 = 0; t0 < tiles; t0 += p.chunk)
             for (int m0 = 0; m0 < d->M; m0 += p.range)
                 if (const int rc = launch(t0, std::min(p.chunk, tiles - t0), m0, std::min(p.range, d->M - m0))) return rc;
@@ -125,12 +126,15 @@ int backward_sweeps(const flare_desc_t *d, int sms, const void *Q, const void *K
         if (p.stages < p.bufs) return FLARE_ERR_UNSUPPORTED;
         if (const int rc = sweep(p, [&](int t0, int nt, int m0, int mc) -> int {
                 const BwdDzArgs a{static_cast<const __nv_bfloat16 *>(Q), Z, lse_dec, at(w.part), at(w.dd), status, d->B, d->H, d->N, mc, d->M, m0, m0 == 0,
-                                  m0 + mc >= d->M, reinterpret_cast<float4 *>(ws + w.dd_other), d->scale * kLog2e, nt, p.stages, t0};
+                                  p.side == 1 && m0 + mc >= d->M, reinterpret_cast<float4 *>(ws + w.dd_other), d->scale * kLog2e, nt, p.stages, t0, p.side};
                 if (p.ranges == 1) return launch_dz_sweep<D, DRT, false>(d, p, K, dY, a, st);
                 if constexpr (D == 16) return launch_dz_sweep<D, DRT, true>(d, p, K, dY, a, st);
                 return FLARE_ERR_UNSUPPORTED;                   // (ranges at D = 32: see use_sweeps)
             }))
             return rc;
+        if (p.side > 1)
+            FLARE_CUDA(launch_after(bwd_join_dd_kernel<kReduceThreads>, dim3((unsigned)(((size_t)d->B * d->H * tiles * kTile + kReduceThreads - 1) / kReduceThreads)), kReduceThreads, 0, st, reinterpret_cast<const float4 *>(ws + w.dd_other), at(w.dd),
+                                    p.side, d->B * d->H, d->N, tiles));
         const int slices = reduce_slices(2 * p.splits, d->D);
         const unsigned row_blocks = reduce_blocks(rows, d->D, slices);
         FLARE_CUDA(launch_after(bwd_dz_reduce_kernel<(DRT ? DRT : D) / 4>, row_blocks, kReduceThreads, 0, st, at(w.part), Z, at(w.dz), at(w.de), 2 * p.splits, rows, slices,
@@ -140,13 +144,16 @@ int backward_sweeps(const flare_desc_t *d, int sms, const void *Q, const void *K
     if (p.stages < p.bufs || BwdGradSmem<D>::log2_accs(p.range) < 0) return FLARE_ERR_UNSUPPORTED;
     if (const int rc = sweep(p, [&](int t0, int nt, int m0, int mc) -> int {
             const BwdGradArgs a{static_cast<const __nv_bfloat16 *>(Q), Z, at(w.dz), lse_enc, at(w.de), lse_dec, at(w.dd), mask, static_cast<__nv_bfloat16 *>(dK),
-                                static_cast<__nv_bfloat16 *>(dV), at(w.part), status, d->B, d->H, d->N, mc, d->M, m0, m0 == 0, m0 + mc >= d->M,
-                                at(w.kvacc), d->scale, d->scale * kLog2e, nt, p.stages, p.bufs, t0};
+                                static_cast<__nv_bfloat16 *>(dV), at(w.part), status, d->B, d->H, d->N, mc, d->M, m0, m0 == 0, p.side == 1 && m0 + mc >= d->M,
+                                at(w.kvacc), d->scale, d->scale * kLog2e, nt, p.stages, p.bufs, t0, p.side};
             if (p.ranges == 1) return launch_grad_sweep<D, DRT, false>(d, p, K, V, dY, a, st);
             if constexpr (D == 16) return launch_grad_sweep<D, DRT, true>(d, p, K, V, dY, a, st);
             return FLARE_ERR_UNSUPPORTED;
         }))
         return rc;
+    if (p.side > 1)
+        FLARE_CUDA(launch_after(bwd_join_rows_kernel<DRT ? DRT : D, kReduceThreads>, dim3((unsigned)(((size_t)2 * d->B * d->H * tiles * (d->D / 4) * kTile + kReduceThreads - 1) / kReduceThreads)), kReduceThreads, 0, st,
+                                reinterpret_cast<const float4 *>(ws + w.kvacc), static_cast<__nv_bfloat16 *>(dK), static_cast<__nv_bfloat16 *>(dV), p.side, d->B, d->H, d->N, tiles, d->scale));
     FLARE_REDUCE(bwd_dq_reduce_kernel, (long)d->H * d->M, d->B * 2 * p.splits, d->D, st, at(w.part), dQ, 2 * p.splits, d->B, (long)d->H * d->M, d->scale);
     return FLARE_OK;
 }

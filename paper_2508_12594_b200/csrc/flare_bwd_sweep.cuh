@@ -138,13 +138,14 @@ struct BwdDzArgs {
     float *part;               // [2 * CTAs per head][B*H*M][D] partial dZ rows
     float *dd;                 // [2][B,H,N]: dd as a float and what is left of it
     uint32_t *status;
-    int B, H, N, M;            // M: latents this launch works on (all of them, or a range)
+    int B, H, N, M;            // M: latents this launch works on (all of them, or a range; the last of several side by side may be shorter)
     int mtot, m0;              // latents per head in memory, and the first one of this launch's range
-    int first, last;           // range of latents (without ranges both)
-    float4 *sums;              // [B,H][tile of this launch][token of the tile]: RowSums of the earlier ranges
+    int first, last;           // range of latents (without ranges both; side by side the first only)
+    float4 *sums;              // [range of those side by side][B,H][tile of this launch][token of the tile]: RowSums of the earlier ranges
     float sl2;                 // scale * log2(e)
     int tiles, stages;         // tiles of tokens this launch works on
     int t0;                    // the first of them (without ranges 0)
+    int side;                  // ranges side by side, in neighbouring blocks (else 1)
 };
 
 template <int D>
@@ -181,7 +182,8 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     constexpr int UNIT = kSwUnit, RING = kSwRing, DR = DRT ? DRT : D;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = ptx::align_1024(smem_raw);
-    const int M = a.M, stages = a.stages;
+    const int side = kRanges ? a.side : 1, which_range = kRanges ? (int)blockIdx.x % side : 0, cta = (int)blockIdx.x / side, ctas = (int)gridDim.x / side;
+    const int m0 = a.m0 + which_range * a.M, M = kRanges ? min(a.M, a.mtot - m0) : a.M, stages = a.stages;
     uint8_t *tiles_s = smem + SM::tile_off;
     float *ring = reinterpret_cast<float *>(smem + SM::ring_off(stages, M));
     float4 *dds = reinterpret_cast<float4 *>(smem + SM::dds_off(stages, M));
@@ -195,8 +197,8 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
 
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int h = blockIdx.y, b = blockIdx.z;
-    const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // tiles of this CTA
-    auto tile_at = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x + (kRanges ? a.t0 : 0); };   // the i-th of them
+    const int nt = (a.tiles - cta + ctas - 1) / ctas;   // tiles of this CTA
+    auto tile_at = [&](int i) { return cta + i * ctas + (kRanges ? a.t0 : 0); };   // the i-th of them
     const int nu = (M + UNIT - 1) / UNIT, wlast = M - (nu - 1) * UNIT;                 // latent units of a tile; columns of the last
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S or A
     const int sets = M <= 32 ? 2 : 1, cps = sets == 2 ? 2 : kSwGroups;                 // sets of warps that take the tiles in turn, column groups of each
@@ -219,7 +221,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     ptx::grid_launch();
     ptx::grid_wait();
-    const size_t bh = (size_t)b * a.H + h, q0 = (size_t)h * a.mtot + a.m0, r0 = bh * a.mtot + a.m0;
+    const size_t bh = (size_t)b * a.H + h, q0 = (size_t)h * a.mtot + m0, r0 = bh * a.mtot + m0;
     z_centre<DR>(centre, a.Z + bh * a.mtot * DR, a.mtot);
     if (DRT != 0)                                               // narrow form: the other columns of every row stay zero
         for (int i = threadIdx.x; i < 3 * M * (G::RB / 16); i += kSwThreads) reinterpret_cast<uint4 *>(smem + SM::lat_off(stages, M, 0))[i] = make_uint4(0, 0, 0, 0);
@@ -305,7 +307,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 const int n = tile_at(i) * kTile + e * 32 + lane;
                 if (n >= a.N) continue;
                 const size_t at = bh * a.N + n;
-                const size_t so_far = ((bh * a.tiles + (tile_at(i) - (kRanges ? a.t0 : 0))) * kTile) + e * 32 + lane;
+                const size_t so_far = ((((size_t)which_range * a.B * a.H + bh) * a.tiles + (tile_at(i) - (kRanges ? a.t0 : 0))) * kTile) + e * 32 + lane;
                 if (kRanges && !a.first) all[e].join(a.sums[so_far]);
                 if (!kRanges || a.last) {
                     const float2 d = all[e].mean();
@@ -451,7 +453,7 @@ bwd_dz_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_consta
                 if (window > 0 && !warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdDz | 11)) break;
                 if (!warp_wait(bar(FL_FULL), window & 1, abort_flag, kErrBwdDz | 10)) break;
                 ptx::tc_fence_after();
-                sweep_flush<D, DR>(acc0 - tm + gcol, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, min(sums_in_turn, i + 1 - window * flush), mine, cps, row, off, window > 0 || (kRanges && a.t0 > 0));
+                sweep_flush<D, DR>(acc0 - tm + gcol, a.part, (size_t)a.B * a.H * a.mtot, cta, r0, M, nu, min(sums_in_turn, i + 1 - window * flush), mine, cps, row, off, window > 0 || (kRanges && a.t0 > 0));
                 ptx::tc_fence_before();
                 __syncwarp();
                 ptx::mbar_arrive_if(bar(FL_DONE), lead);
@@ -489,9 +491,9 @@ struct BwdGradArgs {
     float *part;               // [2 * CTAs per head][B*H*M][D] partial dQ rows (un-scaled)
     uint32_t *status;
     int B, H, N, M, mtot, m0, first, last;   // as in BwdDzArgs
-    float *kvacc;              // float32 dK and dV so far, where there are ranges; the last writes the rows.  [2][B,H][tile of this launch][D / 4][token of the tile][4]
+    float *kvacc;              // float32 dK and dV so far, where there are ranges; the last writes the rows.  [range of those side by side][2][B,H][tile of this launch][D / 4][token of the tile][4]
     float scale, sl2;
-    int tiles, stages, bufs, t0;   // as in BwdDzArgs
+    int tiles, stages, bufs, t0, side;   // as in BwdDzArgs
 };
 
 template <int D>
@@ -534,7 +536,8 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     constexpr int UNIT = kSwUnit, RING = kSwRing, DR = DRT ? DRT : D;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = ptx::align_1024(smem_raw);
-    const int M = a.M, stages = a.stages, bufs = a.bufs;
+    const int side = kRanges ? a.side : 1, which_range = kRanges ? (int)blockIdx.x % side : 0, cta = (int)blockIdx.x / side, ctas = (int)gridDim.x / side;
+    const int m0 = a.m0 + which_range * a.M, M = kRanges ? min(a.M, a.mtot - m0) : a.M, stages = a.stages, bufs = a.bufs;
     uint8_t *tiles_s = smem + SM::tile_off(bufs);
     float *cst = reinterpret_cast<float *>(smem + SM::cst_off(bufs, stages, M));
     float *ring = reinterpret_cast<float *>(smem + SM::ring_off(bufs, stages, M));
@@ -549,8 +552,8 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int h = blockIdx.y, b = blockIdx.z;
-    const int nt = (a.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    auto tile_at = [&](int i) { return (int)blockIdx.x + i * (int)gridDim.x + (kRanges ? a.t0 : 0); };   // the i-th of them
+    const int nt = (a.tiles - cta + ctas - 1) / ctas;
+    auto tile_at = [&](int i) { return cta + i * ctas + (kRanges ? a.t0 : 0); };   // the i-th of them
     const int nu = (M + UNIT - 1) / UNIT, wlast = M - (nu - 1) * UNIT;
     const int sets = M <= 32 ? 2 : 1, cps = sets == 2 ? 2 : kSwGroups;
     const int ucols = min(UNIT, (M + 31) & ~31);                // columns of a region S, A or C
@@ -576,7 +579,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32(tmem_slot), 512);
     ptx::grid_launch();
     ptx::grid_wait();
-    const size_t bh = (size_t)b * a.H + h, q0 = (size_t)h * a.mtot + a.m0, r0 = bh * a.mtot + a.m0;
+    const size_t bh = (size_t)b * a.H + h, q0 = (size_t)h * a.mtot + m0, r0 = bh * a.mtot + m0;
     float K, least, unfolded;                                   // (unfolded != 0: c is 1)
     {
         // K: the middle of the latents' lse_enc (log2 units), leaving out those that saw no valid token and those whose encode is switched off
@@ -923,7 +926,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                     float4 *sums = nullptr;
                     float4 before[PW / 4];
                     if (kRanges) {
-                        sums = reinterpret_cast<float4 *>(a.kvacc) + ((((size_t)which * a.B * a.H + bh) * a.tiles + (t - a.t0)) * (DR / 4) + c0 / 4) * kTile + row;
+                        sums = reinterpret_cast<float4 *>(a.kvacc) + ((((size_t)(2 * which_range + which) * a.B * a.H + bh) * a.tiles + (t - a.t0)) * (DR / 4) + c0 / 4) * kTile + row;
                         if (!a.first) {
 #pragma unroll
                             for (int c = 0; c < PW / 4; ++c) before[c] = sums[c * kTile];
@@ -1082,7 +1085,7 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
                         if (window > 0 && !(ok = warp_wait(bar(FL_DONE), (window - 1) & 1, abort_flag, kErrBwdTok | 15))) break;
                         if (!(ok = warp_wait(bar(FL_FULL), window & 1, abort_flag, kErrBwdTok | 14))) break;
                         ptx::tc_fence_after();
-                        sweep_flush<D, DR>(gcol + dq0, a.part, (size_t)a.B * a.H * a.mtot, blockIdx.x, r0, M, nu, min(sums_in_turn, before + 1 - window * flush), mine, cps, row, off, window > 0 || (kRanges && a.t0 > 0));
+                        sweep_flush<D, DR>(gcol + dq0, a.part, (size_t)a.B * a.H * a.mtot, cta, r0, M, nu, min(sums_in_turn, before + 1 - window * flush), mine, cps, row, off, window > 0 || (kRanges && a.t0 > 0));
                         ptx::tc_fence_before();
                         __syncwarp();
                         ptx::mbar_arrive_if(bar(FL_DONE), lead);
@@ -1101,6 +1104,47 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         ptx::tmem_dealloc(tm, 512);
     }
     if (threadIdx.x == 0 && *abort_flag != 0 && a.status != nullptr) atomicCAS(a.status, 0u, *abort_flag);
+}
+
+// ---------------------------------------------------------------------------------------------------------- ranges side by side
+// dd of every token from the ranges' RowSums, in the order of the latents.
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads)
+bwd_join_dd_kernel(const float4 *sums, float *dd, int side, int BH, int N, int tiles) {
+    ptx::grid_launch();
+    ptx::grid_wait();
+    const size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x, plane = (size_t)BH * tiles * kTile;
+    const size_t bh = i / ((size_t)tiles * kTile), n = i % ((size_t)tiles * kTile);
+    if (i >= plane || n >= (size_t)N) return;
+    RowSums all;
+    all.set(sums[i]);
+#pragma unroll 4
+    for (int r = 1; r < side; ++r) all.join(sums[r * plane + i]);
+    const float2 d = all.mean();
+    dd[bh * N + n] = d.x;
+    dd[((size_t)BH + bh) * N + n] = d.y;
+}
+
+// Rows of dK and dV from the ranges' shares, in the order of the latents: a thread has four columns of a row.
+template <int D, int kThreads>
+__global__ void __launch_bounds__(kThreads)
+bwd_join_rows_kernel(const float4 *shares, __nv_bfloat16 *dK, __nv_bfloat16 *dV, int side, int B, int H, int N, int tiles, float scale) {
+    ptx::grid_launch();
+    ptx::grid_wait();
+    const size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x, plane = (size_t)2 * B * H * tiles * (D / 4) * kTile;
+    if (i >= plane) return;
+    const size_t row = i % kTile, c = i / kTile % (D / 4), t = i / kTile / (D / 4) % tiles, whh = i / kTile / (D / 4) / tiles, bh = whh % ((size_t)B * H), n = t * kTile + row;
+    if (n >= (size_t)N) return;
+    float4 v = shares[i];
+#pragma unroll 4
+    for (int r = 1; r < side; ++r) {
+        const float4 x = shares[r * plane + i];
+        v = make_float4(v.x + x.x, v.y + x.y, v.z + x.z, v.w + x.w);
+    }
+    const bool value = whh >= (size_t)B * H;
+    const float sc = value ? 1.f : scale;
+    const uint2 out = make_uint2(ptx::pack_bf16(v.x * sc, v.y * sc), ptx::pack_bf16(v.z * sc, v.w * sc));
+    *reinterpret_cast<uint2 *>((value ? dV : dK) + ((bh / H * N + n) * H + bh % H) * D + 4 * c) = out;
 }
 
 }  // namespace flare

@@ -221,10 +221,13 @@ inline int balanced_splits(long groups, int tiles, int sms, size_t part_bytes, i
 // `part`: what one more CTA per head costs beyond that, in the same units (some 0.65 us): the two sweeps leave partial results of D floats per latent, two per
 // CTA (the token kernel leaves none), which take about a unit per 8 MB to write and add up.  us per backward of 128 heads of 8192 tokens, M = 1024, D = 16, in seven
 // rounds with 134 MB of them : once over the chip with 17 MB 1905 : 1835; M = 512, D = 8, where 34 MB do not decide, 880 : 899.
-inline int token_splits(const flare_desc_t *d, int tiles, int mc, int sms, double part = 0.0) {
+inline double token_cost(long ctas, int tiles_each, int mc, int sms) {
     const double units = (double)((mc + 63) / 64);
+    return (double)((ctas + sms - 1) / sms) * (tiles_each * units + 6.0 + 0.2 * units);
+}
+inline int token_splits(const flare_desc_t *d, int tiles, int mc, int sms, double part = 0.0) {
     const long heads = (long)d->B * d->H;
-    auto cost = [&](long s) { return (double)((heads * s + sms - 1) / sms) * ((double)((tiles + s - 1) / s) * units + 6.0 + 0.2 * units) + part * (double)s; };
+    auto cost = [&](long s) { return token_cost(heads * s, (int)((tiles + s - 1) / s), mc, sms) + part * (double)s; };
     int best = (int)std::min<long>(std::max(1L, sms / heads), tiles);
     double best_cost = 0.98 * cost(best);
     for (int s = best + 1; s <= std::min(tiles, sms); ++s)
@@ -415,8 +418,15 @@ inline bool token_in_ranges(const flare_desc_t *d) { return use_tc(d) && d->M > 
 inline int token_ranges(const flare_desc_t *d) { return (d->M + token_range_most(d) - 1) / token_range_most(d); }
 inline int token_range(const flare_desc_t *d) { return ((d->M + token_ranges(d) - 1) / token_ranges(d) + 15) / 16 * 16; }
 
-// Two sweeps over the tokens (flare_bwd_sweep.cuh, where both sides are measured): heads up to 16 wide, and 32 wide as long as one launch takes all latents.
-inline bool use_sweeps(const flare_desc_t *d) { return use_tc(d) && (d->D <= 16 || (d->D == 32 && d->M <= 320)); }
+// Two sweeps over the tokens (flare_bwd_sweep.cuh, where both sides are measured): heads up to 16 wide, and 32 wide as long as one launch takes all latents.  Not
+// where that leaves a CTA per tile and few of them, each with many units of latents: the kernels with latents on the lanes share these out.  us per backward, sweeps :
+// the others, D = 32, tiles of all heads: 8, M = 208 29.3 : 29.2, M = 256 31.1 : 29.8, M = 320 35.2 : 31.9; 16, M = 256 31.1 : 30.3, M = 320 35.1 : 32.9; 32, M = 256 31.4 : 31.8, M =
+// 320 35.2 : 34.6; 64, M = 256 33.8 : 35.9, M = 320 37.9 : 36.6; 96, M = 320 40.8 : 40.0; 120, M = 320 42.0 : 46.5.
+inline bool use_sweeps(const flare_desc_t *d) {
+    if (!use_tc(d) || d->D > 32) return false;
+    const long tiles = (long)d->B * d->H * ((d->N + kTile - 1) / kTile);
+    return d->D <= 16 || (d->M <= 320 && !(d->M > 256 && tiles <= 100) && !(d->M == 256 && tiles <= 16));
+}
 // Latents one launch of a sweep takes: what its operands leave of shared memory (beside two tile stages) and the sums over tokens of tensor memory; more are
 // worked off in ranges of about equal size, whole units of 64.
 // Ranges leave float32 rows of dK and dV to one another (in the first sweep RowSums): a launch takes a chunk of each item's tokens, so that the rows stay within
@@ -425,7 +435,13 @@ inline bool use_sweeps(const flare_desc_t *d) { return use_tc(d) && (d->D <= 16 
 // 6394 : 6586 : 6791 : 7136 : 7724, 131072, D = 16 1681 : 1644 : 1745 : 1822 : 1972 (a chunk starts and ends as any launch does, and chunks give 144 CTAs to the 148 SMs
 // where one launch of 1048576 tokens gives two rounds of 148).
 constexpr size_t kRangeBytes = (size_t)128 << 20;
-struct SweepPlan { int range, ranges, chunk, splits, stages, bufs; };
+// Ranges side by side, each with CTAs of its own and rows that a launch of its own adds up, where one after the other (or all latents in one) leaves a few CTAs
+// with many units each.  In the units of token_cost: what a sweep takes to start beyond that, and the launch that joins.  us per backward of 8 heads, one after
+// the other : side by side : the three kernels before, D = 16: 128 tokens, M = 512 34.8 : 27.0 : 31.6, 1024 66.9 : 32.3 : 42.1, 2048 118 : 34 : 73; 1024 tokens, M = 768 48.8 : 39.8 :
+// 47.7, 1024 72.5 : 44.3 : 55.0, 2048 127 : 61 : 94; 16384 tokens, M = 1024 279 : 247 : 293.  Beyond sixteen tiles to an SM it depends on the units alone: 65536 tokens, M = 1024, D = 8 835 : 818,
+// M = 1040 854 : 909.
+constexpr double kSweepStart = 5.0, kSideCost = 5.0;
+struct SweepPlan { int range, ranges, side, chunk, splits, stages, bufs; };
 inline size_t range_tile_bytes(const flare_desc_t *d) {         // of one tile of every item
     return sizeof(float) * kTile * (size_t)d->B * d->H * 2 * d->D;
 }
@@ -435,18 +451,37 @@ inline SweepPlan sweep_ranges(const flare_desc_t *d, int sms) {
     p.ranges = (d->M + most - 1) / most;
     p.range = p.ranges == 1 ? d->M : ((d->M + p.ranges - 1) / p.ranges + 63) / 64 * 64;
     p.ranges = (d->M + p.range - 1) / p.range;
+    p.side = 1;
     const int tiles = (d->N + kTile - 1) / kTile;
     p.chunk = p.ranges == 1 ? tiles : (int)std::min<size_t>(tiles, std::max<size_t>(1, kRangeBytes / range_tile_bytes(d)));
     p.splits = token_splits(d, p.chunk, p.range, sms, (double)d->B * d->H * d->M * d->D * 2 * sizeof(float) / 8.0e6);
     if (p.chunk < tiles) {                                      // chunks of about equal size, each a whole number of tiles to a CTA
         const int chunks = (tiles + p.chunk / p.splits * p.splits - 1) / (p.chunk / p.splits * p.splits);
         p.chunk = ((tiles + chunks - 1) / chunks + p.splits - 1) / p.splits * p.splits;
+        return p;
+    }
+    // Side by side?  Once or twice over the chip, or a tile to a CTA.
+    const long heads = (long)d->B * d->H;
+    if (d->D == 32 || heads * tiles > 16L * sms) return p;
+    auto cost = [&](long ctas, int each, int range) { return token_cost(ctas, each, range, sms) + (double)((ctas + sms - 1) / sms) * kSweepStart; };
+    double best = p.ranges * cost(heads * p.splits, (tiles + p.splits - 1) / p.splits, p.range);
+    for (int range = 64; range < d->M && range <= most; range += 64) {
+        const int side = (d->M + range - 1) / range;
+        if (side * range_tile_bytes(d) * tiles > kRangeBytes) continue;
+        for (int rounds = 1; rounds <= 2; ++rounds) {
+            const int splits = (int)std::min<long>(tiles, std::max(1L, (long)rounds * sms / (heads * side)));
+            const double c = cost(heads * splits * side, (tiles + splits - 1) / splits, range) + kSideCost + (double)side * range_tile_bytes(d) * tiles / 8.0e6;
+            if (c < best) {
+                best = c;
+                p.range = range; p.ranges = p.side = side; p.splits = splits;
+            }
+        }
     }
     return p;
 }
 inline int sweep_launches(const flare_desc_t *d, const SweepPlan &p) {
     const int tiles = (d->N + kTile - 1) / kTile;
-    return p.ranges * ((tiles + p.chunk - 1) / p.chunk);
+    return p.side > 1 ? 2 : p.ranges * ((tiles + p.chunk - 1) / p.chunk);
 }
 inline SweepPlan dz_sweep_plan(const flare_desc_t *d, int sms) {
     SweepPlan p = sweep_ranges(d, sms);
@@ -483,7 +518,7 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     w.dd_other = w.kvacc = off;                                // over latent ranges: dd so far, and float32 sums of the rows
     if (use_sweeps(d)) {                                       // (the two sweeps one after the other, in the same place: a row of either is at least a RowSums)
         const SweepPlan p = grad_sweep_plan(d, sms);
-        if (p.ranges > 1) off += align_up(range_tile_bytes(d) * p.chunk);
+        if (p.ranges > 1) off += align_up(range_tile_bytes(d) * p.side * p.chunk);
     } else if (token_in_ranges(d)) {
         w.kvacc = off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
         off += align_up(sizeof(float) * 3 * (size_t)d->B * d->N * d->H * d->D);

@@ -115,9 +115,11 @@ def test_scratch_at_head_width_64_is_that_of_the_exact_form(lib):
 @pytest.mark.parametrize("M,D,dtype,kernels", [
     (256, 64, flare.DTYPE_F32, 6), (528, 32, flare.DTYPE_F16, 6), (2048, 64, flare.DTYPE_F32, 6),     # one token kernel whatever M is
     (192, 64, flare.DTYPE_BF16, 6), (208, 64, flare.DTYPE_BF16, 7), (400, 64, flare.DTYPE_BF16, 8),   # up to 192 latents a launch at D = 64
-    (512, 32, flare.DTYPE_BF16, 6), (528, 32, flare.DTYPE_BF16, 7)])
+    (512, 32, flare.DTYPE_BF16, 6), (528, 32, flare.DTYPE_BF16, 7),
+    (256, 16, flare.DTYPE_BF16, 5), (512, 16, flare.DTYPE_BF16, 7), (784, 16, flare.DTYPE_BF16, 7), (2048, 8, flare.DTYPE_BF16, 7)])   # two sweeps
 def test_launch_count_of_a_backward(lib, M, D, dtype, kernels):
-    """Header, dZ and its reduction, the token kernel (bfloat16: one per range of latents), dQ and its reduction."""
+    """Header, dZ and its reduction, the token kernel (bfloat16: one per range of latents), dQ and its reduction; two sweeps: header, the sweeps and their
+    reductions, and with ranges of latents side by side, as few tokens want them, a kernel after each sweep that joins them."""
     assert flare.flare_launch_count(flare.FlareDesc(1, 2, 1000, M, D, dtype, 1.0), flare.OP_BACKWARD) == kernels
 
 
@@ -128,3 +130,9 @@ def test_ranges_of_latents_take_bounded_scratch(lib, B, H, N, M, D):
     tokens.  (All else grows as the latents do, or less.)"""
     need = lambda m: flare.flare_workspace_bytes(flare.FlareDesc(B, H, N, m, D, flare.DTYPE_BF16, 1.0), flare.OP_BACKWARD)
     assert 0 < need(M) <= need(768) * M / 768 + (128 << 20)
+
+
+@pytest.mark.parametrize("B,H,N,M,kernels", [(1, 8, 65536, 768, 5), (1, 8, 65536, 784, 7), (1, 8, 65536, 1552, 9), (1, 8, 262144, 784, 15), (4, 8, 262144, 2048, 57)])
+def test_launch_count_of_a_backward_over_ranges(lib, B, H, N, M, kernels):
+    """Many tokens: each sweep is a launch per range of latents (up to 768), and per chunk of tokens where the rows between ranges would take more than 128 MB."""
+    assert flare.flare_launch_count(flare.FlareDesc(B, H, N, M, 16, flare.DTYPE_BF16, 1.0), flare.OP_BACKWARD) == kernels

@@ -1,5 +1,5 @@
 """The two sweeps over the tokens of the bfloat16 backward (heads up to 32 wide) where they can go wrong, against the CPU oracle (needs a B200): latents
-around the units of 64 and the most of one launch, ranges of unequal size, more tiles to a CTA than tensor memory adds up in a row (with one and with two
+around the units of 64 and the most of one launch, ranges of unequal size side by side and one after the other, more tiles to a CTA than tensor memory adds up in a row (with one and with two
 sets of warps), rows that leave by a tile's copy at the end of a batch item, narrow heads."""
 import numpy as np
 import pytest
@@ -8,6 +8,7 @@ import torch
 from paper_2508_12594_b200 import flare, workloads
 from tests._util import dev, to_np64
 from tests.test_gpu_backward import assert_grads_close, gpu_backward, oracle_backward
+from tests.test_gpu_backward_tiles import dk_error_bound
 from tests.test_gpu_fullsize import _float64_z_and_dq
 
 pytestmark = pytest.mark.gpu
@@ -20,21 +21,92 @@ CASES = [  # B, H, N, M, D, masked_fraction
     (1, 2, 385, 176, 32, 0.1),
     (2, 4, 383, 80, 8, 0.1),
     (2, 4, 385, 64, 4, 0.1),
-    (1, 1, 700, 320, 32, 0.1),            # the most latents at D = 32, and one more (other kernels)
+    (1, 1, 700, 320, 32, 0.1),            # the most latents at D = 32, few tiles and more than a hundred, and one more (other kernels)
+    (4, 8, 700, 320, 32, 0.1),
     (1, 1, 700, 336, 32, 0.1),
-    (1, 1, 300, 768, 16, 0.0),            # the most of one launch at D = 16; two ranges, the second shorter; three
+    (1, 1, 300, 768, 16, 0.0),            # few tokens, ranges of latents side by side: the last of all sizes, one and several tiles to a CTA
     (1, 2, 300, 784, 16, 0.1),
     (1, 2, 260, 1552, 8, 0.0),
+    (3, 3, 130, 544, 16, 0.1),
+    (2, 2, 383, 400, 4, 0.1),
+    (1, 4, 4000, 1040, 8, 0.0),
+    (1, 9, 1100, 2048, 16, 0.1),
+    (4, 8, 1024, 768, 16, 0.0),           # the most of one launch at D = 16
+    (1, 64, 4800, 784, 16, 0.1),          # ranges one after the other: two, the second shorter; three
+    (1, 64, 4800, 1552, 8, 0.0),
+    (2, 32, 4800, 1040, 4, 0.1),
     (37, 4, 8400, 16, 8, 0.0),            # 66 tiles to a CTA, two sets of warps
     (37, 4, 8272, 16, 32, 0.0),           # 65 tiles, the last by itself; warps without columns run ahead of the others
     (37, 4, 8400, 48, 16, 0.1),           # one set
 ]
 
 
+def some_heads(inp, heads):
+    """The inputs of these heads alone (the oracle takes minutes for 64)."""
+    cut = lambda x: None if x is None else x[:, :, heads].contiguous()
+    return workloads.Inputs(Q=inp.Q[heads].contiguous(), K=cut(inp.K), V=cut(inp.V), key_mask=inp.key_mask, dY=cut(inp.dY))
+
+
+def gradients_of(inp, heads):
+    got = gpu_backward(inp)
+    return dict(dQ=got["dQ"][heads], dK=got["dK"][:, :, heads], dV=got["dV"][:, :, heads])
+
+
 @pytest.mark.parametrize("B,H,N,M,D,masked", CASES)
 def test_backward_in_two_sweeps(oracle, B, H, N, M, D, masked):
     inp = workloads.make_random(B, H, N, M, D, dtype="bf16", seed=N + M, masked_fraction=masked, with_dy=True, k_std=0.8)
-    assert_grads_close(gpu_backward(inp), oracle_backward(oracle, inp), "bf16", f"{B}x{H}x{N}x{M}x{D}")
+    heads = [0, H - 1] if H >= 32 else list(range(H))
+    assert_grads_close(gradients_of(inp, heads), oracle_backward(oracle, some_heads(inp, heads)), "bf16", f"{B}x{H}x{N}x{M}x{D}")
+
+
+# Ranges of latents side by side (few tokens) and one after the other (many).
+RANGES = [(2, 700, 784, 16), (4, 500, 1552, 8), (4, 500, 1040, 4), (64, 4800, 784, 16), (64, 4800, 1552, 8)]
+
+
+@pytest.mark.parametrize("H,N,M,D", RANGES)
+def test_peaked_softmaxes_over_ranges_of_latents(oracle, H, N, M, D):
+    """dd is what the ranges' shares of it add up to, each a float and what that lost: a token that follows one latent has a small row of dK, left of
+    large numbers, within what its own terms allow element by element."""
+    inp = workloads.make_random(1, H, N, M, D, dtype="bf16", seed=N + M, with_dy=True, k_std=80.0 / D if D > 4 else 12.0)
+    heads = [0, H - 1]
+    few = some_heads(inp, heads)
+    got, want = gradients_of(inp, heads)["dK"], oracle_backward(oracle, few)["dK"]
+    half_ulp = np.maximum(2.0 ** (np.floor(np.log2(np.maximum(np.abs(want), 1e-300))) - 8), 2.0 ** -133)
+    assert (np.abs(got - want) <= half_ulp + dk_error_bound(few, 2.0 ** -17)).all()
+
+
+@pytest.mark.parametrize("H,N,M,D", RANGES)
+def test_very_different_latents_over_ranges(oracle, H, N, M, D):
+    """lse_enc spread over several hundred powers of two within a range and between ranges: a weight of the encode softmax has an exponential of its own."""
+    inp = workloads.make_random(1, H, N, M, D, dtype="bf16", seed=N + M, masked_fraction=0.1, with_dy=True)
+    inp.Q.mul_(torch.linspace(0.05, 30.0, M)[None, :, None].to(inp.Q.dtype))
+    heads = [0, H - 1]
+    assert_grads_close(gradients_of(inp, heads), oracle_backward(oracle, some_heads(inp, heads)), "bf16", f"spread {H}x{N}x{M}x{D}")
+
+
+@pytest.mark.parametrize("H,N,M,D", RANGES)
+def test_features_with_a_mean_over_ranges(oracle, H, N, M, D):
+    """As in test_gpu_backward_tiles.py: dK within 2^-14 of its norm, beyond the rounding of what is stored, where the rows of Z are nearly equal."""
+    inp = workloads.make_random(1, H, N, M, D, dtype="bf16", seed=N + M, with_dy=True, k_std=D ** -0.5)
+    inp.V.mul_(D ** -0.5).add_(1.0)
+    heads = [0, H - 1]
+    got, want = gradients_of(inp, heads)["dK"], oracle_backward(oracle, some_heads(inp, heads))["dK"]
+    half_ulp = 2.0 ** (np.floor(np.log2(np.maximum(np.abs(want), 1e-300))) - 8)
+    assert np.linalg.norm(np.maximum(np.abs(got - want) - half_ulp, 0.0)) <= 2.0 ** -14 * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("H,N,M,first", [(1, 1024, 784, 64), (64, 4800, 784, 448)])
+def test_a_small_weight_of_one_range(oracle, H, N, M, first):
+    """test_small_weights_of_a_range_of_latents of test_gpu_backward_tiles.py at D = 16, with the first range's `first` latents."""
+    inp = workloads.make_random(1, H, N, M, 16, dtype="bf16", seed=4, with_dy=True)
+    inp.Q.zero_()
+    inp.Q[0, 0, 0], inp.Q[0, 1:first, 1], inp.Q[0, first:, 2] = 1.0, 1.0, 1.0
+    inp.K.zero_()
+    inp.K[0, 0, 0, :3] = torch.tensor([-26.25, -13.875, 59.0])
+    inp.K[0, 200, 0, 1], inp.K[0, 300, 0, 2] = 57.5, 132.0
+    got, want = gradients_of(inp, [0])["dV"][0, 0, 0], oracle_backward(oracle, some_heads(inp, [0]))["dV"][0, 0, 0]
+    assert np.linalg.norm(want) > 2.0 ** -60
+    assert np.linalg.norm(got - want) <= 2.0 ** -7 * np.linalg.norm(want)
 
 
 @pytest.mark.parametrize("M,D", [(32, 32), (64, 32), (32, 16)])
