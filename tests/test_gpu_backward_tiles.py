@@ -28,6 +28,8 @@ CASES = [  # B, H, N, M, D, masked_fraction, k_std
     (1, 2, 300, 64, 32, 0.1, 6.0),
     (1, 2, 300, 144, 16, 0.0, 9.0),
     (1, 1, 300, 64, 64, 0.0, 4.0),
+    (1, 2, 300, 336, 32, 0.1, 6.0),       # the same in the kernels that D = 32 takes beyond 320 latents, in one launch and in two
+    (1, 1, 300, 528, 32, 0.0, 6.0),
     (1, 1, 300, 512, 32, 0.1, 0.8),       # the most latents of one launch at D = 32, and ranges beyond
     (1, 1, 300, 528, 32, 0.1, 0.8),
     (1, 1, 260, 400, 64, 0.1, 0.8),       # three and four ranges: launches that neither begin nor end the sums, dd from either array
@@ -37,7 +39,8 @@ CASES = [  # B, H, N, M, D, masked_fraction, k_std
     (1, 2, 40000, 32, 32, 0.1, 0.8),      # two sets of warps, several tiles each
     (2, 1, 40000, 16, 8, 0.0, 0.8),
     (1, 2, 20001, 48, 16, 0.1, 0.8),
-    (8, 4, 20001, 256, 8, 0.0, 0.8),      # several rounds of CTAs over the chip, token side
+    (8, 4, 20001, 256, 8, 0.0, 0.8),      # 32 heads: once over the chip leaves 20 SMs idle
+    (8, 4, 20001, 96, 64, 0.0, 0.8),      # several rounds of CTAs over the chip
 ]
 
 
@@ -128,9 +131,10 @@ def test_rows_of_peaked_softmaxes(oracle, dtype, H, N, M, D, k_std):
 
 
 @pytest.mark.parametrize("value", [float("nan"), float("inf"), 0.0, 1e30])
-@pytest.mark.parametrize("M,D", [(64, 32), (144, 16), (208, 64)])
+@pytest.mark.parametrize("M,D", [(64, 32), (144, 16), (336, 32), (528, 32), (208, 64)])
 def test_any_stored_output(oracle, M, D, value):
-    """The stored Y is a first guess only: what a caller left there has no say in the gradients."""
+    """The stored Y is a first guess only (D = 64, and D = 32 with more than 320 latents, in one launch and in two; the two sweeps do not read it): what a caller
+    left there has no say in the gradients."""
     inp = workloads.make_random(2, 2, 300, M, D, dtype="bf16", seed=M, with_dy=True)
     Q, K, V, dY = (dev(t) for t in (inp.Q, inp.K, inp.V, inp.dY))
     desc = flare.make_desc(Q, K)

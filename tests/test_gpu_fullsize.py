@@ -141,7 +141,8 @@ def _float64_z_and_dq(Q, K, V, dY):
 def test_sums_over_a_million_tokens():
     """The tensor core truncates every float32 sum, so the number of sums in a row bounds how far Z and dQ drift at a million tokens:
     with at most 512 tiles to a split, five groups of warps and two halves of 8 steps to a tile, 1640 truncations of less than 2^-23 of a
-    sum that is half its size on average: 1e-4 of Z.  dQ: eight accumulators of 1024 truncations, 6e-5, beside what Z and dZ carry."""
+    sum that is half its size on average: 1e-4 of Z.  dZ and dQ are drained to float32 after at most 64 tiles of eight steps, 512 truncations of 2^-24 / 3 of
+    the whole on average (sweep_flush_tiles); beside them dQ carries the halves of its factors, 2^-18, and what Z is off by."""
     inp = workloads.make_inputs(workloads.CONFIGS["field_1m"])
     Q, K, V, dY = dev(inp.Q), dev(inp.K), dev(inp.V), dev(inp.dY)
     _, dQ, _, _ = flare.forward_backward(Q, K, V, dY, check=True)
@@ -149,4 +150,5 @@ def test_sums_over_a_million_tokens():
     for h in (0, 5):
         Z_ref, dQ_ref = _float64_z_and_dq(Q[h], K[0, :, h], V[0, :, h], dY[0, :, h])
         assert (Z[0, h] - Z_ref).norm() <= 1e-4 * Z_ref.norm()
-        assert (dQ[h] - dQ_ref).norm() <= 2.6e-4 * dQ_ref.norm()
+        from_z = ((Z[0, h] - Z_ref).norm() / Z_ref.norm()).item()
+        assert (dQ[h] - dQ_ref).norm() <= (2 * 512 * 2.0 ** -24 / 3 + 2.0 ** -18 + from_z) * dQ_ref.norm()

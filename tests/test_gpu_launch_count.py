@@ -34,6 +34,7 @@ def kernels_in(call):
     (1, 2, 1000, 16, 16, "f32"), (1, 2, 5000, 64, 16, "f32"), (1, 1, 300, 256, 64, "f32"), (1, 1, 300, 528, 32, "f16"), (1, 1, 200, 2048, 64, "f32"),
     (1, 2, 1000, 64, 16, "bf16"), (1, 2, 40000, 128, 32, "bf16"), (1, 1, 300, 208, 64, "bf16"), (1, 1, 300, 400, 64, "bf16"),
     (1, 1, 300, 1040, 32, "bf16"), (2, 1, 300, 288, 8, "bf16"),
+    (1, 2, 300, 784, 16, "bf16"), (1, 64, 4800, 784, 16, "bf16"), (1, 64, 25000, 784, 16, "bf16"), (4, 8, 700, 320, 32, "bf16"),
 ])
 def test_counts_are_what_is_launched(B, H, N, M, D, dtype):
     inp = workloads.make_random(B, H, N, M, D, dtype=dtype, seed=N + M, with_dy=True)

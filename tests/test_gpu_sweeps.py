@@ -120,23 +120,27 @@ def test_sums_over_tokens_are_made_of_few_parts(M, D):
     assert (dQ - want).norm() <= (2.0 ** -18 + 2 * 32 * 2.0 ** -24 / 3) * want.norm()
 
 
-def float64_gradients(Q, K, V, dY):
-    """dQ, dK, dV of one head in float64 by plain torch, on the device, a slice of tokens at a time."""
-    Q, step = Q.double(), 1 << 15
+def float64_gradients(Q, K, V, dY, Q_dec=None):
+    """Of one head in float64 by plain torch, on the device, a slice of tokens at a time: dQ, dK and dV; with latent queries of its own for decode dQ of encode and
+    of decode, the parts of dK from encode and from decode, and dV."""
+    Qe, Qd, step = Q.double(), (Q if Q_dec is None else Q_dec).double(), 1 << 15
     at = range(0, K.shape[0], step)
-    S = lambda a: K[a:a + step].double() @ Q.T
-    le = torch.logsumexp(torch.stack([torch.logsumexp(S(a), 0) for a in at]), 0)
-    Z = sum(torch.exp(S(a) - le).T @ V[a:a + step].double() for a in at)
-    dZ = sum(torch.softmax(S(a), 1).T @ dY[a:a + step].double() for a in at)
-    de, dQ, dK, dV = (dZ * Z).sum(1), torch.zeros_like(Q), [], []
+    S = lambda a, q: K[a:a + step].double() @ q.T
+    le = torch.logsumexp(torch.stack([torch.logsumexp(S(a, Qe), 0) for a in at]), 0)
+    Z = sum(torch.exp(S(a, Qe) - le).T @ V[a:a + step].double() for a in at)
+    dZ = sum(torch.softmax(S(a, Qd), 1).T @ dY[a:a + step].double() for a in at)
+    de, dQe, dQd, dKe, dKd, dV = (dZ * Z).sum(1), torch.zeros_like(Qe), torch.zeros_like(Qd), [], [], []
     for a in at:
         k, v, g = (x[a:a + step].double() for x in (K, V, dY))
-        Wd, We, A = torch.softmax(S(a), 1), torch.exp(S(a) - le), g @ Z.T
-        dS = Wd * (A - (Wd * A).sum(1, keepdim=True)) + We * (v @ dZ.T - de)
-        dQ += dS.T @ k
-        dK.append(dS @ Q)
+        Wd, We, A = torch.softmax(S(a, Qd), 1), torch.exp(S(a, Qe) - le), g @ Z.T
+        dSd, dSe = Wd * (A - (Wd * A).sum(1, keepdim=True)), We * (v @ dZ.T - de)
+        dQe += dSe.T @ k
+        dQd += dSd.T @ k
+        dKe.append(dSe @ Qe)
+        dKd.append(dSd @ Qd)
         dV.append(We @ dZ)
-    return dQ, torch.cat(dK), torch.cat(dV)
+    dKe, dKd, dV = torch.cat(dKe), torch.cat(dKd), torch.cat(dV)
+    return (dQe + dQd, dKe + dKd, dV) if Q_dec is None else (dQe, dQd, dKe, dKd, dV)
 
 
 @pytest.mark.parametrize("B,H,N,M,D", [(1, 8, 150001, 784, 16), (2, 8, 140000, 1040, 8), (1, 32, 40000, 784, 16)])
@@ -154,3 +158,25 @@ def test_chunks_of_tokens_between_ranges_of_latents(B, H, N, M, D):
         want = dict(dQ=to_np64(sum(x[0] for x in each)), dK=to_np64(torch.stack([x[1] for x in each])), dV=to_np64(torch.stack([x[2] for x in each])))
         assert_grads_close(got, want, "bf16", f"{B}x{H}x{N}x{M}x{D}")
         assert np.linalg.norm(got["dQ"] - want["dQ"]) <= (2.0 ** -18 + 2 * 512 * 2.0 ** -24 / 3) * np.linalg.norm(want["dQ"])
+
+
+def test_separate_decode_queries_over_ranges_one_after_the_other():
+    """The two runs of the sweeps each store their part of dK in bfloat16: it is off by a rounding of either part and one of their sum."""
+    B, H, N, M, D = 1, 64, 4800, 784, 8
+    inp = workloads.make_random(B, H, N, M, D, dtype="bf16", seed=3, with_dy=True, k_std=0.8)
+    Qe, K, V, dY = dev(inp.Q), dev(inp.K), dev(inp.V), dev(inp.dY)
+    Qd = dev(workloads.make_random(B, H, 1, M, D, dtype="bf16", seed=4).Q)
+    desc = flare.make_desc(Qe, K)
+    scratch = lambda op: torch.empty(flare.flare_variant_workspace_bytes(desc, op, False, True), dtype=torch.uint8, device="cuda")
+    f32 = lambda *shape: torch.empty(*shape, dtype=torch.float32, device="cuda")
+    Y, Z, le, ld, dQe, dQd, dK, dV = torch.empty_like(K), f32(B, H, M, D), f32(B, H, M), f32(B, N, H), f32(H, M, D), f32(H, M, D), torch.empty_like(K), torch.empty_like(V)
+    flare.flare_forward_variant(desc, False, Qe, Qd, K, V, None, Y, Z, le, ld, scratch(flare.OP_FORWARD))
+    ws = scratch(flare.OP_BACKWARD)
+    flare.flare_backward_variant(desc, False, Qe, Qd, K, V, None, Y, dY, Z, le, ld, dQe, dQd, dK, dV, ws)
+    flare.flare_check(ws)
+    for h in (0, H - 1):
+        we, wd, ke, kd, wv = (to_np64(x) for x in float64_gradients(Qe[h], K[0, :, h], V[0, :, h], dY[0, :, h], Qd[h]))
+        got_k, rms = to_np64(dK[0, :, h]), np.sqrt(np.mean((ke + kd) ** 2))
+        assert (np.abs(got_k - ke - kd) - 2.0 ** -8 * (np.abs(ke) + np.abs(kd) + np.abs(ke + kd))).max() <= 2e-2 * rms
+        for got, want in ((dQe, we), (dQd, wd)):
+            assert_grads_close(dict(dQ=to_np64(got[h]), dK=wv, dV=to_np64(dV[0, :, h])), dict(dQ=want, dK=wv, dV=wv), "bf16", f"head {h}")
