@@ -33,7 +33,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # summarised under profiles/ (taken on a 262,144-token slice and scaled by 4: traffic is proportional to N).
 # Valid for the kernels as profiled; set to None when a kernel changes until the capture is redone.
 NCU_TRAFFIC = {("mesh3d_1m", "encode"): 4 * (134.324736e6 + 4.828160e6),     # profiles/encode_lean_mesh3d_N262144.md
-               ("mesh3d_1m", "decode"): 4 * (67.351808e6 + 27.356416e6)}     # profiles/decode_stream_mesh3d_N262144.md
+               ("mesh3d_1m", "decode"): 4 * (67.349248e6 + 28.910592e6)}     # profiles/decode_stream_mesh3d_N262144.md
 
 
 def get_workload(name: str) -> workloads.Workload:

@@ -11,13 +11,14 @@
 //
 // Three kernels before (dZ with latents on the lanes; dK, dV and dd with tokens; dQ with latents) exponentiated every score three times and formed A and C
 // twice; here it is twice and once, and since dd is known when dS is formed, no first guess of it is needed (a pass over Y and dY) and nothing is put right
-// afterwards.  us per training step, before -> now: 16384 tokens, M = 32, D = 32, 8 heads 81 -> 65; 32 x 4096, M = 128, D = 32, 4 heads 289 -> 245; 131072
-// tokens, 8 heads, D = 32: M = 32 340 -> 233, 64 388 -> 298, 256 773 -> 657, 320 1014 -> 826; D = 16: M = 32 238 -> 215, 256 706 -> 624, 1024 2618 -> 2392; D = 8: M = 64 294 -> 262,
-// 1024 2525 -> 2345, 2048 5133 -> 4626; D = 4, 16 heads, M = 64 596 -> 503.  At D = 32 two ranges of latents, with float32 rows to read and write between
+// afterwards.  us per training step, before -> now, both timed in turn: 16384 tokens, M = 32, D = 32, 8 heads 86 -> 68; 32 x 4096, M = 128, D = 32, 4 heads 288 -> 238; 131072
+// tokens, 8 heads, D = 32: M = 32 327 -> 237, 64 375 -> 305, 256 771 -> 663, 320 1026 -> 830; D = 16: M = 16 238 -> 214, 32 239 -> 218, 256 705 -> 604, 1024 2616 -> 2312; D = 8: M = 64 285 -> 248,
+// 1024 2524 -> 2220, 2048 5129 -> 4373; D = 4, 16 heads, M = 64 596 -> 499.  At D = 32 two ranges of latents, with float32 rows to read and write between
 // them, are no faster (M = 400 1312 : 1309, 512 1391 : 1414): more than 320 latents take the kernels of flare_bwd_tc.cuh, and so do heads 64 wide.
 //
-// What bounds them: issue slots (59 to 63 % in use; some 225 warp instructions per 16 columns of a unit in the first, 400 in the second, of which 84 and 144 are the
-// arithmetic) and, lane by lane, latency: a unit takes a warp of the second 1250 cycles of work, 160 of finding its scores ready and 130 around.  Tensor core,
+// What bounds them: issue slots (54 to 64 % in use; some 210 warp instructions per 16 columns of a unit in the first, 340 in the second at D = 16, M = 256, of which
+// 84 and 144 are the arithmetic) and, lane by lane, latency: a unit takes a warp of the second 1250 cycles of work, 160 of finding its scores ready and 130 around.  All
+// forms of the second spill a few registers (8 to 24 bytes at 96 registers; taking them out by chance of code changed no time by more than 2 %).  Tensor core,
 // cycles per unit of 64 latents: S 48, A and C 96 each (D = 32: twice that), dV 100, dK and dZ or dQ 320 each (an instruction with both operands in shared memory takes 40,
 // whichever way its rows lie).  What the loop over a kernel's units should not hold is anything done once per tile: see the second kernel's.
 #pragma once
@@ -815,8 +816,9 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             };
             // What says that the products of unit n + 1 are there says as well that a buffer of dS has been read: with two buffers that of unit n - 1,
             // whose sums come before those products; with three that of n - 2, and dQ of unit n - 1 may come behind them.
-            // us per step, in order : late, 131072 tokens: D = 32, M = 32 233 : 262, 64 298 : 302, 32 x 4096, M = 128 236 : 239; D = 16, M = 64 270 : 262, 256 645 : 620.
-            const bool late = bufs == 3 && D == 16;
+            // us per step, in order : late, 131072 tokens, 8 heads: D = 32, M = 32 237 : 267, 64 305 : 313, 32 x 4096, M = 128 239 : 244; D = 16, M = 32 226 : 218, 64 260 : 258; in
+            // ranges, D = 8, M = 1024 2220 : 2270, D = 16 2312 : 2352.
+            const bool late = bufs == 3 && D == 16 && !kRanges;
             bool ok = products(0);
             for (int n = 0; ok && n < units; ++n) {
                 if (n + 1 < units) {
@@ -1021,13 +1023,13 @@ bwd_grad_sweep_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             }
             ptx::tmem_wait_st();
         };
-        // (what follows a first unsuccessful try: inline at D = 16, where it is 1 to 2 % quicker, a call at D = 32, where inline is slower)
+        // (what follows a first unsuccessful try: inline at D = 16, where it is up to 4 % quicker; a call at D = 32, where the two differ by less than 1 %)
         auto unit_wait = [&](uint32_t at, uint32_t parity, uint32_t code) { return D == 16 ? issue_wait(at, parity, abort_flag, code) : warp_wait(at, parity, abort_flag, code); };
         // The loop over the units has nothing else in it: with the rows in a branch of it, it carried some forty instructions of theirs (131072 tokens, M = 256, D =
-        // 16 649 -> 622 us per step, 32 x 4096, M = 128 259 -> 239 with what follows dd in a warp of its own).
+        // 16 649 -> 622 us per step when that was changed, 32 x 4096, M = 128 259 -> 239 with what follows dd in a warp of its own).
         // Rows of a tile leave after the first unit of the set's next, when they have long been formed; at D = 32 with two sets of warps at once: the other
-        // set is at work, and four tile stages are all there is room for (us per step at once : after the next unit, 131072 tokens: D = 32, M = 32 233 : 253, D = 16,
-        // M = 16 229 : 213, D = 8, M = 32 230 : 214).
+        // set is at work, and four tile stages are all there is room for (us per step at once : after the next unit, 131072 tokens, 8 heads: D = 32, M = 32 237 : 260, D =
+        // 16, M = 16 232 : 214, D = 8, M = 32 231 : 209).
         const bool at_once = D == 32 && sets == 2;
         int n = set;                                            // unit of all
         float r_before = 0.f;

@@ -13,8 +13,8 @@
 // What shapes them.  A tcgen05.mma with both operands in shared memory takes the tensor core 40 cycles at N = 16 or 32, 48 at 64 and 64
 // at 128 (most of it the fetch of its A operand), one with A in tensor memory N / 2; a hand-over between threads and tensor core
 // costs a warp some 100 instructions and a round trip of about 1000 cycles.  Units of 16 columns (dQ kernel at D = 32: ten MMAs of N = 16 for
-// 16 tokens) ran at exactly the tensor limit.  Wider units are shared by all warps (token kernel, up to 32 latents: by half of them, which served better than
-// groups of four warps with units of their own in both kernels).
+// 16 tokens) ran at exactly the tensor limit.  Wider units are shared by all warps, which served better than
+// groups of four warps with units of their own in both kernels.  They run for heads 64 wide, and 32 wide where the two sweeps do not (use_sweeps).
 #pragma once
 
 #include "flare_tc.cuh"
@@ -103,12 +103,9 @@ __device__ __forceinline__ void stage_hilo(uint8_t *hi, uint8_t *lo, const float
 // Units of 64 tokens, shared by sixteen warps, 16 columns each, on two alternating buffers of tensor memory (S | A | C; then the
 // accumulators): while the threads work on one unit the tensor core runs the output contractions of the other and the tiles of the one after.
 // Warps: 0 TMA producer, 1 MMA issue, 3 column constants, 4-19 arithmetic (warp & 3 = the quarter of the lanes it can reach).
-// Measured, us, against units of 16 columns with two exponentials per pair (N = 16384, M = 32, D = 32, 8 heads; 32 x 4096, M = 128, 4 heads;
-// 131072, M = 512, 8 heads; 1048576, M = 1024, D = 8, 8 heads): 22.4, 82, 437, 7844 -> 15.9, 65, 392, 5706; D = 64 (2 x 20011, M = 128, 4
-// heads), on the CUDA cores before: 498 -> 27 (in three
-// parts, see kThird, 31).  Groups of four warps with units and buffers of their own:
-// 21.6, 78, 522, 7485; 44.  Issue slots and the latency of tensor-memory loads share the bound (some 14 instructions per pair, two issued
-// per cycle and SM).
+// Measured, us, against units of 16 columns with two exponentials per pair: 131072 tokens, M = 512, D = 32, 8 heads 437 -> 392; D = 64 (2 x 20011, M = 128, 4
+// heads), on the CUDA cores before, 498 -> 27 (in three parts, see kThird, 31).  Groups of four warps with units and buffers of their own: 522; 44.  Issue
+// slots and the latency of tensor-memory loads share the bound (some 14 instructions per pair, two issued per cycle and SM).
 constexpr int kDqUnit = 64, kDqBuf = 3 * kDqUnit, kDqAcc = 2 * kDqBuf;
 constexpr int kDqThreads = 640, kDqFirstMathWarp = 4;
 
@@ -374,7 +371,7 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         }
     } else if (warp >= kDqFirstMathWarp) {
         const int cg = (warp - kDqFirstMathWarp) >> 2;         // the group of 16 columns this warp works on
-        const int row = ((warp & 3) << 5) + lane;               // TMEM lane = latent within the block (or within the pair)
+        const int row = ((warp & 3) << 5) + lane;               // TMEM lane = latent within the block
         const uint32_t gcol = tm + ((uint32_t)((warp & 3) << 5) << 16);
         const float2 sl2p = make_float2(a.sl2, a.sl2);
         const int m = lb * kTile + row;
@@ -508,10 +505,10 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // e[n], any number that is near dd[n], keeps the two from being large and nearly equal, each with the rounding of its halves, where the rows of Z
 // that a token weighs are nearly equal or one of them has most of the weight.  It comes from the stored Y (bwd_guess), which is dd up to the rounding of
 // Y; A has had a row near the middle of Z taken out as well (z_around).  Against float64, what is left of dK's error when the rounding of the stored value
-// is taken off, of the norm, with dd formed in a sweep of its own first : e = 0 : e from Y.  M = 64, D = 32, mean largest weight 0.70 4.8e-7 : 1.1e-6 : 5.7e-7
+// is taken off, of the norm, with dd formed in a sweep of its own first : e = 0 : e from Y.  M = 64, D = 32 (which the sweeps take now), mean largest weight 0.70 4.8e-7 : 1.1e-6 : 5.7e-7
 // (99th percentile of a row's 2.5e-5 : 1.9e-4 : 2.5e-6), 0.93 9.6e-6 : 1.2e-5 : 5.1e-6, 0.97 3.6e-5 : 3.8e-5 : 1.0e-5; features with
-// a mean of 1, M = 128, D = 32 2.3e-4 : 2.2e-6 : 2.2e-6.  e costs a packed addition per pair of columns and a pass over Y and dY, us per training step, e = 0 -> now: 16384 tokens, M = 32,
-// D = 32 77 -> 82; 32 x 4096, M = 128 266 -> 287; 2 x 20011, M = 128, D = 64 173 -> 180; 131072, M = 1024, D = 8 2472 -> 2530.
+// a mean of 1, M = 128, D = 32 2.3e-4 : 2.2e-6 : 2.2e-6.  e costs a packed addition per pair of columns and a pass over Y and dY, us per training step, e = 0 -> now: 131072 tokens, M =
+// 512, D = 32 1415 -> 1477; 2 x 20011, M = 128, D = 64 173 -> 180.
 // And W_enc = W_dec r[n] c[m] with r = 2^(lse_dec[n] - K), c = 2^(K - lse_enc[m]) and K in the middle of the latents' lse_enc, so that with
 // c dZ in the place of dZ one weight serves everything:
 //     T_n = sum_m W_dec (A - e + r (C' - c de)) q_m,   C' = V (c dZ)^T,     dV_n = r sum_m W_dec (c dZ)_m,
@@ -525,12 +522,11 @@ bwd_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 // whose halves are a third pair of operands (kTwo): 2^(S - K) against c dZ, c at most 2^(kFoldLog2 / 2); for wider ranges of lse_enc all tiles
 // do, and c is 1.
 //
-// Sixteen warps share units of 64 latents, 16 columns each, on two alternating buffers of tensor memory (S | A | C), as in the dQ kernel; up
-// to 32 latents two sets of eight warps take a tile each, so that no warp idles.  Rows leave the accumulators after the first unit of the next tile.
+// Sixteen warps share units of 64 latents, 16 columns each, on two alternating buffers of tensor memory (S | A | C), as in the dQ kernel.  Rows leave the accumulators after the first unit of the next tile.
 // D = 64: units of 32 shared by eight warps (the accumulators take 192 columns).
 // Two sweeps over the latents (dd first; two exponentials and 26 instructions per pair, here one and 20), by groups of four warps with units of their
-// own, took, us per training step -> now: 131072 tokens, M = 512, D = 32 (in two ranges, 448 latents at most) 1905 -> 1513; 1048576, M = 1024, D = 8 20967 -> 20025;
-// 32 x 4096, M = 128, D = 32 300 -> 283; 2 x 20011, M = 128, D = 64 187 -> 178; 16384, M = 32, D = 32 84.2 -> 85.1.
+// own, took, us per training step -> now: 131072 tokens, M = 512, D = 32 (in two ranges, 448 latents at most) 1905 -> 1513;
+// 2 x 20011, M = 128, D = 64 187 -> 178.
 constexpr float kFoldLog2 = 80.f;
 constexpr int kTokFirstMathWarp = 4;                            // warps: 0 TMA producer, 1 and 3 MMA issue, 2 token constants, 4 on arithmetic
 

@@ -12,7 +12,7 @@
 // What bounds it: 4.5 to 5.5 instructions per weight (an exponential on the special-function unit takes 2, on the FMA pipe 4.5; the two
 // share the work of the fast form), issued at 2.4 per cycle and SM; the unit is 60-75 % busy.
 // Measured, us, against units of 32 tokens on two buffers in a kernel with a running-maximum skeleton, four groups bound to halves of the
-// tile: dZ 4377 -> 2703 (million points, M = 1024, D = 8), 261 -> 190 (131072, M = 512, D = 32); weights as two halves 3692 -> 2627, 217 ->
+// tile: dZ 261 -> 190 (131072, M = 512, D = 32); weights as two halves 3692 -> 2627, 217 ->
 // 185; fast 522 -> 492 (million points, M = 256); masked, 262144 tokens, M = 96: 110 -> 82; D = 8 with 64 latents in head pairs: 85 -> 40.
 // Also measured: four groups 4 to 9 % slower than five; the warps of a group issuing in turn instead of a warp of its own 6 %; one guard
 // warp 20 %, three no better than two.
@@ -131,6 +131,7 @@ encode_lean_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constan
     using G = TileGeom<DG>;
     static_assert(!(kPair && DRT), "head pairs are full width");
     static_assert(!(kMask && kKind == kLeanDz), "dZ knows no mask");
+    static_assert(kKind != kLeanDz || (!kPair && DRT == 0), "dZ of head pairs and narrow heads is the sweeps'");
     constexpr bool kDz = kKind == kLeanDz, kTwo = kKind != kLeanFast;
     constexpr int UNIT = LG::UNIT, NG = LG::NG, nstages = LG::kStages, kThreads = LG::kThreads;
     extern __shared__ uint8_t smem_raw[];

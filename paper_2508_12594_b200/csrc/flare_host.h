@@ -411,8 +411,8 @@ struct BwdLayout {
 
 // Latents one launch of the tensor-core token kernel takes: five operands of D-wide bf16 rows (six at D = 64 up to 160 latents) beside two
 // tile stages; more are worked off in ranges of equal size, with three float32 planes and dd to read and write between them.  us per backward, two sweeps with
-// two planes and at most 448 latents a range at D = 32 : now, 8 heads of 131072 tokens: D = 32, M = 528 1778 : 1533, 640 1922 : 1587, 1024 3126 : 2284; D = 8,
-// M = 2048 4668 : 3818; 65536, D = 64, M = 208 852 : 874, 256 939 : 904, 400 1654 : 1671; 4 heads of 131072, M = 384 1128 : 1026.
+// two planes and at most 448 latents a range at D = 32 : now, 8 heads of 131072 tokens: D = 32, M = 528 1778 : 1533, 640 1922 : 1587, 1024 3126 : 2284;
+// 65536, D = 64, M = 208 852 : 874, 256 939 : 904, 400 1654 : 1671; 4 heads of 131072, M = 384 1128 : 1026.
 inline int token_range_most(const flare_desc_t *d) { return d->D == 64 ? 192 : 512; }
 inline bool token_in_ranges(const flare_desc_t *d) { return use_tc(d) && d->M > token_range_most(d); }
 inline int token_ranges(const flare_desc_t *d) { return (d->M + token_range_most(d) - 1) / token_range_most(d); }
@@ -431,9 +431,9 @@ inline bool use_sweeps(const flare_desc_t *d) {
 // worked off in ranges of about equal size, whole units of 64.
 // Ranges leave float32 rows of dK and dV to one another (in the first sweep RowSums): a launch takes a chunk of each item's tokens, so that the rows stay within
 // kRangeBytes (or, if that is more, within a tile to a CTA), and all ranges go over one chunk before the next.  Without a bound they are 1074 MB at 1048576 tokens of
-// 8 heads, D = 16.  us per backward, no bound : 128 : 64 : 32 : 16 MB, 8 heads, M = 1024: 1048576 tokens, D = 8 12408 : 13080 : 13200 : 13450 : 13900, 524288, D = 16
-// 6394 : 6586 : 6791 : 7136 : 7724, 131072, D = 16 1681 : 1644 : 1745 : 1822 : 1972 (a chunk starts and ends as any launch does, and chunks give 144 CTAs to the 148 SMs
-// where one launch of 1048576 tokens gives two rounds of 148).
+// 8 heads, D = 16.  us per training step, no bound : 128 : 64 : 32 MB, 8 heads, M = 1024: 1048576 tokens, D = 8 17000 : 17480 : 17620 : 17870; 524288, D = 16 8830 : 9170 : 9370 : 9720;
+// 131072, D = 16 2357 : 2352 : 2456 : 2534 (a chunk starts and ends as any launch does, and chunks give 144 CTAs to the 148 SMs where one launch over 1048576 tokens
+// gives two rounds of 148).
 constexpr size_t kRangeBytes = (size_t)128 << 20;
 // Ranges side by side, each with CTAs of its own and rows that a launch of its own adds up, where one after the other (or all latents in one) leaves a few CTAs
 // with many units each.  In the units of token_cost: what a sweep takes to start beyond that, and the launch that joins.  us per backward of 8 heads, one after
@@ -510,7 +510,7 @@ inline BwdLayout bwd_layout(const flare_desc_t *d, int sms) {
     w.dz = off;   off += align_up(sizeof(float) * (size_t)rows * d->D);
     w.de = off;   off += align_up(sizeof(float) * (size_t)rows);
     w.dd = off;   off += align_up(sizeof(float) * (use_sweeps(d) ? 2 : 1) * (size_t)d->B * d->N * d->H);
-    w.e = w.around = off;                                      // heads 64 wide: see bwd_guess, z_around
+    w.e = w.around = off;                                      // D = 64, and D = 32 beyond the sweeps: see bwd_guess, z_around
     if (use_tc(d) && !use_sweeps(d)) {
         w.around = off += align_up(sizeof(float) * (size_t)d->B * d->N * d->H);
         off += align_up(sizeof(float) * (size_t)(1 + latent_blocks(d)) * d->B * d->H * d->D);
