@@ -425,7 +425,7 @@ inline int token_range(const flare_desc_t *d) { return ((d->M + token_ranges(d) 
 inline bool use_sweeps(const flare_desc_t *d) {
     if (!use_tc(d) || d->D > 32) return false;
     const long tiles = (long)d->B * d->H * ((d->N + kTile - 1) / kTile);
-    return d->D <= 16 || (d->M <= 320 && !(d->M > 256 && tiles <= 100) && !(d->M == 256 && tiles <= 16));
+    return d->D <= 16 || (d->M <= 320 && tiles > (d->M > 256 ? 100 : d->M > 224 ? 16 : 0));
 }
 // Latents one launch of a sweep takes: what its operands leave of shared memory (beside two tile stages) and the sums over tokens of tensor memory; more are
 // worked off in ranges of about equal size, whole units of 64.

@@ -23,6 +23,8 @@ CASES = [  # B, H, N, M, D, masked_fraction
     (2, 4, 385, 64, 4, 0.1),
     (1, 1, 700, 320, 32, 0.1),            # the most latents at D = 32, few tiles and more than a hundred, and one more (other kernels)
     (4, 8, 700, 320, 32, 0.1),
+    (1, 8, 250, 256, 32, 0.1),            # at 240 and 256 latents sixteen tiles, and more
+    (1, 8, 300, 240, 32, 0.1),
     (1, 1, 700, 336, 32, 0.1),
     (1, 1, 300, 768, 16, 0.0),            # few tokens, ranges of latents side by side: the last of all sizes, one and several tiles to a CTA
     (1, 2, 300, 784, 16, 0.1),
